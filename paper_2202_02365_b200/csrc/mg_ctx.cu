@@ -310,12 +310,15 @@ extern "C" int mg_create(mg_ctx** out, int device, void* stream) {
         cudaMalloc((void**)&c->d_slot_of_part, sizeof(int32_t) * MG_MAX_PARTS) != cudaSuccess ||
         cudaMalloc((void**)&c->d_res_prefix, sizeof(int64_t) * (MG_MAX_PARTS + 1)) != cudaSuccess ||
         cudaMalloc((void**)&c->d_part_start, sizeof(int64_t) * (MG_MAX_PARTS + 1)) != cudaSuccess ||
-        cudaMalloc((void**)&c->d_flags, sizeof(uint32_t)) != cudaSuccess ||
-        cudaMemset(c->d_flags, 0, sizeof(uint32_t)) != cudaSuccess) {
+        cudaHostAlloc((void**)&c->h_flags, 4 * sizeof(uint32_t), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer((void**)&c->d_flags, c->h_flags, 0) != cudaSuccess) {
         cudaGetLastError();
         delete c;
         return MG_ERR_CUDA;
     }
+    *c->h_flags = 0;
+    c->lp_words = reinterpret_cast<int32_t*>(c->h_flags + 2);
+    c->lp_words_dev = reinterpret_cast<int32_t*>(c->d_flags + 2);
     *out = c;
     return MG_OK;
 }
@@ -352,13 +355,12 @@ extern "C" int mg_destroy(mg_ctx* c) {
     free_view(c);
     free_features(c);
     free_out_graph(c);
-    cudaFree(c->row_off); cudaFree(c->nbrs); cudaFree(c->d_slot_of_part); cudaFree(c->d_res_prefix); cudaFree(c->d_flags);
+    cudaFree(c->row_off); cudaFree(c->nbrs); cudaFree(c->d_slot_of_part); cudaFree(c->d_res_prefix); cudaFreeHost(c->h_flags);
     cudaFree(c->view_ws); cudaFree(c->d_part_start); cudaFree(c->d_part_of_node); cudaFree(c->d_local_of_node); cudaFree(c->d_nodes_by_part);
-    cudaFree(c->ws_x); cudaFree(c->ws_h[0]); cudaFree(c->ws_h[1]);
+    cudaFree(c->ws_x); cudaFree(c->ws_meta); cudaFree(c->ws_h[0]); cudaFree(c->ws_h[1]);
     cudaEventDestroy(c->ev_fwd_done); cudaEventDestroy(c->ev_out_done); cudaEventDestroy(c->ev_user);
     for (int i = 0; i < 2; ++i) { if (c->ev_hk_done[i]) cudaEventDestroy(c->ev_hk_done[i]); cudaFree(c->hk_buf[i]); }
     cudaFree(c->lp_ws); cudaFree(c->lp_spare); cudaFree(c->dm_images); cudaFree(c->lp_range);
-    if (c->lp_words) cudaFreeHost(c->lp_words);
     cudaFree(c->bw_g); cudaFree(c->bw_x); cudaFree(c->bw_dx); cudaFree(c->bw_off); cudaFree(c->bw_rev);
     cudaFree(c->gat_x); cudaFree(c->gat_z); cudaFree(c->gat_s); cudaFree(c->gat_h[0]); cudaFree(c->gat_h[1]);
     cudaStreamDestroy(c->sample_stream);

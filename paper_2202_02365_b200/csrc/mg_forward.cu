@@ -24,9 +24,9 @@ int mg_gemm_tf32_splitk_add_rows(mg_ctx* ctx, const float* x, const float* g, fl
 int mg_pack_layer_weights(mg_ctx* ctx, const float* w_cat_dev, float* w_pad_t_dev, int d_in, int N);
 int mg_pack_layer_weights_f16(mg_ctx* ctx, const float* w_cat_dev, void* w_pad_h_dev, int d_in, int N);
 bool mg_layer_fused_supported(int d_in, int d_out);
-int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, int4* row_meta);
+int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int4* meta, const int64_t* start /* [k + 2], layer l at start[l] */);
 int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* w_pad_t, const float* bias,
-                   const float* h_prev, float* h_out, int flags /* 1 = ReLU, 2 = sum instead of mean */, const int4* row_meta,
+                   const float* h_prev, float* h_out, float* h_out2 /* nullable: the rows once more */, int flags /* 1 = ReLU, 2 = sum instead of mean */, const int4* row_meta,
                    int64_t row_lo, int64_t row_hi, int64_t safe_src_row, const void* w_pad_h /* the layer's fp16 weights, nullable */,
                    int in_f16 /* layers >= 2: h_prev holds fp16 rows */, int out_f16 /* h_out receives fp16 rows */);
 
@@ -431,7 +431,8 @@ static int64_t chunk_rows_for(int d_in) {
 enum { OUT_DEVICE = 0, OUT_HOST = 1, OUT_HOST_ASYNC = 2 };
 
 // hands H^k (device, packed) to the caller: device or host copy, blocking or on the side stream
-static int finish_forward(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out, int out_mode, const float* hk) {
+// (out_written: the last layer's kernel has stored the rows there itself)
+static int finish_forward(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out, int out_mode, const float* hk, bool out_written) {
     cudaStream_t st = ctx->stream;
     if (!d->ev_read_done) MG_CUDA(ctx, cudaEventCreateWithFlags(&d->ev_read_done, cudaEventDisableTiming));
     MG_CUDA(ctx, cudaEventRecord(d->ev_read_done, st));   // the next sample into d waits for this
@@ -449,7 +450,7 @@ static int finish_forward(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* ou
         ctx->out_check_gemm = m->precision == MG_GEMM_TF32;
         return MG_OK;
     }
-    MG_CUDA(ctx, cudaMemcpyAsync(out, hk, out_bytes, out_mode == OUT_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
+    if (!out_written) MG_CUDA(ctx, cudaMemcpyAsync(out, hk, out_bytes, out_mode == OUT_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
     MG_CUDA(ctx, cudaStreamSynchronize(st));
     if (m->precision == MG_GEMM_TF32) return mg_gemm_tf32_status(ctx);
     return MG_OK;
@@ -486,14 +487,28 @@ static int forward_impl(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
     // next sub-group before most of it is written back to DRAM.
     bool all_fused = m->precision == MG_GEMM_TF32;
     for (int l = 1; l <= k; ++l) all_fused = all_fused && mg_layer_fused_supported(m->dims[l - 1], m->dims[l]);
+    // row metadata of the layers the fused kernel runs, all in one launch
+    const bool any_fused = m->precision == MG_GEMM_TF32;
+    int64_t meta_at[MG_MAX_HOPS + 2] = {0};
+    for (int l = 1; l <= k; ++l)
+        meta_at[l + 1] = meta_at[l] + (any_fused ? (int64_t)d->h_hdr.rows_total[l] : 0);
+    if (any_fused) {
+        const size_t need = (size_t)meta_at[k + 1];
+        if (ctx->ws_meta_elems < need && (rc = mg_ensure(ctx, &ctx->ws_meta, &ctx->ws_meta_elems, need + need / 4 + 4))) return rc;
+        ProfScope ps(ctx, PH_OTHER, 1);
+        if ((rc = mg_layer_rows(ctx, d, ctx->ws_meta, meta_at))) return rc;
+    }
+    // H^k stays in the library's buffer (mg_layer_output, mg_backward) and goes to the caller's: the last layer's kernel
+    // stores its tiles to both when it can (the copy behind it read and wrote the rows once more: 41 us for 128,000 rows of
+    // 1 KB, and a launch)
+    float* out2 = out_mode == OUT_DEVICE && any_fused && mg_layer_fused_supported(m->dims[k - 1], m->dims[k]) &&
+                  (reinterpret_cast<uintptr_t>(out) & 15) == 0 ? out : nullptr;
     const int sub = ctx->layer_window_batches;
     ctx->layers_kept = !(all_fused && sub > 0 && !ctx->keep_layers && k > 1);
     if (!ctx->layers_kept) {
         const int32_t* rb = d->h_rowbase.data();      // [(k+1)][B+1]
-        size_t ring_off[MG_MAX_HOPS + 1] = {0}, ring_total = 0, meta_off[MG_MAX_HOPS + 1] = {0}, meta_total = 0;
+        size_t ring_off[MG_MAX_HOPS + 1] = {0}, ring_total = 0;
         for (int l = 1; l <= k; ++l) {
-            meta_off[l] = meta_total;
-            meta_total += (size_t)d->h_hdr.rows_total[l];
             ring_off[l] = ring_total;
             if (l == k) break;
             int64_t widest = 0;
@@ -508,21 +523,6 @@ static int forward_impl(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
             if (have < ring_total && (rc = mg_ensure(ctx, &ctx->ws_h[0], &have, ring_total + ring_total / 4))) return rc;
             ctx->ws_h_bytes[0] = have * sizeof(float);
         }
-        int4* meta = reinterpret_cast<int4*>(ctx->ws_x);
-        {
-            size_t have = ctx->ws_x_bytes / sizeof(int4);
-            if (have < meta_total) {
-                rc = mg_ensure(ctx, &meta, &have, meta_total + meta_total / 4);
-                ctx->ws_x = reinterpret_cast<float*>(meta);
-                ctx->ws_x_bytes = have * sizeof(int4);
-                if (rc) return rc;
-            }
-        }
-        {
-            ProfScope ps(ctx, PH_OTHER, k);
-            for (int l = 1; l <= k; ++l)
-                if ((rc = mg_layer_rows(ctx, d, l, m->dims[l - 1], m->dims[l], meta + meta_off[l]))) return rc;
-        }
         float* base = ctx->ws_h[0];
         for (int b0 = 0; b0 < B; b0 += sub) {
             const int b1 = std::min(B, b0 + sub);
@@ -533,13 +533,13 @@ static int forward_impl(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
                 const float* h_prev = l > 1 ? base + ring_off[l - 1] - lo_in * m->dims[l - 1] : nullptr;
                 float* h_out = l == k ? hk : base + ring_off[l] - lo * m->dims[l];
                 ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST, 1);
-                rc = mg_layer_fused(ctx, d, l, m->dims[l - 1], m->dims[l], m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out,
-                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), meta + meta_off[l], lo, hi, l > 1 ? lo_in : 0, l == 1 ? m->w_pad_h[0] : nullptr, 0, 0);
+                rc = mg_layer_fused(ctx, d, l, m->dims[l - 1], m->dims[l], m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
+                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], lo, hi, l > 1 ? lo_in : 0, l == 1 ? m->w_pad_h[0] : nullptr, 0, 0);
                 if (rc) return rc;
             }
         }
         MG_CUDA(ctx, cudaGetLastError());
-        return finish_forward(ctx, m, d, out, out_mode, hk);
+        return finish_forward(ctx, m, d, out, out_mode, hk, out2 != nullptr);
     }
 
     // per-layer outputs H^1..H^k live in one workspace (kept for mg_layer_output).  A model may ask for fp16
@@ -566,12 +566,13 @@ static int forward_impl(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
     char* ws_bytes = reinterpret_cast<char*>(ctx->ws_h[0]);
     int64_t max_x = 0;
     for (int l = 1; l <= k; ++l) {
+        if (m->precision == MG_GEMM_TF32 && mg_layer_fused_supported(m->dims[l - 1], m->dims[l])) continue;
         const int64_t rows = std::min<int64_t>(chunk_rows_for(m->dims[l - 1]), d->h_hdr.rows_total[l]);
         max_x = std::max<int64_t>(max_x, rows * 2 * m->dims[l - 1]);
     }
     {
         size_t have = ctx->ws_x_bytes / sizeof(float);
-        if ((rc = mg_ensure(ctx, &ctx->ws_x, &have, (size_t)max_x))) return rc;
+        if (max_x > 0 && (rc = mg_ensure(ctx, &ctx->ws_x, &have, (size_t)max_x))) return rc;
         ctx->ws_x_bytes = have * sizeof(float);
     }
 
@@ -582,24 +583,11 @@ static int forward_impl(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
         float* h_out = l == k ? hk : reinterpret_cast<float*>(ws_bytes + off[l]);
         const float* h_prev = l > 1 ? reinterpret_cast<const float*>(ws_bytes + off[l - 1]) : nullptr;
         if (m->precision == MG_GEMM_TF32 && mg_layer_fused_supported(d_in, d_out)) {
-            // gather + segment mean + both linear maps in one persistent tensor-core kernel (after a small
-            // pre-pass that resolves every output row's sources)
-            size_t have = ctx->ws_x_bytes / sizeof(int4);
-            int4* meta = reinterpret_cast<int4*>(ctx->ws_x);
-            if (have < (size_t)M) {
-                rc = mg_ensure(ctx, &meta, &have, (size_t)M + (size_t)M / 4);
-                ctx->ws_x = reinterpret_cast<float*>(meta);
-                ctx->ws_x_bytes = have * sizeof(int4);
-                if (rc) return rc;
-            }
-            {
-                ProfScope ps(ctx, PH_OTHER, 1);
-                if ((rc = mg_layer_rows(ctx, d, l, d_in, d_out, meta))) return rc;
-            }
+            // gather + segment mean + both linear maps in one persistent tensor-core kernel
             {
                 ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST, 1);
-                rc = mg_layer_fused(ctx, d, l, d_in, d_out, m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out,
-                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), meta, 0, M, 0,
+                rc = mg_layer_fused(ctx, d, l, d_in, d_out, m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
+                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], 0, M, 0,
                                     (l == 1 || f16_inter) ? m->w_pad_h[l - 1] : nullptr, f16_inter && l > 1, f16_inter && l < k);
             }
             if (rc) return rc;
@@ -644,7 +632,7 @@ static int forward_impl(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
         }
     }
     MG_CUDA(ctx, cudaGetLastError());
-    return finish_forward(ctx, m, d, out, out_mode, hk);
+    return finish_forward(ctx, m, d, out, out_mode, hk, out2 != nullptr);
 }
 
 extern "C" int mg_forward(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out, int out_on_device) {

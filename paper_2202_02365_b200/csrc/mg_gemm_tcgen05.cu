@@ -33,7 +33,7 @@ struct GemmParams {
     int32_t N, K, BN, stages, tmem_cols, relu;
     int32_t kt_per_slice;   // split-K: blockIdx.z owns this many 32-wide K steps and ADDS its product to out (0 = whole K, plain store)
     int32_t mn_major;       // 1: the operands are stored [K, M] and [K, N] (the contraction runs over their rows)
-    uint32_t* error;  // device word: 0 = ok, else the role that gave up waiting
+    uint32_t* error;  // 0 = ok, else the role that gave up waiting
 };
 
 __global__ void __launch_bounds__(kGemmThreads)
@@ -72,7 +72,7 @@ k_gemm_tf32(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         if (lane == 0) {
             for (int kt = 0; kt < kt_total; ++kt) {
                 const int s = kt % p.stages;
-                if (kt >= p.stages && !mbar_wait(&empty_bar[s], ((kt / p.stages) - 1) & 1)) { atomicExch(p.error, 1u); break; }
+                if (kt >= p.stages && !mbar_wait(&empty_bar[s], ((kt / p.stages) - 1) & 1)) { report(p.error, 1u); break; }
                 uint8_t* sa = stage_base + (size_t)s * stage_bytes;
                 mbar_expect_tx(&full_bar[s], stage_bytes);
                 if (p.mn_major) {   // boxes of 32 K rows x 32 floats of M (or N): the tile's 32-float blocks one after the other
@@ -96,7 +96,7 @@ k_gemm_tf32(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             bool ok = true;
             for (int kt = 0; kt < kt_total && ok; ++kt) {
                 const int s = kt % p.stages;
-                if (!mbar_wait(&full_bar[s], (kt / p.stages) & 1)) { atomicExch(p.error, 2u); ok = false; break; }
+                if (!mbar_wait(&full_bar[s], (kt / p.stages) & 1)) { report(p.error, 2u); ok = false; break; }
                 tc_fence_after();
                 const uint32_t sa = smem_u32(stage_base + (size_t)s * stage_bytes);
                 if (p.mn_major) {
@@ -117,7 +117,7 @@ k_gemm_tf32(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         __syncwarp();
     } else {
         const bool ok = mbar_wait(&acc_bar, 0);
-        if (!ok && lane == 0) atomicExch(p.error, 3u);
+        if (!ok && lane == 0) report(p.error, 3u);
         tc_fence_after();
         const int lane_group = warp & 3;                 // tensor-memory lanes this warp may read
         const int64_t row0 = m0 + lane_group * 32;
@@ -192,9 +192,8 @@ int mg_gemm_tf32_splitk_add_rows(mg_ctx* ctx, const float* x, const float* g, fl
 
 // After the stream has drained: MG_ERR_TIMEOUT if a GEMM gave up on a barrier (the word is cleared).
 int mg_gemm_tf32_status(mg_ctx* ctx) {
-    uint32_t flag = 0;
-    MG_CUDA(ctx, cudaMemcpy(&flag, ctx->d_flags, sizeof(uint32_t), cudaMemcpyDeviceToHost));
+    const uint32_t flag = *static_cast<volatile uint32_t*>(ctx->h_flags);
     if (!flag) return MG_OK;
-    cudaMemset(ctx->d_flags, 0, sizeof(uint32_t));
+    *ctx->h_flags = 0;
     return mg_fail(ctx, MG_ERR_TIMEOUT, "tensor-core GEMM gave up waiting on a barrier (role %u)", flag);
 }

@@ -66,7 +66,10 @@ struct mg_ctx {
     std::string err;
     int64_t launches = 0;
     int n_sms = 148;
-    uint32_t* d_flags = nullptr;  // device word the tensor-core GEMM reports a barrier time-out in
+    // word the tensor-core kernels report a barrier time-out in: mapped host memory (a copy of a device word cost a forward pass
+    // 17 us behind its last kernel), read by the host once the stream has drained; d_flags is its device address
+    uint32_t* h_flags = nullptr;
+    uint32_t* d_flags = nullptr;
 
     // graph store (device)
     int64_t n_nodes = 0, n_edges = 0;
@@ -123,7 +126,7 @@ struct mg_ctx {
     // forward workspaces (grown on demand)
     float* ws_x = nullptr; size_t ws_x_bytes = 0;
     float* ws_h[2] = {nullptr, nullptr}; size_t ws_h_bytes[2] = {0, 0};
-    float** ws_layer = nullptr;
+    int4* ws_meta = nullptr; size_t ws_meta_elems = 0;   // row metadata of the fused layers (mg_layer_rows)
 
     // forward schedule
     int32_t layer_window_batches = 0;  // mini-batches per window of the layer schedule; 0 = whole layers
@@ -147,7 +150,7 @@ struct mg_ctx {
     // loop of prepare / free allocates nothing
     char* lp_ws = nullptr; size_t lp_ws_bytes = 0;
     char* lp_spare = nullptr; size_t lp_spare_bytes = 0;
-    int32_t* lp_words = nullptr;       // mapped pinned host words {status, n_targets} that mg_lp_prepare's last kernel writes
+    int32_t* lp_words = nullptr;       // mapped pinned host words {status, n_targets} that mg_lp_prepare's last kernel writes (behind h_flags)
     int32_t* lp_words_dev = nullptr;   // their device address
     int32_t* lp_range = nullptr;       // device {0, 32-word groups of the node bitmap}: the bounds of mg_lp_prepare's scan
     int64_t lp_range_words = -1;
@@ -323,6 +326,14 @@ struct ProfScope {
     ProfScope(mg_ctx* ctx, int phase, int launches) : c(ctx), ph(phase), n(launches) { mg_prof_begin(c, ph); }
     ~ProfScope() { mg_prof_end(c, ph, n); }
 };
+
+// dynamic shared-memory limit of a kernel, raised once per device and not before every launch (`done`: the launch site's own bits)
+static inline cudaError_t mg_smem_limit(uint64_t* done, int device, const void* kernel, int bytes) {
+    if (device < 64 && (*done >> device & 1)) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && device < 64) *done |= 1ull << device;
+    return e;
+}
 
 static inline int mg_grid(const mg_ctx* ctx, int ctas_per_sm) { return ctx->n_sms * ctas_per_sm; }
 

@@ -103,6 +103,7 @@ struct FusedArgs {
     int32_t out_f16;             // the output rows are stored as fp16 (an intermediate layer of a model that keeps them so)
     const float* bias;
     float* out;                  // [M, N]
+    float* out2;                 // the same rows once more, for the caller (the last layer with a device output), or null
     uint32_t* error;
 };
 
@@ -187,7 +188,8 @@ template <> struct PieceSum<true> {
 // the weights in shared memory a half tile waits for eight 16 KB slices through a two-stage ring (4 us of latency).
 template <bool FIRST, bool HALF, bool F16, bool TS = false>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(MG_FUSED_MAXNREG)
-k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_out, FusedArgs a) {
+k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_out,
+                   const __grid_constant__ CUtensorMap map_out2, FusedArgs a) {
     constexpr int KCE = Geo<F16>::kKC, GC = Geo<F16>::kGroup, LC = Geo<F16>::kLaneCols;
     extern __shared__ uint8_t smem_raw[];
     // a_ready and acc_empty are used in the leader CTA only (both CTAs arrive there); a_free, b_empty and acc_full
@@ -303,7 +305,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                         const int gch = min(kSlicesPerGroup, n_chunks - grp * kSlicesPerGroup);
                         for (int c = 0; c < gch; ++c, ++cnt) {
                             const int s = cnt % a.sb;
-                            if (cnt >= (uint32_t)a.sb && !mbar_wait(&b_empty[s], ((cnt / a.sb) - 1) & 1)) { atomicExch(a.error, 11u); ok = false; break; }
+                            if (cnt >= (uint32_t)a.sb && !mbar_wait(&b_empty[s], ((cnt / a.sb) - 1) & 1)) { report(a.error, 11u); ok = false; break; }
                             if (leader) mbar_expect_tx(&b_full[s], 2 * b_bytes);   // both halves are counted on the leader's barrier
                             tma_load_2d_pair(b_base + (size_t)s * b_bytes, &map_w, mapa_u32(smem_u32(&b_full[s]), 0),
                                              (grp * kSlicesPerGroup + c) * KCE, (int)rank * half_n);
@@ -317,14 +319,14 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
             // M = 256 output columns over the pair, N = 128 rows (a half tile of each CTA), fp32 accumulate, K-major
             const uint32_t idesc = (1u << 4) | ((F16 ? 0u : 2u) << 7) | ((F16 ? 0u : 2u) << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
             bool ok = mbar_wait(&w_ready, 0);
-            if (!ok) atomicExch(a.error, 18u);
+            if (!ok) report(a.error, 18u);
             tc_fence_after();
             for (uint32_t it = 0; it < my_iters && ok; ++it)
                 for (int h = 0; h < 2 && ok; ++h) {
                     const uint32_t hu = it * 2 + h, buf = hu & 1;
-                    if (hu >= 2 && !mbar_wait(&acc_empty[buf], ((hu >> 1) - 1) & 1)) { atomicExch(a.error, 12u); ok = false; break; }
+                    if (hu >= 2 && !mbar_wait(&acc_empty[buf], ((hu >> 1) - 1) & 1)) { report(a.error, 12u); ok = false; break; }
                     tc_fence_after();
-                    if (!mbar_wait(&a_ready[h], it & 1)) { atomicExch(a.error, 13u); ok = false; break; }
+                    if (!mbar_wait(&a_ready[h], it & 1)) { report(a.error, 13u); ok = false; break; }
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + kTsAcc0 + buf * kTsAccCols;
                     for (int c = 0; c < n_chunks; ++c) {
@@ -353,16 +355,16 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                         const uint32_t buf = hu % kAccBufs;
                         const uint32_t s_h = it * (uint32_t)n_groups + grp;   // fills of half h's stage rows so far
                         if (grp == 0) {
-                            if (hu >= (uint32_t)kAccBufs && !mbar_wait(&acc_empty[buf], ((hu / kAccBufs) - 1) & 1)) { atomicExch(a.error, 12u); ok = false; break; }
+                            if (hu >= (uint32_t)kAccBufs && !mbar_wait(&acc_empty[buf], ((hu / kAccBufs) - 1) & 1)) { report(a.error, 12u); ok = false; break; }
                             tc_fence_after();
                         }
                         // both CTAs' producers have filled the half's rows of this group's K slices
-                        if (!mbar_wait(&a_ready[h], s_h & 1)) { atomicExch(a.error, 13u); ok = false; break; }
+                        if (!mbar_wait(&a_ready[h], s_h & 1)) { report(a.error, 13u); ok = false; break; }
                         const uint32_t d_tmem = tmem_base + buf * acc_stride;
                         const int gch = min(kSlicesPerGroup, n_chunks - grp * kSlicesPerGroup);
                         for (int c = 0; c < gch; ++c, ++cnt) {
                             const int sb = cnt % a.sb;
-                            if (!mbar_wait(&b_full[sb], (cnt / a.sb) & 1)) { atomicExch(a.error, 13u); ok = false; break; }
+                            if (!mbar_wait(&b_full[sb], (cnt / a.sb) & 1)) { report(a.error, 13u); ok = false; break; }
                             tc_fence_after();
                             const uint64_t da = smem_desc_sw128(smem_u32(a_base + (size_t)c * kABytes + (size_t)h * (HM * 128)));
                             const uint64_t db = smem_desc_sw128(smem_u32(b_base + (size_t)sb * b_bytes));
@@ -388,13 +390,19 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
         constexpr int kPlanners = TS ? kPlannerWarps + 1 : kPlannerWarps;
         const int plw = warp == kTmaWarp ? kPlannerWarps : warp - kFirstPlannerWarp;
         const int32_t* keys = FIRST ? a.ent_nbrs : a.ent_repr;
+        // The kernel may have started while the one before it (the row metadata, the layer below) still runs.  Barriers, tensor
+        // memory and the weights -- which only kernels before the row metadata's write -- do not wait for it; the planners do,
+        // and what the gather and epilogue warps touch comes behind the planners' barriers.  (The two instructions in every
+        // warp cost the gather warps registers: the first layer of 128 mini-batches 1.81 -> 1.86 ms.)
+        pdl_trigger();
+        pdl_wait();
         bool ok = true;
         for (uint32_t q = plw; ok; q += kPlanners) {
             if (q / kBlocksPerTile >= my_iters) break;
             const int64_t t = tile_of(q / kBlocksPerTile);   // past the end for the peer of an odd last tile: all padding
             const int slot = q % kPlanSlots;
             if (q >= (uint32_t)kPlanSlots && !mbar_wait(&plan_empty[slot], ((q / kPlanSlots) - 1) & 1)) {
-                if (lane == 0) atomicExch(a.error, 17u);
+                if (lane == 0) report(a.error, 17u);
                 ok = false;
             }
             ok = __all_sync(0xFFFFFFFFu, ok);
@@ -478,7 +486,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
             uint8_t* stage = reinterpret_cast<uint8_t*>(out_stage[lane_group]);
             for (uint32_t hu = 0; hu < 2 * my_iters && ok; ++hu) {
                 const uint32_t buf = hu & 1;
-                if (!mbar_wait(&acc_full[buf], (hu >> 1) & 1)) { if (lane == 0) atomicExch(a.error, 14u); ok = false; break; }
+                if (!mbar_wait(&acc_full[buf], (hu >> 1) & 1)) { if (lane == 0) report(a.error, 14u); ok = false; break; }
                 tc_fence_after();
                 for (int g = 0; g < 4; ++g) {
                     uint32_t v[32];
@@ -500,8 +508,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                     __syncwarp();
                     if (lane == 0) {
                         // rows past the end of the layer and columns past its width are clipped by the tensor map
-                        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                     ::"l"(&map_out), "r"(smem_u32(stage)), "r"(n0), "r"((int)row0) : "memory");
+                        tma_store_2d(&map_out, stage, n0, (int)row0);
+                        if (a.out2) tma_store_2d(&map_out2, stage, n0, (int)row0);
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
                 }
@@ -516,7 +524,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
         for (uint32_t hu = 0; !TS && hu < 2 * my_iters && ok; ++hu) {
             const int64_t t = tile_of(hu >> 1);
             const uint32_t buf = hu % kAccBufs;
-            if (!mbar_wait(&acc_full[buf], (hu / kAccBufs) & 1)) { if (lane == 0) atomicExch(a.error, 14u); ok = false; break; }
+            if (!mbar_wait(&acc_full[buf], (hu / kAccBufs) & 1)) { if (lane == 0) report(a.error, 14u); ok = false; break; }
             tc_fence_after();
             const int64_t row0 = a.row_lo + t * BM + (hu & 1) * HM + (lane_group & 1) * 32;
             uint8_t* stage = reinterpret_cast<uint8_t*>(out_stage[lane_group]);
@@ -556,8 +564,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                         fence_async_smem();
                         __syncwarp();
                         if (lane == 0) {
-                            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                         ::"l"(&map_out), "r"(smem_u32(stage)), "r"(ncol0 - 48), "r"((int)row0) : "memory");
+                            tma_store_2d(&map_out, stage, ncol0 - 48, (int)row0);
                             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                         }
                     }
@@ -585,8 +592,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                         __syncwarp();
                         if (lane == 0) {
                             // rows past the end of the layer and columns past its width are clipped by the tensor map
-                            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                         ::"l"(&map_out), "r"(smem_u32(stage)), "r"(ncol0 - 16), "r"((int)row0) : "memory");
+                            tma_store_2d(&map_out, stage, ncol0 - 16, (int)row0);
+                            if (a.out2) tma_store_2d(&map_out2, stage, ncol0 - 16, (int)row0);
                             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                         }
                     }
@@ -594,7 +601,6 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                     // the ragged end of the half (BN / 2 is not a multiple of 32): lane = row, plain stores
                     const int64_t row = row0 + lane;
                     if (row < a.M) {
-                        float* orow = a.out + row * a.N;
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
                             const int n = ncol0 + 4 * c;
@@ -603,7 +609,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                                 float4 o = make_float4(__uint_as_float(v[4 * c]) + bb.x, __uint_as_float(v[4 * c + 1]) + bb.y,
                                                        __uint_as_float(v[4 * c + 2]) + bb.z, __uint_as_float(v[4 * c + 3]) + bb.w);
                                 if (a.relu) { o.x = fmaxf(o.x, 0.f); o.y = fmaxf(o.y, 0.f); o.z = fmaxf(o.z, 0.f); o.w = fmaxf(o.w, 0.f); }
-                                *reinterpret_cast<float4*>(orow + n) = o;
+                                *reinterpret_cast<float4*>(a.out + row * a.N + n) = o;
+                                if (a.out2) *reinterpret_cast<float4*>(a.out2 + row * a.N + n) = o;
                             }
                         }
                     }
@@ -643,7 +650,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                     const uint32_t q = it * kBlocksPerTile + blk;     // row block counter of this CTA
                     const int slot = q % kPlanSlots;
                     if (grp == 0 && ok && !mbar_wait(&plan_full[slot], (q / kPlanSlots) & 1)) {
-                        if (lane == 0) atomicExch(a.error, 16u);
+                        if (lane == 0) report(a.error, 16u);
                         ok = false;
                     }
                     ok = __all_sync(0xFFFFFFFFu, ok);
@@ -733,7 +740,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                         // commit frees them all); those MMAs ran while the other half was gathered, and the loads
                         // above are already in flight while this waits
                         if (ok && s_h >= 1 && !mbar_wait(&a_free[h], (s_h - 1) & 1)) {
-                            if (lane == 0) atomicExch(a.error, 15u);
+                            if (lane == 0) report(a.error, 15u);
                             ok = false;
                         }
                         ok = __all_sync(0xFFFFFFFFu, ok);
@@ -774,21 +781,36 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
     }
 }
 
-// Pre-pass: for every output row of the layer, where its own representation lives and which
-// entries it aggregates.  One thread per row, full occupancy; the fused kernel then needs a single
-// coalesced load per row instead of a chain of dependent look-ups.
-template <bool FIRST>
-__global__ void __launch_bounds__(256) k_layer_rows(FusedArgs a, int4* __restrict__ row_meta) {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < a.M; r += (int64_t)gridDim.x * blockDim.x) {
-        const int b = upper_segment(a.rowbase_out, a.B + 1, (int32_t)r);
-        const int32_t l = (int32_t)r - a.rowbase_out[b];
+// Pre-pass: for every output row of every layer, where its own representation lives and which entries it aggregates.  One
+// thread per row, full occupancy; the fused kernels then need a single coalesced load per row instead of a chain of dependent
+// look-ups.  One launch for all layers (one mini-batch, three layers: three launches of 2 us and their gaps before).
+struct RowsArgs {
+    int32_t B, k;
+    const int32_t* rowbase;      // [(k + 1)][B + 1]
+    const int32_t* cum;          // [B][k + 2]
+    const int32_t* node_off;     // [(k + 1)][B + 1]
+    const int32_t* nodes;
+    const int32_t* ent_off;
+    FeatGeom feat;
+    int64_t start[MG_MAX_HOPS + 2];   // layer l's rows go to meta[start[l] .. start[l + 1])
+};
+__global__ void __launch_bounds__(256) k_layer_rows(RowsArgs a, int4* __restrict__ meta) {
+    pdl_trigger();
+    const int64_t total = a.start[a.k + 1];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        int layer = 1;
+        while (i >= a.start[layer + 1]) ++layer;
+        const int32_t* rb = a.rowbase + (int64_t)layer * (a.B + 1);
+        const int32_t r = (int32_t)(i - a.start[layer]);
+        const int b = upper_segment(rb, a.B + 1, r);
+        const int32_t l = r - rb[b];
         const int32_t* cum = a.cum + b * (a.k + 2);
         int h = 0;
-        while (h < a.k - a.layer && l >= cum[h + 1]) ++h;
+        while (h < a.k - layer && l >= cum[h + 1]) ++h;
         const int32_t idx = a.node_off[h * (a.B + 1) + b] + (l - cum[h]);
         const int32_t e0 = a.ent_off[idx];
-        const int32_t in_base = FIRST ? 0 : a.rowbase_in[b];
-        row_meta[r] = make_int4(source_row<FIRST>(a, in_base, FIRST ? a.nodes[idx] : l), e0, a.ent_off[idx + 1] - e0, in_base);
+        const int32_t in_base = layer == 1 ? 0 : rb[b - (a.B + 1)];
+        meta[i] = make_int4(layer == 1 ? (int32_t)feat_row(a.feat, a.nodes[idx]) : in_base + l, e0, a.ent_off[idx + 1] - e0, in_base);
     }
 }
 
@@ -876,22 +898,26 @@ static void fill_args(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d
     a.error = ctx->d_flags;
 }
 
-// Pre-pass of one layer: row_meta[r] for every packed output row r of the layer.
-int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, int4* row_meta) {
-    FusedArgs a;
-    memset(&a, 0, sizeof(a));
-    fill_args(ctx, d, layer, d_in, d_out, &a);
-    if (a.M <= 0) return MG_OK;
-    if (layer == 1) k_layer_rows<true><<<mg_grid(ctx, 8), 256, 0, ctx->stream>>>(a, row_meta);
-    else k_layer_rows<false><<<mg_grid(ctx, 8), 256, 0, ctx->stream>>>(a, row_meta);
+// Pre-pass of a forward pass: meta[start[l] + r] for every packed output row r of every layer l = 1 .. k.
+int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int4* meta, const int64_t* start) {
+    RowsArgs a;
+    a.B = d->n_batches; a.k = d->k;
+    a.rowbase = d->rowbase; a.cum = d->cum; a.node_off = d->node_off; a.nodes = d->nodes; a.ent_off = d->ent_off;
+    a.feat = mg_feat_geom(ctx);
+    for (int l = 1; l <= d->k + 1; ++l) a.start[l] = start[l];
+    const int64_t total = start[d->k + 1];
+    if (total <= 0) return MG_OK;
+    k_layer_rows<<<(int)std::min<int64_t>(mg_grid(ctx, 8), (total + 255) / 256), 256, 0, ctx->stream>>>(a, meta);
     ctx->launches++;
     return MG_OK;
 }
 
 // Runs layer `layer` (1-based) for the packed output rows [row_lo, row_hi).  h_prev and h_out are indexed by
-// GLOBAL packed row (callers that keep only a window of a layer pass pointers shifted accordingly).
+// GLOBAL packed row (callers that keep only a window of a layer pass pointers shifted accordingly).  h_out2 (nullable, 16-byte
+// aligned): receives the same rows.  The kernel is launched as a programmatic dependent of the one queued before it, which
+// must be mg_layer_rows' or another layer's.
 int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* w_pad_t, const float* bias,
-                   const float* h_prev, float* h_out, int flags, const int4* row_meta, int64_t row_lo, int64_t row_hi,
+                   const float* h_prev, float* h_out, float* h_out2, int flags, const int4* row_meta, int64_t row_lo, int64_t row_hi,
                    int64_t safe_src_row, const void* w_pad_h, int in_f16, int out_f16) {
     if (row_hi <= row_lo) return MG_OK;
     FusedArgs a;
@@ -907,7 +933,7 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     a.out_f16 = out_f16;
     a.relu = flags & 1;
     a.sum_aggr = (flags >> 1) & 1;
-    a.bias = bias; a.out = h_out;
+    a.bias = bias; a.out = h_out; a.out2 = h_out2;
     // fp16 operands: first layer over fp16 base representations, mean aggregator (a sum of fp16 values may leave the
     // fp16 range), weights given in fp16 form (the caller withholds them when they do not suit fp16)
     // (later layers: in_f16 says that H^{l-1} was stored as fp16; the caller only does that with fp16 weights at hand)
@@ -942,15 +968,29 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     if (!(out_f16 ? (ts ? make_map_f16_box32(&mo, h_out, row_hi, d_out) : make_map_f16(&mo, h_out, row_hi, d_out, 32))
                   : make_map_f32(&mo, h_out, row_hi, d_out, 32)))
         return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the layer output");
+    CUtensorMap mo2 = mo;
+    if (h_out2 && (out_f16 || !make_map_f32(&mo2, h_out2, row_hi, d_out, 32)))
+        return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the layer output");
     const bool first = layer == 1, half = first && ctx->feat_dtype == MG_DTYPE_F16;
-    auto kern = first ? (f16 ? k_sage_layer_fused<true, true, true> : half ? k_sage_layer_fused<true, true, false> : k_sage_layer_fused<true, false, false>)
-                      : (f16 ? k_sage_layer_fused<false, true, true> : k_sage_layer_fused<false, false, false>);
-    if (ts) kern = first ? (f16 ? k_sage_layer_fused<true, true, true, true> : half ? k_sage_layer_fused<true, true, false, true> : k_sage_layer_fused<true, false, false, true>)
-                         : (f16 ? k_sage_layer_fused<false, true, true, true> : k_sage_layer_fused<false, false, false, true>);
-    MG_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    typedef void (*Kernel)(CUtensorMap, CUtensorMap, CUtensorMap, FusedArgs);
+    static const Kernel kernels[2][5] = {
+        {k_sage_layer_fused<true, false, false>, k_sage_layer_fused<true, true, false>, k_sage_layer_fused<true, true, true>,
+         k_sage_layer_fused<false, false, false>, k_sage_layer_fused<false, true, true>},
+        {k_sage_layer_fused<true, false, false, true>, k_sage_layer_fused<true, true, false, true>, k_sage_layer_fused<true, true, true, true>,
+         k_sage_layer_fused<false, false, false, true>, k_sage_layer_fused<false, true, true, true>}};
+    static uint64_t smem_done[2][5] = {};
+    const int which = first ? (f16 ? 2 : half ? 1 : 0) : (f16 ? 4 : 3);
+    const Kernel kern = kernels[ts][which];
+    MG_CUDA(ctx, mg_smem_limit(&smem_done[ts][which], ctx->device, (const void*)kern, 8 * (int)kABytes + 32 * 1024 + 1024));
     const int64_t n_tiles = (row_hi - row_lo + BM - 1) / BM;
     const int grid = 2 * (int)std::min<int64_t>((n_tiles + 1) / 2, ctx->n_sms / 2);   // CTA pairs
-    kern<<<grid, kFusedThreads, smem, ctx->stream>>>(mw, mo, a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kFusedThreads); cfg.dynamicSmemBytes = smem; cfg.stream = ctx->stream;
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &pdl; cfg.numAttrs = 1;
+    MG_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, mw, mo, mo2, a));
     ctx->launches++;
     MG_CUDA(ctx, cudaGetLastError());
     return MG_OK;

@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
             const int buf = j & 1;
             const int n0 = j * ta.bn_max;
             const int bn = min(ta.bn_max, (a.negs - n0 + 15) / 16 * 16);
-            if (!mbar_wait(&acc_full[buf], (j >> 1) & 1)) { if (lane == 0) atomicExch(ta.error, 21u); ok = false; break; }
+            if (!mbar_wait(&acc_full[buf], (j >> 1) & 1)) { if (lane == 0) report(ta.error, 21u); ok = false; break; }
             tc_fence_after();
             for (int c0 = 32 * half; c0 < bn; c0 += 64) {
                 uint32_t v[32];
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
             int issued = 0;
             for (int j = 0; j < n_blocks && ok; ++j) {
                 const int buf = j & 1;
-                if (j >= 2 && !mbar_wait(&b_empty[buf], ((j >> 1) - 1) & 1)) { atomicExch(ta.error, 22u); ok = false; break; }
+                if (j >= 2 && !mbar_wait(&b_empty[buf], ((j >> 1) - 1) & 1)) { report(ta.error, 22u); ok = false; break; }
                 mbar_expect_tx(&b_full[buf], (uint32_t)b_buf_bytes);
                 for (int sl = 0; sl < ta.n_slices; ++sl)
                     bulk_load(b_smem + (size_t)buf * b_buf_bytes + (size_t)sl * b_slice_bytes,
@@ -394,20 +394,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
             }
             // nothing of this CTA's may be in flight when it ends: the last copy into each buffer has landed
             for (int j = max(0, issued - 2); j < issued; ++j)
-                if (!mbar_wait(&b_full[j & 1], (j >> 1) & 1)) atomicExch(ta.error, 26u);
+                if (!mbar_wait(&b_full[j & 1], (j >> 1) & 1)) report(ta.error, 26u);
         }
         __syncwarp();
     } else if (warp == kTcMmaWarp) {
         // ---------------- MMA issue ----------------
         if (lane == 0) {
             bool ok = mbar_wait(&a_full, 0);
-            if (!ok) atomicExch(ta.error, 23u);
+            if (!ok) report(ta.error, 23u);
             for (int j = 0; j < n_blocks && ok; ++j) {
                 const int buf = j & 1;
                 const int n0 = j * ta.bn_max;
                 const int bn = min(ta.bn_max, (a.negs - n0 + 15) / 16 * 16);
-                if (!mbar_wait(&b_full[buf], (j >> 1) & 1)) { atomicExch(ta.error, 24u); ok = false; break; }
-                if (j >= 2 && !mbar_wait(&acc_empty[buf], ((j >> 1) - 1) & 1)) { atomicExch(ta.error, 25u); ok = false; break; }
+                if (!mbar_wait(&b_full[buf], (j >> 1) & 1)) { report(ta.error, 24u); ok = false; break; }
+                if (j >= 2 && !mbar_wait(&acc_empty[buf], ((j >> 1) - 1) & 1)) { report(ta.error, 25u); ok = false; break; }
                 tc_fence_after();
                 const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
                 const uint8_t* bb = b_smem + (size_t)buf * b_buf_bytes;
@@ -488,13 +488,9 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     uint32_t* scan_tmp = (uint32_t*)take(4 * scan_elems);
     uint32_t* d_status = (uint32_t*)take(4);
     int32_t* d_nt = (int32_t*)take(4);
-    if (!ctx->lp_words) {
-        if (cudaHostAlloc((void**)&ctx->lp_words, 2 * sizeof(int32_t), cudaHostAllocMapped) != cudaSuccess ||
-            cudaHostGetDevicePointer((void**)&ctx->lp_words_dev, ctx->lp_words, 0) != cudaSuccess ||
-            cudaMalloc((void**)&ctx->lp_range, 2 * sizeof(int32_t)) != cudaSuccess) {
-            cudaGetLastError(); delete lp;
-            return mg_fail(ctx, MG_ERR_OOM, "allocation of the link-prediction scratch failed");
-        }
+    if (!ctx->lp_range && cudaMalloc((void**)&ctx->lp_range, 2 * sizeof(int32_t)) != cudaSuccess) {
+        cudaGetLastError(); delete lp;
+        return mg_fail(ctx, MG_ERR_OOM, "allocation of the link-prediction scratch failed");
     }
     if (ctx->lp_range_words != n_words) {   // (once per graph)
         const int32_t h_range[2] = {0, (int32_t)n_groups};

@@ -11,6 +11,14 @@ namespace tc {
 
 constexpr long long kWaitCycles = 2000000000ll;  // ~1 s: far beyond any legitimate wait
 
+// records which role gave up waiting: a word in mapped host memory, so that the host reads it without a copy
+__device__ __forceinline__ void report(uint32_t* word, uint32_t role) { *reinterpret_cast<volatile uint32_t*>(word) = role; }
+
+// Programmatic dependent launch: a kernel launched with that attribute may start while the kernel before it in the stream still
+// runs; pdl_wait returns when that kernel has finished and its writes are visible, pdl_trigger lets the next one start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -44,6 +52,12 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(smem_u32(smem_dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y)
         : "memory");
+}
+
+// box in shared memory -> tensor (the caller commits the bulk group)
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* smem_src, int x, int y) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
+                 ::"l"(map), "r"(smem_u32(smem_src)), "r"(x), "r"(y) : "memory");
 }
 
 // untiled bulk copy global -> shared (both 16-byte aligned, size a multiple of 16); completion counts bytes on `bar`
