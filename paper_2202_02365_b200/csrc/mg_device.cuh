@@ -71,17 +71,6 @@ __device__ __forceinline__ int32_t table_insert(int32_t* keys, int32_t table_siz
     return -1;
 }
 
-__device__ __forceinline__ int32_t table_find(const int32_t* keys, int32_t table_size, int32_t id) {
-    uint32_t slot = table_hash(id, table_size);
-    for (int32_t probe = 0; probe < table_size; ++probe) {
-        const int32_t cur = keys[slot];
-        if (cur == id) return (int32_t)slot;
-        if (cur == -1) return -1;
-        slot = slot + 1u == (uint32_t)table_size ? 0u : slot + 1u;
-    }
-    return -1;
-}
-
 // largest j in [0, n) with arr[j] <= x, for a non-decreasing arr with arr[0] <= x
 __device__ __forceinline__ int upper_segment(const int32_t* arr, int n, int32_t x) {
     int lo = 0, hi = n;  // invariant: arr[lo] <= x, (hi == n or arr[hi] > x)

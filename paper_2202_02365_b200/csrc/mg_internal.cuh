@@ -28,7 +28,10 @@ enum : uint32_t {
 // Device-side header of a sample: counters every kernel sizes itself from.
 struct DenseHeader {
     uint32_t status;
-    uint32_t n_new;                       // length of the new-node list of the current hop
+    uint32_t epoch;                       // number of the sample into this handle: tags the states of k_hop's tiles
+    uint64_t targets;                     // device address the targets are read from
+    uint32_t n_new[MG_MAX_HOPS];          // length of each hop's list of new nodes
+    uint32_t ticket[MG_MAX_HOPS];         // k_hop: the next tile of the hop
     int32_t hop_base[MG_MAX_HOPS + 2];    // node arena: hop h occupies [hop_base[h], hop_base[h+1])
     int32_t ent_base[MG_MAX_HOPS + 1];    // entry arena: hop h occupies [ent_base[h], ent_base[h+1])
     int32_t rows_total[MG_MAX_HOPS + 1];  // rows of H^l summed over batches, l = 0..k
@@ -171,7 +174,7 @@ struct mg_ctx {
 // everything the sampler's captured device work depends on
 struct SampleSignature {
     int32_t B, k, table_size, fanouts[MG_MAX_HOPS];
-    int64_t T, cap_batch, cap_nodes, cap_entries, n_nodes, part_size, inout;
+    int64_t T_bound, cap_batch, cap_nodes, cap_entries, n_nodes, part_size, inout;
     const void* ptrs[32];
 };
 
@@ -189,11 +192,8 @@ struct mg_dense {
     int32_t* nodes = nullptr;       // [cap_nodes] hop-major, batch-major inside a hop
     int32_t* node_batch = nullptr;  // [cap_nodes]
     int32_t* ent_off = nullptr;     // [cap_nodes + 1] start of each sampled node's entries
-    int64_t* node_r0 = nullptr;     // [cap_nodes] start of the node's row in the in-buffer view
-    uint32_t* node_deg = nullptr;   // [cap_nodes] its (resident) degree
-    int64_t* node_r0_out = nullptr; // the same for the outgoing edge list (incoming + outgoing sampling only)
-    uint32_t* node_deg_out = nullptr;
-    int64_t cap_nodes_out = 0;
+    uint64_t* tile_state = nullptr; // k_hop: running entry counts of the tiles, tagged with (epoch, hop)
+    uint32_t epoch = 0;
     int2* pairs = nullptr;          // last hop, shared-memory deduplication: (id, entry) grouped by (batch, share, bucket)
     int32_t* share_off = nullptr;   // its group bounds
     int64_t cap_pairs = 0, cap_share = 0;
@@ -236,9 +236,8 @@ struct mg_dense {
     int perm_batch = -1;
     uint32_t* batch_cnt = nullptr;   // [k][B] new nodes per hop and mini-batch
     // asynchronous sampling: the summary lands in pinned memory, ev_sampled marks its arrival
-    int32_t* h_pinned = nullptr; size_t h_pinned_ints = 0;
-    int32_t* h_pinned_dev = nullptr; // the same memory as the device sees it
-    int32_t* h_stage = nullptr; size_t h_stage_ints = 0;   // pinned, mapped: header, offsets, seeds of the call being queued
+    // one mapped pinned block: header, offsets, seeds and a few targets of the call being queued, then the summary
+    int32_t* h_stage = nullptr; size_t h_stage_ints = 0, h_summary_at = 0;
     int32_t* h_stage_dev = nullptr;                        // the same memory as the device sees it
     cudaGraphExec_t graph_exec = nullptr;                 // the sampler's device work for graph_sig
     SampleSignature graph_sig;

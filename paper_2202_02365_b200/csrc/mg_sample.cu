@@ -24,6 +24,7 @@
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int64_t kStageTargets = 16384;   // targets in host memory that travel in the staging block of a sample
 
 // -------------------------------------------------------------------------------------
 // generic exclusive scan over a device-sized range (three kernels, no inter-block waits)
@@ -70,16 +71,8 @@ __global__ void __launch_bounds__(kThreads) k_scan_reduce(const uint32_t* data, 
     }
 }
 
-// what the scan of a hop's entry counts also does once the total is known: close the hop's entry range, check the arena
-struct HopClose {
-    DenseHeader* hdr;      // null: a plain scan
-    int hop;
-    int32_t* ent_off;
-    int64_t cap_entries;
-};
-
 // single block: exclusive scan of the tile sums in place; total (plus base) to *total_out
-__global__ void __launch_bounds__(1024) k_scan_tiles(uint32_t* tile_sums, ScanRange r, uint32_t* total_out, HopClose hc) {
+__global__ void __launch_bounds__(1024) k_scan_tiles(uint32_t* tile_sums, ScanRange r, uint32_t* total_out) {
     __shared__ uint32_t warp_tot[33];
     const int n = *r.hi - *r.lo;
     const int ntiles = (n + kScanTile - 1) / kScanTile;
@@ -102,18 +95,7 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(uint32_t* tile_sums, ScanRa
         carry += warp_tot[32];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        const uint32_t end = carry + (r.base ? (uint32_t)*r.base : 0u);
-        if (total_out) *total_out = end;
-        if (hc.hdr && !hc.hdr->status) {
-            if ((int64_t)end > hc.cap_entries) atomicOr(&hc.hdr->status, ST_CAP_ENTRIES);
-            else {
-                hc.hdr->ent_base[hc.hop + 1] = (int32_t)end;
-                hc.ent_off[hc.hdr->hop_base[hc.hop + 1]] = (int32_t)end;   // (past the range the scan's last kernel writes)
-                hc.hdr->n_new = 0;
-            }
-        }
-    }
+    if (threadIdx.x == 0 && total_out) *total_out = carry + (r.base ? (uint32_t)*r.base : 0u);
 }
 
 __global__ void __launch_bounds__(kThreads) k_scan_down(uint32_t* data, ScanRange r, const uint32_t* tile_sums) {
@@ -140,244 +122,356 @@ __global__ void __launch_bounds__(kThreads) k_scan_down(uint32_t* data, ScanRang
 }
 
 // -------------------------------------------------------------------------------------
-// hop 0: targets
+// begin of a sample
 // -------------------------------------------------------------------------------------
 struct TableGeom {
-    int32_t size;   // slots per batch (any size)
+    int32_t size;   // slots per batch (a multiple of 8)
 };
 
 // The host-known part of a sample (header, target offsets, per-batch row tables, seeds) is read straight from mapped
 // pinned memory by a kernel instead of being copied by a copy engine: a copy engine may be busy for a long time with
-// a partition that is being swapped in, and the sample would wait behind it.
-__global__ void __launch_bounds__(kThreads)
-k_stage_in(const int32_t* __restrict__ stage, int32_t n_hdr, int32_t n_off, int32_t n_cum, int32_t n_seed_words, int32_t seed_at,
-           int32_t* hdr, int32_t* node_off, int32_t* cum, int32_t* seeds) {
-    const int32_t total = n_hdr + n_off + n_cum + n_seed_words;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        int32_t j = i;
-        if (j < n_hdr) hdr[j] = stage[j];
-        else if ((j -= n_hdr) < n_off) node_off[j] = stage[n_hdr + j];
-        else if ((j -= n_off) < n_cum) cum[j] = stage[n_hdr + n_off + j];
-        else seeds[j - n_cum] = stage[seed_at + (j - n_cum)];
+// a partition that is being swapped in, and the sample would wait behind it.  The same kernel clears the id tables and the
+// counters: a memset node in the captured graph held the kernels behind it up by 10 to 14 us.
+struct BeginArgs {
+    const int32_t* stage;
+    int32_t n_hdr, n_off, n_cum, n_seed_words, seed_at, n_cnt;
+    int64_t n_table4;   // 16-byte pieces of the id tables
+    int32_t *hdr, *node_off, *cum, *seeds, *batch_cnt;
+    int4* hkeys;
+};
+__global__ void __launch_bounds__(kThreads) k_begin(BeginArgs a) {
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    const int32_t total = a.n_hdr + a.n_off + a.n_cum + a.n_seed_words;
+    for (int64_t i = tid; i < total; i += step) {
+        int32_t j = (int32_t)i;
+        if (j < a.n_hdr) a.hdr[j] = a.stage[j];
+        else if ((j -= a.n_hdr) < a.n_off) a.node_off[j] = a.stage[a.n_hdr + j];
+        else if ((j -= a.n_off) < a.n_cum) a.cum[j] = a.stage[a.n_hdr + a.n_off + j];
+        else a.seeds[j - a.n_cum] = a.stage[a.seed_at + (j - a.n_cum)];
     }
-}
-
-__global__ void __launch_bounds__(kThreads) k_copy_i32(const int32_t* __restrict__ src, int32_t* dst, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) dst[i] = src[i];
-}
-
-__global__ void __launch_bounds__(kThreads)
-k_init_targets(DenseHeader* hdr, const int32_t* __restrict__ targets,
-               const int32_t* __restrict__ tgt_off, int32_t B, int32_t* nodes, int32_t* node_batch,
-               int32_t* hkeys, int32_t* hvals, TableGeom tg, int64_t n_nodes, FeatGeom feat) {
-    const int32_t n_total = hdr->hop_base[1];   // read on the device: the launch does not depend on the number of targets
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_total; i += gridDim.x * blockDim.x) {
-        const int b = upper_segment(tgt_off, B + 1, i);
-        const int32_t v = targets[i];
-        nodes[i] = v;
-        node_batch[i] = b;
-        if (v < 0 || (int64_t)v >= n_nodes) { atomicOr(&hdr->status, ST_RANGE); continue; }
-        if (!feat_resident(feat, v)) { atomicOr(&hdr->status, ST_NONRESIDENT); continue; }
-        bool is_new;
-        const int32_t slot = table_insert(hkeys + (int64_t)b * tg.size, tg.size, v, &is_new);
-        if (slot < 0) { atomicOr(&hdr->status, ST_CAP_TABLE); continue; }
-        if (!is_new) { atomicOr(&hdr->status, ST_DUPLICATE); continue; }
-        hvals[(int64_t)b * tg.size + slot] = i - tgt_off[b];
-    }
+    for (int64_t i = tid; i < a.n_cnt; i += step) a.batch_cnt[i] = 0;
+    for (int64_t i = tid; i < a.n_table4; i += step) a.hkeys[i] = make_int4(-1, -1, -1, -1);
 }
 
 // -------------------------------------------------------------------------------------
-// per hop: degree -> count, (scan), pick + id-table insert, (sort), place, relabel
+// per hop: count, scan and pick in one kernel
 // -------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads)
-k_count(const DenseHeader* hdr, int hop, int32_t fanout, const int32_t* __restrict__ nodes,
-        const int64_t* __restrict__ row_off, int32_t* ent_off, int64_t* node_r0, uint32_t* node_deg,
-        const int64_t* __restrict__ row_off_out, int64_t* node_r0_out, uint32_t* node_deg_out) {
-    if (hdr->status) return;
-    const int32_t lo = hdr->hop_base[hop], hi = hdr->hop_base[hop + 1];
-    for (int32_t i = lo + blockIdx.x * blockDim.x + threadIdx.x; i < hi; i += gridDim.x * blockDim.x) {
-        const int32_t v = nodes[i];
-        const int64_t r0 = row_off[v];
-        const int64_t d = row_off[v + 1] - r0;
-        int32_t n = (int32_t)(d < (int64_t)fanout ? d : (int64_t)fanout);
-        node_r0[i] = r0;        // the one random look-up of the row bounds; k_pick reads these coalesced
-        node_deg[i] = (uint32_t)d;
-        if (row_off_out) {      // incoming + outgoing sampling: up to `fanout` of each list
-            const int64_t q0 = row_off_out[v];
-            const int64_t dq = row_off_out[v + 1] - q0;
-            n += (int32_t)(dq < (int64_t)fanout ? dq : (int64_t)fanout);
-            node_r0_out[i] = q0;
-            node_deg_out[i] = (uint32_t)dq;
-        }
-        ent_off[i] = n;
-    }
-}
-
-struct PickArgs {
+// Bound by the latency of random look-ups (a node's row bounds, then one DRAM burst per picked id) and, for small hops, by
+// launches: one thread per node reads the row bounds, the tile's entry counts are scanned in the block, the tiles' running
+// totals are chained through one 64-bit word per tile (decoupled look-back), and the block's warps then pick for the tile's
+// nodes from shared memory.  Before, these were five kernels with the row bounds, degrees and counts going through memory
+// between them (one mini-batch of three hops on 1M nodes: 48 -> 32 us; 128 mini-batches, last hop of 2.7M nodes: 315 -> 288
+// us).  A tile has as few nodes as keeps five blocks per SM busy (hop_tile): the picks of a warp's nodes are one chain after
+// the other, and a hop of 1,000 nodes took 21 us with 256 of them per block, 10 us with 32.  Tiles are handed out by a
+// counter, so a tile's predecessors are always held by running blocks and every wait ends; the polls are bounded all the same.
+// Hop 0 also enters the targets: residency and range checks, the id table (Algorithm 1 wants unique targets).
+struct HopArgs {
     DenseHeader* hdr;
     int hop;
     int32_t fanout;
-    const int32_t* nodes;
-    const int32_t* node_batch;
-    const int64_t* node_r0;
-    const uint32_t* node_deg;
-    const int32_t* row_nbrs;
-    const int32_t* ent_off;
+    int32_t* nodes;
+    int32_t* node_batch;
+    const int64_t* row_off[2];    // [1] null: one direction; else the outgoing list, whose picks follow the first list's
+    const int32_t* row_nbrs[2];
+    int32_t* ent_off;
     int32_t* ent_nbrs;
-    int32_t* ent_repr;  // receives the batch id of the entry (k_insert turns it into the id-table slot)
+    int32_t* ent_repr;            // receives the batch id of the entry (k_insert turns it into the id-table slot)
     const uint64_t* seeds;
-    // second direction of incoming + outgoing sampling: its picks follow the first direction's min(degree, fanout)
-    // entries of the node and its draws use slots slot_base + t
-    const uint32_t* pre_deg;   // nullptr for the first (or only) direction
-    uint32_t slot_base;
+    int64_t cap_entries;
+    uint64_t* tile_state;
+    int32_t tile_cap;             // nodes of a tile that the launch has shared memory for
+    // hop 0
+    int32_t B;
+    const int32_t* tgt_off;
+    int32_t* hkeys;
+    int32_t* hvals;
+    TableGeom tg;
+    int64_t n_nodes;
+    FeatGeom feat;
 };
 
-// first entry of node i's picks in this launch's direction
-__device__ __forceinline__ int32_t pick_base(const PickArgs& a, int32_t i) {
-    int32_t out0 = a.ent_off[i];
-    if (a.pre_deg) {
-        const uint32_t d0 = a.pre_deg[i];
-        out0 += (int32_t)(d0 < (uint32_t)a.fanout ? d0 : (uint32_t)a.fanout);
-    }
-    return out0;
+constexpr uint64_t kTileSum = 1ull << 32, kTileTotal = 2ull << 32;   // a tile's own count / the running total behind it
+// Nodes of a tile.  Below 256 as few as give five blocks (what the registers allow) on each of 148 SMs a tile; above 256
+// where twelve tiles per SM are left all the same: the chain through the tiles costs about 13 ns each (2.7M nodes: 620 us with
+// tiles of 64, 475 with 128, 342 with 256, 288 with 1,024).
+constexpr int kTilesWanted = 740, kTilesLarge = 1776, kTileMax = 1024, kTileSets = kTileMax / kThreads;
+constexpr int kTileParts = kTileSets * kThreads / 32;
+static_assert(kTileParts <= 32, "one warp scans the tile's warp totals");
+__host__ __device__ __forceinline__ int hop_tile(int64_t n) {
+    for (int t = 32; t < kThreads; t <<= 1)
+        if (n <= (int64_t)t * kTilesWanted) return t;
+    for (int t = kTileMax; t > kThreads; t >>= 1)
+        if (n > (int64_t)t * kTilesLarge) return t;
+    return kThreads;
 }
+// shared memory per node of a tile: id, mini-batch, first entry; first edge and length of its row, once per direction
+__host__ __device__ __forceinline__ int hop_node_bytes(bool inout) { return 12 + (inout ? 24 : 12); }
+constexpr int kTilePolls = 1 << 20;   // (a poll is an L2 round trip: far beyond any legitimate wait)
 
-// A pick goes to its place in the entry arena; ent_repr carries the batch id until k_insert replaces it.
-__device__ __forceinline__ void store_pick(const PickArgs& a, bool valid, int32_t b, int32_t u, int32_t out_pos) {
-    if (!valid) return;
-    a.ent_nbrs[out_pos] = u;
-    a.ent_repr[out_pos] = b;
-}
-
-// G lanes per node, fanout <= G <= 32; a warp holds 32 / G nodes (G need not divide 32: the lanes left over idle, and
-// G = 5 or 10 keeps 30 lanes busy where the next power of two keeps 20).
-template <int G>
-__global__ void __launch_bounds__(kThreads) k_pick(PickArgs a) {
-    if (a.hdr->status) return;
-    constexpr int kPerWarp = 32 / G;
-    constexpr int kGroups = (kThreads / 32) * kPerWarp;
-    const int32_t lo = a.hdr->hop_base[a.hop], hi = a.hdr->hop_base[a.hop + 1];
+// the mini-batch of target i: a 32-way search of the warp for its first target, then a walk
+__device__ __forceinline__ int target_batch(const int32_t* __restrict__ off, int B, int32_t first, int32_t i) {
     const int lane = threadIdx.x & 31;
-    const int grp = lane / G;                     // group inside the warp (== kPerWarp: a left-over lane)
-    const int gl = lane - grp * G;                // lane inside the group
-    const int gshift = grp * G;                   // first warp lane of the group
-    const uint32_t gmask = (G == 32) ? 0xFFFFFFFFu : (((1u << G) - 1u) << gshift);
-    const int32_t f = a.fanout;
-    for (int32_t base = lo + blockIdx.x * kGroups; base < hi; base += gridDim.x * kGroups) {
-        const int32_t i = base + (threadIdx.x >> 5) * kPerWarp + grp;
-        const bool node_ok = grp < kPerWarp && i < hi;
-        int32_t v = 0, b = 0, out0 = 0;
-        int64_t r0 = 0, d = 0;
-        if (node_ok) {
-            v = a.nodes[i];
-            b = a.node_batch[i];
-            out0 = pick_base(a, i);
-            r0 = a.node_r0[i];
-            d = (int64_t)a.node_deg[i];
-        }
-        bool valid = false;
-        int32_t u = 0, pos = 0;
-        const bool floyd = node_ok && d > (int64_t)f;
-        // Floyd's subset algorithm: slot t draws x in [0, d-f+t]; it keeps x unless an earlier slot
-        // already holds x, in which case it keeps d-f+t.  Draws are independent of each other, so
-        // all lanes draw at once and only the "already held" test runs slot by slot.
-        uint32_t x = 0xFFFFFFFFu, jt = 0, pick = 0xFFFFFFFFu;
-        if (floyd && gl < f) {
-            jt = (uint32_t)(d - f) + (uint32_t)gl;
-            x = __umulhi(draw_word(a.seeds[b], (uint32_t)v, (uint32_t)a.hop, a.slot_base + (uint32_t)gl), jt + 1u);
-        }
+    int lo = 0, len = B;   // off[lo] <= first, the answer lies in [lo, lo + len)
+    while (len > 1) {
+        const int step = (len + 31) / 32;
+        const uint32_t below = __ballot_sync(0xFFFFFFFFu, lane * step < len && off[lo + min(lane * step, len - 1)] <= first);   // lane 0 always
+        const int last = 31 - __clz(below);
+        lo += last * step;
+        len = min(step, len - last * step);
+    }
+    while (off[lo + 1] <= i) ++lo;
+    return lo;
+}
+
+// Floyd's subset algorithm, G lanes per node: slot t draws x in [0, d-f+t]; it keeps x unless an earlier slot already holds
+// x, in which case it keeps d-f+t.  Draws are independent of each other, so all lanes draw at once and only the "already
+// held" test runs slot by slot.  It is left out when no two draws of a node are alike: slot 0 keeps its draw, and so does
+// every later slot, as the earlier ones hold nothing but their own.  Returns the lane's position in the row, *rank its rank
+// among the f picks.
+template <int G>
+__device__ __forceinline__ uint32_t floyd_pick(bool on, uint32_t d, int32_t f, int gl, int gshift, uint64_t seed, uint32_t v, uint32_t hop,
+                                               uint32_t slot_base, int* rank) {
+    const uint32_t gmask = (G == 32) ? 0xFFFFFFFFu : (((1u << (G & 31)) - 1u) << gshift);
+    uint32_t x = 0xFFFFFFFFu, jt = 0, pick = 0xFFFFFFFFu;
+    if (on && gl < f) {
+        jt = d - (uint32_t)f + (uint32_t)gl;
+        x = __umulhi(draw_word(seed, v, hop, slot_base + (uint32_t)gl), jt + 1u);
+    }
+    const uint32_t same = __match_any_sync(0xFFFFFFFFu, x) & gmask;
+    if (!__any_sync(0xFFFFFFFFu, on && gl < f && same != 1u << (threadIdx.x & 31))) pick = x;
+    else
         for (int t = 0; t < f; ++t) {
             const uint32_t xt = __shfl_sync(0xFFFFFFFFu, x, gshift + t);
             const uint32_t hit = __ballot_sync(0xFFFFFFFFu, gl < t && pick == xt) & gmask;
             if (gl == t) pick = hit ? jt : xt;
         }
-        // rank of this lane's position among the f picks (they are distinct); every lane of the warp
-        // takes part in the shuffles, whatever its node needs
-        int rank = 0;
-        for (int t = 0; t < f; ++t) {
-            const uint32_t pt = __shfl_sync(0xFFFFFFFFu, pick, gshift + t);
-            rank += (pt < pick) ? 1 : 0;
-        }
-        if (floyd) {
-            if (gl < f) {
-                valid = true;
-                u = a.row_nbrs[r0 + (int64_t)pick];
-                pos = out0 + rank;
-            }
-        } else if (node_ok && (int64_t)gl < d) {
-            valid = true;
-            u = a.row_nbrs[r0 + gl];
-            pos = out0 + gl;
-        }
-        store_pick(a, valid, b, u, pos);
+    // (the f picks are distinct; every lane of the warp takes part in the shuffles, whatever its node needs)
+    int r = 0;
+    for (int t = 0; t < f; ++t) {
+        const uint32_t pt = __shfl_sync(0xFFFFFFFFu, pick, gshift + t);
+        r += (pt < pick) ? 1 : 0;
     }
+    *rank = r;
+    return pick;
 }
 
-// Any fanout up to MG_MAX_FANOUT: one warp per node, picks staged in shared memory.
-__global__ void __launch_bounds__(kThreads) k_pick_wide(PickArgs a) {
-    extern __shared__ uint32_t sm_dyn[];  // per warp: x[f], pick[f]
-    if (a.hdr->status) return;
-    constexpr int kWarps = kThreads / 32;
-    const int32_t lo = a.hdr->hop_base[a.hop], hi = a.hdr->hop_base[a.hop + 1];
+// G lanes per node, fanout <= G <= 32; a warp holds 32 / G nodes (G need not divide 32: the lanes left over idle, and
+// G = 5 or 10 keeps 30 lanes busy where the next power of two keeps 20).  G = 0: any fanout up to MG_MAX_FANOUT, a node per
+// warp at a time, picks staged in shared memory.
+template <int G>
+__global__ void __launch_bounds__(kThreads) k_hop(HopArgs a) {
+    extern __shared__ __align__(16) uint8_t hop_sm[];   // the tile's nodes, then (G = 0) per warp x[f], pick[f]
+    __shared__ uint32_t part[kTileParts];
+    __shared__ int32_t sh_tile;
+    __shared__ uint32_t sh_before, sh_end;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t f = a.fanout;
-    uint32_t* xs = sm_dyn + (size_t)warp * 2 * f;
-    uint32_t* picks = xs + f;
-    const int rounds = (f + 31) / 32;
-    for (int32_t base = lo + blockIdx.x * kWarps; base < hi; base += gridDim.x * kWarps) {
-        const int32_t i = base + warp;
-        const bool node_ok = i < hi;
-        int32_t v = 0, b = 0, out0 = 0;
-        int64_t r0 = 0, d = 0;
-        if (node_ok) {
-            v = a.nodes[i];
-            b = a.node_batch[i];
-            out0 = pick_base(a, i);
-            r0 = a.node_r0[i];
-            d = (int64_t)a.node_deg[i];
-        }
-        const bool floyd = node_ok && d > (int64_t)f;
-        if (floyd) {
-            for (int t = lane; t < f; t += 32) {
-                const uint32_t jt = (uint32_t)(d - f) + (uint32_t)t;
-                xs[t] = __umulhi(draw_word(a.seeds[b], (uint32_t)v, (uint32_t)a.hop, a.slot_base + (uint32_t)t), jt + 1u);
+    const bool inout = a.row_off[1] != nullptr;
+    const int32_t lo = a.hdr->hop_base[a.hop], n = a.hdr->hop_base[a.hop + 1] - lo;
+    // (an empty hop has one empty tile: it closes the entry range)
+    const int32_t tile_nodes = min(hop_tile(n), a.tile_cap), n_tiles = max(1, (n + tile_nodes - 1) / tile_nodes);
+    const int sets = (tile_nodes + kThreads - 1) / kThreads;   // nodes per thread
+    int64_t* node_r0 = reinterpret_cast<int64_t*>(hop_sm);                                      // [dirs][tile_cap]
+    uint32_t* node_deg = reinterpret_cast<uint32_t*>(node_r0 + (inout ? 2 : 1) * a.tile_cap);   // [dirs][tile_cap]
+    int32_t* node_id = reinterpret_cast<int32_t*>(node_deg + (inout ? 2 : 1) * a.tile_cap);
+    int32_t* node_b = node_id + a.tile_cap;
+    uint32_t* node_out = reinterpret_cast<uint32_t*>(node_b + a.tile_cap);
+    const uint64_t tag = (((uint64_t)a.hdr->epoch << 3) | (uint64_t)a.hop) << 34;
+    const int32_t* __restrict__ targets = reinterpret_cast<const int32_t*>(a.hdr->targets);
+    for (;;) {
+        __syncthreads();
+        // (after an error no block takes another tile; one that was taken is always closed)
+        if (threadIdx.x == 0) sh_tile = *reinterpret_cast<volatile uint32_t*>(&a.hdr->status) ? INT32_MAX : (int32_t)atomicAdd(&a.hdr->ticket[a.hop], 1u);
+        __syncthreads();
+        const int32_t tile = sh_tile;
+        if (tile >= n_tiles) break;
+        const int32_t n_here = min(tile_nodes, n - tile * tile_nodes);
+        // node t = q * 256 + thread of the tile
+        uint32_t inc[kTileSets];
+#pragma unroll
+        for (int q = 0; q < kTileSets; ++q) {
+            if (q >= sets) break;
+            const int32_t t = q * kThreads + (int32_t)threadIdx.x, local = tile * tile_nodes + t;
+            const bool node_ok = t < n_here;
+            int32_t v = 0, b = 0;
+            bool in_range = node_ok;
+            if (node_ok) {
+                v = a.hop == 0 ? targets[local] : a.nodes[lo + local];
+                if (a.hop > 0) b = a.node_batch[lo + local];
             }
-            __syncwarp();
-            for (int t = 0; t < f; ++t) {
-                const uint32_t xt = xs[t];
-                bool hit = false;
-                for (int s = lane; s < t; s += 32) hit |= (picks[s] == xt);
-                const bool any = __any_sync(0xFFFFFFFFu, hit);
-                if (lane == 0) picks[t] = any ? ((uint32_t)(d - f) + (uint32_t)t) : xt;
-                __syncwarp();
+            if (a.hop == 0) {
+                if (t - lane < n_here) b = target_batch(a.tgt_off, a.B, local - lane, min(local, n - 1));
+                in_range = node_ok && v >= 0 && (int64_t)v < a.n_nodes;
+            }
+            uint32_t cnt = 0;
+            if (in_range) {
+                const int64_t r0 = a.row_off[0][v];
+                const uint32_t d = (uint32_t)(a.row_off[0][v + 1] - r0);
+                cnt = min(d, (uint32_t)f);
+                node_r0[t] = r0;
+                node_deg[t] = d;
+                if (inout) {   // incoming + outgoing sampling: up to `fanout` of each list
+                    const int64_t q0 = a.row_off[1][v];
+                    const uint32_t dq = (uint32_t)(a.row_off[1][v + 1] - q0);
+                    cnt += min(dq, (uint32_t)f);
+                    node_r0[a.tile_cap + t] = q0;
+                    node_deg[a.tile_cap + t] = dq;
+                }
+            } else if (node_ok) {
+                node_r0[t] = 0; node_deg[t] = 0;
+                if (inout) { node_r0[a.tile_cap + t] = 0; node_deg[a.tile_cap + t] = 0; }
+            }
+            if (node_ok) { node_id[t] = v; node_b[t] = b; node_out[t] = cnt; }
+            inc[q] = warp_incl_scan(cnt);
+            if (lane == 31) part[q * (kThreads / 32) + warp] = inc[q];
+        }
+        __syncthreads();
+        // entries before each warp's nodes inside the tile, the tile's count; the tiles before this one
+        if (warp == 0) {
+            const uint32_t w = lane < sets * (kThreads / 32) ? part[lane] : 0u;
+            const uint32_t wi = warp_incl_scan(w);
+            const uint32_t total = __shfl_sync(0xFFFFFFFFu, wi, 31);
+            if (lane < kTileParts) part[lane] = wi - w;
+            volatile uint64_t* state = a.tile_state;
+            uint32_t before = (uint32_t)a.hdr->ent_base[a.hop];
+            if (tile > 0) {
+                if (lane == 0) state[tile] = tag | kTileSum | total;
+                // look back over windows of 32 tiles until one carries a running total
+                before = 0;
+                for (int32_t top = tile - 1; top >= 0; top -= 32) {
+                    const int32_t at = top - lane;
+                    uint64_t s = tag | kTileSum;   // (before tile 0: nothing)
+                    if (at >= 0) {
+                        int polls = 0;
+                        while (((s = state[at]) >> 34 != tag >> 34) && ++polls < kTilePolls) {}
+                        if (polls >= kTilePolls) { atomicOr(&a.hdr->status, ST_INTERNAL); s = tag | kTileTotal; }
+                    }
+                    const uint32_t full = __ballot_sync(0xFFFFFFFFu, (s & kTileTotal) != 0);
+                    const int stop = full ? __ffs(full) - 1 : 31;
+                    before += __reduce_add_sync(0xFFFFFFFFu, lane <= stop ? (uint32_t)s : 0u);
+                    if (full) break;
+                }
+            }
+            if (lane == 0) {
+                const uint32_t end = before + total;
+                state[tile] = tag | kTileTotal | end;
+                sh_before = before;
+                sh_end = end;
+                if ((int64_t)end > a.cap_entries) atomicOr(&a.hdr->status, ST_CAP_ENTRIES);
+                else if (tile == n_tiles - 1) {
+                    a.hdr->ent_base[a.hop + 1] = (int32_t)end;
+                    a.ent_off[lo + n] = (int32_t)end;   // (past the hop's own nodes: the sentinel)
+                }
             }
         }
-        for (int rd = 0; rd < rounds; ++rd) {
-            const int t = rd * 32 + lane;
-            bool valid = false;
-            int32_t u = 0, pos = 0;
-            if (floyd && t < f) {
-                const uint32_t p = picks[t];
-                int rank = 0;
-                for (int s = 0; s < f; ++s) rank += (picks[s] < p) ? 1 : 0;
-                valid = true;
-                u = a.row_nbrs[r0 + (int64_t)p];
-                pos = out0 + rank;
-            } else if (node_ok && !floyd && (int64_t)t < d) {
-                valid = true;
-                u = a.row_nbrs[r0 + t];
-                pos = out0 + t;
+        __syncthreads();
+        const bool fits = (int64_t)sh_end <= a.cap_entries;
+#pragma unroll
+        for (int q = 0; q < kTileSets; ++q) {
+            const int32_t t = q * kThreads + (int32_t)threadIdx.x, local = tile * tile_nodes + t;
+            if (q >= sets || t >= n_here) break;
+            const uint32_t out0 = sh_before + part[q * (kThreads / 32) + warp] + inc[q] - node_out[t];
+            node_out[t] = out0;
+            a.ent_off[lo + local] = (int32_t)out0;
+            if (a.hop == 0) {
+                const int32_t v = node_id[t], b = node_b[t];
+                a.nodes[local] = v;
+                a.node_batch[local] = b;
+                if (v < 0 || (int64_t)v >= a.n_nodes) atomicOr(&a.hdr->status, ST_RANGE);
+                else if (!feat_resident(a.feat, v)) atomicOr(&a.hdr->status, ST_NONRESIDENT);
+                else {
+                    bool is_new;
+                    const int32_t slot = table_insert(a.hkeys + (int64_t)b * a.tg.size, a.tg.size, v, &is_new);
+                    if (slot < 0) atomicOr(&a.hdr->status, ST_CAP_TABLE);
+                    else if (!is_new) atomicOr(&a.hdr->status, ST_DUPLICATE);
+                    else a.hvals[(int64_t)b * a.tg.size + slot] = local - a.tgt_off[b];
+                }
             }
-            store_pick(a, valid, b, u, pos);
         }
-        __syncwarp();
+        if (!fits) break;   // (uniform over the block)
+        __syncthreads();
+        // the picks: warp after warp takes nodes of the tile
+        for (int dir = 0; dir < (inout ? 2 : 1); ++dir) {
+            const int32_t* __restrict__ row_nbrs = a.row_nbrs[dir];
+            const uint32_t slot_base = dir ? (uint32_t)MG_OUT_SLOT_BASE : 0u;
+            const int64_t* dir_r0 = node_r0 + dir * a.tile_cap;
+            const uint32_t* dir_deg = node_deg + dir * a.tile_cap;
+            if (G > 0) {
+                constexpr int GG = G > 0 ? G : 1, kPerWarp = 32 / GG;
+                const int grp = lane / GG;                // group inside the warp (== kPerWarp: a left-over lane)
+                const int gl = lane - grp * GG;           // lane inside the group
+                for (int s = warp * kPerWarp; s < n_here; s += (kThreads / 32) * kPerWarp) {
+                    const bool on = grp < kPerWarp && s + grp < n_here;
+                    const int at = min(s + grp, n_here - 1);
+                    const int32_t gb = node_b[at];
+                    const int64_t gr0 = dir_r0[at];
+                    const uint32_t gd = on ? dir_deg[at] : 0u;
+                    // (the second direction's picks follow the first's)
+                    const uint32_t g0 = node_out[at] + (dir ? min(node_deg[at], (uint32_t)f) : 0u);
+                    const bool floyd = gd > (uint32_t)f;
+                    uint32_t p = (uint32_t)gl;            // all neighbours, in row order
+                    int rank = gl;
+                    if (__any_sync(0xFFFFFFFFu, floyd)) {
+                        int r;
+                        const uint32_t fp = floyd_pick<GG>(floyd, gd, f, gl, grp * GG, floyd ? a.seeds[gb] : 0ull, (uint32_t)node_id[at],
+                                                           (uint32_t)a.hop, slot_base, &r);
+                        if (floyd) { p = fp; rank = r; }
+                    }
+                    if (floyd ? gl < f : (uint32_t)gl < gd) {
+                        a.ent_nbrs[g0 + rank] = row_nbrs[gr0 + (int64_t)p];
+                        a.ent_repr[g0 + rank] = gb;
+                    }
+                }
+            } else {
+                uint32_t* xs = reinterpret_cast<uint32_t*>(node_out + a.tile_cap) + (size_t)warp * 2 * f;
+                uint32_t* picks = xs + f;
+                for (int s = warp; s < n_here; s += kThreads / 32) {
+                    const uint32_t gv = (uint32_t)node_id[s];
+                    const int32_t gb = node_b[s];
+                    const int64_t gr0 = dir_r0[s];
+                    const uint32_t gd = dir_deg[s];
+                    const uint32_t g0 = node_out[s] + (dir ? min(node_deg[s], (uint32_t)f) : 0u);
+                    const bool floyd = gd > (uint32_t)f;   // (uniform over the warp)
+                    if (floyd) {
+                        for (int t = lane; t < f; t += 32) {
+                            const uint32_t jt = gd - (uint32_t)f + (uint32_t)t;
+                            xs[t] = __umulhi(draw_word(a.seeds[gb], gv, (uint32_t)a.hop, slot_base + (uint32_t)t), jt + 1u);
+                        }
+                        __syncwarp();
+                        for (int t = 0; t < f; ++t) {
+                            const uint32_t xt = xs[t];
+                            bool hit = false;
+                            for (int q = lane; q < t; q += 32) hit |= (picks[q] == xt);
+                            const bool any = __any_sync(0xFFFFFFFFu, hit);
+                            if (lane == 0) picks[t] = any ? (gd - (uint32_t)f + (uint32_t)t) : xt;
+                            __syncwarp();
+                        }
+                    }
+                    const int32_t take = (int32_t)min(gd, (uint32_t)f);
+                    for (int t = lane; t < take; t += 32) {
+                        uint32_t p = (uint32_t)t;
+                        int rank = t;
+                        if (floyd) {
+                            p = picks[t];
+                            rank = 0;
+                            for (int q = 0; q < f; ++q) rank += (picks[q] < p) ? 1 : 0;
+                        }
+                        a.ent_nbrs[g0 + rank] = row_nbrs[gr0 + (int64_t)p];
+                        a.ent_repr[g0 + rank] = gb;
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        if (n_tiles <= (int32_t)gridDim.x) break;   // a tile for every block: nothing is left to take
     }
 }
 
-// Deduplication: every entry's neighbour id goes into its batch's id table.  One thread owns eight
-// entries; their first-probe compare-and-swaps are issued back to back (eight atomics in flight per
-// thread), collisions are resolved afterwards.  The keys of the ids that were new are appended to the
-// list with one global atomic per 2048 entries.
+// Deduplication: every entry's neighbour id goes into its batch's id table.  One thread owns four entries; their
+// compare-and-swaps go out back to back and the probes of those that met another id go on in rounds, all open entries of the
+// thread at a time.  Bound by the rounds a warp needs for its longest probe, one L2 round trip each (a bucket load before the
+// compare-and-swap made it slower: 134 -> 160 us for the inner hops of 128 mini-batches), so small tables are kept sparse
+// (mg_sample_many).  The keys of the ids that were new are appended to the list with one global atomic per 1024 entries.
 struct InsertArgs {
     DenseHeader* hdr;
     int hop;
@@ -388,7 +482,6 @@ struct InsertArgs {
     uint64_t* newlist;
     int64_t cap_new;
     int id_bits;
-    // outermost hop only: rows are handed out at insert time
     int32_t k;
     const int32_t* cum;          // [B][k+2]
     int32_t* hvals;
@@ -403,97 +496,98 @@ constexpr int kInsertSpan = 16;   // mini-batches a block's chunk of entries may
 // paper's arrays, with ascending ids, are an export: mg_dense_batch_perm).  A new node takes the next free row of its
 // mini-batch right here -- a count per mini-batch in shared memory, one global atomic per (block, mini-batch) --,
 // its table value is written at once, and its list entry carries (mini-batch, id, rank in the hop).
-__global__ void __launch_bounds__(kThreads) k_insert(InsertArgs a) {
-    constexpr bool OUTER = true;
-    __shared__ uint32_t warp_tot[kThreads / 32 + 1];
+__global__ void __launch_bounds__(kThreads, 6) k_insert(InsertArgs a) {
+    __shared__ uint32_t warp_tot[kThreads / 32];
     __shared__ uint32_t block_base;
     __shared__ uint32_t span_cnt[kInsertSpan], span_base[kInsertSpan];
+    __shared__ int32_t span_row[kInsertSpan];   // first row of the hop's new nodes in the mini-batch
     __shared__ int32_t first_batch;
-    if (a.hdr->status) return;
     const int32_t lo = a.hdr->ent_base[a.hop], hi = a.hdr->ent_base[a.hop + 1];
+    if (__syncthreads_or(a.hdr->status != 0)) return;   // (the whole block: another one may be setting it)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kChunk = kThreads * kInsertPerThread;
     for (int32_t base = lo + blockIdx.x * kChunk; base < hi; base += gridDim.x * kChunk) {
         int32_t u[kInsertPerThread], b[kInsertPerThread], old[kInsertPerThread];
         uint32_t slot[kInsertPerThread];
+        uint32_t open = 0, new_bits = 0;
 #pragma unroll
         for (int j = 0; j < kInsertPerThread; ++j) {
             const int32_t e = base + j * kThreads + threadIdx.x;
-            u[j] = -1; b[j] = 0; old[j] = 0; slot[j] = 0;
+            u[j] = -1; b[j] = 0; old[j] = -1; slot[j] = 0;
             if (e < hi) { u[j] = a.ent_nbrs[e]; b[j] = a.ent_repr[e]; }
         }
+        if (threadIdx.x == 0) first_batch = b[0];   // thread 0's first item is the chunk's first entry
+        if (threadIdx.x < kInsertSpan) span_cnt[threadIdx.x] = 0;
+        __syncthreads();
+        const int32_t b0 = first_batch;   // entries are ordered by mini-batch, so a chunk touches a short run of them
 #pragma unroll
         for (int j = 0; j < kInsertPerThread; ++j)
             if (u[j] >= 0) {
                 slot[j] = table_hash(u[j], a.tg.size);
                 old[j] = atomicCAS(&a.hkeys[(int64_t)b[j] * a.tg.size + slot[j]], -1, u[j]);
             }
-        uint32_t n_mine = 0, new_bits = 0;
 #pragma unroll
         for (int j = 0; j < kInsertPerThread; ++j) {
             if (u[j] < 0) continue;
-            bool fresh = old[j] == -1;
-            if (!fresh && old[j] != u[j]) {   // first slot taken by another id: linear probing
-                int32_t* keys = a.hkeys + (int64_t)b[j] * a.tg.size;
-                int32_t probe = 1;
-                for (; probe < a.tg.size; ++probe) {
-                    slot[j] = slot[j] + 1u == (uint32_t)a.tg.size ? 0u : slot[j] + 1u;
-                    const int32_t o = atomicCAS(&keys[slot[j]], -1, u[j]);
-                    if (o == -1) { fresh = true; break; }
-                    if (o == u[j]) break;
-                }
-                if (probe >= a.tg.size) { atomicOr(&a.hdr->status, ST_CAP_TABLE); slot[j] = 0; }
-            }
-            // an entry that found its node already in the table gets the node's row later (k_relabel): it leaves
-            // -1 - (table index) behind; the entry of a new node gets its row below
-            if (fresh) { new_bits |= 1u << j; ++n_mine; }
-            else a.ent_repr[base + j * kThreads + threadIdx.x] = -1 - (b[j] * a.tg.size + (int32_t)slot[j]);
+            if (old[j] == -1) new_bits |= 1u << j;
+            else if (old[j] != u[j]) open |= 1u << j;
         }
-        // block-wide exclusive scan of the per-thread counts, one global atomic for the block
+        for (int32_t probe = 1; open; ++probe) {   // linear probing
+            if (probe >= a.tg.size) { atomicOr(&a.hdr->status, ST_CAP_TABLE); break; }
+#pragma unroll
+            for (int j = 0; j < kInsertPerThread; ++j)
+                if (open >> j & 1) {
+                    slot[j] = slot[j] + 1u == (uint32_t)a.tg.size ? 0u : slot[j] + 1u;
+                    old[j] = atomicCAS(&a.hkeys[(int64_t)b[j] * a.tg.size + slot[j]], -1, u[j]);
+                }
+#pragma unroll
+            for (int j = 0; j < kInsertPerThread; ++j)
+                if (open >> j & 1) {
+                    if (old[j] == -1) new_bits |= 1u << j;
+                    if (old[j] == -1 || old[j] == u[j]) open &= ~(1u << j);
+                }
+        }
+        const uint32_t n_mine = __popc(new_bits);
+        uint32_t rank[kInsertPerThread];
+#pragma unroll
+        for (int j = 0; j < kInsertPerThread; ++j) {
+            rank[j] = 0;
+            // an entry that found its node already in the table gets the node's row later (k_place): it leaves
+            // -1 - (table index) behind; the entry of a new node gets its row below
+            if (new_bits >> j & 1) {
+                const int32_t bb = b[j] - b0;
+                rank[j] = bb < kInsertSpan ? atomicAdd(&span_cnt[bb], 1u) : atomicAdd(&a.batch_cnt[b[j]], 1u);
+            } else if (u[j] >= 0) a.ent_repr[base + j * kThreads + threadIdx.x] = -1 - (b[j] * a.tg.size + (int32_t)slot[j]);
+        }
         const uint32_t inc = warp_incl_scan(n_mine);
         if (lane == 31) warp_tot[warp] = inc;
         __syncthreads();
+        // the block's run of the list (one thread) and of its mini-batches' rows (another warp's threads): one round trip
         if (threadIdx.x == 0) {
             uint32_t run = 0;
-            for (int w = 0; w < kThreads / 32; ++w) { const uint32_t t = warp_tot[w]; warp_tot[w] = run; run += t; }
-            block_base = run ? atomicAdd(&a.hdr->n_new, run) : 0u;
+            for (int w = 0; w < kThreads / 32; ++w) run += warp_tot[w];
+            block_base = run ? atomicAdd(&a.hdr->n_new[a.hop], run) : 0u;
+        } else if (threadIdx.x >= 32 && threadIdx.x < 32 + kInsertSpan) {
+            const int i = (int)threadIdx.x - 32;
+            const uint32_t c = span_cnt[i];
+            if (c) {
+                span_row[i] = a.cum[(b0 + i) * (a.k + 2) + a.hop + 1];
+                span_base[i] = atomicAdd(&a.batch_cnt[b0 + i], c);
+            }
         }
         __syncthreads();
-        int64_t pos = (int64_t)block_base + warp_tot[warp] + inc - n_mine;
-        uint32_t rank[kInsertPerThread];
-        if (OUTER) {
-            // entries are ordered by mini-batch, so a chunk touches a short run of them
-            if (threadIdx.x == 0) first_batch = b[0];   // thread 0's first item is the chunk's first entry
-            if (threadIdx.x < kInsertSpan) span_cnt[threadIdx.x] = 0;
-            __syncthreads();
-            const int32_t b0 = first_batch;
-#pragma unroll
-            for (int j = 0; j < kInsertPerThread; ++j) {
-                rank[j] = 0;
-                if (new_bits & (1u << j)) {
-                    const int32_t bb = b[j] - b0;
-                    rank[j] = bb < kInsertSpan ? atomicAdd(&span_cnt[bb], 1u) : atomicAdd(&a.batch_cnt[b[j]], 1u);
-                }
-            }
-            __syncthreads();
-            if (threadIdx.x < kInsertSpan && span_cnt[threadIdx.x])
-                span_base[threadIdx.x] = atomicAdd(&a.batch_cnt[b0 + threadIdx.x], span_cnt[threadIdx.x]);
-            __syncthreads();
-#pragma unroll
-            for (int j = 0; j < kInsertPerThread; ++j)
-                if (new_bits & (1u << j)) {
-                    const int32_t bb = b[j] - b0;
-                    if (bb < kInsertSpan) rank[j] += span_base[bb];
-                    const int64_t row = (int64_t)a.cum[b[j] * (a.k + 2) + a.hop + 1] + rank[j];
-                    if (row < a.max_nodes_per_batch) a.hvals[(int64_t)b[j] * a.tg.size + slot[j]] = (int32_t)row;
-                    else atomicOr(&a.hdr->status, ST_CAP_TABLE);
-                    a.ent_repr[base + j * kThreads + threadIdx.x] = (int32_t)row;   // final: no table read for this entry
-                }
-        }
+        int64_t pos = (int64_t)block_base + inc - n_mine;
+        for (int w = 0; w < warp; ++w) pos += warp_tot[w];
 #pragma unroll
         for (int j = 0; j < kInsertPerThread; ++j)
-            if (new_bits & (1u << j)) {
-                const uint64_t key = (uint64_t)(OUTER ? rank[j] : slot[j]) | ((uint64_t)(uint32_t)u[j] << MG_SLOT_BITS) |
+            if (new_bits >> j & 1) {
+                const int32_t bb = b[j] - b0;
+                if (bb < kInsertSpan) rank[j] += span_base[bb];
+                const int64_t row = (int64_t)(bb < kInsertSpan ? span_row[bb] : a.cum[b[j] * (a.k + 2) + a.hop + 1]) + rank[j];
+                if (row < a.max_nodes_per_batch) a.hvals[(int64_t)b[j] * a.tg.size + slot[j]] = (int32_t)row;
+                else atomicOr(&a.hdr->status, ST_CAP_TABLE);
+                a.ent_repr[base + j * kThreads + threadIdx.x] = (int32_t)row;   // final: no table read for this entry
+                const uint64_t key = (uint64_t)rank[j] | ((uint64_t)(uint32_t)u[j] << MG_SLOT_BITS) |
                                      ((uint64_t)(uint32_t)b[j] << (MG_SLOT_BITS + a.id_bits));
                 if (pos < a.cap_new) a.newlist[pos] = key;
                 else atomicOr(&a.hdr->status, ST_CAP_NODES);
@@ -553,7 +647,7 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_entries(DedupArgs a) 
     __shared__ uint32_t cnt[kWarps][kDedupMaxBuckets];
     __shared__ uint32_t base[kDedupMaxBuckets + 1];
     __shared__ int32_t hop_lo[MG_MAX_HOPS + 1], hop_row0[MG_MAX_HOPS + 2];
-    if (a.hdr->status) return;
+    if (__syncthreads_or(a.hdr->status != 0)) return;   // (the whole block: another one may be setting it)
     const uint32_t nb = (uint32_t)a.nb;
     const int32_t b = (int32_t)(blockIdx.x / nb);
     const uint32_t r = blockIdx.x % nb;
@@ -630,7 +724,7 @@ __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
     extern __shared__ int32_t dedup_sm[];
     __shared__ uint32_t row_base, list_base, warp_tot[kDedupThreads / 32];
     __shared__ int32_t run_lo[2][kDedupMaxBuckets], run_start[2][kDedupMaxBuckets + 1];
-    if (a.hdr->status) return;
+    if (__syncthreads_or(a.hdr->status != 0)) return;   // (the whole block: another one may be setting it)
     const uint32_t S = (uint32_t)a.S, nb = (uint32_t)a.nb;
     int32_t* keys = dedup_sm;
     int32_t* vals = dedup_sm + S;
@@ -730,7 +824,7 @@ __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
         if (lane < kDedupThreads / 32) warp_tot[lane] = wi - w;
         if (lane == 31) {
             row_base = wi ? atomicAdd(&a.batch_cnt[b], wi) : 0u;
-            list_base = wi ? atomicAdd(&a.hdr->n_new, wi) : 0u;
+            list_base = wi ? atomicAdd(&a.hdr->n_new[a.hop], wi) : 0u;
         }
     }
     __syncthreads();
@@ -895,124 +989,129 @@ k_radix_scatter(const uint64_t* __restrict__ keys, uint64_t* __restrict__ out, c
 constexpr size_t kScatterSmem = (size_t)kSortTile * 8 + (size_t)(kThreads / 32) * kBins * 4 + 2 * (size_t)kBins * 4;
 
 // -------------------------------------------------------------------------------------
-// place the sorted new nodes as the next hop
+// place the new nodes as the next hop, give the entries their rows
 // -------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads)
-k_relabel(const DenseHeader* hdr, int hop, const int32_t* __restrict__ hvals, int32_t* ent_repr) {
-    if (hdr->status) return;
-    const int32_t lo = hdr->ent_base[hop], hi = hdr->ent_base[hop + 1];
-    for (int32_t e = lo + blockIdx.x * blockDim.x + threadIdx.x; e < hi; e += gridDim.x * blockDim.x) {
-        const int32_t v = ent_repr[e];
-        if (v < 0) ent_repr[e] = hvals[-1 - v];   // entries of nodes that were new got their row at insert time
-    }
-}
+// The hop's new nodes per mini-batch, summed up, are the next hop's node offsets (every block takes the sums for itself, block 0
+// writes them down: a kernel of one block for it cost 2 us and a gap per hop).  Then: list entry (mini-batch, id, rank) -> the
+// node's place in its mini-batch's run; an entry that met a known node -> that node's row (entries of new nodes got theirs at
+// insert time; the shared-memory path of the last hop leaves none).
+// FINAL (last hop): block 0 also writes the packed row bases of every layer and the per-batch entry bounds of every hop, and
+// the sample's summary (header, per-batch tables) for the host, stored straight into mapped pinned memory.  A copy engine
+// is not used on purpose: a large output copy of a forward pass may be queued on it, and the host would wait for that copy
+// before it learned the sample's sizes.  (After an error the summary still goes out: it carries the status word.)
+struct PlaceArgs {
+    DenseHeader* hdr;
+    int hop;
+    const uint64_t* list;
+    int id_bits;
+    const uint32_t* batch_cnt;   // [B] new nodes of the hop
+    int64_t cap_nodes;
+    int32_t* nodes;
+    int32_t* node_batch;
+    const int32_t* hvals;      // null: the entries have their rows
+    int32_t table_limit;       // nodes of a mini-batch that the id tables are meant for
+    int32_t* ent_repr;
+    int32_t B, k;
+    int32_t* cum;
+    int32_t* node_off;
+    // FINAL
+    int32_t n_hdr;
+    const int32_t* ent_off;
+    int32_t* rowbase;
+    int32_t* ent_hop;
+    int32_t* out;              // n_hdr header words, cum, node_off, rowbase, ent_hop
+};
 
-// End of a hop (one block): the node arena's next bound, then per-batch counts -> node offsets of the next hop and the
-// batches' row totals
-__global__ void __launch_bounds__(1024)
-k_outer_offsets(DenseHeader* hdr, int hop, int32_t B, int32_t k, const uint32_t* __restrict__ batch_cnt, int32_t* node_off_next,
-                int32_t* cum, int32_t max_nodes_per_batch, int64_t cap_nodes) {
-    __shared__ uint32_t warp_tot[33];
-    if (hdr->status) return;
+__device__ __forceinline__ void finish_sample(const PlaceArgs& a, bool bad) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int32_t start = hdr->hop_base[hop + 1];
-    const int64_t end = (int64_t)start + hdr->n_new;
-    if (end > cap_nodes) { if (threadIdx.x == 0) atomicOr(&hdr->status, ST_CAP_NODES); return; }
-    if (threadIdx.x == 0) hdr->hop_base[hop + 2] = (int32_t)end;
-    uint32_t carry = 0;
-    for (int s0 = 0; s0 < B; s0 += 1024) {
-        const int b = s0 + threadIdx.x;
-        const uint32_t v = b < B ? batch_cnt[b] : 0u;
-        const uint32_t inc = warp_incl_scan(v);
-        if (lane == 31) warp_tot[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            const uint32_t w = warp_tot[lane];
-            const uint32_t wi = warp_incl_scan(w);
-            warp_tot[lane] = wi - w;
-            if (lane == 31) warp_tot[32] = wi;
-        }
-        __syncthreads();
-        if (b < B) {
-            node_off_next[b] = start + (int32_t)(carry + warp_tot[warp] + inc - v);
-            const int32_t rows = cum[b * (k + 2) + hop + 1] + (int32_t)v;
-            cum[b * (k + 2) + hop + 2] = rows;
-            if (rows > max_nodes_per_batch) atomicOr(&hdr->status, ST_CAP_TABLE);
-        }
-        carry += warp_tot[32];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) node_off_next[B] = start + (int32_t)carry;
-}
-
-// Outermost hop: list entry (mini-batch, id, rank) -> the node's place in its mini-batch's run
-__global__ void __launch_bounds__(kThreads)
-k_place_nodes_outer(const DenseHeader* hdr, const uint64_t* __restrict__ list, int id_bits, const int32_t* __restrict__ node_off_next,
-                    int32_t* nodes, int32_t* node_batch) {
-    if (hdr->status) return;
-    const int32_t n = (int32_t)hdr->n_new;
-    const uint64_t id_mask = (1ull << id_bits) - 1ull;
-    for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        const uint64_t key = list[j];
-        const int32_t b = (int32_t)(key >> (MG_SLOT_BITS + id_bits));
-        const int32_t at = node_off_next[b] + (int32_t)(key & ((1u << MG_SLOT_BITS) - 1u));
-        nodes[at] = (int32_t)((key >> MG_SLOT_BITS) & id_mask);
-        node_batch[at] = b;
-    }
-}
-
-// one block: packed row bases of every layer and the per-batch entry bounds of every hop; then the sample's summary
-// (header, per-batch tables) for the host, stored straight into mapped pinned memory.  A copy engine is not used on
-// purpose: a large output copy of a forward pass may be queued on it, and the host would wait for that copy before it
-// learned the sample's sizes.  (After an error the summary still goes out: it carries the status word.)
-__global__ void __launch_bounds__(1024)
-k_finalize(DenseHeader* hdr, int32_t B, int32_t k, const int32_t* cum, const int32_t* node_off,
-           const int32_t* __restrict__ ent_off, int32_t* rowbase, int32_t* ent_hop, int32_t n_hdr, int32_t* out) {
-    __shared__ uint32_t warp_tot[33];
-    const bool bad = hdr->status != 0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int l = 0; l <= k && !bad; ++l) {
-        uint32_t carry = 0;
-        for (int start = 0; start < B; start += 1024) {
-            const int b = start + threadIdx.x;
-            const uint32_t v = b < B ? (uint32_t)cum[b * (k + 2) + (k - l + 1)] : 0u;
-            const uint32_t inc = warp_incl_scan(v);
-            if (lane == 31) warp_tot[warp] = inc;
-            __syncthreads();
-            if (warp == 0) {
-                const uint32_t w = warp_tot[lane];
-                const uint32_t wi = warp_incl_scan(w);
-                warp_tot[lane] = wi - w;
-                if (lane == 31) warp_tot[32] = wi;
-            }
-            __syncthreads();
-            if (b < B) rowbase[l * (B + 1) + b] = (int32_t)(carry + warp_tot[warp] + inc - v);
-            carry += warp_tot[32];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            rowbase[l * (B + 1) + B] = (int32_t)carry;
-            hdr->rows_total[l] = (int32_t)carry;
-        }
-    }
-    for (int h = 0; h < k && !bad; ++h)
-        for (int b = threadIdx.x; b <= B; b += blockDim.x)
-            ent_hop[h * (B + 1) + b] = ent_off[node_off[h * (B + 1) + b]];
-    __syncthreads();   // (one block: its own writes above are what the summary reads)
+    const int32_t B = a.B, k = a.k;
     const int32_t n_cum = B * (k + 2), n_off = (k + 1) * (B + 1), n_ent = k * (B + 1);
-    const int32_t total = n_hdr + n_cum + 2 * n_off + n_ent;
-    const volatile int32_t* h32 = reinterpret_cast<const volatile int32_t*>(hdr);
-    for (int32_t i = threadIdx.x; i < total; i += blockDim.x) {
-        int32_t j = i, v;
-        if (j < n_hdr) v = j < (int32_t)(sizeof(DenseHeader) / 4) ? h32[j] : 0;
-        else if ((j -= n_hdr) < n_cum) v = cum[j];
-        else if ((j -= n_cum) < n_off) v = node_off[j];
-        else if ((j -= n_off) < n_off) v = rowbase[j];
-        else v = ent_hop[j - n_off];
-        out[i] = v;
+    int32_t* o_cum = a.out + a.n_hdr;
+    int32_t* o_off = o_cum + n_cum;
+    int32_t* o_row = o_off + n_off;
+    int32_t* o_ent = o_row + n_off;
+    const volatile int32_t* h32 = reinterpret_cast<const volatile int32_t*>(a.hdr);
+    for (int32_t i = threadIdx.x; i < a.n_hdr; i += blockDim.x) a.out[i] = h32[i];
+    if (bad) return;
+    for (int l = warp; l <= k; l += kThreads / 32) {   // a warp per layer: rows of the mini-batches, summed up
+        uint32_t carry = 0;
+        for (int s0 = 0; s0 < B; s0 += 32) {
+            const int b = s0 + lane;
+            const uint32_t v = b < B ? (uint32_t)a.cum[b * (k + 2) + (k - l + 1)] : 0u;
+            const uint32_t inc = warp_incl_scan(v);
+            if (b < B) {
+                const int32_t r = (int32_t)(carry + inc - v);
+                a.rowbase[l * (B + 1) + b] = r;
+                o_row[l * (B + 1) + b] = r;
+            }
+            carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
+        }
+        if (lane == 0) { a.rowbase[l * (B + 1) + B] = (int32_t)carry; o_row[l * (B + 1) + B] = (int32_t)carry; }
     }
+    for (int32_t i = threadIdx.x; i < n_ent; i += blockDim.x) {   // (hop h = i / (B + 1), as in node_off)
+        const int32_t e = a.ent_off[a.node_off[i]];
+        a.ent_hop[i] = e;
+        o_ent[i] = e;
+    }
+    for (int32_t i = threadIdx.x; i < n_cum; i += blockDim.x) o_cum[i] = a.cum[i];
+    for (int32_t i = threadIdx.x; i < n_off; i += blockDim.x) o_off[i] = a.node_off[i];
 }
 
+template <bool FINAL>
+__global__ void __launch_bounds__(kThreads) k_place(PlaceArgs a) {
+    extern __shared__ int32_t next_off[];   // [B] first node of the mini-batch in the next hop
+    __shared__ uint32_t part[kThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t n = (int32_t)a.hdr->n_new[a.hop], start = a.hdr->hop_base[a.hop + 1];
+    const int32_t lo = a.hdr->ent_base[a.hop], hi = a.hdr->ent_base[a.hop + 1];
+    // (the whole block alike: block 0 may be adding to the status)
+    bool bad = __syncthreads_or(a.hdr->status != 0);
+    const bool full = !bad && (int64_t)start + n > a.cap_nodes;
+    if (!bad && !full) {
+        uint32_t carry = (uint32_t)start;
+        for (int s0 = 0; s0 < a.B; s0 += kThreads) {
+            const int b = s0 + (int)threadIdx.x;
+            const uint32_t v = b < a.B ? a.batch_cnt[b] : 0u;
+            const uint32_t inc = warp_incl_scan(v);
+            if (lane == 31) part[warp] = inc;
+            __syncthreads();
+            uint32_t before = carry, total = 0;
+            for (int w = 0; w < kThreads / 32; ++w) { if (w < warp) before += part[w]; total += part[w]; }
+            if (b < a.B) {
+                next_off[b] = (int32_t)(before + inc - v);
+                if (blockIdx.x == 0) {
+                    a.node_off[(a.hop + 1) * (a.B + 1) + b] = next_off[b];
+                    const int32_t rows = a.cum[b * (a.k + 2) + a.hop + 1] + (int32_t)v;
+                    a.cum[b * (a.k + 2) + a.hop + 2] = rows;
+                    if (a.hvals && rows > a.table_limit) atomicOr(&a.hdr->status, ST_CAP_TABLE);
+                }
+            }
+            carry += total;
+            __syncthreads();
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            a.hdr->hop_base[a.hop + 2] = start + n;
+            a.node_off[(a.hop + 1) * (a.B + 1) + a.B] = start + n;
+        }
+    } else if (full && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&a.hdr->status, ST_CAP_NODES);
+    bad |= full;
+    if (FINAL && blockIdx.x == 0) { __syncthreads(); finish_sample(a, bad); return; }
+    if (bad) return;
+    const int32_t step = (int32_t)(gridDim.x - FINAL) * kThreads, tid = (int32_t)(blockIdx.x - FINAL) * kThreads + (int32_t)threadIdx.x;
+    const uint64_t id_mask = (1ull << a.id_bits) - 1ull;
+    for (int32_t j = tid; j < n; j += step) {
+        const uint64_t key = a.list[j];
+        const int32_t b = (int32_t)(key >> (MG_SLOT_BITS + a.id_bits));
+        const int32_t at = next_off[b] + (int32_t)(key & ((1u << MG_SLOT_BITS) - 1u));
+        a.nodes[at] = (int32_t)((key >> MG_SLOT_BITS) & id_mask);
+        a.node_batch[at] = b;
+    }
+    if (!a.hvals) return;
+    for (int32_t e = lo + tid; e < hi; e += step) {
+        const int32_t v = a.ent_repr[e];
+        if (v < 0) a.ent_repr[e] = a.hvals[-1 - v];
+    }
+}
 
 // -------------------------------------------------------------------------------------
 // export to the paper's layout (mg_dense_view)
@@ -1273,7 +1372,7 @@ void mg_sort_u64(mg_ctx* ctx, uint64_t* const buf[2], const SortParams* sp, int 
         const int shift = lo_bit + kRadixBits * p;
         k_radix_hist<<<grid, kThreads, 0, st>>>(buf[cur], sp, shift, hist, tiles, p == 0);
         k_scan_reduce<<<grid, kThreads, 0, st>>>(hist, r, scan_tmp);
-        k_scan_tiles<<<1, 1024, 0, st>>>(scan_tmp, r, nullptr, HopClose{nullptr, 0, nullptr, 0});
+        k_scan_tiles<<<1, 1024, 0, st>>>(scan_tmp, r, nullptr);
         k_scan_down<<<grid, kThreads, 0, st>>>(hist, r, scan_tmp);
         k_radix_scatter<<<grid, kThreads, kScatterSmem, st>>>(buf[cur], buf[cur ^ 1], sp, shift, hist, tiles, p == 0);
         cur ^= 1;
@@ -1289,7 +1388,7 @@ void mg_scan_u32(mg_ctx* ctx, uint32_t* data, const int32_t* lo, const int32_t* 
     const int grid = mg_grid(ctx, 8);
     ScanRange r{lo, hi, base};
     k_scan_reduce<<<grid, kThreads, 0, st>>>(data, r, scan_tmp);
-    k_scan_tiles<<<1, 1024, 0, st>>>(scan_tmp, r, total_out, HopClose{nullptr, 0, nullptr, 0});
+    k_scan_tiles<<<1, 1024, 0, st>>>(scan_tmp, r, total_out);
     k_scan_down<<<grid, kThreads, 0, st>>>(data, r, scan_tmp);
     ctx->launches += 3;
 }
@@ -1309,6 +1408,9 @@ static int dev_realloc(mg_ctx* ctx, T** p, size_t elems) {
     return MG_OK;
 }
 
+// tiles of a hop at most (tiles below 256 nodes: at most kTilesWanted)
+static size_t tile_states(int64_t cap_nodes) { return (size_t)cap_nodes / kThreads + kTilesWanted + 2; }
+
 static int dense_alloc(mg_ctx* ctx, mg_dense* d, int32_t B, int32_t k, int64_t cap_nodes, int64_t cap_entries,
                        int32_t table_size, int32_t smem_nb) {
     int rc;
@@ -1321,9 +1423,10 @@ static int dense_alloc(mg_ctx* ctx, mg_dense* d, int32_t B, int32_t k, int64_t c
         if ((rc = dev_realloc(ctx, &d->nodes, (size_t)cap_nodes))) return rc;
         if ((rc = dev_realloc(ctx, &d->node_batch, (size_t)cap_nodes))) return rc;
         if ((rc = dev_realloc(ctx, &d->ent_off, (size_t)cap_nodes + 1))) return rc;
-        if ((rc = dev_realloc(ctx, &d->node_r0, (size_t)cap_nodes))) return rc;
-        if ((rc = dev_realloc(ctx, &d->node_deg, (size_t)cap_nodes))) return rc;
-        d->cap_nodes_out = 0;
+        const size_t n_states = tile_states(cap_nodes);
+        if ((rc = dev_realloc(ctx, &d->tile_state, n_states))) return rc;
+        MG_CUDA(ctx, cudaMemsetAsync(d->tile_state, 0, n_states * sizeof(uint64_t), ctx->stream));   // (no state carries epoch 0)
+        d->epoch = 0;
         if ((rc = dev_realloc(ctx, &d->newlist[0], (size_t)cap_nodes))) return rc;
         if ((rc = dev_realloc(ctx, &d->newlist[1], (size_t)cap_nodes))) return rc;
         d->cap_nodes = cap_nodes;
@@ -1361,12 +1464,6 @@ static int dense_alloc(mg_ctx* ctx, mg_dense* d, int32_t B, int32_t k, int64_t c
             if ((rc = dev_realloc(ctx, &d->share_off, (size_t)need_share))) return rc;
             d->cap_share = need_share;
         }
-    }
-    if (ctx->sample_inout && d->cap_nodes_out < d->cap_nodes) {
-        d->cap_nodes_out = 0;
-        if ((rc = dev_realloc(ctx, &d->node_r0_out, (size_t)d->cap_nodes))) return rc;
-        if ((rc = dev_realloc(ctx, &d->node_deg_out, (size_t)d->cap_nodes))) return rc;
-        d->cap_nodes_out = d->cap_nodes;
     }
     const int64_t need_table = (int64_t)B * table_size;
     if (d->alloc_table < need_table) {
@@ -1437,12 +1534,13 @@ extern "C" int mg_sample_many_end(mg_ctx* ctx, mg_dense* d) {
     d->pending = false;
     MG_CUDA(ctx, cudaEventSynchronize(d->ev_sampled));
     const int B = d->n_batches, k = d->k;
-    const int32_t* p = d->h_pinned;
+    const int32_t* p = d->h_stage + d->h_summary_at;
     memcpy(&d->h_hdr, p, sizeof(DenseHeader)); p += (sizeof(DenseHeader) + 3) / 4;
     d->h_cum.assign(p, p + (size_t)B * (k + 2)); p += (size_t)B * (k + 2);
     d->h_node_off.assign(p, p + (size_t)(k + 1) * (B + 1)); p += (size_t)(k + 1) * (B + 1);
     d->h_rowbase.assign(p, p + (size_t)(k + 1) * (B + 1)); p += (size_t)(k + 1) * (B + 1);
     d->h_ent_hop.assign(p, p + (size_t)k * (B + 1));
+    for (int l = 0; l <= k; ++l) d->h_hdr.rows_total[l] = d->h_rowbase[(size_t)l * (B + 1) + B];
     if (d->h_hdr.status) return mg_fail(ctx, status_code(d->h_hdr.status), "%s", status_text(d->h_hdr.status));
     d->valid = true;
     d->perm_batch = -1;
@@ -1464,8 +1562,8 @@ static void sample_kernel_attributes() {
     if (done) return;
     cudaFuncSetAttribute(k_radix_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
     cudaFuncSetAttribute(k_dedupe_last, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kDedupMaxSlots * 2 * sizeof(int32_t)));
-    cudaFuncSetAttribute(k_pick_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)));
+    cudaFuncSetAttribute(k_hop<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + kTileMax * hop_node_bytes(true));
     done = true;
 }
 
@@ -1540,7 +1638,11 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
         table_nodes = std::min<int64_t>(cap_batch, caps->max_inner_nodes_per_batch);
         for (int b = 0; b < n_batches; ++b) table_nodes = std::max<int64_t>(table_nodes, target_offsets[b + 1] - target_offsets[b]);
     }
-    const int64_t want_slots = std::max<int64_t>(16, (table_nodes + table_nodes / 2 + table_nodes / 8 + 7) / 8 * 8);
+    // (1.625 slots per node; four where all tables together stay within 8 MB: a sparse table saves a small hop the long probes,
+    // 34 -> 17 us for the two inner hops of one mini-batch)
+    int64_t want_slots = std::max<int64_t>(16, (table_nodes + table_nodes / 2 + table_nodes / 8 + 7) / 8 * 8);
+    const int32_t table_limit = (int32_t)std::min<int64_t>(want_slots, INT32_MAX);   // (a sparse table takes no more nodes than a dense one)
+    if (4 * table_nodes * n_batches <= 2ll << 20) want_slots = std::max<int64_t>(16, (4 * table_nodes + 7) / 8 * 8);
     if (want_slots > (1ll << MG_SLOT_BITS)) return mg_fail(ctx, MG_ERR_CAPACITY, "max_nodes_per_batch above %d", (int)((1ll << MG_SLOT_BITS) * 8 / 13));
     const int32_t table_size = (int32_t)want_slots;
     if ((int64_t)table_size * n_batches >= (1ll << 31))
@@ -1572,115 +1674,102 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     // Host-known part of the header, the per-batch tables and the seeds go through a pinned staging block of the
     // sample handle, so that the device work below reads nothing but fixed addresses: it can then be captured once
     // in a CUDA graph and replayed for every later call with the same shape.
-    const size_t n_stage_ints = (sizeof(DenseHeader) + 3) / 4 + (size_t)(B + 1) + (size_t)B * (k + 2) + 2 * (size_t)B + 2;
-    if (d->h_stage_ints < n_stage_ints) {
+    // (mapped, so that no copy engine is involved.)  Up to kStageTargets targets in host memory travel in it too; more are copied.
+    static_assert(sizeof(DenseHeader) % 8 == 0, "the header is staged as 32-bit words");
+    const size_t hdr_ints = sizeof(DenseHeader) / 4;
+    const size_t seeds_at = (hdr_ints + (size_t)(B + 1) + (size_t)B * (k + 2) + 1) & ~(size_t)1;
+    const size_t targets_at = seeds_at + 2 * (size_t)B;
+    const size_t n_staged = !targets_on_device && T <= kStageTargets ? kStageTargets : 0;
+    const size_t n_summary = hdr_ints + (size_t)B * (k + 2) + 2 * (size_t)(k + 1) * (B + 1) + (size_t)k * (B + 1);
+    const size_t summary_at = targets_at + n_staged;
+    if (d->h_stage_ints < summary_at + n_summary) {
         if (d->h_stage) cudaFreeHost(d->h_stage);
         d->h_stage = nullptr; d->h_stage_ints = 0;
-        if (cudaHostAlloc((void**)&d->h_stage, n_stage_ints * sizeof(int32_t), cudaHostAllocMapped) != cudaSuccess ||
+        const size_t ints = summary_at + n_summary;
+        if (cudaHostAlloc((void**)&d->h_stage, ints * sizeof(int32_t), cudaHostAllocMapped) != cudaSuccess ||
             cudaHostGetDevicePointer((void**)&d->h_stage_dev, d->h_stage, 0) != cudaSuccess) {
             cudaGetLastError();
             return mg_fail(ctx, MG_ERR_OOM, "pinned host allocation failed");
         }
-        d->h_stage_ints = n_stage_ints;
+        d->h_stage_ints = ints;
     }
+    d->h_summary_at = summary_at;
     DenseHeader* st_hdr = reinterpret_cast<DenseHeader*>(d->h_stage);
-    int32_t* st_off = d->h_stage + (sizeof(DenseHeader) + 3) / 4;
+    int32_t* st_off = d->h_stage + hdr_ints;
     int32_t* st_cum = st_off + (B + 1);
-    uint64_t* st_seeds = reinterpret_cast<uint64_t*>(d->h_stage + (((sizeof(DenseHeader) + 3) / 4 + (size_t)(B + 1) + (size_t)B * (k + 2) + 1) & ~(size_t)1));
     memset(st_hdr, 0, sizeof(DenseHeader));
     st_hdr->hop_base[0] = 0;
     st_hdr->hop_base[1] = (int32_t)T;
+    if (++d->epoch >= 1u << 27) {   // (27 bits of a tile state's tag; a handle gets here after 134 million samples)
+        MG_CUDA(ctx, cudaMemsetAsync(d->tile_state, 0, tile_states(d->cap_nodes) * sizeof(uint64_t), st));
+        d->epoch = 1;
+    }
+    st_hdr->epoch = d->epoch;
     memset(st_cum, 0, sizeof(int32_t) * (size_t)B * (k + 2));
     for (int b = 0; b <= B; ++b) st_off[b] = (int32_t)target_offsets[b];
     for (int b = 0; b < B; ++b) st_cum[(size_t)b * (k + 2) + 1] = st_off[b + 1] - st_off[b];
-    memcpy(st_seeds, seeds, sizeof(uint64_t) * B);
-
-    // the summary's landing place (mapped pinned memory)
-    const size_t n_ints = (sizeof(DenseHeader) + 3) / 4 + (size_t)B * (k + 2) + 2 * (size_t)(k + 1) * (B + 1) + (size_t)k * (B + 1);
-    if (d->h_pinned_ints < n_ints) {
-        if (d->h_pinned) cudaFreeHost(d->h_pinned);
-        d->h_pinned = nullptr; d->h_pinned_ints = 0;
-        if (cudaHostAlloc((void**)&d->h_pinned, n_ints * sizeof(int32_t), cudaHostAllocMapped) != cudaSuccess ||
-            cudaHostGetDevicePointer((void**)&d->h_pinned_dev, d->h_pinned, 0) != cudaSuccess) {
-            cudaGetLastError();
-            return mg_fail(ctx, MG_ERR_OOM, "pinned host allocation failed");
-        }
-        d->h_pinned_ints = n_ints;
+    memcpy(d->h_stage + seeds_at, seeds, sizeof(uint64_t) * B);
+    if (targets_on_device) st_hdr->targets = (uint64_t)(uintptr_t)targets;
+    else if (n_staged) {
+        if (T > 0) memcpy(d->h_stage + targets_at, targets, sizeof(int32_t) * T);
+        st_hdr->targets = (uint64_t)(uintptr_t)(d->h_stage_dev + targets_at);
+    } else {
+        MG_CUDA(ctx, cudaMemcpyAsync(d->newlist[1], targets, sizeof(int32_t) * T, cudaMemcpyHostToDevice, st));
+        st_hdr->targets = (uint64_t)(uintptr_t)d->newlist[1];
     }
     sample_kernel_attributes();
 
-    // the targets are staged in newlist[1] (outside the graph: their source changes from call to call)
-    if (T > 0) {
-        if (targets_on_device) {
-            k_copy_i32<<<std::max(1, std::min(mg_grid(ctx, 2), (int)((T + kThreads - 1) / kThreads))), kThreads, 0, st>>>(targets, (int32_t*)d->newlist[1], T);
-            ctx->launches++;
-        } else {
-            MG_CUDA(ctx, cudaMemcpyAsync(d->newlist[1], targets, sizeof(int32_t) * T, cudaMemcpyHostToDevice, st));
-        }
+    // Grids follow what a hop can hold at most (the number of targets rounded up to a power of two, so that calls of similar
+    // size share the captured graph): blocks without work cost the small calls as much as the work itself.
+    int64_t T_bound = 1;
+    while (T_bound < T) T_bound <<= 1;
+    int64_t nodes_bound[MG_MAX_HOPS + 1], entries_bound[MG_MAX_HOPS];
+    nodes_bound[0] = std::min<int64_t>(T_bound, d->cap_nodes);
+    for (int h = 0; h < k; ++h) {
+        entries_bound[h] = std::min<int64_t>(nodes_bound[h] * fanouts[h] * (inout ? 2 : 1), d->cap_entries);
+        nodes_bound[h + 1] = std::min<int64_t>({entries_bound[h], d->cap_nodes, (int64_t)B * cap_batch});
     }
-    const int32_t* tgt_dev = (const int32_t*)d->newlist[1];
+    auto blocks_for = [&](int64_t items, int per_block, int ctas_per_sm) {
+        return (unsigned)std::max<int64_t>(1, std::min<int64_t>((items + per_block - 1) / per_block, mg_grid(ctx, ctas_per_sm)));
+    };
 
     // ---- everything the device does for this sample ----
     auto enqueue = [&]() -> int {
+    uint32_t* batch_cnt = d->batch_cnt;   // new nodes per (hop, mini-batch)
     {
         ProfScope ps(ctx, PH_SAMPLE_INIT, 1);
-        static_assert(sizeof(DenseHeader) % 4 == 0, "the header is staged as 32-bit words");
-        k_stage_in<<<4, kThreads, 0, st>>>(d->h_stage_dev, (int32_t)(sizeof(DenseHeader) / 4), B + 1, B * (k + 2), 2 * B,
-                                          (int32_t)(reinterpret_cast<int32_t*>(st_seeds) - d->h_stage), reinterpret_cast<int32_t*>(d->hdr),
-                                          d->node_off, d->cum, reinterpret_cast<int32_t*>(d->d_seeds));
+        BeginArgs a{d->h_stage_dev, (int32_t)hdr_ints, B + 1, B * (k + 2), 2 * B, (int32_t)seeds_at, k * B, (int64_t)B * table_size / 4,
+                    reinterpret_cast<int32_t*>(d->hdr), d->node_off, d->cum, reinterpret_cast<int32_t*>(d->d_seeds),
+                    reinterpret_cast<int32_t*>(batch_cnt), reinterpret_cast<int4*>(d->hkeys)};
+        k_begin<<<blocks_for(a.n_table4, 4 * kThreads, 8), kThreads, 0, st>>>(a);
         ctx->launches++;
-        MG_CUDA(ctx, cudaMemsetAsync(d->hkeys, 0xFF, sizeof(int32_t) * (size_t)B * table_size, st));
-        {
-            k_init_targets<<<mg_grid(ctx, 4), kThreads, 0, st>>>(d->hdr, tgt_dev, d->node_off, B, d->nodes,
-                                                               d->node_batch, d->hkeys, d->hvals, tg, ctx->n_nodes, mg_feat_geom(ctx));
-            ctx->launches++;
-        }
     }
-
-    // new nodes per (hop, mini-batch)
-    uint32_t* batch_cnt = d->batch_cnt;
-    MG_CUDA(ctx, cudaMemsetAsync(batch_cnt, 0, sizeof(uint32_t) * (size_t)k * B, st));
-    uint32_t* scan_total = (uint32_t*)(d->scan_tmp + d->scan_tmp_elems - 4);
-    const int grid = mg_grid(ctx, 8);
     for (int h = 0; h < k; ++h) {
         const int32_t f = fanouts[h];
-        {
-            ProfScope ps(ctx, PH_SAMPLE_COUNT, 1);
-            k_count<<<grid, kThreads, 0, st>>>(d->hdr, h, f, d->nodes, ctx->view_off, d->ent_off, d->node_r0, d->node_deg,
-                                               inout ? ctx->view_off_out : nullptr, d->node_r0_out, d->node_deg_out);
-        }
-        {
-            ProfScope ps(ctx, PH_SAMPLE_SCAN, 3);
-            // (the scan's middle kernel also closes the hop's entry range: ent_base, the sentinel offset, the arena check)
-            const ScanRange sr{&d->hdr->hop_base[h], &d->hdr->hop_base[h + 1], &d->hdr->ent_base[h]};
-            k_scan_reduce<<<grid, kThreads, 0, st>>>((uint32_t*)d->ent_off, sr, (uint32_t*)d->scan_tmp);
-            k_scan_tiles<<<1, 1024, 0, st>>>((uint32_t*)d->scan_tmp, sr, scan_total, HopClose{d->hdr, h, d->ent_off, d->cap_entries});
-            k_scan_down<<<grid, kThreads, 0, st>>>((uint32_t*)d->ent_off, sr, (uint32_t*)d->scan_tmp);
-            ctx->launches += 3;
-        }
+        const bool smem_hop = smem_last && h == k - 1;
         {
             ProfScope ps(ctx, PH_SAMPLE_PICK, 1);
-            for (int dir = 0; dir < (inout ? 2 : 1); ++dir) {
-                PickArgs a{d->hdr, h, f, d->nodes, d->node_batch, dir ? d->node_r0_out : d->node_r0, dir ? d->node_deg_out : d->node_deg,
-                           dir ? ctx->view_nbrs_out : ctx->view_nbrs, d->ent_off, d->ent_nbrs, d->ent_repr, d->d_seeds,
-                           dir ? d->node_deg : nullptr, dir ? (uint32_t)MG_OUT_SLOT_BASE : 0u};
-                // the narrowest group that holds the fanout among those that waste at most two lanes of a warp
-                if (f <= 2) k_pick<2><<<grid, kThreads, 0, st>>>(a);
-                else if (f == 3) k_pick<3><<<grid, kThreads, 0, st>>>(a);
-                else if (f == 4) k_pick<4><<<grid, kThreads, 0, st>>>(a);
-                else if (f == 5) k_pick<5><<<grid, kThreads, 0, st>>>(a);
-                else if (f == 6) k_pick<6><<<grid, kThreads, 0, st>>>(a);
-                else if (f <= 8) k_pick<8><<<grid, kThreads, 0, st>>>(a);
-                else if (f <= 10) k_pick<10><<<grid, kThreads, 0, st>>>(a);
-                else if (f <= 16) k_pick<16><<<grid, kThreads, 0, st>>>(a);
-                else if (f <= 32) k_pick<32><<<grid, kThreads, 0, st>>>(a);
-                else {
-                    const size_t wide_smem = (size_t)(kThreads / 32) * 2 * f * sizeof(uint32_t);   // 64 KiB at the largest fanout
-                    k_pick_wide<<<grid, kThreads, wide_smem, st>>>(a);
-                }
-                if (dir) ctx->launches++;
-            }
-            if (smem_last && h == k - 1) {
+            HopArgs a{d->hdr, h, f, d->nodes, d->node_batch, {ctx->view_off, inout ? ctx->view_off_out : nullptr},
+                      {ctx->view_nbrs, ctx->view_nbrs_out}, d->ent_off, d->ent_nbrs, d->ent_repr, d->d_seeds, d->cap_entries, d->tile_state,
+                      hop_tile(nodes_bound[h]), B, d->node_off, d->hkeys, d->hvals, tg, ctx->n_nodes, mg_feat_geom(ctx)};
+            const unsigned grid = blocks_for(nodes_bound[h], 32, 8);
+            const size_t sm = (size_t)a.tile_cap * hop_node_bytes(inout);   // 36 KiB at most
+            // the narrowest group that holds the fanout among those that waste at most two lanes of a warp
+            if (f <= 2) k_hop<2><<<grid, kThreads, sm, st>>>(a);
+            else if (f == 3) k_hop<3><<<grid, kThreads, sm, st>>>(a);
+            else if (f == 4) k_hop<4><<<grid, kThreads, sm, st>>>(a);
+            else if (f == 5) k_hop<5><<<grid, kThreads, sm, st>>>(a);
+            else if (f == 6) k_hop<6><<<grid, kThreads, sm, st>>>(a);
+            else if (f <= 8) k_hop<8><<<grid, kThreads, sm, st>>>(a);
+            else if (f <= 10) k_hop<10><<<grid, kThreads, sm, st>>>(a);
+            else if (f <= 16) k_hop<16><<<grid, kThreads, sm, st>>>(a);
+            else if (f <= 32) k_hop<32><<<grid, kThreads, sm, st>>>(a);
+            else k_hop<0><<<grid, kThreads, sm + (size_t)(kThreads / 32) * 2 * f * sizeof(uint32_t), st>>>(a);   // 64 KiB more at the largest fanout
+            ctx->launches++;
+        }
+        {
+            ProfScope ps(ctx, PH_SAMPLE_RELABEL, 1);
+            if (smem_hop) {
                 DedupArgs da{d->hdr, h, B, k, (int32_t)dedup_nb, dedup_slots, d->nodes, d->node_off, d->ent_off, d->ent_nbrs,
                              d->ent_repr, d->pairs, d->share_off, d->cum, batch_cnt + (size_t)h * B, d->newlist[0], d->cap_nodes,
                              id_bits, (int32_t)cap_batch, d->cap_entries};
@@ -1691,35 +1780,21 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
                 InsertArgs ia{d->hdr, h, d->ent_nbrs, d->ent_repr, d->hkeys, tg, d->newlist[0], d->cap_nodes, id_bits,
                               k, d->cum, d->hvals, batch_cnt + (size_t)h * B, (int32_t)cap_batch};
                 // many short blocks: measured on the bench's last hop, 0.94 ms at 32 blocks per SM against 1.08 ms at 8
-                // (blocks past the end of the entries return at once)
-                const int igrid = mg_grid(ctx, 32);
-                k_insert<<<igrid, kThreads, 0, st>>>(ia);
+                k_insert<<<blocks_for(entries_bound[h], kThreads * kInsertPerThread, 32), kThreads, 0, st>>>(ia);
                 ctx->launches++;
             }
         }
         {
-            // rows were handed out at insert time, in discovery order: per-batch counts -> offsets, then every list
-            // entry (mini-batch, id, rank) goes to its place.  No sort, no second pass over the id tables.
-            ProfScope ps(ctx, PH_SAMPLE_PLACE, 2);
-            int32_t* off_next = d->node_off + (size_t)(h + 1) * (B + 1);
-            k_outer_offsets<<<1, 1024, 0, st>>>(d->hdr, h, B, k, batch_cnt + (size_t)h * B, off_next, d->cum, (int32_t)cap_batch, d->cap_nodes);
-            k_place_nodes_outer<<<grid, kThreads, 0, st>>>(d->hdr, d->newlist[0], id_bits, off_next, d->nodes, d->node_batch);
-            ctx->launches += 2;
-        }
-        if (!(smem_last && h == k - 1)) {   // (the last hop's shared-memory kernel leaves final rows)
-            ProfScope ps(ctx, PH_SAMPLE_RELABEL, 1);
-            k_relabel<<<grid, kThreads, 0, st>>>(d->hdr, h, d->hvals, d->ent_repr);
+            ProfScope ps(ctx, PH_SAMPLE_PLACE, 1);
+            PlaceArgs pa{d->hdr, h, d->newlist[0], id_bits, batch_cnt + (size_t)h * B, d->cap_nodes, d->nodes, d->node_batch,
+                         smem_hop ? nullptr : d->hvals, table_limit, d->ent_repr, B, k, d->cum, d->node_off, (int32_t)hdr_ints, d->ent_off,
+                         d->rowbase, d->d_ent_hop, d->h_stage_dev + summary_at};
+            const size_t sm = (size_t)B * sizeof(int32_t);   // 16 KiB at the largest number of mini-batches
+            const unsigned grid = blocks_for(std::max<int64_t>(nodes_bound[h + 1], smem_hop ? 0 : entries_bound[h]), kThreads, 8);
+            if (h == k - 1) k_place<true><<<grid + 1, kThreads, sm, st>>>(pa);
+            else k_place<false><<<grid, kThreads, sm, st>>>(pa);
             ctx->launches++;
         }
-        ctx->launches += 1 + 1;  // count, pick
-    }
-    {
-        ProfScope ps(ctx, PH_SAMPLE_FINAL, 1);
-        // (the summary goes to pinned host memory behind the kernels; mg_sample_many_end waits for it)
-        static_assert(sizeof(DenseHeader) % 4 == 0, "the header is copied as 32-bit words");
-        k_finalize<<<1, 1024, 0, st>>>(d->hdr, B, k, d->cum, d->node_off, d->ent_off, d->rowbase, d->d_ent_hop,
-                                       (int32_t)((sizeof(DenseHeader) + 3) / 4), d->h_pinned_dev);
-        ctx->launches++;
     }
     MG_CUDA(ctx, cudaGetLastError());
     return MG_OK;
@@ -1729,15 +1804,15 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     // capture it (again) otherwise.  Profiling runs the launches one by one (its events do not belong in a graph).
     SampleSignature sig;
     memset(&sig, 0, sizeof(sig));
-    sig.B = B; sig.k = k; sig.T = 0; sig.table_size = table_size; sig.cap_batch = cap_batch;   // (the device work does not depend on T)
+    sig.B = B; sig.k = k; sig.T_bound = T_bound; sig.table_size = table_size; sig.cap_batch = cap_batch;
     sig.cap_nodes = d->cap_nodes; sig.cap_entries = d->cap_entries; sig.n_nodes = ctx->n_nodes; sig.part_size = ctx->part_size;
     sig.inout = (inout ? 1 : 0) | (smem_last ? 2 + 4 * dedup_nb : 0);
     for (int h = 0; h < k; ++h) sig.fanouts[h] = fanouts[h];
-    const void* ptrs[] = {d->hdr, d->nodes, d->node_batch, d->ent_off, d->node_r0, d->node_deg, d->newlist[0], d->newlist[1],
-                          d->scan_tmp, d->sort_hist, d->ent_nbrs, d->ent_repr, d->hkeys, d->hvals, d->node_off, d->cum, d->rowbase,
-                          d->d_ent_hop, d->d_seeds, d->h_stage_dev, d->h_pinned_dev, ctx->view_off, ctx->view_nbrs, ctx->d_slot_of_part, st, ctx->d_part_of_node,
-                          inout ? (const void*)ctx->view_off_out : nullptr, inout ? (const void*)ctx->view_nbrs_out : nullptr,
-                          d->node_r0_out, d->node_deg_out, d->pairs, d->share_off};
+    const void* ptrs[] = {d->hdr, d->nodes, d->node_batch, d->ent_off, d->tile_state, d->newlist[0], d->newlist[1],
+                          d->ent_nbrs, d->ent_repr, d->hkeys, d->hvals, d->node_off, d->cum, d->rowbase, d->batch_cnt,
+                          d->d_ent_hop, d->d_seeds, d->h_stage_dev, d->h_stage_dev + summary_at, ctx->view_off, ctx->view_nbrs, ctx->d_slot_of_part, st,
+                          ctx->d_part_of_node, inout ? (const void*)ctx->view_off_out : nullptr, inout ? (const void*)ctx->view_nbrs_out : nullptr,
+                          d->pairs, d->share_off};
     static_assert(sizeof(ptrs) <= sizeof(sig.ptrs), "signature too small");
     memcpy(sig.ptrs, ptrs, sizeof(ptrs));
     const bool use_graph = ctx->sample_graphs && !ctx->prof_on && !getenv("MG_NO_SAMPLE_GRAPH");
@@ -2000,13 +2075,12 @@ extern "C" int mg_dense_free(mg_dense* d) {
     if (!d) return MG_OK;
     cudaSetDevice(d->device);
     if (d->ctx && d->ctx->last_fwd_dense == d) d->ctx->last_fwd_dense = nullptr;
-    cudaFree(d->hdr); cudaFree(d->nodes); cudaFree(d->node_batch); cudaFree(d->ent_off); cudaFree(d->node_r0); cudaFree(d->node_deg); cudaFree(d->node_r0_out); cudaFree(d->node_deg_out); cudaFree(d->pairs); cudaFree(d->share_off);
+    cudaFree(d->hdr); cudaFree(d->nodes); cudaFree(d->node_batch); cudaFree(d->ent_off); cudaFree(d->tile_state); cudaFree(d->pairs); cudaFree(d->share_off);
     cudaFree(d->ent_nbrs); cudaFree(d->ent_repr); cudaFree(d->node_off); cudaFree(d->cum);
     cudaFree(d->rowbase); cudaFree(d->hkeys); cudaFree(d->hvals); cudaFree(d->newlist[0]);
     cudaFree(d->newlist[1]); cudaFree(d->d_seeds); cudaFree(d->batch_cnt); cudaFree(d->scan_tmp); cudaFree(d->sort_hist); cudaFree(d->seg_tiles);
     cudaFree(d->exp_buf); cudaFree(d->perm_buf); cudaFree(d->d_ent_hop); cudaFree(d->expm_buf);
     if (d->ev_exported) cudaEventDestroy(d->ev_exported);
-    if (d->h_pinned) cudaFreeHost(d->h_pinned);
     if (d->h_stage) cudaFreeHost(d->h_stage);
     if (d->graph_exec) cudaGraphExecDestroy(d->graph_exec);
     if (d->ev_sampled) cudaEventDestroy(d->ev_sampled);
