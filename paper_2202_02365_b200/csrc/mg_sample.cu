@@ -16,6 +16,7 @@
 #include <stdarg.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 
 #include "mg_device.cuh"
@@ -609,11 +610,14 @@ __global__ void __launch_bounds__(kThreads, 6) k_insert(InsertArgs a) {
 // enters its bucket's earlier nodes, then its bucket's entries from every share (dense), ranks its new nodes (a scan over
 // the table, no atomics), takes a run of the mini-batch's rows and of the list of new nodes with ONE global atomic
 // each, and gives every entry its node's row.
-// (measured on the bench's last hop: 512 threads x 13,312 slots x 32 buckets and 512 x 6,656 x 64 take the same time)
-constexpr int kDedupThreads = 1024;
+// Both are bound by instruction issue and shared-memory round trips, so the number of buckets follows from how evenly the
+// blocks fill the SMs (dedup_buckets): 4 blocks for one mini-batch of 53,000 nodes left 144 SMs idle (25 + 52 us against 6 + 17
+// with 64), 37 mini-batches of 63,000 nodes go from 84 + 29 to 68 + 22 us, 128 of 95,000 from 285 to 273 us.
 constexpr int kDedupMaxSlots = 26624;    // 208 KiB of keys + rows per block
-constexpr int kDedupMaxBuckets = 16;
+constexpr int kDedupMaxBuckets = 64;
+constexpr int kDedupMaxTables = 16;      // largest tables that a mini-batch may need
 constexpr int kBucketThreads = 512;
+constexpr int kDedupSlots512 = 6656, kDedupSlots256 = 3328;   // tables up to this size: blocks of 512 / 256 threads
 
 struct DedupArgs {
     DenseHeader* hdr;
@@ -636,11 +640,35 @@ struct DedupArgs {
     int64_t node_pairs0;
 };
 
-// bucket and first slot of an id: one multiplicative hash, the bucket from its top, the slot from what is left
-__device__ __forceinline__ uint32_t dedup_bucket(int32_t id, uint32_t nb) { return __umulhi((uint32_t)id * 0x9E3779B1u, nb); }
-__device__ __forceinline__ uint32_t dedup_slot(int32_t id, uint32_t nb, uint32_t S) {
-    return __umulhi((uint32_t)id * 0x9E3779B1u * nb, S);
+// Buckets per mini-batch: work of the SM with the most blocks, in mini-batches, plus 0.004 of one for every block's fixed cost
+// (at least min_nb, so that a bucket's table fits a block; at most 64, and no buckets of fewer than 256 nodes).
+int dedup_buckets(int64_t B, int64_t cap_batch, int64_t min_nb, int n_sms) {
+    const int64_t max_nb = std::max<int64_t>(min_nb, std::min<int64_t>(kDedupMaxBuckets, cap_batch / 256));
+    int64_t best = min_nb;
+    double best_cost = 1e30;
+    for (int64_t nb = min_nb; nb <= max_nb; ++nb) {
+        const double per_sm = (double)((B * nb + n_sms - 1) / n_sms);
+        const double cost = per_sm / (double)nb + 0.004 * per_sm;
+        if (cost < best_cost - 1e-9) { best_cost = cost; best = nb; }
+    }
+    return (int)best;
 }
+
+// slots of a bucket's table: its share of the nodes plus a twelfth plus eight standard deviations of how a hash fills buckets
+int64_t dedup_slots_for(int64_t nodes) {
+    return ((nodes * 13 + 11) / 12 + 8 * (int64_t)std::sqrt((double)nodes) + 64 + 127) / 128 * 128;
+}
+
+// Bucket and first slot of an id: one hash, the bucket from its top, the slot from what is left.  (A multiplication alone puts
+// the multiples of some strides next to each other -- a table for one bucket of 64 would overflow where one of seven did not
+// --, so its upper half is folded into the lower and multiplied again.)
+__device__ __forceinline__ uint32_t dedup_hash(int32_t id) {
+    uint32_t h = (uint32_t)id * 0x9E3779B1u;
+    h ^= h >> 16;
+    return h * 0x85EBCA6Bu;
+}
+__device__ __forceinline__ uint32_t dedup_bucket(int32_t id, uint32_t nb) { return __umulhi(dedup_hash(id), nb); }
+__device__ __forceinline__ uint32_t dedup_slot(int32_t id, uint32_t nb, uint32_t S) { return __umulhi(dedup_hash(id) * nb, S); }
 
 __global__ void __launch_bounds__(kBucketThreads) k_bucket_entries(DedupArgs a) {
     constexpr int kWarps = kBucketThreads / 32;
@@ -695,10 +723,14 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_entries(DedupArgs a) 
             base[threadIdx.x] = run;
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t run = 0;
-            for (uint32_t q = 0; q < nb; ++q) { const uint32_t c = base[q]; base[q] = run; run += c; }
-            base[nb] = run;
+        if (warp == 0) {   // (two buckets per lane)
+            const uint32_t q0 = 2u * (threadIdx.x & 31), q1 = q0 + 1;
+            const uint32_t c0 = q0 < nb ? base[q0] : 0u, c1 = q1 < nb ? base[q1] : 0u;
+            const uint32_t before = warp_incl_scan(c0 + c1) - c0 - c1;
+            __syncwarp();
+            if (q0 <= nb) base[q0] = before;
+            if (q1 <= nb) base[q1] = before + c0;
+            if (q1 + 1 == nb) base[nb] = before + c0 + c1;
         }
         __syncthreads();
         const int64_t dst0 = out0 + (s_lo - first);
@@ -720,6 +752,7 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_entries(DedupArgs a) 
     }
 }
 
+template <int kDedupThreads>
 __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
     extern __shared__ int32_t dedup_sm[];
     __shared__ uint32_t row_base, list_base, warp_tot[kDedupThreads / 32];
@@ -739,10 +772,15 @@ __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
         run_start[which][r + 1] = so[1] - so[0];
     }
     __syncthreads();
-    if (threadIdx.x < 2) {   // ... and their lengths' prefix
-        int32_t run = 0;
-        for (uint32_t r = 0; r < nb; ++r) { const int32_t c = run_start[threadIdx.x][r + 1]; run_start[threadIdx.x][r] = run; run += c; }
-        run_start[threadIdx.x][nb] = run;
+    if (warp < 2) {   // ... and their lengths' prefix (two shares per lane)
+        int32_t* rs = run_start[warp];
+        const uint32_t r0 = 2u * lane, r1 = r0 + 1;
+        const uint32_t c0 = r0 < nb ? (uint32_t)rs[r0 + 1] : 0u, c1 = r1 < nb ? (uint32_t)rs[r1 + 1] : 0u;
+        const uint32_t end = warp_incl_scan(c0 + c1);
+        __syncwarp();
+        if (r0 < nb) rs[r0 + 1] = (int32_t)(end - c1);
+        if (r1 < nb) rs[r1 + 1] = (int32_t)end;
+        if (lane == 0) rs[0] = 0;
     }
     __syncthreads();
     auto pair_at = [&](int which, int32_t i) -> int2* {   // i-th pair of the bucket: which share's run it falls in (run_start ascends)
@@ -1561,7 +1599,8 @@ static void sample_kernel_attributes() {
     static bool done = false;
     if (done) return;
     cudaFuncSetAttribute(k_radix_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
-    cudaFuncSetAttribute(k_dedupe_last, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kDedupMaxSlots * 2 * sizeof(int32_t)));
+    cudaFuncSetAttribute(k_dedupe_last<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kDedupMaxSlots * 2 * sizeof(int32_t)));
+    cudaFuncSetAttribute(k_dedupe_last<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDedupSlots512 * 2 * (int)sizeof(int32_t));
     cudaFuncSetAttribute(k_hop<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + kTileMax * hop_node_bytes(true));
     done = true;
@@ -1625,11 +1664,13 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     // its traffic is random 32-byte sectors, so every slot that is not needed costs DRAM bandwidth
     // (sized below, once it is known whether the last hop goes through it)
     // The last hop is deduplicated in shared memory (k_bucket_entries, k_dedupe_last) when a mini-batch's nodes fit the
-    // tables of a few blocks: S slots per block, filled to 92 % at most when the mini-batch is at its capacity (the
-    // buckets of a hash differ by a per cent or so at these sizes), nb blocks per mini-batch.
-    const int32_t dedup_slots = (int32_t)std::min<int64_t>(kDedupMaxSlots, (cap_batch + cap_batch / 4 + 64 + 1023) / 1024 * 1024);
-    const int64_t dedup_nb = (cap_batch + (cap_batch * 7 + 79) / 80 + dedup_slots - 1) / dedup_slots;
-    const bool smem_last = dedup_nb <= kDedupMaxBuckets && dedup_nb * n_batches < (1ll << 24) && cap_entries + cap_nodes < (1ll << 31) &&
+    // tables of 16 blocks.  Above, the global tables are the faster way (16 mini-batches of room for 480,000 nodes, 320,000 in
+    // use: the sample's kernels take 698 us with k_insert, 723 us with 20 and more blocks per mini-batch).
+    int64_t min_nb = (cap_batch + kDedupMaxSlots - 1) / kDedupMaxSlots;
+    while (min_nb <= kDedupMaxTables && dedup_slots_for((cap_batch + min_nb - 1) / min_nb) > kDedupMaxSlots) ++min_nb;
+    const int64_t dedup_nb = min_nb <= kDedupMaxTables ? dedup_buckets(n_batches, cap_batch, min_nb, ctx->n_sms) : min_nb;
+    const int32_t dedup_slots = (int32_t)std::min<int64_t>(dedup_slots_for((cap_batch + dedup_nb - 1) / dedup_nb), kDedupMaxSlots);
+    const bool smem_last = min_nb <= kDedupMaxTables && dedup_nb * n_batches < (1ll << 24) && cap_entries + cap_nodes < (1ll << 31) &&
                            !getenv("MG_GLOBAL_TABLES");
     // With the last hop deduplicated in shared memory the global tables only ever hold the nodes that are sampled from
     // (targets and the inner deltas): a caller who bounds those gets tables several times smaller.
@@ -1774,7 +1815,12 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
                              d->ent_repr, d->pairs, d->share_off, d->cum, batch_cnt + (size_t)h * B, d->newlist[0], d->cap_nodes,
                              id_bits, (int32_t)cap_batch, d->cap_entries};
                 k_bucket_entries<<<(unsigned)(B * dedup_nb), kBucketThreads, 0, st>>>(da);
-                k_dedupe_last<<<(unsigned)(B * dedup_nb), kDedupThreads, (size_t)dedup_slots * 2 * sizeof(int32_t), st>>>(da);
+                // (threads so that the blocks that shared memory lets onto an SM come to 2,048 threads)
+                const unsigned grid = (unsigned)(B * dedup_nb);
+                const size_t sm = (size_t)dedup_slots * 2 * sizeof(int32_t);
+                if (dedup_slots > kDedupSlots512) k_dedupe_last<1024><<<grid, 1024, sm, st>>>(da);
+                else if (dedup_slots > kDedupSlots256) k_dedupe_last<512><<<grid, 512, sm, st>>>(da);
+                else k_dedupe_last<256><<<grid, 256, sm, st>>>(da);
                 ctx->launches += 2;
             } else {
                 InsertArgs ia{d->hdr, h, d->ent_nbrs, d->ent_repr, d->hkeys, tg, d->newlist[0], d->cap_nodes, id_bits,

@@ -67,3 +67,34 @@ def test_hops_on_either_side_of_the_tile_sizes(graph, ctx, total):
         assert torch.equal(getattr(x, key), getattr(y, key)), key
     d.free()
     one.free()
+
+
+# buckets of the last hop: one (a table of a few hundred nodes), several with tables for blocks of 256, 512 and 1,024 threads, as
+# many tables as a mini-batch may need, and more (through the global tables); ids that are multiples of a Fibonacci
+# number, whose multiplicative hashes lie next to each other
+@pytest.mark.parametrize("room,n_batches", [(300, 1), (12_000, 1), (N, 1), (N, 60), (4_000, 160), (370_000, 2), (420_000, 2)])
+def test_last_hop_buckets(graph, ctx, room, n_batches):
+    off, nbrs = graph.row_offsets.numpy(), graph.nbrs.numpy()
+    per = max(1, min(room // 45, 2_000))
+    ids = torch.arange(0, N, 987, dtype=torch.int32)
+    rows = [torch.cat([ids[:min(per, len(ids)) // 2], torch.tensor([1], dtype=torch.int32)])]
+    rows += [inputs.distinct_targets(N, per, seed=b) for b in range(1, n_batches)]
+    offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    caps = {"max_nodes_per_batch": room, "max_nodes_total": 45 * per * n_batches + 256, "max_entries_total": 48 * per * n_batches + 256}
+    d = ctx.sample_many(torch.cat(rows), offs, [4, 5], list(range(n_batches)), caps=caps)
+    nodes, entries = d.counts()
+    for b in (0, n_batches - 1):
+        v = d.view(b)
+        ids_b, rep, o = v.node_ids.cpu().numpy(), v.repr_map.cpu().numpy(), v.nbr_offsets.cpu().numpy()
+        got = v.nbrs.cpu().numpy()
+        assert len(np.unique(ids_b)) == len(ids_b) == int(nodes[b].sum())
+        assert np.array_equal(ids_b[rep], got)
+        src = ids_b[len(ids_b) - (len(o) - 1):]          # the sampled nodes, in order
+        cnt = np.diff(o)
+        deg = off[src + 1] - off[src]
+        n0 = len(ids_b) - len(src)
+        hop = np.where(np.arange(len(src)) >= len(src) - int(nodes[b, 0]), 4, 5)
+        assert n0 == int(nodes[b, 2]) and np.array_equal(cnt, np.minimum(deg, hop))
+        first = np.unique(got)                           # every node is a target or somebody's neighbour
+        assert np.array_equal(np.unique(np.concatenate([first, rows[b].numpy()])), np.sort(ids_b))
+    d.free()
