@@ -1,0 +1,94 @@
+"""The backward pass at the sizes where its gather is cut differently: source rows named by none, a few, tens and hundreds of
+entries (a star graph's centre), widths of one to eight column blocks; against the layers' definition in fp64."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2202_02365_b200 as mg
+from paper_2202_02365_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+N = 6_000
+
+
+def star_graph():
+    """Node v aggregates from the centres 0 .. 3 by its id's divisors and from two nodes of a random graph; 0 from 20 others."""
+    g = torch.Generator().manual_seed(3)
+    v = torch.arange(4, N)
+    dst = [v, v[::5], v[::40], v[::300], v, v, torch.zeros(20, dtype=torch.int64)]
+    src = [torch.full_like(x, c) for c, x in enumerate(dst[:4])]
+    src += [torch.randint(4, N, (len(v),), generator=g) for _ in range(2)] + [torch.arange(100, 120)]
+    return inputs.build_csr(torch.cat(src), torch.cat(dst), N)
+
+
+def reference(views, feats, layers, d_outs, aggregator):
+    """Loss sum(d_out * H^k) differentiated by torch in fp64: weight gradients, and the rows' gradients by (mini-batch, node)."""
+    params = [[p.double().requires_grad_() for p in layer] for layer in layers]
+    rows, loss = [], 0.0
+    for v, d_out in zip(views, d_outs):
+        ids, nio = v.node_ids.cpu().long(), v.node_id_offsets.cpu().tolist()
+        rep, off = v.repr_map.cpu().long(), v.nbr_offsets.cpu().long()
+        h = feats[ids].double().requires_grad_()
+        rows.append((ids, h))
+        for l, (ws, wn, b) in enumerate(params):
+            first = nio[l + 1] - nio[l]                  # rows of the farthest delta that is left: inputs only
+            drop = nio[l + 1] - nio[1]                   # sampled nodes that are inputs only by now
+            n_out = h.shape[0] - first
+            lo, hi = off[drop], off[drop + n_out]
+            cnt = off[drop + 1:drop + n_out + 1] - off[drop:drop + n_out]
+            dst = torch.repeat_interleave(torch.arange(n_out), cnt)
+            agg = torch.zeros((n_out, h.shape[1]), dtype=torch.float64).index_add(0, dst, h[rep[lo:hi] - nio[l]])
+            if aggregator == "mean":
+                agg = agg / cnt.clamp(min=1).double()[:, None]
+            h = h[first:] @ ws + agg @ wn + b
+            if l + 1 < len(params):
+                h = torch.relu(h)
+        loss = loss + (h * d_out.double().cpu()).sum()
+    loss.backward()
+    return params, rows
+
+
+@pytest.mark.parametrize("dims,fanouts,aggregator", [([16, 8], [6], "mean"), ([132, 128, 12], [6, 4], "mean"), ([16, 260, 8], [6, 6], "sum"),
+                                                     ([1024, 516, 4], [5, 6], "mean")])
+def test_source_rows_named_by_few_and_by_many(dims, fanouts, aggregator):
+    graph = star_graph()
+    feats = inputs.normal_features(N, dims[0], seed=4)
+    layers = inputs.random_bias_layers(dims, seed=5)
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(feats.cuda())
+    ctx.keep_layer_outputs(True)
+    sizes = [700, 0, 1, 90]
+    targets = torch.cat([inputs.distinct_targets(N, s, seed=8 + i) for i, s in enumerate(sizes)])
+    offs = np.concatenate([[0], np.cumsum(sizes)])
+    dense = ctx.sample_many(targets, offs, fanouts, [1, 2, 3, 4])
+    model = ctx.model(layers, mg.GEMM_FP32)
+    model.set_aggregator(aggregator)
+    out = torch.empty((len(targets), dims[-1]), device="cuda")
+    ctx.forward(model, dense, out)
+    d_out = torch.randn(out.shape, generator=torch.Generator("cuda").manual_seed(6), device="cuda")
+    grads, g_rows, ids = ctx.backward(model, dense, d_out, want_h0_grad=True)
+    views = [dense.view(b) for b in range(len(sizes))]
+    params, rows = reference(views, feats, layers, [d_out[offs[b]:offs[b + 1]] for b in range(len(sizes))], aggregator)
+
+    # fp32 sums of up to 800 rows x 700 entries' products in any order: sqrt(n) 2^-24 of the terms' norm, below 1e-5; where terms
+    # cancel the result's norm is smaller, hence 1e-4
+    def near(x, y):
+        return float((x.double().cpu() - y).norm()) <= 1e-4 * max(float(y.norm()), 1e-12)
+
+    for got, want in zip(grads, params):
+        for x, p in zip(got, want):
+            assert near(x.reshape(p.shape), p.grad)
+    at = 0
+    nodes, _ = dense.counts()
+    for b, (want_ids, h) in enumerate(rows):
+        n = int(nodes[b].sum())
+        order = torch.argsort(ids[at:at + n].cpu())
+        want = torch.argsort(want_ids)
+        assert torch.equal(ids[at:at + n].cpu()[order].long(), want_ids[want])
+        if n:
+            assert near(g_rows[at:at + n].cpu()[order], h.grad[want])
+            for i in torch.nonzero(want_ids[want] < 4).flatten().tolist():      # the centres' rows one by one
+                assert near(g_rows[at:at + n].cpu()[order][i], h.grad[want][i])
+        at += n
