@@ -411,7 +411,8 @@ int mg_profile_read(mg_ctx* ctx, int32_t* n_phases, const char** names, double* 
 int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, float* d_h0_dev);
 
 /* DEVICE pointers to the gradients mg_backward left for layer `layer` (1..k): d_w_self and d_w_nbr row-major
- * [dims[layer-1], dims[layer]], d_bias [dims[layer]].  Owned by the model.  Errors: MG_ERR_ARG, MG_ERR_STATE. */
+ * [dims[layer-1], dims[layer]], d_bias [dims[layer]].  Owned by the model; one block, layer after layer d_w_self, d_w_nbr,
+ * d_bias, so that layer 1's d_w_self is the start of all of them.  Errors: MG_ERR_ARG, MG_ERR_STATE. */
 int mg_model_grads(const mg_model* m, int32_t layer, const float** d_w_self, const float** d_w_nbr, const float** d_bias);
 
 /* One step of stochastic gradient descent on every weight and bias of the model with the gradients of the last

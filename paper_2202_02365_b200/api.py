@@ -435,14 +435,13 @@ class Context:
         n_rows = int(nodes.sum())
         g_h0 = torch.empty((n_rows, model.dims[0]), dtype=torch.float32, device=d_out.device) if want_h0_grad else None
         self._check(self.lib.mg_backward(self.handle, model.handle, dense.handle, _ptr(d_out), _ptr(g_h0)))
-        grads = []
-        for l in range(1, len(model.dims)):
-            ps, pn, pb = C.c_void_p(0), C.c_void_p(0), C.c_void_p(0)
-            self._check(self.lib.mg_model_grads(model.handle, C.c_int32(l), C.byref(ps), C.byref(pn), C.byref(pb)))
-            di, dn = model.dims[l - 1], model.dims[l]
-            grads.append((_from_dev_f32(ps.value, di * dn, d_out.device).view(di, dn).clone(),
-                          _from_dev_f32(pn.value, di * dn, d_out.device).view(di, dn).clone(),
-                          _from_dev_f32(pb.value, dn, d_out.device).clone()))
+        # the library keeps the gradients of all layers in one block: one copy of it, handed out in pieces
+        base = C.c_void_p(0)
+        self._check(self.lib.mg_model_grads(model.handle, C.c_int32(1), C.byref(base), None, None))
+        sizes = [n for di, dn in zip(model.dims[:-1], model.dims[1:]) for n in (di * dn, di * dn, dn)]
+        pieces = _from_dev_f32(base.value, sum(sizes), d_out.device).clone().split(sizes)
+        grads = [(pieces[3 * l].view(di, dn), pieces[3 * l + 1].view(di, dn), pieces[3 * l + 2])
+                 for l, (di, dn) in enumerate(zip(model.dims[:-1], model.dims[1:]))]
         if not want_h0_grad:
             return grads
         ids = torch.empty(n_rows, dtype=torch.int32, device=d_out.device)

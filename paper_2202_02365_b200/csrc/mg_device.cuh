@@ -81,6 +81,12 @@ __device__ __forceinline__ int upper_segment(const int32_t* arr, int n, int32_t 
     return lo;
 }
 
+// Where input column `col` of a layer (part 0: its self weight, 1: its neighbour weight) stands in the K order of the fused layer
+// kernel: groups of `gc` columns, inside a group (self, neighbour) pairs of blocks of `kce` columns.
+__device__ __forceinline__ int fused_k_place(int part, int col, int kce, int gc) {
+    return col / gc * 2 * gc + col % gc / kce * 2 * kce + part * kce + col % kce;
+}
+
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
     const int lane = threadIdx.x & 31;
 #pragma unroll

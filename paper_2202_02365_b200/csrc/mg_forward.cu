@@ -21,8 +21,6 @@ int mg_gemm_tf32(mg_ctx* ctx, const float* x, const float* w_t, const float* bia
 int mg_gemm_tf32_status(mg_ctx* ctx);
 int mg_gemm_tf32_splitk_add_rows(mg_ctx* ctx, const float* x, const float* g, float* out, int M, int N, int64_t K, int kt_per_slice);
 // mg_layer_fused.cu
-int mg_pack_layer_weights(mg_ctx* ctx, const float* w_cat_dev, float* w_pad_t_dev, int d_in, int N);
-int mg_pack_layer_weights_f16(mg_ctx* ctx, const float* w_cat_dev, void* w_pad_h_dev, int d_in, int N);
 bool mg_layer_fused_supported(int d_in, int d_out);
 int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int4* meta, const int64_t* start /* [k + 2], layer l at start[l] */);
 int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* w_pad_t, const float* bias,
@@ -271,12 +269,76 @@ __global__ void __launch_bounds__(kThreads) k_gather_h0(H0Args a, float* __restr
     }
 }
 
-__global__ void k_transpose(const float* __restrict__ in, float* __restrict__ out, int rows, int cols, int round_tf32) {
-    const int64_t n = (int64_t)rows * cols;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(i / cols), c = (int)(i % cols);
-        const float v = in[i];
-        out[(int64_t)c * rows + r] = round_tf32 ? to_tf32(v) : v;
+// ---- weights: the optimisers' steps and the copies that the kernels read ------------------------------------------------
+// One launch for all layers: a block takes 32 rows x 32 columns of a layer's [W_self; W_nbr], applies the step, and writes the
+// tile into every copy -- the plain transpose, and the padded K orders of the fused layer kernel -- along the copies' rows.
+// (Five launches per layer before: 15 of 2 to 4 us and the gaps between them for three layers.)
+enum { W_COPY = 0, W_SGD = 1, W_ADAGRAD = 2 };
+struct WeightArgs {
+    int32_t k;
+    int32_t tile_at[MG_MAX_HOPS + 1];   // first tile of the layer; a block per layer for the biases behind the tiles
+    int32_t d_in[MG_MAX_HOPS], d_out[MG_MAX_HOPS];
+    float* w[MG_MAX_HOPS];
+    float* w_t[MG_MAX_HOPS];
+    float* w_pad[MG_MAX_HOPS];
+    __half* w_pad_h[MG_MAX_HOPS];       // null: none
+    float* bias[MG_MAX_HOPS];
+    int64_t g_at[MG_MAX_HOPS];          // the layer's place in the gradient block and the optimiser's state
+    const float* g;
+    float* state;
+    float lr, eps;
+    int32_t round_tf32;                 // w_t holds TF32 values
+};
+
+// SGD: w -= lr * g; Adagrad: state += g^2, w -= lr * g / (sqrt(state) + eps)
+template <int MODE>
+__device__ __forceinline__ float weight_step(const WeightArgs& a, float w, int64_t at) {
+    if (MODE == W_COPY) return w;
+    const float g = a.g[at];
+    if (MODE == W_SGD) return w - a.lr * g;
+    const float s = a.state[at] + g * g;
+    a.state[at] = s;
+    return w - a.lr * g / (sqrtf(s) + a.eps);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kThreads) k_weights(WeightArgs a) {
+    __shared__ float tile[32][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t = (int)blockIdx.x;
+    if (t >= a.tile_at[a.k]) {
+        const int l = t - a.tile_at[a.k];
+        const int64_t g0 = a.g_at[l] + 2 * (int64_t)a.d_in[l] * a.d_out[l];
+        for (int n = threadIdx.x; n < a.d_out[l]; n += kThreads) a.bias[l][n] = weight_step<MODE>(a, a.bias[l][n], g0 + n);
+        return;
+    }
+    int l = 0;
+    while (t >= a.tile_at[l + 1]) ++l;
+    const int di = a.d_in[l], dn = a.d_out[l];
+    const int col_blocks = (di + 31) / 32, n_blocks = (dn + 31) / 32;
+    int q = t - a.tile_at[l];
+    const int n0 = q % n_blocks * 32;
+    q /= n_blocks;
+    const int c0 = q % col_blocks * 32, part = q / col_blocks;   // 32 input columns of the self (0) or the neighbour (1) weights
+    for (int r = warp; r < 32; r += kThreads / 32) {
+        const int c = c0 + r, n = n0 + lane;
+        float w = 0.f;
+        if (c < di && n < dn) {
+            const int64_t i = (int64_t)(part * di + c) * dn + n;
+            w = weight_step<MODE>(a, a.w[l][i], a.g_at[l] + i);
+            if (MODE != W_COPY) a.w[l][i] = w;
+        }
+        tile[r][lane] = w;
+    }
+    __syncthreads();
+    const int pad32 = (di + kPackCols32 - 1) / kPackCols32 * kPackCols32, pad16 = (di + kPackCols16 - 1) / kPackCols16 * kPackCols16;
+    for (int r = warp; r < 32; r += kThreads / 32) {
+        const int c = c0 + lane, n = n0 + r;
+        if (c >= di || n >= dn) continue;
+        const float w = tile[lane][r], w32 = to_tf32(w);
+        a.w_t[l][(int64_t)n * 2 * di + part * di + c] = a.round_tf32 ? w32 : w;
+        a.w_pad[l][(int64_t)n * 2 * pad32 + fused_k_place(part, c, kPackCols32, kPackGroup32)] = w32;
+        if (a.w_pad_h[l]) a.w_pad_h[l][(int64_t)n * 2 * pad16 + fused_k_place(part, c, kPackCols16, kPackGroup16)] = __float2half_rn(w);
     }
 }
 
@@ -314,6 +376,26 @@ void fill_row_export(const mg_dense* d, int batch, int first_delta, int dim, Row
 
 }  // namespace
 
+// A model's weights: MODE's step, then every copy, on ctx's stream
+template <int MODE>
+static void launch_weights(mg_ctx* ctx, mg_model* m, float lr, float eps) {
+    WeightArgs a;
+    memset(&a, 0, sizeof(a));
+    a.k = m->k;
+    int64_t at = 0;
+    for (int l = 0; l < m->k; ++l) {
+        const int di = m->dims[l], dn = m->dims[l + 1];
+        a.tile_at[l + 1] = a.tile_at[l] + 2 * ((di + 31) / 32) * ((dn + 31) / 32);
+        a.d_in[l] = di; a.d_out[l] = dn;
+        a.w[l] = m->w_cat[l]; a.w_t[l] = m->w_cat_t[l]; a.w_pad[l] = m->w_pad_t[l]; a.w_pad_h[l] = static_cast<__half*>(m->w_pad_h[l]); a.bias[l] = m->bias[l];
+        a.g_at[l] = at;
+        at += 2 * (int64_t)di * dn + dn;
+    }
+    a.g = m->g_block; a.state = m->s_block; a.lr = lr; a.eps = eps; a.round_tf32 = m->precision == MG_GEMM_TF32;
+    k_weights<MODE><<<a.tile_at[m->k] + m->k, kThreads, 0, ctx->stream>>>(a);
+    ctx->launches++;
+}
+
 // ---------------------------------------------------------------------------------------
 extern "C" int mg_model_create(mg_ctx* ctx, int32_t k, const int32_t* dims, const float* const* w_self,
                                const float* const* w_nbr, const float* const* bias, int gemm_precision, mg_model** out) {
@@ -345,11 +427,7 @@ extern "C" int mg_model_create(mg_ctx* ctx, int32_t k, const int32_t* dims, cons
         cudaMemcpyAsync(m->w_cat[l], w_self[l], sizeof(float) * di * dn, cudaMemcpyHostToDevice, ctx->stream);
         cudaMemcpyAsync(m->w_cat[l] + di * dn, w_nbr[l], sizeof(float) * di * dn, cudaMemcpyHostToDevice, ctx->stream);
         cudaMemcpyAsync(m->bias[l], bias[l], sizeof(float) * dn, cudaMemcpyHostToDevice, ctx->stream);
-        // K-major copy [d_out, 2 d_in], rounded to nearest TF32 once, for the tensor-core path
-        k_transpose<<<mg_grid(ctx, 2), kThreads, 0, ctx->stream>>>(m->w_cat[l], m->w_cat_t[l], (int)(2 * di), (int)dn,
-                                                                  gemm_precision == MG_GEMM_TF32);
-        ctx->launches++;
-        mg_pack_layer_weights(ctx, m->w_cat[l], m->w_pad_t[l], (int)di, (int)dn);
+        cudaMemsetAsync(m->w_pad_t[l], 0, sizeof(float) * 2 * ((di + 31) / 32 * 32) * dn, ctx->stream);   // (the padding stays zero)
     }
     // Every layer's weights in fp16 form too, for layers whose input rows are fp16 (layer 1 over fp16 base
     // representations; later layers when the model stores its intermediate outputs as fp16).  fp16 keeps the 10-bit
@@ -371,8 +449,10 @@ extern "C" int mg_model_create(mg_ctx* ctx, int32_t k, const int32_t* dims, cons
             mg_model_free(m);
             return mg_fail(ctx, MG_ERR_OOM, "weight allocation failed");
         }
-        mg_pack_layer_weights_f16(ctx, m->w_cat[l], m->w_pad_h[l], (int)di, (int)dn);
+        cudaMemsetAsync(m->w_pad_h[l], 0, sizeof(uint16_t) * 2 * ((di + 63) / 64 * 64) * dn, ctx->stream);
     }
+    // K-major copies [d_out, 2 d_in], rounded to nearest TF32 once, for the tensor-core path
+    launch_weights<W_COPY>(ctx, m, 0.f, 0.f);
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { mg_model_free(m); return mg_cuda_fail(ctx, e, "weight upload"); }
@@ -399,9 +479,8 @@ extern "C" int mg_model_free(mg_model* m) {
     cudaSetDevice(m->device);
     for (int l = 0; l < MG_MAX_HOPS; ++l) {
         cudaFree(m->w_cat[l]); cudaFree(m->w_cat_t[l]); cudaFree(m->w_pad_t[l]); cudaFree(m->bias[l]);
-        cudaFree(m->g_w_cat[l]); cudaFree(m->g_bias[l]); cudaFree(m->s_w_cat[l]); cudaFree(m->s_bias[l]);
     }
-    cudaFree(m->zeros);
+    cudaFree(m->zeros); cudaFree(m->g_block); cudaFree(m->s_block);
     for (int l = 0; l < MG_MAX_HOPS; ++l) cudaFree(m->w_pad_h[l]);
     if (m->ctx && m->ctx->last_fwd_model == m) m->ctx->last_fwd_model = nullptr;
     delete m;
@@ -1119,10 +1198,6 @@ __global__ void __launch_bounds__(kThreads, MASK ? 4 : 1) k_grad_gather(GatherAr
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_sgd(float* w, const float* __restrict__ g, float lr, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) w[i] -= lr * g[i];
-}
-
 struct PackedIdArgs {
     RowGeom g;
     const int32_t* nodes;
@@ -1151,16 +1226,18 @@ extern "C" int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
     const int k = d->k, B = d->n_batches;
     cudaStream_t st = ctx->stream;
-    // gradient buffers of the model (allocated once), cleared for this pass
-    int widest2 = 8;
-    for (int l = 1; l <= k; ++l) widest2 = std::max(widest2, 2 * m->dims[l - 1]);
-    for (int l = 0; l < k; ++l) {
-        const size_t n_w = (size_t)2 * m->dims[l] * m->dims[l + 1], n_b = (size_t)m->dims[l + 1];
-        if (!m->g_w_cat[l] && cudaMalloc((void**)&m->g_w_cat[l], n_w * sizeof(float)) != cudaSuccess) { cudaGetLastError(); return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
-        if (!m->g_bias[l] && cudaMalloc((void**)&m->g_bias[l], n_b * sizeof(float)) != cudaSuccess) { cudaGetLastError(); return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
-        MG_CUDA(ctx, cudaMemsetAsync(m->g_w_cat[l], 0, n_w * sizeof(float), st));
-        MG_CUDA(ctx, cudaMemsetAsync(m->g_bias[l], 0, n_b * sizeof(float), st));
+    // gradient block of the model (allocated once), cleared for this pass
+    if (!m->g_block) {
+        m->g_elems = 0;
+        for (int l = 0; l < k; ++l) m->g_elems += (size_t)(2 * m->dims[l] + 1) * m->dims[l + 1];
+        if (cudaMalloc((void**)&m->g_block, m->g_elems * sizeof(float)) != cudaSuccess) { cudaGetLastError(); m->g_block = nullptr; return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
+        float* g = m->g_block;
+        for (int l = 0; l < k; ++l) {
+            m->g_w_cat[l] = g; g += (size_t)2 * m->dims[l] * m->dims[l + 1];
+            m->g_bias[l] = g; g += m->dims[l + 1];
+        }
     }
+    MG_CUDA(ctx, cudaMemsetAsync(m->g_block, 0, m->g_elems * sizeof(float), st));
     if (!m->zeros) {
         if (cudaMalloc((void**)&m->zeros, sizeof(float) * 2 * 1024) != cudaSuccess) { cudaGetLastError(); return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
         MG_CUDA(ctx, cudaMemsetAsync(m->zeros, 0, sizeof(float) * 2 * 1024, st));
@@ -1309,71 +1386,38 @@ extern "C" int mg_model_grads(const mg_model* m, int32_t layer, const float** d_
     return MG_OK;
 }
 
-namespace {
-// Adagrad: state += g^2; w -= lr * g / (sqrt(state) + eps)
-__global__ void __launch_bounds__(kThreads) k_adagrad(float* w, const float* __restrict__ g, float* state, float lr, float eps, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float s = state[i] + gi * gi;
-        state[i] = s;
-        w[i] -= lr * gi / (sqrtf(s) + eps);
-    }
-}
-}  // namespace
-
-// the copies of a layer's weights that the forward kernels read
-static int refresh_weight_copies(mg_ctx* ctx, mg_model* m, int l) {
-    const size_t di = m->dims[l], dn = m->dims[l + 1];
-    k_transpose<<<mg_grid(ctx, 2), kThreads, 0, ctx->stream>>>(m->w_cat[l], m->w_cat_t[l], (int)(2 * di), (int)dn, m->precision == MG_GEMM_TF32);
-    ctx->launches++;
-    if (m->w_pad_h[l]) mg_pack_layer_weights_f16(ctx, m->w_cat[l], m->w_pad_h[l], (int)di, (int)dn);
-    return mg_pack_layer_weights(ctx, m->w_cat[l], m->w_pad_t[l], (int)di, (int)dn);
+static int optimizer_checks(mg_ctx* ctx, const mg_model* m) {
+    if (!m || m->ctx != ctx) return mg_fail(ctx, MG_ERR_ARG, "bad model handle");
+    if (!m->g_block) return mg_fail(ctx, MG_ERR_STATE, "mg_backward has not run");
+    return MG_OK;
 }
 
 extern "C" int mg_model_adagrad_step(mg_ctx* ctx, mg_model* m, float lr, float eps) {
     if (!ctx) return MG_ERR_ARG;
-    if (!m || m->ctx != ctx) return mg_fail(ctx, MG_ERR_ARG, "bad model handle");
-    if (!m->g_w_cat[0]) return mg_fail(ctx, MG_ERR_STATE, "mg_backward has not run");
+    if (int rc = optimizer_checks(ctx, m)) return rc;
     if (!(eps > 0.f)) return mg_fail(ctx, MG_ERR_ARG, "eps must be positive");
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
-    cudaStream_t st = ctx->stream;
-    for (int l = 0; l < m->k; ++l) {
-        const size_t n_w = (size_t)2 * m->dims[l] * m->dims[l + 1], n_b = (size_t)m->dims[l + 1];
-        if (!m->s_w_cat[l]) {   // accumulated squared gradients start at zero
-            if (cudaMalloc((void**)&m->s_w_cat[l], n_w * sizeof(float)) != cudaSuccess || cudaMalloc((void**)&m->s_bias[l], n_b * sizeof(float)) != cudaSuccess) {
-                cudaGetLastError();
-                return mg_fail(ctx, MG_ERR_OOM, "optimizer state allocation failed");
-            }
-            MG_CUDA(ctx, cudaMemsetAsync(m->s_w_cat[l], 0, n_w * sizeof(float), st));
-            MG_CUDA(ctx, cudaMemsetAsync(m->s_bias[l], 0, n_b * sizeof(float), st));
+    if (!m->s_block) {   // accumulated squared gradients start at zero
+        if (cudaMalloc((void**)&m->s_block, m->g_elems * sizeof(float)) != cudaSuccess) {
+            cudaGetLastError();
+            m->s_block = nullptr;
+            return mg_fail(ctx, MG_ERR_OOM, "optimizer state allocation failed");
         }
-        k_adagrad<<<mg_grid(ctx, 2), kThreads, 0, st>>>(m->w_cat[l], m->g_w_cat[l], m->s_w_cat[l], lr, eps, (int64_t)n_w);
-        k_adagrad<<<1, kThreads, 0, st>>>(m->bias[l], m->g_bias[l], m->s_bias[l], lr, eps, (int64_t)n_b);
-        ctx->launches += 2;
-        const int rc = refresh_weight_copies(ctx, m, l);
-        if (rc) return rc;
+        MG_CUDA(ctx, cudaMemsetAsync(m->s_block, 0, m->g_elems * sizeof(float), ctx->stream));
     }
+    launch_weights<W_ADAGRAD>(ctx, m, lr, eps);
     MG_CUDA(ctx, cudaGetLastError());
-    MG_CUDA(ctx, cudaStreamSynchronize(st));
+    MG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return MG_OK;
 }
 
 extern "C" int mg_model_sgd_step(mg_ctx* ctx, mg_model* m, float lr) {
     if (!ctx) return MG_ERR_ARG;
-    if (!m || m->ctx != ctx) return mg_fail(ctx, MG_ERR_ARG, "bad model handle");
-    if (!m->g_w_cat[0]) return mg_fail(ctx, MG_ERR_STATE, "mg_backward has not run");
+    if (int rc = optimizer_checks(ctx, m)) return rc;
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
-    cudaStream_t st = ctx->stream;
-    for (int l = 0; l < m->k; ++l) {
-        const size_t di = m->dims[l], dn = m->dims[l + 1];
-        k_sgd<<<mg_grid(ctx, 2), kThreads, 0, st>>>(m->w_cat[l], m->g_w_cat[l], lr, (int64_t)(2 * di * dn));
-        k_sgd<<<1, kThreads, 0, st>>>(m->bias[l], m->g_bias[l], lr, (int64_t)dn);
-        ctx->launches += 2;
-        const int rc = refresh_weight_copies(ctx, m, l);
-        if (rc) return rc;
-    }
+    launch_weights<W_SGD>(ctx, m, lr, 0.f);
     MG_CUDA(ctx, cudaGetLastError());
-    MG_CUDA(ctx, cudaStreamSynchronize(st));
+    MG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return MG_OK;
 }
 

@@ -263,10 +263,12 @@ struct mg_model {
     bool f16_intermediates = false;   // store H^1 .. H^{k-1} as fp16 (mg_model_set_intermediates)
     float* bias[MG_MAX_HOPS] = {nullptr};
     // mg_backward: gradients of w_cat and bias (allocated by the first backward pass), a zero vector
+    // (one block: layer after layer its weights' gradients, then its bias's)
+    float* g_block = nullptr;
+    size_t g_elems = 0;
     float* g_w_cat[MG_MAX_HOPS] = {nullptr};
     float* g_bias[MG_MAX_HOPS] = {nullptr};
-    float* s_w_cat[MG_MAX_HOPS] = {nullptr};   // Adagrad: accumulated squared gradients
-    float* s_bias[MG_MAX_HOPS] = {nullptr};
+    float* s_block = nullptr;                  // Adagrad: accumulated squared gradients, laid out like them
     float* zeros = nullptr;
 };
 
@@ -346,6 +348,9 @@ static inline FeatGeom mg_feat_geom(const mg_ctx* ctx) {
     g.identity = ctx->backing == MG_BACKING_HBM ? 1 : 0;   // the whole table in device memory, in node order
     return g;
 }
+
+// K order of the fused layer kernel's weights (fused_k_place): columns per block and per group, TF32 and fp16 operands
+constexpr int kPackCols32 = 32, kPackGroup32 = 128, kPackCols16 = 64, kPackGroup16 = 256;
 
 // ---- generic device-sized scan and sort (mg_sample.cu) -------------------------------------
 struct SortParams {   // device-resident

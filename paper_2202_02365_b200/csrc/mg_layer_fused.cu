@@ -60,6 +60,8 @@ template <bool F16> struct Geo {
     static constexpr int kLaneCols = F16 ? 8 : 4;    // columns of a group one lane owns (16 bytes of operand)
     static constexpr int kGroup = 32 * kLaneCols;    // columns per group
 };
+static_assert(Geo<false>::kKC == kPackCols32 && Geo<false>::kGroup == kPackGroup32 && Geo<true>::kKC == kPackCols16 && Geo<true>::kGroup == kPackGroup16,
+              "the order the weights are packed in");
 constexpr int kRowsInFlight = 2;                 // rows a producer warp builds at the same time
 constexpr int kBlockRows = kProducerWarps * kRowsInFlight;   // 32: rows of a tile the producers build in one round
 constexpr int kBlocksPerTile = BM / kBlockRows;              // 4
@@ -814,26 +816,6 @@ __global__ void __launch_bounds__(256) k_layer_rows(RowsArgs a, int4* __restrict
     }
 }
 
-// slice order of the fused kernel: groups of kGroup input columns; inside a group (self, mean) pairs of kKC-column blocks
-template <bool F16>
-__global__ void k_pack_weights(const float* __restrict__ w_cat /*[2 d_in, N]*/, void* __restrict__ w_pad_t /*[N, 2 d_in_pad]*/,
-                               int d_in, int d_in_pad, int N) {
-    constexpr int KCE = Geo<F16>::kKC, GC = Geo<F16>::kGroup;
-    const int K = 2 * d_in_pad;
-    const int64_t total = (int64_t)N * K;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int n = (int)(i / K), kx = (int)(i % K);
-        const int slice = kx / KCE;
-        int grp = 0, rem = slice, pairs = min(GC / KCE, d_in_pad / KCE);
-        while (rem >= 2 * pairs) { rem -= 2 * pairs; ++grp; pairs = min(GC / KCE, (d_in_pad - grp * GC) / KCE); }
-        const int part = rem & 1;
-        const int col = grp * GC + (rem >> 1) * KCE + (kx % KCE);
-        const float w = col < d_in ? w_cat[(int64_t)(part * d_in + col) * N + n] : 0.f;
-        if (F16) reinterpret_cast<__half*>(w_pad_t)[i] = __float2half_rn(w);
-        else reinterpret_cast<float*>(w_pad_t)[i] = to_tf32(w);
-    }
-}
-
 // row-major [rows, K] fp16 matrix, boxes of 64 halves x box_rows, 128-byte swizzle, zero fill
 // the same matrix in boxes of 32 halves x 32 rows, not swizzled (the transposed epilogue's fp16 stores)
 static bool make_map_f16_box32(CUtensorMap* map, const void* base, int64_t rows, int K) {
@@ -860,23 +842,6 @@ static bool make_map_f16(CUtensorMap* map, const void* base, int64_t rows, int K
 }
 
 }  // namespace
-
-// K-major, zero-padded, TF32-rounded copy of [W_self ; W_nbr] for the fused layer kernel
-int mg_pack_layer_weights(mg_ctx* ctx, const float* w_cat_dev, float* w_pad_t_dev, int d_in, int N) {
-    const int d_in_pad = (d_in + KC - 1) / KC * KC;
-    k_pack_weights<false><<<mg_grid(ctx, 2), 256, 0, ctx->stream>>>(w_cat_dev, w_pad_t_dev, d_in, d_in_pad, N);
-    ctx->launches++;
-    return MG_OK;
-}
-
-// The same rounded to fp16 (64-column slices), [N, 2 * roundup64(d_in)] halves: the first layer's weights when the base
-// representations are fp16 and the layer's GEMM runs on fp16 operands
-int mg_pack_layer_weights_f16(mg_ctx* ctx, const float* w_cat_dev, void* w_pad_h_dev, int d_in, int N) {
-    const int d_in_pad = (d_in + 63) / 64 * 64;
-    k_pack_weights<true><<<mg_grid(ctx, 2), 256, 0, ctx->stream>>>(w_cat_dev, w_pad_h_dev, d_in, d_in_pad, N);
-    ctx->launches++;
-    return MG_OK;
-}
 
 bool mg_layer_fused_supported(int d_in, int d_out) { return d_out <= 256 && d_out % 4 == 0 && d_in % 4 == 0; }
 
