@@ -1374,6 +1374,26 @@ __global__ void __launch_bounds__(kThreads) k_export_many_entries(ExportManyArgs
     }
 }
 
+// the five arrays of one mini-batch, one behind the other (mg_dense_arrays_copy); blockIdx.y = array, four loads in flight
+struct ArraysCopy {
+    const int32_t* src[5];
+    int32_t len[5];
+};
+__global__ void __launch_bounds__(kThreads) k_copy_arrays(ArraysCopy a, int32_t* __restrict__ dst) {
+    const int q = blockIdx.y;
+    for (int p = 0; p < q; ++p) dst += a.len[p];
+    const int32_t* __restrict__ src = a.src[q];
+    const int32_t n = a.len[q];
+    for (int32_t i0 = blockIdx.x * 4 * kThreads + threadIdx.x; i0 < n; i0 += gridDim.x * 4 * kThreads) {
+        int32_t v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = i0 + u * kThreads < n ? src[i0 + u * kThreads] : 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i0 + u * kThreads < n) dst[i0 + u * kThreads] = v[u];
+    }
+}
+
 int ilog2_ceil(int64_t x) {
     int b = 0;
     while (((int64_t)1 << b) < x) ++b;
@@ -2114,6 +2134,20 @@ extern "C" int mg_dense_export_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_
     out->nbrs = d->expm_buf + L.nbrs + e_before;
     out->repr_map = d->expm_buf + L.repr + e_before;
     out->nbr_offsets = d->expm_buf + L.nbr_off + row0 + b;
+    return MG_OK;
+}
+
+extern "C" int mg_dense_arrays_copy(mg_ctx* ctx, const mg_dense_arrays* v, int32_t* dst_dev, void* stream) {
+    if (!ctx) return MG_ERR_ARG;
+    if (!v || !dst_dev) return mg_fail(ctx, MG_ERR_ARG, "null argument");
+    MG_CUDA(ctx, cudaSetDevice(ctx->device));
+    const ArraysCopy a{{v->node_ids, v->node_id_offsets, v->nbrs, v->nbr_offsets, v->repr_map},
+                       {v->n_nodes, v->k + 2, v->n_entries, v->n_sampled + 1, v->n_entries}};
+    const int longest = std::max(std::max(v->n_nodes, v->n_entries), v->n_sampled + 1);
+    const int blocks = std::max(1, std::min(mg_grid(ctx, 2), (longest + 4 * kThreads - 1) / (4 * kThreads)));
+    k_copy_arrays<<<dim3((unsigned)blocks, 5), kThreads, 0, (cudaStream_t)stream>>>(a, dst_dev);
+    ctx->launches++;
+    MG_CUDA(ctx, cudaGetLastError());
     return MG_OK;
 }
 
