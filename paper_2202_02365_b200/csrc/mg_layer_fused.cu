@@ -72,7 +72,13 @@ constexpr int kAccBufs = 4;                                  // accumulator buff
 constexpr int kSlicesPerGroup = 2 * kGroupCols / KC;         // 8 K slices: (self, mean) x four 32-column blocks
 constexpr int kUnroll = 5;                       // neighbour rows per output row fetched before the first add
 static_assert(kUnroll == 5, "the first-round table is read as four + one source rows");
-constexpr uint32_t kABytes = BM * KC * 4;  // 16 KiB per A stage
+// an A stage: a 128-byte slice row per row of the tile (16 or 8 KiB)
+__host__ __device__ constexpr uint32_t stage_bytes(int halves) { return (uint32_t)(HM * halves) * 128; }
+// Shared memory of a weight ring.  Two halves: shallow on purpose -- with 128 KB of A stages the CTA then fits the 196 KB
+// carve-out, which leaves the gathers twice the L1 (measured: layer 1 of the bench 2.92 -> 2.75 ms).  One half: what the
+// smaller A stages leave of the same carve-out.
+constexpr int ring_bytes(int halves) { return (halves == 1 ? 96 : 32) * 1024; }
+constexpr int fused_smem_limit(int halves) { return 8 * (int)stage_bytes(halves) + ring_bytes(halves) + 1024; }
 
 struct FusedArgs {
     // DENSE (device arrays of the sample)
@@ -188,11 +194,18 @@ template <> struct PieceSum<true> {
 // the pair, a CTA's 128 in its 128 lanes, K <= 256 columns), the gathered rows the second (N = 128: a half tile of either
 // CTA); the accumulator is the transposed output, [output column][row].  Nothing is streamed per half tile then -- with
 // the weights in shared memory a half tile waits for eight 16 KB slices through a two-stage ring (4 us of latency).
-template <bool FIRST, bool HALF, bool F16, bool TS = false>
+//
+// HALVES = 1: tiles of 64 rows per CTA (one half only) for layers of few rows.  Such a layer is one chain -- plan, gather, weight
+// slices, epilogue -- whose links are halved, on twice the CTAs, with six weight slices in flight instead of two (the operand
+// stages are half as large); layers of many rows want the second half, whose gather runs under the first half's MMAs.
+template <bool FIRST, bool HALF, bool F16, bool TS, int HALVES>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(MG_FUSED_MAXNREG)
 k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_out,
                    const __grid_constant__ CUtensorMap map_out2, FusedArgs a) {
     constexpr int KCE = Geo<F16>::kKC, GC = Geo<F16>::kGroup, LC = Geo<F16>::kLaneCols;
+    constexpr int TM = HM * HALVES;                          // rows of a tile
+    constexpr int kBlocks = kBlocksPerHalf * HALVES;         // row blocks of a tile
+    constexpr uint32_t kStage = stage_bytes(HALVES);
     extern __shared__ uint8_t smem_raw[];
     // a_ready and acc_empty are used in the leader CTA only (both CTAs arrive there); a_free, b_empty and acc_full
     // exist in both CTAs and are signalled in both by the leader's commits; b_full counts both halves' bytes in
@@ -217,9 +230,9 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
     const int half_n = a.BN / 2;                  // weight rows (output columns) this CTA stages
     const uint32_t b_bytes = (uint32_t)half_n * 128;   // one 128-byte slice row per staged output column
     uint8_t* a_base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* b_base = a_base + (size_t)a.sa * kABytes;
+    uint8_t* b_base = a_base + (size_t)a.sa * kStage;
     const int n_chunks = 2 * a.d_in_pad / KCE;
-    const int64_t n_tiles = (a.M - a.row_lo + BM - 1) / BM;
+    const int64_t n_tiles = (a.M - a.row_lo + TM - 1) / TM;
     const int64_t n_tile_pairs = (n_tiles + 1) / 2;
     // iteration `it` of this pair works on tile pair (pair + it * n_pairs): the leader on its even tile, the peer
     // on the odd one (which may lie past the end: then all its rows are padding)
@@ -303,7 +316,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
             // the weight slices of a group are streamed once per half tile, in the order the MMAs consume them
             for (uint32_t it = 0; it < my_iters && ok; ++it)
                 for (int grp = 0; grp < n_groups && ok; ++grp)
-                    for (int h = 0; h < 2 && ok; ++h) {
+                    for (int h = 0; h < HALVES && ok; ++h) {
                         const int gch = min(kSlicesPerGroup, n_chunks - grp * kSlicesPerGroup);
                         for (int c = 0; c < gch; ++c, ++cnt) {
                             const int s = cnt % a.sb;
@@ -324,15 +337,15 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
             if (!ok) report(a.error, 18u);
             tc_fence_after();
             for (uint32_t it = 0; it < my_iters && ok; ++it)
-                for (int h = 0; h < 2 && ok; ++h) {
-                    const uint32_t hu = it * 2 + h, buf = hu & 1;
+                for (int h = 0; h < HALVES && ok; ++h) {
+                    const uint32_t hu = it * HALVES + h, buf = hu & 1;
                     if (hu >= 2 && !mbar_wait(&acc_empty[buf], ((hu >> 1) - 1) & 1)) { report(a.error, 12u); ok = false; break; }
                     tc_fence_after();
                     if (!mbar_wait(&a_ready[h], it & 1)) { report(a.error, 13u); ok = false; break; }
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + kTsAcc0 + buf * kTsAccCols;
                     for (int c = 0; c < n_chunks; ++c) {
-                        const uint64_t db = smem_desc_sw128(smem_u32(a_base + (size_t)c * kABytes + (size_t)h * (HM * 128)));
+                        const uint64_t db = smem_desc_sw128(smem_u32(a_base + (size_t)c * kStage + (size_t)h * (HM * 128)));
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {   // 32 bytes of every slice row = 8 columns of the weights per instruction
                             if (F16) mma_f16_pair_ts(d_tmem, tmem_base + (uint32_t)(c * 32 + kk * 8), db + (uint64_t)(kk * 2), idesc, (c | kk) ? 1u : 0u);
@@ -352,8 +365,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
             bool ok = true;
             for (uint32_t it = 0; it < my_iters && ok; ++it)
                 for (int grp = 0; grp < n_groups && ok; ++grp)
-                    for (int h = 0; h < 2 && ok; ++h) {
-                        const uint32_t hu = it * 2 + h;                       // half tiles of this CTA, in order
+                    for (int h = 0; h < HALVES && ok; ++h) {
+                        const uint32_t hu = it * HALVES + h;                       // half tiles of this CTA, in order
                         const uint32_t buf = hu % kAccBufs;
                         const uint32_t s_h = it * (uint32_t)n_groups + grp;   // fills of half h's stage rows so far
                         if (grp == 0) {
@@ -368,7 +381,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                             const int sb = cnt % a.sb;
                             if (!mbar_wait(&b_full[sb], (cnt / a.sb) & 1)) { report(a.error, 13u); ok = false; break; }
                             tc_fence_after();
-                            const uint64_t da = smem_desc_sw128(smem_u32(a_base + (size_t)c * kABytes + (size_t)h * (HM * 128)));
+                            const uint64_t da = smem_desc_sw128(smem_u32(a_base + (size_t)c * kStage + (size_t)h * (HM * 128)));
                             const uint64_t db = smem_desc_sw128(smem_u32(b_base + (size_t)sb * b_bytes));
 #pragma unroll
                             for (int kk = 0; kk < 4; ++kk) {   // 32 bytes of every slice row per instruction: K = 8 (TF32) or 16 (fp16)
@@ -400,8 +413,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
         pdl_wait();
         bool ok = true;
         for (uint32_t q = plw; ok; q += kPlanners) {
-            if (q / kBlocksPerTile >= my_iters) break;
-            const int64_t t = tile_of(q / kBlocksPerTile);   // past the end for the peer of an odd last tile: all padding
+            if (q / kBlocks >= my_iters) break;
+            const int64_t t = tile_of(q / kBlocks);   // past the end for the peer of an odd last tile: all padding
             const int slot = q % kPlanSlots;
             if (q >= (uint32_t)kPlanSlots && !mbar_wait(&plan_empty[slot], ((q / kPlanSlots) - 1) & 1)) {
                 if (lane == 0) report(a.error, 17u);
@@ -409,7 +422,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
             }
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
-            const int64_t r = a.row_lo + t * BM + (q % kBlocksPerTile) * kBlockRows + lane;
+            const int64_t r = a.row_lo + t * TM + (q % kBlocks) * kBlockRows + lane;
             int4 rm = make_int4(a.safe_src, 0, -1, 0);
             if (r < a.M) rm = __ldg(a.row_meta + r);   // (self source row, first entry, count, first H^{l-1} row of the batch)
             const int32_t end = (int32_t)warp_incl_scan((uint32_t)max(rm.z, 0));   // end of the row's cached entries
@@ -486,7 +499,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
             const int n0 = (int)rank * 128 + lane_group * 32;
             const float bias_n = n0 + lane < a.N ? __ldg(a.bias + n0 + lane) : 0.f;
             uint8_t* stage = reinterpret_cast<uint8_t*>(out_stage[lane_group]);
-            for (uint32_t hu = 0; hu < 2 * my_iters && ok; ++hu) {
+            for (uint32_t hu = 0; hu < HALVES * my_iters && ok; ++hu) {
                 const uint32_t buf = hu & 1;
                 if (!mbar_wait(&acc_full[buf], (hu >> 1) & 1)) { if (lane == 0) report(a.error, 14u); ok = false; break; }
                 tc_fence_after();
@@ -494,8 +507,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                     uint32_t v[32];
                     tmem_ld_32(tmem_base + kTsAcc0 + buf * kTsAccCols + ((uint32_t)(lane_group * 32) << 16) + (uint32_t)(g * 32), v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    const int64_t t = 2 * ((int64_t)pair + (int64_t)(hu >> 1) * n_pairs) + (g >> 1);   // the tile of CTA g / 2
-                    const int64_t row0 = a.row_lo + t * BM + (hu & 1) * HM + (g & 1) * 32;
+                    const int64_t t = 2 * ((int64_t)pair + (int64_t)(hu / HALVES) * n_pairs) + (g >> 1);   // the tile of CTA g / 2
+                    const int64_t row0 = a.row_lo + t * TM + (hu % HALVES) * HM + (g & 1) * 32;
                     if (row0 >= a.M || n0 >= a.N) continue;
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the previous box has left the tile
                     __syncwarp();
@@ -523,12 +536,12 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                 }
             }
         }
-        for (uint32_t hu = 0; !TS && hu < 2 * my_iters && ok; ++hu) {
-            const int64_t t = tile_of(hu >> 1);
+        for (uint32_t hu = 0; !TS && hu < HALVES * my_iters && ok; ++hu) {
+            const int64_t t = tile_of(hu / HALVES);
             const uint32_t buf = hu % kAccBufs;
             if (!mbar_wait(&acc_full[buf], (hu / kAccBufs) & 1)) { if (lane == 0) report(a.error, 14u); ok = false; break; }
             tc_fence_after();
-            const int64_t row0 = a.row_lo + t * BM + (hu & 1) * HM + (lane_group & 1) * 32;
+            const int64_t row0 = a.row_lo + t * TM + (hu % HALVES) * HM + (lane_group & 1) * 32;
             uint8_t* stage = reinterpret_cast<uint8_t*>(out_stage[lane_group]);
             // 16 accumulator columns at a time (few registers); two such steps fill one 32-column fp32 box of the TMA
             // store, four a 64-column fp16 box
@@ -647,9 +660,9 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                 const bool lane_on = (lane >> 3) < pairs;
                 const bool col_ok = lane_on && col < a.d_in;
                 const char* src = a.src_base + (size_t)col * (HALF ? 2 : 4);
-                for (int blk = 0; blk < kBlocksPerTile; ++blk) {
+                for (int blk = 0; blk < kBlocks; ++blk) {
                     const int h = blk / kBlocksPerHalf;               // the half tile this block belongs to
-                    const uint32_t q = it * kBlocksPerTile + blk;     // row block counter of this CTA
+                    const uint32_t q = it * kBlocks + blk;     // row block counter of this CTA
                     const int slot = q % kPlanSlots;
                     if (grp == 0 && ok && !mbar_wait(&plan_full[slot], (q / kPlanSlots) & 1)) {
                         if (lane == 0) report(a.error, 16u);
@@ -750,8 +763,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                     if (ok && lane_on) {
                         // K-major, 128-byte swizzle: 16-byte slot gl of row r lands in slot gl ^ (r % 8)
                         const uint32_t s_self = 2 * (lane >> 3), s_mean = 2 * (lane >> 3) + 1;   // the group's slice = its stage
-                        uint8_t* stage_self = a_base + (size_t)s_self * kABytes;
-                        uint8_t* stage_mean = a_base + (size_t)s_mean * kABytes;
+                        uint8_t* stage_self = a_base + (size_t)s_self * kStage;
+                        uint8_t* stage_mean = a_base + (size_t)s_mean * kStage;
 #pragma unroll
                         for (int q2 = 0; q2 < kRowsInFlight; ++q2) {
                             const int row = blk * kBlockRows + brow + q2;
@@ -913,9 +926,13 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     const int b_bytes = (a.BN / 2) * 128;       // each CTA of a pair stages half of the output columns
     const int n_chunks = 2 * a.d_in_pad / kce;
     a.sa = std::min(8, n_chunks);   // one group of (self, mean) slice pairs: 128 input columns
-    // A shallow weight ring (32 KB) on purpose: with 128 KB of A stages the CTA then fits the 196 KB shared-memory
-    // carve-out, which leaves the gathers twice the L1 (measured: layer 1 of the bench 2.92 -> 2.75 ms).
-    a.sb = std::max(2, std::min({kMaxStages, n_chunks, (32 * 1024) / b_bytes}));
+    // Halves per tile: the CTA pair with the most rows sets the time, and a row of a one-half tile costs about a seventh more
+    // where its pair has several of them.  (The three layers of one mini-batch on 1M nodes, 23,400, 4,300 and 1,000 rows: 93 us in
+    // 128-row tiles, the whole call 214 -> 195 us; 128 mini-batches keep them: 4.0 ms either way.)
+    const int64_t rows = row_hi - row_lo, pairs = ctx->n_sms / 2;
+    const int64_t rounds1 = (rows + 2 * HM * pairs - 1) / (2 * HM * pairs), rounds2 = (rows + 4 * HM * pairs - 1) / (4 * HM * pairs);
+    const int halves = rounds1 * 8 < rounds2 * 14 ? 1 : 2;
+    a.sb = std::max(2, std::min({kMaxStages, n_chunks, ring_bytes(halves) / b_bytes}));
     // weights in tensor memory: TF32 operands, fp32 output, all of K in 256 columns, at most 256 output columns
     // ... and rows with few entries: a half tile of long rows is gathered for longer than its weight slices take to
     // arrive, so the stream costs nothing there, while the transposed epilogue does (measured: 5.3 entries per row,
@@ -923,7 +940,7 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     const int64_t layer_entries = d->h_hdr.ent_base[d->k - layer + 1], layer_rows = d->h_hdr.rows_total[layer];
     const bool ts = n_chunks <= 8 && d_out <= 256 && layer_entries <= kTsMaxEntriesPerRow * layer_rows && !getenv("MG_FUSED_NO_TS");
     if (ts) { a.tmem_cols = 512; a.sb = 0; a.w_rows = f16 ? (const void*)w_pad_h : (const void*)w_pad_t; }
-    const size_t smem = (size_t)a.sa * kABytes + (size_t)a.sb * b_bytes + 1024;
+    const size_t smem = (size_t)a.sa * stage_bytes(halves) + (size_t)a.sb * b_bytes + 1024;
     CUtensorMap mw;
     if (!(f16 ? make_map_f16(&mw, w_pad_h, d_out, 2 * a.d_in_pad, a.BN / 2) : make_map_f32(&mw, w_pad_t, d_out, 2 * a.d_in_pad, a.BN / 2)))
         return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the layer weights");
@@ -938,17 +955,17 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
         return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the layer output");
     const bool first = layer == 1, half = first && ctx->feat_dtype == MG_DTYPE_F16;
     typedef void (*Kernel)(CUtensorMap, CUtensorMap, CUtensorMap, FusedArgs);
-    static const Kernel kernels[2][5] = {
-        {k_sage_layer_fused<true, false, false>, k_sage_layer_fused<true, true, false>, k_sage_layer_fused<true, true, true>,
-         k_sage_layer_fused<false, false, false>, k_sage_layer_fused<false, true, true>},
-        {k_sage_layer_fused<true, false, false, true>, k_sage_layer_fused<true, true, false, true>, k_sage_layer_fused<true, true, true, true>,
-         k_sage_layer_fused<false, false, false, true>, k_sage_layer_fused<false, true, true, true>}};
-    static uint64_t smem_done[2][5] = {};
+#define MG_FUSED_KERNELS(TS, HALVES) \
+    {k_sage_layer_fused<true, false, false, TS, HALVES>, k_sage_layer_fused<true, true, false, TS, HALVES>, k_sage_layer_fused<true, true, true, TS, HALVES>, \
+     k_sage_layer_fused<false, false, false, TS, HALVES>, k_sage_layer_fused<false, true, true, TS, HALVES>}
+    static const Kernel kernels[2][2][5] = {{MG_FUSED_KERNELS(false, 1), MG_FUSED_KERNELS(true, 1)}, {MG_FUSED_KERNELS(false, 2), MG_FUSED_KERNELS(true, 2)}};
+#undef MG_FUSED_KERNELS
+    static uint64_t smem_done[2][2][5] = {};
     const int which = first ? (f16 ? 2 : half ? 1 : 0) : (f16 ? 4 : 3);
-    const Kernel kern = kernels[ts][which];
-    MG_CUDA(ctx, mg_smem_limit(&smem_done[ts][which], ctx->device, (const void*)kern, 8 * (int)kABytes + 32 * 1024 + 1024));
-    const int64_t n_tiles = (row_hi - row_lo + BM - 1) / BM;
-    const int grid = 2 * (int)std::min<int64_t>((n_tiles + 1) / 2, ctx->n_sms / 2);   // CTA pairs
+    const Kernel kern = kernels[halves - 1][ts][which];
+    MG_CUDA(ctx, mg_smem_limit(&smem_done[halves - 1][ts][which], ctx->device, (const void*)kern, fused_smem_limit(halves)));
+    const int64_t n_tiles = (rows + HM * halves - 1) / (HM * halves);
+    const int grid = 2 * (int)std::min<int64_t>((n_tiles + 1) / 2, pairs);   // CTA pairs
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kFusedThreads); cfg.dynamicSmemBytes = smem; cfg.stream = ctx->stream;
     cudaLaunchAttribute pdl;

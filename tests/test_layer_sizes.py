@@ -1,0 +1,48 @@
+"""The fused layer kernel cuts a layer's rows into tiles of 64 or 128 per CTA by how many rows there are: row counts on either
+side of every cut, with the weights in tensor memory and streamed, against the layer's definition in fp64."""
+import pytest
+import torch
+
+import paper_2202_02365_b200 as mg
+from paper_2202_02365_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+N = 40_000
+
+
+@pytest.fixture(scope="module")
+def graph():
+    return inputs.rmat_graph(N, 6 * N, seed=31)
+
+
+def last_layer(view, feats, ws, wn, b):
+    """One layer over a one-hop sample in fp64: self rows, mean of the sampled neighbours, linear maps."""
+    h = feats[view.node_ids.long()].double()
+    off, n = view.nbr_offsets.long(), view.nbr_offsets.numel() - 1
+    cnt = off[1:] - off[:-1]
+    dst = torch.repeat_interleave(torch.arange(n, device=h.device), cnt)
+    mean = torch.zeros((n, h.shape[1]), dtype=torch.float64, device=h.device).index_add(0, dst, h[view.repr_map.long()])
+    mean = mean / cnt.clamp(min=1).double()[:, None]
+    return h[h.shape[0] - n:] @ ws.double().cuda() + mean @ wn.double().cuda() + b.double().cuda()
+
+
+# (148 SMs: one round of 64-row tiles holds 9,472 rows, of 128-row tiles 18,944); widths with K of one to three groups
+@pytest.mark.parametrize("rows", [1, 64, 65, 129, 9_472, 9_473, 18_944, 18_945, 28_417, 37_889])
+@pytest.mark.parametrize("d_in,d_out,half,fanout", [(128, 256, False, 4), (256, 100, False, 9), (384, 36, True, 3)])
+def test_rows_on_either_side_of_the_tile_sizes(graph, rows, d_in, d_out, half, fanout):
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    feats = inputs.normal_features(N, d_in, seed=5, device="cuda", dtype=torch.float16 if half else torch.float32)
+    ctx.load_features(feats)
+    (layer,) = inputs.random_bias_layers([d_in, d_out], seed=6)
+    dense = ctx.sample(inputs.distinct_targets(N, rows, seed=7), [fanout], seed=8)
+    out = torch.full((rows + 1, d_out), 7.0, device="cuda")
+    ctx.forward(ctx.model([layer]), dense, out[:rows])
+    want = last_layer(dense.view(0), feats, *layer)
+    # operands rounded to 10 bits (2^-11 each), sums of up to 768 products of random sign: rms error below 1e-3 of the rows' rms, the
+    # largest of 10^7 values below 6 times that
+    err = (out[:rows].double() - want).abs()
+    rms = want.square().mean().sqrt()
+    assert float(err.square().mean().sqrt() / rms) < 1e-3 and float((err / torch.maximum(want.abs(), rms)).max()) < 6e-3
+    assert torch.equal(out[rows], torch.full_like(out[rows], 7.0))
