@@ -155,8 +155,6 @@ struct mg_ctx {
     char* lp_spare = nullptr; size_t lp_spare_bytes = 0;
     int32_t* lp_words = nullptr;       // mapped pinned host words {status, n_targets} that mg_lp_prepare's last kernel writes (behind h_flags)
     int32_t* lp_words_dev = nullptr;   // their device address
-    int32_t* lp_range = nullptr;       // device {0, 32-word groups of the node bitmap}: the bounds of mg_lp_prepare's scan
-    int64_t lp_range_words = -1;
     float* gat_x = nullptr; float* gat_z = nullptr; float* gat_s = nullptr; float* gat_h[2] = {nullptr, nullptr};   // mg_gat_forward scratch
     size_t gat_x_elems = 0, gat_z_elems = 0, gat_s_elems = 0, gat_h_elems[2] = {0, 0};
     const struct mg_model* last_fwd_model = nullptr; const struct mg_dense* last_fwd_dense = nullptr;   // what mg_backward may follow
@@ -365,7 +363,6 @@ void mg_sort_params_host(SortParams* sp, int64_t n);
 // (perm[c] = local row of canonical row c: deltas in the paper's order, ids ascending inside a delta, targets in the
 // caller's order; inv = its inverse).  Device arrays owned by d; on ctx->stream, synchronous, off the hot path.
 int mg_dense_batch_perm(mg_ctx* ctx, mg_dense* d, int b, const int32_t** perm, const int32_t** inv);
-size_t mg_scan_tmp_elems(int64_t max_elems);
 void mg_sort_u64(mg_ctx* ctx, uint64_t* const buf[2], const SortParams* sp, int lo_bit, int bits, uint32_t* hist,
                  uint32_t* scan_tmp, int* res_buf, const void* seg_tiles = nullptr);
 void mg_scan_u32(mg_ctx* ctx, uint32_t* data, const int32_t* lo, const int32_t* hi, const int32_t* base,

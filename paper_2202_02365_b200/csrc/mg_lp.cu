@@ -13,10 +13,9 @@ namespace {
 constexpr int kThreads = 256;
 
 // The target union of a batch = the distinct ids among sources, destinations and negatives, ascending.  It is taken
-// with a bit per node: every id sets its bit (k_lp_mark, which also draws the negatives), the words' population counts
-// are scanned, a word's set bits are written out from its prefix on (k_lp_emit), and the row of an id is its word's prefix
-// plus the set bits below it (k_lp_index); counts and prefixes are kept per group of 32 words, so the scan runs over
-// n_nodes / 1024 values.  Seven short launches, none of them a sort.
+// with a bit per node: every id sets its bit (k_lp_mark, which also draws the negatives), one pass over the bitmap counts the
+// set bits before every word and writes the ids out (k_lp_scan), and the row of an id is its word's count plus the set bits below
+// it (k_lp_index).  Three short launches, none of them a sort.
 // Origins: [0, E) sources, [E, 2E) destinations, [2E, 2E + C * negs) negatives.
 __global__ void __launch_bounds__(kThreads)
 k_lp_mark(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t E, int32_t n_chunks, int32_t negs,
@@ -47,33 +46,77 @@ k_lp_mark(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int6
     }
 }
 
-// population count of every group of 32 words (1,024 nodes): the scan then runs over n_words / 32 counts
-constexpr int kLpGroup = 32;
-__global__ void __launch_bounds__(kThreads) k_lp_popc(const uint32_t* __restrict__ bitmap, int32_t n_words, int32_t n_groups, uint32_t* counts) {
-    const int lane = threadIdx.x & 31;
-    const int32_t warps = gridDim.x * (kThreads / 32);
-    for (int32_t g = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); g < n_groups; g += warps) {
-        const int32_t w = g * kLpGroup + lane;
-        uint32_t c = w < n_words ? __popc(bitmap[w]) : 0u;
-        for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
-        if (lane == 0) counts[g] = c;
+// One pass over the bitmap (8 words per thread): set bits are counted, the tiles' running totals chained through a 64-bit state each
+// (decoupled look-back; tiles come from a counter, so that a tile's predecessors are held by running blocks, and the polls are
+// bounded), the set bits' ids written from their place on, and the count before every word that holds any kept.  Bound by launch
+// and look-back latency: 8M nodes 7 us, where a population count, a three-kernel scan and a pass for the ids took 14 us and
+// four gaps.
+constexpr int kLpWords = kThreads * 8;   // words of a tile: 65,536 nodes
+struct LpScanArgs {
+    const uint32_t* bitmap;    // padded with zero words to whole tiles
+    uint64_t* state;
+    uint32_t* ticket;
+    int32_t n_tiles;
+    uint32_t* before;          // [words] set bits before the word (words with set bits only)
+    int32_t* targets;
+    int32_t* n_targets;
+    uint32_t* status;
+};
+__global__ void __launch_bounds__(kThreads) k_lp_scan(LpScanArgs a) {
+    __shared__ uint32_t part[kThreads / 32];
+    __shared__ uint32_t sh_before;
+    __shared__ int32_t sh_tile;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr uint64_t kSum = 1ull << 62, kTotal = 2ull << 62;
+    constexpr int kPolls = 1 << 20;
+    if (threadIdx.x == 0) sh_tile = (int32_t)atomicAdd(a.ticket, 1u);   // (a block per tile)
+    __syncthreads();
+    const int32_t tile = sh_tile;
+    const int32_t w0 = tile * kLpWords + (int32_t)threadIdx.x * 8;
+    const uint4 lo = *reinterpret_cast<const uint4*>(a.bitmap + w0), hi = *reinterpret_cast<const uint4*>(a.bitmap + w0 + 4);
+    const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    uint32_t s = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s += __popc(w[i]);
+    const uint32_t inc = warp_incl_scan(s);
+    if (lane == 31) part[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t p = lane < kThreads / 32 ? part[lane] : 0u;
+        const uint32_t pi = warp_incl_scan(p);
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, pi, 31);
+        if (lane < kThreads / 32) part[lane] = pi - p;
+        volatile uint64_t* state = a.state;
+        uint32_t before = 0;
+        if (tile > 0 && lane == 0) state[tile] = kSum | total;
+        for (int32_t top = tile - 1; top >= 0; top -= 32) {   // windows of 32 tiles until one carries a running total
+            const int32_t at = top - lane;
+            uint64_t st = kSum;   // (before tile 0: nothing)
+            if (at >= 0) {
+                int polls = 0;
+                while ((st = state[at]) == 0 && ++polls < kPolls) {}
+                if (polls >= kPolls) { atomicOr(a.status, ST_INTERNAL); st = kTotal; }
+            }
+            const uint32_t full = __ballot_sync(0xFFFFFFFFu, (st & kTotal) != 0);
+            const int stop = full ? __ffs(full) - 1 : 31;
+            before += __reduce_add_sync(0xFFFFFFFFu, lane <= stop ? (uint32_t)st : 0u);
+            if (full) break;
+        }
+        if (lane == 0) {
+            state[tile] = kTotal | (before + total);
+            sh_before = before;
+            if (tile == a.n_tiles - 1) *a.n_targets = (int32_t)(before + total);
+        }
     }
-}
-
-// after the exclusive scan of the group counts: the ids of the set bits, ascending (a warp per group: lane = word)
-__global__ void __launch_bounds__(kThreads)
-k_lp_emit(const uint32_t* __restrict__ bitmap, const uint32_t* __restrict__ prefix, int32_t n_words, int32_t n_groups, int32_t* targets) {
-    const int lane = threadIdx.x & 31;
-    const int32_t warps = gridDim.x * (kThreads / 32);
-    for (int32_t g = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); g < n_groups; g += warps) {
-        const int32_t w = g * kLpGroup + lane;
-        uint32_t bits = w < n_words ? bitmap[w] : 0u;
-        if (!__any_sync(0xFFFFFFFFu, bits != 0u)) continue;
-        const uint32_t c = __popc(bits);
-        uint32_t at = prefix[g] + warp_incl_scan(c) - c;
+    __syncthreads();
+    uint32_t at = sh_before + part[warp] + inc - s;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        uint32_t bits = w[i];
+        if (!bits) continue;
+        a.before[w0 + i] = at;
         while (bits) {
-            const int bpos = __ffs(bits) - 1;
-            targets[at++] = w * 32 + bpos;
+            a.targets[at++] = (w0 + i) * 32 + (__ffs(bits) - 1);
             bits &= bits - 1;
         }
     }
@@ -81,7 +124,7 @@ k_lp_emit(const uint32_t* __restrict__ bitmap, const uint32_t* __restrict__ pref
 
 __global__ void __launch_bounds__(kThreads)
 k_lp_index(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, const int32_t* __restrict__ neg_ids, int64_t E,
-           int64_t total, int64_t n_nodes, const uint32_t* __restrict__ bitmap, const uint32_t* __restrict__ prefix,
+           int64_t total, int64_t n_nodes, const uint32_t* __restrict__ bitmap, const uint32_t* __restrict__ before,
            int32_t* src_idx, int32_t* dst_idx, int32_t* neg_idx, const uint32_t* status, const int32_t* n_targets, int32_t* host_words) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {   // the call's two results, straight into mapped host memory
         host_words[0] = (int32_t)*status;
@@ -91,9 +134,7 @@ k_lp_index(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, con
         int32_t id = i < E ? src[i] : (i < 2 * E ? dst[i - E] : neg_ids[i - 2 * E]);
         if (id < 0 || (int64_t)id >= n_nodes) id = 0;   // (as k_lp_mark: the call fails with the range error anyway)
         const uint32_t w = (uint32_t)id >> 5;
-        // the group's prefix, the set bits of the group's words before this one, the set bits below the id in its word
-        uint32_t rank = prefix[w / kLpGroup] + __popc(bitmap[w] & ((1u << (id & 31)) - 1u));
-        for (uint32_t v = w - w % kLpGroup; v < w; ++v) rank += __popc(bitmap[v]);
+        const uint32_t rank = before[w] + __popc(bitmap[w] & ((1u << (id & 31)) - 1u));
         if (i < E) src_idx[i] = (int32_t)rank;
         else if (i < 2 * E) dst_idx[i - E] = (int32_t)rank;
         else neg_idx[i - 2 * E] = (int32_t)rank;
@@ -193,7 +234,7 @@ __global__ void __launch_bounds__(256) k_distmult_neg(NegArgs a) {
 
 // ---- tensor-core negative scoring ------------------------------------------------------------
 // The right operand -- the chunk's negatives h[neg], rounded to TF32 -- is the same for every 128-edge tile of a chunk:
-// k_stage_negs writes it once per call as ready-made operand images (blocks of up to 128 negatives, K-major slices of
+// k_distmult_prepare writes it once per call as ready-made operand images (blocks of up to 128 negatives, K-major slices of
 // 32 columns, 128-byte swizzle), a few MB that stay in L2, and the scoring kernel fetches a block with one bulk copy
 // per slice.
 // One CTA of the scoring kernel owns 128 edges of one chunk and one corrupted side.  The left operand rows
@@ -221,26 +262,64 @@ __device__ __forceinline__ size_t swz_off(int row, int slot) {   // 16-byte slot
     return (size_t)(row >> 3) * 1024 + (size_t)(row & 7) * 128 + (size_t)((slot ^ (row & 7)) << 4);
 }
 
-// operand images of the negatives: item = (chunk, block, row of the block, 16-byte slot of the row)
-__global__ void __launch_bounds__(kThreads)
-k_stage_negs(const float* __restrict__ h, const int32_t* __restrict__ neg_idx, int32_t n_chunks, int32_t negs, int32_t dim,
-             int32_t n_slices, int32_t bn_max, uint8_t* images) {
-    const int n_slots = n_slices * 8;
-    const int n_blocks = (negs + bn_max - 1) / bn_max;
-    const int64_t total = (int64_t)n_chunks * n_blocks * bn_max * n_slots;
-    const size_t slice_bytes = (size_t)bn_max * 128;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+// What the tensor-core kernels wait for, and the scores of the positives beside it: the first `pos_blocks` blocks take edges,
+// the others make the operand images (item = (chunk, block, row of the block, 16-byte slot of the row)).  Both are bound by the
+// latency of scattered row reads, so a warp has the three rows of four edges in flight and the two run together: 50,000 edges
+// and 10,000 negatives of 100 columns, 14.6 + 6.8 us and a gap in two kernels of an edge per warp at a time.
+constexpr int kPosEdges = 4;
+struct PrepareArgs {
+    const float* h;
+    const float* rel_emb;
+    const int32_t *src_idx, *dst_idx, *rel, *neg_idx;
+    int64_t E;
+    float* pos;
+    int32_t pos_blocks, n_chunks, negs, dim, n_slices, bn_max;
+    uint8_t* images;
+};
+__global__ void __launch_bounds__(kThreads) k_distmult_prepare(PrepareArgs a) {
+    if ((int)blockIdx.x < a.pos_blocks) {
+        const int lane = threadIdx.x & 31, n4 = a.dim / 4;   // (dim <= 128: a lane has at most one 16-byte piece of a row)
+        const int64_t step = (int64_t)a.pos_blocks * (kThreads / 32) * kPosEdges;
+        for (int64_t i0 = (blockIdx.x * (int64_t)(kThreads / 32) + (threadIdx.x >> 5)) * kPosEdges; i0 < a.E; i0 += step) {
+            float4 s[kPosEdges], r[kPosEdges], o[kPosEdges];
+#pragma unroll
+            for (int u = 0; u < kPosEdges; ++u) {
+                const int64_t i = min(i0 + u, a.E - 1);
+                s[u] = r[u] = o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (lane >= n4) continue;
+                s[u] = __ldg(reinterpret_cast<const float4*>(a.h + (int64_t)a.src_idx[i] * a.dim) + lane);
+                o[u] = __ldg(reinterpret_cast<const float4*>(a.h + (int64_t)a.dst_idx[i] * a.dim) + lane);
+                r[u] = __ldg(reinterpret_cast<const float4*>(a.rel_emb + (int64_t)a.rel[i] * a.dim) + lane);
+            }
+#pragma unroll
+            for (int u = 0; u < kPosEdges; ++u) {
+                float v = s[u].x * r[u].x * o[u].x;
+                v = fmaf(s[u].y * r[u].y, o[u].y, v);
+                v = fmaf(s[u].z * r[u].z, o[u].z, v);
+                v = fmaf(s[u].w * r[u].w, o[u].w, v);
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, d);
+                if (lane == 0 && i0 + u < a.E) a.pos[i0 + u] = v;
+            }
+        }
+        return;
+    }
+    const int n_slots = a.n_slices * 8;
+    const int n_blocks = (a.negs + a.bn_max - 1) / a.bn_max;
+    const int64_t total = (int64_t)a.n_chunks * n_blocks * a.bn_max * n_slots;
+    const size_t slice_bytes = (size_t)a.bn_max * 128;
+    for (int64_t i = (blockIdx.x - a.pos_blocks) * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)(gridDim.x - a.pos_blocks) * blockDim.x) {
         const int q = (int)(i % n_slots);
-        const int r = (int)((i / n_slots) % bn_max);
-        const int64_t cb = i / ((int64_t)n_slots * bn_max);   // chunk * n_blocks + block
-        const int n = (int)(cb % n_blocks) * bn_max + r;
+        const int r = (int)((i / n_slots) % a.bn_max);
+        const int64_t cb = i / ((int64_t)n_slots * a.bn_max);   // chunk * n_blocks + block
+        const int n = (int)(cb % n_blocks) * a.bn_max + r;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (n < negs && q * 4 < dim) {
-            const int32_t src = neg_idx[(cb / n_blocks) * negs + n];
-            const float4 x = __ldg(reinterpret_cast<const float4*>(h + (int64_t)src * dim) + q);
+        if (n < a.negs && q * 4 < a.dim) {
+            const int32_t src = a.neg_idx[(cb / n_blocks) * a.negs + n];
+            const float4 x = __ldg(reinterpret_cast<const float4*>(a.h + (int64_t)src * a.dim) + q);
             v = make_float4(tc::to_tf32(x.x), tc::to_tf32(x.y), tc::to_tf32(x.z), tc::to_tf32(x.w));
         }
-        *reinterpret_cast<float4*>(images + ((size_t)cb * n_slices + (q >> 3)) * slice_bytes + swz_off(r, q & 7)) = v;
+        *reinterpret_cast<float4*>(a.images + ((size_t)cb * a.n_slices + (q >> 3)) * slice_bytes + swz_off(r, q & 7)) = v;
     }
 }
 
@@ -464,12 +543,10 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     lp->ctx = ctx; lp->device = ctx->device; lp->n_edges = n_edges; lp->n_chunks = n_chunks; lp->negs = negs;
 
     const size_t n_neg = (size_t)std::max<int64_t>((int64_t)n_chunks * negs, 1);
-    const int64_t n_words = (ctx->n_nodes + 31) / 32;
-    const int64_t n_groups = (n_words + kLpGroup - 1) / kLpGroup;
-    const size_t scan_elems = mg_scan_tmp_elems(n_groups);
+    const int64_t n_tiles = ((ctx->n_nodes + 31) / 32 + kLpWords - 1) / kLpWords, n_words = n_tiles * kLpWords;
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     // scratch: one block of the context that only grows
-    const size_t ws_bytes = 2 * up(4 * (size_t)n_edges) + up(4 * (size_t)n_words) + up(4 * (size_t)n_groups) + up(4 * scan_elems) + 3 * 256;
+    const size_t ws_bytes = 2 * up(4 * (size_t)n_edges) + 256 + up(8 * (size_t)n_tiles) + 2 * up(4 * (size_t)n_words);
     if (ctx->lp_ws_bytes < ws_bytes) {
         cudaFree(ctx->lp_ws);
         ctx->lp_ws = nullptr; ctx->lp_ws_bytes = 0;
@@ -483,24 +560,14 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     auto take = [&](size_t b) { char* p = w; w += up(b); return p; };
     int32_t* d_src = (int32_t*)take(4 * (size_t)n_edges);
     int32_t* d_dst = (int32_t*)take(4 * (size_t)n_edges);
+    // cleared by one memset: the status, the scan's ticket and states, the bitmap
+    uint32_t* d_status = (uint32_t*)take(256);
+    uint64_t* states = (uint64_t*)take(8 * (size_t)n_tiles);
     uint32_t* bitmap = (uint32_t*)take(4 * (size_t)n_words);
-    uint32_t* prefix = (uint32_t*)take(4 * (size_t)n_groups);
-    uint32_t* scan_tmp = (uint32_t*)take(4 * scan_elems);
-    uint32_t* d_status = (uint32_t*)take(4);
-    int32_t* d_nt = (int32_t*)take(4);
-    if (!ctx->lp_range && cudaMalloc((void**)&ctx->lp_range, 2 * sizeof(int32_t)) != cudaSuccess) {
-        cudaGetLastError(); delete lp;
-        return mg_fail(ctx, MG_ERR_OOM, "allocation of the link-prediction scratch failed");
-    }
-    if (ctx->lp_range_words != n_words) {   // (once per graph)
-        const int32_t h_range[2] = {0, (int32_t)n_groups};
-        if (cudaMemcpy(ctx->lp_range, h_range, sizeof(h_range), cudaMemcpyHostToDevice) != cudaSuccess) {
-            cudaGetLastError(); delete lp;
-            return mg_fail(ctx, MG_ERR_CUDA, "copy failed");
-        }
-        ctx->lp_range_words = n_words;
-    }
-    const int32_t* d_range = ctx->lp_range;
+    const size_t cleared = (size_t)(w - (char*)d_status);
+    uint32_t* before = (uint32_t*)take(4 * (size_t)n_words);
+    uint32_t* ticket = d_status + 1;
+    int32_t* d_nt = (int32_t*)(d_status + 2);
     // results: one block, taken from the context's spare when that is large enough
     const size_t blk_bytes = up(4 * (size_t)total) + 3 * up(4 * (size_t)n_edges) + 2 * up(4 * n_neg);
     if (ctx->lp_spare && ctx->lp_spare_bytes >= blk_bytes) {
@@ -519,30 +586,27 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     lp->rel = (int32_t*)take(4 * (size_t)n_edges);
     lp->neg_ids = (int32_t*)take(4 * n_neg);
     lp->neg_idx = (int32_t*)take(4 * n_neg);
-    auto cleanup = [&]() {};
 
     cudaMemcpyAsync(d_src, src, 4 * n_edges, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_dst, dst, 4 * n_edges, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(lp->rel, rel, 4 * n_edges, cudaMemcpyHostToDevice, st);
-    cudaMemsetAsync(d_status, 0, 4, st);
-    cudaMemsetAsync(bitmap, 0, 4 * (size_t)n_words, st);
+    cudaMemsetAsync(d_status, 0, cleared, st);
     const int grid = mg_grid(ctx, 4);
     k_lp_mark<<<grid, kThreads, 0, st>>>(d_src, d_dst, n_edges, n_chunks, negs, seed, ctx->d_res_prefix, ctx->n_parts,
                                          ctx->n_resident_nodes, ctx->n_nodes, mg_feat_geom(ctx), ctx->d_part_start, ctx->d_nodes_by_part,
                                          lp->neg_ids, bitmap, d_status);
-    k_lp_popc<<<grid, kThreads, 0, st>>>(bitmap, (int32_t)n_words, (int32_t)n_groups, prefix);
-    mg_scan_u32(ctx, prefix, d_range, d_range + 1, nullptr, scan_tmp, reinterpret_cast<uint32_t*>(d_nt));
-    k_lp_emit<<<grid, kThreads, 0, st>>>(bitmap, prefix, (int32_t)n_words, (int32_t)n_groups, lp->targets);
-    k_lp_index<<<grid, kThreads, 0, st>>>(d_src, d_dst, lp->neg_ids, n_edges, total, ctx->n_nodes, bitmap, prefix, lp->src_idx,
+    k_lp_scan<<<(unsigned)n_tiles, kThreads, 0, st>>>(LpScanArgs{bitmap, states, ticket, (int32_t)n_tiles, before, lp->targets, d_nt, d_status});
+    k_lp_index<<<grid, kThreads, 0, st>>>(d_src, d_dst, lp->neg_ids, n_edges, total, ctx->n_nodes, bitmap, before, lp->src_idx,
                                           lp->dst_idx, lp->neg_idx, d_status, d_nt, ctx->lp_words_dev);
-    ctx->launches += 4;
+    ctx->launches += 3;
+    // (not needed above: the host's part of this copy runs beside the kernels)
+    cudaMemcpyAsync(lp->rel, rel, 4 * n_edges, cudaMemcpyHostToDevice, st);
     cudaError_t e = cudaStreamSynchronize(st);
     const uint32_t h_status = e == cudaSuccess ? (uint32_t)ctx->lp_words[0] : 0u;
     lp->n_targets = e == cudaSuccess ? ctx->lp_words[1] : 0;
     if (e == cudaSuccess) e = cudaGetLastError();
-    cleanup();
     if (e != cudaSuccess) { mg_lp_free(lp); return mg_cuda_fail(ctx, e, "mg_lp_prepare"); }
     if (h_status & ST_RANGE) { mg_lp_free(lp); return mg_fail(ctx, MG_ERR_ARG, "an edge endpoint is outside [0, n_nodes)"); }
+    if (h_status & ST_INTERNAL) { mg_lp_free(lp); return mg_fail(ctx, MG_ERR_TIMEOUT, "the scan of the target union gave up waiting"); }
     if (h_status & ST_NONRESIDENT) { mg_lp_free(lp); return mg_fail(ctx, MG_ERR_NONRESIDENT, "an edge endpoint lies in a partition that is not resident"); }
     *out = lp;
     return MG_OK;
@@ -571,15 +635,17 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
     cudaStream_t st = ctx->stream;
     ProfScope ps(ctx, PH_DISTMULT, 3);
-    k_distmult_pos<<<mg_grid(ctx, 8), kThreads, 0, st>>>(h_dev, rel_emb_dev, lp->src_idx, lp->dst_idx, lp->rel, lp->n_edges, dim, pos_out);
-    ctx->launches++;
+    const bool tensor = gemm_precision == MG_GEMM_TF32 && dim % 4 == 0 && dim <= 32 * kTcMaxSlices && lp->negs > 0;
+    if (!tensor) {
+        k_distmult_pos<<<mg_grid(ctx, 8), kThreads, 0, st>>>(h_dev, rel_emb_dev, lp->src_idx, lp->dst_idx, lp->rel, lp->n_edges, dim, pos_out);
+        ctx->launches++;
+    }
     if (lp->negs > 0) {
         const int64_t max_chunk = (lp->n_edges + lp->n_chunks - 1) / lp->n_chunks;
         NegArgs a;
         a.h = h_dev; a.rel_emb = rel_emb_dev; a.rel = lp->rel; a.neg_idx = lp->neg_idx; a.E = lp->n_edges;
         a.n_chunks = lp->n_chunks; a.negs = lp->negs; a.dim = dim;
         a.tiles_per_chunk = (int32_t)((max_chunk + 63) / 64);
-        const bool tensor = gemm_precision == MG_GEMM_TF32 && dim % 4 == 0 && dim <= 32 * kTcMaxSlices;
         if (tensor) {
             NegTcArgs ta;
             ta.n_slices = (dim + 31) / 32;
@@ -601,8 +667,12 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
                 }
                 ctx->dm_images_bytes = image_bytes;
             }
-            k_stage_negs<<<mg_grid(ctx, 8), kThreads, 0, st>>>(h_dev, lp->neg_idx, lp->n_chunks, lp->negs, dim, ta.n_slices, ta.bn_max,
-                                                             (uint8_t*)ctx->dm_images);
+            const int64_t items = (int64_t)lp->n_chunks * n_blocks * ta.bn_max * ta.n_slices * 8;
+            const int pos_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(mg_grid(ctx, 4), (lp->n_edges + kPosEdges * kThreads / 32 - 1) / (kPosEdges * kThreads / 32)));
+            const int image_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(mg_grid(ctx, 4), (items + kThreads - 1) / kThreads));
+            k_distmult_prepare<<<pos_blocks + image_blocks, kThreads, 0, st>>>(PrepareArgs{h_dev, rel_emb_dev, lp->src_idx, lp->dst_idx, lp->rel, lp->neg_idx, lp->n_edges,
+                                                                                          pos_out, pos_blocks, lp->n_chunks, lp->negs, dim, ta.n_slices, ta.bn_max,
+                                                                                          (uint8_t*)ctx->dm_images});
             ctx->launches++;
             ta.b_images = (const uint8_t*)ctx->dm_images;
             const size_t smem = (size_t)ta.n_slices * 16384 + 2 * (size_t)ta.n_slices * ta.bn_max * 128 + 1024;

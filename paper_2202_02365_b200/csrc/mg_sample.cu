@@ -1409,7 +1409,6 @@ size_t mg_sort_hist_elems(int64_t max_keys) { return (size_t)kBins * ((max_keys 
 void mg_sort_params_host(SortParams* sp, int64_t n) {
     sp->zero = 0; sp->n = (int32_t)n; sp->ntiles = (int32_t)((n + kSortTile - 1) / kSortTile); sp->hist_len = kBins * sp->ntiles;
 }
-size_t mg_scan_tmp_elems(int64_t max_elems) { return (size_t)((max_elems + kScanTile - 1) / kScanTile) + 16; }
 
 static void sample_kernel_attributes();
 
