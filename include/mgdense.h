@@ -375,6 +375,9 @@ int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel, const int
 int mg_lp_view(const mg_lp_batch* lp, int32_t* n_targets, const int32_t** targets,
                const int32_t** src_idx, const int32_t** dst_idx, const int32_t** neg_ids,
                const int32_t** neg_idx);
+/* Copy the target ids (n_targets of mg_lp_view) to a DEVICE buffer of the caller's on `stream` (a cudaStream_t of the context's
+ * device; NULL = the default stream); not waited for. */
+int mg_lp_targets(mg_ctx* ctx, const mg_lp_batch* lp, int32_t* dst_dev, void* stream);
 int mg_lp_free(mg_lp_batch* lp);
 
 /* DistMult: pos[i] = sum_d h[s_i,d] rel_emb[r_i,d] h[o_i,d]; neg_dst[i,t] the same with the

@@ -30,7 +30,7 @@ EXPORTS = [
     "mg_create", "mg_destroy", "mg_last_error", "mg_load_graph", "mg_load_out_graph", "mg_set_sample_direction", "mg_set_partitioning",
     "mg_load_features", "mg_set_partition_source", "mg_set_resident", "mg_commit_resident", "mg_sample_many", "mg_sample_many_begin", "mg_sample_many_end", "mg_sample",
     "mg_dense_counts", "mg_dense_view", "mg_dense_export_many", "mg_dense_export_view", "mg_dense_arrays_copy", "mg_dense_free", "mg_model_create", "mg_model_set_aggregator", "mg_model_set_intermediates", "mg_model_free",
-    "mg_forward", "mg_set_layer_window", "mg_keep_layer_outputs", "mg_forward_host_async", "mg_wait_output", "mg_forward_noalloc", "mg_gather_h0", "mg_layer_output", "mg_lp_prepare", "mg_lp_view", "mg_lp_free",
+    "mg_forward", "mg_set_layer_window", "mg_keep_layer_outputs", "mg_forward_host_async", "mg_wait_output", "mg_forward_noalloc", "mg_gather_h0", "mg_layer_output", "mg_lp_prepare", "mg_lp_view", "mg_lp_targets", "mg_lp_free",
     "mg_distmult_score", "mg_kernel_launches", "mg_profile", "mg_profile_read", "mg_comet_plan", "mg_comet_bias", "mg_comet_autotune", "mg_gat_model_create", "mg_gat_model_set_heads", "mg_gat_model_free", "mg_gat_forward", "mg_backward", "mg_model_grads", "mg_model_sgd_step", "mg_model_adagrad_step", "mg_dense_packed_ids", "mg_apply_embedding_sgd",
 ]
 
@@ -70,6 +70,15 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
 
 def _ptr(t: torch.Tensor | None):
     return C.c_void_p(t.data_ptr()) if t is not None else C.c_void_p(0)
+
+
+def _raw_stream(device: torch.device):
+    """The stream torch queues on, as the library takes it."""
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(device.index))
+
+
+def _fanouts(fanouts):
+    return (C.c_int32 * len(fanouts))(*[int(f) for f in fanouts])
 
 
 def _host(x, dtype) -> torch.Tensor:
@@ -180,7 +189,7 @@ class Dense:
         dev = self.ctx.device
         out = torch.empty(sum(sizes), dtype=torch.int32, device=dev)
         self.ctx._check(self.ctx.lib.mg_dense_arrays_copy(self.ctx.handle, C.byref(arr), _ptr(out),
-                                                          C.c_void_p(torch._C._cuda_getCurrentRawStream(dev.index))))
+                                                          _raw_stream(dev)))
         return DenseView(*out.split_with_sizes(sizes))
 
     def export_many(self):
@@ -293,9 +302,10 @@ class LpBatch:
     def targets(self) -> torch.Tensor:
         """The batch's target union (distinct ids, ascending) alone: what the sampler is called with."""
         n = C.c_int32(0)
-        p = C.c_void_p(0)
-        self.ctx._check(self.ctx.lib.mg_lp_view(self.handle, C.byref(n), C.byref(p), None, None, None, None))
-        return _from_dev(p.value, n.value, self.ctx.device)
+        self.ctx._check(self.ctx.lib.mg_lp_view(self.handle, C.byref(n), None, None, None, None, None))
+        out = torch.empty(n.value, dtype=torch.int32, device=self.ctx.device)
+        self.ctx._check(self.ctx.lib.mg_lp_targets(self.ctx.handle, self.handle, _ptr(out), _raw_stream(self.ctx.device)))
+        return out
 
     def view(self):
         n = C.c_int32(0)
@@ -472,7 +482,7 @@ class Context:
         assert targets.dtype == torch.int32
         targets = targets.contiguous()
         offs = _host(target_offsets, torch.int64)
-        fo = _host(list(fanouts), torch.int32)
+        fo = _fanouts(fanouts)
         sd = np.ascontiguousarray(np.array([int(s) & 0xFFFFFFFFFFFFFFFF for s in seeds], dtype=np.uint64))
         d = out if out is not None else Dense(self)
         cp = None
@@ -480,7 +490,7 @@ class Context:
             cp = SampleCaps(int(caps.get("max_nodes_total", 0)), int(caps.get("max_entries_total", 0)),
                             int(caps.get("max_nodes_per_batch", 0)), int(caps.get("max_inner_nodes_per_batch", 0)))
         self._check(fn(self.handle, _ptr(targets), C.c_int(targets.is_cuda), _ptr(offs),
-                       C.c_int32(offs.numel() - 1), _ptr(fo), C.c_int32(fo.numel()), C.c_void_p(sd.ctypes.data),
+                       C.c_int32(offs.numel() - 1), fo, C.c_int32(len(fo)), C.c_void_p(sd.ctypes.data),
                        C.byref(cp) if cp is not None else None, C.byref(d.handle)))
         d._targets_keepalive = targets     # device targets must outlive the queued kernels
         return d
@@ -498,14 +508,14 @@ class Context:
     def sample(self, targets: torch.Tensor, fanouts, seed: int, caps=None, out: Dense | None = None) -> Dense:
         assert targets.dtype == torch.int32
         targets = targets.contiguous()
-        fo = _host(list(fanouts), torch.int32)
+        fo = _fanouts(fanouts)
         d = out if out is not None else Dense(self)
         cp = None
         if caps is not None:
             cp = SampleCaps(int(caps.get("max_nodes_total", 0)), int(caps.get("max_entries_total", 0)),
                             int(caps.get("max_nodes_per_batch", 0)), int(caps.get("max_inner_nodes_per_batch", 0)))
         self._check(self.lib.mg_sample(self.handle, _ptr(targets), C.c_int(targets.is_cuda), C.c_int32(targets.numel()),
-                                       _ptr(fo), C.c_int32(fo.numel()), C.c_uint64(int(seed) & 0xFFFFFFFFFFFFFFFF),
+                                       fo, C.c_int32(len(fo)), C.c_uint64(int(seed) & 0xFFFFFFFFFFFFFFFF),
                                        C.byref(cp) if cp is not None else None, C.byref(d.handle)))
         return d
 

@@ -624,6 +624,13 @@ extern "C" int mg_lp_view(const mg_lp_batch* lp, int32_t* n_targets, const int32
     return MG_OK;
 }
 
+extern "C" int mg_lp_targets(mg_ctx* ctx, const mg_lp_batch* lp, int32_t* dst_dev, void* stream) {
+    if (!ctx) return MG_ERR_ARG;
+    if (!lp || !dst_dev) return mg_fail(ctx, MG_ERR_ARG, "null argument");
+    MG_CUDA(ctx, cudaMemcpyAsync(dst_dev, lp->targets, sizeof(int32_t) * (size_t)lp->n_targets, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
+    return MG_OK;
+}
+
 extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float* h_dev, int32_t dim, const float* rel_emb_dev,
                                  int32_t n_relations, int corrupt, int gemm_precision, float* pos_out, float* neg_dst_out, float* neg_src_out) {
     if (!ctx) return MG_ERR_ARG;
@@ -676,7 +683,8 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
             ctx->launches++;
             ta.b_images = (const uint8_t*)ctx->dm_images;
             const size_t smem = (size_t)ta.n_slices * 16384 + 2 * (size_t)ta.n_slices * ta.bn_max * 128 + 1024;
-            MG_CUDA(ctx, cudaFuncSetAttribute(k_distmult_neg_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            static uint64_t smem_done = 0;
+            MG_CUDA(ctx, mg_smem_limit(&smem_done, ctx->device, (const void*)k_distmult_neg_tc, kTcMaxSlices * (16384 + 2 * kTcBlockN * 128) + 1024));
             const unsigned blocks = (unsigned)(a.tiles_per_chunk * lp->n_chunks);
             if (corrupt & MG_CORRUPT_DST) {
                 a.keep_idx = lp->src_idx; a.out = neg_dst_out; ta.base = a;
