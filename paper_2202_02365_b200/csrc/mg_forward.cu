@@ -19,7 +19,6 @@
 int mg_gemm_tf32(mg_ctx* ctx, const float* x, const float* w_t, const float* bias, float* out, int64_t M, int N, int K,
                  bool relu);  // mg_gemm_tcgen05.cu
 int mg_gemm_tf32_status(mg_ctx* ctx);
-int mg_gemm_tf32_splitk_add_rows(mg_ctx* ctx, const float* x, const float* g, float* out, int M, int N, int64_t K, int kt_per_slice);
 // mg_layer_fused.cu
 bool mg_layer_fused_supported(int d_in, int d_out);
 int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int4* meta, const int64_t* start /* [k + 2], layer l at start[l] */);
@@ -27,6 +26,9 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
                    const float* h_prev, float* h_out, float* h_out2 /* nullable: the rows once more */, int flags /* 1 = ReLU, 2 = sum instead of mean */, const int4* row_meta,
                    int64_t row_lo, int64_t row_hi, int64_t safe_src_row, const void* w_pad_h /* the layer's fp16 weights, nullable */,
                    int in_f16 /* layers >= 2: h_prev holds fp16 rows */, int out_f16 /* h_out receives fp16 rows */);
+
+int mg_layer_grad_weights(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* h_prev, const float* dpre, const int4* row_meta,
+                          int sum_aggr, float* dw);
 
 namespace {
 
@@ -1242,7 +1244,7 @@ extern "C" int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d
         if (cudaMalloc((void**)&m->zeros, sizeof(float) * 2 * 1024) != cudaSuccess) { cudaGetLastError(); return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
         MG_CUDA(ctx, cudaMemsetAsync(m->zeros, 0, sizeof(float) * 2 * 1024, st));
     }
-    // scratch: dH^1 .. dH^{k-1}, the X and dX rows of a chunk, the turned-round entries of the layers whose dX is handed down
+    // scratch: dH^1 .. dH^{k-1}, the X rows of a chunk (fp32 products only), dX of a layer, the turned-round entries of the layers whose dX is handed down
     size_t g_off[MG_MAX_HOPS + 1] = {0}, g_total = 0, h_off[MG_MAX_HOPS + 1] = {0}, h_total = 0;
     for (int l = 1; l < k; ++l) {
         g_off[l] = g_total; g_total += ((size_t)d->h_hdr.rows_total[l] * m->dims[l] + 7) / 8 * 8;   // (32-byte aligned starts)
@@ -1256,7 +1258,8 @@ extern "C" int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d
     memset(&ra, 0, sizeof(ra));
     ra.l0 = d_h0_dev ? 1 : 2;
     for (int l = 1; l <= k; ++l) {
-        max_x = std::max<int64_t>(max_x, std::min<int64_t>(bw_mult * chunk_rows_for(m->dims[l - 1]), d->h_hdr.rows_total[l]) * 2 * m->dims[l - 1]);
+        if (m->precision == MG_GEMM_FP32)
+            max_x = std::max<int64_t>(max_x, std::min<int64_t>(bw_mult * chunk_rows_for(m->dims[l - 1]), d->h_hdr.rows_total[l]) * 2 * m->dims[l - 1]);
         const bool down = l >= ra.l0;
         const int64_t entries = down ? d->h_hdr.ent_base[k - l + 1] : 0;
         if (down) max_dx = std::max<int64_t>(max_dx, (int64_t)d->h_hdr.rows_total[l] * 2 * m->dims[l - 1]);
@@ -1315,8 +1318,17 @@ extern "C" int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d
         }
         const float* h_prev = l > 1 ? ctx->ws_h[0] + h_off[l - 1] : nullptr;
         float* g_in = l > 1 ? ctx->bw_g + g_off[l - 1] : d_h0_dev;
+        int64_t meta_at = 0;   // the layer's rows in ws_meta
+        for (int q = 1; q < l; ++q) meta_at += d->h_hdr.rows_total[q];
+        if (m->precision == MG_GEMM_TF32) {
+            // dW += X^T dPre with X gathered again inside the kernel; the row metadata is what the forward pass left (its layers all
+            // have it, mg_forward of this very model and sample was the last to write it)
+            if ((rc = mg_layer_grad_weights(ctx, d, l, d_in, d_out, h_prev, dpre_all, ctx->ws_meta + meta_at, m->sum_aggr ? 1 : 0, m->g_w_cat[l - 1]))) return rc;
+            // dX = dPre W^T on the tensor cores: the K-major operand the kernel wants is W itself ([2 d_in, d_out])
+            if (g_in && (rc = mg_gemm_tf32(ctx, dpre_all, m->w_cat[l - 1], m->zeros, ctx->bw_dx, M, 2 * d_in, d_out, false))) return rc;
+        }
         const int64_t chunk = bw_mult * chunk_rows_for(d_in);
-        for (int64_t r0 = 0; r0 < M; r0 += chunk) {
+        for (int64_t r0 = 0; r0 < M && m->precision == MG_GEMM_FP32; r0 += chunk) {
             const int64_t r1 = std::min(M, r0 + chunk), rows = r1 - r0;
             AggArgs a;
             a.B = B; a.k = k; a.layer = l; a.d_in = d_in;
@@ -1333,30 +1345,14 @@ extern "C" int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d
             if (l == 1) { if (half) launch_aggregate<true, true>(a, grid, st); else launch_aggregate<true, false>(a, grid, st); }
             else launch_aggregate<false, false>(a, grid, st);
             const float* dpre = dpre_all + r0 * d_out;
-            if (m->precision == MG_GEMM_TF32) {
-                // dW += X^T dPre as a tcgen05 GEMM whose contraction runs over the chunk's rows: both operands are read
-                // as they lie (rows x columns, the columns contiguous), the contraction is split over CTAs
-                const int m_tiles = (2 * d_in + 127) / 128, n_tiles = (d_out + 255) / 256;
-                const int64_t steps = (rows + 31) / 32;
-                const int per_slice = (int)std::max<int64_t>(16, (steps * m_tiles * n_tiles + 4 * ctx->n_sms - 1) / (4 * ctx->n_sms));
-                if ((rc = mg_gemm_tf32_splitk_add_rows(ctx, ctx->bw_x, dpre, m->g_w_cat[l - 1], 2 * d_in, d_out, rows, per_slice))) return rc;
-            } else {
-                const unsigned slices = (unsigned)((rows + kGradRowsPerBlock - 1) / kGradRowsPerBlock);
-                dim3 gw((unsigned)((2 * d_in + 63) / 64), (unsigned)((d_out + 63) / 64), slices);
-                k_grad_weights<<<gw, 256, 0, st>>>(ctx->bw_x, dpre, m->g_w_cat[l - 1], rows, 2 * d_in, d_out);
-                ctx->launches++;
-            }
-            ctx->launches++;   // (the aggregation above)
+            const unsigned slices = (unsigned)((rows + kGradRowsPerBlock - 1) / kGradRowsPerBlock);
+            dim3 gw((unsigned)((2 * d_in + 63) / 64), (unsigned)((d_out + 63) / 64), slices);
+            k_grad_weights<<<gw, 256, 0, st>>>(ctx->bw_x, dpre, m->g_w_cat[l - 1], rows, 2 * d_in, d_out);
+            ctx->launches += 2;
             if (!g_in) continue;   // layer 1 without a gradient of the base representations
-            float* dx = ctx->bw_dx + r0 * 2 * d_in;
-            if (m->precision == MG_GEMM_TF32) {
-                // dX = dPre W^T on the tensor cores: the K-major operand the kernel wants is W itself ([2 d_in, d_out])
-                if ((rc = mg_gemm_tf32(ctx, dpre, m->w_cat[l - 1], m->zeros, dx, rows, 2 * d_in, d_out, false))) return rc;
-            } else {
-                dim3 gx((unsigned)((rows + 63) / 64), (unsigned)((2 * d_in + 63) / 64));
-                k_gemm_fp32<false><<<gx, 256, 0, st>>>(dpre, m->w_cat_t[l - 1], m->zeros, dx, rows, 2 * d_in, d_out);
-                ctx->launches++;
-            }
+            dim3 gx((unsigned)((rows + 63) / 64), (unsigned)((2 * d_in + 63) / 64));
+            k_gemm_fp32<false><<<gx, 256, 0, st>>>(dpre, m->w_cat_t[l - 1], m->zeros, ctx->bw_dx + r0 * 2 * d_in, rows, 2 * d_in, d_out);
+            ctx->launches++;
         }
         const int64_t rows_in = d->h_hdr.rows_total[l - 1];
         if (!g_in || rows_in == 0) continue;

@@ -190,6 +190,152 @@ template <> struct PieceSum<true> {
     static __device__ __forceinline__ uint4 self_operand(const uint4& r) { return r; }   // fp16 rows are operands as they are
 };
 
+// A planner warp's work on one row block, lane = row: the rows' metadata, their entries translated to source rows, each row's
+// first kUnroll source rows, all in shared memory.
+template <bool FIRST>
+__device__ __forceinline__ void plan_block(const FusedArgs& a, const int32_t* keys, int4 rm, RowMeta* meta, int32_t* src_rows, int32_t (*first_rows)[8],
+                                           int32_t* plan_total) {
+    const int lane = threadIdx.x & 31;
+    const int32_t end = (int32_t)warp_incl_scan((uint32_t)max(rm.z, 0));   // end of the row's cached entries
+    const int32_t total = __shfl_sync(0xFFFFFFFFu, end, 31);
+    const bool cached = total <= kKeyCap;
+    const int32_t in_base = rm.w, koff = end - max(rm.z, 0);
+    meta[lane] = make_int4(rm.x, rm.y, rm.z, cached ? koff : in_base);
+    const int32_t zmax = (int32_t)__reduce_max_sync(0xFFFFFFFFu, (uint32_t)max(rm.z, 0));
+    if (cached && zmax <= kLaneEntries) {
+        // short rows (the usual case): every lane translates its own row's entries, kUnroll loads in flight
+        // (the entries of consecutive rows are consecutive, so the lanes' loads share their cache lines)
+        for (int32_t i0 = 0; i0 < zmax; i0 += kUnroll) {
+            int32_t key[kUnroll];
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) key[u] = i0 + u < rm.z ? __ldg(keys + rm.y + i0 + u) : 0;
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u)
+                if (i0 + u < rm.z) src_rows[koff + i0 + u] = source_row<FIRST>(a, in_base, key[u]);
+        }
+    } else if (cached) {
+        // entry j belongs to the first row whose end exceeds j
+        for (int32_t j0 = 0; j0 < total; j0 += 32 * 4) {
+            int32_t key[4], base[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int32_t j = j0 + u * 32 + lane;
+                int lo = 0, hi = 31;
+#pragma unroll
+                for (int s = 0; s < 5; ++s) {
+                    const int mid = (lo + hi) >> 1;
+                    const int32_t e = __shfl_sync(0xFFFFFFFFu, end, mid);
+                    if (lo < hi) { if (e > j) hi = mid; else lo = mid + 1; }
+                }
+                const int32_t e0 = __shfl_sync(0xFFFFFFFFu, rm.y, lo), k0 = __shfl_sync(0xFFFFFFFFu, koff, lo);
+                base[u] = __shfl_sync(0xFFFFFFFFu, in_base, lo);
+                key[u] = j < total ? __ldg(keys + e0 + (j - k0)) : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int32_t j = j0 + u * 32 + lane;
+                if (j < total) src_rows[j] = source_row<FIRST>(a, base[u], key[u]);
+            }
+        }
+    }
+    if (lane == 0) *plan_total = cached ? total : -1;
+    __syncwarp();
+    if (cached) {
+        // lane = row: its first kUnroll source rows, padded with its own source row
+        int32_t fr[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) fr[j] = (j < kUnroll && j < rm.z) ? src_rows[koff + j] : rm.x;
+        fr[5] = __float_as_int(rm.z > 0 ? (a.sum_aggr ? 1.f : 1.f / (float)rm.z) : 0.f);   // the mean's factor (1 for a sum)
+        *reinterpret_cast<int4*>(&first_rows[lane][0]) = make_int4(fr[0], fr[1], fr[2], fr[3]);
+        *reinterpret_cast<int4*>(&first_rows[lane][4]) = make_int4(fr[4], fr[5], fr[6], fr[7]);
+        __syncwarp();
+    }
+}
+
+// A gather warp's work on two planned rows: the lane's 16-byte operand pieces of each row's self part and aggregate.
+// (RAW: fp32 values as they are, not rounded to the operand's precision.)
+template <bool FIRST, bool HALF, bool F16, bool RAW = false>
+__device__ __forceinline__ void gather_rows(const FusedArgs& a, const char* src, bool on, bool cached, const RowMeta* meta, const int32_t (*first_rows)[8],
+                                            const int32_t* rows_of, uint4* selfv, uint4* meanv) {
+    RowMeta mq[kRowsInFlight];
+    PieceSum<F16> acc[kRowsInFlight];
+    int top = 0;
+#pragma unroll
+    for (int q2 = 0; q2 < kRowsInFlight; ++q2) {
+        mq[q2] = meta[q2];
+        selfv[q2] = make_uint4(0u, 0u, 0u, 0u);
+        meanv[q2] = selfv[q2];
+        acc[q2].zero();
+        top = max(top, mq[q2].z);
+    }
+    if (on) {
+#pragma unroll
+        for (int q2 = 0; q2 < kRowsInFlight; ++q2)
+            selfv[q2] = load_piece<HALF, F16>(src + (size_t)(uint32_t)mq[q2].x * (size_t)a.src_row_bytes);
+        if (cached) {
+            // Every load is issued unconditionally: a slot past the end of a row's entries re-reads
+            // the row's own representation (a cache hit) and is not added.  Branch-free code is what
+            // lets all loads of a round be in flight together.  First round: the planner has laid
+            // out the kUnroll source rows per row, padding included.
+            {
+                uint4 v[kRowsInFlight][kUnroll];
+#pragma unroll
+                for (int q2 = 0; q2 < kRowsInFlight; ++q2) {
+                    const int4 f4 = *reinterpret_cast<const int4*>(first_rows[q2]);
+                    const int32_t f5 = first_rows[q2][4];
+                    v[q2][0] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f4.x * (size_t)a.src_row_bytes);
+                    v[q2][1] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f4.y * (size_t)a.src_row_bytes);
+                    v[q2][2] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f4.z * (size_t)a.src_row_bytes);
+                    v[q2][3] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f4.w * (size_t)a.src_row_bytes);
+                    v[q2][4] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f5 * (size_t)a.src_row_bytes);
+                }
+#pragma unroll
+                for (int j = 0; j < kUnroll; ++j)   // entry order
+#pragma unroll
+                    for (int q2 = 0; q2 < kRowsInFlight; ++q2)
+                        if (j < mq[q2].z) acc[q2].add(v[q2][j]);
+            }
+            for (int e = kUnroll; e < top; e += kUnroll) {
+                uint4 v[kRowsInFlight][kUnroll];
+#pragma unroll
+                for (int j = 0; j < kUnroll; ++j)
+#pragma unroll
+                    for (int q2 = 0; q2 < kRowsInFlight; ++q2) {
+                        const bool live = e + j < mq[q2].z;
+                        const int32_t sr = rows_of[live ? mq[q2].w + e + j : 0];
+                        v[q2][j] = load_piece<HALF, F16>(src + (size_t)(uint32_t)(live ? sr : mq[q2].x) * (size_t)a.src_row_bytes);
+                    }
+#pragma unroll
+                for (int j = 0; j < kUnroll; ++j)   // entry order
+#pragma unroll
+                    for (int q2 = 0; q2 < kRowsInFlight; ++q2)
+                        if (e + j < mq[q2].z) acc[q2].add(v[q2][j]);   // warp-uniform: predicated adds, not a branch around a load
+            }
+        } else {
+            // a row block with more entries than the shared-memory cache holds: plain per-entry loop
+            const int32_t* keys = FIRST ? a.ent_nbrs : a.ent_repr;
+#pragma unroll
+            for (int q2 = 0; q2 < kRowsInFlight; ++q2)
+                for (int e = 0; e < mq[q2].z; ++e) {
+                    const int32_t sr = source_row<FIRST>(a, mq[q2].w, __ldg(keys + mq[q2].y + e));
+                    acc[q2].add(load_piece<HALF, F16>(src + (size_t)(uint32_t)sr * (size_t)a.src_row_bytes));
+                }
+        }
+#pragma unroll
+        for (int q2 = 0; q2 < kRowsInFlight; ++q2) {
+            const float inv = cached ? __int_as_float(first_rows[q2][5])
+                                     : (mq[q2].z > 0 ? (a.sum_aggr ? 1.f : 1.f / (float)mq[q2].z) : 0.f);
+            if (RAW) {
+                meanv[q2] = make_uint4(__float_as_uint(acc[q2].a[0] * inv), __float_as_uint(acc[q2].a[1] * inv), __float_as_uint(acc[q2].a[2] * inv),
+                                       __float_as_uint(acc[q2].a[3] * inv));
+                continue;
+            }
+            meanv[q2] = acc[q2].operand(inv);
+            selfv[q2] = PieceSum<F16>::self_operand(selfv[q2]);
+        }
+    }
+}
+
 // TS: the weights stay in tensor memory for the whole kernel and are the MMAs' first operand (M = 256 output columns over
 // the pair, a CTA's 128 in its 128 lanes, K <= 256 columns), the gathered rows the second (N = 128: a half tile of either
 // CTA); the accumulator is the transposed output, [output column][row].  Nothing is streamed per half tile then -- with
@@ -425,60 +571,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
             const int64_t r = a.row_lo + t * TM + (q % kBlocks) * kBlockRows + lane;
             int4 rm = make_int4(a.safe_src, 0, -1, 0);
             if (r < a.M) rm = __ldg(a.row_meta + r);   // (self source row, first entry, count, first H^{l-1} row of the batch)
-            const int32_t end = (int32_t)warp_incl_scan((uint32_t)max(rm.z, 0));   // end of the row's cached entries
-            const int32_t total = __shfl_sync(0xFFFFFFFFu, end, 31);
-            const bool cached = total <= kKeyCap;
-            const int32_t in_base = rm.w, koff = end - max(rm.z, 0);
-            meta[slot][lane] = make_int4(rm.x, rm.y, rm.z, cached ? koff : in_base);
-            const int32_t zmax = (int32_t)__reduce_max_sync(0xFFFFFFFFu, (uint32_t)max(rm.z, 0));
-            if (cached && zmax <= kLaneEntries) {
-                // short rows (the usual case): every lane translates its own row's entries, kUnroll loads in flight
-                // (the entries of consecutive rows are consecutive, so the lanes' loads share their cache lines)
-                for (int32_t i0 = 0; i0 < zmax; i0 += kUnroll) {
-                    int32_t key[kUnroll];
-#pragma unroll
-                    for (int u = 0; u < kUnroll; ++u) key[u] = i0 + u < rm.z ? __ldg(keys + rm.y + i0 + u) : 0;
-#pragma unroll
-                    for (int u = 0; u < kUnroll; ++u)
-                        if (i0 + u < rm.z) src_rows[slot][koff + i0 + u] = source_row<FIRST>(a, in_base, key[u]);
-                }
-            } else if (cached) {
-                // entry j belongs to the first row whose end exceeds j
-                for (int32_t j0 = 0; j0 < total; j0 += 32 * 4) {
-                    int32_t key[4], base[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int32_t j = j0 + u * 32 + lane;
-                        int lo = 0, hi = 31;
-#pragma unroll
-                        for (int s = 0; s < 5; ++s) {
-                            const int mid = (lo + hi) >> 1;
-                            const int32_t e = __shfl_sync(0xFFFFFFFFu, end, mid);
-                            if (lo < hi) { if (e > j) hi = mid; else lo = mid + 1; }
-                        }
-                        const int32_t e0 = __shfl_sync(0xFFFFFFFFu, rm.y, lo), k0 = __shfl_sync(0xFFFFFFFFu, koff, lo);
-                        base[u] = __shfl_sync(0xFFFFFFFFu, in_base, lo);
-                        key[u] = j < total ? __ldg(keys + e0 + (j - k0)) : 0;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int32_t j = j0 + u * 32 + lane;
-                        if (j < total) src_rows[slot][j] = source_row<FIRST>(a, base[u], key[u]);
-                    }
-                }
-            }
-            if (lane == 0) plan_total[slot] = cached ? total : -1;
-            __syncwarp();
-            if (cached) {
-                // lane = row: its first kUnroll source rows, padded with its own source row
-                int32_t fr[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) fr[j] = (j < kUnroll && j < rm.z) ? src_rows[slot][koff + j] : rm.x;
-                fr[5] = __float_as_int(rm.z > 0 ? (a.sum_aggr ? 1.f : 1.f / (float)rm.z) : 0.f);   // the mean's factor (1 for a sum)
-                *reinterpret_cast<int4*>(&first_rows[slot][lane][0]) = make_int4(fr[0], fr[1], fr[2], fr[3]);
-                *reinterpret_cast<int4*>(&first_rows[slot][lane][4]) = make_int4(fr[4], fr[5], fr[6], fr[7]);
-                __syncwarp();
-            }
+            plan_block<FIRST>(a, keys, rm, meta[slot], src_rows[slot], first_rows[slot], &plan_total[slot]);
             if (lane == 0) mbar_arrive(&plan_full[slot]);
         }
     }
@@ -672,79 +765,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                     const bool cached = plan_total[slot] >= 0;
                     const int32_t* rows_of = src_rows[slot];
                     const int brow = pw * kRowsInFlight;              // this warp's first row inside the block
-                    RowMeta mq[kRowsInFlight];
                     uint4 selfv[kRowsInFlight], meanv[kRowsInFlight];   // the two operand pieces of each row
-                    PieceSum<F16> acc[kRowsInFlight];
-                    int top = 0;
-#pragma unroll
-                    for (int q2 = 0; q2 < kRowsInFlight; ++q2) {
-                        mq[q2] = meta[slot][brow + q2];
-                        selfv[q2] = make_uint4(0u, 0u, 0u, 0u);
-                        meanv[q2] = selfv[q2];
-                        acc[q2].zero();
-                        top = max(top, mq[q2].z);
-                    }
-                    if (col_ok && ok) {
-#pragma unroll
-                        for (int q2 = 0; q2 < kRowsInFlight; ++q2)
-                            selfv[q2] = load_piece<HALF, F16>(src + (size_t)(uint32_t)mq[q2].x * (size_t)a.src_row_bytes);
-                        if (cached) {
-                            // Every load is issued unconditionally: a slot past the end of a row's entries re-reads
-                            // the row's own representation (a cache hit) and is not added.  Branch-free code is what
-                            // lets all loads of a round be in flight together.  First round: the planner has laid
-                            // out the kUnroll source rows per row, padding included.
-                            {
-                                uint4 v[kRowsInFlight][kUnroll];
-#pragma unroll
-                                for (int q2 = 0; q2 < kRowsInFlight; ++q2) {
-                                    const int4 f4 = *reinterpret_cast<const int4*>(first_rows[slot][brow + q2]);
-                                    const int32_t f5 = first_rows[slot][brow + q2][4];
-                                    v[q2][0] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f4.x * (size_t)a.src_row_bytes);
-                                    v[q2][1] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f4.y * (size_t)a.src_row_bytes);
-                                    v[q2][2] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f4.z * (size_t)a.src_row_bytes);
-                                    v[q2][3] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f4.w * (size_t)a.src_row_bytes);
-                                    v[q2][4] = load_piece<HALF, F16>(src + (size_t)(uint32_t)f5 * (size_t)a.src_row_bytes);
-                                }
-#pragma unroll
-                                for (int j = 0; j < kUnroll; ++j)   // entry order
-#pragma unroll
-                                    for (int q2 = 0; q2 < kRowsInFlight; ++q2)
-                                        if (j < mq[q2].z) acc[q2].add(v[q2][j]);
-                            }
-                            for (int e = kUnroll; e < top; e += kUnroll) {
-                                uint4 v[kRowsInFlight][kUnroll];
-#pragma unroll
-                                for (int j = 0; j < kUnroll; ++j)
-#pragma unroll
-                                    for (int q2 = 0; q2 < kRowsInFlight; ++q2) {
-                                        const bool live = e + j < mq[q2].z;
-                                        const int32_t sr = rows_of[live ? mq[q2].w + e + j : 0];
-                                        v[q2][j] = load_piece<HALF, F16>(src + (size_t)(uint32_t)(live ? sr : mq[q2].x) * (size_t)a.src_row_bytes);
-                                    }
-#pragma unroll
-                                for (int j = 0; j < kUnroll; ++j)   // entry order
-#pragma unroll
-                                    for (int q2 = 0; q2 < kRowsInFlight; ++q2)
-                                        if (e + j < mq[q2].z) acc[q2].add(v[q2][j]);   // warp-uniform: predicated adds, not a branch around a load
-                            }
-                        } else {
-                            // a row block with more entries than the shared-memory cache holds: plain per-entry loop
-                            const int32_t* keys = FIRST ? a.ent_nbrs : a.ent_repr;
-#pragma unroll
-                            for (int q2 = 0; q2 < kRowsInFlight; ++q2)
-                                for (int e = 0; e < mq[q2].z; ++e) {
-                                    const int32_t sr = source_row<FIRST>(a, mq[q2].w, __ldg(keys + mq[q2].y + e));
-                                    acc[q2].add(load_piece<HALF, F16>(src + (size_t)(uint32_t)sr * (size_t)a.src_row_bytes));
-                                }
-                        }
-#pragma unroll
-                        for (int q2 = 0; q2 < kRowsInFlight; ++q2) {
-                            const float inv = cached ? __int_as_float(first_rows[slot][brow + q2][5])
-                                                     : (mq[q2].z > 0 ? (a.sum_aggr ? 1.f : 1.f / (float)mq[q2].z) : 0.f);
-                            meanv[q2] = acc[q2].operand(inv);
-                            selfv[q2] = PieceSum<F16>::self_operand(selfv[q2]);
-                        }
-                    }
+                    gather_rows<FIRST, HALF, F16>(a, src, col_ok && ok, cached, &meta[slot][brow], &first_rows[slot][brow], rows_of, selfv, meanv);
                     if (grp == n_groups - 1) {
                         // the block's plan has been read for the last time: its slot may be planned again
                         __syncwarp();
@@ -793,6 +815,180 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
     if (warp == kMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)a.tmem_cols) : "memory");
+    }
+}
+
+// ---- weight gradients: dW += [self | aggregate]^T dPre --------------------------------------------------------------------
+// The layer's operand is gathered again, block by block of 32 rows, straight into shared memory, and contracted over the rows with
+// the gradient rows that TMA brings; it never exists in memory (before: an aggregation kernel wrote it, 1 to 2 KB per row, and a
+// product over split chunks read it back).  Bound by the gather like the forward layer.  A CTA owns 128 input columns -- their
+// self and aggregate halves are the two M = 128 tiles of its accumulators, all 512 columns of tensor memory with 256 output
+// columns -- and every n_slices-th block of rows; at the end it adds its 256 x 256 sums to dW with 16-byte reductions.  24 mini-batches of
+// 1,000 targets on 2M nodes: 540k rows of 2 x 128 in 252 us (257 + 190 before), 91k + 24k rows of 2 x 256 in 188 us (178 + 100).
+// Both operands lie with the contraction across rows ("MN-major"): boxes of 32 rows x 32 floats, swizzled in 32-byte units.
+//   warps 0..15  gather, two rows each per block     warps 16..19  planners     warp 20  TMA     warp 21  MMA, tensor memory
+constexpr int kGradPlanners = 4, kGradFirstPlanner = 16, kGradTmaWarp = 20, kGradMmaWarp = 21;
+constexpr int kGradThreads = (kGradMmaWarp + 1) * 32;   // 704
+constexpr int kGradStages = 2;                          // (two leave the gathers 92 KB of L1: the MMAs of a block take a fifth of its gather)
+constexpr uint32_t kGradBox = kBlockRows * 128, kGradStageX = 8 * kGradBox;
+
+struct GradWArgs {
+    FusedArgs f;          // rows, entries, sources of the layer; N, d_in, M
+    int32_t n_slices, col_groups, n_cols;   // n_cols: output columns of a CTA, a multiple of 32, at most 256
+    float* dw;            // [2 d_in, N]
+};
+
+template <bool FIRST, bool HALF>
+__global__ void __launch_bounds__(kGradThreads, 1) k_sage_grad_weights(const __grid_constant__ CUtensorMap map_g, GradWArgs p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t x_ready[kGradStages], g_full[kGradStages], stage_free[kGradStages], acc_full;
+    __shared__ uint64_t plan_full[kPlanSlots], plan_empty[kPlanSlots];
+    __shared__ uint32_t tmem_slot;
+    __shared__ RowMeta meta[kPlanSlots][kBlockRows];
+    __shared__ int32_t src_rows[kPlanSlots][kKeyCap];
+    __shared__ int32_t plan_total[kPlanSlots];
+    __shared__ __align__(16) int32_t first_rows[kPlanSlots][kBlockRows][8];
+    const FusedArgs& a = p.f;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int col0 = (int)(blockIdx.y % p.col_groups) * kGroupCols, n0 = (int)(blockIdx.y / p.col_groups) * 256;
+    const int bn = min(p.n_cols, (a.N - n0 + 31) / 32 * 32);
+    uint8_t* x_base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* g_base = x_base + kGradStages * kGradStageX;
+    const uint32_t g_bytes = (uint32_t)(p.n_cols / 32) * kGradBox;   // a stage of gradient rows
+    const int64_t blocks = (a.M + kBlockRows - 1) / kBlockRows;
+    const uint32_t my = (int64_t)blockIdx.x < blocks ? (uint32_t)((blocks - blockIdx.x + p.n_slices - 1) / p.n_slices) : 0u;
+    auto first_row = [&](uint32_t it) -> int64_t { return ((int64_t)blockIdx.x + (int64_t)it * p.n_slices) * kBlockRows; };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kGradStages; ++s) { mbar_init(&x_ready[s], kProducerWarps); mbar_init(&g_full[s], 1); mbar_init(&stage_free[s], 1); }
+        mbar_init(&acc_full, 1);
+        for (int s = 0; s < kPlanSlots; ++s) { mbar_init(&plan_full[s], 1); mbar_init(&plan_empty[s], kProducerWarps); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_g) : "memory");
+    }
+    if (warp == kGradMmaWarp) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"((uint32_t)a.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_slot;
+    const uint32_t acc_cols = (uint32_t)a.tmem_cols / 2;   // the aggregate half's accumulator starts here
+
+    if (warp < kProducerWarps) {
+        const int col = col0 + lane * 4;
+        const bool col_ok = col < a.d_in;
+        const char* src = a.src_base + (size_t)col * (HALF ? 2 : 4);
+        const int brow = warp * kRowsInFlight;
+        bool ok = true;
+        for (uint32_t it = 0; it < my; ++it) {
+            const int slot = it % kPlanSlots, s = it % kGradStages;
+            if (ok && !mbar_wait(&plan_full[slot], (it / kPlanSlots) & 1)) { if (lane == 0) report(a.error, 41u); ok = false; }
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (!ok) break;
+            uint4 selfv[kRowsInFlight], meanv[kRowsInFlight];
+            gather_rows<FIRST, HALF, false, true>(a, src, col_ok, plan_total[slot] >= 0, &meta[slot][brow], &first_rows[slot][brow], src_rows[slot], selfv, meanv);
+#pragma unroll
+            for (int q = 0; q < kRowsInFlight; ++q)   // a row past the end meets a gradient row of zeros: it only has to be finite
+                if (meta[slot][brow + q].z < 0) selfv[q] = make_uint4(0u, 0u, 0u, 0u);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&plan_empty[slot]);
+            if (it >= (uint32_t)kGradStages && !mbar_wait(&stage_free[s], ((it / kGradStages) - 1) & 1)) { if (lane == 0) report(a.error, 42u); ok = false; }
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (!ok) break;
+            if (col_ok) {
+                // box lane / 8 of the half; the 32-byte pieces of a row are exchanged by the row number mod 4
+                uint8_t* xs = x_base + (size_t)s * kGradStageX + (size_t)(lane >> 3) * kGradBox;
+#pragma unroll
+                for (int q = 0; q < kRowsInFlight; ++q) {
+                    const int row = brow + q;
+                    const size_t off = (size_t)row * 128 + (size_t)((((lane & 7) >> 1) ^ (row & 3)) << 5) + (size_t)((lane & 1) << 4);
+                    *reinterpret_cast<uint4*>(xs + off) = selfv[q];
+                    *reinterpret_cast<uint4*>(xs + 4 * kGradBox + off) = meanv[q];
+                }
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&x_ready[s]);
+        }
+        // the CTA's sums: warp = a quarter of the accumulators' lanes (input columns) x every fourth 32 output columns
+        if (my > 0 && ok) {
+            ok = mbar_wait(&acc_full, 0);
+            if (!ok && lane == 0) report(a.error, 43u);
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            tc_fence_after();
+            const int quarter = warp & 3, c = col0 + quarter * 32 + lane;
+            for (int part = 0; part < 2 && ok; ++part)
+                for (int j0 = (warp >> 2) * 32; j0 < bn; j0 += 128) {
+                    uint32_t v[32];
+                    tmem_ld_32(tmem_base + part * acc_cols + ((uint32_t)(quarter * 32) << 16) + (uint32_t)j0, v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (c >= a.d_in) continue;
+                    float4* dst = reinterpret_cast<float4*>(p.dw + (int64_t)(part * a.d_in + c) * a.N + n0 + j0);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (n0 + j0 + 4 * j < a.N)
+                            atomicAdd(dst + j, make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]), __uint_as_float(v[4 * j + 2]),
+                                                           __uint_as_float(v[4 * j + 3])));
+                }
+        }
+    } else if (warp < kGradTmaWarp) {
+        const int32_t* keys = FIRST ? a.ent_nbrs : a.ent_repr;
+        bool ok = true;
+        for (uint32_t it = warp - kGradFirstPlanner; it < my; it += kGradPlanners) {
+            const int slot = it % kPlanSlots;
+            if (it >= (uint32_t)kPlanSlots && !mbar_wait(&plan_empty[slot], ((it / kPlanSlots) - 1) & 1)) { if (lane == 0) report(a.error, 44u); ok = false; }
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (!ok) break;
+            const int64_t r = first_row(it) + lane;
+            int4 rm = make_int4(a.safe_src, 0, -1, 0);
+            if (r < a.M) rm = __ldg(a.row_meta + r);
+            plan_block<FIRST>(a, keys, rm, meta[slot], src_rows[slot], first_rows[slot], &plan_total[slot]);
+            if (lane == 0) mbar_arrive(&plan_full[slot]);
+        }
+    } else if (warp == kGradTmaWarp) {
+        if (lane == 0) {
+            uint32_t it = 0;
+            for (; it < my; ++it) {
+                const int s = it % kGradStages;
+                if (it >= (uint32_t)kGradStages && !mbar_wait(&stage_free[s], ((it / kGradStages) - 1) & 1)) { report(a.error, 45u); break; }
+                mbar_expect_tx(&g_full[s], (uint32_t)(bn / 32) * kGradBox);
+                for (int j = 0; j < bn / 32; ++j)   // (rows past the end and columns past the width come as zeros)
+                    tma_load_2d(g_base + (size_t)s * g_bytes + (size_t)j * kGradBox, &map_g, &g_full[s], n0 + 32 * j, (int)first_row(it));
+            }
+            // nothing of this CTA's may be in flight when it ends
+            for (uint32_t i = it >= (uint32_t)kGradStages ? it - kGradStages : 0; i < it; ++i)
+                if (!mbar_wait(&g_full[i % kGradStages], (i / kGradStages) & 1)) report(a.error, 46u);
+        }
+        __syncwarp();
+    } else {
+        if (lane == 0 && my > 0) {
+            // fp32 accumulate, TF32 x TF32, the contiguous dimension of both operands is M (N): bits 15 and 16
+            const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+            bool ok = true;
+            for (uint32_t it = 0; it < my && ok; ++it) {
+                const int s = it % kGradStages;
+                if (!mbar_wait(&g_full[s], (it / kGradStages) & 1) || !mbar_wait(&x_ready[s], (it / kGradStages) & 1)) { report(a.error, 47u); ok = false; break; }
+                tc_fence_after();
+                const uint64_t db = smem_desc_sw128_mn(smem_u32(g_base + (size_t)s * g_bytes), kGradBox);
+                for (int part = 0; part < 2; ++part) {
+                    const uint64_t da = smem_desc_sw128_mn(smem_u32(x_base + (size_t)s * kGradStageX + (size_t)part * 4 * kGradBox), kGradBox);
+#pragma unroll
+                    for (int kk = 0; kk < kBlockRows / 8; ++kk)   // 8 rows of every box = 1024 bytes further on
+                        mma_tf32(tmem_base + part * acc_cols, da + (uint64_t)(kk * 64), db + (uint64_t)(kk * 64), idesc, (it | kk) ? 1u : 0u);
+                }
+                mma_commit(&stage_free[s]);
+            }
+            if (ok) mma_commit(&acc_full);
+        }
+        __syncwarp();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == kGradMmaWarp) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)a.tmem_cols) : "memory");
     }
 }
 
@@ -973,6 +1169,43 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     pdl.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &pdl; cfg.numAttrs = 1;
     MG_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, mw, mo, mo2, a));
+    ctx->launches++;
+    MG_CUDA(ctx, cudaGetLastError());
+    return MG_OK;
+}
+
+// dw [2 d_in, d_out] += X^T dpre over the packed rows of layer `layer`, X = [self | aggregate]; row_meta: the layer's part of
+// mg_layer_rows' result.  dpre: DEVICE [rows, d_out], 16-byte aligned.
+int mg_layer_grad_weights(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* h_prev, const float* dpre, const int4* row_meta,
+                          int sum_aggr, float* dw) {
+    GradWArgs p;
+    memset(&p, 0, sizeof(p));
+    FusedArgs& a = p.f;
+    fill_args(ctx, d, layer, d_in, d_out, &a);
+    if (a.M <= 0) return MG_OK;
+    a.row_meta = row_meta;
+    a.src_base = layer == 1 ? ctx->slots : reinterpret_cast<const char*>(h_prev);
+    a.src_row_bytes = layer == 1 ? (uint32_t)ctx->row_bytes : (uint32_t)d_in * 4u;
+    a.sum_aggr = sum_aggr;
+    p.n_cols = std::min(256, (d_out + 31) / 32 * 32);
+    int cols = 32;
+    while (cols < p.n_cols) cols <<= 1;
+    a.tmem_cols = 2 * cols;
+    p.col_groups = (d_in + kGroupCols - 1) / kGroupCols;
+    const int groups = p.col_groups * ((d_out + 255) / 256);
+    // a CTA per SM; below eight blocks of rows each, the sums' way into dW would cost more than the rows
+    const int64_t blocks = (a.M + kBlockRows - 1) / kBlockRows;
+    p.n_slices = (int)std::max<int64_t>(1, std::min<int64_t>(ctx->n_sms / groups, (blocks + 7) / 8));
+    p.dw = dw;
+    CUtensorMap mg;
+    if (!make_map_f32(&mg, dpre, a.M, d_out, kBlockRows, true)) return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the gradient rows");
+    const size_t smem = kGradStages * (kGradStageX + (size_t)(p.n_cols / 32) * kGradBox) + 1024;
+    typedef void (*Kernel)(CUtensorMap, GradWArgs);
+    static const Kernel kernels[3] = {k_sage_grad_weights<true, false>, k_sage_grad_weights<true, true>, k_sage_grad_weights<false, false>};
+    static uint64_t smem_done[3] = {};
+    const int which = layer > 1 ? 2 : ctx->feat_dtype == MG_DTYPE_F16 ? 1 : 0;
+    MG_CUDA(ctx, mg_smem_limit(&smem_done[which], ctx->device, (const void*)kernels[which], (int)(kGradStages * (kGradStageX + 8 * kGradBox) + 1024)));
+    kernels[which]<<<dim3((unsigned)p.n_slices, (unsigned)groups), kGradThreads, smem, ctx->stream>>>(mg, p);
     ctx->launches++;
     MG_CUDA(ctx, cudaGetLastError());
     return MG_OK;

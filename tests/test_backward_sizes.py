@@ -92,3 +92,32 @@ def test_source_rows_named_by_few_and_by_many(dims, fanouts, aggregator):
             for i in torch.nonzero(want_ids[want] < 4).flatten().tolist():      # the centres' rows one by one
                 assert near(g_rows[at:at + n].cpu()[order][i], h.grad[want][i])
         at += n
+
+
+# one layer (no ReLU whose branch could differ): rows around a block of 32, around the rows that one CTA takes; widths of one to three
+# groups of input columns and one to three tiles of output columns
+@pytest.mark.parametrize("rows", [1, 31, 33, 257, 5_990])
+@pytest.mark.parametrize("d_in,d_out,half,aggregator", [(4, 4, False, "mean"), (128, 256, False, "mean"), (132, 300, False, "sum"), (264, 36, True, "mean"),
+                                                        (260, 516, False, "mean")])
+def test_weight_gradients_on_the_tensor_cores(rows, d_in, d_out, half, aggregator):
+    graph = star_graph()
+    feats = inputs.normal_features(N, d_in, seed=4, dtype=torch.float16 if half else torch.float32)
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(feats.cuda())
+    ctx.keep_layer_outputs(True)
+    layers = inputs.random_bias_layers([d_in, d_out], seed=5)
+    model = ctx.model(layers)
+    model.set_aggregator(aggregator)
+    dense = ctx.sample(inputs.distinct_targets(N, rows, seed=6), [6], 7)
+    out = torch.empty((rows, d_out), device="cuda")
+    ctx.forward(model, dense, out)
+    d_out_rows = torch.randn(out.shape, generator=torch.Generator("cuda").manual_seed(8), device="cuda")
+    grads, g_rows, ids = ctx.backward(model, dense, d_out_rows, want_h0_grad=True)
+    (want,), ((want_ids, h),) = reference([dense.view(0)], feats.float(), layers, [d_out_rows], aggregator)
+    # the tensor cores drop what is beyond ten bits of an operand that was not rounded before (gradient rows, the weights of dX): up to
+    # 2^-10 relative for each of the two, all in one direction where a row stands alone, so 2^-9 of the result's norm
+    for x, p in zip(grads[0], want):
+        assert float((x.double().cpu().reshape(p.shape) - p.grad).norm()) <= 2 ** -9 * float(p.grad.norm())
+    order, want_order = torch.argsort(ids.cpu()), torch.argsort(want_ids)
+    assert float((g_rows.double().cpu()[order] - h.grad[want_order]).norm()) <= 2 ** -9 * float(h.grad.norm())
