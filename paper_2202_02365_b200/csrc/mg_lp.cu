@@ -254,6 +254,12 @@ constexpr int kTcBlockN = 128;    // negatives per block
 struct NegTcArgs {
     NegArgs base;
     int32_t n_slices, bn_max, tmem_cols;
+    // Both corrupted sides run in one launch.  CTAs [0, n_whole) take a tile each, tile t of side t / (tiles of a side); the tiles
+    // behind them are cut into `parts` runs of negatives, so that the last round of CTAs fills the SMs (800 tiles on 148 SMs: five
+    // rounds and a half instead of twice three, 141 us either way; 80 tiles of 5,000 edges: one round, 2 x 16 -> 18 us).
+    const int32_t* keep_idx[2];
+    float* out[2];
+    int32_t n_whole, parts;
     const uint8_t* b_images;   // [n_chunks][n_blocks][n_slices][bn_max x 128 bytes]
     uint32_t* error;
 };
@@ -329,6 +335,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
     __shared__ uint64_t a_full, b_full[2], b_empty[2], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_slot;
     __shared__ int32_t a_row[128], a_rel[128];
+    // the CTA's tile (in shared memory: as registers they made the gather spill): its rows [m0, hi), its run of negative blocks, ...
+    __shared__ int64_t job_m0, job_hi;
+    __shared__ int32_t job_first, job_blocks, job_side;
+    __shared__ const uint8_t* job_images;
     __shared__ __align__(16) float out_stage[kTcEpilogueWarps][32 * 32];
     const NegArgs& a = ta.base;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -337,11 +347,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
     const size_t b_buf_bytes = (size_t)ta.n_slices * b_slice_bytes;
     uint8_t* b_smem = a_smem + (size_t)ta.n_slices * 16384;                          // 2 x n_slices x bn_max x 128 B
 
-    const int c = blockIdx.x / a.tiles_per_chunk, tile = blockIdx.x % a.tiles_per_chunk;
-    const int64_t lo = ((int64_t)c * a.E + a.n_chunks - 1) / a.n_chunks;
-    const int64_t hi = ((int64_t)(c + 1) * a.E + a.n_chunks - 1) / a.n_chunks;
-    const int64_t m0 = lo + (int64_t)tile * 128;
-    const int n_blocks = (a.negs + ta.bn_max - 1) / ta.bn_max;
     const int n_slots = ta.n_slices * 8;                  // 16-byte slots per operand row
     constexpr int kGatherThreads = kTcGatherWarps * 32, kGatherUnroll = 8;
 
@@ -358,9 +363,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x < 128) {
+        const int behind = (int)blockIdx.x - ta.n_whole;   // >= 0: a part of a tile
+        const int unit = behind < 0 ? (int)blockIdx.x : ta.n_whole + behind / ta.parts;
+        const int side_tiles = a.tiles_per_chunk * a.n_chunks;
+        const int side = unit / side_tiles, c = unit % side_tiles / a.tiles_per_chunk, tile = unit % a.tiles_per_chunk;
+        const int64_t lo = ((int64_t)c * a.E + a.n_chunks - 1) / a.n_chunks;
+        const int64_t hi = ((int64_t)(c + 1) * a.E + a.n_chunks - 1) / a.n_chunks;
+        const int64_t m0 = lo + (int64_t)tile * 128;
+        const int all_blocks = (a.negs + ta.bn_max - 1) / ta.bn_max;
+        const int first_block = behind < 0 ? 0 : behind % ta.parts * all_blocks / ta.parts;
+        const int n_blocks = (behind < 0 ? all_blocks : (behind % ta.parts + 1) * all_blocks / ta.parts) - first_block;
         const int64_t i = m0 + threadIdx.x;
-        a_row[threadIdx.x] = i < hi ? a.keep_idx[i] : -1;
+        a_row[threadIdx.x] = i < hi ? ta.keep_idx[side][i] : -1;
         a_rel[threadIdx.x] = i < hi ? a.rel[i] : 0;
+        if (threadIdx.x == 0) {
+            job_m0 = m0; job_hi = hi; job_first = first_block; job_blocks = n_blocks; job_side = side;
+            job_images = ta.b_images + ((size_t)c * all_blocks + first_block) * b_buf_bytes;
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -405,11 +424,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
         // 32-column slice of them
         bool ok = true;
         const int quarter = warp & 3, half = warp >> 2;
-        const int64_t row0 = m0 + quarter * 32;
-        const bool vec4 = a.negs % 4 == 0 && (reinterpret_cast<uintptr_t>(a.out) & 15) == 0;   // rows start 16-byte aligned
+        const int64_t row0 = job_m0 + quarter * 32, hi = job_hi;
+        const int first_block = job_first, n_blocks = job_blocks;
+        float* out = ta.out[job_side];
+        const bool vec4 = a.negs % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;   // rows start 16-byte aligned
         for (int j = 0; j < n_blocks && ok; ++j) {
             const int buf = j & 1;
-            const int n0 = j * ta.bn_max;
+            const int n0 = (first_block + j) * ta.bn_max;
             const int bn = min(ta.bn_max, (a.negs - n0 + 15) / 16 * 16);
             if (!mbar_wait(&acc_full[buf], (j >> 1) & 1)) { if (lane == 0) report(ta.error, 21u); ok = false; break; }
             tc_fence_after();
@@ -436,7 +457,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
                         for (int r4 = 0; r4 < 32; r4 += 4) {
                             const int rr = r4 + (lane >> 3);
                             if (rr < rows && n < a.negs)
-                                *reinterpret_cast<float4*>(a.out + (row0 + rr) * a.negs + n) =
+                                *reinterpret_cast<float4*>(out + (row0 + rr) * a.negs + n) =
                                     *reinterpret_cast<const float4*>(sb + rr * 128 + ((p ^ (rr & 7)) << 4));
                         }
                     } else {
@@ -447,7 +468,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
                         __syncwarp();
                         const int n = n0 + c0 + lane;
                         if (n < a.negs)
-                            for (int rr = 0; rr < rows; ++rr) a.out[(row0 + rr) * a.negs + n] = st[rr * 32 + (lane ^ rr)];
+                            for (int rr = 0; rr < rows; ++rr) out[(row0 + rr) * a.negs + n] = st[rr * 32 + (lane ^ rr)];
                     }
                     __syncwarp();
                 }
@@ -460,7 +481,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
         // ---------------- operand images of the negatives: one bulk copy per slice ----------------
         if (lane == 0) {
             bool ok = true;
-            const uint8_t* images = ta.b_images + (size_t)c * n_blocks * b_buf_bytes;
+            const uint8_t* images = job_images;
+            const int n_blocks = job_blocks;
             int issued = 0;
             for (int j = 0; j < n_blocks && ok; ++j) {
                 const int buf = j & 1;
@@ -479,11 +501,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
     } else if (warp == kTcMmaWarp) {
         // ---------------- MMA issue ----------------
         if (lane == 0) {
+            const int first_block = job_first, n_blocks = job_blocks;
             bool ok = mbar_wait(&a_full, 0);
             if (!ok) report(ta.error, 23u);
             for (int j = 0; j < n_blocks && ok; ++j) {
                 const int buf = j & 1;
-                const int n0 = j * ta.bn_max;
+                const int n0 = (first_block + j) * ta.bn_max;
                 const int bn = min(ta.bn_max, (a.negs - n0 + 15) / 16 * 16);
                 if (!mbar_wait(&b_full[buf], (j >> 1) & 1)) { report(ta.error, 24u); ok = false; break; }
                 if (j >= 2 && !mbar_wait(&acc_empty[buf], ((j >> 1) - 1) & 1)) { report(ta.error, 25u); ok = false; break; }
@@ -655,6 +678,7 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
         a.tiles_per_chunk = (int32_t)((max_chunk + 63) / 64);
         if (tensor) {
             NegTcArgs ta;
+            memset(&ta, 0, sizeof(ta));
             ta.n_slices = (dim + 31) / 32;
             ta.bn_max = std::min(kTcBlockN, (lp->negs + 15) / 16 * 16);
             int cols = 32;
@@ -685,15 +709,21 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
             const size_t smem = (size_t)ta.n_slices * 16384 + 2 * (size_t)ta.n_slices * ta.bn_max * 128 + 1024;
             static uint64_t smem_done = 0;
             MG_CUDA(ctx, mg_smem_limit(&smem_done, ctx->device, (const void*)k_distmult_neg_tc, kTcMaxSlices * (16384 + 2 * kTcBlockN * 128) + 1024));
-            const unsigned blocks = (unsigned)(a.tiles_per_chunk * lp->n_chunks);
-            if (corrupt & MG_CORRUPT_DST) {
-                a.keep_idx = lp->src_idx; a.out = neg_dst_out; ta.base = a;
-                k_distmult_neg_tc<<<blocks, kTcThreads, smem, st>>>(ta);
-                ctx->launches++;
+            int sides = 0;
+            for (int q = 0; q < 2; ++q) {
+                const bool dst = q == 0;
+                if (!(corrupt & (dst ? MG_CORRUPT_DST : MG_CORRUPT_SRC))) continue;
+                ta.keep_idx[sides] = dst ? lp->src_idx : lp->dst_idx;
+                ta.out[sides] = dst ? neg_dst_out : neg_src_out;
+                ++sides;
             }
-            if (corrupt & MG_CORRUPT_SRC) {
-                a.keep_idx = lp->dst_idx; a.out = neg_src_out; ta.base = a;
-                k_distmult_neg_tc<<<blocks, kTcThreads, smem, st>>>(ta);
+            const int64_t tiles = (int64_t)sides * a.tiles_per_chunk * lp->n_chunks;
+            const int64_t left = tiles % ctx->n_sms;
+            ta.parts = left ? (int)std::min<int64_t>({4, n_blocks, ctx->n_sms / left}) : 1;
+            ta.n_whole = (int32_t)(tiles - left);
+            a.keep_idx = nullptr; a.out = nullptr; ta.base = a;
+            if (sides) {
+                k_distmult_neg_tc<<<(unsigned)(tiles - left + left * ta.parts), kTcThreads, smem, st>>>(ta);
                 ctx->launches++;
             }
         } else {

@@ -48,3 +48,32 @@ def test_positive_scores_beside_the_operand_images(dim, edges):
     assert float(((pos.double() - (s * w * o).sum(1)).abs() / terms).max()) < 1e-5
     for got, want in ((nd, (s * w) @ n.T), (ns, (o * w) @ n.T)):
         assert float((got.double() - want).norm() / want.norm()) < 1e-3      # operands rounded to ten bits
+
+
+# tiles of both sides in one launch: none left over a round of 148, some that are cut into parts, too many to cut; parts of unequal
+# runs of negatives; one side alone
+@pytest.mark.parametrize("edges,chunks,negs,corrupt", [(9_472, 1, 40, mg.CORRUPT_BOTH), (20_000, 1, 600, mg.CORRUPT_BOTH), (18_000, 9, 130, mg.CORRUPT_BOTH),
+                                                       (3_001, 2, 1_000, mg.CORRUPT_SRC), (127, 1, 333, mg.CORRUPT_DST)])
+def test_negative_scores_by_the_number_of_tiles(edges, chunks, negs, corrupt):
+    nodes, dim = 30_000, 36
+    ctx = mg.Context(0)
+    g = inputs.erdos_renyi_graph(nodes, 2 * nodes, seed=1, device="cuda")
+    ctx.load_graph(g.row_offsets, g.nbrs)
+    ctx.load_features(torch.zeros((nodes, 4), device="cuda"))
+    rng = np.random.RandomState(4)
+    src, dst, rel = (torch.from_numpy(rng.randint(0, n, edges).astype(np.int32)) for n in (nodes, nodes, 50))
+    lp = ctx.lp_prepare(src, rel, dst, chunks, negs, seed=5)
+    v = lp.view()
+    h = inputs.normal_features(v["targets"].numel(), dim, seed=6, device="cuda")
+    r = inputs.normal_features(50, dim, seed=7, device="cuda")
+    _, nd, ns = ctx.distmult_score(lp, h, r, corrupt)
+    w = r[rel.cuda().long()].double()
+    chunk = torch.arange(edges, device="cuda") * chunks // edges
+    for got, keep in ((nd, v["src_idx"]), (ns, v["dst_idx"])):
+        assert (got is None) == (not corrupt & (mg.CORRUPT_DST if keep is v["src_idx"] else mg.CORRUPT_SRC))
+        for c in range(chunks if got is not None else 0):
+            mine = chunk == c
+            want = (h[keep.long()][mine].double() * w[mine]) @ h[v["neg_idx"][c].long()].double().T
+            # operands rounded to ten bits, sums of 36 products: below 1e-3 of the norm, no value off by 1 % of the rows' rms
+            err = got[mine].double() - want
+            assert float(err.norm() / want.norm()) < 1e-3 and float(err.abs().max() / want.square().mean().sqrt()) < 1e-2
