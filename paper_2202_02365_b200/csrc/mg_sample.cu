@@ -616,6 +616,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_insert(InsertArgs a) {
 constexpr int kDedupMaxSlots = 26624;    // 208 KiB of keys + rows per block
 constexpr int kDedupMaxBuckets = 64;
 constexpr int kDedupMaxTables = 16;      // largest tables that a mini-batch may need
+constexpr int64_t kDedupMinNodes = 1 << 20;   // room for nodes of all mini-batches up to which the global tables are the faster way
 constexpr int kBucketThreads = 512;
 constexpr int kDedupSlots512 = 6656, kDedupSlots256 = 3328;   // tables up to this size: blocks of 512 / 256 threads
 
@@ -1047,7 +1048,7 @@ struct PlaceArgs {
     int32_t* nodes;
     int32_t* node_batch;
     const int32_t* hvals;      // null: the entries have their rows
-    int32_t table_limit;       // nodes of a mini-batch that the id tables are meant for
+    int32_t node_limit;        // nodes that a mini-batch may have after this hop
     int32_t* ent_repr;
     int32_t B, k;
     int32_t* cum;
@@ -1121,7 +1122,7 @@ __global__ void __launch_bounds__(kThreads) k_place(PlaceArgs a) {
                     a.node_off[(a.hop + 1) * (a.B + 1) + b] = next_off[b];
                     const int32_t rows = a.cum[b * (a.k + 2) + a.hop + 1] + (int32_t)v;
                     a.cum[b * (a.k + 2) + a.hop + 2] = rows;
-                    if (a.hvals && rows > a.table_limit) atomicOr(&a.hdr->status, ST_CAP_TABLE);
+                    if (rows > a.node_limit) atomicOr(&a.hdr->status, ST_CAP_TABLE);
                 }
             }
             carry += total;
@@ -1689,19 +1690,24 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     while (min_nb <= kDedupMaxTables && dedup_slots_for((cap_batch + min_nb - 1) / min_nb) > kDedupMaxSlots) ++min_nb;
     const int64_t dedup_nb = min_nb <= kDedupMaxTables ? dedup_buckets(n_batches, cap_batch, min_nb, ctx->n_sms) : min_nb;
     const int32_t dedup_slots = (int32_t)std::min<int64_t>(dedup_slots_for((cap_batch + dedup_nb - 1) / dedup_nb), kDedupMaxSlots);
-    const bool smem_last = min_nb <= kDedupMaxTables && dedup_nb * n_batches < (1ll << 24) && cap_entries + cap_nodes < (1ll << 31) &&
-                           !getenv("MG_GLOBAL_TABLES");
+    const bool smem_fits = min_nb <= kDedupMaxTables && dedup_nb * n_batches < (1ll << 24) && cap_entries + cap_nodes < (1ll << 31);
+    // Small samples go through the global tables in any case: these stay in L2, and k_insert takes one launch where the shared tables
+    // take two (room for 14,000 nodes: the whole call 94 -> 84 us, 80,000: 192 -> 175 us, 8 x 83,000: 893 -> 883 us, 64 x 42,000:
+    // equal, 37 x 100,000: 867 us with the shared tables, 880 without).
+    const bool smem_last = smem_fits && (int64_t)n_batches * cap_batch > kDedupMinNodes && !getenv("MG_GLOBAL_TABLES");
     // With the last hop deduplicated in shared memory the global tables only ever hold the nodes that are sampled from
-    // (targets and the inner deltas): a caller who bounds those gets tables several times smaller.
-    int64_t table_nodes = cap_batch;
-    if (smem_last && caps && caps->max_inner_nodes_per_batch > 0) {
-        table_nodes = std::min<int64_t>(cap_batch, caps->max_inner_nodes_per_batch);
-        for (int b = 0; b < n_batches; ++b) table_nodes = std::max<int64_t>(table_nodes, target_offsets[b + 1] - target_offsets[b]);
+    // (targets and the inner deltas): a caller who bounds those gets tables several times smaller.  (The bound holds either way.)
+    int64_t inner_nodes = cap_batch;
+    if (smem_fits && caps && caps->max_inner_nodes_per_batch > 0) {
+        inner_nodes = std::min<int64_t>(cap_batch, caps->max_inner_nodes_per_batch);
+        for (int b = 0; b < n_batches; ++b) inner_nodes = std::max<int64_t>(inner_nodes, target_offsets[b + 1] - target_offsets[b]);
     }
+    const int64_t table_nodes = smem_last ? inner_nodes : cap_batch;
     // (1.625 slots per node; four where all tables together stay within 8 MB: a sparse table saves a small hop the long probes,
     // 34 -> 17 us for the two inner hops of one mini-batch)
-    int64_t want_slots = std::max<int64_t>(16, (table_nodes + table_nodes / 2 + table_nodes / 8 + 7) / 8 * 8);
-    const int32_t table_limit = (int32_t)std::min<int64_t>(want_slots, INT32_MAX);   // (a sparse table takes no more nodes than a dense one)
+    auto slots_for = [](int64_t nodes) { return std::max<int64_t>(16, (nodes + nodes / 2 + nodes / 8 + 7) / 8 * 8); };
+    const int32_t inner_limit = (int32_t)std::min<int64_t>(slots_for(inner_nodes), INT32_MAX);
+    int64_t want_slots = slots_for(table_nodes);
     if (4 * table_nodes * n_batches <= 2ll << 20) want_slots = std::max<int64_t>(16, (4 * table_nodes + 7) / 8 * 8);
     if (want_slots > (1ll << MG_SLOT_BITS)) return mg_fail(ctx, MG_ERR_CAPACITY, "max_nodes_per_batch above %d", (int)((1ll << MG_SLOT_BITS) * 8 / 13));
     const int32_t table_size = (int32_t)want_slots;
@@ -1852,7 +1858,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
         {
             ProfScope ps(ctx, PH_SAMPLE_PLACE, 1);
             PlaceArgs pa{d->hdr, h, d->newlist[0], id_bits, batch_cnt + (size_t)h * B, d->cap_nodes, d->nodes, d->node_batch,
-                         smem_hop ? nullptr : d->hvals, table_limit, d->ent_repr, B, k, d->cum, d->node_off, (int32_t)hdr_ints, d->ent_off,
+                         smem_hop ? nullptr : d->hvals, h < k - 1 ? inner_limit : (int32_t)cap_batch, d->ent_repr, B, k, d->cum, d->node_off, (int32_t)hdr_ints, d->ent_off,
                          d->rowbase, d->d_ent_hop, d->h_stage_dev + summary_at};
             const size_t sm = (size_t)B * sizeof(int32_t);   // 16 KiB at the largest number of mini-batches
             const unsigned grid = blocks_for(std::max<int64_t>(nodes_bound[h + 1], smem_hop ? 0 : entries_bound[h]), kThreads, 8);
@@ -1871,7 +1877,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     memset(&sig, 0, sizeof(sig));
     sig.B = B; sig.k = k; sig.T_bound = T_bound; sig.table_size = table_size; sig.cap_batch = cap_batch;
     sig.cap_nodes = d->cap_nodes; sig.cap_entries = d->cap_entries; sig.n_nodes = ctx->n_nodes; sig.part_size = ctx->part_size;
-    sig.inout = (inout ? 1 : 0) | (smem_last ? 2 + 4 * dedup_nb : 0);
+    sig.inout = (inout ? 1 : 0) | (smem_last ? 2 + 4 * dedup_nb : 0) | ((int64_t)inner_limit << 16);
     for (int h = 0; h < k; ++h) sig.fanouts[h] = fanouts[h];
     const void* ptrs[] = {d->hdr, d->nodes, d->node_batch, d->ent_off, d->tile_state, d->newlist[0], d->newlist[1],
                           d->ent_nbrs, d->ent_repr, d->hkeys, d->hvals, d->node_off, d->cum, d->rowbase, d->batch_cnt,

@@ -69,10 +69,10 @@ def test_hops_on_either_side_of_the_tile_sizes(graph, ctx, total):
     one.free()
 
 
-# buckets of the last hop: one (a table of a few hundred nodes), several with tables for blocks of 256, 512 and 1,024 threads, as
-# many tables as a mini-batch may need, and more (through the global tables); ids that are multiples of a Fibonacci
+# the last hop: through the global tables (little room in all); buckets in shared memory, one (a table of a few hundred nodes), several
+# with tables for blocks of 256, 512 and 1,024 threads, as many tables as a mini-batch may need, and more (global tables again); ids that are multiples of a Fibonacci
 # number, whose multiplicative hashes lie next to each other
-@pytest.mark.parametrize("room,n_batches", [(300, 1), (12_000, 1), (N, 1), (N, 60), (4_000, 160), (370_000, 2), (420_000, 2)])
+@pytest.mark.parametrize("room,n_batches", [(300, 1), (N, 1), (300, 3_600), (4_000, 300), (12_000, 120), (N, 9), (370_000, 4), (420_000, 4)])
 def test_last_hop_buckets(graph, ctx, room, n_batches):
     off, nbrs = graph.row_offsets.numpy(), graph.nbrs.numpy()
     per = max(1, min(room // 45, 2_000))
