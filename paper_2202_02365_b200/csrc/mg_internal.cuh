@@ -30,7 +30,6 @@ struct DenseHeader {
     uint32_t status;
     uint32_t epoch;                       // number of the sample into this handle: tags the states of k_hop's tiles
     uint64_t targets;                     // device address the targets are read from
-    uint32_t n_new[MG_MAX_HOPS];          // length of each hop's list of new nodes
     uint32_t ticket[MG_MAX_HOPS];         // k_hop: the next tile of the hop
     int32_t hop_base[MG_MAX_HOPS + 2];    // node arena: hop h occupies [hop_base[h], hop_base[h+1])
     int32_t ent_base[MG_MAX_HOPS + 1];    // entry arena: hop h occupies [ent_base[h], ent_base[h+1])
@@ -202,7 +201,8 @@ struct mg_dense {
     int32_t* rowbase = nullptr;     // [(k+1) * (B+1)] first packed row of batch b in H^l
     int32_t* hkeys = nullptr;       // [B * table_size]
     int32_t* hvals = nullptr;       // [B * table_size]
-    uint64_t* newlist[2] = {nullptr, nullptr};  // [cap_nodes] composite keys
+    int32_t* new_ids = nullptr;     // [cap_entries] a hop's new ids by rank, a mini-batch's from the place of its first entry on
+    uint64_t* newlist[2] = {nullptr, nullptr};  // [cap_nodes] sort keys of an export
     uint64_t* d_seeds = nullptr;    // [B]
     int32_t* scan_tmp = nullptr;    // block sums
     uint32_t* sort_hist = nullptr;  // radix histograms

@@ -468,11 +468,12 @@ __global__ void __launch_bounds__(kThreads) k_hop(HopArgs a) {
     }
 }
 
-// Deduplication: every entry's neighbour id goes into its batch's id table.  One thread owns four entries; their
+// Deduplication: every entry's neighbour id goes into its batch's id table.  One thread owns PER entries; their
 // compare-and-swaps go out back to back and the probes of those that met another id go on in rounds, all open entries of the
-// thread at a time.  Bound by the rounds a warp needs for its longest probe, one L2 round trip each (a bucket load before the
-// compare-and-swap made it slower: 134 -> 160 us for the inner hops of 128 mini-batches), so small tables are kept sparse
-// (mg_sample_many).  The keys of the ids that were new are appended to the list with one global atomic per 1024 entries.
+// thread at a time.  Bound by the rounds a block needs for its longest probe, one L2 round trip each (reads of four or eight
+// slots in place of the next compare-and-swap made it slower: 134 -> 160 us for the inner hops of 128 mini-batches, 292 -> 339 us
+// for 12.6M entries of 16 large ones), so small tables are kept sparse (mg_sample_many), and by the counter of the mini-batch
+// that all blocks in flight add to.
 struct InsertArgs {
     DenseHeader* hdr;
     int hop;
@@ -480,55 +481,66 @@ struct InsertArgs {
     int32_t* ent_repr;   // in: batch id; out: the node's row (new node) or -1 - (batch * table_size + slot)
     int32_t* hkeys;
     TableGeom tg;
-    uint64_t* newlist;
-    int64_t cap_new;
-    int id_bits;
-    int32_t k;
+    int32_t* new_ids;            // [cap_entries] a mini-batch's new ids, from its first entry's place on
+    int32_t B, k;
+    const int32_t* node_off;     // [hop + 1][B + 1] valid
+    const int32_t* ent_off;
     const int32_t* cum;          // [B][k+2]
     int32_t* hvals;
     uint32_t* batch_cnt;         // [B] new nodes of the hop per mini-batch, zero before the launch
     int32_t max_nodes_per_batch;
 };
 
+constexpr int kInsertThreads = 128, kInsertBlocks = 12;   // per SM
 constexpr int kInsertPerThread = 4;
 constexpr int kInsertSpan = 16;   // mini-batches a block's chunk of entries may touch on the fast path
 
 // New nodes are not sorted on the device: nothing the path computes depends on the order of ids inside a delta (the
 // paper's arrays, with ascending ids, are an export: mg_dense_batch_perm).  A new node takes the next free row of its
-// mini-batch right here -- a count per mini-batch in shared memory, one global atomic per (block, mini-batch) --,
-// its table value is written at once, and its list entry carries (mini-batch, id, rank in the hop).
-__global__ void __launch_bounds__(kThreads, 6) k_insert(InsertArgs a) {
-    __shared__ uint32_t warp_tot[kThreads / 32];
-    __shared__ uint32_t block_base;
+// mini-batch right here -- one global atomic per (block, mini-batch) --, its table value is written at once, and its id goes to
+// its rank in the mini-batch's run of new_ids (a mini-batch has no more new nodes than entries, so the run starts where its
+// entries do and no second counter is needed: with one list of (mini-batch, id, rank) for all, which wants a counter for its
+// length, 16 mini-batches of 790,000 entries took 284 us instead of 254, and 128 of 29,000 119 instead of 95).
+template <int PER>
+__global__ void __launch_bounds__(kInsertThreads, kInsertBlocks) k_insert(InsertArgs a) {
+    constexpr int kWarps = kInsertThreads / 32, kChunk = kInsertThreads * PER;
+    __shared__ uint32_t warp_tot[kWarps];
     __shared__ uint32_t span_cnt[kInsertSpan], span_base[kInsertSpan];
     __shared__ int32_t span_row[kInsertSpan];   // first row of the hop's new nodes in the mini-batch
-    __shared__ int32_t first_batch;
+    __shared__ int32_t span_list[kInsertSpan];  // its run of new_ids
+    __shared__ int32_t first_batch, last_batch;
     const int32_t lo = a.hdr->ent_base[a.hop], hi = a.hdr->ent_base[a.hop + 1];
     if (__syncthreads_or(a.hdr->status != 0)) return;   // (the whole block: another one may be setting it)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kChunk = kThreads * kInsertPerThread;
+    auto row_of = [&](int32_t batch) { return a.cum[batch * (a.k + 2) + a.hop + 1]; };
+    auto list_of = [&](int32_t batch) { return a.ent_off[a.node_off[a.hop * (a.B + 1) + batch]]; };
     for (int32_t base = lo + blockIdx.x * kChunk; base < hi; base += gridDim.x * kChunk) {
-        int32_t u[kInsertPerThread], b[kInsertPerThread], old[kInsertPerThread];
-        uint32_t slot[kInsertPerThread];
+        int32_t u[PER], b[PER], old[PER];
+        uint32_t slot[PER], rank[PER];
         uint32_t open = 0, new_bits = 0;
 #pragma unroll
-        for (int j = 0; j < kInsertPerThread; ++j) {
-            const int32_t e = base + j * kThreads + threadIdx.x;
+        for (int j = 0; j < PER; ++j) {
+            const int32_t e = base + j * kInsertThreads + threadIdx.x;
             u[j] = -1; b[j] = 0; old[j] = -1; slot[j] = 0;
             if (e < hi) { u[j] = a.ent_nbrs[e]; b[j] = a.ent_repr[e]; }
         }
         if (threadIdx.x == 0) first_batch = b[0];   // thread 0's first item is the chunk's first entry
+        if (threadIdx.x == 32) last_batch = a.ent_repr[min(hi - base, kChunk) - 1 + base];
         if (threadIdx.x < kInsertSpan) span_cnt[threadIdx.x] = 0;
         __syncthreads();
         const int32_t b0 = first_batch;   // entries are ordered by mini-batch, so a chunk touches a short run of them
+        const bool one_batch = b0 == last_batch;
+        const int span = (int)threadIdx.x - 32;   // threads 32..47: a mini-batch of the run each
+        int32_t my_row = 0, my_list = 0;
+        if (span >= 0 && span < (one_batch ? 1 : kInsertSpan) && b0 + span < a.B) { my_row = row_of(b0 + span); my_list = list_of(b0 + span); }
 #pragma unroll
-        for (int j = 0; j < kInsertPerThread; ++j)
+        for (int j = 0; j < PER; ++j)
             if (u[j] >= 0) {
                 slot[j] = table_hash(u[j], a.tg.size);
                 old[j] = atomicCAS(&a.hkeys[(int64_t)b[j] * a.tg.size + slot[j]], -1, u[j]);
             }
 #pragma unroll
-        for (int j = 0; j < kInsertPerThread; ++j) {
+        for (int j = 0; j < PER; ++j) {
             if (u[j] < 0) continue;
             if (old[j] == -1) new_bits |= 1u << j;
             else if (old[j] != u[j]) open |= 1u << j;
@@ -536,63 +548,63 @@ __global__ void __launch_bounds__(kThreads, 6) k_insert(InsertArgs a) {
         for (int32_t probe = 1; open; ++probe) {   // linear probing
             if (probe >= a.tg.size) { atomicOr(&a.hdr->status, ST_CAP_TABLE); break; }
 #pragma unroll
-            for (int j = 0; j < kInsertPerThread; ++j)
+            for (int j = 0; j < PER; ++j)
                 if (open >> j & 1) {
                     slot[j] = slot[j] + 1u == (uint32_t)a.tg.size ? 0u : slot[j] + 1u;
                     old[j] = atomicCAS(&a.hkeys[(int64_t)b[j] * a.tg.size + slot[j]], -1, u[j]);
                 }
 #pragma unroll
-            for (int j = 0; j < kInsertPerThread; ++j)
+            for (int j = 0; j < PER; ++j)
                 if (open >> j & 1) {
                     if (old[j] == -1) new_bits |= 1u << j;
                     if (old[j] == -1 || old[j] == u[j]) open &= ~(1u << j);
                 }
         }
-        const uint32_t n_mine = __popc(new_bits);
-        uint32_t rank[kInsertPerThread];
+        __syncwarp();
+        uint32_t in_warp = 0;
 #pragma unroll
-        for (int j = 0; j < kInsertPerThread; ++j) {
-            rank[j] = 0;
+        for (int j = 0; j < PER; ++j) {
+            const bool fresh = new_bits >> j & 1;
             // an entry that found its node already in the table gets the node's row later (k_place): it leaves
             // -1 - (table index) behind; the entry of a new node gets its row below
-            if (new_bits >> j & 1) {
+            if (!fresh && u[j] >= 0) a.ent_repr[base + j * kInsertThreads + threadIdx.x] = -1 - (b[j] * a.tg.size + (int32_t)slot[j]);
+            rank[j] = 0;
+            if (one_batch) {
+                const uint32_t ballot = __ballot_sync(0xFFFFFFFFu, fresh);
+                rank[j] = in_warp + __popc(ballot & ((1u << lane) - 1u));
+                in_warp += __popc(ballot);
+            } else if (fresh) {
                 const int32_t bb = b[j] - b0;
                 rank[j] = bb < kInsertSpan ? atomicAdd(&span_cnt[bb], 1u) : atomicAdd(&a.batch_cnt[b[j]], 1u);
-            } else if (u[j] >= 0) a.ent_repr[base + j * kThreads + threadIdx.x] = -1 - (b[j] * a.tg.size + (int32_t)slot[j]);
-        }
-        const uint32_t inc = warp_incl_scan(n_mine);
-        if (lane == 31) warp_tot[warp] = inc;
-        __syncthreads();
-        // the block's run of the list (one thread) and of its mini-batches' rows (another warp's threads): one round trip
-        if (threadIdx.x == 0) {
-            uint32_t run = 0;
-            for (int w = 0; w < kThreads / 32; ++w) run += warp_tot[w];
-            block_base = run ? atomicAdd(&a.hdr->n_new[a.hop], run) : 0u;
-        } else if (threadIdx.x >= 32 && threadIdx.x < 32 + kInsertSpan) {
-            const int i = (int)threadIdx.x - 32;
-            const uint32_t c = span_cnt[i];
-            if (c) {
-                span_row[i] = a.cum[(b0 + i) * (a.k + 2) + a.hop + 1];
-                span_base[i] = atomicAdd(&a.batch_cnt[b0 + i], c);
             }
         }
+        if (lane == 0) warp_tot[warp] = in_warp;
+        if (span >= 0 && span < kInsertSpan) { span_row[span] = my_row; span_list[span] = my_list; }
         __syncthreads();
-        int64_t pos = (int64_t)block_base + inc - n_mine;
-        for (int w = 0; w < warp; ++w) pos += warp_tot[w];
+        if (threadIdx.x < kInsertSpan) {   // the block's run of its mini-batches' rows: one round trip
+            uint32_t c = span_cnt[threadIdx.x];
+            if (one_batch) {
+                c = 0;
+                if (threadIdx.x == 0)
+                    for (int w = 0; w < kWarps; ++w) c += warp_tot[w];
+            }
+            if (c) span_base[threadIdx.x] = atomicAdd(&a.batch_cnt[b0 + (int)threadIdx.x], c);
+        }
+        __syncthreads();
+        uint32_t before = 0;
+        if (one_batch)
+            for (int w = 0; w < warp; ++w) before += warp_tot[w];
 #pragma unroll
-        for (int j = 0; j < kInsertPerThread; ++j)
+        for (int j = 0; j < PER; ++j)
             if (new_bits >> j & 1) {
                 const int32_t bb = b[j] - b0;
-                if (bb < kInsertSpan) rank[j] += span_base[bb];
-                const int64_t row = (int64_t)(bb < kInsertSpan ? span_row[bb] : a.cum[b[j] * (a.k + 2) + a.hop + 1]) + rank[j];
+                const bool near = bb < kInsertSpan;
+                rank[j] += near ? before + span_base[bb] : 0u;
+                const int64_t row = (int64_t)(near ? span_row[bb] : row_of(b[j])) + rank[j];
                 if (row < a.max_nodes_per_batch) a.hvals[(int64_t)b[j] * a.tg.size + slot[j]] = (int32_t)row;
                 else atomicOr(&a.hdr->status, ST_CAP_TABLE);
-                a.ent_repr[base + j * kThreads + threadIdx.x] = (int32_t)row;   // final: no table read for this entry
-                const uint64_t key = (uint64_t)rank[j] | ((uint64_t)(uint32_t)u[j] << MG_SLOT_BITS) |
-                                     ((uint64_t)(uint32_t)b[j] << (MG_SLOT_BITS + a.id_bits));
-                if (pos < a.cap_new) a.newlist[pos] = key;
-                else atomicOr(&a.hdr->status, ST_CAP_NODES);
-                ++pos;
+                a.ent_repr[base + j * kInsertThreads + threadIdx.x] = (int32_t)row;   // final: no table read for this entry
+                a.new_ids[(int64_t)(near ? span_list[bb] : list_of(b[j])) + rank[j]] = u[j];
             }
         __syncthreads();
     }
@@ -634,9 +646,7 @@ struct DedupArgs {
     int32_t* share_off;         // [2][B][nb][nb + 1] group bounds (positions in pairs): entries, then earlier nodes
     const int32_t* cum;         // [B][k + 2]
     uint32_t* batch_cnt;        // [B] new nodes of the hop per mini-batch, zero before the launch
-    uint64_t* newlist;
-    int64_t cap_new;
-    int id_bits;
+    int32_t* new_ids;           // [cap_entries] a mini-batch's new ids, from its first entry's place on
     int32_t max_nodes_per_batch;
     int64_t node_pairs0;
 };
@@ -756,7 +766,7 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_entries(DedupArgs a) 
 template <int kDedupThreads>
 __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
     extern __shared__ int32_t dedup_sm[];
-    __shared__ uint32_t row_base, list_base, warp_tot[kDedupThreads / 32];
+    __shared__ uint32_t row_base, warp_tot[kDedupThreads / 32];
     __shared__ int32_t run_lo[2][kDedupMaxBuckets], run_start[2][kDedupMaxBuckets + 1];
     if (__syncthreads_or(a.hdr->status != 0)) return;   // (the whole block: another one may be setting it)
     const uint32_t S = (uint32_t)a.S, nb = (uint32_t)a.nb;
@@ -851,7 +861,7 @@ __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
         }
     }
     __syncthreads();
-    // rank the new nodes of this block's table, take a run of the mini-batch's rows and of the list of new nodes
+    // rank the new nodes of this block's table, take a run of the mini-batch's rows
     uint32_t mine = 0;
     for (uint32_t i = threadIdx.x; i < S; i += kDedupThreads) mine += (keys[i] != -1 && vals[i] < 0) ? 1u : 0u;
     const uint32_t inc = warp_incl_scan(mine);
@@ -861,13 +871,11 @@ __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
         const uint32_t w = lane < kDedupThreads / 32 ? warp_tot[lane] : 0u;
         const uint32_t wi = warp_incl_scan(w);
         if (lane < kDedupThreads / 32) warp_tot[lane] = wi - w;
-        if (lane == 31) {
-            row_base = wi ? atomicAdd(&a.batch_cnt[b], wi) : 0u;
-            list_base = wi ? atomicAdd(&a.hdr->n_new[a.hop], wi) : 0u;
-        }
+        if (lane == 31) row_base = wi ? atomicAdd(&a.batch_cnt[b], wi) : 0u;
     }
     __syncthreads();
     const int32_t first_row = a.cum[b * (a.k + 2) + a.hop + 1];
+    int32_t* list = a.new_ids + a.ent_off[a.node_off[a.hop * (a.B + 1) + b]];
     uint32_t rk = warp_tot[warp] + inc - mine;
     for (uint32_t i = threadIdx.x; i < S; i += kDedupThreads) {
         if (keys[i] == -1 || vals[i] >= 0) continue;
@@ -875,11 +883,7 @@ __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
         const int64_t row = (int64_t)first_row + rank;
         if (row >= a.max_nodes_per_batch) atomicOr(&a.hdr->status, ST_CAP_TABLE);
         vals[i] = (int32_t)row;
-        const int64_t pos = (int64_t)list_base + rk;
-        if (pos < a.cap_new)
-            a.newlist[pos] = (uint64_t)rank | ((uint64_t)(uint32_t)keys[i] << MG_SLOT_BITS) |
-                             ((uint64_t)(uint32_t)b << (MG_SLOT_BITS + a.id_bits));
-        else atomicOr(&a.hdr->status, ST_CAP_NODES);
+        list[rank] = keys[i];
         ++rk;
     }
     __syncthreads();
@@ -1031,8 +1035,8 @@ constexpr size_t kScatterSmem = (size_t)kSortTile * 8 + (size_t)(kThreads / 32) 
 // place the new nodes as the next hop, give the entries their rows
 // -------------------------------------------------------------------------------------
 // The hop's new nodes per mini-batch, summed up, are the next hop's node offsets (every block takes the sums for itself, block 0
-// writes them down: a kernel of one block for it cost 2 us and a gap per hop).  Then: list entry (mini-batch, id, rank) -> the
-// node's place in its mini-batch's run; an entry that met a known node -> that node's row (entries of new nodes got theirs at
+// writes them down: a kernel of one block for it cost 2 us and a gap per hop).  Then: the mini-batches' runs of new ids are put
+// one behind the other (a warp takes 128 nodes at a time, four loads in flight per thread); an entry that met a known node -> that node's row (entries of new nodes got theirs at
 // insert time; the shared-memory path of the last hop leaves none).
 // FINAL (last hop): block 0 also writes the packed row bases of every layer and the per-batch entry bounds of every hop, and
 // the sample's summary (header, per-batch tables) for the host, stored straight into mapped pinned memory.  A copy engine
@@ -1041,8 +1045,7 @@ constexpr size_t kScatterSmem = (size_t)kSortTile * 8 + (size_t)(kThreads / 32) 
 struct PlaceArgs {
     DenseHeader* hdr;
     int hop;
-    const uint64_t* list;
-    int id_bits;
+    const int32_t* new_ids;      // the hop's new ids by rank, mini-batch b's from the place of its first entry on
     const uint32_t* batch_cnt;   // [B] new nodes of the hop
     int64_t cap_nodes;
     int32_t* nodes;
@@ -1096,21 +1099,25 @@ __device__ __forceinline__ void finish_sample(const PlaceArgs& a, bool bad) {
     for (int32_t i = threadIdx.x; i < n_off; i += blockDim.x) o_off[i] = a.node_off[i];
 }
 
+constexpr int kPlacePerThread = 4;
+
 template <bool FINAL>
-__global__ void __launch_bounds__(kThreads) k_place(PlaceArgs a) {
-    extern __shared__ int32_t next_off[];   // [B] first node of the mini-batch in the next hop
+__global__ void __launch_bounds__(kThreads, 8) k_place(PlaceArgs a) {
+    extern __shared__ int32_t next_off[];   // [B] first node of the mini-batch in the next hop ...
+    int32_t* list_at = next_off + a.B;      // ... and its run of new_ids
     __shared__ uint32_t part[kThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int32_t n = (int32_t)a.hdr->n_new[a.hop], start = a.hdr->hop_base[a.hop + 1];
+    const int32_t start = a.hdr->hop_base[a.hop + 1];
     const int32_t lo = a.hdr->ent_base[a.hop], hi = a.hdr->ent_base[a.hop + 1];
     // (the whole block alike: block 0 may be adding to the status)
     bool bad = __syncthreads_or(a.hdr->status != 0);
-    const bool full = !bad && (int64_t)start + n > a.cap_nodes;
-    if (!bad && !full) {
+    int64_t end = start;
+    if (!bad) {
         uint32_t carry = (uint32_t)start;
         for (int s0 = 0; s0 < a.B; s0 += kThreads) {
             const int b = s0 + (int)threadIdx.x;
             const uint32_t v = b < a.B ? a.batch_cnt[b] : 0u;
+            const int32_t run = b < a.B ? a.ent_off[a.node_off[a.hop * (a.B + 1) + b]] : 0;
             const uint32_t inc = warp_incl_scan(v);
             if (lane == 31) part[warp] = inc;
             __syncthreads();
@@ -1118,6 +1125,7 @@ __global__ void __launch_bounds__(kThreads) k_place(PlaceArgs a) {
             for (int w = 0; w < kThreads / 32; ++w) { if (w < warp) before += part[w]; total += part[w]; }
             if (b < a.B) {
                 next_off[b] = (int32_t)(before + inc - v);
+                list_at[b] = run;
                 if (blockIdx.x == 0) {
                     a.node_off[(a.hop + 1) * (a.B + 1) + b] = next_off[b];
                     const int32_t rows = a.cum[b * (a.k + 2) + a.hop + 1] + (int32_t)v;
@@ -1128,27 +1136,48 @@ __global__ void __launch_bounds__(kThreads) k_place(PlaceArgs a) {
             carry += total;
             __syncthreads();
         }
+        end = carry;
+        if (end > a.cap_nodes) bad = true;   // (nothing is written outside the arenas; the kernels that follow see the status)
         if (blockIdx.x == 0 && threadIdx.x == 0) {
-            a.hdr->hop_base[a.hop + 2] = start + n;
-            a.node_off[(a.hop + 1) * (a.B + 1) + a.B] = start + n;
+            if (bad) atomicOr(&a.hdr->status, ST_CAP_NODES);
+            else {
+                a.hdr->hop_base[a.hop + 2] = (int32_t)end;
+                a.node_off[(a.hop + 1) * (a.B + 1) + a.B] = (int32_t)end;
+            }
         }
-    } else if (full && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&a.hdr->status, ST_CAP_NODES);
-    bad |= full;
+    }
     if (FINAL && blockIdx.x == 0) { __syncthreads(); finish_sample(a, bad); return; }
     if (bad) return;
     const int32_t step = (int32_t)(gridDim.x - FINAL) * kThreads, tid = (int32_t)(blockIdx.x - FINAL) * kThreads + (int32_t)threadIdx.x;
-    const uint64_t id_mask = (1ull << a.id_bits) - 1ull;
-    for (int32_t j = tid; j < n; j += step) {
-        const uint64_t key = a.list[j];
-        const int32_t b = (int32_t)(key >> (MG_SLOT_BITS + a.id_bits));
-        const int32_t at = next_off[b] + (int32_t)(key & ((1u << MG_SLOT_BITS) - 1u));
-        a.nodes[at] = (int32_t)((key >> MG_SLOT_BITS) & id_mask);
-        a.node_batch[at] = b;
+    for (int64_t at0 = start + (int64_t)(tid >> 5) * (32 * kPlacePerThread); at0 < end; at0 += (int64_t)step * kPlacePerThread) {
+        int32_t b = 0;   // the mini-batch of the warp's first node
+        for (int32_t above = a.B; above - b > 1;) {
+            const int32_t mid = (b + above) >> 1;
+            if (next_off[mid] <= at0) b = mid; else above = mid;
+        }
+        int32_t id[kPlacePerThread], batch[kPlacePerThread];
+#pragma unroll
+        for (int j = 0; j < kPlacePerThread; ++j) {
+            const int64_t at = at0 + j * 32 + lane;
+            if (at < end) {
+                while (b + 1 < a.B && next_off[b + 1] <= at) ++b;
+                id[j] = a.new_ids[list_at[b] + (int32_t)(at - next_off[b])];
+                batch[j] = b;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kPlacePerThread; ++j) {
+            const int64_t at = at0 + j * 32 + lane;
+            if (at < end) { a.nodes[at] = id[j]; a.node_batch[at] = batch[j]; }
+        }
     }
     if (!a.hvals) return;
-    for (int32_t e = lo + tid; e < hi; e += step) {
-        const int32_t v = a.ent_repr[e];
-        if (v < 0) a.ent_repr[e] = a.hvals[-1 - v];
+    for (int64_t e0 = lo + tid; e0 < hi; e0 += (int64_t)step * kPlacePerThread) {
+        int32_t v[kPlacePerThread];
+#pragma unroll
+        for (int j = 0; j < kPlacePerThread; ++j) { const int64_t e = e0 + (int64_t)j * step; v[j] = e < hi ? a.ent_repr[e] : 0; }
+#pragma unroll
+        for (int j = 0; j < kPlacePerThread; ++j) if (v[j] < 0) a.ent_repr[e0 + (int64_t)j * step] = a.hvals[-1 - v[j]];
     }
 }
 
@@ -1507,6 +1536,7 @@ static int dense_alloc(mg_ctx* ctx, mg_dense* d, int32_t B, int32_t k, int64_t c
         d->cap_entries = 0;
         if ((rc = dev_realloc(ctx, &d->ent_nbrs, (size_t)cap_entries))) return rc;
         if ((rc = dev_realloc(ctx, &d->ent_repr, (size_t)cap_entries))) return rc;
+        if ((rc = dev_realloc(ctx, &d->new_ids, (size_t)cap_entries))) return rc;
         d->cap_entries = cap_entries;
         d->cap_pairs = 0;
     }
@@ -1837,8 +1867,8 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
             ProfScope ps(ctx, PH_SAMPLE_RELABEL, 1);
             if (smem_hop) {
                 DedupArgs da{d->hdr, h, B, k, (int32_t)dedup_nb, dedup_slots, d->nodes, d->node_off, d->ent_off, d->ent_nbrs,
-                             d->ent_repr, d->pairs, d->share_off, d->cum, batch_cnt + (size_t)h * B, d->newlist[0], d->cap_nodes,
-                             id_bits, (int32_t)cap_batch, d->cap_entries};
+                             d->ent_repr, d->pairs, d->share_off, d->cum, batch_cnt + (size_t)h * B, d->new_ids,
+                             (int32_t)cap_batch, d->cap_entries};
                 k_bucket_entries<<<(unsigned)(B * dedup_nb), kBucketThreads, 0, st>>>(da);
                 // (threads so that the blocks that shared memory lets onto an SM come to 2,048 threads)
                 const unsigned grid = (unsigned)(B * dedup_nb);
@@ -1848,19 +1878,24 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
                 else k_dedupe_last<256><<<grid, 256, sm, st>>>(da);
                 ctx->launches += 2;
             } else {
-                InsertArgs ia{d->hdr, h, d->ent_nbrs, d->ent_repr, d->hkeys, tg, d->newlist[0], d->cap_nodes, id_bits,
-                              k, d->cum, d->hvals, batch_cnt + (size_t)h * B, (int32_t)cap_batch};
-                // many short blocks: measured on the bench's last hop, 0.94 ms at 32 blocks per SM against 1.08 ms at 8
-                k_insert<<<blocks_for(entries_bound[h], kThreads * kInsertPerThread, 32), kThreads, 0, st>>>(ia);
+                InsertArgs ia{d->hdr, h, d->ent_nbrs, d->ent_repr, d->hkeys, tg, d->new_ids, B, k, d->node_off, d->ent_off,
+                              d->cum, d->hvals, batch_cnt + (size_t)h * B, (int32_t)cap_batch};
+                // many short blocks (64 threads: 340 us for the 254 of the large mini-batches, the counters are the limit then; 256: 255);
+                // an entry per thread where the SMs hold all of the hop's at once that way (the three hops of one mini-batch 23 -> 15 us,
+                // of a tiny graph 9.6 -> 7.4; with 12M entries it takes twice the time of four per thread)
+                if (entries_bound[h] <= (int64_t)mg_grid(ctx, kInsertBlocks) * kInsertThreads)
+                    k_insert<1><<<blocks_for(entries_bound[h], kInsertThreads, kInsertBlocks), kInsertThreads, 0, st>>>(ia);
+                else
+                    k_insert<kInsertPerThread><<<blocks_for(entries_bound[h], kInsertThreads * kInsertPerThread, 64), kInsertThreads, 0, st>>>(ia);
                 ctx->launches++;
             }
         }
         {
             ProfScope ps(ctx, PH_SAMPLE_PLACE, 1);
-            PlaceArgs pa{d->hdr, h, d->newlist[0], id_bits, batch_cnt + (size_t)h * B, d->cap_nodes, d->nodes, d->node_batch,
+            PlaceArgs pa{d->hdr, h, d->new_ids, batch_cnt + (size_t)h * B, d->cap_nodes, d->nodes, d->node_batch,
                          smem_hop ? nullptr : d->hvals, h < k - 1 ? inner_limit : (int32_t)cap_batch, d->ent_repr, B, k, d->cum, d->node_off, (int32_t)hdr_ints, d->ent_off,
                          d->rowbase, d->d_ent_hop, d->h_stage_dev + summary_at};
-            const size_t sm = (size_t)B * sizeof(int32_t);   // 16 KiB at the largest number of mini-batches
+            const size_t sm = 2 * (size_t)B * sizeof(int32_t);   // 32 KiB at the largest number of mini-batches
             const unsigned grid = blocks_for(std::max<int64_t>(nodes_bound[h + 1], smem_hop ? 0 : entries_bound[h]), kThreads, 8);
             if (h == k - 1) k_place<true><<<grid + 1, kThreads, sm, st>>>(pa);
             else k_place<false><<<grid, kThreads, sm, st>>>(pa);
@@ -1883,7 +1918,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
                           d->ent_nbrs, d->ent_repr, d->hkeys, d->hvals, d->node_off, d->cum, d->rowbase, d->batch_cnt,
                           d->d_ent_hop, d->d_seeds, d->h_stage_dev, d->h_stage_dev + summary_at, ctx->view_off, ctx->view_nbrs, ctx->d_slot_of_part, st,
                           ctx->d_part_of_node, inout ? (const void*)ctx->view_off_out : nullptr, inout ? (const void*)ctx->view_nbrs_out : nullptr,
-                          d->pairs, d->share_off};
+                          d->pairs, d->share_off, d->new_ids};
     static_assert(sizeof(ptrs) <= sizeof(sig.ptrs), "signature too small");
     memcpy(sig.ptrs, ptrs, sizeof(ptrs));
     const bool use_graph = ctx->sample_graphs && !ctx->prof_on && !getenv("MG_NO_SAMPLE_GRAPH");
@@ -2162,7 +2197,7 @@ extern "C" int mg_dense_free(mg_dense* d) {
     if (d->ctx && d->ctx->last_fwd_dense == d) d->ctx->last_fwd_dense = nullptr;
     cudaFree(d->hdr); cudaFree(d->nodes); cudaFree(d->node_batch); cudaFree(d->ent_off); cudaFree(d->tile_state); cudaFree(d->pairs); cudaFree(d->share_off);
     cudaFree(d->ent_nbrs); cudaFree(d->ent_repr); cudaFree(d->node_off); cudaFree(d->cum);
-    cudaFree(d->rowbase); cudaFree(d->hkeys); cudaFree(d->hvals); cudaFree(d->newlist[0]);
+    cudaFree(d->rowbase); cudaFree(d->hkeys); cudaFree(d->hvals); cudaFree(d->newlist[0]); cudaFree(d->new_ids);
     cudaFree(d->newlist[1]); cudaFree(d->d_seeds); cudaFree(d->batch_cnt); cudaFree(d->scan_tmp); cudaFree(d->sort_hist); cudaFree(d->seg_tiles);
     cudaFree(d->exp_buf); cudaFree(d->perm_buf); cudaFree(d->d_ent_hop); cudaFree(d->expm_buf);
     if (d->ev_exported) cudaEventDestroy(d->ev_exported);

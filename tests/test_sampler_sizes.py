@@ -98,3 +98,21 @@ def test_last_hop_buckets(graph, ctx, room, n_batches):
         first = np.unique(got)                           # every node is a target or somebody's neighbour
         assert np.array_equal(np.unique(np.concatenate([first, rows[b].numpy()])), np.sort(ids_b))
     d.free()
+
+
+# entries go into the id tables 128 at a time, an entry per thread, or (hops with room for more than the SMs hold at once that way) 512 at
+# a time: either form with blocks that touch a few mini-batches, and more mini-batches than a block keeps counts for
+@pytest.mark.parametrize("per,fanout", [(1, 14), (4, 13), (4, 14)])
+def test_id_table_blocks_over_many_mini_batches(graph, ctx, per, fanout):
+    n_batches = 4_000
+    rows = [inputs.distinct_targets(N, per, seed=b) for b in range(n_batches)]
+    rows[17] = rows[17][:0]
+    offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    d = ctx.sample_many(torch.cat(rows), offs, [fanout, 3], list(range(n_batches)), caps={"max_nodes_per_batch": 600})
+    for b in (0, 16, 17, 18, 1_999, n_batches - 1):
+        one = ctx.sample(rows[b], [fanout, 3], b)
+        x, y = d.view(b), one.view(0)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
+        one.free()
+    d.free()
