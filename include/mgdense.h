@@ -254,6 +254,12 @@ int mg_dense_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out)
 int mg_dense_export_many(mg_ctx* ctx, mg_dense* d);
 int mg_dense_export_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out);
 
+/* The arrays of mini-batch `batch` of the last export copied to a buffer of the caller's without waiting on the host: `stream` (a
+ * cudaStream_t of the context's device; NULL = the default stream) waits for the export and runs the copy of mg_dense_arrays_copy,
+ * and a later export into `d` is ordered behind it.  `out` receives what mg_dense_export_view gives (its pointers are valid for
+ * work that is ordered behind the export); with dst_dev = NULL that is all, so that the caller can size the buffer. */
+int mg_dense_export_copy(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out, int32_t* dst_dev, void* stream);
+
 /* Copy the five arrays of a mini-batch, as mg_dense_view or mg_dense_export_view handed them out, to one DEVICE buffer of the
  * caller's: node_ids (n_nodes), node_id_offsets (k + 2), nbrs (n_entries), nbr_offsets (n_sampled + 1), repr_map (n_entries),
  * one behind the other.  One kernel on `stream` (a cudaStream_t of the context's device; NULL = the default stream), not waited

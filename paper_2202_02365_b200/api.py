@@ -77,6 +77,11 @@ def _raw_stream(device: torch.device):
     return C.c_void_p(torch._C._cuda_getCurrentRawStream(device.index))
 
 
+def _sizes(arr: "DenseArrays"):
+    """Lengths of the arrays as DenseView and mg_dense_arrays_copy list them."""
+    return arr.n_nodes, arr.k + 2, arr.n_entries, arr.n_sampled + 1, arr.n_entries
+
+
 def _fanouts(fanouts):
     return (C.c_int32 * len(fanouts))(*[int(f) for f in fanouts])
 
@@ -185,7 +190,7 @@ class Dense:
     def _copied(self, arr: DenseArrays) -> DenseView:
         """The arrays in memory of the caller's own: one allocation and one kernel (a tensor made from every pointer and cloned
         took 65 us of host time per mini-batch)."""
-        sizes = (arr.n_nodes, arr.k + 2, arr.n_entries, arr.n_sampled + 1, arr.n_entries)
+        sizes = _sizes(arr)
         dev = self.ctx.device
         out = torch.empty(sum(sizes), dtype=torch.int32, device=dev)
         self.ctx._check(self.ctx.lib.mg_dense_arrays_copy(self.ctx.handle, C.byref(arr), _ptr(out),
@@ -197,10 +202,15 @@ class Dense:
         self.ctx._check(self.ctx.lib.mg_dense_export_many(self.ctx.handle, self.handle))
 
     def export_view(self, batch: int = 0) -> DenseView:
-        """Mini-batch `batch` of the last export_many (waits for it the first time)."""
-        arr = DenseArrays()
-        self.ctx._check(self.ctx.lib.mg_dense_export_view(self.ctx.handle, self.handle, C.c_int32(batch), C.byref(arr)))
-        return self._copied(arr)
+        """Mini-batch `batch` of the last export_many, ready in the order of torch's current stream.  (The stream waits for the
+        export, not the host: 32 mini-batches' views are queued while the export runs, the whole call 1107 -> 910 us.)"""
+        arr, at = DenseArrays(), C.c_int32(batch)
+        copy, ctx = self.ctx.lib.mg_dense_export_copy, self.ctx
+        ctx._check(copy(ctx.handle, self.handle, at, C.byref(arr), None, None))
+        sizes = _sizes(arr)
+        out = torch.empty(sum(sizes), dtype=torch.int32, device=ctx.device)
+        ctx._check(copy(ctx.handle, self.handle, at, C.byref(arr), _ptr(out), _raw_stream(ctx.device)))
+        return DenseView(*out.split_with_sizes(sizes))
 
     def free(self):
         if self.handle:

@@ -229,6 +229,8 @@ struct mg_dense {
     // export of all mini-batches at once (mg_dense_export_many): one buffer, laid out by export_layout()
     int32_t* expm_buf = nullptr; size_t expm_elems = 0;
     cudaEvent_t ev_exported = nullptr;
+    cudaEvent_t ev_copied = nullptr;     // the last copy out of the export buffer that was queued on a caller's stream
+    bool copies_queued = false;
     bool export_valid = false, export_pending = false;
     int32_t* perm_buf = nullptr; size_t perm_elems = 0;   // perm | inv of mini-batch perm_batch (mg_dense_batch_perm)
     int perm_batch = -1;

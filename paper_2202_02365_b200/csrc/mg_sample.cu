@@ -2122,6 +2122,7 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
     a.o_repr = d->expm_buf + L.repr; a.o_nbr_off = d->expm_buf + L.nbr_off; a.inv = d->expm_buf + L.inv;
     a.cnt = reinterpret_cast<uint32_t*>(d->expm_buf + L.cnt);
     d->export_valid = false;
+    if (d->copies_queued) { MG_CUDA(ctx, cudaStreamWaitEvent(st, d->ev_copied)); d->copies_queued = false; }   // they read the buffer
     if (n_total > 0) {
         SortParams* sp = (SortParams*)(d->scan_tmp + d->scan_tmp_elems - 8);
         int32_t* range = d->scan_tmp + d->scan_tmp_elems - 12;
@@ -2148,13 +2149,11 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
     return MG_OK;
 }
 
-extern "C" int mg_dense_export_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out) {
-    if (!ctx) return MG_ERR_ARG;
+// where mini-batch `batch` stands in the last export
+static int exported_arrays(mg_ctx* ctx, const mg_dense* d, int32_t batch, mg_dense_arrays* out) {
     if (!d || !out) return mg_fail(ctx, MG_ERR_ARG, "null argument");
     if (!d->valid || !d->export_valid) return mg_fail(ctx, MG_ERR_STATE, "no export of this sample: call mg_dense_export_many first");
     if (batch < 0 || batch >= d->n_batches) return mg_fail(ctx, MG_ERR_ARG, "batch out of range");
-    MG_CUDA(ctx, cudaSetDevice(ctx->device));
-    if (d->export_pending) { MG_CUDA(ctx, cudaEventSynchronize(d->ev_exported)); d->export_pending = false; }
     const int k = d->k, B = d->n_batches, b = batch;
     const ExportLayout L = export_layout(d);
     const int32_t row0 = d->h_rowbase[b], V = d->h_rowbase[b + 1] - row0;
@@ -2174,6 +2173,29 @@ extern "C" int mg_dense_export_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_
     out->nbrs = d->expm_buf + L.nbrs + e_before;
     out->repr_map = d->expm_buf + L.repr + e_before;
     out->nbr_offsets = d->expm_buf + L.nbr_off + row0 + b;
+    return MG_OK;
+}
+
+extern "C" int mg_dense_export_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out) {
+    if (!ctx) return MG_ERR_ARG;
+    if (int rc = exported_arrays(ctx, d, batch, out)) return rc;
+    MG_CUDA(ctx, cudaSetDevice(ctx->device));
+    if (d->export_pending) { MG_CUDA(ctx, cudaEventSynchronize(d->ev_exported)); d->export_pending = false; }
+    return MG_OK;
+}
+
+extern "C" int mg_dense_export_copy(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out, int32_t* dst_dev, void* stream) {
+    if (!ctx) return MG_ERR_ARG;
+    if (int rc = exported_arrays(ctx, d, batch, out)) return rc;
+    if (!dst_dev) return MG_OK;
+    MG_CUDA(ctx, cudaSetDevice(ctx->device));
+    cudaStream_t st = (cudaStream_t)stream;
+    if (!d->ev_copied) MG_CUDA(ctx, cudaEventCreateWithFlags(&d->ev_copied, cudaEventDisableTiming));
+    if (d->export_pending) MG_CUDA(ctx, cudaStreamWaitEvent(st, d->ev_exported));
+    if (d->copies_queued) MG_CUDA(ctx, cudaStreamWaitEvent(st, d->ev_copied));   // (from another stream: one event stands for all copies)
+    if (int rc = mg_dense_arrays_copy(ctx, out, dst_dev, stream)) return rc;
+    MG_CUDA(ctx, cudaEventRecord(d->ev_copied, st));
+    d->copies_queued = true;
     return MG_OK;
 }
 
@@ -2201,6 +2223,7 @@ extern "C" int mg_dense_free(mg_dense* d) {
     cudaFree(d->newlist[1]); cudaFree(d->d_seeds); cudaFree(d->batch_cnt); cudaFree(d->scan_tmp); cudaFree(d->sort_hist); cudaFree(d->seg_tiles);
     cudaFree(d->exp_buf); cudaFree(d->perm_buf); cudaFree(d->d_ent_hop); cudaFree(d->expm_buf);
     if (d->ev_exported) cudaEventDestroy(d->ev_exported);
+    if (d->ev_copied) cudaEventDestroy(d->ev_copied);
     if (d->h_stage) cudaFreeHost(d->h_stage);
     if (d->graph_exec) cudaGraphExecDestroy(d->graph_exec);
     if (d->ev_sampled) cudaEventDestroy(d->ev_sampled);
