@@ -425,6 +425,15 @@ int mg_profile_read(mg_ctx* ctx, int32_t* n_phases, const char** names, double* 
  * forward pass, layers not kept), MG_ERR_OOM. */
 int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, float* d_h0_dev);
 
+/* The same in two calls, so that the caller's host work runs beside the pass: mg_backward_begin queues it (arguments and errors of
+ * mg_backward), with ids_dev (DEVICE, nullable) also what mg_dense_packed_ids writes, and with grads_dev (DEVICE, nullable) a copy of
+ * the whole block of gradients (mg_model_grads) on `grads_stream`, behind the pass.  mg_backward_end waits for the pass -- for the
+ * copy only as far as grads_stream's own order goes -- and returns its status.  Every successful begin wants its end before the next
+ * call on the context. */
+int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, float* d_h0_dev, int32_t* ids_dev, float* grads_dev,
+                      void* grads_stream);
+int mg_backward_end(mg_ctx* ctx);
+
 /* DEVICE pointers to the gradients mg_backward left for layer `layer` (1..k): d_w_self and d_w_nbr row-major
  * [dims[layer-1], dims[layer]], d_bias [dims[layer]].  Owned by the model; one block, layer after layer d_w_self, d_w_nbr,
  * d_bias, so that layer 1's d_w_self is the start of all of them.  Errors: MG_ERR_ARG, MG_ERR_STATE. */

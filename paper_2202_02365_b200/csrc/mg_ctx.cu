@@ -359,6 +359,7 @@ extern "C" int mg_destroy(mg_ctx* c) {
     cudaFree(c->view_ws); cudaFree(c->d_part_start); cudaFree(c->d_part_of_node); cudaFree(c->d_local_of_node); cudaFree(c->d_nodes_by_part);
     cudaFree(c->ws_x); cudaFree(c->ws_meta); cudaFree(c->ws_h[0]); cudaFree(c->ws_h[1]);
     cudaEventDestroy(c->ev_fwd_done); cudaEventDestroy(c->ev_out_done); cudaEventDestroy(c->ev_user);
+    if (c->ev_backward) cudaEventDestroy(c->ev_backward);
     for (int i = 0; i < 2; ++i) { if (c->ev_hk_done[i]) cudaEventDestroy(c->ev_hk_done[i]); cudaFree(c->hk_buf[i]); }
     cudaFree(c->lp_ws); cudaFree(c->lp_spare); cudaFree(c->dm_images);
     cudaFree(c->bw_g); cudaFree(c->bw_x); cudaFree(c->bw_dx); cudaFree(c->bw_off); cudaFree(c->bw_rev);

@@ -1217,7 +1217,15 @@ __global__ void __launch_bounds__(kThreads) k_packed_ids(PackedIdArgs a) {
 
 }  // namespace
 
-extern "C" int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, float* d_h0_dev) {
+static void launch_packed_ids(mg_ctx* ctx, const mg_dense* d, int32_t* ids_dev) {
+    PackedIdArgs a{{d->n_batches, d->k, d->rowbase, d->cum, d->node_off}, d->nodes, d->h_hdr.rows_total[0], ids_dev};
+    if (a.n_rows <= 0) return;
+    k_packed_ids<<<mg_grid(ctx, 4), kThreads, 0, ctx->stream>>>(a);
+    ctx->launches++;
+}
+
+extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, float* d_h0_dev, int32_t* ids_dev,
+                                 float* grads_dev, void* grads_stream) {
     if (!ctx) return MG_ERR_ARG;
     int rc = forward_checks(ctx, m, d);
     if (rc) return rc;
@@ -1366,9 +1374,29 @@ extern "C" int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d
         else k_grad_gather<false><<<ggrid, kThreads, 0, st>>>(ga);
         ctx->launches++;
     }
+    if (ids_dev) launch_packed_ids(ctx, d, ids_dev);
+    if (!ctx->ev_backward) MG_CUDA(ctx, cudaEventCreateWithFlags(&ctx->ev_backward, cudaEventDisableTiming));
     MG_CUDA(ctx, cudaGetLastError());
-    MG_CUDA(ctx, cudaStreamSynchronize(st));
+    MG_CUDA(ctx, cudaEventRecord(ctx->ev_backward, st));
+    if (grads_dev) {
+        cudaStream_t gs = (cudaStream_t)grads_stream;
+        if (gs != st) MG_CUDA(ctx, cudaStreamWaitEvent(gs, ctx->ev_backward));
+        MG_CUDA(ctx, cudaMemcpyAsync(grads_dev, m->g_block, m->g_elems * sizeof(float), cudaMemcpyDeviceToDevice, gs));
+    }
+    return MG_OK;
+}
+
+extern "C" int mg_backward_end(mg_ctx* ctx) {
+    if (!ctx) return MG_ERR_ARG;
+    if (!ctx->ev_backward) return mg_fail(ctx, MG_ERR_STATE, "mg_backward_begin has not run");
+    MG_CUDA(ctx, cudaSetDevice(ctx->device));
+    MG_CUDA(ctx, cudaEventSynchronize(ctx->ev_backward));
     return mg_gemm_tf32_status(ctx);
+}
+
+extern "C" int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, float* d_h0_dev) {
+    if (int rc = mg_backward_begin(ctx, m, d, d_out_dev, d_h0_dev, nullptr, nullptr, nullptr)) return rc;
+    return mg_backward_end(ctx);
 }
 
 extern "C" int mg_model_grads(const mg_model* m, int32_t layer, const float** d_w_self, const float** d_w_nbr, const float** d_bias) {
@@ -1504,11 +1532,7 @@ extern "C" int mg_dense_packed_ids(mg_ctx* ctx, mg_dense* d, int32_t* ids_dev) {
     if (d->pending) return mg_fail(ctx, MG_ERR_STATE, "a sample is in flight on this mg_dense: call mg_sample_many_end first");
     if (!d->valid) return mg_fail(ctx, MG_ERR_STATE, "mg_dense holds no completed sample");
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
-    PackedIdArgs a{{d->n_batches, d->k, d->rowbase, d->cum, d->node_off}, d->nodes, d->h_hdr.rows_total[0], ids_dev};
-    if (a.n_rows > 0) {
-        k_packed_ids<<<mg_grid(ctx, 4), kThreads, 0, ctx->stream>>>(a);
-        ctx->launches++;
-    }
+    launch_packed_ids(ctx, d, ids_dev);
     MG_CUDA(ctx, cudaGetLastError());
     MG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return MG_OK;

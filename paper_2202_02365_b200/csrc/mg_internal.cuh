@@ -137,6 +137,7 @@ struct mg_ctx {
 
     // asynchronous output copy of mg_forward_host_async
     cudaEvent_t ev_fwd_done = nullptr, ev_out_done = nullptr;
+    cudaEvent_t ev_backward = nullptr;   // the end of the last mg_backward_begin
     bool out_check_gemm = false;
     // H^k goes to one of two buffers in turn, so that a forward pass need not wait for the copy of the previous
     // pass's output to the host
