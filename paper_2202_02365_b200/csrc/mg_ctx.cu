@@ -303,6 +303,7 @@ extern "C" int mg_create(mg_ctx** out, int device, void* stream) {
     int prio_least = 0, prio_greatest = 0;
     cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);
     if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&c->prep_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithPriority(&c->sample_stream, cudaStreamNonBlocking, prio_least) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_user, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fwd_done, cudaEventDisableTiming) != cudaSuccess ||
@@ -350,6 +351,7 @@ extern "C" int mg_destroy(mg_ctx* c) {
     cudaStreamSynchronize(c->stream);
     cudaStreamSynchronize(c->side);
     cudaStreamSynchronize(c->sample_stream);
+    cudaStreamSynchronize(c->prep_stream);
     for (auto ev : c->pending_events) cudaEventDestroy(ev);
     for (auto& p : c->prof_pending) { cudaEventDestroy(p.second.first); cudaEventDestroy(p.second.second); }
     free_view(c);
@@ -361,7 +363,9 @@ extern "C" int mg_destroy(mg_ctx* c) {
     cudaEventDestroy(c->ev_fwd_done); cudaEventDestroy(c->ev_out_done); cudaEventDestroy(c->ev_user);
     if (c->ev_backward) cudaEventDestroy(c->ev_backward);
     for (int i = 0; i < 2; ++i) { if (c->ev_hk_done[i]) cudaEventDestroy(c->ev_hk_done[i]); cudaFree(c->hk_buf[i]); }
-    cudaFree(c->lp_ws); cudaFree(c->lp_spare); cudaFree(c->dm_images);
+    cudaFree(c->lp_ws); cudaFree(c->dm_images);
+    for (auto& s : c->lp_spare) { cudaFree(s.block); if (s.idle) cudaEventDestroy(s.idle); }
+    cudaStreamDestroy(c->prep_stream);
     cudaFree(c->bw_g); cudaFree(c->bw_x); cudaFree(c->bw_dx); cudaFree(c->bw_off); cudaFree(c->bw_rev);
     cudaFree(c->gat_x); cudaFree(c->gat_z); cudaFree(c->gat_s); cudaFree(c->gat_h[0]); cudaFree(c->gat_h[1]);
     cudaStreamDestroy(c->sample_stream);

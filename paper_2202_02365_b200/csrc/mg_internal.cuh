@@ -152,7 +152,11 @@ struct mg_ctx {
     // link-prediction batches: scratch of mg_lp_prepare (grows, never shrinks) and one spare result block, so that a
     // loop of prepare / free allocates nothing
     char* lp_ws = nullptr; size_t lp_ws_bytes = 0;
-    char* lp_spare = nullptr; size_t lp_spare_bytes = 0;
+    // blocks of freed link-prediction batches, for the next ones: two, so that a batch can be prepared while the scores of the one
+    // before it are still being computed; `idle` is recorded on the context's stream when the batch is freed
+    struct LpSpare { char* block = nullptr; size_t bytes = 0; cudaEvent_t idle = nullptr; };
+    LpSpare lp_spare[2];
+    cudaStream_t prep_stream = nullptr;   // mg_lp_prepare's copies and kernels
     int32_t* lp_words = nullptr;       // mapped pinned host words {status, n_targets} that mg_lp_prepare's last kernel writes (behind h_flags)
     int32_t* lp_words_dev = nullptr;   // their device address
     float* gat_x = nullptr; float* gat_z = nullptr; float* gat_s = nullptr; float* gat_h[2] = {nullptr, nullptr};   // mg_gat_forward scratch

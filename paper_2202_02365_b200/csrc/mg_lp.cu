@@ -540,13 +540,17 @@ extern "C" int mg_lp_free(mg_lp_batch* lp) {
     if (!lp) return MG_OK;
     cudaSetDevice(lp->device);
     mg_ctx* ctx = lp->ctx;
-    // the block becomes the context's spare (the next mg_lp_prepare takes it) unless the spare is already larger
-    if (ctx && lp->block && lp->block_bytes > ctx->lp_spare_bytes) {
-        cudaFree(ctx->lp_spare);
-        ctx->lp_spare = lp->block; ctx->lp_spare_bytes = lp->block_bytes;
-    } else {
-        cudaFree(lp->block);
+    // the block takes the place of the context's smaller spare (a later mg_lp_prepare takes it) unless that is larger still
+    char* gone = lp->block;
+    if (ctx && lp->block) {
+        mg_ctx::LpSpare& s = ctx->lp_spare[ctx->lp_spare[0].bytes <= ctx->lp_spare[1].bytes ? 0 : 1];
+        if (lp->block_bytes > s.bytes && (s.idle || cudaEventCreateWithFlags(&s.idle, cudaEventDisableTiming) == cudaSuccess) &&
+            cudaEventRecord(s.idle, ctx->stream) == cudaSuccess) {
+            gone = s.block;
+            s.block = lp->block; s.bytes = lp->block_bytes;
+        }
     }
+    cudaFree(gone);
     delete lp;
     return MG_OK;
 }
@@ -561,7 +565,10 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     const int64_t total = 2 * n_edges + (int64_t)n_chunks * negs;
     if (total >= (1ll << 31)) return mg_fail(ctx, MG_ERR_ARG, "batch too large");
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
-    cudaStream_t st = ctx->stream;
+    // Its own stream: the edges come from the host, so nothing here waits for the layers and scores of the batch before, which may
+    // still be running on the context's (50,000 edges against 1,000 negatives a chunk: a step 444 -> 408 us).  The call ends with a
+    // host wait, so whatever follows it sees its results; the partition maps are uploaded with one.
+    cudaStream_t st = ctx->prep_stream;
     mg_lp_batch* lp = new mg_lp_batch();
     lp->ctx = ctx; lp->device = ctx->device; lp->n_edges = n_edges; lp->n_chunks = n_chunks; lp->negs = negs;
 
@@ -591,11 +598,20 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     uint32_t* before = (uint32_t*)take(4 * (size_t)n_words);
     uint32_t* ticket = d_status + 1;
     int32_t* d_nt = (int32_t*)(d_status + 2);
-    // results: one block, taken from the context's spare when that is large enough
+    // results: one block, one of the context's spares when that is large enough: one that nothing reads any more, or, when both are
+    // still read, the first of them (the stream then waits)
     const size_t blk_bytes = up(4 * (size_t)total) + 3 * up(4 * (size_t)n_edges) + 2 * up(4 * n_neg);
-    if (ctx->lp_spare && ctx->lp_spare_bytes >= blk_bytes) {
-        lp->block = ctx->lp_spare; lp->block_bytes = ctx->lp_spare_bytes;
-        ctx->lp_spare = nullptr; ctx->lp_spare_bytes = 0;
+    mg_ctx::LpSpare* spare = nullptr;
+    for (auto& s : ctx->lp_spare)
+        if (s.block && s.bytes >= blk_bytes && cudaEventQuery(s.idle) == cudaSuccess) { spare = &s; break; }
+    cudaGetLastError();   // (a spare that is still read is no error)
+    if (!spare && ctx->lp_spare[0].block && ctx->lp_spare[1].block)
+        for (auto& s : ctx->lp_spare)
+            if (s.bytes >= blk_bytes) { spare = &s; break; }
+    if (spare) {
+        lp->block = spare->block; lp->block_bytes = spare->bytes;
+        spare->block = nullptr; spare->bytes = 0;
+        cudaStreamWaitEvent(st, spare->idle);
     } else if (cudaMalloc((void**)&lp->block, blk_bytes) != cudaSuccess) {
         cudaGetLastError(); delete lp;
         return mg_fail(ctx, MG_ERR_OOM, "allocation of the link-prediction batch failed");

@@ -77,3 +77,44 @@ def test_negative_scores_by_the_number_of_tiles(edges, chunks, negs, corrupt):
             # operands rounded to ten bits, sums of 36 products: below 1e-3 of the norm, no value off by 1 % of the rows' rms
             err = got[mine].double() - want
             assert float(err.norm() / want.norm()) < 1e-3 and float(err.abs().max() / want.square().mean().sqrt()) < 1e-2
+
+
+# batches are prepared while the scores of the ones before are computed, in the blocks of freed batches: growing, shrinking, two alive at once
+@pytest.mark.parametrize("sizes", [[40_000] * 6, [100, 40_000, 300, 50_000, 20_000, 60_000]])
+def test_batches_prepared_beside_scores(sizes):
+    nodes, dim = 400_000, 64
+    ctx = mg.Context(0)
+    g = inputs.erdos_renyi_graph(nodes, 2 * nodes, seed=1, device="cuda")
+    ctx.load_graph(g.row_offsets, g.nbrs)
+    ctx.load_features(torch.zeros((nodes, 4), device="cuda"))
+    r = inputs.normal_features(50, dim, seed=7, device="cuda")
+    table = inputs.normal_features(nodes, dim, seed=6, device="cuda")
+    rng = np.random.RandomState(4)
+    batches = [tuple(torch.from_numpy(rng.randint(0, n, e).astype(np.int32)) for n in (nodes, 50, nodes)) for e in sizes]
+
+    def score(i, wait):
+        lp = ctx.lp_prepare(*batches[i], 4, 500, seed=i)
+        h = table[lp.targets().long()]
+        if wait:
+            torch.cuda.synchronize()
+        out = ctx.distmult_score(lp, h, r)
+        if wait:
+            torch.cuda.synchronize()
+        return lp, out
+
+    got, held = [], None
+    for i in range(len(sizes)):
+        lp, out = score(i, False)
+        got.append(out)
+        if i % 3 == 1:
+            held = lp                       # freed a batch later
+        else:
+            lp.free()
+            if held is not None:
+                held.free()
+                held = None
+    for i in range(len(sizes)):
+        lp, want = score(i, True)
+        lp.free()
+        for x, y in zip(got[i], want):
+            assert torch.equal(x, y), i
