@@ -1754,6 +1754,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     d->valid = false;
     d->pending = false;
     d->export_valid = false;
+    if (ctx->last_fwd_dense == d) ctx->last_fwd_dense = nullptr;   // (that pass was of the sample that ends here: mg_backward may not follow it)
     if (d->ev_read_done) MG_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, d->ev_read_done, 0));
     int rc = dense_alloc(ctx, d, n_batches, k, cap_nodes, std::max<int64_t>(cap_entries, 1), table_size, smem_last ? (int32_t)dedup_nb : 0);
     if (rc) { if (created) mg_dense_free(d); return rc; }

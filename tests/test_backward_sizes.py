@@ -121,3 +121,29 @@ def test_weight_gradients_on_the_tensor_cores(rows, d_in, d_out, half, aggregato
         assert float((x.double().cpu().reshape(p.shape) - p.grad).norm()) <= 2 ** -9 * float(p.grad.norm())
     order, want_order = torch.argsort(ids.cpu()), torch.argsort(want_ids)
     assert float((g_rows.double().cpu()[order] - h.grad[want_order]).norm()) <= 2 ** -9 * float(h.grad.norm())
+
+
+# the row metadata and the kept outputs are the old sample's: with another sample in the handle they would be read past their end
+@pytest.mark.parametrize("precision", [mg.GEMM_TF32, mg.GEMM_FP32])
+@pytest.mark.parametrize("fails", [False, True])
+def test_sample_between_forward_and_backward_is_refused(precision, fails):
+    graph = star_graph()
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(inputs.normal_features(N, 16, seed=4).cuda())
+    ctx.keep_layer_outputs(True)
+    model = ctx.model(inputs.random_bias_layers([16, 8], seed=5), precision)
+    dense = ctx.sample(inputs.distinct_targets(N, 40, seed=6), [6], 7)
+    out = torch.empty((40, 8), device="cuda")
+    ctx.forward(model, dense, out)
+    if fails:                                                # a sample that ends in an error leaves nothing to go back through either
+        with pytest.raises(mg.MgError):
+            ctx.sample(torch.tensor([1, 1], dtype=torch.int32), [6], 7, out=dense)
+    else:
+        ctx.sample(inputs.distinct_targets(N, 40, seed=6), [6], 8, out=dense)
+    with pytest.raises(mg.MgError) as e:
+        ctx.backward(model, dense, torch.ones_like(out))
+    assert e.value.code == -2                                # MG_ERR_STATE
+    if not fails:
+        ctx.forward(model, dense, out)
+        ctx.backward(model, dense, torch.ones_like(out))
