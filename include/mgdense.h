@@ -195,7 +195,8 @@ int mg_commit_resident(mg_ctx* ctx, int32_t timeout_ms);
  * (seed, node, hop, slot), kept in row order.  Each new delta is the ascending list of
  * unique new neighbours not yet in node_ids (computeNextDelta).
  * `targets` is a host pointer, or a device pointer if targets_on_device; target_offsets,
- * fanouts and seeds are host pointers.  *out: NULL to allocate a new mg_dense, or an
+ * fanouts and seeds are host pointers.  Targets in device or pinned host memory are read behind
+ * the work queued on the context's stream before the call.  *out: NULL to allocate a new mg_dense, or an
  * existing one (of this context) to reuse its buffers.
  * The call is synchronous: on return the sample is complete and its status checked.  The kernels run
  * on a library-owned sampling stream, ordered after the work queued on the context's stream so far.

@@ -341,6 +341,22 @@ static inline cudaError_t mg_smem_limit(uint64_t* done, int device, const void* 
     return e;
 }
 
+// Host memory that a call was handed.  Pageable memory is what the host's own program order says it is, and may be read at once.
+// Pinned memory may be the destination of a copy that is still queued: it is read in stream order, by a copy or, where the whole range
+// is mapped, through `*mapped` by a kernel.
+enum HostMemory { HOST_PAGEABLE, HOST_PINNED, HOST_MAPPED };
+static inline HostMemory mg_host_memory(const void* p, size_t bytes, const void** mapped) {
+    cudaPointerAttributes first, last;
+    const char* end = static_cast<const char*>(p) + (bytes ? bytes - 1 : 0);
+    if (cudaPointerGetAttributes(&first, p) != cudaSuccess || cudaPointerGetAttributes(&last, end) != cudaSuccess) { cudaGetLastError(); return HOST_PINNED; }
+    if (first.type == cudaMemoryTypeUnregistered && last.type == cudaMemoryTypeUnregistered) return HOST_PAGEABLE;
+    if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer ||
+        static_cast<const char*>(last.devicePointer) - static_cast<const char*>(first.devicePointer) != end - static_cast<const char*>(p))
+        return HOST_PINNED;
+    *mapped = first.devicePointer;
+    return HOST_MAPPED;
+}
+
 static inline int mg_grid(const mg_ctx* ctx, int ctas_per_sm) { return ctx->n_sms * ctas_per_sm; }
 
 // how kernels find a node's partition and its row in the feature buffer

@@ -25,7 +25,7 @@
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int64_t kStageTargets = 16384;   // targets in host memory that travel in the staging block of a sample
+constexpr int64_t kStageTargets = 16384;   // targets in host memory that are read without a copy of their own
 
 // -------------------------------------------------------------------------------------
 // generic exclusive scan over a device-sized range (three kernels, no inter-block waits)
@@ -1776,7 +1776,9 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     const size_t hdr_ints = sizeof(DenseHeader) / 4;
     const size_t seeds_at = (hdr_ints + (size_t)(B + 1) + (size_t)B * (k + 2) + 1) & ~(size_t)1;
     const size_t targets_at = seeds_at + 2 * (size_t)B;
-    const size_t n_staged = !targets_on_device && T <= kStageTargets ? kStageTargets : 0;
+    const void* mapped = nullptr;
+    const HostMemory kind = targets_on_device || T == 0 ? HOST_PAGEABLE : mg_host_memory(targets, sizeof(int32_t) * (size_t)T, &mapped);
+    const size_t n_staged = !targets_on_device && T <= kStageTargets && kind == HOST_PAGEABLE ? kStageTargets : 0;
     const size_t n_summary = hdr_ints + (size_t)B * (k + 2) + 2 * (size_t)(k + 1) * (B + 1) + (size_t)k * (B + 1);
     const size_t summary_at = targets_at + n_staged;
     if (d->h_stage_ints < summary_at + n_summary) {
@@ -1810,6 +1812,8 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     else if (n_staged) {
         if (T > 0) memcpy(d->h_stage + targets_at, targets, sizeof(int32_t) * T);
         st_hdr->targets = (uint64_t)(uintptr_t)(d->h_stage_dev + targets_at);
+    } else if (kind == HOST_MAPPED && T <= kStageTargets) {
+        st_hdr->targets = (uint64_t)(uintptr_t)mapped;
     } else {
         MG_CUDA(ctx, cudaMemcpyAsync(d->newlist[1], targets, sizeof(int32_t) * T, cudaMemcpyHostToDevice, st));
         st_hdr->targets = (uint64_t)(uintptr_t)d->newlist[1];

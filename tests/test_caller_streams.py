@@ -1,0 +1,45 @@
+"""Calls whose caller works on a stream of its own, or hands over host memory that a stream still writes: what is copied out for the
+caller is the call's result however late the caller's stream runs, and what is read from the caller is what its stream wrote."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2202_02365_b200 as mg
+from paper_2202_02365_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+N = 30_000
+LATE = 200_000_000     # cycles that the caller's stream sleeps: a tenth of a second
+
+
+@pytest.fixture(scope="module")
+def graph():
+    return inputs.erdos_renyi_graph(N, 8 * N, seed=41)
+
+
+def context(graph, dim=32, stream=None):
+    ctx = mg.Context(0, stream)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(inputs.normal_features(N, dim, seed=42, device="cuda"))
+    torch.cuda.synchronize()
+    return ctx
+
+
+def arrays(view):
+    return [x.cpu() for x in (view.node_ids, view.node_id_offsets, view.nbrs, view.nbr_offsets, view.repr_map)]
+
+
+# up to 16,384 targets travel in the staging block of the call, more are copied
+@pytest.mark.parametrize("count", [137, 20_000])
+def test_pinned_targets_that_the_stream_still_writes(graph, count):
+    ctx = context(graph)
+    ids = inputs.distinct_targets(N, count, seed=1)
+    want = arrays(ctx.sample(ids, [4, 3], 5).view(0))
+    host = inputs.distinct_targets(N, count, seed=2).pin_memory()
+    device = ids.cuda()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(LATE)
+    host.copy_(device, non_blocking=True)
+    got = arrays(ctx.sample(host, [4, 3], 5).view(0))
+    assert torch.equal(host, ids) and all(torch.equal(x, y) for x, y in zip(got, want))
