@@ -368,8 +368,8 @@ int mg_forward_noalloc(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out_d
 
 /* ---- link prediction: shared negatives, target union, DistMult ------------------------ */
 
-/* Prepare a batch of n_edges training edges (HOST int32 src / rel / dst; dst aggregates
- * from src).  Edge i belongs to chunk floor(i * n_chunks / n_edges); chunk c shares
+/* Prepare a batch of n_edges training edges (HOST int32 src / rel / dst, in pinned memory read behind
+ * the work queued on the context's stream before the call; dst aggregates from src).  Edge i belongs to chunk floor(i * n_chunks / n_edges); chunk c shares
  * negs_per_chunk negatives, negative t being the resident node number
  * mulhi(Philox4x32-10(counter = (c, t, 0xFFFFFFFF, 0), key = seed).word0, #resident nodes)
  * counted in ascending partition order.  The targets of the batch are the ascending unique

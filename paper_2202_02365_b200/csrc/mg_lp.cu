@@ -565,8 +565,8 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     const int64_t total = 2 * n_edges + (int64_t)n_chunks * negs;
     if (total >= (1ll << 31)) return mg_fail(ctx, MG_ERR_ARG, "batch too large");
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
-    // Its own stream: the edges come from the host, so nothing here waits for the layers and scores of the batch before, which may
-    // still be running on the context's (50,000 edges against 1,000 negatives a chunk: a step 444 -> 408 us).  The call ends with a
+    // Its own stream: edges in pageable memory are the host's, so nothing here waits for the layers and scores of the batch before, which
+    // may still be running on the context's (50,000 edges against 1,000 negatives a chunk: a step 444 -> 408 us).  The call ends with a
     // host wait, so whatever follows it sees its results; the partition maps are uploaded with one.
     cudaStream_t st = ctx->prep_stream;
     mg_lp_batch* lp = new mg_lp_batch();
@@ -626,6 +626,13 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     lp->neg_ids = (int32_t*)take(4 * n_neg);
     lp->neg_idx = (int32_t*)take(4 * n_neg);
 
+    // (edges in pinned memory may be the destination of a copy that is still queued on the context's stream)
+    const void* mapped;
+    for (const int32_t* p : {src, rel, dst})
+        if (mg_host_memory(p, 4 * (size_t)n_edges, &mapped) != HOST_PAGEABLE) {
+            if (cudaEventRecord(ctx->ev_user, ctx->stream) == cudaSuccess) cudaStreamWaitEvent(st, ctx->ev_user);
+            break;
+        }
     cudaMemcpyAsync(d_src, src, 4 * n_edges, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_dst, dst, 4 * n_edges, cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(d_status, 0, cleared, st);

@@ -43,3 +43,18 @@ def test_pinned_targets_that_the_stream_still_writes(graph, count):
     host.copy_(device, non_blocking=True)
     got = arrays(ctx.sample(host, [4, 3], 5).view(0))
     assert torch.equal(host, ids) and all(torch.equal(x, y) for x, y in zip(got, want))
+
+
+def test_pinned_edges_that_the_stream_still_writes(graph):
+    ctx = context(graph)
+    rng = np.random.RandomState(3)
+    edges = [torch.from_numpy(rng.randint(0, n, 5_000).astype(np.int32)) for n in (N, 50, N)]
+    want = ctx.lp_prepare(*edges, 4, 100, seed=6).view()
+    host = [torch.zeros(5_000, dtype=torch.int32).pin_memory() for _ in edges]
+    device = [e.cuda() for e in edges]
+    torch.cuda.synchronize()
+    torch.cuda._sleep(LATE)
+    for h, d in zip(host, device):
+        h.copy_(d, non_blocking=True)
+    got = ctx.lp_prepare(*host, 4, 100, seed=6).view()
+    assert all(torch.equal(got[key], want[key]) for key in want)
