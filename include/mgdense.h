@@ -385,6 +385,10 @@ int mg_lp_view(const mg_lp_batch* lp, int32_t* n_targets, const int32_t** target
 /* Copy the target ids (n_targets of mg_lp_view) to a DEVICE buffer of the caller's on `stream` (a cudaStream_t of the context's
  * device; NULL = the default stream); not waited for. */
 int mg_lp_targets(mg_ctx* ctx, const mg_lp_batch* lp, int32_t* dst_dev, void* stream);
+/* Reads of mg_lp_view's arrays that the caller has queued on `stream` (a cudaStream_t of the context's device; NULL = the default
+ * stream) come before any reuse of the batch's memory after mg_lp_free.  (mg_lp_targets does this for its own copy; work on the
+ * context's stream needs no call.) */
+int mg_lp_record_stream(mg_ctx* ctx, const mg_lp_batch* lp, void* stream);
 int mg_lp_free(mg_lp_batch* lp);
 
 /* DistMult: pos[i] = sum_d h[s_i,d] rel_emb[r_i,d] h[o_i,d]; neg_dst[i,t] the same with the

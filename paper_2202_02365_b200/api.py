@@ -30,7 +30,7 @@ EXPORTS = [
     "mg_create", "mg_destroy", "mg_last_error", "mg_load_graph", "mg_load_out_graph", "mg_set_sample_direction", "mg_set_partitioning",
     "mg_load_features", "mg_set_partition_source", "mg_set_resident", "mg_commit_resident", "mg_sample_many", "mg_sample_many_begin", "mg_sample_many_end", "mg_sample",
     "mg_dense_counts", "mg_dense_view", "mg_dense_export_many", "mg_dense_export_view", "mg_dense_export_copy", "mg_dense_arrays_copy", "mg_dense_free", "mg_model_create", "mg_model_set_aggregator", "mg_model_set_intermediates", "mg_model_free",
-    "mg_forward", "mg_set_layer_window", "mg_keep_layer_outputs", "mg_forward_host_async", "mg_wait_output", "mg_forward_noalloc", "mg_gather_h0", "mg_layer_output", "mg_lp_prepare", "mg_lp_view", "mg_lp_targets", "mg_lp_free",
+    "mg_forward", "mg_set_layer_window", "mg_keep_layer_outputs", "mg_forward_host_async", "mg_wait_output", "mg_forward_noalloc", "mg_gather_h0", "mg_layer_output", "mg_lp_prepare", "mg_lp_view", "mg_lp_targets", "mg_lp_record_stream", "mg_lp_free",
     "mg_distmult_score", "mg_kernel_launches", "mg_profile", "mg_profile_read", "mg_comet_plan", "mg_comet_bias", "mg_comet_autotune", "mg_gat_model_create", "mg_gat_model_set_heads", "mg_gat_model_free", "mg_gat_forward", "mg_backward", "mg_backward_begin", "mg_backward_end", "mg_model_grads", "mg_model_sgd_step", "mg_model_adagrad_step", "mg_dense_packed_ids", "mg_apply_embedding_sgd",
 ]
 
@@ -311,12 +311,14 @@ class LpBatch:
         self.ctx._check(self.ctx.lib.mg_lp_view(self.handle, C.byref(n), *[C.byref(x) for x in p]))
         dev = self.ctx.device
         nt = n.value
-        return {
+        arrays = {
             "targets": _from_dev(p[0].value, nt, dev), "src_idx": _from_dev(p[1].value, self.n_edges, dev),
             "dst_idx": _from_dev(p[2].value, self.n_edges, dev),
             "neg_ids": _from_dev(p[3].value, self.n_chunks * self.negs, dev).view(self.n_chunks, self.negs),
             "neg_idx": _from_dev(p[4].value, self.n_chunks * self.negs, dev).view(self.n_chunks, self.negs),
         }
+        self.ctx._check(self.ctx.lib.mg_lp_record_stream(self.ctx.handle, self.handle, _raw_stream(dev)))
+        return arrays
 
     def free(self):
         if self.handle:

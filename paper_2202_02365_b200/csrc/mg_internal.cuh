@@ -59,6 +59,12 @@ enum {
     PH_COUNT
 };
 
+// Reads of memory of the library's that callers have queued on streams of their own; one event stands for all of them.
+struct QueuedReads {
+    cudaEvent_t done = nullptr;
+    bool queued = false;
+};
+
 struct mg_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -153,8 +159,9 @@ struct mg_ctx {
     // loop of prepare / free allocates nothing
     char* lp_ws = nullptr; size_t lp_ws_bytes = 0;
     // blocks of freed link-prediction batches, for the next ones: two, so that a batch can be prepared while the scores of the one
-    // before it are still being computed; `idle` is recorded on the context's stream when the batch is freed
-    struct LpSpare { char* block = nullptr; size_t bytes = 0; cudaEvent_t idle = nullptr; };
+    // before it are still being computed; `idle` is recorded on the context's stream when the batch is freed, `reads` stands for the
+    // reads that callers queued on streams of their own
+    struct LpSpare { char* block = nullptr; size_t bytes = 0; cudaEvent_t idle = nullptr; QueuedReads reads; };
     LpSpare lp_spare[2];
     cudaStream_t prep_stream = nullptr;   // mg_lp_prepare's copies and kernels
     int32_t* lp_words = nullptr;       // mapped pinned host words {status, n_targets} that mg_lp_prepare's last kernel writes (behind h_flags)
@@ -290,6 +297,7 @@ struct mg_lp_batch {
     int32_t* neg_idx = nullptr;
     char* block = nullptr;       // the one device allocation the six arrays above live in
     size_t block_bytes = 0;
+    mutable QueuedReads reads;       // of the block
 };
 
 // ---------------------------------------------------------------------------------------
@@ -339,6 +347,22 @@ static inline cudaError_t mg_smem_limit(uint64_t* done, int device, const void* 
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess && device < 64) *done |= 1ull << device;
     return e;
+}
+
+// `stream` has just been given a read: `r` stands for it too
+static inline cudaError_t mg_reads_add(QueuedReads* r, cudaStream_t stream) {
+    cudaError_t e = cudaSuccess;
+    if (!r->done) e = cudaEventCreateWithFlags(&r->done, cudaEventDisableTiming);
+    if (e == cudaSuccess && r->queued) e = cudaStreamWaitEvent(stream, r->done);   // (from another stream)
+    if (e == cudaSuccess) e = cudaEventRecord(r->done, stream);
+    if (e == cudaSuccess) r->queued = true;
+    return e;
+}
+// what `stream` is given from here on comes behind the reads
+static inline cudaError_t mg_reads_wait(QueuedReads* r, cudaStream_t stream) { return r->queued ? cudaStreamWaitEvent(stream, r->done) : cudaSuccess; }
+static inline void mg_reads_free(QueuedReads* r) {
+    if (r->done) cudaEventDestroy(r->done);
+    r->done = nullptr; r->queued = false;
 }
 
 // Host memory that a call was handed.  Pageable memory is what the host's own program order says it is, and may be read at once.

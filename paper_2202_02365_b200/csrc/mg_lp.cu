@@ -548,9 +548,11 @@ extern "C" int mg_lp_free(mg_lp_batch* lp) {
             cudaEventRecord(s.idle, ctx->stream) == cudaSuccess) {
             gone = s.block;
             s.block = lp->block; s.bytes = lp->block_bytes;
+            std::swap(s.reads, lp->reads);
         }
     }
-    cudaFree(gone);
+    cudaFree(gone);   // (waits for what still reads it)
+    mg_reads_free(&lp->reads);
     delete lp;
     return MG_OK;
 }
@@ -603,7 +605,10 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     const size_t blk_bytes = up(4 * (size_t)total) + 3 * up(4 * (size_t)n_edges) + 2 * up(4 * n_neg);
     mg_ctx::LpSpare* spare = nullptr;
     for (auto& s : ctx->lp_spare)
-        if (s.block && s.bytes >= blk_bytes && cudaEventQuery(s.idle) == cudaSuccess) { spare = &s; break; }
+        if (s.block && s.bytes >= blk_bytes && cudaEventQuery(s.idle) == cudaSuccess && (!s.reads.queued || cudaEventQuery(s.reads.done) == cudaSuccess)) {
+            spare = &s;
+            break;
+        }
     cudaGetLastError();   // (a spare that is still read is no error)
     if (!spare && ctx->lp_spare[0].block && ctx->lp_spare[1].block)
         for (auto& s : ctx->lp_spare)
@@ -612,6 +617,8 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
         lp->block = spare->block; lp->block_bytes = spare->bytes;
         spare->block = nullptr; spare->bytes = 0;
         cudaStreamWaitEvent(st, spare->idle);
+        mg_reads_wait(&spare->reads, st);
+        spare->reads.queued = false;
     } else if (cudaMalloc((void**)&lp->block, blk_bytes) != cudaSuccess) {
         cudaGetLastError(); delete lp;
         return mg_fail(ctx, MG_ERR_OOM, "allocation of the link-prediction batch failed");
@@ -673,7 +680,17 @@ extern "C" int mg_lp_view(const mg_lp_batch* lp, int32_t* n_targets, const int32
 extern "C" int mg_lp_targets(mg_ctx* ctx, const mg_lp_batch* lp, int32_t* dst_dev, void* stream) {
     if (!ctx) return MG_ERR_ARG;
     if (!lp || !dst_dev) return mg_fail(ctx, MG_ERR_ARG, "null argument");
+    MG_CUDA(ctx, cudaSetDevice(ctx->device));
     MG_CUDA(ctx, cudaMemcpyAsync(dst_dev, lp->targets, sizeof(int32_t) * (size_t)lp->n_targets, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
+    return mg_lp_record_stream(ctx, lp, stream);
+}
+
+extern "C" int mg_lp_record_stream(mg_ctx* ctx, const mg_lp_batch* lp, void* stream) {
+    if (!ctx) return MG_ERR_ARG;
+    if (!lp) return mg_fail(ctx, MG_ERR_ARG, "null argument");
+    if ((cudaStream_t)stream == ctx->stream) return MG_OK;   // (mg_lp_free's own event covers it)
+    MG_CUDA(ctx, cudaSetDevice(ctx->device));
+    MG_CUDA(ctx, mg_reads_add(&lp->reads, (cudaStream_t)stream));
     return MG_OK;
 }
 

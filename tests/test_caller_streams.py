@@ -58,3 +58,25 @@ def test_pinned_edges_that_the_stream_still_writes(graph):
         h.copy_(d, non_blocking=True)
     got = ctx.lp_prepare(*host, 4, 100, seed=6).view()
     assert all(torch.equal(got[key], want[key]) for key in want)
+
+
+@pytest.mark.parametrize("what", ["targets", "view"])
+def test_arrays_of_a_freed_link_prediction_batch_copied_on_a_late_stream(graph, what):
+    ctx = context(graph)
+    rng = np.random.RandomState(3)
+    batches = [[torch.from_numpy(rng.randint(0, n, 5_000).astype(np.int32)) for n in (N, 50, N)] for _ in range(3)]
+    lps = [ctx.lp_prepare(*b, 4, 100, seed=6) for b in batches]
+    take = (lambda lp: {"targets": lp.targets()}) if what == "targets" else (lambda lp: lp.view())
+    want = [{k: x.cpu() for k, x in take(lp).items()} for lp in lps]
+    for lp in lps:
+        lp.free()
+    got = []
+    with torch.cuda.stream(torch.cuda.Stream()):
+        torch.cuda._sleep(LATE)
+        for b in batches:
+            lp = ctx.lp_prepare(*b, 4, 100, seed=6)
+            got.append(take(lp))
+            lp.free()
+    torch.cuda.synchronize()
+    for g, w in zip(got, want):
+        assert all(torch.equal(g[k].cpu(), w[k]) for k in w)
