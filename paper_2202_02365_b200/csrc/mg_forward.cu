@@ -483,6 +483,7 @@ extern "C" int mg_model_free(mg_model* m) {
         cudaFree(m->w_cat[l]); cudaFree(m->w_cat_t[l]); cudaFree(m->w_pad_t[l]); cudaFree(m->bias[l]);
     }
     cudaFree(m->zeros); cudaFree(m->g_block); cudaFree(m->s_block);
+    mg_reads_free(&m->g_reads);
     for (int l = 0; l < MG_MAX_HOPS; ++l) cudaFree(m->w_pad_h[l]);
     if (m->ctx && m->ctx->last_fwd_model == m) m->ctx->last_fwd_model = nullptr;
     delete m;
@@ -1247,6 +1248,8 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
             m->g_bias[l] = g; g += m->dims[l + 1];
         }
     }
+    MG_CUDA(ctx, mg_reads_wait(&m->g_reads, st));   // (the last pass's gradients may still be on their way to the caller)
+    m->g_reads.queued = false;
     MG_CUDA(ctx, cudaMemsetAsync(m->g_block, 0, m->g_elems * sizeof(float), st));
     if (!m->zeros) {
         if (cudaMalloc((void**)&m->zeros, sizeof(float) * 2 * 1024) != cudaSuccess) { cudaGetLastError(); return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
@@ -1382,6 +1385,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         cudaStream_t gs = (cudaStream_t)grads_stream;
         if (gs != st) MG_CUDA(ctx, cudaStreamWaitEvent(gs, ctx->ev_backward));
         MG_CUDA(ctx, cudaMemcpyAsync(grads_dev, m->g_block, m->g_elems * sizeof(float), cudaMemcpyDeviceToDevice, gs));
+        if (gs != st) MG_CUDA(ctx, mg_reads_add(&m->g_reads, gs));
     }
     return MG_OK;
 }

@@ -280,6 +280,7 @@ struct mg_model {
     size_t g_elems = 0;
     float* g_w_cat[MG_MAX_HOPS] = {nullptr};
     float* g_bias[MG_MAX_HOPS] = {nullptr};
+    QueuedReads g_reads;                       // copies of the block that mg_backward_begin queued on a caller's stream
     float* s_block = nullptr;                  // Adagrad: accumulated squared gradients, laid out like them
     float* zeros = nullptr;
 };

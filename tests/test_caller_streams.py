@@ -80,3 +80,30 @@ def test_arrays_of_a_freed_link_prediction_batch_copied_on_a_late_stream(graph, 
     torch.cuda.synchronize()
     for g, w in zip(got, want):
         assert all(torch.equal(g[k].cpu(), w[k]) for k in w)
+
+
+def training(graph, stream=None):
+    ctx = context(graph, stream=stream)
+    ctx.keep_layer_outputs(True)
+    model = ctx.model(inputs.random_bias_layers([32, 16, 8], seed=7))
+    dense = ctx.sample(inputs.distinct_targets(N, 300, seed=8), [5, 4], 9)
+    out = torch.empty((300, 8), device="cuda")
+    ctx.forward(model, dense, out)
+    d_out = [torch.randn(out.shape, generator=torch.Generator("cuda").manual_seed(i), device="cuda") for i in (1, 2)]
+    torch.cuda.synchronize()
+    return ctx, model, dense, d_out
+
+
+def test_gradients_of_two_passes_copied_on_a_late_stream(graph):
+    ctx, model, dense, d_out = training(graph, torch.cuda.Stream())
+    want = []
+    for d in d_out:
+        want.append(ctx.backward(model, dense, d))
+        torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        torch.cuda._sleep(LATE)
+        got = [ctx.backward(model, dense, d) for d in d_out]
+    torch.cuda.synchronize()
+    for g, w in zip(got, want):
+        for x, y in zip((t for layer in g for t in layer), (t for layer in w for t in layer)):
+            assert float((x - y).norm()) <= 1e-4 * float(y.norm())      # (sums over rows meet in any order)
