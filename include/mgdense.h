@@ -432,9 +432,10 @@ int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, f
 
 /* The same in two calls, so that the caller's host work runs beside the pass: mg_backward_begin queues it (arguments and errors of
  * mg_backward), with ids_dev (DEVICE, nullable) also what mg_dense_packed_ids writes, and with grads_dev (DEVICE, nullable) a copy of
- * the whole block of gradients (mg_model_grads) on `grads_stream`, behind the pass.  mg_backward_end waits for the pass -- for the
- * copy only as far as grads_stream's own order goes -- and returns its status.  Every successful begin wants its end before the next
- * call on the context. */
+ * the whole block of gradients (mg_model_grads) on `grads_stream`, behind the pass.  The pass then also comes behind what is queued on
+ * `grads_stream`, so that d_out_dev may come from there and d_h0_dev, ids_dev may be memory that it still uses.  mg_backward_end waits
+ * for the pass -- for the copy only as far as grads_stream's own order goes -- and returns its status.  Every successful begin wants its
+ * end before the next call on the context. */
 int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, float* d_h0_dev, int32_t* ids_dev, float* grads_dev,
                       void* grads_stream);
 int mg_backward_end(mg_ctx* ctx);

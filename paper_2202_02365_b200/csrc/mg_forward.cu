@@ -1237,6 +1237,10 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
     const int k = d->k, B = d->n_batches;
     cudaStream_t st = ctx->stream;
+    if (grads_dev && (cudaStream_t)grads_stream != st) {   // the caller's buffers are as its stream leaves them
+        MG_CUDA(ctx, cudaEventRecord(ctx->ev_user, (cudaStream_t)grads_stream));
+        MG_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_user));
+    }
     // gradient block of the model (allocated once), cleared for this pass
     if (!m->g_block) {
         m->g_elems = 0;

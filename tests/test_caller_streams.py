@@ -107,3 +107,24 @@ def test_gradients_of_two_passes_copied_on_a_late_stream(graph):
     for g, w in zip(got, want):
         for x, y in zip((t for layer in g for t in layer), (t for layer in w for t in layer)):
             assert float((x - y).norm()) <= 1e-4 * float(y.norm())      # (sums over rows meet in any order)
+
+
+def test_gradient_rows_in_memory_that_the_callers_stream_still_reads(graph):
+    ctx, model, dense, d_out = training(graph, torch.cuda.Stream())
+    rows = int(dense.counts()[0].sum())
+    ctx.backward(model, dense, d_out[0], want_h0_grad=True)
+    torch.cuda.synchronize()
+    user = torch.cuda.Stream()
+    with torch.cuda.stream(user):
+        before = torch.full((rows, 32), 5.0, device="cuda")
+        user.synchronize()
+        at = before.data_ptr()
+        (before * 1.0).sum()                         # (a kernel's first launch loads it, and waits)
+        user.synchronize()
+        torch.cuda._sleep(LATE)
+        read = before * 1.0
+        del before                                   # (the stream's own next allocation may take its place: it comes behind the read)
+        _, g_rows, _ = ctx.backward(model, dense, d_out[0], want_h0_grad=True)
+    torch.cuda.synchronize()
+    assert g_rows.data_ptr() == at
+    assert torch.equal(read, torch.full_like(read, 5.0))
