@@ -264,7 +264,7 @@ int mg_dense_export_copy(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_array
 /* Copy the five arrays of a mini-batch, as mg_dense_view or mg_dense_export_view handed them out, to one DEVICE buffer of the
  * caller's: node_ids (n_nodes), node_id_offsets (k + 2), nbrs (n_entries), nbr_offsets (n_sampled + 1), repr_map (n_entries),
  * one behind the other.  One kernel on `stream` (a cudaStream_t of the context's device; NULL = the default stream), not waited
- * for. */
+ * for; a later mg_dense_view or export is ordered behind it. */
 int mg_dense_arrays_copy(mg_ctx* ctx, const mg_dense_arrays* arrays, int32_t* dst_dev, void* stream);
 
 int mg_dense_free(mg_dense* d);

@@ -362,6 +362,7 @@ extern "C" int mg_destroy(mg_ctx* c) {
     cudaFree(c->ws_x); cudaFree(c->ws_meta); cudaFree(c->ws_h[0]); cudaFree(c->ws_h[1]);
     cudaEventDestroy(c->ev_fwd_done); cudaEventDestroy(c->ev_out_done); cudaEventDestroy(c->ev_user);
     if (c->ev_backward) cudaEventDestroy(c->ev_backward);
+    mg_reads_free(&c->array_reads);
     for (int i = 0; i < 2; ++i) { if (c->ev_hk_done[i]) cudaEventDestroy(c->ev_hk_done[i]); cudaFree(c->hk_buf[i]); }
     cudaFree(c->lp_ws); cudaFree(c->dm_images);
     for (auto& s : c->lp_spare) { cudaFree(s.block); if (s.idle) cudaEventDestroy(s.idle); mg_reads_free(&s.reads); }

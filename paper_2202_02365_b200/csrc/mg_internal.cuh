@@ -154,6 +154,8 @@ struct mg_ctx {
     int hk_cur = 0;
     const float* last_hk = nullptr;
 
+    QueuedReads array_reads;   // copies of mini-batches' arrays that mg_dense_arrays_copy queued on a caller's stream
+
     // profiling
     // link-prediction batches: scratch of mg_lp_prepare (grows, never shrinks) and one spare result block, so that a
     // loop of prepare / free allocates nothing
@@ -241,8 +243,7 @@ struct mg_dense {
     // export of all mini-batches at once (mg_dense_export_many): one buffer, laid out by export_layout()
     int32_t* expm_buf = nullptr; size_t expm_elems = 0;
     cudaEvent_t ev_exported = nullptr;
-    cudaEvent_t ev_copied = nullptr;     // the last copy out of the export buffer that was queued on a caller's stream
-    bool copies_queued = false;
+    QueuedReads expm_reads;              // copies out of the export buffer that were queued on a caller's stream (mg_dense_export_copy)
     bool export_valid = false, export_pending = false;
     int32_t* perm_buf = nullptr; size_t perm_elems = 0;   // perm | inv of mini-batch perm_batch (mg_dense_batch_perm)
     int perm_batch = -1;

@@ -2059,6 +2059,7 @@ extern "C" int mg_dense_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_a
     a.o_nbrs = a.o_nio + (k + 2);
     a.o_nbr_off = a.o_nbrs + n_entries;
     a.o_repr = a.o_nbr_off + n_s + 1;
+    MG_CUDA(ctx, mg_reads_wait(&ctx->array_reads, ctx->stream));   // (the last call's arrays may still be read)
     const int grid = std::max(1, std::min(mg_grid(ctx, 4), (a.g.V + kThreads - 1) / kThreads));
     k_export_nodes<<<grid, kThreads, 0, ctx->stream>>>(a);
     k_export_scan<<<1, 1024, 0, ctx->stream>>>(a.o_nbr_off, n_s);
@@ -2127,7 +2128,9 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
     a.o_repr = d->expm_buf + L.repr; a.o_nbr_off = d->expm_buf + L.nbr_off; a.inv = d->expm_buf + L.inv;
     a.cnt = reinterpret_cast<uint32_t*>(d->expm_buf + L.cnt);
     d->export_valid = false;
-    if (d->copies_queued) { MG_CUDA(ctx, cudaStreamWaitEvent(st, d->ev_copied)); d->copies_queued = false; }   // they read the buffer
+    MG_CUDA(ctx, mg_reads_wait(&d->expm_reads, st));   // (the last export's arrays may still be read)
+    MG_CUDA(ctx, mg_reads_wait(&ctx->array_reads, st));
+    d->expm_reads.queued = false;
     if (n_total > 0) {
         SortParams* sp = (SortParams*)(d->scan_tmp + d->scan_tmp_elems - 8);
         int32_t* range = d->scan_tmp + d->scan_tmp_elems - 12;
@@ -2189,18 +2192,26 @@ extern "C" int mg_dense_export_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_
     return MG_OK;
 }
 
+static int copy_arrays(mg_ctx* ctx, const mg_dense_arrays* v, int32_t* dst_dev, cudaStream_t st) {
+    const ArraysCopy a{{v->node_ids, v->node_id_offsets, v->nbrs, v->nbr_offsets, v->repr_map},
+                       {v->n_nodes, v->k + 2, v->n_entries, v->n_sampled + 1, v->n_entries}};
+    const int longest = std::max(std::max(v->n_nodes, v->n_entries), v->n_sampled + 1);
+    const int blocks = std::max(1, std::min(mg_grid(ctx, 2), (longest + 4 * kThreads - 1) / (4 * kThreads)));
+    k_copy_arrays<<<dim3((unsigned)blocks, 5), kThreads, 0, st>>>(a, dst_dev);
+    ctx->launches++;
+    MG_CUDA(ctx, cudaGetLastError());
+    return MG_OK;
+}
+
 extern "C" int mg_dense_export_copy(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out, int32_t* dst_dev, void* stream) {
     if (!ctx) return MG_ERR_ARG;
     if (int rc = exported_arrays(ctx, d, batch, out)) return rc;
     if (!dst_dev) return MG_OK;
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
     cudaStream_t st = (cudaStream_t)stream;
-    if (!d->ev_copied) MG_CUDA(ctx, cudaEventCreateWithFlags(&d->ev_copied, cudaEventDisableTiming));
     if (d->export_pending) MG_CUDA(ctx, cudaStreamWaitEvent(st, d->ev_exported));
-    if (d->copies_queued) MG_CUDA(ctx, cudaStreamWaitEvent(st, d->ev_copied));   // (from another stream: one event stands for all copies)
-    if (int rc = mg_dense_arrays_copy(ctx, out, dst_dev, stream)) return rc;
-    MG_CUDA(ctx, cudaEventRecord(d->ev_copied, st));
-    d->copies_queued = true;
+    if (int rc = copy_arrays(ctx, out, dst_dev, st)) return rc;
+    MG_CUDA(ctx, mg_reads_add(&d->expm_reads, st));
     return MG_OK;
 }
 
@@ -2208,13 +2219,8 @@ extern "C" int mg_dense_arrays_copy(mg_ctx* ctx, const mg_dense_arrays* v, int32
     if (!ctx) return MG_ERR_ARG;
     if (!v || !dst_dev) return mg_fail(ctx, MG_ERR_ARG, "null argument");
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
-    const ArraysCopy a{{v->node_ids, v->node_id_offsets, v->nbrs, v->nbr_offsets, v->repr_map},
-                       {v->n_nodes, v->k + 2, v->n_entries, v->n_sampled + 1, v->n_entries}};
-    const int longest = std::max(std::max(v->n_nodes, v->n_entries), v->n_sampled + 1);
-    const int blocks = std::max(1, std::min(mg_grid(ctx, 2), (longest + 4 * kThreads - 1) / (4 * kThreads)));
-    k_copy_arrays<<<dim3((unsigned)blocks, 5), kThreads, 0, (cudaStream_t)stream>>>(a, dst_dev);
-    ctx->launches++;
-    MG_CUDA(ctx, cudaGetLastError());
+    if (int rc = copy_arrays(ctx, v, dst_dev, (cudaStream_t)stream)) return rc;
+    MG_CUDA(ctx, mg_reads_add(&ctx->array_reads, (cudaStream_t)stream));
     return MG_OK;
 }
 
@@ -2228,7 +2234,7 @@ extern "C" int mg_dense_free(mg_dense* d) {
     cudaFree(d->newlist[1]); cudaFree(d->d_seeds); cudaFree(d->batch_cnt); cudaFree(d->scan_tmp); cudaFree(d->sort_hist); cudaFree(d->seg_tiles);
     cudaFree(d->exp_buf); cudaFree(d->perm_buf); cudaFree(d->d_ent_hop); cudaFree(d->expm_buf);
     if (d->ev_exported) cudaEventDestroy(d->ev_exported);
-    if (d->ev_copied) cudaEventDestroy(d->ev_copied);
+    mg_reads_free(&d->expm_reads);
     if (d->h_stage) cudaFreeHost(d->h_stage);
     if (d->graph_exec) cudaGraphExecDestroy(d->graph_exec);
     if (d->ev_sampled) cudaEventDestroy(d->ev_sampled);

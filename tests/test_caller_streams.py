@@ -128,3 +128,27 @@ def test_gradient_rows_in_memory_that_the_callers_stream_still_reads(graph):
     torch.cuda.synchronize()
     assert g_rows.data_ptr() == at
     assert torch.equal(read, torch.full_like(read, 5.0))
+
+
+@pytest.mark.parametrize("export", [False, True])
+def test_views_copied_on_a_late_stream(graph, export):
+    ctx = context(graph)
+    offs = np.array([0, 200, 500, 650])
+    samples = [ctx.sample_many(torch.cat([inputs.distinct_targets(N, n, seed=s + i) for i, n in enumerate(np.diff(offs))]), offs, [4, 3], [1, 2, 3])
+               for s in (11, 21)]
+    want = [[arrays(d.view(b)) for b in range(3)] for d in samples]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        torch.cuda._sleep(LATE)
+        if export:
+            got = []
+            for d in samples:
+                d.export_many()
+                got.append([d.export_view(b) for b in range(3)])
+                d.export_many()      # (the same arrays, into the buffer that is still to be read)
+        else:
+            got = [[d.view(b) for b in range(3)] for d in samples]
+    torch.cuda.synchronize()
+    for g, w in zip(got, want):
+        for x, y in zip(g, w):
+            assert all(torch.equal(p, q) for p, q in zip(arrays(x), y))
