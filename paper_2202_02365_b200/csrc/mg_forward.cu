@@ -930,12 +930,15 @@ struct RevArgs {
     uint32_t* n_units;                 // [k + 1]
     float* g_in[MG_MAX_HOPS + 1];      // the layer's source rows' gradients; rows of several units are cleared here
     int32_t d_in[MG_MAX_HOPS + 1];
-    uint32_t* status;
+    int32_t polls;                     // reads of a tile's state before the scan gives up
+    uint32_t* bad;                     // set when it has: the lists are then wrong, and the kernels behind it leave them alone
+    uint32_t* status;                  // the host's word
 };
 
 // 8 lanes per output row
 template <bool FILL>
 __global__ void __launch_bounds__(kThreads) k_rev_entries(RevArgs a) {
+    if (FILL && *a.bad) return;
     const int gl = threadIdx.x & 7;
     for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3; i < a.out_at[a.g.k + 1]; i += ((int64_t)gridDim.x * blockDim.x) >> 3) {
         int layer = a.l0;
@@ -956,7 +959,7 @@ __global__ void __launch_bounds__(kThreads) k_rev_entries(RevArgs a) {
 
 // exclusive scan of the counts in place, the total behind them; the rows with long lists are cut into units on the way.
 // Tiles come from a counter, so a tile's predecessors are held by running blocks; the polls are bounded all the same.
-constexpr int kRevTile = kThreads * 16, kRevPolls = 1 << 20;
+constexpr int kRevTile = kThreads * 16, kRevPolls = 1 << 20;   // (a poll is an L2 round trip: far beyond any legitimate wait)
 __global__ void __launch_bounds__(kThreads) k_rev_scan(RevArgs a) {
     __shared__ uint32_t part[kThreads / 32];
     __shared__ uint32_t sh_before;
@@ -998,8 +1001,8 @@ __global__ void __launch_bounds__(kThreads) k_rev_scan(RevArgs a) {
             uint64_t st = kSum;   // (before tile 0: nothing)
             if (at >= 0) {
                 int polls = 0;
-                while ((st = state[at]) == 0 && ++polls < kRevPolls) {}
-                if (polls >= kRevPolls) { *reinterpret_cast<volatile uint32_t*>(a.status) = 31u; st = kTotal; }
+                while ((st = state[at]) == 0 && ++polls < a.polls) {}
+                if (polls >= a.polls) { *a.bad = 1u; *reinterpret_cast<volatile uint32_t*>(a.status) = MG_ROLE_REV_SCAN; st = kTotal; }
             }
             const uint32_t full = __ballot_sync(0xFFFFFFFFu, (st & kTotal) != 0);
             const int stop = full ? __ffs(full) - 1 : 31;
@@ -1055,6 +1058,7 @@ struct GatherArgs {
     const int2* rev;
     const int2* units;
     const uint32_t* n_units;
+    const uint32_t* bad;       // the scan gave up: there are no lists
     const float* dx;           // [rows of layer, 2 d_in]
     int32_t d_in;
     const float* y;            // [rows_in, d_in] kept outputs of layer - 1 (MASK), else null
@@ -1080,6 +1084,7 @@ __global__ void __launch_bounds__(kThreads, MASK ? 4 : 1) k_grad_gather(GatherAr
     __shared__ int32_t rows_sm[kWarps][kGradRows];
     __shared__ float sums[MASK ? 1024 : 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (*a.bad) return;
     int2* items = items_sm[warp];
     int32_t* rows = rows_sm[warp];
     const int n4 = a.d_in / 4;
@@ -1289,7 +1294,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     if (ctx->bw_g_elems < g_total && (rc = mg_ensure(ctx, &ctx->bw_g, &ctx->bw_g_elems, g_total + g_total / 4 + 16))) return rc;
     if (ctx->bw_x_elems < (size_t)max_x && (rc = mg_ensure(ctx, &ctx->bw_x, &ctx->bw_x_elems, (size_t)max_x + 16))) return rc;
     if (ctx->bw_dx_elems < (size_t)max_dx && (rc = mg_ensure(ctx, &ctx->bw_dx, &ctx->bw_dx_elems, (size_t)max_dx + 16))) return rc;
-    // cleared by one memset: the scan's ticket, the unit counts, its states, the counts; then the entries' places
+    // cleared by one memset: the scan's ticket, the unit counts, whether it gave up, its states, the counts; then the entries' places
     const size_t cnt_at = ((MG_MAX_HOPS + 4) + 2 * (size_t)rev_tiles + 3) / 4 * 4;
     const size_t cleared = cnt_at + (size_t)in_total + 1;
     const size_t need_off = cleared + (size_t)ent_total;
@@ -1310,6 +1315,9 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         ra.pos = ra.cnt + in_total + 1;
         ra.rev = ctx->bw_rev;
         ra.units = ctx->bw_rev + ent_total;
+        ra.bad = ra.n_units + MG_MAX_HOPS + 1;
+        const char* polls = getenv("MG_REV_POLLS");
+        ra.polls = polls ? atoi(polls) : kRevPolls;
         ra.status = ctx->d_flags;
         for (int l = ra.l0; l <= k; ++l) { ra.g_in[l] = l > 1 ? ctx->bw_g + g_off[l - 1] : d_h0_dev; ra.d_in[l] = m->dims[l - 1]; }
         MG_CUDA(ctx, cudaMemsetAsync(ctx->bw_off, 0, sizeof(uint32_t) * cleared, st));
@@ -1372,7 +1380,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         const int64_t rows_in = d->h_hdr.rows_total[l - 1];
         if (!g_in || rows_in == 0) continue;
         // dX -> the gradient of the layer's input rows
-        GatherArgs ga{geom, l, rows_in, ra.cnt + ra.in_at[l], ra.rev, ra.units + ra.unit_at[l], ra.n_units + l, ctx->bw_dx, d_in,
+        GatherArgs ga{geom, l, rows_in, ra.cnt + ra.in_at[l], ra.rev, ra.units + ra.unit_at[l], ra.n_units + l, ra.bad, ctx->bw_dx, d_in,
                       l > 1 ? ctx->ws_h[0] + h_off[l - 1] : nullptr, g_in, l > 1 ? m->g_bias[l - 2] : nullptr};
         // (groups of 16 rows, a warp per 128 columns; the units come on top, the loop takes what does not fit the grid)
         const int64_t warps = (rows_in + kGradRows - 1) / kGradRows * std::max(1, (d_in + 127) / 128);

@@ -147,10 +147,11 @@ int mg_gemm_tf32(mg_ctx* ctx, const float* x, const float* w_t, const float* bia
     return MG_OK;
 }
 
-// After the stream has drained: MG_ERR_TIMEOUT if a GEMM gave up on a barrier (the word is cleared).
+// After the stream has drained: MG_ERR_TIMEOUT if a kernel gave up waiting (the word is cleared).
 int mg_gemm_tf32_status(mg_ctx* ctx) {
     const uint32_t flag = *static_cast<volatile uint32_t*>(ctx->h_flags);
     if (!flag) return MG_OK;
     *ctx->h_flags = 0;
+    if (flag == MG_ROLE_REV_SCAN) return mg_fail(ctx, MG_ERR_TIMEOUT, "the scan of the backward pass's entry lists gave up waiting");
     return mg_fail(ctx, MG_ERR_TIMEOUT, "tensor-core GEMM gave up waiting on a barrier (role %u)", flag);
 }

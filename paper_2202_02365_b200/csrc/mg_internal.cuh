@@ -25,6 +25,9 @@ enum : uint32_t {
     ST_INTERNAL = 64u,     // an invariant did not hold (bug guard; access skipped)
 };
 
+// what a kernel leaves in mg_ctx::d_flags besides the roles of the tensor-core kernels
+constexpr uint32_t MG_ROLE_REV_SCAN = 31u;   // the scan of the backward pass's turned-round entries
+
 // Device-side header of a sample: counters every kernel sizes itself from.
 struct DenseHeader {
     uint32_t status;

@@ -147,3 +147,27 @@ def test_sample_between_forward_and_backward_is_refused(precision, fails):
     if not fails:
         ctx.forward(model, dense, out)
         ctx.backward(model, dense, torch.ones_like(out))
+
+
+# a wait of the scan that cuts the entry lists runs out (here at once): an error, and a context that goes on working
+@pytest.mark.parametrize("precision", [mg.GEMM_TF32, mg.GEMM_FP32])
+def test_scan_that_gives_up_ends_in_an_error(monkeypatch, precision):
+    graph = star_graph()
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(inputs.normal_features(N, 16, seed=4).cuda())
+    ctx.keep_layer_outputs(True)
+    model = ctx.model(inputs.random_bias_layers([16, 12, 8], seed=5), precision)
+    dense = ctx.sample(inputs.distinct_targets(N, 5_000, seed=6), [6, 4], 7)      # (more source rows than a tile of the scan has, 4,096)
+    out = torch.empty((5_000, 8), device="cuda")
+    ctx.forward(model, dense, out)
+    d_out = torch.randn(out.shape, generator=torch.Generator("cuda").manual_seed(8), device="cuda")
+    want, want_rows, _ = ctx.backward(model, dense, d_out, want_h0_grad=True)
+    monkeypatch.setenv("MG_REV_POLLS", "0")
+    with pytest.raises(mg.MgError, match="entry lists") as e:
+        ctx.backward(model, dense, d_out, want_h0_grad=True)
+    assert e.value.code == -7                                                     # MG_ERR_TIMEOUT
+    monkeypatch.delenv("MG_REV_POLLS")
+    got, got_rows, _ = ctx.backward(model, dense, d_out, want_h0_grad=True)
+    for x, y in zip([t for layer in got for t in layer] + [got_rows], [t for layer in want for t in layer] + [want_rows]):
+        assert float((x - y).norm()) <= 1e-5 * float(y.norm())                    # (sums over rows meet in any order)
