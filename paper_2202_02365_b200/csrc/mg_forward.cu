@@ -538,15 +538,10 @@ static int finish_forward(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* ou
     return MG_OK;
 }
 
-static int forward_impl(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out, int out_mode) {
-    if (!ctx) return MG_ERR_ARG;
-    int rc = forward_checks(ctx, m, d);
-    if (rc) return rc;
-    if (!out) return mg_fail(ctx, MG_ERR_ARG, "null output");
-    MG_CUDA(ctx, cudaSetDevice(ctx->device));
+static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out, int out_mode) {
+    int rc;
     const int k = d->k, B = d->n_batches;
     cudaStream_t st = ctx->stream;
-    ctx->last_fwd_model = m; ctx->last_fwd_dense = d;
     // H^k of this pass goes to the buffer the pass before last used; an output copy of that pass to the host (side
     // stream) may still read it.  The copy of the previous pass reads the other buffer and is not waited for.
     float* hk = nullptr;
@@ -715,6 +710,19 @@ static int forward_impl(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
     }
     MG_CUDA(ctx, cudaGetLastError());
     return finish_forward(ctx, m, d, out, out_mode, hk, out2 != nullptr);
+}
+
+static int forward_impl(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out, int out_mode) {
+    if (!ctx) return MG_ERR_ARG;
+    if (int rc = forward_checks(ctx, m, d)) return rc;
+    if (!out) return mg_fail(ctx, MG_ERR_ARG, "null output");
+    MG_CUDA(ctx, cudaSetDevice(ctx->device));
+    // a pass that ends in an error leaves neither layer outputs nor anything that mg_backward may follow
+    ctx->last_fwd_model = nullptr; ctx->last_fwd_dense = nullptr; ctx->last_hk = nullptr;
+    const int rc = forward_pass(ctx, m, d, out, out_mode);
+    if (rc) { ctx->last_hk = nullptr; return rc; }
+    ctx->last_fwd_model = m; ctx->last_fwd_dense = d;
+    return MG_OK;
 }
 
 extern "C" int mg_forward(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out, int out_on_device) {

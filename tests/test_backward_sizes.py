@@ -171,3 +171,40 @@ def test_scan_that_gives_up_ends_in_an_error(monkeypatch, precision):
     got, got_rows, _ = ctx.backward(model, dense, d_out, want_h0_grad=True)
     for x, y in zip([t for layer in got for t in layer] + [got_rows], [t for layer in want for t in layer] + [want_rows]):
         assert float((x - y).norm()) <= 1e-5 * float(y.norm())                    # (sums over rows meet in any order)
+
+
+# no memory for the pass's rows: it frees smaller buffers before it fails, and what it leaves is not to be gone back through
+def test_backward_after_a_failed_forward_is_refused():
+    graph = star_graph()
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(inputs.normal_features(N, 16, seed=4).cuda())
+    ctx.keep_layer_outputs(True)
+    model = ctx.model(inputs.random_bias_layers([16, 1024], seed=5))
+    few, many = (ctx.sample(inputs.distinct_targets(N, n, seed=6), [6], 7) for n in (40, 5_990))
+    out = torch.empty((5_990, 1024), device="cuda")
+    d_out = torch.ones_like(out)
+    ctx.forward(model, few, out)
+    ctx.backward(model, few, d_out)
+    held = []
+    try:
+        for size in (torch.cuda.mem_get_info()[0] - (64 << 20), 8 << 20, 2 << 20):
+            try:
+                while True:
+                    held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            except torch.OutOfMemoryError:
+                pass
+        with pytest.raises(mg.MgError) as e:
+            ctx.forward(model, many, out)                    # (24 MB of rows)
+        assert e.value.code == -6                            # MG_ERR_OOM
+    finally:
+        held.clear()
+        torch.cuda.empty_cache()
+    for dense in (few, many):
+        with pytest.raises(mg.MgError) as e:
+            ctx.backward(model, dense, d_out)
+        assert e.value.code == -2                            # MG_ERR_STATE
+        with pytest.raises(mg.MgError):
+            ctx.layer_output(model, dense, 1, 0, 40)
+    ctx.forward(model, many, out)
+    ctx.backward(model, many, d_out)
