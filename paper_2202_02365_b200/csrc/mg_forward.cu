@@ -1312,7 +1312,8 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     const RowGeom geom{B, k, d->rowbase, d->cum, d->node_off};
     const bool half = ctx->feat_dtype == MG_DTYPE_F16;
     const int grid = mg_grid(ctx, 8);
-    if (in_total > 0 && ra.out_at[k + 1] > 0) {
+    // (behind the last layer's products: the scan clears rows of the inputs' gradients, and d_h0_dev may lie where d_out_dev does)
+    auto turn_entries_round = [&]() -> int {
         ra.g = geom;
         ra.ent_off = d->ent_off; ra.ent_repr = d->ent_repr; ra.sum_aggr = m->sum_aggr ? 1 : 0;
         ra.ticket = ctx->bw_off;
@@ -1334,7 +1335,9 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         k_rev_scan<<<(unsigned)rev_tiles, kThreads, 0, st>>>(ra);
         k_rev_entries<true><<<rgrid, kThreads, 0, st>>>(ra);
         ctx->launches += 3;
-    }
+        return MG_OK;
+    };
+    bool turned = false;
     for (int l = k; l >= 1; --l) {
         const int d_in = m->dims[l - 1], d_out = m->dims[l];
         const int64_t M = d->h_hdr.rows_total[l];
@@ -1387,6 +1390,8 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         }
         const int64_t rows_in = d->h_hdr.rows_total[l - 1];
         if (!g_in || rows_in == 0) continue;
+        if (!turned && (rc = turn_entries_round())) return rc;
+        turned = true;
         // dX -> the gradient of the layer's input rows
         GatherArgs ga{geom, l, rows_in, ra.cnt + ra.in_at[l], ra.rev, ra.units + ra.unit_at[l], ra.n_units + l, ra.bad, ctx->bw_dx, d_in,
                       l > 1 ? ctx->ws_h[0] + h_off[l - 1] : nullptr, g_in, l > 1 ? m->g_bias[l - 2] : nullptr};

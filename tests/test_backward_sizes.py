@@ -1,11 +1,13 @@
 """The backward pass at the sizes where its gather is cut differently: source rows named by none, a few, tens and hundreds of
 entries (a star graph's centre), widths of one to eight column blocks; against the layers' definition in fp64."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
 import paper_2202_02365_b200 as mg
-from paper_2202_02365_b200 import inputs
+from paper_2202_02365_b200 import api, inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -208,3 +210,31 @@ def test_backward_after_a_failed_forward_is_refused():
             ctx.layer_output(model, dense, 1, 0, 40)
     ctx.forward(model, many, out)
     ctx.backward(model, many, d_out)
+
+
+# the rows' gradients may go where the loss's gradient lies: it is read before any of them is written (rows named by hundreds of entries
+# are cleared before they are added up)
+@pytest.mark.parametrize("precision", [mg.GEMM_TF32, mg.GEMM_FP32])
+@pytest.mark.parametrize("dims", [[16, 16], [16, 12, 16]])
+def test_row_gradients_over_the_output_gradient(precision, dims):
+    graph = star_graph()
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(inputs.normal_features(N, dims[0], seed=4).cuda())
+    ctx.keep_layer_outputs(True)
+    model = ctx.model(inputs.random_bias_layers(dims, seed=5), precision)
+    dense = ctx.sample(inputs.distinct_targets(N, 4_000, seed=6), [6] * (len(dims) - 1), 7)
+    out = torch.empty((4_000, dims[-1]), device="cuda")
+    ctx.forward(model, dense, out)
+    d_out = torch.randn(out.shape, generator=torch.Generator("cuda").manual_seed(8), device="cuda")
+    want, want_rows, _ = ctx.backward(model, dense, d_out, want_h0_grad=True)
+    both = torch.zeros(want_rows.numel(), device="cuda")
+    both[:d_out.numel()] = d_out.flatten()
+    at = ctypes.c_void_p(both.data_ptr())
+    torch.cuda.synchronize()
+    ctx._check(ctx.lib.mg_backward(ctx.handle, model.handle, dense.handle, at, at))
+    w_self = ctypes.c_void_p(0)
+    ctx._check(ctx.lib.mg_model_grads(model.handle, 1, ctypes.byref(w_self), None, None))
+    got = torch.as_tensor(api._DeviceInts(w_self.value, want[0][0].numel()), device="cuda").view(torch.float32)
+    for x, y in ((got, want[0][0].flatten()), (both, want_rows.flatten())):
+        assert float((x - y).norm()) <= 1e-5 * float(y.norm())                    # (sums over rows meet in any order)
