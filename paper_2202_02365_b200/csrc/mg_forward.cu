@@ -577,9 +577,12 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
     }
     // H^k stays in the library's buffer (mg_layer_output, mg_backward) and goes to the caller's: the last layer's kernel
     // stores its tiles to both when it can (the copy behind it read and wrote the rows once more: 41 us for 128,000 rows of
-    // 1 KB, and a launch)
-    float* out2 = out_mode == OUT_DEVICE && any_fused && mg_layer_fused_supported(m->dims[k - 1], m->dims[k]) &&
-                  (reinterpret_cast<uintptr_t>(out) & 15) == 0 ? out : nullptr;
+    // 1 KB, and a launch).  Not into the feature table, which other tiles still read.
+    const uintptr_t out_at = reinterpret_cast<uintptr_t>(out), table_at = reinterpret_cast<uintptr_t>(ctx->slots);
+    const size_t out_bytes = (size_t)d->h_hdr.rows_total[k] * m->dims[k] * sizeof(float);
+    const size_t table_bytes = ctx->backing == MG_BACKING_HBM ? (size_t)ctx->n_nodes * ctx->row_bytes : (size_t)ctx->n_slots * ctx->slot_bytes;
+    const bool in_table = out_at < table_at + table_bytes && table_at < out_at + out_bytes;
+    float* out2 = out_mode == OUT_DEVICE && any_fused && mg_layer_fused_supported(m->dims[k - 1], m->dims[k]) && out_at % 16 == 0 && !in_table ? out : nullptr;
     const int sub = ctx->layer_window_batches;
     ctx->layers_kept = !(all_fused && sub > 0 && !ctx->keep_layers && k > 1);
     if (!ctx->layers_kept) {

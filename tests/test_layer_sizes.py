@@ -46,3 +46,23 @@ def test_rows_on_either_side_of_the_tile_sizes(graph, rows, d_in, d_out, half, f
     rms = want.square().mean().sqrt()
     assert float(err.square().mean().sqrt() / rms) < 1e-3 and float((err / torch.maximum(want.abs(), rms)).max()) < 6e-3
     assert torch.equal(out[rows], torch.full_like(out[rows], 7.0))
+
+
+# the rows may go into the table that they are made from: it is read before any of them is there, also where the layers run over a few
+# mini-batches at a time
+@pytest.mark.parametrize("hops,window", [(1, 0), (2, 0), (2, 1)])
+def test_rows_written_over_the_table(graph, hops, window):
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    table = inputs.normal_features(N, 128, seed=5, device="cuda")
+    ctx.load_features(table)
+    ctx.set_layer_window(window)
+    per, count = 9_000, 4
+    targets = torch.cat([inputs.distinct_targets(N, per, seed=b) for b in range(count)])
+    dense = ctx.sample_many(targets, [per * b for b in range(count + 1)], [5, 4][:hops], [1, 2, 3, 4])
+    model = ctx.model(inputs.random_bias_layers([128] * (hops + 1), seed=6))
+    want = torch.empty((per * count, 128), device="cuda")
+    ctx.forward(model, dense, want)
+    got = table[1_000:1_000 + per * count]
+    ctx.forward(model, dense, got)
+    assert torch.equal(got, want)
