@@ -267,6 +267,12 @@ int mg_dense_export_copy(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_array
  * for; a later mg_dense_view or export is ordered behind it. */
 int mg_dense_arrays_copy(mg_ctx* ctx, const mg_dense_arrays* arrays, int32_t* dst_dev, void* stream);
 
+/* The same two copies with every array at the next multiple of `align` elements (a power of two up to 1024) of dst_dev, which must have
+ * room for the lengths rounded up to it: 4 makes 16-byte loads of every array possible, 128 starts each as an allocation would. */
+int mg_dense_export_copy_aligned(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out, int32_t* dst_dev, int32_t align,
+                                 void* stream);
+int mg_dense_arrays_copy_aligned(mg_ctx* ctx, const mg_dense_arrays* arrays, int32_t* dst_dev, int32_t align, void* stream);
+
 int mg_dense_free(mg_dense* d);
 
 /* ---- GraphSage forward over DENSE (Section 4.2, Algorithms 2 and 3) -------------------- */

@@ -29,7 +29,7 @@ CORRUPT_DST, CORRUPT_SRC, CORRUPT_BOTH = 1, 2, 3
 EXPORTS = [
     "mg_create", "mg_destroy", "mg_last_error", "mg_load_graph", "mg_load_out_graph", "mg_set_sample_direction", "mg_set_partitioning",
     "mg_load_features", "mg_set_partition_source", "mg_set_resident", "mg_commit_resident", "mg_sample_many", "mg_sample_many_begin", "mg_sample_many_end", "mg_sample",
-    "mg_dense_counts", "mg_dense_view", "mg_dense_export_many", "mg_dense_export_view", "mg_dense_export_copy", "mg_dense_arrays_copy", "mg_dense_free", "mg_model_create", "mg_model_set_aggregator", "mg_model_set_intermediates", "mg_model_free",
+    "mg_dense_counts", "mg_dense_view", "mg_dense_export_many", "mg_dense_export_view", "mg_dense_export_copy", "mg_dense_arrays_copy", "mg_dense_export_copy_aligned", "mg_dense_arrays_copy_aligned", "mg_dense_free", "mg_model_create", "mg_model_set_aggregator", "mg_model_set_intermediates", "mg_model_free",
     "mg_forward", "mg_set_layer_window", "mg_keep_layer_outputs", "mg_forward_host_async", "mg_wait_output", "mg_forward_noalloc", "mg_gather_h0", "mg_layer_output", "mg_lp_prepare", "mg_lp_view", "mg_lp_targets", "mg_lp_record_stream", "mg_lp_free",
     "mg_distmult_score", "mg_kernel_launches", "mg_profile", "mg_profile_read", "mg_comet_plan", "mg_comet_bias", "mg_comet_autotune", "mg_gat_model_create", "mg_gat_model_set_heads", "mg_gat_model_free", "mg_gat_forward", "mg_backward", "mg_backward_begin", "mg_backward_end", "mg_model_grads", "mg_model_sgd_step", "mg_model_adagrad_step", "mg_dense_packed_ids", "mg_apply_embedding_sgd",
 ]
@@ -77,9 +77,20 @@ def _raw_stream(device: torch.device):
     return C.c_void_p(torch._C._cuda_getCurrentRawStream(device.index))
 
 
-def _sizes(arr: "DenseArrays"):
-    """Lengths of the arrays as DenseView and mg_dense_arrays_copy list them."""
-    return arr.n_nodes, arr.k + 2, arr.n_entries, arr.n_sampled + 1, arr.n_entries
+_ALIGN = 128     # elements: the arrays of a view start 512 bytes apart, as allocations of their own would
+
+
+def _room(arr: "DenseArrays"):
+    """Lengths of the arrays as DenseView lists them and mg_dense_arrays_copy_aligned places them, each with what is left to the next."""
+    n, o, e, s = arr.n_nodes, arr.k + 2, arr.n_entries, arr.n_sampled + 1
+    left = -e % _ALIGN
+    return n, -n % _ALIGN, o, -o % _ALIGN, e, left, s, -s % _ALIGN, e, left
+
+
+def _pieces(block: torch.Tensor, sizes):
+    """Consecutive pieces of a block of memory, each with an autograd life of its own: what is done to one in place is no change of the
+    others (the "unsafe" form of the split is the one whose pieces are no views of the block, and the cheapest)."""
+    return torch.unsafe_split_with_sizes(block, sizes)
 
 
 def _fanouts(fanouts):
@@ -147,7 +158,8 @@ def _from_dev(ptr, n: int, device) -> torch.Tensor:
 
 @dataclass
 class DenseView:
-    """One batch's DENSE in the paper's layout (device int32 tensors)."""
+    """One batch's DENSE in the paper's layout (device int32 tensors).  The five lie in one allocation, 512-byte aligned: keeping one
+    keeps the memory of all."""
     node_ids: torch.Tensor
     node_id_offsets: torch.Tensor
     nbrs: torch.Tensor
@@ -178,12 +190,12 @@ class Dense:
     def _copied(self, arr: DenseArrays) -> DenseView:
         """The arrays in memory of the caller's own: one allocation and one kernel (a tensor made from every pointer and cloned
         took 65 us of host time per mini-batch)."""
-        sizes = _sizes(arr)
+        room = _room(arr)
         dev = self.ctx.device
-        out = torch.empty(sum(sizes), dtype=torch.int32, device=dev)
-        self.ctx._check(self.ctx.lib.mg_dense_arrays_copy(self.ctx.handle, C.byref(arr), _ptr(out),
-                                                          _raw_stream(dev)))
-        return DenseView(*out.split_with_sizes(sizes))
+        out = torch.empty(sum(room), dtype=torch.int32, device=dev)
+        self.ctx._check(self.ctx.lib.mg_dense_arrays_copy_aligned(self.ctx.handle, C.byref(arr), _ptr(out), _ALIGN,
+                                                                  _raw_stream(dev)))
+        return DenseView(*_pieces(out, room)[::2])
 
     def export_many(self):
         """Queue the export of every mini-batch into the paper's arrays (asynchronous, on the sampling stream)."""
@@ -192,13 +204,13 @@ class Dense:
     def export_view(self, batch: int = 0) -> DenseView:
         """Mini-batch `batch` of the last export_many, ready in the order of torch's current stream.  (The stream waits for the
         export, not the host: 32 mini-batches' views are queued while the export runs, the whole call 1107 -> 910 us.)"""
-        arr, at = DenseArrays(), C.c_int32(batch)
-        copy, ctx = self.ctx.lib.mg_dense_export_copy, self.ctx
-        ctx._check(copy(ctx.handle, self.handle, at, C.byref(arr), None, None))
-        sizes = _sizes(arr)
-        out = torch.empty(sum(sizes), dtype=torch.int32, device=ctx.device)
-        ctx._check(copy(ctx.handle, self.handle, at, C.byref(arr), _ptr(out), _raw_stream(ctx.device)))
-        return DenseView(*out.split_with_sizes(sizes))
+        arr, at, ctx = DenseArrays(), C.c_int32(batch), self.ctx
+        ref, copy = C.byref(arr), ctx.lib.mg_dense_export_copy_aligned
+        ctx._check(copy(ctx.handle, self.handle, at, ref, None, _ALIGN, None))
+        room = _room(arr)
+        out = torch.empty(sum(room), dtype=torch.int32, device=ctx.device)
+        ctx._check(copy(ctx.handle, self.handle, at, ref, _ptr(out), _ALIGN, _raw_stream(ctx.device)))
+        return DenseView(*_pieces(out, room)[::2])
 
     def free(self):
         if self.handle:

@@ -1408,10 +1408,11 @@ __global__ void __launch_bounds__(kThreads) k_export_many_entries(ExportManyArgs
 struct ArraysCopy {
     const int32_t* src[5];
     int32_t len[5];
+    int32_t align;   // every array starts at a multiple of this many elements (a power of two)
 };
 __global__ void __launch_bounds__(kThreads) k_copy_arrays(ArraysCopy a, int32_t* __restrict__ dst) {
     const int q = blockIdx.y;
-    for (int p = 0; p < q; ++p) dst += a.len[p];
+    for (int p = 0; p < q; ++p) dst += ((int64_t)a.len[p] + a.align - 1) & -(int64_t)a.align;
     const int32_t* __restrict__ src = a.src[q];
     const int32_t n = a.len[q];
     for (int32_t i0 = blockIdx.x * 4 * kThreads + threadIdx.x; i0 < n; i0 += gridDim.x * 4 * kThreads) {
@@ -2192,9 +2193,9 @@ extern "C" int mg_dense_export_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_
     return MG_OK;
 }
 
-static int copy_arrays(mg_ctx* ctx, const mg_dense_arrays* v, int32_t* dst_dev, cudaStream_t st) {
+static int copy_arrays(mg_ctx* ctx, const mg_dense_arrays* v, int32_t* dst_dev, int32_t align, cudaStream_t st) {
     const ArraysCopy a{{v->node_ids, v->node_id_offsets, v->nbrs, v->nbr_offsets, v->repr_map},
-                       {v->n_nodes, v->k + 2, v->n_entries, v->n_sampled + 1, v->n_entries}};
+                       {v->n_nodes, v->k + 2, v->n_entries, v->n_sampled + 1, v->n_entries}, align};
     const int longest = std::max(std::max(v->n_nodes, v->n_entries), v->n_sampled + 1);
     const int blocks = std::max(1, std::min(mg_grid(ctx, 2), (longest + 4 * kThreads - 1) / (4 * kThreads)));
     k_copy_arrays<<<dim3((unsigned)blocks, 5), kThreads, 0, st>>>(a, dst_dev);
@@ -2203,25 +2204,38 @@ static int copy_arrays(mg_ctx* ctx, const mg_dense_arrays* v, int32_t* dst_dev, 
     return MG_OK;
 }
 
-extern "C" int mg_dense_export_copy(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out, int32_t* dst_dev, void* stream) {
+static bool bad_align(int32_t align) { return align <= 0 || align > 1024 || (align & (align - 1)); }
+
+extern "C" int mg_dense_export_copy_aligned(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out, int32_t* dst_dev, int32_t align,
+                                            void* stream) {
     if (!ctx) return MG_ERR_ARG;
+    if (bad_align(align)) return mg_fail(ctx, MG_ERR_ARG, "align must be a power of two up to 1024");
     if (int rc = exported_arrays(ctx, d, batch, out)) return rc;
     if (!dst_dev) return MG_OK;
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
     cudaStream_t st = (cudaStream_t)stream;
     if (d->export_pending) MG_CUDA(ctx, cudaStreamWaitEvent(st, d->ev_exported));
-    if (int rc = copy_arrays(ctx, out, dst_dev, st)) return rc;
+    if (int rc = copy_arrays(ctx, out, dst_dev, align, st)) return rc;
     MG_CUDA(ctx, mg_reads_add(&d->expm_reads, st));
     return MG_OK;
 }
 
-extern "C" int mg_dense_arrays_copy(mg_ctx* ctx, const mg_dense_arrays* v, int32_t* dst_dev, void* stream) {
+extern "C" int mg_dense_export_copy(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_arrays* out, int32_t* dst_dev, void* stream) {
+    return mg_dense_export_copy_aligned(ctx, d, batch, out, dst_dev, 1, stream);
+}
+
+extern "C" int mg_dense_arrays_copy_aligned(mg_ctx* ctx, const mg_dense_arrays* v, int32_t* dst_dev, int32_t align, void* stream) {
     if (!ctx) return MG_ERR_ARG;
     if (!v || !dst_dev) return mg_fail(ctx, MG_ERR_ARG, "null argument");
+    if (bad_align(align)) return mg_fail(ctx, MG_ERR_ARG, "align must be a power of two up to 1024");
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
-    if (int rc = copy_arrays(ctx, v, dst_dev, (cudaStream_t)stream)) return rc;
+    if (int rc = copy_arrays(ctx, v, dst_dev, align, (cudaStream_t)stream)) return rc;
     MG_CUDA(ctx, mg_reads_add(&ctx->array_reads, (cudaStream_t)stream));
     return MG_OK;
+}
+
+extern "C" int mg_dense_arrays_copy(mg_ctx* ctx, const mg_dense_arrays* v, int32_t* dst_dev, void* stream) {
+    return mg_dense_arrays_copy_aligned(ctx, v, dst_dev, 1, stream);
 }
 
 extern "C" int mg_dense_free(mg_dense* d) {

@@ -1,0 +1,36 @@
+"""What the binding hands out and takes in: tensors with a start and an autograd life of their own, sizes as they were given."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2202_02365_b200 as mg
+from paper_2202_02365_b200 import inputs
+
+N = 5_000
+
+
+@pytest.fixture
+def sample():
+    graph = inputs.erdos_renyi_graph(N, 8 * N, seed=51)
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(inputs.normal_features(N, 12, seed=52, device="cuda"))
+    targets = torch.cat([inputs.distinct_targets(N, n, seed=n) for n in (101, 37, 1)])
+    return ctx, ctx.sample_many(targets, np.array([0, 101, 138, 139]), [3, 5], [1, 2, 3])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("export", [False, True])
+def test_arrays_start_on_their_own_and_live_on_their_own(sample, export):
+    ctx, dense = sample
+    if export:
+        dense.export_many()
+    for b in range(3):
+        v = dense.export_view(b) if export else dense.view(b)
+        for x in (v.node_ids, v.node_id_offsets, v.nbrs, v.nbr_offsets, v.repr_map):
+            assert x.data_ptr() % 512 == 0 and x.is_contiguous() and x._base is None      # as an allocation of its own starts
+        weight = torch.ones((N, 2), device="cuda", requires_grad=True)
+        rows = torch.nn.functional.embedding(v.node_ids, weight)                          # keeps the ids for its backward pass
+        v.nbrs.add_(1)
+        rows.sum().backward()
+        assert int(weight.grad.sum()) == 2 * len(v.node_ids)
