@@ -89,7 +89,7 @@ def _room(arr: "DenseArrays"):
 
 def _pieces(block: torch.Tensor, sizes):
     """Consecutive pieces of a block of memory, each with an autograd life of its own: what is done to one in place is no change of the
-    others (the "unsafe" form of the split is the one whose pieces are no views of the block, and the cheapest)."""
+    others, and autograd may record it (the "unsafe" form of the split is the one whose pieces are no views of the block, and the cheapest)."""
     return torch.unsafe_split_with_sizes(block, sizes)
 
 
@@ -453,7 +453,8 @@ class Context:
 
     def backward(self, model: "Model", dense: "Dense", d_out: torch.Tensor, want_h0_grad: bool = False):
         """Gradients through the last forward(model, dense) (keep_layer_outputs(True) must be set).  Returns the list of
-        (dW_self, dW_nbr, dbias) device tensors per layer and, on request, (dH0 rows, their node ids)."""
+        (dW_self, dW_nbr, dbias) device tensors per layer and, on request, (dH0 rows, their node ids).  The gradients of all layers
+        lie in one allocation, 16-byte aligned: keeping one keeps the memory of all."""
         assert d_out.is_cuda and d_out.dtype == torch.float32 and d_out.is_contiguous()
         dims, dev = list(zip(model.dims[:-1], model.dims[1:])), d_out.device
         g_h0 = ids = None
@@ -467,7 +468,7 @@ class Context:
         flat = torch.empty(sum(sizes), dtype=torch.float32, device=dev)
         self._check(self.lib.mg_backward_begin(self.handle, model.handle, dense.handle, _ptr(d_out), _ptr(g_h0), _ptr(ids), _ptr(flat),
                                                _raw_stream(dev)))
-        pieces = flat.split(sizes)
+        pieces = _pieces(flat, sizes)
         grads = [(pieces[3 * l].view(di, dn), pieces[3 * l + 1].view(di, dn), pieces[3 * l + 2]) for l, (di, dn) in enumerate(dims)]
         self._check(self.lib.mg_backward_end(self.handle))
         return (grads, g_h0, ids) if want_h0_grad else grads

@@ -34,3 +34,19 @@ def test_arrays_start_on_their_own_and_live_on_their_own(sample, export):
         v.nbrs.add_(1)
         rows.sum().backward()
         assert int(weight.grad.sum()) == 2 * len(v.node_ids)
+
+
+@pytest.mark.gpu
+def test_gradients_may_be_changed_in_place(sample):
+    ctx, dense = sample
+    ctx.keep_layer_outputs(True)
+    layers = inputs.random_bias_layers([12, 16, 4], seed=53)
+    model = ctx.model(layers)
+    out = torch.empty((139, 4), device="cuda")
+    ctx.forward(model, dense, out)
+    weight = torch.ones((12, 16), device="cuda", requires_grad=True)
+    grads = ctx.backward(model, dense, torch.ones_like(out))
+    assert all(x.data_ptr() % 16 == 0 for layer in grads for x in layer)
+    kept = grads[0][0].clone()
+    grads[0][0].add_(weight)                # a penalty's share, recorded by autograd
+    assert torch.equal(grads[0][0].detach(), kept + 1) and not grads[0][1].requires_grad
