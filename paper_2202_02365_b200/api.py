@@ -94,7 +94,10 @@ def _pieces(block: torch.Tensor, sizes):
 
 
 def _fanouts(fanouts):
-    return (C.c_int32 * len(fanouts))(*[int(f) for f in fanouts])
+    values = [int(f) for f in fanouts]
+    if any(not -2 ** 31 <= f < 2 ** 31 for f in values):     # (a C array takes the low 32 bits of anything)
+        raise OverflowError("a fanout does not fit 32 bits")
+    return (C.c_int32 * len(values))(*values)
 
 
 def _host(x, dtype) -> torch.Tensor:

@@ -4,9 +4,20 @@ import pytest
 import torch
 
 import paper_2202_02365_b200 as mg
-from paper_2202_02365_b200 import inputs
+from paper_2202_02365_b200 import api, inputs
 
 N = 5_000
+
+
+def test_fanouts_from_any_iterable():
+    for given in ([5, 4], (5, 4), iter([5, 4]), (f for f in (5, 4)), np.array([5, 4]), torch.tensor([5, 4])):
+        assert list(api._fanouts(given)) == [5, 4]
+
+
+@pytest.mark.parametrize("too_large", [2 ** 31, 2 ** 32 + 5, -2 ** 31 - 1])
+def test_fanouts_that_do_not_fit_are_refused(too_large):
+    with pytest.raises((RuntimeError, OverflowError)):
+        api._fanouts([5, too_large])
 
 
 @pytest.fixture
