@@ -2167,11 +2167,11 @@ static int exported_arrays(mg_ctx* ctx, const mg_dense* d, int32_t batch, mg_den
     const ExportLayout L = export_layout(d);
     const int32_t row0 = d->h_rowbase[b], V = d->h_rowbase[b + 1] - row0;
     const int32_t n0 = d->h_cum[(size_t)b * (k + 2) + k + 1] - d->h_cum[(size_t)b * (k + 2) + k];
-    int64_t e_before = 0, e_mine = 0;
+    int64_t e_before = 0, e_mine = 0;   // entries are packed mini-batch after mini-batch in the export
     for (int h = 0; h < k; ++h) {
-        // entries are packed mini-batch after mini-batch in the export
-        for (int bb = 0; bb < b; ++bb) e_before += d->h_ent_hop[(size_t)h * (B + 1) + bb + 1] - d->h_ent_hop[(size_t)h * (B + 1) + bb];
-        e_mine += d->h_ent_hop[(size_t)h * (B + 1) + b + 1] - d->h_ent_hop[(size_t)h * (B + 1) + b];
+        const int32_t* at = d->h_ent_hop.data() + (size_t)h * (B + 1);
+        e_before += at[b] - at[0];
+        e_mine += at[b + 1] - at[b];
     }
     out->k = k;
     out->n_nodes = V;

@@ -116,3 +116,19 @@ def test_id_table_blocks_over_many_mini_batches(graph, ctx, per, fanout):
             assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
         one.free()
     d.free()
+
+
+# as many mini-batches as a call may have: where each stands in the export
+def test_export_of_as_many_mini_batches_as_a_call_may_have(graph, ctx):
+    n_batches = 4_096
+    rows = [inputs.distinct_targets(N, 1 + b % 3, seed=b) for b in range(n_batches)]
+    rows[17] = rows[17][:0]
+    offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    d = ctx.sample_many(torch.cat(rows), offs, [3, 2, 2], list(range(n_batches)), caps={"max_nodes_per_batch": 200})
+    d.export_many()
+    views = [d.export_view(b) for b in range(n_batches)]
+    for b in (0, 1, 16, 17, 18, 2_047, n_batches - 2, n_batches - 1):
+        x, y = views[b], d.view(b)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
+    d.free()
