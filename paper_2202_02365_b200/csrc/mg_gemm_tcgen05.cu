@@ -138,8 +138,7 @@ int mg_gemm_tf32(mg_ctx* ctx, const float* x, const float* w_t, const float* bia
     CUtensorMap ma, mb;
     if (!make_map_f32(&ma, x, M, K, BM) || !make_map_f32(&mb, w_t, N, K, p.BN))
         return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed (M %lld N %d K %d)", (long long)M, N, K);
-    static uint64_t smem_done = 0;
-    MG_CUDA(ctx, mg_smem_limit(&smem_done, ctx->device, (const void*)k_gemm_tf32, 100 * 1024));
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_gemm_tf32, 100 * 1024));
     dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + p.BN - 1) / p.BN));
     k_gemm_tf32<<<grid, kGemmThreads, smem, ctx->stream>>>(ma, mb, p);
     ctx->launches++;

@@ -77,6 +77,7 @@ struct mg_ctx {
     std::string err;
     int64_t launches = 0;
     int n_sms = 148;
+    std::vector<const void*> smem_raised;   // kernels whose shared-memory limit this context has raised (mg_smem_limit)
     // word the tensor-core kernels report a barrier time-out in: mapped host memory (a copy of a device word cost a forward pass
     // 17 us behind its last kernel), read by the host once the stream has drained; d_flags is its device address
     uint32_t* h_flags = nullptr;
@@ -346,11 +347,11 @@ struct ProfScope {
     ~ProfScope() { mg_prof_end(c, ph, n); }
 };
 
-// dynamic shared-memory limit of a kernel, raised once per device and not before every launch (`done`: the launch site's own bits)
-static inline cudaError_t mg_smem_limit(uint64_t* done, int device, const void* kernel, int bytes) {
-    if (device < 64 && (*done >> device & 1)) return cudaSuccess;
+// dynamic shared-memory limit of a kernel, raised once per context (a context has one device, and belongs to one thread)
+static inline cudaError_t mg_smem_limit(mg_ctx* ctx, const void* kernel, int bytes) {
+    for (const void* k : ctx->smem_raised) if (k == kernel) return cudaSuccess;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && device < 64) *done |= 1ull << device;
+    if (e == cudaSuccess) ctx->smem_raised.push_back(kernel);
     return e;
 }
 

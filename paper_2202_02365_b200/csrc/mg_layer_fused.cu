@@ -1156,10 +1156,9 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
      k_sage_layer_fused<false, false, false, TS, HALVES>, k_sage_layer_fused<false, true, true, TS, HALVES>}
     static const Kernel kernels[2][2][5] = {{MG_FUSED_KERNELS(false, 1), MG_FUSED_KERNELS(true, 1)}, {MG_FUSED_KERNELS(false, 2), MG_FUSED_KERNELS(true, 2)}};
 #undef MG_FUSED_KERNELS
-    static uint64_t smem_done[2][2][5] = {};
     const int which = first ? (f16 ? 2 : half ? 1 : 0) : (f16 ? 4 : 3);
     const Kernel kern = kernels[halves - 1][ts][which];
-    MG_CUDA(ctx, mg_smem_limit(&smem_done[halves - 1][ts][which], ctx->device, (const void*)kern, fused_smem_limit(halves)));
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)kern, fused_smem_limit(halves)));
     const int64_t n_tiles = (rows + HM * halves - 1) / (HM * halves);
     const int grid = 2 * (int)std::min<int64_t>((n_tiles + 1) / 2, pairs);   // CTA pairs
     cudaLaunchConfig_t cfg = {};
@@ -1202,9 +1201,8 @@ int mg_layer_grad_weights(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, i
     const size_t smem = kGradStages * (kGradStageX + (size_t)(p.n_cols / 32) * kGradBox) + 1024;
     typedef void (*Kernel)(CUtensorMap, GradWArgs);
     static const Kernel kernels[3] = {k_sage_grad_weights<true, false>, k_sage_grad_weights<true, true>, k_sage_grad_weights<false, false>};
-    static uint64_t smem_done[3] = {};
     const int which = layer > 1 ? 2 : ctx->feat_dtype == MG_DTYPE_F16 ? 1 : 0;
-    MG_CUDA(ctx, mg_smem_limit(&smem_done[which], ctx->device, (const void*)kernels[which], (int)(kGradStages * (kGradStageX + 8 * kGradBox) + 1024)));
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)kernels[which], (int)(kGradStages * (kGradStageX + 8 * kGradBox) + 1024)));
     kernels[which]<<<dim3((unsigned)p.n_slices, (unsigned)groups), kGradThreads, smem, ctx->stream>>>(mg, p);
     ctx->launches++;
     MG_CUDA(ctx, cudaGetLastError());

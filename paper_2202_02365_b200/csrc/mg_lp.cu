@@ -747,8 +747,7 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
             ctx->launches++;
             ta.b_images = (const uint8_t*)ctx->dm_images;
             const size_t smem = (size_t)ta.n_slices * 16384 + 2 * (size_t)ta.n_slices * ta.bn_max * 128 + 1024;
-            static uint64_t smem_done = 0;
-            MG_CUDA(ctx, mg_smem_limit(&smem_done, ctx->device, (const void*)k_distmult_neg_tc, kTcMaxSlices * (16384 + 2 * kTcBlockN * 128) + 1024));
+            MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_distmult_neg_tc, kTcMaxSlices * (16384 + 2 * kTcBlockN * 128) + 1024));
             int sides = 0;
             for (int q = 0; q < 2; ++q) {
                 const bool dst = q == 0;

@@ -1441,8 +1441,6 @@ void mg_sort_params_host(SortParams* sp, int64_t n) {
     sp->zero = 0; sp->n = (int32_t)n; sp->ntiles = (int32_t)((n + kSortTile - 1) / kSortTile); sp->hist_len = kBins * sp->ntiles;
 }
 
-static void sample_kernel_attributes();
-
 // LSD radix sort of 64-bit keys on bits [lo_bit, lo_bit + bits); sp (device) holds the key count.
 // Keys start in buf[0]; *res_buf tells which buffer holds the result.
 // With a tile table (seg_tiles, SegTile per tile; sp->ntiles tiles): a sort inside segments -- the first pass reads
@@ -1454,7 +1452,7 @@ void mg_sort_u64(mg_ctx* ctx, uint64_t* const buf[2], const SortParams* sp, int 
     const int grid = mg_grid(ctx, 8);
     const int passes = (bits + kRadixBits - 1) / kRadixBits;
     ScanRange r{&sp->zero, &sp->hist_len, nullptr};
-    sample_kernel_attributes();
+    mg_smem_limit(ctx, (const void*)k_radix_scatter, (int)kScatterSmem);   // (an error shows at the launch)
     int cur = 0;
     for (int p = 0; p < passes; ++p) {
         const int shift = lo_bit + kRadixBits * p;
@@ -1645,16 +1643,13 @@ extern "C" int mg_sample_many(mg_ctx* ctx, const int32_t* targets, int targets_o
 }
 
 
-// dynamic shared-memory limits of the sampler's kernels, set once (not inside a stream capture)
-static void sample_kernel_attributes() {
-    static bool done = false;
-    if (done) return;
-    cudaFuncSetAttribute(k_radix_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
-    cudaFuncSetAttribute(k_dedupe_last<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kDedupMaxSlots * 2 * sizeof(int32_t)));
-    cudaFuncSetAttribute(k_dedupe_last<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDedupSlots512 * 2 * (int)sizeof(int32_t));
-    cudaFuncSetAttribute(k_hop<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + kTileMax * hop_node_bytes(true));
-    done = true;
+// dynamic shared-memory limits of the sampler's kernels (not inside a stream capture)
+static int sample_kernel_limits(mg_ctx* ctx) {
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_dedupe_last<1024>, (int)(kDedupMaxSlots * 2 * sizeof(int32_t))));
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_dedupe_last<512>, kDedupSlots512 * 2 * (int)sizeof(int32_t)));
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_hop<0>,
+                               (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + kTileMax * hop_node_bytes(true)));
+    return MG_OK;
 }
 
 static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on_device,
@@ -1819,7 +1814,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
         MG_CUDA(ctx, cudaMemcpyAsync(d->newlist[1], targets, sizeof(int32_t) * T, cudaMemcpyHostToDevice, st));
         st_hdr->targets = (uint64_t)(uintptr_t)d->newlist[1];
     }
-    sample_kernel_attributes();
+    if ((rc = sample_kernel_limits(ctx))) return rc;
 
     // Grids follow what a hop can hold at most (the number of targets rounded up to a power of two, so that calls of similar
     // size share the captured graph): blocks without work cost the small calls as much as the work itself.
