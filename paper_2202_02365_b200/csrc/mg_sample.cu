@@ -1739,9 +1739,6 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     const int32_t table_size = (int32_t)want_slots;
     if ((int64_t)table_size * n_batches >= (1ll << 31))
         return mg_fail(ctx, MG_ERR_CAPACITY, "n_batches x id-table size must stay below 2^31: pass a smaller max_nodes_per_batch or fewer batches");
-    const int id_bits = std::max(1, ilog2_ceil(N));
-    const int b_bits = std::max(1, ilog2_ceil(n_batches));
-    if (MG_SLOT_BITS + id_bits + b_bits > 64) return mg_fail(ctx, MG_ERR_ARG, "id and batch bits do not fit the sort key");
 
     mg_dense* d = *out;
     const bool created = (d == nullptr);

@@ -132,3 +132,25 @@ def test_export_of_as_many_mini_batches_as_a_call_may_have(graph, ctx):
         for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
             assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
     d.free()
+
+
+# ids of 29 bits and mini-batches of 12: no part of a sample packs both into one word
+def test_many_mini_batches_on_a_graph_of_many_nodes():
+    n, n_batches = 2 ** 28 + 1, 2_049
+    rows = torch.arange(n_batches, device="cuda") * ((n - 1) // (n_batches - 1))             # a target each, the first and the last node among them
+    assert int(rows[-1]) == n - 1
+    off = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    off[rows + 1] = 3
+    off = torch.cumsum(off, 0)
+    nbrs = torch.stack([(rows + 1) % n, (rows + 12_345) % n, (rows + n // 2) % n], 1).sort(1).values
+    c = mg.Context(0)
+    c.load_graph(off, nbrs.flatten().to(torch.int32))
+    del off
+    d = c.sample_many(rows.to(torch.int32), list(range(n_batches + 1)), [3], list(range(n_batches)), caps={"max_nodes_per_batch": 16})
+    d.export_many()
+    for b in (0, 1, 1_024, n_batches - 1):
+        for v in (d.export_view(b), d.view(b)):
+            assert torch.equal(v.nbrs.long(), nbrs[b]) and int(v.node_ids[-1]) == int(rows[b])
+            assert torch.equal(v.node_ids[v.repr_map.long()].long(), nbrs[b])
+    c.close()
+    torch.cuda.empty_cache()
