@@ -433,7 +433,7 @@ int mg_profile_read(mg_ctx* ctx, int32_t* n_phases, const char** names, double* 
  * of dims[0] floats per node of every mini-batch in the library's packed row order -- mg_dense_packed_ids gives the
  * node id of each row -- i.e. the gradient rows of the base representations.  fp32 arithmetic; sums over rows use
  * atomic adds (low-order bits vary from run to run).  Synchronous.  Errors: MG_ERR_ARG, MG_ERR_STATE (no matching
- * forward pass, layers not kept), MG_ERR_OOM, MG_ERR_TIMEOUT (a bounded wait on the device ran out: the gradients are not
+ * forward pass, layers not kept), MG_ERR_OOM, MG_ERR_CAPACITY (2^30 rows of one layer or more), MG_ERR_TIMEOUT (a bounded wait on the device ran out: the gradients are not
  * to be used).  The environment variable MG_REV_POLLS (for diagnosis) sets how often one of these waits looks. */
 int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, float* d_h0_dev);
 

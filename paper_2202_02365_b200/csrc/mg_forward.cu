@@ -1087,6 +1087,8 @@ struct GatherArgs {
 // three at 72 take 481 / 178 us.)
 constexpr int kGradRows = 16, kGradItems = kGradRows * (kGradLight + 1);
 static_assert(kGradItems >= kGradUnit + 1, "a unit's items fit the list");
+constexpr int64_t kGradMaxRows = (1ll << 30) - 1;   // an item holds twice its output row, and one more, in 31 bits; the largest value means none
+static_assert(2 * (kGradMaxRows - 1) + 1 < 0x7FFFFFFFll, "an output row's item is not the one that means none");
 template <bool MASK>
 __global__ void __launch_bounds__(kThreads, MASK ? 4 : 1) k_grad_gather(GatherArgs a) {
     constexpr int U = MASK ? 4 : 8, kWarps = kThreads / 32;
@@ -1302,6 +1304,8 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     const int64_t in_total = ra.in_at[k + 1], ent_total = ra.ent_at[k + 1];
     const int64_t rev_tiles = (in_total + kRevTile - 1) / kRevTile;
     if (ent_total >= (1ll << 32)) return mg_fail(ctx, MG_ERR_CAPACITY, "too many entries for one backward pass");
+    for (int l = ra.l0; l <= k; ++l)
+        if (d->h_hdr.rows_total[l] > kGradMaxRows) return mg_fail(ctx, MG_ERR_CAPACITY, "too many rows for one backward pass");
     if (ctx->bw_g_elems < g_total && (rc = mg_ensure(ctx, &ctx->bw_g, &ctx->bw_g_elems, g_total + g_total / 4 + 16))) return rc;
     if (ctx->bw_x_elems < (size_t)max_x && (rc = mg_ensure(ctx, &ctx->bw_x, &ctx->bw_x_elems, (size_t)max_x + 16))) return rc;
     if (ctx->bw_dx_elems < (size_t)max_dx && (rc = mg_ensure(ctx, &ctx->bw_dx, &ctx->bw_dx_elems, (size_t)max_dx + 16))) return rc;
