@@ -431,10 +431,13 @@ int mg_profile_read(mg_ctx* ctx, int32_t* n_phases, const char** names, double* 
  * mg_forward's output.  The weight and bias gradients of every layer are left in buffers owned by the model
  * (mg_model_grads), overwriting those of the previous call.  d_h0_dev (DEVICE, nullable): receives dL/dH^0, one row
  * of dims[0] floats per node of every mini-batch in the library's packed row order -- mg_dense_packed_ids gives the
- * node id of each row -- i.e. the gradient rows of the base representations.  fp32 arithmetic; sums over rows use
- * atomic adds (low-order bits vary from run to run).  Synchronous.  Errors: MG_ERR_ARG, MG_ERR_STATE (no matching
- * forward pass, layers not kept), MG_ERR_OOM, MG_ERR_CAPACITY (2^30 rows of one layer or more), MG_ERR_TIMEOUT (a bounded wait on the device ran out: the gradients are not
- * to be used).  The environment variable MG_REV_POLLS (for diagnosis) sets how often one of these waits looks. */
+ * node id of each row -- i.e. the gradient rows of the base representations.  A model with MG_GEMM_TF32 takes the
+ * products for the weights' and the input rows' gradients on the tensor cores (operands cut to TF32's ten bits, fp32
+ * accumulate), one with MG_GEMM_FP32 in fp32; the other sums are fp32.  Sums over rows use atomic adds (low-order bits
+ * vary from run to run).  Synchronous.  Errors: MG_ERR_ARG, MG_ERR_STATE (no matching forward pass, layers not kept),
+ * MG_ERR_OOM, MG_ERR_CAPACITY (2^30 rows of one layer or more), MG_ERR_TIMEOUT (a bounded wait on the device ran out:
+ * the gradients are not to be used).  The environment variable MG_REV_POLLS (for diagnosis) sets how often one of these
+ * waits looks. */
 int mg_backward(mg_ctx* ctx, mg_model* m, mg_dense* d, const float* d_out_dev, float* d_h0_dev);
 
 /* The same in two calls, so that the caller's host work runs beside the pass: mg_backward_begin queues it (arguments and errors of

@@ -804,13 +804,14 @@ extern "C" int mg_layer_output(mg_ctx* ctx, const mg_model* m, mg_dense* d, int3
 
 // ---------------------------------------------------------------------------------------
 // Backward pass through the GraphSage layers (Section 3: the gradients of a mini-batch update the model and the
-// base representations).  Chain rule through Algorithm 3 and Algorithm 2, layer k down to layer 1, over the same
-// row chunks as the unfused forward path:
-//   X = [self | aggregate] of the chunk is recomputed from H^{l-1} (kept by the forward pass),
+// base representations).  Chain rule through Algorithm 3 and Algorithm 2, layer k down to layer 1, whole layers at a time:
 //   dPre = dH^l (masked by H^l > 0 below the last layer),
-//   dW += X^T dPre, dbias += column sums of dPre, dX = dPre W^T,
-//   dH^{l-1}[self row] += dX[:, :d_in];  dH^{l-1}[source row of entry e] += dX[:, d_in:] / count (or x 1 for a sum).
-// All arithmetic is fp32 on CUDA cores; sums over rows use atomic adds, so low-order bits vary from run to run.
+//   dW += X^T dPre with X = [self | aggregate] gathered again from H^{l-1} (kept by the forward pass), dbias += column
+//   sums of dPre, dX = dPre W^T,
+//   dH^{l-1}[row] = its self part of dX + the neighbour parts of every entry that names it, times 1 / count (1 for a sum).
+// A model with TF32 products takes dW and dX on the tensor cores (X, dPre and W as they lie in memory, of which the tensor cores
+// read ten bits of the mantissa; fp32 accumulate), one with fp32 products on CUDA cores, there with X in chunks of rows.  All
+// other sums are fp32.  Sums over rows meet by atomic adds, so low-order bits vary from run to run.
 // ---------------------------------------------------------------------------------------
 namespace {
 
@@ -837,11 +838,10 @@ __device__ __forceinline__ void locate_row(const RowGeom& g, int layer, int64_t 
     *node_out = g.node_off[(int64_t)j * (g.B + 1) + lo] + (local - cum[j]);
 }
 
-// The gradient of a layer's pre-activations and of its bias in one pass: g *= (y > 0) where the layer has a ReLU
-// (MASK; y = the layer's kept outputs), db += column sums of g.  A thread keeps four columns and walks down the rows
-// (16-byte accesses, a block covers whole rows); column sums meet in shared memory, one atomic add per column and block.
-template <bool MASK>
-__global__ void __launch_bounds__(kThreads) k_grad_pre_bias(float* g, const float* __restrict__ y, float* db, int64_t rows, int N) {
+// The gradient of the last layer's bias: db += column sums of g (below it, k_grad_gather sums the bias on its way).  A thread keeps
+// four columns and walks down the rows (16-byte accesses, two rows in flight, a block covers whole rows); column sums meet in shared
+// memory, one atomic add per column and block.
+__global__ void __launch_bounds__(kThreads) k_grad_bias(const float* __restrict__ g, float* db, int64_t rows, int N) {
     __shared__ float sums[1024];
     const int n4 = N / 4;                       // (widths are multiples of 4, at most 1024)
     const int rows_per_pass = kThreads / n4;    // >= 1
@@ -850,21 +850,10 @@ __global__ void __launch_bounds__(kThreads) k_grad_pre_bias(float* g, const floa
     const int c4 = threadIdx.x % n4, rr = threadIdx.x / n4;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (rr < rows_per_pass) {
-        float4* g4 = reinterpret_cast<float4*>(g);
-        const float4* y4 = reinterpret_cast<const float4*>(y);
+        const float4* g4 = reinterpret_cast<const float4*>(g);
         const int64_t step = (int64_t)gridDim.x * rows_per_pass;
         for (int64_t r = (int64_t)blockIdx.x * rows_per_pass + rr; r < rows; r += 2 * step) {
-            const int64_t i0 = r * n4 + c4, i1 = (r + step) * n4 + c4;
-            const bool two = r + step < rows;
-            float4 v0 = g4[i0], v1 = two ? g4[i1] : make_float4(0.f, 0.f, 0.f, 0.f);
-            if (MASK) {
-                const float4 a0 = y4[i0], a1 = two ? y4[i1] : make_float4(1.f, 1.f, 1.f, 1.f);
-                const float4 m0 = make_float4(a0.x > 0.f ? v0.x : 0.f, a0.y > 0.f ? v0.y : 0.f, a0.z > 0.f ? v0.z : 0.f, a0.w > 0.f ? v0.w : 0.f);
-                const float4 m1 = make_float4(a1.x > 0.f ? v1.x : 0.f, a1.y > 0.f ? v1.y : 0.f, a1.z > 0.f ? v1.z : 0.f, a1.w > 0.f ? v1.w : 0.f);
-                g4[i0] = m0;
-                if (two) g4[i1] = m1;
-                v0 = m0; v1 = m1;
-            }
+            const float4 v0 = g4[r * n4 + c4], v1 = r + step < rows ? g4[(r + step) * n4 + c4] : make_float4(0.f, 0.f, 0.f, 0.f);
             s.x += v0.x + v1.x; s.y += v0.y + v1.y; s.z += v0.z + v1.z; s.w += v0.w + v1.w;
         }
         atomicAdd(&sums[4 * c4], s.x); atomicAdd(&sums[4 * c4 + 1], s.y); atomicAdd(&sums[4 * c4 + 2], s.z); atomicAdd(&sums[4 * c4 + 3], s.w);
@@ -1354,7 +1343,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         if (l == k && M > 0) {
             // (few blocks: every one ends with an atomic add per column; 8,000 x 256 in 1,184 blocks took 13 us, in 148 6.5 us)
             const int blocks = (int)std::min<int64_t>(ctx->n_sms, (M + kThreads / (d_out / 4) - 1) / (kThreads / (d_out / 4)));
-            k_grad_pre_bias<false><<<blocks, kThreads, 0, st>>>(const_cast<float*>(d_out_dev), nullptr, m->g_bias[l - 1], M, d_out);
+            k_grad_bias<<<blocks, kThreads, 0, st>>>(d_out_dev, m->g_bias[l - 1], M, d_out);
             ctx->launches++;
         }
         const float* h_prev = l > 1 ? ctx->ws_h[0] + h_off[l - 1] : nullptr;
