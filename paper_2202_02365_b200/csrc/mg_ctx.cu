@@ -12,8 +12,8 @@
 #include "mg_internal.cuh"
 
 static const char* kPhaseNames[PH_COUNT] = {
-    "sample_init", "sample_count", "sample_scan", "sample_pick", "sample_sort", "sample_place",
-    "sample_relabel", "sample_final", "aggregate_l1", "aggregate_rest", "gemm", "distmult", "other"};
+    "sample_init", "sample_pick", "sample_sort", "sample_place",
+    "sample_relabel", "aggregate_l1", "aggregate_rest", "gemm", "distmult", "other"};
 
 int mg_fail(mg_ctx* ctx, int code, const char* fmt, ...) {
     if (ctx) {
@@ -51,7 +51,7 @@ void mg_prof_begin(mg_ctx* ctx, int phase) {
     ctx->prof_pending.push_back({phase, {a, b}});
 }
 
-void mg_prof_end(mg_ctx* ctx, int phase, int n_launches) {
+void mg_prof_end(mg_ctx* ctx, int phase, int64_t n_launches) {
     if (!ctx->prof_on) return;
     for (size_t i = ctx->prof_pending.size(); i-- > 0;) {
         if (ctx->prof_pending[i].first == phase) {

@@ -572,7 +572,7 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
     if (any_fused) {
         const size_t need = (size_t)meta_at[k + 1];
         if (ctx->ws_meta_elems < need && (rc = mg_ensure(ctx, &ctx->ws_meta, &ctx->ws_meta_elems, need + need / 4 + 4))) return rc;
-        ProfScope ps(ctx, PH_OTHER, 1);
+        ProfScope ps(ctx, PH_OTHER);
         if ((rc = mg_layer_rows(ctx, d, ctx->ws_meta, meta_at))) return rc;
     }
     // H^k stays in the library's buffer (mg_layer_output, mg_backward) and goes to the caller's: the last layer's kernel
@@ -612,7 +612,7 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
                 // pointers shifted so that the kernel's global packed row indices land inside the windows
                 const float* h_prev = l > 1 ? base + ring_off[l - 1] - lo_in * m->dims[l - 1] : nullptr;
                 float* h_out = l == k ? hk : base + ring_off[l] - lo * m->dims[l];
-                ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST, 1);
+                ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST);
                 rc = mg_layer_fused(ctx, d, l, m->dims[l - 1], m->dims[l], m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
                                     (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], lo, hi, l > 1 ? lo_in : 0, l == 1 ? m->w_pad_h[0] : nullptr, 0, 0);
                 if (rc) return rc;
@@ -665,7 +665,7 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
         if (m->precision == MG_GEMM_TF32 && mg_layer_fused_supported(d_in, d_out)) {
             // gather + segment mean + both linear maps in one persistent tensor-core kernel
             {
-                ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST, 1);
+                ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST);
                 rc = mg_layer_fused(ctx, d, l, d_in, d_out, m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
                                     (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], 0, M, 0,
                                     (l == 1 || f16_inter) ? m->w_pad_h[l - 1] : nullptr, f16_inter && l > 1, f16_inter && l < k);
@@ -689,14 +689,14 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
             a.round_tf32 = m->precision == MG_GEMM_TF32;
             a.sum_aggr = m->sum_aggr ? 1 : 0;
             {
-                ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST, 1);
+                ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST);
                 const int grid = mg_grid(ctx, 8);
                 if (l == 1) { if (half) launch_aggregate<true, true>(a, grid, st); else launch_aggregate<true, false>(a, grid, st); }
                 else launch_aggregate<false, false>(a, grid, st);
                 ctx->launches++;
             }
             {
-                ProfScope ps(ctx, PH_GEMM, 1);
+                ProfScope ps(ctx, PH_GEMM);
                 const int64_t rows = r1 - r0;
                 const bool relu = l < k;
                 if (m->precision == MG_GEMM_FP32) {

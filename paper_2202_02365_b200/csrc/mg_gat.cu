@@ -502,7 +502,7 @@ extern "C" int mg_gat_forward(mg_ctx* ctx, const mg_gat_model* m, mg_dense* d, f
             const int d_in = m->dims[l - 1], d_out = m->dims[l];
             const int64_t rows_out = d->h_hdr.rows_total[l];
             {
-                ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST, 1);
+                ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST);
                 InAttendArgs a;
                 a.g = geom; a.layer = l; a.nodes = d->nodes; a.ent_off = d->ent_off; a.ent_nbrs = d->ent_nbrs; a.ent_repr = d->ent_repr;
                 a.slots = ctx->slots; a.feat = mg_feat_geom(ctx); a.row_bytes = ctx->row_bytes; a.h_prev = h_in;
@@ -518,7 +518,7 @@ extern "C" int mg_gat_forward(mg_ctx* ctx, const mg_gat_model* m, mg_dense* d, f
             }
             float* out_l = l == k ? out_dev : ctx->gat_h[l & 1];
             {
-                ProfScope ps(ctx, PH_GEMM, 1);
+                ProfScope ps(ctx, PH_GEMM);
                 if (tf32) {
                     if ((rc = mg_gemm_tf32(ctx, ctx->gat_x, m->w_t[l - 1], m->bias[l - 1], out_l, rows_out, d_out, d_in, l < k))) return rc;
                 } else {
@@ -548,7 +548,7 @@ extern "C" int mg_gat_forward(mg_ctx* ctx, const mg_gat_model* m, mg_dense* d, f
         if ((rc = grow(&ctx->gat_h[i], &ctx->gat_h_elems[i], need_h))) return rc;
     if (d->h_hdr.rows_total[k] == 0) return MG_OK;
     {
-        ProfScope ps(ctx, PH_AGG_L1, 1);
+        ProfScope ps(ctx, PH_AGG_L1);
         GatherArgs a;
         a.g = geom; a.nodes = d->nodes; a.slots = ctx->slots; a.feat = mg_feat_geom(ctx);
         a.row_bytes = ctx->row_bytes; a.n_rows = d->h_hdr.rows_total[0];
@@ -565,7 +565,7 @@ extern "C" int mg_gat_forward(mg_ctx* ctx, const mg_gat_model* m, mg_dense* d, f
         const int H = m->heads;
         float* s_dst = ctx->gat_s + rows_in * H;
         {
-            ProfScope ps(ctx, PH_GEMM, 1);
+            ProfScope ps(ctx, PH_GEMM);
             if (tf32) {
                 if ((rc = mg_gemm_tf32(ctx, h_prev, m->w_t[l - 1], m->zeros, ctx->gat_z, rows_in, d_out, d_in, false))) return rc;
             } else {
@@ -574,7 +574,7 @@ extern "C" int mg_gat_forward(mg_ctx* ctx, const mg_gat_model* m, mg_dense* d, f
                 ctx->launches++;
             }
         }
-        ProfScope ps(ctx, PH_AGG_REST, 2);
+        ProfScope ps(ctx, PH_AGG_REST);
         k_gat_scores_heads<<<grid, kThreads, 0, st>>>(ctx->gat_z, m->a_src[l - 1], m->a_dst[l - 1], rows_in, d_out, H, s_src, s_dst);
         AttendArgs a;
         a.g = geom; a.layer = l; a.ent_off = d->ent_off; a.ent_repr = d->ent_repr; a.z = ctx->gat_z; a.s_src = s_src; a.s_dst = s_dst;

@@ -47,13 +47,10 @@ struct ProfPhase {
 
 enum {
     PH_SAMPLE_INIT = 0,
-    PH_SAMPLE_COUNT,
-    PH_SAMPLE_SCAN,
     PH_SAMPLE_PICK,
     PH_SAMPLE_SORT,
     PH_SAMPLE_PLACE,
     PH_SAMPLE_RELABEL,
-    PH_SAMPLE_FINAL,
     PH_AGG_L1,
     PH_AGG_REST,
     PH_GEMM,
@@ -339,12 +336,12 @@ static inline int mg_ensure(mg_ctx* ctx, T** ptr, size_t* have_elems, size_t nee
 }
 
 void mg_prof_begin(mg_ctx* ctx, int phase);
-void mg_prof_end(mg_ctx* ctx, int phase, int n_launches);
+void mg_prof_end(mg_ctx* ctx, int phase, int64_t n_launches);
 
-struct ProfScope {
-    mg_ctx* c; int ph; int n;
-    ProfScope(mg_ctx* ctx, int phase, int launches) : c(ctx), ph(phase), n(launches) { mg_prof_begin(c, ph); }
-    ~ProfScope() { mg_prof_end(c, ph, n); }
+struct ProfScope {   // the kernels launched while it lives belong to the phase
+    mg_ctx* c; int ph; int64_t before;
+    ProfScope(mg_ctx* ctx, int phase) : c(ctx), ph(phase), before(ctx->launches) { mg_prof_begin(c, ph); }
+    ~ProfScope() { mg_prof_end(c, ph, c->launches - before); }
 };
 
 // dynamic shared-memory limit of a kernel, raised once per context (a context has one device, and belongs to one thread)

@@ -704,7 +704,7 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
     if ((corrupt & MG_CORRUPT_SRC) && lp->negs > 0 && !neg_src_out) return mg_fail(ctx, MG_ERR_ARG, "null neg_src_out");
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
     cudaStream_t st = ctx->stream;
-    ProfScope ps(ctx, PH_DISTMULT, 3);
+    ProfScope ps(ctx, PH_DISTMULT);
     const bool tensor = gemm_precision == MG_GEMM_TF32 && dim % 4 == 0 && dim <= 32 * kTcMaxSlices && lp->negs > 0;
     if (!tensor) {
         k_distmult_pos<<<mg_grid(ctx, 8), kThreads, 0, st>>>(h_dev, rel_emb_dev, lp->src_idx, lp->dst_idx, lp->rel, lp->n_edges, dim, pos_out);

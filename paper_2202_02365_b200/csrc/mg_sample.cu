@@ -1831,7 +1831,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     auto enqueue = [&]() -> int {
     uint32_t* batch_cnt = d->batch_cnt;   // new nodes per (hop, mini-batch)
     {
-        ProfScope ps(ctx, PH_SAMPLE_INIT, 1);
+        ProfScope ps(ctx, PH_SAMPLE_INIT);
         BeginArgs a{d->h_stage_dev, (int32_t)hdr_ints, B + 1, B * (k + 2), 2 * B, (int32_t)seeds_at, k * B, (int64_t)B * table_size / 4,
                     reinterpret_cast<int32_t*>(d->hdr), d->node_off, d->cum, reinterpret_cast<int32_t*>(d->d_seeds),
                     reinterpret_cast<int32_t*>(batch_cnt), reinterpret_cast<int4*>(d->hkeys)};
@@ -1842,7 +1842,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
         const int32_t f = fanouts[h];
         const bool smem_hop = smem_last && h == k - 1;
         {
-            ProfScope ps(ctx, PH_SAMPLE_PICK, 1);
+            ProfScope ps(ctx, PH_SAMPLE_PICK);
             HopArgs a{d->hdr, h, f, d->nodes, d->node_batch, {ctx->view_off, inout ? ctx->view_off_out : nullptr},
                       {ctx->view_nbrs, ctx->view_nbrs_out}, d->ent_off, d->ent_nbrs, d->ent_repr, d->d_seeds, d->cap_entries, d->tile_state,
                       hop_tile(nodes_bound[h]), B, d->node_off, d->hkeys, d->hvals, tg, ctx->n_nodes, mg_feat_geom(ctx)};
@@ -1862,7 +1862,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
             ctx->launches++;
         }
         {
-            ProfScope ps(ctx, PH_SAMPLE_RELABEL, 1);
+            ProfScope ps(ctx, PH_SAMPLE_RELABEL);
             if (smem_hop) {
                 DedupArgs da{d->hdr, h, B, k, (int32_t)dedup_nb, dedup_slots, d->nodes, d->node_off, d->ent_off, d->ent_nbrs,
                              d->ent_repr, d->pairs, d->share_off, d->cum, batch_cnt + (size_t)h * B, d->new_ids,
@@ -1889,7 +1889,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
             }
         }
         {
-            ProfScope ps(ctx, PH_SAMPLE_PLACE, 1);
+            ProfScope ps(ctx, PH_SAMPLE_PLACE);
             PlaceArgs pa{d->hdr, h, d->new_ids, batch_cnt + (size_t)h * B, d->cap_nodes, d->nodes, d->node_batch,
                          smem_hop ? nullptr : d->hvals, h < k - 1 ? inner_limit : (int32_t)cap_batch, d->ent_repr, B, k, d->cum, d->node_off, (int32_t)hdr_ints, d->ent_off,
                          d->rowbase, d->d_ent_hop, d->h_stage_dev + summary_at};
@@ -2130,7 +2130,7 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
         const int grid = mg_grid(ctx, 8);
         ctx->stream = st;   // the sort and scan helpers (and the phase events) use ctx->stream
         {
-        ProfScope ps(ctx, PH_SAMPLE_SORT, 0);
+        ProfScope ps(ctx, PH_SAMPLE_SORT);
         k_export_tiles<<<1, 1024, 0, st>>>(a, static_cast<SegTile*>(d->seg_tiles), sp, range);
         k_export_keys<<<grid, kThreads, 0, st>>>(a, d->newlist[0]);
         int res = 0;
@@ -2138,9 +2138,9 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
         k_export_place<<<grid, kThreads, 0, st>>>(a, d->newlist[res]);
         mg_scan_u32(ctx, a.cnt, &range[0], &range[1], nullptr, (uint32_t*)d->scan_tmp, nullptr);
         k_export_many_entries<<<grid, kThreads, 0, st>>>(a);
+        ctx->launches += 4;
         }
         ctx->stream = user;
-        ctx->launches += 4;
     }
     MG_CUDA(ctx, cudaGetLastError());
     MG_CUDA(ctx, cudaEventRecord(d->ev_exported, st));

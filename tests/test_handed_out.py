@@ -61,3 +61,24 @@ def test_gradients_may_be_changed_in_place(sample):
     kept = grads[0][0].clone()
     grads[0][0].add_(weight)                # a penalty's share, recorded by autograd
     assert torch.equal(grads[0][0].detach(), kept + 1) and not grads[0][1].requires_grad
+
+
+@pytest.mark.gpu
+def test_profile_counts_the_kernels_of_its_phases(sample):
+    ctx, dense = sample
+    model = ctx.model(inputs.random_bias_layers([12, 16, 4], seed=53))
+    out = torch.empty((139, 4), device="cuda")
+    rel = torch.ones((3, 4), device="cuda")
+    lp = ctx.lp_prepare(torch.arange(40), torch.zeros(40), torch.arange(40, 80), 2, 20, seed=1)
+    rows = torch.ones((lp.targets().numel(), 4), device="cuda")
+    ctx.profile(True)
+    ctx.profile_read(reset=True)
+    before = ctx.kernel_launches()
+    ctx.sample_many(torch.arange(139, dtype=torch.int32), [0, 139], [3, 5], [1], out=dense)
+    dense.export_many()
+    ctx.forward(model, dense, out)
+    ctx.distmult_score(lp, rows, rel)
+    phases = ctx.profile_read(reset=True)
+    ctx.profile(False)
+    assert sum(p["launches"] for p in phases.values()) == ctx.kernel_launches() - before
+    assert all(p["launches"] for name, p in phases.items() if name != "gemm")      # (no phase that nothing enters; these layers need no separate product)
