@@ -95,9 +95,10 @@ def _pieces(block: torch.Tensor, sizes):
 
 def _fanouts(fanouts):
     values = [int(f) for f in fanouts]
-    if any(not -2 ** 31 <= f < 2 ** 31 for f in values):     # (a C array takes the low 32 bits of anything)
+    array = (C.c_int32 * len(values))(*values)
+    if array[:] != values:                       # (a C array takes the low 32 bits of anything)
         raise OverflowError("a fanout does not fit 32 bits")
-    return (C.c_int32 * len(values))(*values)
+    return array
 
 
 def _host(x, dtype) -> torch.Tensor:

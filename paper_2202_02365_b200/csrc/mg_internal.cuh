@@ -374,12 +374,14 @@ static inline void mg_reads_free(QueuedReads* r) {
 enum HostMemory { HOST_PAGEABLE, HOST_PINNED, HOST_MAPPED };
 static inline HostMemory mg_host_memory(const void* p, size_t bytes, const void** mapped) {
     cudaPointerAttributes first, last;
+    if (cudaPointerGetAttributes(&first, p) != cudaSuccess) { cudaGetLastError(); return HOST_PINNED; }
+    if (first.type == cudaMemoryTypeUnregistered) return HOST_PAGEABLE;
     const char* end = static_cast<const char*>(p) + (bytes ? bytes - 1 : 0);
-    if (cudaPointerGetAttributes(&first, p) != cudaSuccess || cudaPointerGetAttributes(&last, end) != cudaSuccess) { cudaGetLastError(); return HOST_PINNED; }
-    if (first.type == cudaMemoryTypeUnregistered && last.type == cudaMemoryTypeUnregistered) return HOST_PAGEABLE;
-    if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer ||
-        static_cast<const char*>(last.devicePointer) - static_cast<const char*>(first.devicePointer) != end - static_cast<const char*>(p))
+    if (first.type != cudaMemoryTypeHost || !first.devicePointer || cudaPointerGetAttributes(&last, end) != cudaSuccess || last.type != cudaMemoryTypeHost ||
+        static_cast<const char*>(last.devicePointer) - static_cast<const char*>(first.devicePointer) != end - static_cast<const char*>(p)) {
+        cudaGetLastError();
         return HOST_PINNED;
+    }
     *mapped = first.devicePointer;
     return HOST_MAPPED;
 }

@@ -636,7 +636,7 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     // (edges in pinned memory may be the destination of a copy that is still queued on the context's stream)
     const void* mapped;
     for (const int32_t* p : {src, rel, dst})
-        if (mg_host_memory(p, 4 * (size_t)n_edges, &mapped) != HOST_PAGEABLE) {
+        if (mg_host_memory(p, 0, &mapped) != HOST_PAGEABLE) {
             if (cudaEventRecord(ctx->ev_user, ctx->stream) == cudaSuccess) cudaStreamWaitEvent(st, ctx->ev_user);
             break;
         }
