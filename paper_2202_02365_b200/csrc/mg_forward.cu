@@ -1488,7 +1488,8 @@ struct EmbSgdArgs {
 // the gradient rows coming in and the reductions in L2: a warp looks `group` consecutive rows up at once (lane = row: a
 // binary search and two look-ups per row otherwise stood between any two rows), then reads four rows ahead of their
 // 16-byte reductions (1.56M rows x 128 onto 2M nodes: 538 -> 294 us against a row and 4-byte reductions at a time).
-__global__ void __launch_bounds__(kThreads) k_embedding_sgd(EmbSgdArgs a, int group, bool aligned) {
+// (A borrowed table or the caller's gradient rows may start anywhere: then 4 bytes at a time.)
+__global__ void __launch_bounds__(kThreads) k_embedding_sgd(EmbSgdArgs a, int group, bool grad_aligned, bool table_aligned) {
     const int lane = threadIdx.x & 31;
     const int n4 = a.dim / 4;
     const int64_t warps = (int64_t)gridDim.x * (kThreads / 32);
@@ -1508,14 +1509,16 @@ __global__ void __launch_bounds__(kThreads) k_embedding_sgd(EmbSgdArgs a, int gr
                     v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (r + u >= n || c >= n4) continue;
                     const float* g = a.grad + (s0 + r + u) * a.dim + 4 * c;
-                    v[u] = aligned ? __ldcs(reinterpret_cast<const float4*>(g)) : make_float4(g[0], g[1], g[2], g[3]);
+                    v[u] = grad_aligned ? __ldcs(reinterpret_cast<const float4*>(g)) : make_float4(g[0], g[1], g[2], g[3]);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int64_t row = __shfl_sync(0xFFFFFFFFu, at, min(r + u, 31));
-                    if (v[u].x != 0.f || v[u].y != 0.f || v[u].z != 0.f || v[u].w != 0.f)
-                        atomicAdd(reinterpret_cast<float4*>(a.slots + row * a.row_bytes) + c,
-                                  make_float4(-a.lr * v[u].x, -a.lr * v[u].y, -a.lr * v[u].z, -a.lr * v[u].w));
+                    if (v[u].x == 0.f && v[u].y == 0.f && v[u].z == 0.f && v[u].w == 0.f) continue;
+                    const float4 step = make_float4(-a.lr * v[u].x, -a.lr * v[u].y, -a.lr * v[u].z, -a.lr * v[u].w);
+                    float* dst = reinterpret_cast<float*>(a.slots + row * a.row_bytes) + 4 * c;
+                    if (table_aligned) atomicAdd(reinterpret_cast<float4*>(dst), step);
+                    else { atomicAdd(dst, step.x); atomicAdd(dst + 1, step.y); atomicAdd(dst + 2, step.z); atomicAdd(dst + 3, step.w); }
                 }
             }
     }
@@ -1540,7 +1543,8 @@ extern "C" int mg_apply_embedding_sgd(mg_ctx* ctx, mg_dense* d, const float* d_h
         while (group < 32 && a.n_rows > (int64_t)group * mg_grid(ctx, 8) * (kThreads / 32)) group *= 2;
         const int64_t groups = (a.n_rows + group - 1) / group;
         const int blocks = (int)std::min<int64_t>(mg_grid(ctx, 8), (groups + kThreads / 32 - 1) / (kThreads / 32));
-        k_embedding_sgd<<<blocks, kThreads, 0, ctx->stream>>>(a, group, (reinterpret_cast<uintptr_t>(d_h0_dev) & 15) == 0);
+        k_embedding_sgd<<<blocks, kThreads, 0, ctx->stream>>>(a, group, reinterpret_cast<uintptr_t>(d_h0_dev) % 16 == 0,
+                                                              reinterpret_cast<uintptr_t>(ctx->slots) % 16 == 0);
         ctx->launches++;
     }
     // with host backing the updated slots go back to the host table when their partitions are evicted

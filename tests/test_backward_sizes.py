@@ -238,3 +238,27 @@ def test_row_gradients_over_the_output_gradient(precision, dims):
     got = torch.as_tensor(api._DeviceInts(w_self.value, want[0][0].numel()), device="cuda").view(torch.float32)
     for x, y in ((got, want[0][0].flatten()), (both, want_rows.flatten())):
         assert float((x - y).norm()) <= 1e-5 * float(y.norm())                    # (sums over rows meet in any order)
+
+
+# a table and gradient rows that start anywhere (the step reads and adds 16 bytes at a time where it may)
+@pytest.mark.parametrize("table_at,grad_at", [(0, 0), (1, 0), (0, 3), (2, 1)])
+@pytest.mark.parametrize("dim", [4, 132])
+def test_base_rows_step_at_any_alignment(table_at, grad_at, dim):
+    graph = star_graph()
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    table = torch.zeros(N * dim + 4, device="cuda")[table_at:table_at + N * dim].view(N, dim)
+    table.copy_(inputs.normal_features(N, dim, seed=4, device="cuda"))
+    before = table.clone()
+    ctx.load_features(table)
+    sizes = [300, 0, 20]
+    targets = torch.cat([inputs.distinct_targets(N, s, seed=8 + i) for i, s in enumerate(sizes)])
+    dense = ctx.sample_many(targets, np.concatenate([[0], np.cumsum(sizes)]), [6, 4], [1, 2, 3])
+    rows = int(dense.counts()[0].sum())
+    grad = torch.zeros(rows * dim + 4, device="cuda")[grad_at:grad_at + rows * dim].view(rows, dim)
+    grad.copy_(torch.randn((rows, dim), generator=torch.Generator("cuda").manual_seed(5), device="cuda"))
+    ids = torch.empty(rows, dtype=torch.int32, device="cuda")
+    ctx._check(ctx.lib.mg_dense_packed_ids(ctx.handle, dense.handle, ctypes.c_void_p(ids.data_ptr())))
+    ctx.apply_embedding_sgd(dense, grad, 0.25)
+    want = before.double().index_add(0, ids.long(), grad.double(), alpha=-0.25)
+    assert float((table.double() - want).abs().max()) <= 4 * 2 ** -24 * 8      # (a handful of fp32 sums of magnitude below 8)
