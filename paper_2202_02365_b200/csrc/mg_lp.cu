@@ -705,7 +705,8 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
     cudaStream_t st = ctx->stream;
     ProfScope ps(ctx, PH_DISTMULT);
-    const bool tensor = gemm_precision == MG_GEMM_TF32 && dim % 4 == 0 && dim <= 32 * kTcMaxSlices && lp->negs > 0;
+    // (with no side corrupted there is nothing for the tensor cores, and the relations' rows may start anywhere)
+    const bool tensor = gemm_precision == MG_GEMM_TF32 && dim % 4 == 0 && dim <= 32 * kTcMaxSlices && lp->negs > 0 && (corrupt & MG_CORRUPT_BOTH);
     if (!tensor) {
         k_distmult_pos<<<mg_grid(ctx, 8), kThreads, 0, st>>>(h_dev, rel_emb_dev, lp->src_idx, lp->dst_idx, lp->rel, lp->n_edges, dim, pos_out);
         ctx->launches++;
@@ -761,10 +762,8 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
             ta.parts = left ? (int)std::min<int64_t>({4, n_blocks, ctx->n_sms / left}) : 1;
             ta.n_whole = (int32_t)(tiles - left);
             a.keep_idx = nullptr; a.out = nullptr; ta.base = a;
-            if (sides) {
-                k_distmult_neg_tc<<<(unsigned)(tiles - left + left * ta.parts), kTcThreads, smem, st>>>(ta);
-                ctx->launches++;
-            }
+            k_distmult_neg_tc<<<(unsigned)(tiles - left + left * ta.parts), kTcThreads, smem, st>>>(ta);
+            ctx->launches++;
         } else {
         dim3 grid((unsigned)(a.tiles_per_chunk * lp->n_chunks), (unsigned)((lp->negs + 63) / 64));
         if (corrupt & MG_CORRUPT_DST) {

@@ -118,3 +118,27 @@ def test_batches_prepared_beside_scores(sizes):
         lp.free()
         for x, y in zip(got[i], want):
             assert torch.equal(x, y), i
+
+
+# neither side corrupted: only the positives, from rows that may start anywhere
+@pytest.mark.parametrize("start", [0, 1])
+@pytest.mark.parametrize("precision", [mg.GEMM_TF32, mg.GEMM_FP32])
+def test_positive_scores_alone(start, precision):
+    nodes, dim, edges = 5_000, 36, 700
+    ctx = mg.Context(0)
+    g = inputs.erdos_renyi_graph(nodes, 2 * nodes, seed=1, device="cuda")
+    ctx.load_graph(g.row_offsets, g.nbrs)
+    rng = np.random.RandomState(4)
+    src, dst, rel = (torch.from_numpy(rng.randint(0, n, edges).astype(np.int32)) for n in (nodes, nodes, 50))
+    lp = ctx.lp_prepare(src, rel, dst, 2, 30, seed=5)
+    v = lp.view()
+
+    def rows(n, seed):
+        x = torch.zeros(n * dim + 4, device="cuda")[start:start + n * dim].view(n, dim)
+        return x.copy_(inputs.normal_features(n, dim, seed=seed, device="cuda"))
+
+    h, r = inputs.normal_features(v["targets"].numel(), dim, seed=6, device="cuda"), rows(50, 7)
+    pos, nd, ns = ctx.distmult_score(lp, h, r, 0, precision)
+    terms = h[v["src_idx"].long()].double() * r[rel.cuda().long()].double() * h[v["dst_idx"].long()].double()
+    assert nd is None and ns is None
+    assert float(((pos.double() - terms.sum(1)).abs() / terms.square().sum(1).sqrt()).max()) < 1e-5
