@@ -96,3 +96,36 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
     }
     return v;
 }
+
+// Single-pass scan over tiles (decoupled look-back): a 64-bit word per tile holds a tag (whose scan it belongs to; a word that was
+// cleared belongs to none), whether its count is the tile's own or the running total behind it, and the count.  Called by one warp of
+// the block that has the tile: publishes the tile's count, adds up what stands before it over windows of 32 tiles until one carries a
+// running total, publishes its own.  Returns what stands before the tile (`first` before tile 0).  Tiles come from a counter, so a tile's
+// predecessors are held by running blocks and every wait ends; the reads are bounded all the same, and *gave_up says when they ran out
+// (the count is then too small, and what is returned points into the range all the same).
+constexpr uint64_t kChainTag = 1ull << 34, kChainOwn = 1ull << 32, kChainTotal = 2ull << 32;
+constexpr int kChainPolls = 1 << 20;   // (a poll is an L2 round trip: far beyond any legitimate wait)
+__device__ __forceinline__ uint32_t chain_tiles(uint64_t* states, int32_t tile, uint64_t tag, uint32_t first, uint32_t total, int max_polls, bool* gave_up) {
+    const int lane = threadIdx.x & 31;
+    volatile uint64_t* state = states;
+    uint32_t before = first;
+    if (tile > 0) {
+        if (lane == 0) state[tile] = tag | kChainOwn | total;
+        before = 0;
+        for (int32_t top = tile - 1; top >= 0; top -= 32) {
+            const int32_t at = top - lane;
+            uint64_t s = tag | kChainOwn;   // (before tile 0: nothing)
+            if (at >= 0) {
+                int polls = 0;
+                while (((s = state[at]) >> 34 != tag >> 34) && ++polls < max_polls) {}
+                if (polls >= max_polls) { *gave_up = true; s = tag | kChainTotal; }
+            }
+            const uint32_t full = __ballot_sync(0xFFFFFFFFu, (s & kChainTotal) != 0);
+            const int stop = full ? __ffs(full) - 1 : 31;
+            before += __reduce_add_sync(0xFFFFFFFFu, lane <= stop ? (uint32_t)s : 0u);
+            if (full) break;
+        }
+    }
+    if (lane == 0) state[tile] = tag | kChainTotal | (before + total);
+    return before;
+}

@@ -958,19 +958,17 @@ __global__ void __launch_bounds__(kThreads) k_rev_entries(RevArgs a) {
 }
 
 // exclusive scan of the counts in place, the total behind them; the rows with long lists are cut into units on the way.
-// Tiles come from a counter, so a tile's predecessors are held by running blocks; the polls are bounded all the same.
-constexpr int kRevTile = kThreads * 16, kRevPolls = 1 << 20;   // (a poll is an L2 round trip: far beyond any legitimate wait)
+constexpr int kRevTile = kThreads * 16;
 __global__ void __launch_bounds__(kThreads) k_rev_scan(RevArgs a) {
     __shared__ uint32_t part[kThreads / 32];
     __shared__ uint32_t sh_before;
-    __shared__ int64_t sh_tile;
+    __shared__ int32_t sh_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n = a.in_at[a.g.k + 1], n_tiles = (n + kRevTile - 1) / kRevTile;
-    constexpr uint64_t kSum = 1ull << 62, kTotal = 2ull << 62;
-    if (threadIdx.x == 0) sh_tile = atomicAdd(a.ticket, 1u);   // (a block per tile)
+    if (threadIdx.x == 0) sh_tile = (int32_t)atomicAdd(a.ticket, 1u);   // (a block per tile)
     __syncthreads();
-    const int64_t tile = sh_tile;
-    const int64_t t0 = tile * kRevTile + (int64_t)threadIdx.x * 16;   // 16 consecutive elements per thread
+    const int32_t tile = sh_tile;
+    const int64_t t0 = (int64_t)tile * kRevTile + (int64_t)threadIdx.x * 16;   // 16 consecutive elements per thread
     uint32_t v[16], s = 0, my_units = 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {   // (the counts start on a 16-byte boundary)
@@ -993,24 +991,10 @@ __global__ void __launch_bounds__(kThreads) k_rev_scan(RevArgs a) {
         const uint32_t wi = warp_incl_scan(w);
         const uint32_t total = __shfl_sync(0xFFFFFFFFu, wi, 31);
         if (lane < kThreads / 32) part[lane] = wi - w;
-        volatile uint64_t* state = a.state;
-        uint32_t before = 0;
-        if (tile > 0 && lane == 0) state[tile] = kSum | total;
-        for (int64_t top = tile - 1; top >= 0; top -= 32) {
-            const int64_t at = top - lane;
-            uint64_t st = kSum;   // (before tile 0: nothing)
-            if (at >= 0) {
-                int polls = 0;
-                while ((st = state[at]) == 0 && ++polls < a.polls) {}
-                if (polls >= a.polls) { *a.bad = 1u; *reinterpret_cast<volatile uint32_t*>(a.status) = MG_ROLE_REV_SCAN; st = kTotal; }
-            }
-            const uint32_t full = __ballot_sync(0xFFFFFFFFu, (st & kTotal) != 0);
-            const int stop = full ? __ffs(full) - 1 : 31;
-            before += __reduce_add_sync(0xFFFFFFFFu, lane <= stop ? (uint32_t)st : 0u);
-            if (full) break;
-        }
+        bool gave_up = false;
+        const uint32_t before = chain_tiles(a.state, tile, kChainTag, 0u, total, a.polls, &gave_up);
+        if (gave_up) { *a.bad = 1u; *reinterpret_cast<volatile uint32_t*>(a.status) = MG_ROLE_REV_SCAN; }
         if (lane == 0) {
-            state[tile] = kTotal | (before + total);
             sh_before = before;
             if (tile == n_tiles - 1) a.cnt[n] = before + total;
         }
@@ -1322,7 +1306,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         ra.units = ctx->bw_rev + ent_total;
         ra.bad = ra.n_units + MG_MAX_HOPS + 1;
         const char* polls = getenv("MG_REV_POLLS");
-        ra.polls = polls ? atoi(polls) : kRevPolls;
+        ra.polls = polls ? atoi(polls) : kChainPolls;
         ra.status = ctx->d_flags;
         for (int l = ra.l0; l <= k; ++l) { ra.g_in[l] = l > 1 ? ctx->bw_g + g_off[l - 1] : d_h0_dev; ra.d_in[l] = m->dims[l - 1]; }
         MG_CUDA(ctx, cudaMemsetAsync(ctx->bw_off, 0, sizeof(uint32_t) * cleared, st));

@@ -46,9 +46,8 @@ k_lp_mark(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int6
     }
 }
 
-// One pass over the bitmap (8 words per thread): set bits are counted, the tiles' running totals chained through a 64-bit state each
-// (decoupled look-back; tiles come from a counter, so that a tile's predecessors are held by running blocks, and the polls are
-// bounded), the set bits' ids written from their place on, and the count before every word that holds any kept.  Bound by launch
+// One pass over the bitmap (8 words per thread): set bits are counted, the tiles' running totals chained (chain_tiles), the
+// set bits' ids written from their place on, and the count before every word that holds any kept.  Bound by launch
 // and look-back latency: 8M nodes 7 us, where a population count, a three-kernel scan and a pass for the ids took 14 us and
 // four gaps.
 constexpr int kLpWords = kThreads * 8;   // words of a tile: 65,536 nodes
@@ -67,8 +66,6 @@ __global__ void __launch_bounds__(kThreads) k_lp_scan(LpScanArgs a) {
     __shared__ uint32_t sh_before;
     __shared__ int32_t sh_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr uint64_t kSum = 1ull << 62, kTotal = 2ull << 62;
-    constexpr int kPolls = 1 << 20;
     if (threadIdx.x == 0) sh_tile = (int32_t)atomicAdd(a.ticket, 1u);   // (a block per tile)
     __syncthreads();
     const int32_t tile = sh_tile;
@@ -86,24 +83,10 @@ __global__ void __launch_bounds__(kThreads) k_lp_scan(LpScanArgs a) {
         const uint32_t pi = warp_incl_scan(p);
         const uint32_t total = __shfl_sync(0xFFFFFFFFu, pi, 31);
         if (lane < kThreads / 32) part[lane] = pi - p;
-        volatile uint64_t* state = a.state;
-        uint32_t before = 0;
-        if (tile > 0 && lane == 0) state[tile] = kSum | total;
-        for (int32_t top = tile - 1; top >= 0; top -= 32) {   // windows of 32 tiles until one carries a running total
-            const int32_t at = top - lane;
-            uint64_t st = kSum;   // (before tile 0: nothing)
-            if (at >= 0) {
-                int polls = 0;
-                while ((st = state[at]) == 0 && ++polls < kPolls) {}
-                if (polls >= kPolls) { atomicOr(a.status, ST_INTERNAL); st = kTotal; }
-            }
-            const uint32_t full = __ballot_sync(0xFFFFFFFFu, (st & kTotal) != 0);
-            const int stop = full ? __ffs(full) - 1 : 31;
-            before += __reduce_add_sync(0xFFFFFFFFu, lane <= stop ? (uint32_t)st : 0u);
-            if (full) break;
-        }
+        bool gave_up = false;
+        const uint32_t before = chain_tiles(a.state, tile, kChainTag, 0u, total, kChainPolls, &gave_up);
+        if (gave_up) atomicOr(a.status, ST_INTERNAL);
         if (lane == 0) {
-            state[tile] = kTotal | (before + total);
             sh_before = before;
             if (tile == a.n_tiles - 1) *a.n_targets = (int32_t)(before + total);
         }

@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kThreads) k_begin(BeginArgs a) {
 // between them (one mini-batch of three hops on 1M nodes: 48 -> 32 us; 128 mini-batches, last hop of 2.7M nodes: 315 -> 288
 // us).  A tile has as few nodes as keeps five blocks per SM busy (hop_tile): the picks of a warp's nodes are one chain after
 // the other, and a hop of 1,000 nodes took 21 us with 256 of them per block, 10 us with 32.  Tiles are handed out by a
-// counter, so a tile's predecessors are always held by running blocks and every wait ends; the polls are bounded all the same.
+// counter, as chain_tiles wants it.
 // Hop 0 also enters the targets: residency and range checks, the id table (Algorithm 1 wants unique targets).
 struct HopArgs {
     DenseHeader* hdr;
@@ -191,7 +191,6 @@ struct HopArgs {
     FeatGeom feat;
 };
 
-constexpr uint64_t kTileSum = 1ull << 32, kTileTotal = 2ull << 32;   // a tile's own count / the running total behind it
 // Nodes of a tile.  Below 256 as few as give five blocks (what the registers allow) on each of 148 SMs a tile; above 256
 // where twelve tiles per SM are left all the same: the chain through the tiles costs about 13 ns each (2.7M nodes: 620 us with
 // tiles of 64, 475 with 128, 342 with 256, 288 with 1,024).
@@ -207,7 +206,6 @@ __host__ __device__ __forceinline__ int hop_tile(int64_t n) {
 }
 // shared memory per node of a tile: id, mini-batch, first entry; first edge and length of its row, once per direction
 __host__ __device__ __forceinline__ int hop_node_bytes(bool inout) { return 12 + (inout ? 24 : 12); }
-constexpr int kTilePolls = 1 << 20;   // (a poll is an L2 round trip: far beyond any legitimate wait)
 
 // the mini-batch of target i: a 32-way search of the warp for its first target, then a walk
 __device__ __forceinline__ int target_batch(const int32_t* __restrict__ off, int B, int32_t first, int32_t i) {
@@ -277,7 +275,7 @@ __global__ void __launch_bounds__(kThreads) k_hop(HopArgs a) {
     int32_t* node_id = reinterpret_cast<int32_t*>(node_deg + (inout ? 2 : 1) * a.tile_cap);
     int32_t* node_b = node_id + a.tile_cap;
     uint32_t* node_out = reinterpret_cast<uint32_t*>(node_b + a.tile_cap);
-    const uint64_t tag = (((uint64_t)a.hdr->epoch << 3) | (uint64_t)a.hop) << 34;
+    const uint64_t tag = (((uint64_t)a.hdr->epoch << 3) | (uint64_t)a.hop) * kChainTag;
     const int32_t* __restrict__ targets = reinterpret_cast<const int32_t*>(a.hdr->targets);
     for (;;) {
         __syncthreads();
@@ -333,29 +331,11 @@ __global__ void __launch_bounds__(kThreads) k_hop(HopArgs a) {
             const uint32_t wi = warp_incl_scan(w);
             const uint32_t total = __shfl_sync(0xFFFFFFFFu, wi, 31);
             if (lane < kTileParts) part[lane] = wi - w;
-            volatile uint64_t* state = a.tile_state;
-            uint32_t before = (uint32_t)a.hdr->ent_base[a.hop];
-            if (tile > 0) {
-                if (lane == 0) state[tile] = tag | kTileSum | total;
-                // look back over windows of 32 tiles until one carries a running total
-                before = 0;
-                for (int32_t top = tile - 1; top >= 0; top -= 32) {
-                    const int32_t at = top - lane;
-                    uint64_t s = tag | kTileSum;   // (before tile 0: nothing)
-                    if (at >= 0) {
-                        int polls = 0;
-                        while (((s = state[at]) >> 34 != tag >> 34) && ++polls < kTilePolls) {}
-                        if (polls >= kTilePolls) { atomicOr(&a.hdr->status, ST_INTERNAL); s = tag | kTileTotal; }
-                    }
-                    const uint32_t full = __ballot_sync(0xFFFFFFFFu, (s & kTileTotal) != 0);
-                    const int stop = full ? __ffs(full) - 1 : 31;
-                    before += __reduce_add_sync(0xFFFFFFFFu, lane <= stop ? (uint32_t)s : 0u);
-                    if (full) break;
-                }
-            }
+            bool gave_up = false;
+            const uint32_t before = chain_tiles(a.tile_state, tile, tag, (uint32_t)a.hdr->ent_base[a.hop], total, kChainPolls, &gave_up);
+            if (gave_up) atomicOr(&a.hdr->status, ST_INTERNAL);
             if (lane == 0) {
                 const uint32_t end = before + total;
-                state[tile] = tag | kTileTotal | end;
                 sh_before = before;
                 sh_end = end;
                 if ((int64_t)end > a.cap_entries) atomicOr(&a.hdr->status, ST_CAP_ENTRIES);
