@@ -904,7 +904,7 @@ __global__ void __launch_bounds__(256) k_grad_weights(const float* __restrict__ 
 // A source row receives the self part of its own output row and a share of the neighbour part of every output row that
 // aggregates it.  Instead of adding row by row with atomics (a read-modify-write of the target for every sampled
 // entry), the entries of all layers are first turned round -- for every source row the list of (output row, weight) that
-// name it: a count per source row, an exclusive scan, a fill; four launches for all layers together, as none of it depends on
+// name it: a count per source row, an exclusive scan, a fill; three kernels for all layers together, as none of it depends on
 // a gradient -- and a warp then sums a source row's contributions in registers and stores the row once, through the ReLU of
 // the layer below and into that layer's bias gradient on the way.
 constexpr int kGradLight = 8;     // a source row named by more entries than this is cut into units of its own

@@ -157,9 +157,7 @@ struct mg_ctx {
 
     QueuedReads array_reads;   // copies of mini-batches' arrays that mg_dense_arrays_copy queued on a caller's stream
 
-    // profiling
-    // link-prediction batches: scratch of mg_lp_prepare (grows, never shrinks) and one spare result block, so that a
-    // loop of prepare / free allocates nothing
+    // link-prediction batches: scratch of mg_lp_prepare (grows, never shrinks)
     char* lp_ws = nullptr; size_t lp_ws_bytes = 0;
     // blocks of freed link-prediction batches, for the next ones: two, so that a batch can be prepared while the scores of the one
     // before it are still being computed; `idle` is recorded on the context's stream when the batch is freed, `reads` stands for the
@@ -174,9 +172,10 @@ struct mg_ctx {
     const struct mg_model* last_fwd_model = nullptr; const struct mg_dense* last_fwd_dense = nullptr;   // what mg_backward may follow
     float* bw_g = nullptr; float* bw_x = nullptr; float* bw_dx = nullptr;   // mg_backward scratch
     size_t bw_g_elems = 0, bw_x_elems = 0, bw_dx_elems = 0;
-    uint32_t* bw_off = nullptr; int2* bw_rev = nullptr;   // mg_backward: the turned-round entries of a layer
+    uint32_t* bw_off = nullptr; int2* bw_rev = nullptr;   // mg_backward: the turned-round entries of all layers whose dX is handed down
     size_t bw_off_elems = 0, bw_rev_elems = 0;
     char* dm_images = nullptr; size_t dm_images_bytes = 0;   // TF32 operand images of the negatives (mg_distmult_score)
+    // profiling
     bool prof_on = false;
     bool sample_graphs = true;   // replay the sampler's launches from a CUDA graph
     ProfPhase prof[PH_COUNT];

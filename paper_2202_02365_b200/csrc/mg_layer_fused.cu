@@ -3,14 +3,15 @@
 //
 //     H^l[r] = act([ self_r | mean_r ] . [W_self ; W_nbr] + b)
 //
-// The [self | mean] operand never goes to global memory.  Producer warps gather the rows a tile of
-// 128 output rows needs (layer 1: base representations straight from the partition buffer; later
-// layers: rows of H^{l-1}), reduce each segment in entry order, round to TF32 and write 32-float
-// K slices directly into 128-byte-swizzled shared-memory stages.  One thread issues tcgen05.mma
-// kind::tf32 against weight slices that a TMA thread streams from L2 (no multicast); the fp32
-// accumulator lives in tensor memory, double-buffered so that the epilogue of one tile (bias,
-// ReLU, store) overlaps the gather and MMAs of the next.  Tiles are handed out round-robin in
-// packed row order, so all SMs work on the same mini-batch at a time and its rows stay in L2.
+// The [self | mean] operand never goes to global memory.  Two CTAs work as a pair; producer warps of each gather the
+// rows its tile of 128 output rows needs (64 in layers of few rows; layer 1: base representations straight from the
+// partition buffer; later layers: rows of H^{l-1}), reduce each segment in entry order, round to the operand's
+// precision (TF32, or fp16 over fp16 rows) and write 128-byte K slices directly into swizzled shared-memory stages.  One
+// thread of the pair issues tcgen05.mma (cta_group::2) against weights that stay in tensor memory, or against weight
+// slices that a TMA thread streams from L2 (no multicast); the fp32 accumulators of the tiles' halves live in tensor
+// memory, so that the epilogue of one (bias, ReLU, store) overlaps the gather and MMAs of the next.  Tiles are handed
+// out round-robin in packed row order, so all SMs work on the same mini-batch at a time and its rows stay in L2.
+// The same gather feeds the kernel of the weights' gradients (k_sage_grad_weights).
 // Every mbarrier wait is bounded; on a time-out the role records a code and stops.
 
 #include <cuda_fp16.h>
@@ -1025,8 +1026,7 @@ __global__ void __launch_bounds__(256) k_layer_rows(RowsArgs a, int4* __restrict
     }
 }
 
-// row-major [rows, K] fp16 matrix, boxes of 64 halves x box_rows, 128-byte swizzle, zero fill
-// the same matrix in boxes of 32 halves x 32 rows, not swizzled (the transposed epilogue's fp16 stores)
+// row-major [rows, K] fp16 matrix in boxes of 32 halves x 32 rows, not swizzled (the transposed epilogue's fp16 stores)
 static bool make_map_f16_box32(CUtensorMap* map, const void* base, int64_t rows, int K) {
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
@@ -1038,6 +1038,7 @@ static bool make_map_f16_box32(CUtensorMap* map, const void* base, int64_t rows,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+// the same in boxes of 64 halves x box_rows, 128-byte swizzle, zero fill
 static bool make_map_f16(CUtensorMap* map, const void* base, int64_t rows, int K, int box_rows) {
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;

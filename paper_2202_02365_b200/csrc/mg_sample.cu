@@ -2,13 +2,14 @@
 //
 // Layout kept on the device (hop-major, sampling order):
 //   nodes[]     hop 0 = the targets of all batches, hop h+1 = the deltas found from hop h,
-//               inside a hop batch after batch, inside a batch ascending id (targets: caller order)
+//               inside a hop batch after batch, inside a batch in the order found (targets: caller order)
 //   ent_off[]   for each sampled node its first entry in ent_nbrs / ent_repr (same order as nodes)
 //   ent_repr[]  the neighbour's LOCAL row: its position in the batch's node list taken in
 //               sampling order (targets first).  In that order the rows layer l needs are the
 //               prefix [0, N_l) of the batch, which is what Algorithm 2 achieves by cutting the
 //               front of node_ids in the paper's (reversed) order.
-// The paper's arrays are produced from this by mg_dense_view.
+// The paper's arrays, with ascending ids inside a delta, are produced from this by mg_dense_view and
+// mg_dense_export_many.
 //
 // Every kernel sizes itself from counters in device memory (DenseHeader), so a k-hop sample is
 // issued without a host round trip per hop; the host reads the header once at the end.
@@ -879,14 +880,13 @@ __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
 }
 
 // -------------------------------------------------------------------------------------
-// radix sort of the new-node list on bits [lo_bit, lo_bit + bits) of the composite key
+// radix sort of 64-bit keys on bits [lo_bit, lo_bit + bits), for the exports
 // -------------------------------------------------------------------------------------
 constexpr int kSortKeysPerThread = 16;
 constexpr int kSortTile = kThreads * kSortKeysPerThread;  // 4096
-constexpr int kRadixBits = 9;                              // 34 key bits (27 id + 7 batch) take four passes
+constexpr int kRadixBits = 9;                              // ids of up to 27 bits, sorted inside segments, take three passes
 constexpr int kBins = 1 << kRadixBits;
 constexpr int kBinsPerThread = kBins / kThreads;
-
 
 // A tile of a segmented sort: a run of at most kSortTile keys of one segment.  Its histogram sits with its segment's
 // (digit-major inside the segment), so that one exclusive scan over all histograms in segment order gives every
@@ -1986,7 +1986,7 @@ int mg_dense_batch_perm(mg_ctx* ctx, mg_dense* d, int b, const int32_t** perm, c
     const int grid = std::max(1, std::min(mg_grid(ctx, 4), (g.V + kThreads - 1) / kThreads));
     int res = 0;
     if (n > 0) {
-        SortParams* sp = (SortParams*)(d->scan_tmp + d->scan_tmp_elems - 8);   // tail of the scratch block, as in the sampler
+        SortParams* sp = (SortParams*)(d->scan_tmp + d->scan_tmp_elems - 8);   // tail of the scratch block, as in mg_dense_export_many
         SortParams h_sp;
         mg_sort_params_host(&h_sp, n);
         MG_CUDA(ctx, cudaMemcpyAsync(sp, &h_sp, sizeof(h_sp), cudaMemcpyHostToDevice, st));
