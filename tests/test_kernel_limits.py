@@ -22,7 +22,7 @@ static cudaError_t write_down(const void* kernel, cudaFuncAttribute, int) { ++as
 int mg_fail(mg_ctx*, int code, const char*, ...) { return code; }
 int mg_cuda_fail(mg_ctx*, cudaError_t, const char*) { return MG_ERR_CUDA; }
 void mg_prof_begin(mg_ctx*, int) {}
-void mg_prof_end(mg_ctx*, int, int) {}
+void mg_prof_end(mg_ctx*, int, int64_t) {}
 
 int main() {
     for (int round = 0; round < 2; ++round)
