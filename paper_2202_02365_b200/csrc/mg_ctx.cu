@@ -297,6 +297,7 @@ extern "C" int mg_create(mg_ctx** out, int device, void* stream) {
     c->stream = (cudaStream_t)stream;
     cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, device);
     if (c->n_sms <= 0) c->n_sms = 148;
+    c->smem_raised.reserve(64);   // (more kernels than have a raised limit: nothing grows it later)
     for (int i = 0; i < PH_COUNT; ++i) c->prof[i] = ProfPhase{kPhaseNames[i], 0.0, 0};
     // the sampling stream has the lowest priority: when a layer kernel and sampler kernels are both ready, the layer
     // kernel's blocks are placed first and the sampler's short blocks fill what is left of every SM

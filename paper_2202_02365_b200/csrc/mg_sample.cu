@@ -182,6 +182,7 @@ struct HopArgs {
     int64_t cap_entries;
     uint64_t* tile_state;
     int32_t tile_cap;             // nodes of a tile that the launch has shared memory for
+    int32_t n_sms;
     // hop 0
     int32_t B;
     const int32_t* tgt_off;
@@ -192,17 +193,17 @@ struct HopArgs {
     FeatGeom feat;
 };
 
-// Nodes of a tile.  Below 256 as few as give five blocks (what the registers allow) on each of 148 SMs a tile; above 256
+// Nodes of a tile.  Below 256 as few as give five blocks (what the registers allow) on each SM a tile; above 256
 // where twelve tiles per SM are left all the same: the chain through the tiles costs about 13 ns each (2.7M nodes: 620 us with
 // tiles of 64, 475 with 128, 342 with 256, 288 with 1,024).
-constexpr int kTilesWanted = 740, kTilesLarge = 1776, kTileMax = 1024, kTileSets = kTileMax / kThreads;
+constexpr int kTilesPerSm = 5, kTilesPerSmLarge = 12, kTileMax = 1024, kTileSets = kTileMax / kThreads;
 constexpr int kTileParts = kTileSets * kThreads / 32;
 static_assert(kTileParts <= 32, "one warp scans the tile's warp totals");
-__host__ __device__ __forceinline__ int hop_tile(int64_t n) {
+__host__ __device__ __forceinline__ int hop_tile(int64_t n, int n_sms) {
     for (int t = 32; t < kThreads; t <<= 1)
-        if (n <= (int64_t)t * kTilesWanted) return t;
+        if (n <= (int64_t)t * kTilesPerSm * n_sms) return t;
     for (int t = kTileMax; t > kThreads; t >>= 1)
-        if (n > (int64_t)t * kTilesLarge) return t;
+        if (n > (int64_t)t * kTilesPerSmLarge * n_sms) return t;
     return kThreads;
 }
 // shared memory per node of a tile: id, mini-batch, first entry; first edge and length of its row, once per direction
@@ -269,7 +270,7 @@ __global__ void __launch_bounds__(kThreads) k_hop(HopArgs a) {
     const bool inout = a.row_off[1] != nullptr;
     const int32_t lo = a.hdr->hop_base[a.hop], n = a.hdr->hop_base[a.hop + 1] - lo;
     // (an empty hop has one empty tile: it closes the entry range)
-    const int32_t tile_nodes = min(hop_tile(n), a.tile_cap), n_tiles = max(1, (n + tile_nodes - 1) / tile_nodes);
+    const int32_t tile_nodes = min(hop_tile(n, a.n_sms), a.tile_cap), n_tiles = max(1, (n + tile_nodes - 1) / tile_nodes);
     const int sets = (tile_nodes + kThreads - 1) / kThreads;   // nodes per thread
     int64_t* node_r0 = reinterpret_cast<int64_t*>(hop_sm);                                      // [dirs][tile_cap]
     uint32_t* node_deg = reinterpret_cast<uint32_t*>(node_r0 + (inout ? 2 : 1) * a.tile_cap);   // [dirs][tile_cap]
@@ -1474,8 +1475,8 @@ static int dev_realloc(mg_ctx* ctx, T** p, size_t elems) {
     return MG_OK;
 }
 
-// tiles of a hop at most (tiles below 256 nodes: at most kTilesWanted)
-static size_t tile_states(int64_t cap_nodes) { return (size_t)cap_nodes / kThreads + kTilesWanted + 2; }
+// tiles of a hop at most (tiles below 256 nodes: at most five per SM)
+static size_t tile_states(const mg_ctx* ctx, int64_t cap_nodes) { return (size_t)cap_nodes / kThreads + (size_t)kTilesPerSm * ctx->n_sms + 2; }
 
 static int dense_alloc(mg_ctx* ctx, mg_dense* d, int32_t B, int32_t k, int64_t cap_nodes, int64_t cap_entries,
                        int32_t table_size, int32_t smem_nb) {
@@ -1489,7 +1490,7 @@ static int dense_alloc(mg_ctx* ctx, mg_dense* d, int32_t B, int32_t k, int64_t c
         if ((rc = dev_realloc(ctx, &d->nodes, (size_t)cap_nodes))) return rc;
         if ((rc = dev_realloc(ctx, &d->node_batch, (size_t)cap_nodes))) return rc;
         if ((rc = dev_realloc(ctx, &d->ent_off, (size_t)cap_nodes + 1))) return rc;
-        const size_t n_states = tile_states(cap_nodes);
+        const size_t n_states = tile_states(ctx, cap_nodes);
         if ((rc = dev_realloc(ctx, &d->tile_state, n_states))) return rc;
         MG_CUDA(ctx, cudaMemsetAsync(d->tile_state, 0, n_states * sizeof(uint64_t), ctx->stream));   // (no state carries epoch 0)
         d->epoch = 0;
@@ -1773,7 +1774,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     st_hdr->hop_base[0] = 0;
     st_hdr->hop_base[1] = (int32_t)T;
     if (++d->epoch >= 1u << 27) {   // (27 bits of a tile state's tag; a handle gets here after 134 million samples)
-        MG_CUDA(ctx, cudaMemsetAsync(d->tile_state, 0, tile_states(d->cap_nodes) * sizeof(uint64_t), st));
+        MG_CUDA(ctx, cudaMemsetAsync(d->tile_state, 0, tile_states(ctx, d->cap_nodes) * sizeof(uint64_t), st));
         d->epoch = 1;
     }
     st_hdr->epoch = d->epoch;
@@ -1825,7 +1826,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
             ProfScope ps(ctx, PH_SAMPLE_PICK);
             HopArgs a{d->hdr, h, f, d->nodes, d->node_batch, {ctx->view_off, inout ? ctx->view_off_out : nullptr},
                       {ctx->view_nbrs, ctx->view_nbrs_out}, d->ent_off, d->ent_nbrs, d->ent_repr, d->d_seeds, d->cap_entries, d->tile_state,
-                      hop_tile(nodes_bound[h]), B, d->node_off, d->hkeys, d->hvals, tg, ctx->n_nodes, mg_feat_geom(ctx)};
+                      hop_tile(nodes_bound[h], ctx->n_sms), ctx->n_sms, B, d->node_off, d->hkeys, d->hvals, tg, ctx->n_nodes, mg_feat_geom(ctx)};
             const unsigned grid = blocks_for(nodes_bound[h], 32, 8);
             const size_t sm = (size_t)a.tile_cap * hop_node_bytes(inout);   // 36 KiB at most
             // the narrowest group that holds the fanout among those that waste at most two lanes of a warp
