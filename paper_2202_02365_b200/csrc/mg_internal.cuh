@@ -216,13 +216,13 @@ struct mg_dense {
     int32_t* hkeys = nullptr;       // [B * table_size]
     int32_t* hvals = nullptr;       // [B * table_size]
     int32_t* new_ids = nullptr;     // [cap_entries] a hop's new ids by rank, a mini-batch's from the place of its first entry on
-    uint64_t* newlist[2] = {nullptr, nullptr};  // [cap_nodes] sort keys of an export
+    uint64_t* newlist[2] = {nullptr, nullptr};  // [cap_nodes] keys of an export
     uint64_t* d_seeds = nullptr;    // [B]
     int32_t* scan_tmp = nullptr;    // block sums
-    uint32_t* sort_hist = nullptr;  // radix histograms
+    uint32_t* sort_hist = nullptr;  // radix histograms; bins of an export
     size_t scan_tmp_elems = 0, sort_hist_elems = 0;
-    void* seg_tiles = nullptr;      // tile table of the export's sort inside (mini-batch, delta) segments
-    int64_t cap_sort_tiles = 0;     // tiles the sort scratch (histograms, block sums, tile table) is sized for
+    void* seg_tiles = nullptr;      // export: the (mini-batch, delta) segments and their tiles
+    int64_t cap_sort_tiles = 0;     // tiles the sort scratch (histograms, block sums, segment and tile tables) is sized for
     int64_t alloc_batches = 0, alloc_table = 0;
 
     // export buffer for mg_dense_view
@@ -415,6 +415,5 @@ void mg_sort_params_host(SortParams* sp, int64_t n);
 // caller's order; inv = its inverse).  Device arrays owned by d; on ctx->stream, synchronous, off the hot path.
 int mg_dense_batch_perm(mg_ctx* ctx, mg_dense* d, int b, const int32_t** perm, const int32_t** inv);
 void mg_sort_u64(mg_ctx* ctx, uint64_t* const buf[2], const SortParams* sp, int lo_bit, int bits, uint32_t* hist,
-                 uint32_t* scan_tmp, int* res_buf, const void* seg_tiles = nullptr);
-void mg_scan_u32(mg_ctx* ctx, uint32_t* data, const int32_t* lo, const int32_t* hi, const int32_t* base,
-                 uint32_t* scan_tmp, uint32_t* total_out);
+                 uint32_t* scan_tmp, int* res_buf);
+

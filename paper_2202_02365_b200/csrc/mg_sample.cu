@@ -881,37 +881,23 @@ __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
 }
 
 // -------------------------------------------------------------------------------------
-// radix sort of 64-bit keys on bits [lo_bit, lo_bit + bits), for the exports
+// radix sort of 64-bit keys on bits [lo_bit, lo_bit + bits), for the export of one mini-batch
 // -------------------------------------------------------------------------------------
 constexpr int kSortKeysPerThread = 16;
 constexpr int kSortTile = kThreads * kSortKeysPerThread;  // 4096
-constexpr int kRadixBits = 9;                              // ids of up to 27 bits, sorted inside segments, take three passes
+constexpr int kRadixBits = 9;
 constexpr int kBins = 1 << kRadixBits;
 constexpr int kBinsPerThread = kBins / kThreads;
 
-// A tile of a segmented sort: a run of at most kSortTile keys of one segment.  Its histogram sits with its segment's
-// (digit-major inside the segment), so that one exclusive scan over all histograms in segment order gives every
-// (segment, digit, tile) its place in the output, where segment follows segment.
-struct SegTile {
-    int32_t in0;      // first key of the tile in the input of the first pass (the segments lie elsewhere there)
-    int32_t out0;     // first key of the tile in every pass's output and the later passes' input
-    int32_t count;
-    int32_t hist0;    // index of the tile's count of digit 0
-    int32_t stride;   // distance between its counts of consecutive digits: the segment's tiles
-};
-
-// (tiles == nullptr: one segment, tile t = keys [t * kSortTile, ...), histograms digit-major over all tiles)
 __global__ void __launch_bounds__(kThreads)
-k_radix_hist(const uint64_t* __restrict__ keys, const SortParams* sp, int shift, uint32_t* hist,
-             const SegTile* __restrict__ tiles, bool first_pass) {
+k_radix_hist(const uint64_t* __restrict__ keys, const SortParams* sp, int shift, uint32_t* hist) {
     __shared__ uint32_t sh[kBins];
     const int32_t n = sp->n, ntiles = sp->ntiles;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
 #pragma unroll
         for (int q = 0; q < kBinsPerThread; ++q) sh[threadIdx.x + q * kThreads] = 0;
         __syncthreads();
-        int32_t tb = t * kSortTile, tn = min(kSortTile, n - tb), h0 = t, hs = ntiles;
-        if (tiles) { const SegTile st = tiles[t]; tb = first_pass ? st.in0 : st.out0; tn = st.count; h0 = st.hist0; hs = st.stride; }
+        const int32_t tb = t * kSortTile, tn = min(kSortTile, n - tb);
 #pragma unroll 4
         for (int j = 0; j < kSortKeysPerThread; ++j) {
             const int32_t l = j * kThreads + threadIdx.x;
@@ -921,7 +907,7 @@ k_radix_hist(const uint64_t* __restrict__ keys, const SortParams* sp, int shift,
 #pragma unroll
         for (int q = 0; q < kBinsPerThread; ++q) {
             const int bin = threadIdx.x + q * kThreads;
-            hist[(size_t)h0 + (size_t)bin * hs] = sh[bin];
+            hist[(size_t)t + (size_t)bin * ntiles] = sh[bin];
         }
         __syncthreads();
     }
@@ -932,7 +918,7 @@ k_radix_hist(const uint64_t* __restrict__ keys, const SortParams* sp, int shift,
 // equal digits leaves the SM as consecutive addresses.
 __global__ void __launch_bounds__(kThreads)
 k_radix_scatter(const uint64_t* __restrict__ keys, uint64_t* __restrict__ out, const SortParams* sp, int shift,
-                const uint32_t* __restrict__ hist_scanned, const SegTile* __restrict__ tiles, bool first_pass) {
+                const uint32_t* __restrict__ hist_scanned) {
     extern __shared__ __align__(16) uint8_t sort_smem[];
     uint64_t* stage = reinterpret_cast<uint64_t*>(sort_smem);                          // [kSortTile]
     uint32_t (*cnt)[kBins] = reinterpret_cast<uint32_t (*)[kBins]>(stage + kSortTile);   // [warps][kBins]
@@ -950,8 +936,7 @@ k_radix_scatter(const uint64_t* __restrict__ keys, uint64_t* __restrict__ out, c
         __syncthreads();
         uint64_t key[kSortKeysPerThread];
         uint32_t rank[kSortKeysPerThread];
-        int32_t tb = t * kSortTile, tile_n = min(kSortTile, n - tb), h0 = t, hs = ntiles;
-        if (tiles) { const SegTile st = tiles[t]; tb = first_pass ? st.in0 : st.out0; tile_n = st.count; h0 = st.hist0; hs = st.stride; }
+        const int32_t tb = t * kSortTile, tile_n = min(kSortTile, n - tb);
         const int32_t wl = warp * kPerWarp;   // the warp's first key inside the tile
 #pragma unroll
         for (int r = 0; r < kSortKeysPerThread; ++r) {
@@ -989,7 +974,7 @@ k_radix_scatter(const uint64_t* __restrict__ keys, uint64_t* __restrict__ out, c
         for (int q = 0; q < kBinsPerThread; ++q) {
             const int bin = threadIdx.x * kBinsPerThread + q;
             tile_base[bin] = before;
-            glob_base[bin] = hist_scanned[(size_t)h0 + (size_t)bin * hs];
+            glob_base[bin] = hist_scanned[(size_t)t + (size_t)bin * ntiles];
             before += mine[q];
         }
         __syncthreads();
@@ -1267,120 +1252,440 @@ __global__ void __launch_bounds__(kThreads) k_export_entries(ExportArgs a) {
 // -------------------------------------------------------------------------------------
 // export of every mini-batch at once (mg_dense_export_many): the canonical DENSE ordering for the whole sample
 // -------------------------------------------------------------------------------------
-// One sort orders all nodes of the sample by (mini-batch, delta, id); a node's position in that order is its row in
-// the packed canonical node list (mini-batch after mini-batch, each [Delta_0 .. Delta_k]).  Targets keep the caller's
-// order: their "id" field is their position.
+// A segment is a (mini-batch, delta) pair; in output order mini-batch follows mini-batch, inside it the farthest delta comes
+// first.  Its ids are distinct, so a node's place in it is the number of smaller ids.  The ids are split by their top bits
+// into bins -- counted per tile (k_export_count), written bin after bin in any order (k_export_split) --, and then ordered bin by bin
+// (k_export_order): a warp compares the ids of a bin of up to 128 all with all, a block takes a larger one through a bitmap of the
+// bin's range in shared memory, whose set bits below an id are its rank.  The same bins carry the sampled nodes' entry counts,
+// so that a node's place in the packed entries falls out of its place in the bin.  Targets keep the caller's order and take no part.
+// Bound by the latency of a few dependent passes over what stays in L2.  Before, a radix sort of three passes with a scan each, a kernel
+// for the order and a scan of all counts, 24 kernels: 310 us for 32 mini-batches of 114,000 nodes on a graph of 8M, now 175 us (begin 5,
+// count 16, split 31, order 76, entries 37, and their gaps).
+struct ExportSeg {
+    int32_t in0, len;        // its nodes in the arena
+    int32_t out0;            // its first row in the packed canonical node list
+    int32_t row0, lrow0;     // first packed row of the mini-batch; local row of the segment's first node in sampling order
+    int32_t hop, n_tiles;
+    int32_t bin0, bins, shift;   // bin of an id: bin0 + (id >> shift)
+    int32_t off_shift;       // canonical row c has its offset at o_nbr_off[c + off_shift]
+    int32_t ent_rel, ent0;   // its first entry in the mini-batch's packed entries, and where those start
+    uint32_t ticket;         // tiles that have been counted
+};
+struct ExportCounts { int32_t n_tiles, n_bins, n_dense; };
 struct ExportManyArgs {
-    int32_t B, k, n_nodes_total, pay_bits, id_bits;
+    int32_t B, k, id_bits, n_bins_max;
     int32_t hop_base[MG_MAX_HOPS + 2];
-    const int32_t *nodes, *node_batch, *node_off, *cum, *rowbase0, *ent_off, *ent_nbrs, *ent_repr;
-    int32_t *o_node_ids, *o_nio, *o_nbrs, *o_repr, *o_nbr_off, *inv;
-    uint32_t* cnt;   // per canonical row: entry count, then (scanned) its first entry in the packed entry list
+    const int32_t *nodes, *node_batch, *node_off, *cum, *rowbase0, *ent_hop, *ent_off, *ent_nbrs, *ent_repr;
+    int32_t *o_node_ids, *o_nio, *o_nbrs, *o_repr, *o_nbr_off;
+    int32_t* inv;            // per packed row in sampling order: the canonical row in the mini-batch
+    int32_t* ent_to;         // per sampled node (arena): its first entry in the packed entry list
+    ExportSeg* segs;         // [B (k + 1)]
+    int2* tiles;             // (segment, tile inside it)
+    ExportCounts* counts;
+    uint32_t* bin_end;       // per bin: nodes, then where the next one goes, at last where the bin ends
+    uint32_t* bin_ents;      // per bin: entries, then the bin's first in the mini-batch's packed entries
+    int32_t* bin_seg;
+    int2* keys;              // (id, local row in sampling order) in place of the packed rows, ordered by bin
+    int32_t* dense_bins;     // the bins of more than kExportWarpKeys nodes
 };
 
-__device__ __forceinline__ int hop_of_arena(const ExportManyArgs& a, int32_t i) {
-    int h = 0;
-    while (h < a.k && i >= a.hop_base[h + 1]) ++h;
-    return h;
+constexpr int kExportBinsLog = 9;      // bins of a segment at most
+constexpr int kExportWarpKeys = 128;   // keys that a warp compares all with all
+constexpr int kExportPairKeys = 1024;  // ... and a block, where the bin's range takes more than one bitmap
+constexpr int kExportMapLog = 17;      // ids of a bitmap
+static_assert((1 << kExportBinsLog) == 2 * kThreads, "two bins per thread");
+
+// bins of a segment: a power of two that gives them 32 to 64 nodes on average (more in the longest segments); none where nothing
+// is to be ordered
+__device__ __forceinline__ int export_bins_log(int32_t len, int id_bits) {
+    const int want = len <= 64 ? 0 : 32 - __clz((len - 1) >> 6);
+    return min(want, min(kExportBinsLog, id_bits));
 }
 
-// The segments of the export's sort in output order -- mini-batch after mini-batch, inside it the farthest delta
-// first -- cut into tiles: where a tile's keys lie in the arenas (hop-major), where in the output, and where its
-// histogram goes.  One block; also the sort's parameters and the range of the entry-count scan.
-__global__ void __launch_bounds__(1024) k_export_tiles(ExportManyArgs a, SegTile* tiles, SortParams* sp, int32_t* range) {
-    __shared__ int32_t warp_t[32], warp_n[32];
-    __shared__ int32_t carry_t, carry_n;
+// Block 0: the segments in output order and their tiles.  The others: bins to zero, and what is known of every mini-batch.
+__global__ void __launch_bounds__(1024) k_export_begin(ExportManyArgs a) {
+    const int32_t k = a.k, B = a.B;
+    auto entries = [&](int32_t b, int32_t h) { return a.ent_hop[h * (B + 1) + b + 1] - a.ent_hop[h * (B + 1) + b]; };
+    if (blockIdx.x > 0) {
+        const int32_t step = (int32_t)(gridDim.x - 1) * 1024, t0 = (int32_t)(blockIdx.x - 1) * 1024 + (int32_t)threadIdx.x;
+        for (int32_t i = t0; i < 2 * a.n_bins_max; i += step) a.bin_end[i] = 0u;   // (bin_ents follows)
+        for (int32_t b = t0; b < B; b += step) {
+            const int32_t* cum = a.cum + (int64_t)b * (k + 2);
+            int32_t run = 0, ents = 0;
+            a.o_nio[(int64_t)b * (k + 2)] = 0;
+            for (int j = 0; j <= k; ++j) { run += cum[k - j + 1] - cum[k - j]; a.o_nio[(int64_t)b * (k + 2) + j + 1] = run; }
+            for (int h = 0; h < k; ++h) ents += entries(b, h);
+            a.o_nbr_off[a.rowbase0[b] + b + cum[k]] = ents;   // the terminal entry, behind the sampled nodes'
+        }
+        return;
+    }
+    __shared__ int32_t warp_sum[3][32];
+    __shared__ int32_t carry[3];   // tiles, nodes, bins
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) { carry_t = 0; carry_n = 0; }
+    if (threadIdx.x < 3) carry[threadIdx.x] = 0;
     __syncthreads();
-    const int32_t n_seg = a.B * (a.k + 1);
+    const int32_t n_seg = B * (k + 1);
     for (int32_t s0 = 0; s0 < n_seg; s0 += 1024) {
-        const int32_t s = s0 + (int32_t)threadIdx.x;
-        int32_t in0 = 0, len = 0;
+        const int32_t s = s0 + (int32_t)threadIdx.x, b = s / (k + 1), h = k - s % (k + 1);
+        ExportSeg g;
+        g.in0 = 0; g.len = 0; g.bins = 0; g.shift = 0;
         if (s < n_seg) {
-            const int32_t b = s / (a.k + 1), h = a.k - s % (a.k + 1);
-            in0 = a.node_off[h * (a.B + 1) + b];
-            len = a.node_off[h * (a.B + 1) + b + 1] - in0;
+            g.in0 = a.node_off[h * (B + 1) + b];
+            g.len = a.node_off[h * (B + 1) + b + 1] - g.in0;
+            if (h > 0 && g.len > 0) {
+                const int lg = export_bins_log(g.len, a.id_bits);
+                g.bins = 1 << lg;
+                g.shift = a.id_bits - lg;
+            }
         }
-        const int32_t nt = (len + kSortTile - 1) / kSortTile;
-        const int32_t it = (int32_t)warp_incl_scan((uint32_t)nt), in = (int32_t)warp_incl_scan((uint32_t)len);
-        if (lane == 31) { warp_t[warp] = it; warp_n[warp] = in; }
-        __syncthreads();
-        int32_t t0 = carry_t + it - nt, o0 = carry_n + in - len;
-        for (int w = 0; w < warp; ++w) { t0 += warp_t[w]; o0 += warp_n[w]; }
-        for (int32_t t = 0; t < nt; ++t) {
-            SegTile st;
-            st.in0 = in0 + t * kSortTile;
-            st.out0 = o0 + t * kSortTile;
-            st.count = min(kSortTile, len - t * kSortTile);
-            st.hist0 = t0 * kBins + t;
-            st.stride = nt;
-            tiles[t0 + t] = st;
+        g.n_tiles = (g.len + kSortTile - 1) / kSortTile;
+        const int32_t mine[3] = {g.n_tiles, g.len, g.bins};
+        int32_t at[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int32_t inc = (int32_t)warp_incl_scan((uint32_t)mine[q]);
+            if (lane == 31) warp_sum[q][warp] = inc;
+            at[q] = inc - mine[q];
         }
         __syncthreads();
-        if (threadIdx.x == 1023) { carry_t = t0 + nt; carry_n = o0 + len; }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            at[q] += carry[q];
+            for (int w = 0; w < warp; ++w) at[q] += warp_sum[q][w];
+        }
+        __syncthreads();
+        if (threadIdx.x == 1023)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) carry[q] = at[q] + mine[q];
+        if (s < n_seg) {
+            const int32_t* cum = a.cum + (int64_t)b * (k + 2);
+            g.out0 = at[1];
+            g.row0 = a.rowbase0[b];
+            g.lrow0 = cum[h];
+            g.hop = h;
+            g.bin0 = at[2];
+            g.off_shift = b - (cum[k + 1] - cum[k]);
+            g.ent_rel = 0;
+            g.ent0 = 0;
+            for (int j = 0; j < k; ++j) {   // entries are packed mini-batch after mini-batch, inside one in the order of its nodes
+                g.ent0 += a.ent_hop[j * (B + 1) + b] - a.ent_hop[j * (B + 1)];
+                if (j > h) g.ent_rel += entries(b, j);
+            }
+            g.ticket = 0u;
+            a.segs[s] = g;
+            for (int32_t t = 0; t < g.n_tiles; ++t) a.tiles[at[0] + t] = make_int2(s, t);
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        sp->zero = 0; sp->n = a.n_nodes_total; sp->ntiles = carry_t; sp->hist_len = kBins * carry_t;
-        range[0] = 0; range[1] = a.n_nodes_total;
+    if (threadIdx.x == 0) { a.counts->n_tiles = carry[0]; a.counts->n_bins = carry[2]; a.counts->n_dense = 0; }
+}
+
+// Nodes and entries per bin; the block that counts a segment's last tile sums them up over its bins.
+__global__ void __launch_bounds__(kThreads) k_export_count(ExportManyArgs a) {
+    constexpr int kMaxBins = 1 << kExportBinsLog, kPer = kSortTile / kThreads;
+    __shared__ uint32_t cnt[kMaxBins], ents[kMaxBins], part[2][kThreads / 32];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t n_tiles = a.counts->n_tiles;
+    for (int32_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const int2 tile = a.tiles[t];
+        const ExportSeg g = a.segs[tile.x];
+        if (g.bins == 0) continue;   // (the whole block)
+        const bool sampled = g.hop < a.k;
+        __syncthreads();
+        for (int i = threadIdx.x; i < g.bins; i += kThreads) { cnt[i] = 0u; ents[i] = 0u; }
+        __syncthreads();
+        const int32_t i0 = g.in0 + tile.y * kSortTile, n = min(kSortTile, g.len - tile.y * kSortTile);
+        int32_t id[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) { const int32_t i = j * kThreads + (int32_t)threadIdx.x; id[j] = i < n ? a.nodes[i0 + i] : -1; }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) if (id[j] >= 0) atomicAdd(&cnt[id[j] >> g.shift], 1u);
+        if (sampled) {
+            uint32_t e[kPer];
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                const int32_t i = i0 + j * kThreads + (int32_t)threadIdx.x;
+                e[j] = id[j] >= 0 ? (uint32_t)(a.ent_off[i + 1] - a.ent_off[i]) : 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) if (e[j]) atomicAdd(&ents[id[j] >> g.shift], e[j]);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < g.bins; i += kThreads)
+            if (cnt[i]) {
+                atomicAdd(&a.bin_end[g.bin0 + i], cnt[i]);
+                if (ents[i]) atomicAdd(&a.bin_ents[g.bin0 + i], ents[i]);
+            }
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&a.segs[tile.x].ticket, 1u) == (uint32_t)g.n_tiles - 1u;
+        __syncthreads();
+        if (!last) continue;
+        __threadfence();
+        const int q0 = 2 * (int)threadIdx.x;   // two bins per thread
+        uint32_t c[2], e[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const bool on = q0 + q < g.bins;
+            c[q] = on ? __ldcg(&a.bin_end[g.bin0 + q0 + q]) : 0u;
+            e[q] = on ? __ldcg(&a.bin_ents[g.bin0 + q0 + q]) : 0u;
+        }
+        const uint32_t ci = warp_incl_scan(c[0] + c[1]), ei = warp_incl_scan(e[0] + e[1]);
+        if (lane == 31) { part[0][warp] = ci; part[1][warp] = ei; }
+        __syncthreads();
+        uint32_t c_at = (uint32_t)g.out0 + ci - c[0] - c[1], e_at = (uint32_t)g.ent_rel + ei - e[0] - e[1];
+        for (int w = 0; w < warp; ++w) { c_at += part[0][w]; e_at += part[1][w]; }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q0 + q >= g.bins) break;
+            const int32_t bin = g.bin0 + q0 + q;
+            a.bin_end[bin] = c_at;
+            a.bin_ents[bin] = e_at;
+            a.bin_seg[bin] = tile.x;
+            if (c[q] > (uint32_t)kExportWarpKeys) a.dense_bins[atomicAdd(&a.counts->n_dense, 1)] = bin;
+            c_at += c[q];
+            e_at += e[q];
+        }
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_export_keys(ExportManyArgs a, uint64_t* keys) {
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n_nodes_total; i += gridDim.x * blockDim.x) {
-        const int h = hop_of_arena(a, i);
-        const int32_t b = a.node_batch[i];
-        const uint32_t id = h == 0 ? (uint32_t)(i - a.node_off[b]) : (uint32_t)a.nodes[i];
-        keys[i] = ((uint64_t)id << a.pay_bits) | (uint64_t)(uint32_t)i;   // sorted inside its (mini-batch, delta) segment
-    }
-    // node_id_offsets of every mini-batch
-    for (int32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < a.B; t += gridDim.x * blockDim.x) {
-        const int32_t* cum = a.cum + (int64_t)t * (a.k + 2);
-        int32_t run = 0;
-        a.o_nio[(int64_t)t * (a.k + 2)] = 0;
-        a.o_nbr_off[a.rowbase0[t] + t] = 0;   // (an empty mini-batch has this terminal entry only)
-        for (int j = 0; j <= a.k; ++j) { run += cum[a.k - j + 1] - cum[a.k - j]; a.o_nio[(int64_t)t * (a.k + 2) + j + 1] = run; }
+// a node at its place: canonical row c of the packed list
+__device__ __forceinline__ void export_node(const ExportManyArgs& a, const ExportSeg& g, int32_t c, int32_t id, int32_t local) {
+    a.o_node_ids[c] = id;
+    a.inv[g.row0 + local] = c - g.row0;
+}
+// ... and its entries: the first one stands at `rel` of the mini-batch's
+__device__ __forceinline__ void export_offset(const ExportManyArgs& a, const ExportSeg& g, int32_t c, int32_t local, int32_t rel) {
+    a.o_nbr_off[c + g.off_shift] = rel;
+    a.ent_to[g.in0 + local - g.lrow0] = g.ent0 + rel;
+}
+
+// Every node to its bin (one global atomic per tile and bin); targets stay where they are.
+__global__ void __launch_bounds__(kThreads) k_export_split(ExportManyArgs a) {
+    constexpr int kMaxBins = 1 << kExportBinsLog, kPer = kSortTile / kThreads;
+    __shared__ uint32_t cnt[kMaxBins], base[kMaxBins];
+    const int32_t n_tiles = a.counts->n_tiles;
+    for (int32_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const int2 tile = a.tiles[t];
+        const ExportSeg g = a.segs[tile.x];
+        const int32_t first = tile.y * kSortTile, n = min(kSortTile, g.len - first);
+        if (g.bins == 0) {
+            for (int32_t i = threadIdx.x; i < n; i += kThreads) {
+                const int32_t at = g.in0 + first + i, local = g.lrow0 + first + i, c = g.out0 + first + i;
+                export_node(a, g, c, a.nodes[at], local);
+                if (g.hop < a.k) export_offset(a, g, c, local, g.ent_rel + a.ent_off[at] - a.ent_off[g.in0]);
+            }
+            continue;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < g.bins; i += kThreads) cnt[i] = 0u;
+        __syncthreads();
+        int32_t id[kPer];
+        uint32_t rank[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) { const int32_t i = j * kThreads + (int32_t)threadIdx.x; id[j] = i < n ? a.nodes[g.in0 + first + i] : -1; }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) rank[j] = id[j] >= 0 ? atomicAdd(&cnt[id[j] >> g.shift], 1u) : 0u;
+        __syncthreads();
+        for (int i = threadIdx.x; i < g.bins; i += kThreads) if (cnt[i]) base[i] = atomicAdd(&a.bin_end[g.bin0 + i], cnt[i]);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kPer; ++j)
+            if (id[j] >= 0) a.keys[base[id[j] >> g.shift] + rank[j]] = make_int2(id[j], g.lrow0 + first + j * kThreads + (int32_t)threadIdx.x);
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_export_place(ExportManyArgs a, const uint64_t* __restrict__ sorted) {
-    const uint64_t pay_mask = (1ull << a.pay_bits) - 1ull;
-    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < a.n_nodes_total; c += gridDim.x * blockDim.x) {
-        const uint64_t key = sorted[c];
-        const int32_t i = (int32_t)(key & pay_mask);
-        a.inv[i] = c;
-        // the key carries the node id (for the targets their position: they keep the caller's order)
-        a.o_node_ids[c] = i < a.hop_base[1] ? a.nodes[i] : (int32_t)((key >> a.pay_bits) & ((1ull << a.id_bits) - 1ull));
-        a.cnt[c] = i < a.hop_base[a.k] ? (uint32_t)(a.ent_off[i + 1] - a.ent_off[i]) : 0u;   // the farthest delta has no entries
+__global__ void __launch_bounds__(kThreads) k_export_order(ExportManyArgs a) {
+    constexpr int kWarps = kThreads / 32, kMapWords = (1 << kExportMapLog) / 32, kBinsPerWarp = 8;
+    __shared__ __align__(16) uint32_t map[kMapWords];   // a bitmap, or the ids of bins that are compared all with all
+    __shared__ uint16_t below[kMapWords];               // set bits before a word among those of its warp
+    __shared__ uint32_t warp_tot[kWarps];
+    static_assert(kWarps * kExportWarpKeys <= kMapWords && kExportPairKeys <= kMapWords, "ids fit the bitmap's place");
+    static_assert(kMapWords / kWarps * 32 <= 65536 && kMapWords % (32 * kWarps) == 0, "a warp's words");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t n_bins = a.counts->n_bins, n_dense = a.counts->n_dense;
+    auto bin_start = [&](const ExportSeg& g, int32_t bin) { return bin == g.bin0 ? g.out0 : (int32_t)a.bin_end[bin - 1]; };
+    // large bins: a block each
+    for (int32_t w = blockIdx.x; w < n_dense; w += gridDim.x) {
+        const int32_t bin = a.dense_bins[w];
+        const ExportSeg g = a.segs[a.bin_seg[bin]];
+        const int32_t start = bin_start(g, bin), n = (int32_t)a.bin_end[bin] - start;
+        const int2* __restrict__ keys = a.keys + start;
+        const bool sampled = g.hop < a.k;
+        if (n <= kExportPairKeys && g.shift > kExportMapLog) {
+            constexpr int kPer = kExportPairKeys / kThreads;
+            __syncthreads();
+            int2 key[kPer];
+            int32_t rank[kPer];
+#pragma unroll
+            for (int r = 0; r < kPer; ++r) {
+                const int i = r * kThreads + (int)threadIdx.x;
+                key[r] = i < n ? keys[i] : make_int2(INT32_MAX, 0);
+                rank[r] = 0;
+                map[i] = (uint32_t)key[r].x;
+            }
+            __syncthreads();
+            for (int i = 0; i < n; i += 4) {
+                const int4 v = *reinterpret_cast<const int4*>(&map[i]);
+#pragma unroll
+                for (int r = 0; r < kPer; ++r) rank[r] += (v.x < key[r].x) + (v.y < key[r].x) + (v.z < key[r].x) + (v.w < key[r].x);
+            }
+#pragma unroll
+            for (int r = 0; r < kPer; ++r)
+                if (r * kThreads + (int)threadIdx.x < n) {
+                    export_node(a, g, start + rank[r], key[r].x, key[r].y);
+                    if (sampled) a.o_nbr_off[start + rank[r] + g.off_shift] = key[r].y;   // (until the counts are summed up below)
+                }
+        } else {
+            const int map_log = max(5, min(g.shift, kExportMapLog));
+            const int words = 1 << (map_log - 5), warp_words = max(32, words / kWarps);
+            const int32_t id0 = (bin - g.bin0) << g.shift;
+            uint32_t before = 0;   // ids in the bitmaps so far
+            for (int64_t sub = 0; sub < 1ll << g.shift; sub += 1ll << map_log) {
+                __syncthreads();
+                for (int i = threadIdx.x; i < words; i += kThreads) map[i] = 0u;
+                __syncthreads();
+                for (int32_t i = threadIdx.x; i < n; i += kThreads) {
+                    const int64_t at = (int64_t)(keys[i].x - id0) - sub;
+                    if (at >= 0 && at < 1ll << map_log) atomicOr(&map[at >> 5], 1u << (at & 31));
+                }
+                __syncthreads();
+                uint32_t run = 0;
+                for (int i = warp * warp_words + lane; i < min(words, (warp + 1) * warp_words) + lane; i += 32) {
+                    const uint32_t c = i < words ? (uint32_t)__popc(map[i]) : 0u;
+                    const uint32_t inc = warp_incl_scan(c);
+                    if (i < words) below[i] = (uint16_t)(run + inc - c);
+                    run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+                }
+                if (lane == 0) warp_tot[warp] = run;
+                __syncthreads();
+                for (int32_t i = threadIdx.x; i < n; i += kThreads) {
+                    const int2 key = keys[i];
+                    const int64_t at = (int64_t)(key.x - id0) - sub;
+                    if (at < 0 || at >= 1ll << map_log) continue;
+                    const int wd = (int)(at >> 5);
+                    uint32_t rank = before + below[wd] + (uint32_t)__popc(map[wd] & ((1u << (at & 31)) - 1u));
+                    for (int q = 0; q < wd / warp_words; ++q) rank += warp_tot[q];
+                    export_node(a, g, start + (int32_t)rank, key.x, key.y);
+                    if (sampled) a.o_nbr_off[start + (int32_t)rank + g.off_shift] = key.y;
+                }
+                for (int q = 0; q < kWarps; ++q) before += warp_tot[q];
+            }
+        }
+        if (!sampled) continue;
+        // in order now: the nodes' entry counts, summed up from the bin's first entry on
+        uint32_t run = a.bin_ents[bin];
+        for (int32_t i0 = 0; i0 < n; i0 += kThreads) {
+            __syncthreads();
+            const int32_t i = i0 + (int32_t)threadIdx.x, c = start + i;
+            int32_t local = 0;
+            uint32_t ents = 0;
+            if (i < n) {
+                local = a.o_nbr_off[c + g.off_shift];
+                const int32_t at = g.in0 + local - g.lrow0;
+                ents = (uint32_t)(a.ent_off[at + 1] - a.ent_off[at]);
+            }
+            const uint32_t inc = warp_incl_scan(ents);
+            if (lane == 31) warp_tot[warp] = inc;
+            __syncthreads();
+            uint32_t rel = run + inc - ents;
+            for (int q = 0; q < kWarps; ++q) { if (q < warp) rel += warp_tot[q]; run += warp_tot[q]; }
+            if (i < n) export_offset(a, g, c, local, (int32_t)rel);
+        }
+    }
+    __syncthreads();
+    // the others: a warp looks eight consecutive bins up at once (lane = bin) and takes them one after the other
+    int32_t* ids = reinterpret_cast<int32_t*>(map) + warp * kExportWarpKeys;
+    for (int32_t b0 = ((int32_t)blockIdx.x * kWarps + warp) * kBinsPerWarp; b0 < n_bins; b0 += (int32_t)gridDim.x * kWarps * kBinsPerWarp) {
+        int32_t my_seg = 0, my_start = 0, my_n = 0;
+        uint32_t my_ents = 0;
+        if (lane < kBinsPerWarp && b0 + lane < n_bins) {
+            const int32_t bin = b0 + lane;
+            my_seg = a.bin_seg[bin];
+            my_start = bin == a.segs[my_seg].bin0 ? a.segs[my_seg].out0 : (int32_t)a.bin_end[bin - 1];
+            my_n = (int32_t)a.bin_end[bin] - my_start;
+            my_ents = a.bin_ents[bin];
+        }
+        for (int q = 0; q < kBinsPerWarp; ++q) {
+            const int32_t n = __shfl_sync(0xFFFFFFFFu, my_n, q);
+            if (n <= 0 || n > kExportWarpKeys) continue;
+            const int32_t start = __shfl_sync(0xFFFFFFFFu, my_start, q);
+            const ExportSeg g = a.segs[__shfl_sync(0xFFFFFFFFu, my_seg, q)];
+            constexpr int kPer = kExportWarpKeys / 32;
+            int2 key[kPer];
+            int32_t rank[kPer];
+#pragma unroll
+            for (int r = 0; r < kPer; ++r) key[r] = r * 32 + lane < n ? a.keys[start + r * 32 + lane] : make_int2(INT32_MAX, 0);
+#pragma unroll
+            for (int r = 0; r < kPer; ++r) { ids[r * 32 + lane] = key[r].x; rank[r] = 0; }
+            __syncwarp();
+            for (int i = 0; i < n; i += 4) {
+                const int4 v = *reinterpret_cast<const int4*>(ids + i);
+#pragma unroll
+                for (int r = 0; r < kPer; ++r)
+                    if (r == 0 || n > r * 32) rank[r] += (v.x < key[r].x) + (v.y < key[r].x) + (v.z < key[r].x) + (v.w < key[r].x);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < kPer; ++r) if (r * 32 + lane < n) export_node(a, g, start + rank[r], key[r].x, key[r].y);
+            if (g.hop == a.k) continue;
+#pragma unroll
+            for (int r = 0; r < kPer; ++r)
+                if (r * 32 + lane < n) {
+                    const int32_t at = g.in0 + key[r].y - g.lrow0;
+                    ids[rank[r]] = a.ent_off[at + 1] - a.ent_off[at];
+                }
+            __syncwarp();
+            uint32_t run = __shfl_sync(0xFFFFFFFFu, my_ents, q);
+#pragma unroll
+            for (int r = 0; r < kPer; ++r) {
+                const uint32_t e = r * 32 + lane < n ? (uint32_t)ids[r * 32 + lane] : 0u;
+                const uint32_t inc = warp_incl_scan(e);
+                ids[r * 32 + lane] = (int32_t)(run + inc - e);
+                run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < kPer; ++r) if (r * 32 + lane < n) export_offset(a, g, start + rank[r], key[r].y, ids[rank[r]]);
+            __syncwarp();
+        }
     }
 }
 
-// 8 lanes per sampled node: its entries go to their place in the packed canonical entry list, neighbours translated to
-// canonical rows of the mini-batch; the node's offset (relative to its mini-batch) goes to nbr_offsets
+// A warp takes 32 sampled nodes; their entries lie one behind the other in the arena and are read as one stream, four loads in flight
+// per lane, each lane looking up whose its entry is.  They go to their place in the packed canonical entry list, the neighbours
+// translated to canonical rows of the mini-batch.
 __global__ void __launch_bounds__(kThreads) k_export_many_entries(ExportManyArgs a) {
-    const int gl = threadIdx.x & 7;
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31;
     const int32_t n_sampled = a.hop_base[a.k];
-    for (int32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < n_sampled; i += (gridDim.x * blockDim.x) >> 3) {
-        const int32_t b = a.node_batch[i];
-        const int32_t c = a.inv[i];
-        const int32_t row0 = a.rowbase0[b];                        // first packed row of the mini-batch
-        const int32_t* cum = a.cum + (int64_t)b * (a.k + 2);
-        const int32_t n0 = cum[a.k + 1] - cum[a.k];                // |Delta_0|
-        const uint32_t o0 = a.cnt[c], batch_e0 = a.cnt[row0];
-        const int32_t e0 = a.ent_off[i], n = a.ent_off[i + 1] - e0;
-        if (gl == 0) {
-            int32_t* off = a.o_nbr_off + row0 + b;                 // the mini-batch's nbr_offsets: |sampled| + 1 entries
-            off[c - row0 - n0] = (int32_t)(o0 - batch_e0);
-            if (c + 1 == a.rowbase0[b + 1]) off[c + 1 - row0 - n0] = (int32_t)(o0 - batch_e0) + n;   // terminal entry
-        }
-        for (int32_t j = gl; j < n; j += 8) {
-            const int32_t l = a.ent_repr[e0 + j];                  // the neighbour's local row in the mini-batch
-            int h = 0;
-            while (h < a.k && l >= cum[h + 1]) ++h;
-            const int32_t ai = a.node_off[h * (a.B + 1) + b] + (l - cum[h]);
-            a.o_nbrs[o0 + j] = a.ent_nbrs[e0 + j];
-            a.o_repr[o0 + j] = a.inv[ai] - row0;
+    for (int32_t i0 = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x) & ~31; i0 < n_sampled; i0 += (int32_t)(gridDim.x * blockDim.x)) {
+        const int32_t i = min(i0 + lane, n_sampled - 1);
+        const int32_t off = i0 + lane < n_sampled ? a.ent_off[i] : INT32_MAX;
+        const int32_t to = a.ent_to[i] - off, row0 = a.rowbase0[a.node_batch[i]];   // (lanes behind the last node: never asked for)
+        const int32_t end = a.ent_off[min(i0 + 32, n_sampled)];
+        for (int32_t e0 = __shfl_sync(0xFFFFFFFFu, off, 0); e0 < end; e0 += 32 * U) {
+            int32_t nbr[U], row[U], at[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int32_t e = min(e0 + u * 32 + lane, end - 1);
+                nbr[u] = a.ent_nbrs[e];
+                row[u] = a.ent_repr[e];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int32_t e = min(e0 + u * 32 + lane, end - 1);
+                int owner = 0;   // the last node whose entries start at or before e
+#pragma unroll
+                for (int s = 16; s > 0; s >>= 1)
+                    if (__shfl_sync(0xFFFFFFFFu, off, owner + s) <= e) owner += s;
+                at[u] = __shfl_sync(0xFFFFFFFFu, to, owner) + e;
+                row[u] = a.inv[__shfl_sync(0xFFFFFFFFu, row0, owner) + row[u]];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (e0 + u * 32 + lane < end) { a.o_nbrs[at[u]] = nbr[u]; a.o_repr[at[u]] = row[u]; }
         }
     }
 }
@@ -1424,11 +1729,8 @@ void mg_sort_params_host(SortParams* sp, int64_t n) {
 
 // LSD radix sort of 64-bit keys on bits [lo_bit, lo_bit + bits); sp (device) holds the key count.
 // Keys start in buf[0]; *res_buf tells which buffer holds the result.
-// With a tile table (seg_tiles, SegTile per tile; sp->ntiles tiles): a sort inside segments -- the first pass reads
-// every segment where its tiles say and all passes write segment after segment.
 void mg_sort_u64(mg_ctx* ctx, uint64_t* const buf[2], const SortParams* sp, int lo_bit, int bits, uint32_t* hist,
-                 uint32_t* scan_tmp, int* res_buf, const void* seg_tiles) {
-    const SegTile* tiles = static_cast<const SegTile*>(seg_tiles);
+                 uint32_t* scan_tmp, int* res_buf) {
     cudaStream_t st = ctx->stream;
     const int grid = mg_grid(ctx, 8);
     const int passes = (bits + kRadixBits - 1) / kRadixBits;
@@ -1437,27 +1739,15 @@ void mg_sort_u64(mg_ctx* ctx, uint64_t* const buf[2], const SortParams* sp, int 
     int cur = 0;
     for (int p = 0; p < passes; ++p) {
         const int shift = lo_bit + kRadixBits * p;
-        k_radix_hist<<<grid, kThreads, 0, st>>>(buf[cur], sp, shift, hist, tiles, p == 0);
+        k_radix_hist<<<grid, kThreads, 0, st>>>(buf[cur], sp, shift, hist);
         k_scan_reduce<<<grid, kThreads, 0, st>>>(hist, r, scan_tmp);
         k_scan_tiles<<<1, 1024, 0, st>>>(scan_tmp, r, nullptr);
         k_scan_down<<<grid, kThreads, 0, st>>>(hist, r, scan_tmp);
-        k_radix_scatter<<<grid, kThreads, kScatterSmem, st>>>(buf[cur], buf[cur ^ 1], sp, shift, hist, tiles, p == 0);
+        k_radix_scatter<<<grid, kThreads, kScatterSmem, st>>>(buf[cur], buf[cur ^ 1], sp, shift, hist);
         cur ^= 1;
     }
     ctx->launches += 5 * passes;
     *res_buf = cur;
-}
-
-// in-place exclusive scan of data[*lo .. *hi) (+ *base); total (+ *base) to *total_out (nullable)
-void mg_scan_u32(mg_ctx* ctx, uint32_t* data, const int32_t* lo, const int32_t* hi, const int32_t* base,
-                 uint32_t* scan_tmp, uint32_t* total_out) {
-    cudaStream_t st = ctx->stream;
-    const int grid = mg_grid(ctx, 8);
-    ScanRange r{lo, hi, base};
-    k_scan_reduce<<<grid, kThreads, 0, st>>>(data, r, scan_tmp);
-    k_scan_tiles<<<1, 1024, 0, st>>>(scan_tmp, r, total_out);
-    k_scan_down<<<grid, kThreads, 0, st>>>(data, r, scan_tmp);
-    ctx->launches += 3;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1507,9 +1797,9 @@ static int dense_alloc(mg_ctx* ctx, mg_dense* d, int32_t B, int32_t k, int64_t c
         if ((rc = dev_realloc(ctx, &d->scan_tmp, d->scan_tmp_elems))) return rc;
         d->sort_hist_elems = (size_t)kBins * sort_tiles + kBins;
         if ((rc = dev_realloc(ctx, &d->sort_hist, d->sort_hist_elems))) return rc;
-        SegTile* tiles = static_cast<SegTile*>(d->seg_tiles);
-        if ((rc = dev_realloc(ctx, &tiles, (size_t)sort_tiles + 1))) { d->seg_tiles = nullptr; return rc; }
-        d->seg_tiles = tiles;
+        char* tables = static_cast<char*>(d->seg_tiles);   // the segments, then the tiles: there are no more of the former than of the latter
+        if ((rc = dev_realloc(ctx, &tables, (size_t)sort_tiles * (sizeof(ExportSeg) + sizeof(int2))))) { d->seg_tiles = nullptr; return rc; }
+        d->seg_tiles = tables;
         d->cap_sort_tiles = sort_tiles;
     }
     if (d->cap_entries < cap_entries) {
@@ -2054,7 +2344,7 @@ extern "C" int mg_dense_view(mg_ctx* ctx, mg_dense* d, int32_t batch, mg_dense_a
 }
 
 // Layout of the export buffer (int32 elements), from the sample's capacities so that it is allocated once per handle.
-struct ExportLayout { size_t node_ids, nio, nbrs, repr, nbr_off, inv, cnt, total; };
+struct ExportLayout { size_t node_ids, nio, nbrs, repr, nbr_off, inv, ent_to, total; };
 static ExportLayout export_layout(const mg_dense* d) {
     ExportLayout L;
     const size_t cn = (size_t)d->cap_nodes, ce = (size_t)d->cap_entries, B = (size_t)d->n_batches;
@@ -2065,7 +2355,7 @@ static ExportLayout export_layout(const mg_dense* d) {
     L.repr = at; at += ce;
     L.nbr_off = at; at += cn + B + 1;
     L.inv = at; at += cn;
-    L.cnt = at; at += cn + 1;
+    L.ent_to = at; at += cn;
     L.total = at + 16;
     return L;
 }
@@ -2079,11 +2369,8 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
     const int k = d->k, B = d->n_batches;
     const int32_t n_total = d->h_hdr.hop_base[k + 1];
-    const int id_bits = std::max({1, ilog2_ceil(ctx->n_nodes), ilog2_ceil(d->n_targets_total + 1)});
-    const int pay_bits = std::max(1, ilog2_ceil((int64_t)n_total + 1));
-    if (id_bits + pay_bits > 64)
-        return mg_fail(ctx, MG_ERR_CAPACITY, "sample too large for a one-pass export (%d key bits): export fewer mini-batches per sample", id_bits + pay_bits);
-    if ((int64_t)(n_total + kSortTile - 1) / kSortTile + (int64_t)B * (k + 1) > d->cap_sort_tiles)
+    const int64_t n_segs = (int64_t)B * (k + 1);
+    if ((int64_t)(n_total + kSortTile - 1) / kSortTile + n_segs > d->cap_sort_tiles)
         return mg_fail(ctx, MG_ERR_STATE, "the sort scratch of this mg_dense is too small for its sample");
     const ExportLayout L = export_layout(d);
     int rc = mg_ensure(ctx, &d->expm_buf, &d->expm_elems, L.total);
@@ -2094,32 +2381,39 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
     cudaStream_t st = ctx->sample_stream;
     ExportManyArgs a;
     memset(&a, 0, sizeof(a));
-    a.B = B; a.k = k; a.n_nodes_total = n_total; a.pay_bits = pay_bits; a.id_bits = id_bits;
+    a.B = B; a.k = k; a.id_bits = std::max(1, ilog2_ceil(ctx->n_nodes));
     for (int h = 0; h <= k + 1; ++h) a.hop_base[h] = d->h_hdr.hop_base[h];
     a.nodes = d->nodes; a.node_batch = d->node_batch; a.node_off = d->node_off; a.cum = d->cum; a.rowbase0 = d->rowbase;
-    a.ent_off = d->ent_off; a.ent_nbrs = d->ent_nbrs; a.ent_repr = d->ent_repr;
+    a.ent_hop = d->d_ent_hop; a.ent_off = d->ent_off; a.ent_nbrs = d->ent_nbrs; a.ent_repr = d->ent_repr;
     a.o_node_ids = d->expm_buf + L.node_ids; a.o_nio = d->expm_buf + L.nio; a.o_nbrs = d->expm_buf + L.nbrs;
-    a.o_repr = d->expm_buf + L.repr; a.o_nbr_off = d->expm_buf + L.nbr_off; a.inv = d->expm_buf + L.inv;
-    a.cnt = reinterpret_cast<uint32_t*>(d->expm_buf + L.cnt);
+    a.o_repr = d->expm_buf + L.repr; a.o_nbr_off = d->expm_buf + L.nbr_off; a.inv = d->expm_buf + L.inv; a.ent_to = d->expm_buf + L.ent_to;
+    a.segs = static_cast<ExportSeg*>(d->seg_tiles);
+    a.tiles = reinterpret_cast<int2*>(a.segs + n_segs);
+    a.n_bins_max = (int32_t)(n_segs + n_total / 32);   // (export_bins: a segment of more than 64 nodes has at most a bin for 32 of them)
+    a.bin_end = d->sort_hist;                          // (kBins places for every tile that the scratch is sized for, and these are three for every bin)
+    a.bin_ents = a.bin_end + a.n_bins_max;
+    a.bin_seg = reinterpret_cast<int32_t*>(a.bin_ents + a.n_bins_max);
+    a.counts = reinterpret_cast<ExportCounts*>(d->scan_tmp + d->scan_tmp_elems - 12);
+    a.keys = reinterpret_cast<int2*>(d->newlist[0]);
+    a.dense_bins = reinterpret_cast<int32_t*>(d->newlist[1]);
     d->export_valid = false;
     MG_CUDA(ctx, mg_reads_wait(&d->expm_reads, st));   // (the last export's arrays may still be read)
     MG_CUDA(ctx, mg_reads_wait(&ctx->array_reads, st));
     d->expm_reads.queued = false;
     if (n_total > 0) {
-        SortParams* sp = (SortParams*)(d->scan_tmp + d->scan_tmp_elems - 8);
-        int32_t* range = d->scan_tmp + d->scan_tmp_elems - 12;
-        const int grid = mg_grid(ctx, 8);
-        ctx->stream = st;   // the sort and scan helpers (and the phase events) use ctx->stream
+        const int64_t n_tiles_max = n_segs + n_total / kSortTile;
+        auto blocks_for = [&](int64_t items, int per_block, int ctas_per_sm) {
+            return (unsigned)std::max<int64_t>(1, std::min<int64_t>((items + per_block - 1) / per_block, mg_grid(ctx, ctas_per_sm)));
+        };
+        ctx->stream = st;   // (the phase events use ctx->stream)
         {
         ProfScope ps(ctx, PH_SAMPLE_SORT);
-        k_export_tiles<<<1, 1024, 0, st>>>(a, static_cast<SegTile*>(d->seg_tiles), sp, range);
-        k_export_keys<<<grid, kThreads, 0, st>>>(a, d->newlist[0]);
-        int res = 0;
-        mg_sort_u64(ctx, d->newlist, sp, pay_bits, id_bits, d->sort_hist, (uint32_t*)d->scan_tmp, &res, d->seg_tiles);
-        k_export_place<<<grid, kThreads, 0, st>>>(a, d->newlist[res]);
-        mg_scan_u32(ctx, a.cnt, &range[0], &range[1], nullptr, (uint32_t*)d->scan_tmp, nullptr);
-        k_export_many_entries<<<grid, kThreads, 0, st>>>(a);
-        ctx->launches += 4;
+        k_export_begin<<<1 + blocks_for(a.n_bins_max + B, 1024, 1), 1024, 0, st>>>(a);
+        k_export_count<<<blocks_for(n_tiles_max, 1, 8), kThreads, 0, st>>>(a);
+        k_export_split<<<blocks_for(n_tiles_max, 1, 8), kThreads, 0, st>>>(a);
+        k_export_order<<<blocks_for(a.n_bins_max, kThreads / 32, 8), kThreads, 0, st>>>(a);
+        k_export_many_entries<<<blocks_for(d->h_hdr.hop_base[k], kThreads, 8), kThreads, 0, st>>>(a);
+        ctx->launches += 5;
         }
         ctx->stream = user;
     }

@@ -154,3 +154,46 @@ def test_many_mini_batches_on_a_graph_of_many_nodes():
             assert torch.equal(v.node_ids[v.repr_map.long()].long(), nbrs[b])
     c.close()
     torch.cuda.empty_cache()
+
+
+# an export orders the ids of a delta bin by bin: deltas on either side of the number of bins (65), of what a warp compares (129), of what
+# a block compares where the bin's range takes several bitmaps (1,025), ranges of one bitmap and of more, consecutive ids (one bin has all)
+# and spread ones, before and behind the last hop (sampled nodes carry their entries along)
+@pytest.mark.parametrize("stride", [1, 61, 200])
+def test_export_orders_deltas_of_any_size_and_spread(stride):
+    n, base = 2 ** 25 + 3, 5 * 2 ** 20 + 77
+    sizes = [1, 64, 65, 128, 129, 1_000, 1_024, 1_025, 4_096, 4_097, 40_000, 0]
+    tg = [np.arange(-(-m // 1_000), dtype=np.int64) + 100 * s for s, m in enumerate(sizes)]      # 1,000 of the delta's ids from each target
+    counts = np.zeros(n, np.int32)
+    inner = base + stride * np.arange(max(sizes))
+    counts[inner] = np.arange(len(inner)) % 4
+    for t, m in zip(tg, sizes):
+        counts[t] = np.minimum(1_000, m - 1_000 * np.arange(len(t)))
+    off = np.concatenate([[0], np.cumsum(counts, dtype=np.int64)])
+    nbrs = np.empty(off[-1], np.int32)
+    for t, m in zip(tg, sizes):
+        if m: nbrs[off[t[0]]:off[t[0]] + m] = np.sort(inner[:m])
+    for q in range(3):      # the last deltas: consecutive ids (stride 1) or spread ones
+        has = np.nonzero(np.arange(len(inner)) % 4 > q)[0]
+        nbrs[off[inner[has]] + q] = 2 ** 24 + stride * (2 * has + q)
+    c = mg.Context(0)
+    c.load_graph(torch.from_numpy(off).cuda(), torch.from_numpy(nbrs).cuda())
+    rng = np.random.default_rng(3)
+    targets = torch.from_numpy(np.concatenate([rng.permutation(t) for t in tg]).astype(np.int32))
+    offs = np.concatenate([[0], np.cumsum([len(t) for t in tg])])
+    room = 40 + 1_000 + 4 * 40_000
+    d = c.sample_many(targets, offs, [1_000, 3], list(range(len(tg))), caps={"max_nodes_total": 3 * room, "max_entries_total": 3 * room, "max_nodes_per_batch": room})
+    nodes, _ = d.counts()
+    assert nodes[:, 1].tolist() == sizes
+    d.export_many()
+    views = [d.export_view(b) for b in range(len(tg))]
+    for b, x in enumerate(views):
+        y = d.view(b)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
+        at = x.node_id_offsets.tolist()
+        for lo, hi in zip(at[:-2], at[1:-1]):
+            assert bool((x.node_ids[lo:hi].diff() > 0).all())
+        assert torch.equal(x.node_ids[x.repr_map.long()], x.nbrs)
+    c.close()
+    torch.cuda.empty_cache()
