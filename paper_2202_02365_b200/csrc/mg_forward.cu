@@ -25,7 +25,8 @@ int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int4* meta, const int64_t* sta
 int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* w_pad_t, const float* bias,
                    const float* h_prev, float* h_out, float* h_out2 /* nullable: the rows once more */, int flags /* 1 = ReLU, 2 = sum instead of mean */, const int4* row_meta,
                    int64_t row_lo, int64_t row_hi, int64_t safe_src_row, const void* w_pad_h /* the layer's fp16 weights, nullable */,
-                   int in_f16 /* layers >= 2: h_prev holds fp16 rows */, int out_f16 /* h_out receives fp16 rows */);
+                   int in_f16 /* layers >= 2: h_prev holds fp16 rows */, int out_f16 /* h_out receives fp16 rows */,
+                   uint32_t* positive /* nullable: a bit per value of h_out, above zero */);
 
 int mg_layer_grad_weights(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* h_prev, const float* dpre, const int4* row_meta,
                           int sum_aggr, float* dw);
@@ -614,7 +615,7 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
                 float* h_out = l == k ? hk : base + ring_off[l] - lo * m->dims[l];
                 ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST);
                 rc = mg_layer_fused(ctx, d, l, m->dims[l - 1], m->dims[l], m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
-                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], lo, hi, l > 1 ? lo_in : 0, l == 1 ? m->w_pad_h[0] : nullptr, 0, 0);
+                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], lo, hi, l > 1 ? lo_in : 0, l == 1 ? m->w_pad_h[0] : nullptr, 0, 0, nullptr);
                 if (rc) return rc;
             }
         }
@@ -656,6 +657,19 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
         ctx->ws_x_bytes = have * sizeof(float);
     }
 
+    // Kept outputs go through a ReLU once more in the backward pass, which only has to know which values were above zero: the
+    // fused kernel leaves a bit for each, a thirty-second of what reading the rows again takes.
+    {
+        int64_t words = 0;
+        for (int l = 1; l <= k; ++l) {
+            const bool bits = ctx->keep_layers && l < k && m->precision == MG_GEMM_TF32 && mg_layer_fused_supported(m->dims[l - 1], m->dims[l]);
+            ctx->positive_at[l] = bits ? words : -1;
+            if (bits) words += mg_positive_words(d->h_hdr.rows_total[l], m->dims[l]);
+        }
+        if (words > 0 && ctx->ws_positive_elems < (size_t)words && mg_ensure(ctx, &ctx->ws_positive, &ctx->ws_positive_elems, (size_t)(words + words / 4)))
+            for (int l = 1; l <= k; ++l) ctx->positive_at[l] = -1;   // (no room: the rows are read)
+    }
+
     const bool half = ctx->feat_dtype == MG_DTYPE_F16;
     for (int l = 1; l <= k; ++l) {
         const int d_in = m->dims[l - 1], d_out = m->dims[l];
@@ -668,7 +682,8 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
                 ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST);
                 rc = mg_layer_fused(ctx, d, l, d_in, d_out, m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
                                     (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], 0, M, 0,
-                                    (l == 1 || f16_inter) ? m->w_pad_h[l - 1] : nullptr, f16_inter && l > 1, f16_inter && l < k);
+                                    (l == 1 || f16_inter) ? m->w_pad_h[l - 1] : nullptr, f16_inter && l > 1, f16_inter && l < k,
+                                    ctx->positive_at[l] >= 0 ? ctx->ws_positive + ctx->positive_at[l] : nullptr);
             }
             if (rc) return rc;
             continue;
@@ -1045,26 +1060,30 @@ struct GatherArgs {
     const uint32_t* bad;       // the scan gave up: there are no lists
     const float* dx;           // [rows of layer, 2 d_in]
     int32_t d_in;
-    const float* y;            // [rows_in, d_in] kept outputs of layer - 1 (MASK), else null
+    const float* y;            // [rows_in, d_in] kept outputs of layer - 1 (RELU_ROWS), else null
+    const uint32_t* positive;  // which of them are above zero, mg_positive_words (RELU_BITS), else null
     float* g_in;               // [rows_in, d_in]
-    float* db;                 // [d_in] bias gradient of layer - 1 (MASK)
+    float* db;                 // [d_in] bias gradient of layer - 1 (with a ReLU)
 };
 
 // Bound by the latency of scattered 512-byte row reads.  A warp works on 128 columns of 16 consecutive source rows, or of one
 // unit of a row with a long list (a hub of the graph is named by hundreds of entries; one warp reading them one after the
 // other set the kernel's time).  Its contributions -- self parts and entries, row after row -- are first listed in shared
 // memory, lane = row, and then read as one stream, U loads of 512 bytes in flight whatever rows they belong to, with the kept
-// outputs of the rows that end among them (MASK) beside.  Rows of several units are added up by atomics: mask and bias are
+// outputs of the rows that end among them beside, or, where the forward pass has left bits of them, one word per column for
+// all rows of the group.  Rows of several units are added up by atomics: mask and bias are
 // linear in the sum.  24 mini-batches of 1,000 targets on 2M nodes: 1.56M rows x 128 in 685 -> 367 us, 543k + 92k rows x 256 in
-// 445 -> 388 us; 8 mini-batches on 1M nodes, 181k + 34k rows x 256 in 250 -> 141 us.  (MASK: four blocks per SM at 64 registers;
-// three at 72 take 481 / 178 us.)
+// 445 -> 388 us (bits: 213 us); 8 mini-batches on 1M nodes, 181k + 34k rows x 256 in 250 -> 141 us (bits: 83 us).  (With the outputs
+// read: four blocks per SM at 64 registers; three at 72 take 481 / 178 us.)
 constexpr int kGradRows = 16, kGradItems = kGradRows * (kGradLight + 1);
 static_assert(kGradItems >= kGradUnit + 1, "a unit's items fit the list");
 constexpr int64_t kGradMaxRows = (1ll << 30) - 1;   // an item holds twice its output row, and one more, in 31 bits; the largest value means none
 static_assert(2 * (kGradMaxRows - 1) + 1 < 0x7FFFFFFFll, "an output row's item is not the one that means none");
-template <bool MASK>
-__global__ void __launch_bounds__(kThreads, MASK ? 4 : 1) k_grad_gather(GatherArgs a) {
-    constexpr int U = MASK ? 4 : 8, kWarps = kThreads / 32;
+enum { RELU_NONE = 0, RELU_ROWS = 1, RELU_BITS = 2 };
+template <int RELU>
+__global__ void __launch_bounds__(kThreads, RELU ? 4 : 1) k_grad_gather(GatherArgs a) {
+    constexpr bool MASK = RELU != RELU_NONE;
+    constexpr int U = RELU == RELU_NONE ? 8 : 4, kWarps = kThreads / 32;
     constexpr uint32_t kNone = 0x7FFFFFFFu;       // an item without a contribution
     __shared__ int2 items_sm[kWarps][kGradItems];   // 2 x output row + (1: its neighbour part), weight; sign: the row's last item
     __shared__ int32_t rows_sm[kWarps][kGradRows];
@@ -1141,11 +1160,17 @@ __global__ void __launch_bounds__(kThreads, MASK ? 4 : 1) k_grad_gather(GatherAr
                 rows[__popc(rowmask & ((1u << lane) - 1u))] = (int32_t)s;
             }
         }
+        // (16 consecutive rows that start at a multiple of 16, or one row: their bits share a word per column)
+        uint4 pos = make_uint4(0u, 0u, 0u, 0u);
+        if (RELU == RELU_BITS && on) {
+            const int64_t row = w < n_units ? a.units[w].x : (w - n_units) * kGradRows;
+            pos = __ldg(reinterpret_cast<const uint4*>(a.positive) + (row >> 5) * n4 + c4);
+        }
         __syncwarp();
         float4 acc = zero4;
         int row_i = 0, row_l = 0;   // the row that the sums and the loads have come to
         for (int t = 0; t < n_items; t += U) {
-            float4 v[U], yv[MASK ? U : 1];
+            float4 v[U], yv[RELU == RELU_ROWS ? U : 1];
             int2 it[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -1153,7 +1178,7 @@ __global__ void __launch_bounds__(kThreads, MASK ? 4 : 1) k_grad_gather(GatherAr
                 const uint32_t src = (uint32_t)it[u].x & 0x7FFFFFFFu;
                 v[u] = zero4;
                 if (on && t + u < n_items && src != kNone) v[u] = __ldg(dx + (int64_t)src * n4);
-                if (MASK) {
+                if (RELU == RELU_ROWS) {
                     yv[u] = zero4;
                     if (t + u < n_items && it[u].x < 0) {
                         if (on) yv[u] = __ldg(reinterpret_cast<const float4*>(a.y) + (int64_t)rows[row_l] * n4 + c4);
@@ -1168,7 +1193,13 @@ __global__ void __launch_bounds__(kThreads, MASK ? 4 : 1) k_grad_gather(GatherAr
                 acc.x = fmaf(wt, v[u].x, acc.x); acc.y = fmaf(wt, v[u].y, acc.y); acc.z = fmaf(wt, v[u].z, acc.z); acc.w = fmaf(wt, v[u].w, acc.w);
                 if (it[u].x >= 0) continue;
                 if (MASK) {
-                    acc = make_float4(yv[u].x > 0.f ? acc.x : 0.f, yv[u].y > 0.f ? acc.y : 0.f, yv[u].z > 0.f ? acc.z : 0.f, yv[u].w > 0.f ? acc.w : 0.f);
+                    if (RELU == RELU_ROWS)
+                        acc = make_float4(yv[u].x > 0.f ? acc.x : 0.f, yv[u].y > 0.f ? acc.y : 0.f, yv[u].z > 0.f ? acc.z : 0.f, yv[u].w > 0.f ? acc.w : 0.f);
+                    else {
+                        const int bit = rows[row_i] & 31;
+                        acc = make_float4(pos.x >> bit & 1u ? acc.x : 0.f, pos.y >> bit & 1u ? acc.y : 0.f, pos.z >> bit & 1u ? acc.z : 0.f,
+                                          pos.w >> bit & 1u ? acc.w : 0.f);
+                    }
                     bias.x += acc.x; bias.y += acc.y; bias.z += acc.z; bias.w += acc.w;
                 }
                 if (on) {
@@ -1373,13 +1404,15 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         if (!turned && (rc = turn_entries_round())) return rc;
         turned = true;
         // dX -> the gradient of the layer's input rows
+        const bool bits = l > 1 && ctx->positive_at[l - 1] >= 0;
         GatherArgs ga{geom, l, rows_in, ra.cnt + ra.in_at[l], ra.rev, ra.units + ra.unit_at[l], ra.n_units + l, ra.bad, ctx->bw_dx, d_in,
-                      l > 1 ? ctx->ws_h[0] + h_off[l - 1] : nullptr, g_in, l > 1 ? m->g_bias[l - 2] : nullptr};
+                      l > 1 ? ctx->ws_h[0] + h_off[l - 1] : nullptr, bits ? ctx->ws_positive + ctx->positive_at[l - 1] : nullptr, g_in, l > 1 ? m->g_bias[l - 2] : nullptr};
         // (groups of 16 rows, a warp per 128 columns; the units come on top, the loop takes what does not fit the grid)
         const int64_t warps = (rows_in + kGradRows - 1) / kGradRows * std::max(1, (d_in + 127) / 128);
         const int ggrid = (int)std::max<int64_t>(1, std::min<int64_t>(mg_grid(ctx, l > 1 ? 4 : 8), (warps + kThreads / 32 - 1) / (kThreads / 32) + 16));
-        if (l > 1) k_grad_gather<true><<<ggrid, kThreads, 0, st>>>(ga);
-        else k_grad_gather<false><<<ggrid, kThreads, 0, st>>>(ga);
+        if (bits) k_grad_gather<RELU_BITS><<<ggrid, kThreads, 0, st>>>(ga);
+        else if (l > 1) k_grad_gather<RELU_ROWS><<<ggrid, kThreads, 0, st>>>(ga);
+        else k_grad_gather<RELU_NONE><<<ggrid, kThreads, 0, st>>>(ga);
         ctx->launches++;
     }
     if (ids_dev) launch_packed_ids(ctx, d, ids_dev);

@@ -136,11 +136,13 @@ struct mg_ctx {
     float* ws_x = nullptr; size_t ws_x_bytes = 0;
     float* ws_h[2] = {nullptr, nullptr}; size_t ws_h_bytes[2] = {0, 0};
     int4* ws_meta = nullptr; size_t ws_meta_elems = 0;   // row metadata of the fused layers (mg_layer_rows)
+    uint32_t* ws_positive = nullptr; size_t ws_positive_elems = 0;   // kept layer outputs: a bit per value, above zero
 
     // forward schedule
     int32_t layer_window_batches = 0;  // mini-batches per window of the layer schedule; 0 = whole layers
     bool keep_layers = false;          // keep H^1..H^{k-1} for mg_layer_output (whole-layer schedule)
     bool layers_kept = false;          // what the last forward did
+    int64_t positive_at[MG_MAX_HOPS + 1] = {0};   // where layer l's bits of ws_positive start (32-bit words); below zero: it left none
 
     // asynchronous output copy of mg_forward_host_async
     cudaEvent_t ev_fwd_done = nullptr, ev_out_done = nullptr;
@@ -384,6 +386,9 @@ static inline HostMemory mg_host_memory(const void* p, size_t bytes, const void*
     *mapped = first.devicePointer;
     return HOST_MAPPED;
 }
+
+// 32-bit words of a layer in mg_ctx::ws_positive: bit r % 32 of word (r / 32) * width + c stands for row r, column c
+static inline int64_t mg_positive_words(int64_t rows, int width) { return (rows + 31) / 32 * width; }
 
 static inline int mg_grid(const mg_ctx* ctx, int ctas_per_sm) { return ctx->n_sms * ctas_per_sm; }
 

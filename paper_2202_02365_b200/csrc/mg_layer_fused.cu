@@ -113,6 +113,7 @@ struct FusedArgs {
     const float* bias;
     float* out;                  // [M, N]
     float* out2;                 // the same rows once more, for the caller (the last layer with a device output), or null
+    uint32_t* positive;          // a bit per output value: above zero (kept layers of a ReLU, for the backward pass), or null
     uint32_t* error;
 };
 
@@ -345,7 +346,9 @@ __device__ __forceinline__ void gather_rows(const FusedArgs& a, const char* src,
 // HALVES = 1: tiles of 64 rows per CTA (one half only) for layers of few rows.  Such a layer is one chain -- plan, gather, weight
 // slices, epilogue -- whose links are halved, on twice the CTAs, with six weight slices in flight instead of two (the operand
 // stages are half as large); layers of many rows want the second half, whose gather runs under the first half's MMAs.
-template <bool FIRST, bool HALF, bool F16, bool TS, int HALVES>
+//
+// KEEP: what the backward pass wants is left on the way (its own instances, so that the others keep their registers).
+template <bool FIRST, bool HALF, bool F16, bool TS, int HALVES, bool KEEP>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(MG_FUSED_MAXNREG)
 k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_out,
                    const __grid_constant__ CUtensorMap map_out2, FusedArgs a) {
@@ -613,6 +616,12 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                         if (a.out_f16) *reinterpret_cast<__half*>(stage + j * 64 + lane * 2) = __float2half_rn(o);   // (boxes of 32 fp16 columns, not swizzled)
                         else *reinterpret_cast<float*>(stage + j * 128 + (((lane >> 2) ^ (j & 7)) << 4) + ((lane & 3) << 2)) = o;
                     }
+                    if (KEEP && a.positive) {   // lane = column: a word for its 32 rows
+                        uint32_t bits = 0;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) if (__uint_as_float(v[j]) + bias_n > 0.f) bits |= 1u << j;
+                        if (n0 + lane < a.N) a.positive[(row0 >> 5) * a.N + n0 + lane] = bits;
+                    }
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0) {
@@ -645,6 +654,21 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                 const int ncol0 = col_base + c0;   // first output column of this step
                 if (row0 >= a.M || ncol0 >= a.N) continue;
+                if (KEEP && a.positive) {   // lane = row: 32 rows of a column are one vote, lane c keeps column c's
+                    uint32_t bits = 0;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        if (c0 + 4 * c >= n_cols || ncol0 + 4 * c >= a.N) break;
+                        const float4 bb = __ldg(reinterpret_cast<const float4*>(a.bias + ncol0 + 4 * c));
+                        const float b4[4] = {bb.x, bb.y, bb.z, bb.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const uint32_t w = __ballot_sync(0xFFFFFFFFu, __uint_as_float(v[4 * c + i]) + b4[i] > 0.f);
+                            if (lane == 4 * c + i) bits = w;
+                        }
+                    }
+                    if (lane < 16 && c0 + lane < n_cols && ncol0 + lane < a.N) a.positive[(row0 >> 5) * a.N + ncol0 + lane] = bits;
+                }
                 if (a.out_f16) {
                     // fp16 output (widths that are multiples of 128 only): 128 bytes per row and box, so a row of the next
                     // layer's input is again fetched in 512-byte requests
@@ -1089,11 +1113,11 @@ int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int4* meta, const int64_t* sta
 
 // Runs layer `layer` (1-based) for the packed output rows [row_lo, row_hi).  h_prev and h_out are indexed by
 // GLOBAL packed row (callers that keep only a window of a layer pass pointers shifted accordingly).  h_out2 (nullable, 16-byte
-// aligned): receives the same rows.  The kernel is launched as a programmatic dependent of the one queued before it, which
+// aligned): receives the same rows.  positive (nullable): mg_positive_words of the layer.  The kernel is launched as a programmatic dependent of the one queued before it, which
 // must be mg_layer_rows' or another layer's.
 int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* w_pad_t, const float* bias,
                    const float* h_prev, float* h_out, float* h_out2, int flags, const int4* row_meta, int64_t row_lo, int64_t row_hi,
-                   int64_t safe_src_row, const void* w_pad_h, int in_f16, int out_f16) {
+                   int64_t safe_src_row, const void* w_pad_h, int in_f16, int out_f16, uint32_t* positive) {
     if (row_hi <= row_lo) return MG_OK;
     FusedArgs a;
     memset(&a, 0, sizeof(a));
@@ -1108,7 +1132,7 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     a.out_f16 = out_f16;
     a.relu = flags & 1;
     a.sum_aggr = (flags >> 1) & 1;
-    a.bias = bias; a.out = h_out; a.out2 = h_out2;
+    a.bias = bias; a.out = h_out; a.out2 = h_out2; a.positive = positive;
     // fp16 operands: first layer over fp16 base representations, mean aggregator (a sum of fp16 values may leave the
     // fp16 range), weights given in fp16 form (the caller withholds them when they do not suit fp16)
     // (later layers: in_f16 says that H^{l-1} was stored as fp16; the caller only does that with fp16 weights at hand)
@@ -1152,12 +1176,16 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
         return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the layer output");
     const bool first = layer == 1, half = first && ctx->feat_dtype == MG_DTYPE_F16;
     typedef void (*Kernel)(CUtensorMap, CUtensorMap, CUtensorMap, FusedArgs);
-#define MG_FUSED_KERNELS(TS, HALVES) \
-    {k_sage_layer_fused<true, false, false, TS, HALVES>, k_sage_layer_fused<true, true, false, TS, HALVES>, k_sage_layer_fused<true, true, true, TS, HALVES>, \
-     k_sage_layer_fused<false, false, false, TS, HALVES>, k_sage_layer_fused<false, true, true, TS, HALVES>}
-    static const Kernel kernels[2][2][5] = {{MG_FUSED_KERNELS(false, 1), MG_FUSED_KERNELS(true, 1)}, {MG_FUSED_KERNELS(false, 2), MG_FUSED_KERNELS(true, 2)}};
+    // (kept outputs are fp32: fp16 rows as a later layer's input have no instance that keeps)
+#define MG_FUSED_KERNELS(TS, HALVES, KEEP) \
+    k_sage_layer_fused<true, false, false, TS, HALVES, KEEP>, k_sage_layer_fused<true, true, false, TS, HALVES, KEEP>, \
+    k_sage_layer_fused<true, true, true, TS, HALVES, KEEP>, k_sage_layer_fused<false, false, false, TS, HALVES, KEEP>
+#define MG_FUSED_FORMS(TS, HALVES) {MG_FUSED_KERNELS(TS, HALVES, false), k_sage_layer_fused<false, true, true, TS, HALVES, false>, MG_FUSED_KERNELS(TS, HALVES, true)}
+    static const Kernel kernels[2][2][9] = {{MG_FUSED_FORMS(false, 1), MG_FUSED_FORMS(true, 1)}, {MG_FUSED_FORMS(false, 2), MG_FUSED_FORMS(true, 2)}};
+#undef MG_FUSED_FORMS
 #undef MG_FUSED_KERNELS
-    const int which = first ? (f16 ? 2 : half ? 1 : 0) : (f16 ? 4 : 3);
+    if (positive && (in_f16 || out_f16)) return mg_fail(ctx, MG_ERR_STATE, "fp16 layer outputs are not kept");
+    const int which = (first ? (f16 ? 2 : half ? 1 : 0) : (f16 ? 4 : 3)) + (positive ? 5 : 0);
     const Kernel kern = kernels[halves - 1][ts][which];
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)kern, fused_smem_limit(halves)));
     const int64_t n_tiles = (rows + HM * halves - 1) / (HM * halves);

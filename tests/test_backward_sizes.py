@@ -262,3 +262,31 @@ def test_base_rows_step_at_any_alignment(table_at, grad_at, dim):
     ctx.apply_embedding_sgd(dense, grad, 0.25)
     want = before.double().index_add(0, ids.long(), grad.double(), alpha=-0.25)
     assert float((table.double() - want).abs().max()) <= 4 * 2 ** -24 * 8      # (a handful of fp32 sums of magnitude below 8)
+
+
+# what the forward pass leaves for the backward pass when it is asked to keep its layers (a bit for each output above zero; the aggregates of
+# layers of several entries per row), against the same read and gathered again; rows around a row block and a tile, widths around a
+# word, a 16-column step, a half tile of output columns
+@pytest.mark.parametrize("sizes", [[1], [31, 2], [0, 33, 64], [700, 90], [5_000]])
+@pytest.mark.parametrize("dims,aggregator", [([16, 4, 8], "mean"), ([20, 36, 100, 12], "sum"), ([128, 132, 256, 8], "mean"), ([12, 256, 64, 16], "mean")])
+def test_what_the_forward_pass_keeps_for_the_backward_pass(sizes, dims, aggregator):
+    graph = inputs.erdos_renyi_graph(N, 9 * N, seed=31)
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(inputs.normal_features(N, dims[0], seed=32, device="cuda"))
+    targets = torch.cat([inputs.distinct_targets(N, s, seed=33 + i) for i, s in enumerate(sizes)])
+    dense = ctx.sample_many(targets, np.concatenate([[0], np.cumsum(sizes)]), [7, 5, 4][:len(dims) - 1], list(range(len(sizes))))
+    model = ctx.model(inputs.random_bias_layers(dims, seed=34))
+    model.set_aggregator(aggregator)
+    d_out = torch.randn((len(targets), dims[-1]), generator=torch.Generator("cuda").manual_seed(35), device="cuda")
+    got = []
+    for keep in (False, True):
+        ctx.keep_layer_outputs(keep)
+        out = torch.empty_like(d_out)
+        ctx.forward(model, dense, out)
+        grads, rows, ids = ctx.backward(model, dense, d_out, want_h0_grad=True)
+        got.append([out, rows.clone(), ids.clone()] + [x.clone() for layer in grads for x in layer])
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][2], got[1][2])
+    # the same operands; fp32 sums over up to 6,000 rows meet in any order: sqrt(6,000) 2^-24 of the terms' norm, where terms cancel more
+    for x, y in zip(got[0][1:2] + got[0][3:], got[1][1:2] + got[1][3:]):
+        assert float((x.double() - y.double()).norm()) <= 1e-4 * max(float(x.double().norm()), 1e-12)
