@@ -360,7 +360,7 @@ extern "C" int mg_destroy(mg_ctx* c) {
     free_out_graph(c);
     cudaFree(c->row_off); cudaFree(c->nbrs); cudaFree(c->d_slot_of_part); cudaFree(c->d_res_prefix); cudaFreeHost(c->h_flags);
     cudaFree(c->view_ws); cudaFree(c->d_part_start); cudaFree(c->d_part_of_node); cudaFree(c->d_local_of_node); cudaFree(c->d_nodes_by_part);
-    cudaFree(c->ws_x); cudaFree(c->ws_meta); cudaFree(c->ws_positive); cudaFree(c->ws_h[0]); cudaFree(c->ws_h[1]);
+    cudaFree(c->ws_x); cudaFree(c->ws_meta); cudaFree(c->ws_positive); cudaFree(c->ws_agg); cudaFree(c->ws_h[0]); cudaFree(c->ws_h[1]);
     cudaEventDestroy(c->ev_fwd_done); cudaEventDestroy(c->ev_out_done); cudaEventDestroy(c->ev_user);
     if (c->ev_backward) cudaEventDestroy(c->ev_backward);
     mg_reads_free(&c->array_reads);

@@ -26,10 +26,10 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
                    const float* h_prev, float* h_out, float* h_out2 /* nullable: the rows once more */, int flags /* 1 = ReLU, 2 = sum instead of mean */, const int4* row_meta,
                    int64_t row_lo, int64_t row_hi, int64_t safe_src_row, const void* w_pad_h /* the layer's fp16 weights, nullable */,
                    int in_f16 /* layers >= 2: h_prev holds fp16 rows */, int out_f16 /* h_out receives fp16 rows */,
-                   uint32_t* positive /* nullable: a bit per value of h_out, above zero */);
+                   uint32_t* positive /* nullable: a bit per value of h_out, above zero */, float* kept_agg /* nullable: the rows' aggregates */);
 
 int mg_layer_grad_weights(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* h_prev, const float* dpre, const int4* row_meta,
-                          int sum_aggr, float* dw);
+                          int sum_aggr, const float* kept_agg /* nullable: what mg_layer_fused left */, float* dw);
 
 namespace {
 
@@ -511,6 +511,8 @@ static int64_t chunk_rows_for(int d_in) {
     return rows;
 }
 
+constexpr int64_t kKeepEntriesPerRow = 3;   // layers with more entries per row leave their aggregates for the backward pass
+
 enum { OUT_DEVICE = 0, OUT_HOST = 1, OUT_HOST_ASYNC = 2 };
 
 // hands H^k (device, packed) to the caller: device or host copy, blocking or on the side stream
@@ -615,7 +617,7 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
                 float* h_out = l == k ? hk : base + ring_off[l] - lo * m->dims[l];
                 ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST);
                 rc = mg_layer_fused(ctx, d, l, m->dims[l - 1], m->dims[l], m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
-                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], lo, hi, l > 1 ? lo_in : 0, l == 1 ? m->w_pad_h[0] : nullptr, 0, 0, nullptr);
+                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], lo, hi, l > 1 ? lo_in : 0, l == 1 ? m->w_pad_h[0] : nullptr, 0, 0, nullptr, nullptr);
                 if (rc) return rc;
             }
         }
@@ -657,6 +659,20 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
         ctx->ws_x_bytes = have * sizeof(float);
     }
 
+    // The weights' gradients want the rows' aggregates again.  Where a row has several entries of a layer's outputs the forward pass leaves
+    // the aggregate behind: a row to write and to read in place of a row for each entry.  (Layer 1's rows have few entries and come from
+    // the table, where the other mini-batches' copies are as many: it gathers again.)
+    {
+        int64_t floats = 0;
+        for (int l = 1; l <= k; ++l) {
+            const bool kept = ctx->keep_layers && l > 1 && m->precision == MG_GEMM_TF32 && mg_layer_fused_supported(m->dims[l - 1], m->dims[l]) &&
+                              (int64_t)d->h_hdr.ent_base[k - l + 1] > kKeepEntriesPerRow * d->h_hdr.rows_total[l];
+            ctx->agg_at[l] = kept ? floats : -1;
+            if (kept) floats += (int64_t)d->h_hdr.rows_total[l] * m->dims[l - 1];
+        }
+        if (floats > 0 && ctx->ws_agg_elems < (size_t)floats && mg_ensure(ctx, &ctx->ws_agg, &ctx->ws_agg_elems, (size_t)(floats + floats / 4)))
+            for (int l = 1; l <= k; ++l) ctx->agg_at[l] = -1;   // (no room: gathered again)
+    }
     // Kept outputs go through a ReLU once more in the backward pass, which only has to know which values were above zero: the
     // fused kernel leaves a bit for each, a thirty-second of what reading the rows again takes.
     {
@@ -683,7 +699,8 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
                 rc = mg_layer_fused(ctx, d, l, d_in, d_out, m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
                                     (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], 0, M, 0,
                                     (l == 1 || f16_inter) ? m->w_pad_h[l - 1] : nullptr, f16_inter && l > 1, f16_inter && l < k,
-                                    ctx->positive_at[l] >= 0 ? ctx->ws_positive + ctx->positive_at[l] : nullptr);
+                                    ctx->positive_at[l] >= 0 ? ctx->ws_positive + ctx->positive_at[l] : nullptr,
+                                    ctx->agg_at[l] >= 0 ? ctx->ws_agg + ctx->agg_at[l] : nullptr);
             }
             if (rc) return rc;
             continue;
@@ -1368,7 +1385,8 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         if (m->precision == MG_GEMM_TF32) {
             // dW += X^T dPre with X gathered again inside the kernel; the row metadata is what the forward pass left (its layers all
             // have it, mg_forward of this very model and sample was the last to write it)
-            if ((rc = mg_layer_grad_weights(ctx, d, l, d_in, d_out, h_prev, dpre_all, ctx->ws_meta + meta_at, m->sum_aggr ? 1 : 0, m->g_w_cat[l - 1]))) return rc;
+            if ((rc = mg_layer_grad_weights(ctx, d, l, d_in, d_out, h_prev, dpre_all, ctx->ws_meta + meta_at, m->sum_aggr ? 1 : 0,
+                                            ctx->agg_at[l] >= 0 ? ctx->ws_agg + ctx->agg_at[l] : nullptr, m->g_w_cat[l - 1]))) return rc;
             // dX = dPre W^T on the tensor cores: the K-major operand the kernel wants is W itself ([2 d_in, d_out])
             if (g_in && (rc = mg_gemm_tf32(ctx, dpre_all, m->w_cat[l - 1], m->zeros, ctx->bw_dx, M, 2 * d_in, d_out, false))) return rc;
         }

@@ -136,12 +136,14 @@ struct mg_ctx {
     float* ws_x = nullptr; size_t ws_x_bytes = 0;
     float* ws_h[2] = {nullptr, nullptr}; size_t ws_h_bytes[2] = {0, 0};
     int4* ws_meta = nullptr; size_t ws_meta_elems = 0;   // row metadata of the fused layers (mg_layer_rows)
+    float* ws_agg = nullptr; size_t ws_agg_elems = 0;                // aggregates of the kept layers' rows
     uint32_t* ws_positive = nullptr; size_t ws_positive_elems = 0;   // kept layer outputs: a bit per value, above zero
 
     // forward schedule
     int32_t layer_window_batches = 0;  // mini-batches per window of the layer schedule; 0 = whole layers
     bool keep_layers = false;          // keep H^1..H^{k-1} for mg_layer_output (whole-layer schedule)
     bool layers_kept = false;          // what the last forward did
+    int64_t agg_at[MG_MAX_HOPS + 1] = {0};        // where layer l's rows of ws_agg start (floats); below zero: it left none
     int64_t positive_at[MG_MAX_HOPS + 1] = {0};   // where layer l's bits of ws_positive start (32-bit words); below zero: it left none
 
     // asynchronous output copy of mg_forward_host_async

@@ -113,6 +113,7 @@ struct FusedArgs {
     const float* bias;
     float* out;                  // [M, N]
     float* out2;                 // the same rows once more, for the caller (the last layer with a device output), or null
+    float* kept_agg;             // the rows' aggregates, [M, d_in] fp32 and not rounded (for the backward pass), or null
     uint32_t* positive;          // a bit per output value: above zero (kept layers of a ReLU, for the backward pass), or null
     uint32_t* error;
 };
@@ -255,10 +256,11 @@ __device__ __forceinline__ void plan_block(const FusedArgs& a, const int32_t* ke
 }
 
 // A gather warp's work on two planned rows: the lane's 16-byte operand pieces of each row's self part and aggregate.
-// (RAW: fp32 values as they are, not rounded to the operand's precision.)
-template <bool FIRST, bool HALF, bool F16, bool RAW = false>
+// (RAW: fp32 values as they are, not rounded to the operand's precision.  KEEP: the aggregates go to `keep`, if it is given, as well:
+// its rows are a.d_in floats apart.)
+template <bool FIRST, bool HALF, bool F16, bool RAW = false, bool KEEP = false>
 __device__ __forceinline__ void gather_rows(const FusedArgs& a, const char* src, bool on, bool cached, const RowMeta* meta, const int32_t (*first_rows)[8],
-                                            const int32_t* rows_of, uint4* selfv, uint4* meanv) {
+                                            const int32_t* rows_of, uint4* selfv, uint4* meanv, float* keep = nullptr) {
     RowMeta mq[kRowsInFlight];
     PieceSum<F16> acc[kRowsInFlight];
     int top = 0;
@@ -332,6 +334,8 @@ __device__ __forceinline__ void gather_rows(const FusedArgs& a, const char* src,
                                        __float_as_uint(acc[q2].a[3] * inv));
                 continue;
             }
+            if (KEEP && keep && mq[q2].z >= 0)
+                *reinterpret_cast<float4*>(keep + q2 * a.d_in) = make_float4(acc[q2].a[0] * inv, acc[q2].a[1] * inv, acc[q2].a[2] * inv, acc[q2].a[3] * inv);
             meanv[q2] = acc[q2].operand(inv);
             selfv[q2] = PieceSum<F16>::self_operand(selfv[q2]);
         }
@@ -791,7 +795,9 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                     const int32_t* rows_of = src_rows[slot];
                     const int brow = pw * kRowsInFlight;              // this warp's first row inside the block
                     uint4 selfv[kRowsInFlight], meanv[kRowsInFlight];   // the two operand pieces of each row
-                    gather_rows<FIRST, HALF, F16>(a, src, col_ok && ok, cached, &meta[slot][brow], &first_rows[slot][brow], rows_of, selfv, meanv);
+                    constexpr bool kKeepAgg = KEEP && !FIRST;
+                    float* keep = kKeepAgg && a.kept_agg ? a.kept_agg + (a.row_lo + tile_of(it) * TM + blk * kBlockRows + brow) * a.d_in + col : nullptr;
+                    gather_rows<FIRST, HALF, F16, false, kKeepAgg>(a, src, col_ok && ok, cached, &meta[slot][brow], &first_rows[slot][brow], rows_of, selfv, meanv, keep);
                     if (grp == n_groups - 1) {
                         // the block's plan has been read for the last time: its slot may be planned again
                         __syncwarp();
@@ -854,7 +860,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
 //   warps 0..15  gather, two rows each per block     warps 16..19  planners     warp 20  TMA     warp 21  MMA, tensor memory
 constexpr int kGradPlanners = 4, kGradFirstPlanner = 16, kGradTmaWarp = 20, kGradMmaWarp = 21;
 constexpr int kGradThreads = (kGradMmaWarp + 1) * 32;   // 704
-constexpr int kGradStages = 2;                          // (two leave the gathers 92 KB of L1: the MMAs of a block take a fifth of its gather)
+// (two stages leave the gathers 92 KB of L1: the MMAs of a block take a fifth of its gather; kept aggregates come by TMA, three deep)
+__host__ __device__ constexpr int grad_stages(bool kept) { return kept ? 3 : 2; }
 constexpr uint32_t kGradBox = kBlockRows * 128, kGradStageX = 8 * kGradBox;
 
 struct GradWArgs {
@@ -863,8 +870,12 @@ struct GradWArgs {
     float* dw;            // [2 d_in, N]
 };
 
-template <bool FIRST, bool HALF>
-__global__ void __launch_bounds__(kGradThreads, 1) k_sage_grad_weights(const __grid_constant__ CUtensorMap map_g, GradWArgs p) {
+// KEPT: the forward pass has left the aggregates (FusedArgs::kept_agg).  They lie as they are wanted, so TMA brings them like the gradient
+// rows, and the gather warps read the rows themselves only (92k + 24k rows of 2 x 256: 183 -> 110 us, 34k + 8k: 98 -> 62).
+template <bool FIRST, bool HALF, bool KEPT>
+__global__ void __launch_bounds__(kGradThreads, 1) k_sage_grad_weights(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_x,
+                                                                       GradWArgs p) {
+    constexpr int kGradStages = grad_stages(KEPT);
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t x_ready[kGradStages], g_full[kGradStages], stage_free[kGradStages], acc_full;
     __shared__ uint64_t plan_full[kPlanSlots], plan_empty[kPlanSlots];
@@ -913,7 +924,13 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_sage_grad_weights(const __g
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             uint4 selfv[kRowsInFlight], meanv[kRowsInFlight];
-            gather_rows<FIRST, HALF, false, true>(a, src, col_ok, plan_total[slot] >= 0, &meta[slot][brow], &first_rows[slot][brow], src_rows[slot], selfv, meanv);
+            if (KEPT) {
+#pragma unroll
+                for (int q = 0; q < kRowsInFlight; ++q)
+                    selfv[q] = col_ok ? load_piece<HALF, false>(src + (size_t)(uint32_t)meta[slot][brow + q].x * (size_t)a.src_row_bytes) : make_uint4(0u, 0u, 0u, 0u);
+            } else {
+                gather_rows<FIRST, HALF, false, true>(a, src, col_ok, plan_total[slot] >= 0, &meta[slot][brow], &first_rows[slot][brow], src_rows[slot], selfv, meanv);
+            }
 #pragma unroll
             for (int q = 0; q < kRowsInFlight; ++q)   // a row past the end meets a gradient row of zeros: it only has to be finite
                 if (meta[slot][brow + q].z < 0) selfv[q] = make_uint4(0u, 0u, 0u, 0u);
@@ -930,7 +947,7 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_sage_grad_weights(const __g
                     const int row = brow + q;
                     const size_t off = (size_t)row * 128 + (size_t)((((lane & 7) >> 1) ^ (row & 3)) << 5) + (size_t)((lane & 1) << 4);
                     *reinterpret_cast<uint4*>(xs + off) = selfv[q];
-                    *reinterpret_cast<uint4*>(xs + 4 * kGradBox + off) = meanv[q];
+                    if (!KEPT) *reinterpret_cast<uint4*>(xs + 4 * kGradBox + off) = meanv[q];
                 }
             }
             fence_async_smem();
@@ -969,18 +986,26 @@ __global__ void __launch_bounds__(kGradThreads, 1) k_sage_grad_weights(const __g
             const int64_t r = first_row(it) + lane;
             int4 rm = make_int4(a.safe_src, 0, -1, 0);
             if (r < a.M) rm = __ldg(a.row_meta + r);
-            plan_block<FIRST>(a, keys, rm, meta[slot], src_rows[slot], first_rows[slot], &plan_total[slot]);
+            if (KEPT) {
+                meta[slot][lane] = rm;
+                __syncwarp();
+            } else {
+                plan_block<FIRST>(a, keys, rm, meta[slot], src_rows[slot], first_rows[slot], &plan_total[slot]);
+            }
             if (lane == 0) mbar_arrive(&plan_full[slot]);
         }
     } else if (warp == kGradTmaWarp) {
         if (lane == 0) {
+            const int n_agg = KEPT ? min(4, (a.d_in - col0 + 31) / 32) : 0;   // boxes of this CTA's input columns
             uint32_t it = 0;
             for (; it < my; ++it) {
                 const int s = it % kGradStages;
                 if (it >= (uint32_t)kGradStages && !mbar_wait(&stage_free[s], ((it / kGradStages) - 1) & 1)) { report(a.error, 45u); break; }
-                mbar_expect_tx(&g_full[s], (uint32_t)(bn / 32) * kGradBox);
+                mbar_expect_tx(&g_full[s], (uint32_t)(bn / 32 + n_agg) * kGradBox);
                 for (int j = 0; j < bn / 32; ++j)   // (rows past the end and columns past the width come as zeros)
                     tma_load_2d(g_base + (size_t)s * g_bytes + (size_t)j * kGradBox, &map_g, &g_full[s], n0 + 32 * j, (int)first_row(it));
+                for (int j = 0; j < n_agg; ++j)
+                    tma_load_2d(x_base + (size_t)s * kGradStageX + (size_t)(4 + j) * kGradBox, &map_x, &g_full[s], col0 + 32 * j, (int)first_row(it));
             }
             // nothing of this CTA's may be in flight when it ends
             for (uint32_t i = it >= (uint32_t)kGradStages ? it - kGradStages : 0; i < it; ++i)
@@ -1113,11 +1138,12 @@ int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int4* meta, const int64_t* sta
 
 // Runs layer `layer` (1-based) for the packed output rows [row_lo, row_hi).  h_prev and h_out are indexed by
 // GLOBAL packed row (callers that keep only a window of a layer pass pointers shifted accordingly).  h_out2 (nullable, 16-byte
-// aligned): receives the same rows.  positive (nullable): mg_positive_words of the layer.  The kernel is launched as a programmatic dependent of the one queued before it, which
+// aligned): receives the same rows.  positive (nullable): mg_positive_words of the layer; kept_agg (nullable, layers >= 2):
+// [rows of the layer, d_in].  The kernel is launched as a programmatic dependent of the one queued before it, which
 // must be mg_layer_rows' or another layer's.
 int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* w_pad_t, const float* bias,
                    const float* h_prev, float* h_out, float* h_out2, int flags, const int4* row_meta, int64_t row_lo, int64_t row_hi,
-                   int64_t safe_src_row, const void* w_pad_h, int in_f16, int out_f16, uint32_t* positive) {
+                   int64_t safe_src_row, const void* w_pad_h, int in_f16, int out_f16, uint32_t* positive, float* kept_agg) {
     if (row_hi <= row_lo) return MG_OK;
     FusedArgs a;
     memset(&a, 0, sizeof(a));
@@ -1132,7 +1158,7 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     a.out_f16 = out_f16;
     a.relu = flags & 1;
     a.sum_aggr = (flags >> 1) & 1;
-    a.bias = bias; a.out = h_out; a.out2 = h_out2; a.positive = positive;
+    a.bias = bias; a.out = h_out; a.out2 = h_out2; a.positive = positive; a.kept_agg = kept_agg;
     // fp16 operands: first layer over fp16 base representations, mean aggregator (a sum of fp16 values may leave the
     // fp16 range), weights given in fp16 form (the caller withholds them when they do not suit fp16)
     // (later layers: in_f16 says that H^{l-1} was stored as fp16; the caller only does that with fp16 weights at hand)
@@ -1184,8 +1210,9 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     static const Kernel kernels[2][2][9] = {{MG_FUSED_FORMS(false, 1), MG_FUSED_FORMS(true, 1)}, {MG_FUSED_FORMS(false, 2), MG_FUSED_FORMS(true, 2)}};
 #undef MG_FUSED_FORMS
 #undef MG_FUSED_KERNELS
-    if (positive && (in_f16 || out_f16)) return mg_fail(ctx, MG_ERR_STATE, "fp16 layer outputs are not kept");
-    const int which = (first ? (f16 ? 2 : half ? 1 : 0) : (f16 ? 4 : 3)) + (positive ? 5 : 0);
+    const bool keep = positive || kept_agg;
+    if (keep && (in_f16 || out_f16)) return mg_fail(ctx, MG_ERR_STATE, "fp16 layer outputs are not kept");
+    const int which = (first ? (f16 ? 2 : half ? 1 : 0) : (f16 ? 4 : 3)) + (keep ? 5 : 0);
     const Kernel kern = kernels[halves - 1][ts][which];
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)kern, fused_smem_limit(halves)));
     const int64_t n_tiles = (rows + HM * halves - 1) / (HM * halves);
@@ -1203,9 +1230,9 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
 }
 
 // dw [2 d_in, d_out] += X^T dpre over the packed rows of layer `layer`, X = [self | aggregate]; row_meta: the layer's part of
-// mg_layer_rows' result.  dpre: DEVICE [rows, d_out], 16-byte aligned.
+// mg_layer_rows' result.  dpre: DEVICE [rows, d_out], 16-byte aligned.  kept_agg (nullable, layers >= 2): what mg_layer_fused left.
 int mg_layer_grad_weights(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* h_prev, const float* dpre, const int4* row_meta,
-                          int sum_aggr, float* dw) {
+                          int sum_aggr, const float* kept_agg, float* dw) {
     GradWArgs p;
     memset(&p, 0, sizeof(p));
     FusedArgs& a = p.f;
@@ -1227,12 +1254,16 @@ int mg_layer_grad_weights(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, i
     p.dw = dw;
     CUtensorMap mg;
     if (!make_map_f32(&mg, dpre, a.M, d_out, kBlockRows, true)) return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the gradient rows");
-    const size_t smem = kGradStages * (kGradStageX + (size_t)(p.n_cols / 32) * kGradBox) + 1024;
-    typedef void (*Kernel)(CUtensorMap, GradWArgs);
-    static const Kernel kernels[3] = {k_sage_grad_weights<true, false>, k_sage_grad_weights<true, true>, k_sage_grad_weights<false, false>};
-    const int which = layer > 1 ? 2 : ctx->feat_dtype == MG_DTYPE_F16 ? 1 : 0;
-    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)kernels[which], (int)(kGradStages * (kGradStageX + 8 * kGradBox) + 1024)));
-    kernels[which]<<<dim3((unsigned)p.n_slices, (unsigned)groups), kGradThreads, smem, ctx->stream>>>(mg, p);
+    CUtensorMap mx = mg;
+    if (kept_agg && !make_map_f32(&mx, kept_agg, a.M, d_in, kBlockRows, true)) return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the aggregates");
+    const int stages = grad_stages(kept_agg != nullptr);
+    const size_t smem = stages * (kGradStageX + (size_t)(p.n_cols / 32) * kGradBox) + 1024;
+    typedef void (*Kernel)(CUtensorMap, CUtensorMap, GradWArgs);
+    static const Kernel kernels[4] = {k_sage_grad_weights<true, false, false>, k_sage_grad_weights<true, true, false>, k_sage_grad_weights<false, false, false>,
+                                      k_sage_grad_weights<false, false, true>};
+    const int which = kept_agg ? 3 : layer > 1 ? 2 : ctx->feat_dtype == MG_DTYPE_F16 ? 1 : 0;
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)kernels[which], (int)(stages * (kGradStageX + 8 * kGradBox) + 1024)));
+    kernels[which]<<<dim3((unsigned)p.n_slices, (unsigned)groups), kGradThreads, smem, ctx->stream>>>(mg, mx, p);
     ctx->launches++;
     MG_CUDA(ctx, cudaGetLastError());
     return MG_OK;
