@@ -68,7 +68,6 @@ constexpr int kBlockRows = kProducerWarps * kRowsInFlight;   // 32: rows of a ti
 constexpr int kBlocksPerTile = BM / kBlockRows;              // 4
 constexpr int kPlanSlots = kBlocksPerTile;                   // planned row blocks in shared memory (one tile's worth)
 constexpr int HM = BM / 2;                                   // rows of a half tile: the unit the MMAs work on
-constexpr int kBlocksPerHalf = kBlocksPerTile / 2;
 constexpr int kAccBufs = 4;                                  // accumulator buffers in tensor memory (two tiles' halves)
 constexpr int kSlicesPerGroup = 2 * kGroupCols / KC;         // 8 K slices: (self, mean) x four 32-column blocks
 constexpr int kUnroll = 5;                       // neighbour rows per output row fetched before the first add
@@ -347,18 +346,21 @@ __device__ __forceinline__ void gather_rows(const FusedArgs& a, const char* src,
 // CTA); the accumulator is the transposed output, [output column][row].  Nothing is streamed per half tile then -- with
 // the weights in shared memory a half tile waits for eight 16 KB slices through a two-stage ring (4 us of latency).
 //
-// HALVES = 1: tiles of 64 rows per CTA (one half only) for layers of few rows.  Such a layer is one chain -- plan, gather, weight
+// ROWS: 128 output rows per tile and CTA, or 64 (one half only) for layers of few rows.  Such a layer is one chain -- plan, gather, weight
 // slices, epilogue -- whose links are halved, on twice the CTAs, with six weight slices in flight instead of two (the operand
-// stages are half as large); layers of many rows want the second half, whose gather runs under the first half's MMAs.
+// stages are half as large); layers of many rows want the second half, whose gather runs under the first half's MMAs.  32: a tile is
+// one row block, for layers that all SMs together take in one round that way; the other half of a 64-row stage is then never
+// written, and what the MMAs make of it never read (one mini-batch on 1M nodes, layers of 4,300 and 1,000 rows: 82 -> 62 us; two layers on
+// a graph of 10,000: 24 -> 18 us).
 //
 // KEEP: what the backward pass wants is left on the way (its own instances, so that the others keep their registers).
-template <bool FIRST, bool HALF, bool F16, bool TS, int HALVES, bool KEEP>
+template <bool FIRST, bool HALF, bool F16, bool TS, int ROWS, bool KEEP>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(MG_FUSED_MAXNREG)
 k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_out,
                    const __grid_constant__ CUtensorMap map_out2, FusedArgs a) {
     constexpr int KCE = Geo<F16>::kKC, GC = Geo<F16>::kGroup, LC = Geo<F16>::kLaneCols;
-    constexpr int TM = HM * HALVES;                          // rows of a tile
-    constexpr int kBlocks = kBlocksPerHalf * HALVES;         // row blocks of a tile
+    constexpr int HALVES = ROWS > HM ? 2 : 1, TM = ROWS;     // rows of a tile
+    constexpr int kBlocks = ROWS / kBlockRows, kHalfBlocks = kBlocks / HALVES;   // row blocks of a tile, of a half
     constexpr uint32_t kStage = stage_bytes(HALVES);
     extern __shared__ uint8_t smem_raw[];
     // a_ready and acc_empty are used in the leader CTA only (both CTAs arrive there); a_free, b_empty and acc_full
@@ -610,7 +612,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     const int64_t t = 2 * ((int64_t)pair + (int64_t)(hu / HALVES) * n_pairs) + (g >> 1);   // the tile of CTA g / 2
                     const int64_t row0 = a.row_lo + t * TM + (hu % HALVES) * HM + (g & 1) * 32;
-                    if (row0 >= a.M || n0 >= a.N) continue;
+                    if (row0 >= a.M || n0 >= a.N || (ROWS < HM && (g & 1))) continue;
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the previous box has left the tile
                     __syncwarp();
 #pragma unroll
@@ -657,7 +659,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                 tmem_ld_16(tmem_base + buf * acc_stride + ((uint32_t)(lane_group * 32) << 16) + (uint32_t)c0, v);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                 const int ncol0 = col_base + c0;   // first output column of this step
-                if (row0 >= a.M || ncol0 >= a.N) continue;
+                if (row0 >= a.M || ncol0 >= a.N || (ROWS < HM && (lane_group & 1))) continue;
                 if (KEEP && a.positive) {   // lane = row: 32 rows of a column are one vote, lane c keeps column c's
                     uint32_t bits = 0;
 #pragma unroll
@@ -783,7 +785,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                 const bool col_ok = lane_on && col < a.d_in;
                 const char* src = a.src_base + (size_t)col * (HALF ? 2 : 4);
                 for (int blk = 0; blk < kBlocks; ++blk) {
-                    const int h = blk / kBlocksPerHalf;               // the half tile this block belongs to
+                    const int h = blk / kHalfBlocks;               // the half tile this block belongs to
                     const uint32_t q = it * kBlocks + blk;     // row block counter of this CTA
                     const int slot = q % kPlanSlots;
                     if (grp == 0 && ok && !mbar_wait(&plan_full[slot], (q / kPlanSlots) & 1)) {
@@ -803,7 +805,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&plan_empty[slot]);
                     }
-                    if (blk % kBlocksPerHalf == 0) {
+                    if (blk % kHalfBlocks == 0) {
                         // the half's rows of the stages must have been read by the MMAs of their previous fill (one
                         // commit frees them all); those MMAs ran while the other half was gathered, and the loads
                         // above are already in flight while this waits
@@ -826,7 +828,7 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
                             *reinterpret_cast<uint4*>(stage_mean + off) = meanv[q2];
                         }
                     }
-                    if (blk % kBlocksPerHalf == kBlocksPerHalf - 1) {
+                    if (blk % kHalfBlocks == kHalfBlocks - 1) {
                         // this warp's rows of the half are in place: tell the leader's MMA thread
                         fence_async_smem();
                         __syncwarp();
@@ -1178,7 +1180,7 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     // 128-row tiles, the whole call 214 -> 195 us; 128 mini-batches keep them: 4.0 ms either way.)
     const int64_t rows = row_hi - row_lo, pairs = ctx->n_sms / 2;
     const int64_t rounds1 = (rows + 2 * HM * pairs - 1) / (2 * HM * pairs), rounds2 = (rows + 4 * HM * pairs - 1) / (4 * HM * pairs);
-    const int halves = rounds1 * 8 < rounds2 * 14 ? 1 : 2;
+    const int tile_rows = rows <= 2 * kBlockRows * pairs ? kBlockRows : rounds1 * 8 < rounds2 * 14 ? HM : BM, halves = tile_rows > HM ? 2 : 1;
     a.sb = std::max(2, std::min({kMaxStages, n_chunks, ring_bytes(halves) / b_bytes}));
     // weights in tensor memory: TF32 operands, fp32 output, all of K in 256 columns, at most 256 output columns
     // ... and rows with few entries: a half tile of long rows is gathered for longer than its weight slices take to
@@ -1203,19 +1205,20 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     const bool first = layer == 1, half = first && ctx->feat_dtype == MG_DTYPE_F16;
     typedef void (*Kernel)(CUtensorMap, CUtensorMap, CUtensorMap, FusedArgs);
     // (kept outputs are fp32: fp16 rows as a later layer's input have no instance that keeps)
-#define MG_FUSED_KERNELS(TS, HALVES, KEEP) \
-    k_sage_layer_fused<true, false, false, TS, HALVES, KEEP>, k_sage_layer_fused<true, true, false, TS, HALVES, KEEP>, \
-    k_sage_layer_fused<true, true, true, TS, HALVES, KEEP>, k_sage_layer_fused<false, false, false, TS, HALVES, KEEP>
-#define MG_FUSED_FORMS(TS, HALVES) {MG_FUSED_KERNELS(TS, HALVES, false), k_sage_layer_fused<false, true, true, TS, HALVES, false>, MG_FUSED_KERNELS(TS, HALVES, true)}
-    static const Kernel kernels[2][2][9] = {{MG_FUSED_FORMS(false, 1), MG_FUSED_FORMS(true, 1)}, {MG_FUSED_FORMS(false, 2), MG_FUSED_FORMS(true, 2)}};
+#define MG_FUSED_KERNELS(TS, ROWS, KEEP) \
+    k_sage_layer_fused<true, false, false, TS, ROWS, KEEP>, k_sage_layer_fused<true, true, false, TS, ROWS, KEEP>, \
+    k_sage_layer_fused<true, true, true, TS, ROWS, KEEP>, k_sage_layer_fused<false, false, false, TS, ROWS, KEEP>
+#define MG_FUSED_FORMS(TS, ROWS) {MG_FUSED_KERNELS(TS, ROWS, false), k_sage_layer_fused<false, true, true, TS, ROWS, false>, MG_FUSED_KERNELS(TS, ROWS, true)}
+    static const Kernel kernels[3][2][9] = {{MG_FUSED_FORMS(false, kBlockRows), MG_FUSED_FORMS(true, kBlockRows)}, {MG_FUSED_FORMS(false, HM), MG_FUSED_FORMS(true, HM)},
+                                            {MG_FUSED_FORMS(false, BM), MG_FUSED_FORMS(true, BM)}};
 #undef MG_FUSED_FORMS
 #undef MG_FUSED_KERNELS
     const bool keep = positive || kept_agg;
     if (keep && (in_f16 || out_f16)) return mg_fail(ctx, MG_ERR_STATE, "fp16 layer outputs are not kept");
     const int which = (first ? (f16 ? 2 : half ? 1 : 0) : (f16 ? 4 : 3)) + (keep ? 5 : 0);
-    const Kernel kern = kernels[halves - 1][ts][which];
+    const Kernel kern = kernels[tile_rows == BM ? 2 : tile_rows == HM ? 1 : 0][ts][which];
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)kern, fused_smem_limit(halves)));
-    const int64_t n_tiles = (rows + HM * halves - 1) / (HM * halves);
+    const int64_t n_tiles = (rows + tile_rows - 1) / tile_rows;
     const int grid = 2 * (int)std::min<int64_t>((n_tiles + 1) / 2, pairs);   // CTA pairs
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kFusedThreads); cfg.dynamicSmemBytes = smem; cfg.stream = ctx->stream;

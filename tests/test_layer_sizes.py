@@ -66,3 +66,10 @@ def test_rows_written_over_the_table(graph, hops, window):
     got = table[1_000:1_000 + per * count]
     ctx.forward(model, dense, got)
     assert torch.equal(got, want)
+
+
+# tiles of 32 rows: one row, a full tile, one more, all that the SMs take in one round of them (148 SMs: 4,736), one more
+@pytest.mark.parametrize("rows", [31, 32, 33, 63, 96, 4_736, 4_737])
+@pytest.mark.parametrize("d_in,d_out,half,fanout", [(128, 256, False, 4), (256, 100, False, 9), (384, 36, True, 3)])
+def test_rows_on_either_side_of_the_smallest_tiles(graph, rows, d_in, d_out, half, fanout):
+    test_rows_on_either_side_of_the_tile_sizes(graph, rows, d_in, d_out, half, fanout)
