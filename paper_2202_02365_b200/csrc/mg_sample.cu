@@ -166,7 +166,10 @@ __global__ void __launch_bounds__(kThreads) k_begin(BeginArgs a) {
 // us).  A tile has as few nodes as keeps five blocks per SM busy (hop_tile): the picks of a warp's nodes are one chain after
 // the other, and a hop of 1,000 nodes took 21 us with 256 of them per block, 10 us with 32.  Tiles are handed out by a
 // counter, as chain_tiles wants it.
-// Hop 0 also enters the targets: residency and range checks, the id table (Algorithm 1 wants unique targets).
+// Hop 0 also enters the targets: residency and range checks, the id table (Algorithm 1 wants unique targets).  The other hops start from the
+// counts of new nodes per mini-batch: every block sums them up for itself (block 0 writes the sums down), and the tiles' nodes are
+// read from the mini-batches' runs of new ids and put one behind the other on the way (a kernel of its own for
+// that took 3.4 to 5 us per hop of one mini-batch, 26 us for the two inner hops of 128).
 struct HopArgs {
     DenseHeader* hdr;
     int hop;
@@ -183,8 +186,15 @@ struct HopArgs {
     uint64_t* tile_state;
     int32_t tile_cap;             // nodes of a tile that the launch has shared memory for
     int32_t n_sms;
+    int32_t B, k;
+    // hops > 0: the nodes are what k_insert found new in the hop before
+    const int32_t* new_ids;       // by rank, mini-batch b's from the place of its first entry on
+    const uint32_t* batch_cnt;    // [B] how many
+    int64_t cap_nodes;
+    int32_t node_limit;           // nodes that a mini-batch may have with them
+    int32_t* cum;
+    int32_t* node_off;
     // hop 0
-    int32_t B;
     const int32_t* tgt_off;
     int32_t* hkeys;
     int32_t* hvals;
@@ -256,11 +266,59 @@ __device__ __forceinline__ uint32_t floyd_pick(bool on, uint32_t d, int32_t f, i
     return pick;
 }
 
+// A hop's nodes per mini-batch, summed up over the mini-batches: the new nodes of hop - 1 are hop's.  Every block takes the sums for itself
+// (a kernel of one block for it cost 2 us and a gap per hop); block 0 writes them down.  Returns one past the hop's last node.
+struct NewNodes {
+    DenseHeader* hdr;
+    int32_t hop, B, k;
+    const uint32_t* batch_cnt;   // [B] new nodes of hop - 1
+    int64_t cap_nodes;
+    int32_t node_limit;          // nodes that a mini-batch may have with them
+    const int32_t* ent_off;
+    int32_t* cum;
+    int32_t* node_off;
+};
+__device__ __forceinline__ int64_t sum_new_nodes(const NewNodes& a, int32_t* next_off, int32_t* list_at, uint32_t* part /* [kThreads / 32] */) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t carry = (uint32_t)a.hdr->hop_base[a.hop];
+    for (int s0 = 0; s0 < a.B; s0 += kThreads) {
+        const int b = s0 + (int)threadIdx.x;
+        const uint32_t v = b < a.B ? a.batch_cnt[b] : 0u;
+        const int32_t run = b < a.B ? a.ent_off[a.node_off[(a.hop - 1) * (a.B + 1) + b]] : 0;
+        const uint32_t inc = warp_incl_scan(v);
+        if (lane == 31) part[warp] = inc;
+        __syncthreads();
+        uint32_t before = carry, total = 0;
+        for (int w = 0; w < kThreads / 32; ++w) { if (w < warp) before += part[w]; total += part[w]; }
+        if (b < a.B) {
+            next_off[b] = (int32_t)(before + inc - v);
+            list_at[b] = run;
+            if (blockIdx.x == 0) {
+                a.node_off[a.hop * (a.B + 1) + b] = next_off[b];
+                const int32_t rows = a.cum[b * (a.k + 2) + a.hop] + (int32_t)v;
+                a.cum[b * (a.k + 2) + a.hop + 1] = rows;
+                if (rows > a.node_limit) atomicOr(&a.hdr->status, ST_CAP_TABLE);
+            }
+        }
+        carry += total;
+        __syncthreads();
+    }
+    const int64_t end = carry;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (end > a.cap_nodes) atomicOr(&a.hdr->status, ST_CAP_NODES);
+        else {
+            a.hdr->hop_base[a.hop + 1] = (int32_t)end;
+            a.node_off[a.hop * (a.B + 1) + a.B] = (int32_t)end;
+        }
+    }
+    return end;
+}
+
 // G lanes per node, fanout <= G <= 32; a warp holds 32 / G nodes (G need not divide 32: the lanes left over idle, and
 // G = 5 or 10 keeps 30 lanes busy where the next power of two keeps 20).  G = 0: any fanout up to MG_MAX_FANOUT, a node per
 // warp at a time, picks staged in shared memory.
 template <int G>
-__global__ void __launch_bounds__(kThreads) k_hop(HopArgs a) {
+__global__ void __launch_bounds__(kThreads, 4) k_hop(HopArgs a) {
     extern __shared__ __align__(16) uint8_t hop_sm[];   // the tile's nodes, then (G = 0) per warp x[f], pick[f]
     __shared__ uint32_t part[kTileParts];
     __shared__ int32_t sh_tile;
@@ -268,11 +326,21 @@ __global__ void __launch_bounds__(kThreads) k_hop(HopArgs a) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t f = a.fanout;
     const bool inout = a.row_off[1] != nullptr;
-    const int32_t lo = a.hdr->hop_base[a.hop], n = a.hdr->hop_base[a.hop + 1] - lo;
+    int32_t* next_off = reinterpret_cast<int32_t*>(hop_sm);   // [B] (hops > 0) first node of the mini-batch in the hop ...
+    int32_t* list_at = next_off + a.B;                        // ... and its run of new_ids
+    const int32_t lo = a.hdr->hop_base[a.hop];
+    int32_t n;
+    if (a.hop == 0) n = a.hdr->hop_base[1] - lo;
+    else {
+        if (__syncthreads_or(a.hdr->status != 0)) return;   // (the whole block: another one may be setting it)
+        const int64_t end = sum_new_nodes({a.hdr, a.hop, a.B, a.k, a.batch_cnt, a.cap_nodes, a.node_limit, a.ent_off, a.cum, a.node_off}, next_off, list_at, part);
+        if (end > a.cap_nodes) return;   // (nothing is written outside the arenas; the kernels that follow see the status)
+        n = (int32_t)(end - lo);
+    }
     // (an empty hop has one empty tile: it closes the entry range)
     const int32_t tile_nodes = min(hop_tile(n, a.n_sms), a.tile_cap), n_tiles = max(1, (n + tile_nodes - 1) / tile_nodes);
     const int sets = (tile_nodes + kThreads - 1) / kThreads;   // nodes per thread
-    int64_t* node_r0 = reinterpret_cast<int64_t*>(hop_sm);                                      // [dirs][tile_cap]
+    int64_t* node_r0 = reinterpret_cast<int64_t*>(hop_sm + (a.hop > 0 ? 8 * (size_t)a.B : 0));   // [dirs][tile_cap]
     uint32_t* node_deg = reinterpret_cast<uint32_t*>(node_r0 + (inout ? 2 : 1) * a.tile_cap);   // [dirs][tile_cap]
     int32_t* node_id = reinterpret_cast<int32_t*>(node_deg + (inout ? 2 : 1) * a.tile_cap);
     int32_t* node_b = node_id + a.tile_cap;
@@ -297,8 +365,13 @@ __global__ void __launch_bounds__(kThreads) k_hop(HopArgs a) {
             int32_t v = 0, b = 0;
             bool in_range = node_ok;
             if (node_ok) {
-                v = a.hop == 0 ? targets[local] : a.nodes[lo + local];
-                if (a.hop > 0) b = a.node_batch[lo + local];
+                if (a.hop == 0) v = targets[local];
+                else {
+                    b = upper_segment(next_off, a.B, lo + local);
+                    v = a.new_ids[list_at[b] + (lo + local - next_off[b])];
+                    a.nodes[lo + local] = v;
+                    a.node_batch[lo + local] = b;
+                }
             }
             if (a.hop == 0) {
                 if (t - lane < n_here) b = target_batch(a.tgt_off, a.B, local - lane, min(local, n - 1));
@@ -998,36 +1071,33 @@ k_radix_scatter(const uint64_t* __restrict__ keys, uint64_t* __restrict__ out, c
 constexpr size_t kScatterSmem = (size_t)kSortTile * 8 + (size_t)(kThreads / 32) * kBins * 4 + 2 * (size_t)kBins * 4;
 
 // -------------------------------------------------------------------------------------
-// place the new nodes as the next hop, give the entries their rows
+// place the last hop's new nodes, give the entries their rows
 // -------------------------------------------------------------------------------------
-// The hop's new nodes per mini-batch, summed up, are the next hop's node offsets (every block takes the sums for itself, block 0
-// writes them down: a kernel of one block for it cost 2 us and a gap per hop).  Then: the mini-batches' runs of new ids are put
-// one behind the other (a warp takes 128 nodes at a time, four loads in flight per thread); an entry that met a known node -> that node's row (entries of new nodes got theirs at
-// insert time; the shared-memory path of the last hop leaves none).
-// FINAL (last hop): block 0 also writes the packed row bases of every layer and the per-batch entry bounds of every hop, and
-// the sample's summary (header, per-batch tables) for the host, stored straight into mapped pinned memory.  A copy engine
-// is not used on purpose: a large output copy of a forward pass may be queued on it, and the host would wait for that copy
-// before it learned the sample's sizes.  (After an error the summary still goes out: it carries the status word.)
+// The new nodes per mini-batch are summed up as in k_hop, and their runs of new ids put one behind the other (a warp takes 128 nodes at a
+// time, four loads in flight per thread); an entry, of whatever hop, that met a known node -> that node's row (entries of new nodes got
+// theirs at insert time; the shared-memory path of the last hop leaves none).  Block 0 writes the packed row bases of every layer and the
+// per-batch entry bounds of every hop, and the sample's summary (header, per-batch tables) for the host, stored straight into mapped pinned
+// memory.  A copy engine is not used on purpose: a large output copy of a forward pass may be queued on it, and the host would wait for
+// that copy before it learned the sample's sizes.  (After an error the summary still goes out: it carries the status word.)
 struct PlaceArgs {
     DenseHeader* hdr;
-    int hop;
-    const int32_t* new_ids;      // the hop's new ids by rank, mini-batch b's from the place of its first entry on
-    const uint32_t* batch_cnt;   // [B] new nodes of the hop
+    const int32_t* new_ids;      // the last hop's new ids by rank, mini-batch b's from the place of its first entry on
+    const uint32_t* batch_cnt;   // [B] new nodes of the last hop
     int64_t cap_nodes;
     int32_t* nodes;
     int32_t* node_batch;
-    const int32_t* hvals;      // null: the entries have their rows
-    int32_t node_limit;        // nodes that a mini-batch may have after this hop
+    const int32_t* hvals;
+    int32_t hops_in_table;       // hops whose entries went through the global tables: k, or k - 1
+    int32_t node_limit;          // nodes that a mini-batch may have in all
     int32_t* ent_repr;
     int32_t B, k;
     int32_t* cum;
     int32_t* node_off;
-    // FINAL
     int32_t n_hdr;
     const int32_t* ent_off;
     int32_t* rowbase;
     int32_t* ent_hop;
-    int32_t* out;              // n_hdr header words, cum, node_off, rowbase, ent_hop
+    int32_t* out;                // n_hdr header words, cum, node_off, rowbase, ent_hop
 };
 
 __device__ __forceinline__ void finish_sample(const PlaceArgs& a, bool bad) {
@@ -1067,54 +1137,22 @@ __device__ __forceinline__ void finish_sample(const PlaceArgs& a, bool bad) {
 
 constexpr int kPlacePerThread = 4;
 
-template <bool FINAL>
 __global__ void __launch_bounds__(kThreads, 8) k_place(PlaceArgs a) {
-    extern __shared__ int32_t next_off[];   // [B] first node of the mini-batch in the next hop ...
+    extern __shared__ int32_t next_off[];   // [B] first node of the mini-batch among the new ones ...
     int32_t* list_at = next_off + a.B;      // ... and its run of new_ids
     __shared__ uint32_t part[kThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int32_t start = a.hdr->hop_base[a.hop + 1];
-    const int32_t lo = a.hdr->ent_base[a.hop], hi = a.hdr->ent_base[a.hop + 1];
+    const int lane = threadIdx.x & 31;
+    const int32_t start = a.hdr->hop_base[a.k], hi = a.hdr->ent_base[a.hops_in_table];
     // (the whole block alike: block 0 may be adding to the status)
     bool bad = __syncthreads_or(a.hdr->status != 0);
     int64_t end = start;
     if (!bad) {
-        uint32_t carry = (uint32_t)start;
-        for (int s0 = 0; s0 < a.B; s0 += kThreads) {
-            const int b = s0 + (int)threadIdx.x;
-            const uint32_t v = b < a.B ? a.batch_cnt[b] : 0u;
-            const int32_t run = b < a.B ? a.ent_off[a.node_off[a.hop * (a.B + 1) + b]] : 0;
-            const uint32_t inc = warp_incl_scan(v);
-            if (lane == 31) part[warp] = inc;
-            __syncthreads();
-            uint32_t before = carry, total = 0;
-            for (int w = 0; w < kThreads / 32; ++w) { if (w < warp) before += part[w]; total += part[w]; }
-            if (b < a.B) {
-                next_off[b] = (int32_t)(before + inc - v);
-                list_at[b] = run;
-                if (blockIdx.x == 0) {
-                    a.node_off[(a.hop + 1) * (a.B + 1) + b] = next_off[b];
-                    const int32_t rows = a.cum[b * (a.k + 2) + a.hop + 1] + (int32_t)v;
-                    a.cum[b * (a.k + 2) + a.hop + 2] = rows;
-                    if (rows > a.node_limit) atomicOr(&a.hdr->status, ST_CAP_TABLE);
-                }
-            }
-            carry += total;
-            __syncthreads();
-        }
-        end = carry;
-        if (end > a.cap_nodes) bad = true;   // (nothing is written outside the arenas; the kernels that follow see the status)
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            if (bad) atomicOr(&a.hdr->status, ST_CAP_NODES);
-            else {
-                a.hdr->hop_base[a.hop + 2] = (int32_t)end;
-                a.node_off[(a.hop + 1) * (a.B + 1) + a.B] = (int32_t)end;
-            }
-        }
+        end = sum_new_nodes({a.hdr, a.k, a.B, a.k, a.batch_cnt, a.cap_nodes, a.node_limit, a.ent_off, a.cum, a.node_off}, next_off, list_at, part);
+        bad = end > a.cap_nodes;   // (nothing is written outside the arenas)
     }
-    if (FINAL && blockIdx.x == 0) { __syncthreads(); finish_sample(a, bad); return; }
+    if (blockIdx.x == 0) { __syncthreads(); finish_sample(a, bad); return; }
     if (bad) return;
-    const int32_t step = (int32_t)(gridDim.x - FINAL) * kThreads, tid = (int32_t)(blockIdx.x - FINAL) * kThreads + (int32_t)threadIdx.x;
+    const int32_t step = (int32_t)(gridDim.x - 1) * kThreads, tid = (int32_t)(blockIdx.x - 1) * kThreads + (int32_t)threadIdx.x;
     for (int64_t at0 = start + (int64_t)(tid >> 5) * (32 * kPlacePerThread); at0 < end; at0 += (int64_t)step * kPlacePerThread) {
         int32_t b = 0;   // the mini-batch of the warp's first node
         for (int32_t above = a.B; above - b > 1;) {
@@ -1137,8 +1175,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_place(PlaceArgs a) {
             if (at < end) { a.nodes[at] = id[j]; a.node_batch[at] = batch[j]; }
         }
     }
-    if (!a.hvals) return;
-    for (int64_t e0 = lo + tid; e0 < hi; e0 += (int64_t)step * kPlacePerThread) {
+    for (int64_t e0 = tid; e0 < hi; e0 += (int64_t)step * kPlacePerThread) {
         int32_t v[kPlacePerThread];
 #pragma unroll
         for (int j = 0; j < kPlacePerThread; ++j) { const int64_t e = e0 + (int64_t)j * step; v[j] = e < hi ? a.ent_repr[e] : 0; }
@@ -1918,8 +1955,11 @@ extern "C" int mg_sample_many(mg_ctx* ctx, const int32_t* targets, int targets_o
 static int sample_kernel_limits(mg_ctx* ctx) {
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_dedupe_last<1024>, (int)(kDedupMaxSlots * 2 * sizeof(int32_t))));
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_dedupe_last<512>, kDedupSlots512 * 2 * (int)sizeof(int32_t)));
-    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_hop<0>,
-                               (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + kTileMax * hop_node_bytes(true)));
+    const int hop_bytes = kTileMax * hop_node_bytes(true) + 8 * MG_MAX_BATCHES;
+    const void* hops[] = {(const void*)k_hop<2>, (const void*)k_hop<3>, (const void*)k_hop<4>, (const void*)k_hop<5>, (const void*)k_hop<6>,
+                          (const void*)k_hop<8>, (const void*)k_hop<10>, (const void*)k_hop<16>, (const void*)k_hop<32>};
+    for (const void* hop : hops) MG_CUDA(ctx, mg_smem_limit(ctx, hop, hop_bytes));
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_hop<0>, (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + hop_bytes));
     return MG_OK;
 }
 
@@ -2116,9 +2156,10 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
             ProfScope ps(ctx, PH_SAMPLE_PICK);
             HopArgs a{d->hdr, h, f, d->nodes, d->node_batch, {ctx->view_off, inout ? ctx->view_off_out : nullptr},
                       {ctx->view_nbrs, ctx->view_nbrs_out}, d->ent_off, d->ent_nbrs, d->ent_repr, d->d_seeds, d->cap_entries, d->tile_state,
-                      hop_tile(nodes_bound[h], ctx->n_sms), ctx->n_sms, B, d->node_off, d->hkeys, d->hvals, tg, ctx->n_nodes, mg_feat_geom(ctx)};
+                      hop_tile(nodes_bound[h], ctx->n_sms), ctx->n_sms, B, k, d->new_ids, batch_cnt + (size_t)(h > 0 ? h - 1 : 0) * B, d->cap_nodes,
+                      inner_limit, d->cum, d->node_off, d->node_off, d->hkeys, d->hvals, tg, ctx->n_nodes, mg_feat_geom(ctx)};
             const unsigned grid = blocks_for(nodes_bound[h], 32, 8);
-            const size_t sm = (size_t)a.tile_cap * hop_node_bytes(inout);   // 36 KiB at most
+            const size_t sm = (size_t)a.tile_cap * hop_node_bytes(inout) + (h > 0 ? 8 * (size_t)B : 0);   // 36 KiB, and 32 at the largest number of mini-batches
             // the narrowest group that holds the fanout among those that waste at most two lanes of a warp
             if (f <= 2) k_hop<2><<<grid, kThreads, sm, st>>>(a);
             else if (f == 3) k_hop<3><<<grid, kThreads, sm, st>>>(a);
@@ -2159,17 +2200,17 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
                 ctx->launches++;
             }
         }
-        {
-            ProfScope ps(ctx, PH_SAMPLE_PLACE);
-            PlaceArgs pa{d->hdr, h, d->new_ids, batch_cnt + (size_t)h * B, d->cap_nodes, d->nodes, d->node_batch,
-                         smem_hop ? nullptr : d->hvals, h < k - 1 ? inner_limit : (int32_t)cap_batch, d->ent_repr, B, k, d->cum, d->node_off, (int32_t)hdr_ints, d->ent_off,
-                         d->rowbase, d->d_ent_hop, d->h_stage_dev + summary_at};
-            const size_t sm = 2 * (size_t)B * sizeof(int32_t);   // 32 KiB at the largest number of mini-batches
-            const unsigned grid = blocks_for(std::max<int64_t>(nodes_bound[h + 1], smem_hop ? 0 : entries_bound[h]), kThreads, 8);
-            if (h == k - 1) k_place<true><<<grid + 1, kThreads, sm, st>>>(pa);
-            else k_place<false><<<grid, kThreads, sm, st>>>(pa);
-            ctx->launches++;
-        }
+    }
+    {
+        ProfScope ps(ctx, PH_SAMPLE_PLACE);
+        const int in_table = smem_last ? k - 1 : k;
+        int64_t table_entries = 0;
+        for (int h = 0; h < in_table; ++h) table_entries += entries_bound[h];
+        PlaceArgs pa{d->hdr, d->new_ids, batch_cnt + (size_t)(k - 1) * B, d->cap_nodes, d->nodes, d->node_batch, d->hvals, in_table, (int32_t)cap_batch,
+                     d->ent_repr, B, k, d->cum, d->node_off, (int32_t)hdr_ints, d->ent_off, d->rowbase, d->d_ent_hop, d->h_stage_dev + summary_at};
+        const size_t sm = 2 * (size_t)B * sizeof(int32_t);   // 32 KiB at the largest number of mini-batches
+        k_place<<<blocks_for(std::max(nodes_bound[k], table_entries), kThreads, 8) + 1, kThreads, sm, st>>>(pa);
+        ctx->launches++;
     }
     MG_CUDA(ctx, cudaGetLastError());
     return MG_OK;
