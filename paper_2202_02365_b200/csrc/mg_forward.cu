@@ -1089,7 +1089,8 @@ struct GatherArgs {
 // memory, lane = row, and then read as one stream, U loads of 512 bytes in flight whatever rows they belong to, with the kept
 // outputs of the rows that end among them beside, or, where the forward pass has left bits of them, one word per column for
 // all rows of the group.  Rows of several units are added up by atomics: mask and bias are
-// linear in the sum.  24 mini-batches of 1,000 targets on 2M nodes: 1.56M rows x 128 in 685 -> 367 us, 543k + 92k rows x 256 in
+// linear in the sum.  24 mini-batches of 1,000 targets on 2M nodes: 1.56M rows x 128 in 685 -> 367 us with eight loads in flight and three
+// blocks per SM, 342 with six and four (four and five: 362), 543k + 92k rows x 256 in
 // 445 -> 388 us (bits: 213 us); 8 mini-batches on 1M nodes, 181k + 34k rows x 256 in 250 -> 141 us (bits: 83 us).  (With the outputs
 // read: four blocks per SM at 64 registers; three at 72 take 481 / 178 us.)
 constexpr int kGradRows = 16, kGradItems = kGradRows * (kGradLight + 1);
@@ -1098,9 +1099,9 @@ constexpr int64_t kGradMaxRows = (1ll << 30) - 1;   // an item holds twice its o
 static_assert(2 * (kGradMaxRows - 1) + 1 < 0x7FFFFFFFll, "an output row's item is not the one that means none");
 enum { RELU_NONE = 0, RELU_ROWS = 1, RELU_BITS = 2 };
 template <int RELU>
-__global__ void __launch_bounds__(kThreads, RELU ? 4 : 1) k_grad_gather(GatherArgs a) {
+__global__ void __launch_bounds__(kThreads, 4) k_grad_gather(GatherArgs a) {
     constexpr bool MASK = RELU != RELU_NONE;
-    constexpr int U = RELU == RELU_NONE ? 8 : 4, kWarps = kThreads / 32;
+    constexpr int U = RELU == RELU_NONE ? 6 : 4, kWarps = kThreads / 32;
     constexpr uint32_t kNone = 0x7FFFFFFFu;       // an item without a contribution
     __shared__ int2 items_sm[kWarps][kGradItems];   // 2 x output row + (1: its neighbour part), weight; sign: the row's last item
     __shared__ int32_t rows_sm[kWarps][kGradRows];
