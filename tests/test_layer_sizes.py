@@ -73,3 +73,11 @@ def test_rows_written_over_the_table(graph, hops, window):
 @pytest.mark.parametrize("d_in,d_out,half,fanout", [(128, 256, False, 4), (256, 100, False, 9), (384, 36, True, 3)])
 def test_rows_on_either_side_of_the_smallest_tiles(graph, rows, d_in, d_out, half, fanout):
     test_rows_on_either_side_of_the_tile_sizes(graph, rows, d_in, d_out, half, fanout)
+
+
+# layers wider than the fused kernel's go through a product of their own: by tile, or (148 SMs: from 296 blocks of 256 rows x 256 columns on)
+# by persistent CTA pairs; K of one and of eight slices, a ragged last block of rows and of columns
+@pytest.mark.parametrize("rows", [37_632, 37_633, 39_999])
+@pytest.mark.parametrize("d_in,d_out", [(16, 300), (128, 512), (100, 260)])
+def test_rows_on_either_side_of_the_persistent_product(graph, rows, d_in, d_out):
+    test_rows_on_either_side_of_the_tile_sizes(graph, rows, d_in, d_out, False, 4)
