@@ -541,6 +541,16 @@ static int finish_forward(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* ou
     return MG_OK;
 }
 
+// mg_layer_rows of all layers into ws_meta, layer l's at meta_at[l]
+static int row_metadata(mg_ctx* ctx, const mg_dense* d, int64_t* meta_at) {
+    for (int l = 1; l <= d->k; ++l) meta_at[l + 1] = meta_at[l] + (int64_t)d->h_hdr.rows_total[l];
+    const size_t need = (size_t)meta_at[d->k + 1];
+    if (ctx->ws_meta_elems < need)
+        if (int rc = mg_ensure(ctx, &ctx->ws_meta, &ctx->ws_meta_elems, need + need / 4 + 4)) return rc;
+    ProfScope ps(ctx, PH_OTHER);
+    return mg_layer_rows(ctx, d, ctx->ws_meta, meta_at);
+}
+
 static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out, int out_mode) {
     int rc;
     const int k = d->k, B = d->n_batches;
@@ -570,14 +580,7 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
     // row metadata of the layers the fused kernel runs, all in one launch
     const bool any_fused = m->precision == MG_GEMM_TF32;
     int64_t meta_at[MG_MAX_HOPS + 2] = {0};
-    for (int l = 1; l <= k; ++l)
-        meta_at[l + 1] = meta_at[l] + (any_fused ? (int64_t)d->h_hdr.rows_total[l] : 0);
-    if (any_fused) {
-        const size_t need = (size_t)meta_at[k + 1];
-        if (ctx->ws_meta_elems < need && (rc = mg_ensure(ctx, &ctx->ws_meta, &ctx->ws_meta_elems, need + need / 4 + 4))) return rc;
-        ProfScope ps(ctx, PH_OTHER);
-        if ((rc = mg_layer_rows(ctx, d, ctx->ws_meta, meta_at))) return rc;
-    }
+    if (any_fused && (rc = row_metadata(ctx, d, meta_at))) return rc;
     // H^k stays in the library's buffer (mg_layer_output, mg_backward) and goes to the caller's: the last layer's kernel
     // stores its tiles to both when it can (the copy behind it read and wrote the rows once more: 41 us for 128,000 rows of
     // 1 KB, and a launch).  Not into the feature table, which other tiles still read.
@@ -947,7 +950,8 @@ struct RevArgs {
     int64_t out_at[MG_MAX_HOPS + 2];   // layer l's output rows are items [out_at[l], out_at[l + 1])
     int64_t in_at[MG_MAX_HOPS + 2];    // its source rows are places [in_at[l], in_at[l + 1]) of cnt
     int64_t ent_at[MG_MAX_HOPS + 2];   // its entries' places in pos
-    const int32_t* ent_off;
+    int32_t rows_per_warp;             // of k_rev_entries: 4 to 32
+    const int4* meta;                  // of the output rows: first entry, entries, first source row of the mini-batch (mg_layer_rows)
     const int32_t* ent_repr;
     uint32_t* cnt;                     // [in_at[k + 1] + 1]: counts, then (scanned) where the lists start
     uint32_t* pos;                     // an entry's place in its source row's list, left by the count for the fill
@@ -967,24 +971,59 @@ struct RevArgs {
     uint32_t* status;                  // the host's word
 };
 
-// 8 lanes per output row
+// A warp takes 32 output rows (fewer where there would not be a warp for every slot of the SMs), lane = row: its metadata is one load.  Their entries are then read as one stream, four per lane in flight,
+// each lane looking up whose its entry is.  Bound by the scattered atomics and list places in L2.  (Eight lanes per row, each row
+// found by a search over the mini-batches, took 2 x 55 us for the 3.7M entries of 24 mini-batches, now 34 + 36.)
 template <bool FILL>
 __global__ void __launch_bounds__(kThreads) k_rev_entries(RevArgs a) {
     if (FILL && *a.bad) return;
-    const int gl = threadIdx.x & 7;
-    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3; i < a.out_at[a.g.k + 1]; i += ((int64_t)gridDim.x * blockDim.x) >> 3) {
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31;
+    const int64_t total = a.out_at[a.g.k + 1], step = (int64_t)gridDim.x * (kThreads / 32) * a.rows_per_warp;
+    for (int64_t i0 = (blockIdx.x * (int64_t)(kThreads / 32) + (threadIdx.x >> 5)) * a.rows_per_warp; i0 < total; i0 += step) {
+        const int64_t i = min(i0 + lane, total - 1);
         int layer = a.l0;
         while (i >= a.out_at[layer + 1]) ++layer;
-        const int64_t row = i - a.out_at[layer];
-        int32_t b, local, node;
-        locate_row(a.g, layer, row, &b, &local, &node);
-        const int32_t e0 = a.ent_off[node], e1 = a.ent_off[node + 1];
-        const int64_t in0 = a.in_at[layer] + a.g.rowbase[(int64_t)(layer - 1) * (a.g.B + 1) + b];
-        const float w = a.sum_aggr ? 1.f : 1.f / (float)(e1 - e0);
-        for (int32_t e = e0 + gl; e < e1; e += 8) {
-            const int64_t src = in0 + a.ent_repr[e];
-            if (FILL) a.rev[a.cnt[src] + a.pos[a.ent_at[layer] + e]] = make_int2((int32_t)row, __float_as_int(w));
-            else a.pos[a.ent_at[layer] + e] = atomicAdd(&a.cnt[src], 1u);
+        const int4 m = __ldg(a.meta + i);
+        const int32_t n = lane < a.rows_per_warp && i0 + lane < total ? m.z : 0;
+        const int32_t end = (int32_t)warp_incl_scan((uint32_t)n), all = __shfl_sync(0xFFFFFFFFu, end, 31);
+        const int32_t row = (int32_t)(i - a.out_at[layer]);
+        const int32_t ent = m.y - (end - n);                        // entry j of the stream is ent + j of the arena
+        const int64_t src0 = a.in_at[layer] + m.w;                  // row 0 of the mini-batch among the layer's source rows
+        const int64_t pos0 = a.ent_at[layer] + ent;
+        const float w = a.sum_aggr ? 1.f : 1.f / (float)m.z;
+        for (int32_t j0 = 0; j0 < all; j0 += 32 * U) {
+            int32_t repr[U], own[U];
+            uint32_t at[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int32_t j = min(j0 + u * 32 + lane, all - 1);
+                int o = 0;   // the first row whose entries end behind j
+#pragma unroll
+                for (int s = 16; s > 0; s >>= 1)
+                    if (__shfl_sync(0xFFFFFFFFu, end, o + s - 1) <= j) o += s;
+                own[u] = o;
+                repr[u] = __ldg(a.ent_repr + __shfl_sync(0xFFFFFFFFu, ent, o) + j);
+                if (FILL) at[u] = a.pos[__shfl_sync(0xFFFFFFFFu, pos0, o) + j];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t src = __shfl_sync(0xFFFFFFFFu, src0, own[u]) + repr[u];
+                const bool on = j0 + u * 32 + lane < all;
+                if (FILL) at[u] += a.cnt[src];
+                else if (on) at[u] = atomicAdd(&a.cnt[src], 1u);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int32_t j = j0 + u * 32 + lane;
+                if (FILL) {
+                    const int2 item = make_int2(__shfl_sync(0xFFFFFFFFu, row, own[u]), __shfl_sync(0xFFFFFFFFu, __float_as_int(w), own[u]));
+                    if (j < all) a.rev[at[u]] = item;
+                } else {
+                    const int64_t p = __shfl_sync(0xFFFFFFFFu, pos0, own[u]) + j;
+                    if (j < all) a.pos[p] = at[u];
+                }
+            }
         }
     }
 }
@@ -1341,10 +1380,15 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     const RowGeom geom{B, k, d->rowbase, d->cum, d->node_off};
     const bool half = ctx->feat_dtype == MG_DTYPE_F16;
     const int grid = mg_grid(ctx, 8);
+    if (m->precision == MG_GEMM_FP32) {   // (the forward pass of the others has left it)
+        int64_t meta_at[MG_MAX_HOPS + 2] = {0};
+        if ((rc = row_metadata(ctx, d, meta_at))) return rc;
+    }
     // (behind the last layer's products: the scan clears rows of the inputs' gradients, and d_h0_dev may lie where d_out_dev does)
     auto turn_entries_round = [&]() -> int {
         ra.g = geom;
-        ra.ent_off = d->ent_off; ra.ent_repr = d->ent_repr; ra.sum_aggr = m->sum_aggr ? 1 : 0;
+        ra.meta = ctx->ws_meta + (ra.l0 > 1 ? (int64_t)d->h_hdr.rows_total[1] : 0);
+        ra.ent_repr = d->ent_repr; ra.sum_aggr = m->sum_aggr ? 1 : 0;
         ra.ticket = ctx->bw_off;
         ra.n_units = ra.ticket + 1;
         static_assert(MG_MAX_HOPS % 2 == 0, "the states are 8-byte aligned behind the counters");
@@ -1359,7 +1403,10 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         ra.status = ctx->d_flags;
         for (int l = ra.l0; l <= k; ++l) { ra.g_in[l] = l > 1 ? ctx->bw_g + g_off[l - 1] : d_h0_dev; ra.d_in[l] = m->dims[l - 1]; }
         MG_CUDA(ctx, cudaMemsetAsync(ctx->bw_off, 0, sizeof(uint32_t) * cleared, st));
-        const int rgrid = (int)std::min<int64_t>(grid, (8 * ra.out_at[k + 1] + kThreads - 1) / kThreads);
+        ra.rows_per_warp = 4;
+        while (ra.rows_per_warp < 32 && ra.out_at[k + 1] > (int64_t)ra.rows_per_warp * grid * (kThreads / 32)) ra.rows_per_warp *= 2;
+        const int64_t per_block = (int64_t)ra.rows_per_warp * (kThreads / 32);
+        const int rgrid = (int)std::min<int64_t>(grid, (ra.out_at[k + 1] + per_block - 1) / per_block);
         k_rev_entries<false><<<rgrid, kThreads, 0, st>>>(ra);
         k_rev_scan<<<(unsigned)rev_tiles, kThreads, 0, st>>>(ra);
         k_rev_entries<true><<<rgrid, kThreads, 0, st>>>(ra);

@@ -1072,7 +1072,7 @@ __global__ void __launch_bounds__(256) k_layer_rows(RowsArgs a, int4* __restrict
         while (h < a.k - layer && l >= cum[h + 1]) ++h;
         const int32_t idx = a.node_off[h * (a.B + 1) + b] + (l - cum[h]);
         const int32_t e0 = a.ent_off[idx];
-        const int32_t in_base = layer == 1 ? 0 : rb[b - (a.B + 1)];
+        const int32_t in_base = rb[b - (a.B + 1)];
         meta[i] = make_int4(layer == 1 ? (int32_t)feat_row(a.feat, a.nodes[idx]) : in_base + l, e0, a.ent_off[idx + 1] - e0, in_base);
     }
 }
