@@ -1297,7 +1297,8 @@ __global__ void __launch_bounds__(kThreads) k_export_entries(ExportArgs a) {
 // so that a node's place in the packed entries falls out of its place in the bin.  Targets keep the caller's order and take no part.
 // Bound by the latency of a few dependent passes over what stays in L2.  Before, a radix sort of three passes with a scan each, a kernel
 // for the order and a scan of all counts, 24 kernels: 310 us for 32 mini-batches of 114,000 nodes on a graph of 8M, now 175 us (begin 5,
-// count 16, split 31, order 76, entries 37, and their gaps).
+// count 16, split 31, order 76, entries 37, and their gaps).  (Two bins per warp and not eight: ordering 4 mini-batches of
+// 300 targets takes 12 us instead of 34, one of 1,000 14 instead of 25.)
 struct ExportSeg {
     int32_t in0, len;        // its nodes in the arena
     int32_t out0;            // its first row in the packed canonical node list
@@ -1533,8 +1534,8 @@ __global__ void __launch_bounds__(kThreads) k_export_split(ExportManyArgs a) {
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_export_order(ExportManyArgs a) {
-    constexpr int kWarps = kThreads / 32, kMapWords = (1 << kExportMapLog) / 32, kBinsPerWarp = 8;
+__global__ void __launch_bounds__(kThreads, 6) k_export_order(ExportManyArgs a) {
+    constexpr int kWarps = kThreads / 32, kMapWords = (1 << kExportMapLog) / 32, kBinsPerWarp = 2;
     __shared__ __align__(16) uint32_t map[kMapWords];   // a bitmap, or the ids of bins that are compared all with all
     __shared__ uint16_t below[kMapWords];               // set bits before a word among those of its warp
     __shared__ uint32_t warp_tot[kWarps];
@@ -1550,7 +1551,11 @@ __global__ void __launch_bounds__(kThreads) k_export_order(ExportManyArgs a) {
         const int32_t start = bin_start(g, bin), n = (int32_t)a.bin_end[bin] - start;
         const int2* __restrict__ keys = a.keys + start;
         const bool sampled = g.hop < a.k;
-        if (n <= kExportPairKeys && g.shift > kExportMapLog) {
+        // All with all: instructions by the square of the bin; bitmaps: by their number, where the bin's range takes several (in
+        // units of what a warp issues for 512 words; a graph of 111M nodes has two bitmaps per bin, and comparing its bins of up
+        // to 1,024 ids all with all took the export of 128 mini-batches from 1.27 to 1.96 ms)
+        const int64_t bitmaps = g.shift > kExportMapLog ? 1ll << (g.shift - kExportMapLog) : 1;
+        if (n <= kExportPairKeys && bitmaps > 1 && (int64_t)((n + kThreads - 1) / kThreads) * n * 2 <= bitmaps * 512) {
             constexpr int kPer = kExportPairKeys / kThreads;
             __syncthreads();
             int2 key[kPer];
@@ -1566,7 +1571,8 @@ __global__ void __launch_bounds__(kThreads) k_export_order(ExportManyArgs a) {
             for (int i = 0; i < n; i += 4) {
                 const int4 v = *reinterpret_cast<const int4*>(&map[i]);
 #pragma unroll
-                for (int r = 0; r < kPer; ++r) rank[r] += (v.x < key[r].x) + (v.y < key[r].x) + (v.z < key[r].x) + (v.w < key[r].x);
+                for (int r = 0; r < kPer; ++r)
+                    if (r == 0 || n > r * kThreads) rank[r] += (v.x < key[r].x) + (v.y < key[r].x) + (v.z < key[r].x) + (v.w < key[r].x);
             }
 #pragma unroll
             for (int r = 0; r < kPer; ++r)
@@ -1632,7 +1638,7 @@ __global__ void __launch_bounds__(kThreads) k_export_order(ExportManyArgs a) {
         }
     }
     __syncthreads();
-    // the others: a warp looks eight consecutive bins up at once (lane = bin) and takes them one after the other
+    // the others: a warp looks two consecutive bins up at once (lane = bin) and takes them one after the other
     int32_t* ids = reinterpret_cast<int32_t*>(map) + warp * kExportWarpKeys;
     for (int32_t b0 = ((int32_t)blockIdx.x * kWarps + warp) * kBinsPerWarp; b0 < n_bins; b0 += (int32_t)gridDim.x * kWarps * kBinsPerWarp) {
         int32_t my_seg = 0, my_start = 0, my_n = 0;
