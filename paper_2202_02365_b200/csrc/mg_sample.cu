@@ -1958,14 +1958,20 @@ extern "C" int mg_sample_many(mg_ctx* ctx, const int32_t* targets, int targets_o
 
 
 // dynamic shared-memory limits of the sampler's kernels (not inside a stream capture)
+constexpr int kHopSmem = kTileMax * (12 + 24) + 8 * MG_MAX_BATCHES;   // of k_hop at most: a tile with both directions, the mini-batches' tables
 static int sample_kernel_limits(mg_ctx* ctx) {
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_dedupe_last<1024>, (int)(kDedupMaxSlots * 2 * sizeof(int32_t))));
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_dedupe_last<512>, kDedupSlots512 * 2 * (int)sizeof(int32_t)));
-    const int hop_bytes = kTileMax * hop_node_bytes(true) + 8 * MG_MAX_BATCHES;
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_hop<0>, (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + kHopSmem));
+    return MG_OK;
+}
+
+// ... and of the others where the mini-batches' tables of k_hop, beside its tile, come to more than a kernel has without asking
+static int hop_kernel_limits(mg_ctx* ctx, int32_t n_batches, bool inout) {
+    if (kTileMax * hop_node_bytes(inout) + 8 * n_batches <= 47 * 1024) return MG_OK;   // (48 KiB, of which k_hop has some for itself)
     const void* hops[] = {(const void*)k_hop<2>, (const void*)k_hop<3>, (const void*)k_hop<4>, (const void*)k_hop<5>, (const void*)k_hop<6>,
                           (const void*)k_hop<8>, (const void*)k_hop<10>, (const void*)k_hop<16>, (const void*)k_hop<32>};
-    for (const void* hop : hops) MG_CUDA(ctx, mg_smem_limit(ctx, hop, hop_bytes));
-    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_hop<0>, (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + hop_bytes));
+    for (const void* hop : hops) MG_CUDA(ctx, mg_smem_limit(ctx, hop, kHopSmem));
     return MG_OK;
 }
 
@@ -2129,6 +2135,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
         st_hdr->targets = (uint64_t)(uintptr_t)d->newlist[1];
     }
     if ((rc = sample_kernel_limits(ctx))) return rc;
+    if ((rc = hop_kernel_limits(ctx, B, inout))) return rc;
 
     // Grids follow what a hop can hold at most (the number of targets rounded up to a power of two, so that calls of similar
     // size share the captured graph): blocks without work cost the small calls as much as the work itself.

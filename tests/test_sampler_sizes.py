@@ -197,3 +197,20 @@ def test_export_orders_deltas_of_any_size_and_spread(stride):
         assert torch.equal(x.node_ids[x.repr_map.long()], x.nbrs)
     c.close()
     torch.cuda.empty_cache()
+
+
+# the tables of k_hop over the mini-batches beside its largest tile: more shared memory than a kernel has without asking
+@pytest.mark.parametrize("fanout", [9, 40])
+def test_largest_tiles_with_as_many_mini_batches_as_a_call_may_have(graph, ctx, fanout):
+    n_batches, per = 4_096, 40
+    rows = [inputs.distinct_targets(N, per - b % 7, seed=b) for b in range(n_batches)]
+    offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    d = ctx.sample_many(torch.cat(rows), offs, [fanout, fanout], list(range(n_batches)), caps={"max_nodes_per_batch": 4_000, "max_nodes_total": 4_000_000 * 3,
+                                                                                              "max_entries_total": 4_000_000 * 3})
+    for b in (0, 1, 2_047, n_batches - 1):
+        one = ctx.sample(rows[b], [fanout, fanout], b)
+        x, y = d.view(b), one.view(0)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
+        one.free()
+    d.free()
