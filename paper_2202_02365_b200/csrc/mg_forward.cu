@@ -673,6 +673,7 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
             ctx->agg_at[l] = kept ? floats : -1;
             if (kept) floats += (int64_t)d->h_hdr.rows_total[l] * m->dims[l - 1];
         }
+        ctx->agg_sum = m->sum_aggr;
         if (floats > 0 && ctx->ws_agg_elems < (size_t)floats && mg_ensure(ctx, &ctx->ws_agg, &ctx->ws_agg_elems, (size_t)(floats + floats / 4)))
             for (int l = 1; l <= k; ++l) ctx->agg_at[l] = -1;   // (no room: gathered again)
     }
@@ -1434,7 +1435,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
             // dW += X^T dPre with X gathered again inside the kernel; the row metadata is what the forward pass left (its layers all
             // have it, mg_forward of this very model and sample was the last to write it)
             if ((rc = mg_layer_grad_weights(ctx, d, l, d_in, d_out, h_prev, dpre_all, ctx->ws_meta + meta_at, m->sum_aggr ? 1 : 0,
-                                            ctx->agg_at[l] >= 0 ? ctx->ws_agg + ctx->agg_at[l] : nullptr, m->g_w_cat[l - 1]))) return rc;
+                                            ctx->agg_at[l] >= 0 && ctx->agg_sum == m->sum_aggr ? ctx->ws_agg + ctx->agg_at[l] : nullptr, m->g_w_cat[l - 1]))) return rc;
             // dX = dPre W^T on the tensor cores: the K-major operand the kernel wants is W itself ([2 d_in, d_out])
             if (g_in && (rc = mg_gemm_tf32(ctx, dpre_all, m->w_cat[l - 1], m->zeros, ctx->bw_dx, M, 2 * d_in, d_out, false))) return rc;
         }

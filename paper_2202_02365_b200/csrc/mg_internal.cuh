@@ -144,6 +144,7 @@ struct mg_ctx {
     bool keep_layers = false;          // keep H^1..H^{k-1} for mg_layer_output (whole-layer schedule)
     bool layers_kept = false;          // what the last forward did
     int64_t agg_at[MG_MAX_HOPS + 1] = {0};        // where layer l's rows of ws_agg start (floats); below zero: it left none
+    bool agg_sum = false;                         // ... by the model's aggregator at the time
     int64_t positive_at[MG_MAX_HOPS + 1] = {0};   // where layer l's bits of ws_positive start (32-bit words); below zero: it left none
 
     // asynchronous output copy of mg_forward_host_async

@@ -290,3 +290,23 @@ def test_what_the_forward_pass_keeps_for_the_backward_pass(sizes, dims, aggregat
     # the same operands; fp32 sums over up to 6,000 rows meet in any order: sqrt(6,000) 2^-24 of the terms' norm, where terms cancel more
     for x, y in zip(got[0][1:2] + got[0][3:], got[1][1:2] + got[1][3:]):
         assert float((x.double() - y.double()).norm()) <= 1e-4 * max(float(x.double().norm()), 1e-12)
+
+
+# an aggregator that is set between the two passes: the backward pass takes its own, whatever the forward pass has left
+def test_aggregator_set_between_the_passes():
+    graph = inputs.erdos_renyi_graph(N, 9 * N, seed=31)
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.load_features(inputs.normal_features(N, 16, seed=32, device="cuda"))
+    dense = ctx.sample(inputs.distinct_targets(N, 300, seed=33), [7, 5], seed=34)
+    model = ctx.model(inputs.random_bias_layers([16, 32, 8], seed=35))
+    d_out = torch.randn((300, 8), generator=torch.Generator("cuda").manual_seed(36), device="cuda")
+    got = []
+    for keep in (False, True):
+        ctx.keep_layer_outputs(keep)
+        model.set_aggregator("mean")
+        ctx.forward(model, dense, torch.empty_like(d_out))
+        model.set_aggregator("sum")
+        got.append([x.clone() for layer in ctx.backward(model, dense, d_out) for x in layer])
+    for x, y in zip(*got):      # (the same operands, sums in any order)
+        assert float((x.double() - y.double()).norm()) <= 1e-4 * float(x.double().norm())
