@@ -202,6 +202,7 @@ struct mg_dense {
     int64_t cap_nodes = 0, cap_entries = 0;
     int32_t table_size = 0;  // slots per batch, power of two
     int64_t n_targets_total = 0;
+    int64_t n_nodes = 0;     // of the graph that was sampled: ids lie below it (the context may have loaded another one since)
 
     // device arrays
     DenseHeader* hdr = nullptr;

@@ -2077,6 +2077,7 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     *out = d;
     for (int h = 0; h < k; ++h) d->fanouts[h] = fanouts[h];
     d->n_targets_total = T;
+    d->n_nodes = N;
     d->resident_serial = ctx->resident_serial;
     d->slot_of_part_at_sample = ctx->slot_of_part;
 
@@ -2327,7 +2328,7 @@ int mg_dense_batch_perm(mg_ctx* ctx, mg_dense* d, int b, const int32_t** perm, c
     cudaStream_t st = ctx->stream;
     if (d->export_pending) MG_CUDA(ctx, cudaStreamWaitEvent(st, d->ev_exported, 0));   // the export uses the same sort scratch
     const int32_t n = g.V - g.n_targets;
-    const int id_bits = std::max(1, ilog2_ceil(ctx->n_nodes)), hop_bits = std::max(1, ilog2_ceil(g.k + 1));
+    const int id_bits = std::max(1, ilog2_ceil(d->n_nodes)), hop_bits = std::max(1, ilog2_ceil(g.k + 1));
     const int grid = std::max(1, std::min(mg_grid(ctx, 4), (g.V + kThreads - 1) / kThreads));
     int res = 0;
     if (n > 0) {
@@ -2435,7 +2436,7 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
     cudaStream_t st = ctx->sample_stream;
     ExportManyArgs a;
     memset(&a, 0, sizeof(a));
-    a.B = B; a.k = k; a.id_bits = std::max(1, ilog2_ceil(ctx->n_nodes));
+    a.B = B; a.k = k; a.id_bits = std::max(1, ilog2_ceil(d->n_nodes));
     for (int h = 0; h <= k + 1; ++h) a.hop_base[h] = d->h_hdr.hop_base[h];
     a.nodes = d->nodes; a.node_batch = d->node_batch; a.node_off = d->node_off; a.cum = d->cum; a.rowbase0 = d->rowbase;
     a.ent_hop = d->d_ent_hop; a.ent_off = d->ent_off; a.ent_nbrs = d->ent_nbrs; a.ent_repr = d->ent_repr;

@@ -214,3 +214,24 @@ def test_largest_tiles_with_as_many_mini_batches_as_a_call_may_have(graph, ctx, 
             assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
         one.free()
     d.free()
+
+
+# ids are as wide as the graph that was sampled has them, whatever the context has loaded since
+@pytest.mark.parametrize("n_later", [500, 4 * N])
+def test_arrays_of_a_sample_whose_graph_has_been_replaced(graph, n_later):
+    c = mg.Context(0)
+    c.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    rows = [inputs.distinct_targets(N, n, seed=n) for n in (700, 1, 90)]
+    offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    keys = ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map")
+    d = c.sample_many(torch.cat(rows), offs, [4, 3], [1, 2, 3])
+    d.export_many()
+    want = [{key: getattr(d.export_view(b), key).clone() for key in keys} for b in range(len(rows))]
+    later = inputs.erdos_renyi_graph(n_later, 4 * n_later, seed=5)
+    c.load_graph(later.row_offsets.cuda(), later.nbrs.cuda())
+    d.export_many()
+    for b, arrays in enumerate(want):
+        for v in (d.export_view(b), d.view(b)):
+            for key in keys:
+                assert torch.equal(getattr(v, key), arrays[key]), (b, key)
+    c.close()
