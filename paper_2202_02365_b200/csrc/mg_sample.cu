@@ -1292,13 +1292,16 @@ __global__ void __launch_bounds__(kThreads) k_export_entries(ExportArgs a) {
 // A segment is a (mini-batch, delta) pair; in output order mini-batch follows mini-batch, inside it the farthest delta comes
 // first.  Its ids are distinct, so a node's place in it is the number of smaller ids.  The ids are split by their top bits
 // into bins -- counted per tile (k_export_count), written bin after bin in any order (k_export_split) --, and then ordered bin by bin
-// (k_export_order): a warp compares the ids of a bin of up to 128 all with all, a block takes a larger one through a bitmap of the
-// bin's range in shared memory, whose set bits below an id are its rank.  The same bins carry the sampled nodes' entry counts,
+// (k_export_order): a warp compares the ids of a bin of up to 128 all with all, a block takes a larger one through bitmaps in
+// shared memory, whose set bits below an id are its rank.  The same bins carry the sampled nodes' entry counts,
 // so that a node's place in the packed entries falls out of its place in the bin.  Targets keep the caller's order and take no part.
 // Bound by the latency of a few dependent passes over what stays in L2.  Before, a radix sort of three passes with a scan each, a kernel
-// for the order and a scan of all counts, 24 kernels: 310 us for 32 mini-batches of 114,000 nodes on a graph of 8M, now 175 us (begin 5,
-// count 16, split 31, order 76, entries 37, and their gaps).  (Two bins per warp and not eight: ordering 4 mini-batches of
+// for the order and a scan of all counts, 24 kernels: 310 us for 32 mini-batches of 114,000 nodes on a graph of 8M, now 150 us (begin 6,
+// count 18, split 28, order 50, entries 35, and their gaps).  (Two bins per warp and not eight: ordering 4 mini-batches of
 // 300 targets takes 12 us instead of 34, one of 1,000 14 instead of 25.)
+// A segment has as many bins as give it 32 to 64 nodes each, up to 4,096.  With 512 at most the bins of a delta of 100,000 nodes went to blocks
+// instead of warps, and ids next to each other into a handful of bins: the export of 128 mini-batches on a graph of 111M nodes 1.26 ms (now 0.69;
+// the radix sort 1.29), there the order alone of 32 deltas of 100,000 spread ids 246 us (now 54) and of 100,000 consecutive ones 278 (now 139).
 struct ExportSeg {
     int32_t in0, len;        // its nodes in the arena
     int32_t out0;            // its first row in the packed canonical node list
@@ -1327,13 +1330,13 @@ struct ExportManyArgs {
     int32_t* dense_bins;     // the bins of more than kExportWarpKeys nodes
 };
 
-constexpr int kExportBinsLog = 9;      // bins of a segment at most
+constexpr int kExportBinsLog = 12;     // bins of a segment at most
 constexpr int kExportWarpKeys = 128;   // keys that a warp compares all with all
 constexpr int kExportPairKeys = 1024;  // ... and a block, where the bin's range takes more than one bitmap
 constexpr int kExportMapLog = 17;      // ids of a bitmap
-static_assert((1 << kExportBinsLog) == 2 * kThreads, "two bins per thread");
+constexpr int kExportBinsPerThread = (1 << kExportBinsLog) / kThreads;
 
-// bins of a segment: a power of two that gives them 32 to 64 nodes on average (more in the longest segments); none where nothing
+// bins of a segment: a power of two that gives them 32 to 64 nodes on average (more in segments of over 262,144); none where nothing
 // is to be ordered
 __device__ __forceinline__ int export_bins_log(int32_t len, int id_bits) {
     const int want = len <= 64 ? 0 : 32 - __clz((len - 1) >> 6);
@@ -1461,22 +1464,24 @@ __global__ void __launch_bounds__(kThreads) k_export_count(ExportManyArgs a) {
         __syncthreads();
         if (!last) continue;
         __threadfence();
-        const int q0 = 2 * (int)threadIdx.x;   // two bins per thread
-        uint32_t c[2], e[2];
+        const int per = max(1, g.bins / kThreads), q0 = per * (int)threadIdx.x;   // (bins are a power of two)
+        uint32_t c[kExportBinsPerThread], e[kExportBinsPerThread], c_sum = 0, e_sum = 0;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const bool on = q0 + q < g.bins;
+        for (int q = 0; q < kExportBinsPerThread; ++q) {
+            const bool on = q < per && q0 + q < g.bins;
             c[q] = on ? __ldcg(&a.bin_end[g.bin0 + q0 + q]) : 0u;
             e[q] = on ? __ldcg(&a.bin_ents[g.bin0 + q0 + q]) : 0u;
         }
-        const uint32_t ci = warp_incl_scan(c[0] + c[1]), ei = warp_incl_scan(e[0] + e[1]);
+#pragma unroll
+        for (int q = 0; q < kExportBinsPerThread; ++q) { c_sum += c[q]; e_sum += e[q]; }
+        const uint32_t ci = warp_incl_scan(c_sum), ei = warp_incl_scan(e_sum);
         if (lane == 31) { part[0][warp] = ci; part[1][warp] = ei; }
         __syncthreads();
-        uint32_t c_at = (uint32_t)g.out0 + ci - c[0] - c[1], e_at = (uint32_t)g.ent_rel + ei - e[0] - e[1];
+        uint32_t c_at = (uint32_t)g.out0 + ci - c_sum, e_at = (uint32_t)g.ent_rel + ei - e_sum;
         for (int w = 0; w < warp; ++w) { c_at += part[0][w]; e_at += part[1][w]; }
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            if (q0 + q >= g.bins) break;
+        for (int q = 0; q < kExportBinsPerThread; ++q) {
+            if (q >= per || q0 + q >= g.bins) break;
             const int32_t bin = g.bin0 + q0 + q;
             a.bin_end[bin] = c_at;
             a.bin_ents[bin] = e_at;
@@ -1534,11 +1539,11 @@ __global__ void __launch_bounds__(kThreads) k_export_split(ExportManyArgs a) {
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 6) k_export_order(ExportManyArgs a) {
+__global__ void __launch_bounds__(kThreads, 5) k_export_order(ExportManyArgs a) {
     constexpr int kWarps = kThreads / 32, kMapWords = (1 << kExportMapLog) / 32, kBinsPerWarp = 2;
     __shared__ __align__(16) uint32_t map[kMapWords];   // a bitmap, or the ids of bins that are compared all with all
     __shared__ uint16_t below[kMapWords];               // set bits before a word among those of its warp
-    __shared__ uint32_t warp_tot[kWarps];
+    __shared__ uint32_t warp_tot[kWarps], warp_lo[kWarps], warp_hi[kWarps], warp_next[kWarps];
     static_assert(kWarps * kExportWarpKeys <= kMapWords && kExportPairKeys <= kMapWords, "ids fit the bitmap's place");
     static_assert(kMapWords / kWarps * 32 <= 65536 && kMapWords % (32 * kWarps) == 0, "a warp's words");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1551,10 +1556,33 @@ __global__ void __launch_bounds__(kThreads, 6) k_export_order(ExportManyArgs a) 
         const int32_t start = bin_start(g, bin), n = (int32_t)a.bin_end[bin] - start;
         const int2* __restrict__ keys = a.keys + start;
         const bool sampled = g.hop < a.k;
-        // All with all: instructions by the square of the bin; bitmaps: by their number, where the bin's range takes several (in
-        // units of what a warp issues for 512 words; a graph of 111M nodes has two bitmaps per bin, and comparing its bins of up
-        // to 1,024 ids all with all took the export of 128 mini-batches from 1.27 to 1.96 ms)
-        const int64_t bitmaps = g.shift > kExportMapLog ? 1ll << (g.shift - kExportMapLog) : 1;
+        const uint32_t id0 = (uint32_t)(bin - g.bin0) << g.shift;
+        auto for_keys = [&](auto&& f) {   // (id inside the bin's range, local row), four loads in flight per thread
+            for (int32_t i0 = threadIdx.x; i0 < n; i0 += 4 * kThreads) {
+                int2 key[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) key[u] = i0 + u * kThreads < n ? keys[i0 + u * kThreads] : make_int2(-1, 0);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) if (key[u].x >= 0) f((uint32_t)key[u].x - id0, key[u].y);
+            }
+        };
+        // The range that the bin's ids really have: bitmaps start at the smallest id and skip what has none, so that their number
+        // follows the ids and not the width of a bin (of a graph of 111M nodes: 27,000 ids in a segment of more than 131,072 nodes, up to
+        // all of them in one of 64).
+        uint32_t lo = 0, hi = (1u << g.shift) - 1u;
+        if (g.shift > kExportMapLog) {
+            uint32_t first = hi, last = 0;
+            for_keys([&](uint32_t at, int32_t) { first = min(first, at); last = max(last, at); });
+            first = __reduce_min_sync(0xFFFFFFFFu, first);
+            last = __reduce_max_sync(0xFFFFFFFFu, last);
+            if (lane == 0) { warp_lo[warp] = first; warp_hi[warp] = last; }
+            __syncthreads();
+            lo = warp_lo[0]; hi = warp_hi[0];
+            for (int q = 1; q < kWarps; ++q) { lo = min(lo, warp_lo[q]); hi = max(hi, warp_hi[q]); }
+        }
+        // All with all: instructions by the square of the bin; bitmaps: by their words, where the ids' range takes several (in
+        // units of what a warp issues for 512 words)
+        const int64_t bitmaps = ((hi - lo) >> kExportMapLog) + 1;
         if (n <= kExportPairKeys && bitmaps > 1 && (int64_t)((n + kThreads - 1) / kThreads) * n * 2 <= bitmaps * 512) {
             constexpr int kPer = kExportPairKeys / kThreads;
             __syncthreads();
@@ -1581,18 +1609,19 @@ __global__ void __launch_bounds__(kThreads, 6) k_export_order(ExportManyArgs a) 
                     if (sampled) a.o_nbr_off[start + rank[r] + g.off_shift] = key[r].y;   // (until the counts are summed up below)
                 }
         } else {
-            const int map_log = max(5, min(g.shift, kExportMapLog));
-            const int words = 1 << (map_log - 5), warp_words = max(32, words / kWarps);
-            const int32_t id0 = (bin - g.bin0) << g.shift;
             uint32_t before = 0;   // ids in the bitmaps so far
-            for (int64_t sub = 0; sub < 1ll << g.shift; sub += 1ll << map_log) {
+            for (;;) {
+                const int words = (int)min((hi - lo) / 32 + 1, (uint32_t)kMapWords);
+                const int warp_words = (words + 32 * kWarps - 1) / (32 * kWarps) * 32;
+                uint32_t next = UINT32_MAX;   // the smallest id behind this bitmap
                 __syncthreads();
                 for (int i = threadIdx.x; i < words; i += kThreads) map[i] = 0u;
                 __syncthreads();
-                for (int32_t i = threadIdx.x; i < n; i += kThreads) {
-                    const int64_t at = (int64_t)(keys[i].x - id0) - sub;
-                    if (at >= 0 && at < 1ll << map_log) atomicOr(&map[at >> 5], 1u << (at & 31));
-                }
+                for_keys([&](uint32_t at, int32_t) {
+                    if (at < lo) return;
+                    if (at - lo < 32u * kMapWords) atomicOr(&map[(at - lo) >> 5], 1u << ((at - lo) & 31));
+                    else next = min(next, at);
+                });
                 __syncthreads();
                 uint32_t run = 0;
                 for (int i = warp * warp_words + lane; i < min(words, (warp + 1) * warp_words) + lane; i += 32) {
@@ -1601,40 +1630,47 @@ __global__ void __launch_bounds__(kThreads, 6) k_export_order(ExportManyArgs a) 
                     if (i < words) below[i] = (uint16_t)(run + inc - c);
                     run += __shfl_sync(0xFFFFFFFFu, inc, 31);
                 }
-                if (lane == 0) warp_tot[warp] = run;
+                next = __reduce_min_sync(0xFFFFFFFFu, next);
+                if (lane == 0) { warp_tot[warp] = run; warp_next[warp] = next; }
                 __syncthreads();
-                for (int32_t i = threadIdx.x; i < n; i += kThreads) {
-                    const int2 key = keys[i];
-                    const int64_t at = (int64_t)(key.x - id0) - sub;
-                    if (at < 0 || at >= 1ll << map_log) continue;
-                    const int wd = (int)(at >> 5);
-                    uint32_t rank = before + below[wd] + (uint32_t)__popc(map[wd] & ((1u << (at & 31)) - 1u));
+                for_keys([&](uint32_t at, int32_t local) {
+                    if (at < lo || at - lo >= 32u * kMapWords) return;
+                    const int wd = (int)((at - lo) >> 5);
+                    uint32_t rank = before + below[wd] + (uint32_t)__popc(map[wd] & ((1u << ((at - lo) & 31)) - 1u));
                     for (int q = 0; q < wd / warp_words; ++q) rank += warp_tot[q];
-                    export_node(a, g, start + (int32_t)rank, key.x, key.y);
-                    if (sampled) a.o_nbr_off[start + (int32_t)rank + g.off_shift] = key.y;
-                }
-                for (int q = 0; q < kWarps; ++q) before += warp_tot[q];
+                    export_node(a, g, start + (int32_t)rank, (int32_t)(id0 + at), local);
+                    if (sampled) a.o_nbr_off[start + (int32_t)rank + g.off_shift] = local;
+                });
+                for (int q = 0; q < kWarps; ++q) { before += warp_tot[q]; next = min(next, warp_next[q]); }
+                if (next == UINT32_MAX) break;
+                lo = next;
             }
         }
         if (!sampled) continue;
-        // in order now: the nodes' entry counts, summed up from the bin's first entry on
+        // in order now: the nodes' entry counts, summed up from the bin's first entry on, four consecutive nodes per thread
         uint32_t run = a.bin_ents[bin];
-        for (int32_t i0 = 0; i0 < n; i0 += kThreads) {
+        for (int32_t i0 = 0; i0 < n; i0 += 4 * kThreads) {
             __syncthreads();
-            const int32_t i = i0 + (int32_t)threadIdx.x, c = start + i;
-            int32_t local = 0;
-            uint32_t ents = 0;
-            if (i < n) {
-                local = a.o_nbr_off[c + g.off_shift];
-                const int32_t at = g.in0 + local - g.lrow0;
-                ents = (uint32_t)(a.ent_off[at + 1] - a.ent_off[at]);
+            const int32_t i = i0 + 4 * (int32_t)threadIdx.x, c = start + i;
+            int32_t local[4];
+            uint32_t ents[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) local[u] = i + u < n ? a.o_nbr_off[c + u + g.off_shift] : -1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int32_t at = g.in0 + local[u] - g.lrow0;
+                ents[u] = local[u] >= 0 ? (uint32_t)(a.ent_off[at + 1] - a.ent_off[at]) : 0u;
             }
-            const uint32_t inc = warp_incl_scan(ents);
+            const uint32_t mine = ents[0] + ents[1] + ents[2] + ents[3], inc = warp_incl_scan(mine);
             if (lane == 31) warp_tot[warp] = inc;
             __syncthreads();
-            uint32_t rel = run + inc - ents;
+            uint32_t rel = run + inc - mine;
             for (int q = 0; q < kWarps; ++q) { if (q < warp) rel += warp_tot[q]; run += warp_tot[q]; }
-            if (i < n) export_offset(a, g, c, local, (int32_t)rel);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (local[u] >= 0) export_offset(a, g, c + u, local[u], (int32_t)rel);
+                rel += ents[u];
+            }
         }
     }
     __syncthreads();
@@ -2444,7 +2480,7 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
     a.o_repr = d->expm_buf + L.repr; a.o_nbr_off = d->expm_buf + L.nbr_off; a.inv = d->expm_buf + L.inv; a.ent_to = d->expm_buf + L.ent_to;
     a.segs = static_cast<ExportSeg*>(d->seg_tiles);
     a.tiles = reinterpret_cast<int2*>(a.segs + n_segs);
-    a.n_bins_max = (int32_t)(n_segs + n_total / 32);   // (export_bins: a segment of more than 64 nodes has at most a bin for 32 of them)
+    a.n_bins_max = (int32_t)(n_segs + n_total / 32);   // (export_bins_log: a segment of more than 64 nodes has at most a bin for 32 of them)
     a.bin_end = d->sort_hist;                          // (kBins places for every tile that the scratch is sized for, and these are three for every bin)
     a.bin_ents = a.bin_end + a.n_bins_max;
     a.bin_seg = reinterpret_cast<int32_t*>(a.bin_ents + a.n_bins_max);

@@ -235,3 +235,78 @@ def test_arrays_of_a_sample_whose_graph_has_been_replaced(graph, n_later):
             for key in keys:
                 assert torch.equal(getattr(v, key), arrays[key]), (b, key)
     c.close()
+
+
+# ... and deltas with as many bins as there are (131,073 nodes and more), spread and in one run of a graph of many nodes, and runs of ids that lie
+# further apart than a bitmap reaches, several in a bin; targets with a thousand entries each and too few of them for a warp's share
+@pytest.mark.parametrize("place,sizes,n", [(lambda i: 2 ** 18 * (i % 5) + i // 5, (64, 129, 1_000, 1_025, 4_097, 40_000), 2 ** 25),
+                                           (lambda i: 61 * i, (131_072, 131_073, 150_000), 2 ** 26), (lambda i: i, (150_000,), 2 ** 27 - 1)],
+                         ids=["runs", "long", "one-run"])
+def test_export_orders_long_deltas_and_ids_in_runs(place, sizes, n):
+    base, most = 5 * 2 ** 20 + 77, max(sizes)
+    tg = [np.arange(-(-m // 1_000), dtype=np.int64) + 1_000 * s for s, m in enumerate(sizes)]      # 1,000 of the delta's ids from each target
+    inner = base + place(np.arange(most, dtype=np.int64))
+    has = np.nonzero(np.arange(most) % 4)[0]
+    rows, ids = [], []
+    for t, m in zip(tg, sizes):
+        rows.append(np.repeat(t, np.minimum(1_000, m - 1_000 * np.arange(len(t)))))
+        ids.append(inner[:m])
+    for q in range(3):      # the last deltas: placed alike, up to three of their ids from each node
+        at = has[has % 4 > q]
+        rows.append(inner[at])
+        ids.append(2 ** 24 + place(2 * at + q))
+    rows, ids = np.concatenate(rows), np.concatenate(ids)
+    assert inner.max() < 2 ** 24 and ids.max() < n
+    off = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=n), dtype=np.int64)])
+    c = mg.Context(0)
+    c.load_graph(torch.from_numpy(off).cuda(), torch.from_numpy(ids[np.lexsort((ids, rows))].astype(np.int32)).cuda())
+    offs = np.concatenate([[0], np.cumsum([len(t) for t in tg])])
+    room = 1_000 + 4 * most
+    d = c.sample_many(torch.from_numpy(np.concatenate(tg).astype(np.int32)), offs, [1_000, 3], list(range(len(tg))),
+                      caps={"max_nodes_total": 3 * room, "max_entries_total": 3 * room, "max_nodes_per_batch": room})
+    assert d.counts()[0][:, 1].tolist() == list(sizes)
+    d.export_many()
+    for b in range(len(tg)):
+        x, y = d.export_view(b), d.view(b)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
+        at = x.node_id_offsets.tolist()
+        for lo, hi in zip(at[:-2], at[1:-1]):
+            assert bool((x.node_ids[lo:hi].diff() > 0).all())
+        assert torch.equal(x.node_ids[x.repr_map.long()], x.nbrs)
+    c.close()
+    torch.cuda.empty_cache()
+
+
+# an export runs on the sampling stream, beside the layers of another sample and before the next one is drawn
+def test_exports_beside_the_layers_of_other_samples(graph):
+    c = mg.Context(0)
+    c.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    c.load_features(inputs.normal_features(N, 32, seed=8, device="cuda"))
+    model = c.model(inputs.random_bias_layers([32, 64, 64], seed=9))
+    keys = ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map")
+    n_batches, per = 24, 600
+    offs = per * np.arange(n_batches + 1)
+    rows = [torch.cat([inputs.distinct_targets(N, per, seed=100 * g + b) for b in range(n_batches)]).cuda() for g in range(5)]
+    seeds = [[1_000 * g + b for b in range(n_batches)] for g in range(5)]
+    outs, arrays = [], []
+    for g in range(5):      # one behind the other
+        d = c.sample_many(rows[g], offs, [8, 4], seeds[g])
+        outs.append(c.forward(model, d, torch.empty((n_batches * per, 64), device="cuda")))
+        arrays.append([{key: getattr(v, key).clone() for key in keys} for v in (d.view(b) for b in (0, 11, n_batches - 1))])
+        d.free()
+    held = [c.sample_many(rows[0], offs, [8, 4], seeds[0]) for _ in range(3)]
+    for g in range(2):
+        c.sample_many_begin(rows[g], offs, [8, 4], seeds[g], out=held[g])
+    for g in range(5):
+        d = held[g % 3]
+        c.sample_many_end(d)
+        d.export_many()
+        if g + 2 < 5:
+            c.sample_many_begin(rows[g + 2], offs, [8, 4], seeds[g + 2], out=held[(g + 2) % 3])
+        assert torch.equal(c.forward(model, d, torch.empty((n_batches * per, 64), device="cuda")), outs[g])
+        for want, b in zip(arrays[g], (0, 11, n_batches - 1)):
+            v = d.export_view(b)
+            for key in keys:
+                assert torch.equal(getattr(v, key), want[key]), (g, b, key)
+    c.close()
