@@ -1315,6 +1315,7 @@ struct ExportSeg {
 struct ExportCounts { int32_t n_tiles, n_bins, n_dense; };
 struct ExportManyArgs {
     int32_t B, k, id_bits, n_bins_max;
+    int32_t nodes_per_warp;  // of k_export_many_entries: 1 to 32
     int32_t hop_base[MG_MAX_HOPS + 2];
     const int32_t *nodes, *node_batch, *node_off, *cum, *rowbase0, *ent_hop, *ent_off, *ent_nbrs, *ent_repr;
     int32_t *o_node_ids, *o_nio, *o_nbrs, *o_repr, *o_nbr_off;
@@ -1732,18 +1733,20 @@ __global__ void __launch_bounds__(kThreads, 5) k_export_order(ExportManyArgs a) 
     }
 }
 
-// A warp takes 32 sampled nodes; their entries lie one behind the other in the arena and are read as one stream, four loads in flight
-// per lane, each lane looking up whose its entry is.  They go to their place in the packed canonical entry list, the neighbours
-// translated to canonical rows of the mini-batch.
+// A warp takes 32 sampled nodes (fewer where there would not be a warp for every slot of the SMs); their entries lie one behind the other in
+// the arena and are read as one stream, four loads in flight per lane, each lane looking up whose its entry is.  They go to their place in the
+// packed canonical entry list, the neighbours translated to canonical rows of the mini-batch.  (With 32 nodes per warp whatever their number, 100
+// targets of 1,000 entries were four warps' work: 206 us, now 9; 8 mini-batches of 100 targets with 3,000 entries 9 -> 3.)
 __global__ void __launch_bounds__(kThreads) k_export_many_entries(ExportManyArgs a) {
     constexpr int U = 4;
     const int lane = threadIdx.x & 31;
-    const int32_t n_sampled = a.hop_base[a.k];
-    for (int32_t i0 = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x) & ~31; i0 < n_sampled; i0 += (int32_t)(gridDim.x * blockDim.x)) {
-        const int32_t i = min(i0 + lane, n_sampled - 1);
-        const int32_t off = i0 + lane < n_sampled ? a.ent_off[i] : INT32_MAX;
+    const int32_t n_sampled = a.hop_base[a.k], npw = a.nodes_per_warp;
+    const int64_t step = (int64_t)gridDim.x * (kThreads / 32) * npw;
+    for (int64_t w0 = (blockIdx.x * (int64_t)(kThreads / 32) + (threadIdx.x >> 5)) * npw; w0 < n_sampled; w0 += step) {
+        const int32_t i0 = (int32_t)w0, i = min(i0 + lane, n_sampled - 1);
+        const int32_t off = lane < npw && i0 + lane < n_sampled ? a.ent_off[i] : INT32_MAX;
         const int32_t to = a.ent_to[i] - off, row0 = a.rowbase0[a.node_batch[i]];   // (lanes behind the last node: never asked for)
-        const int32_t end = a.ent_off[min(i0 + 32, n_sampled)];
+        const int32_t end = a.ent_off[min(i0 + npw, n_sampled)];
         for (int32_t e0 = __shfl_sync(0xFFFFFFFFu, off, 0); e0 < end; e0 += 32 * U) {
             int32_t nbr[U], row[U], at[U];
 #pragma unroll
@@ -2503,7 +2506,10 @@ extern "C" int mg_dense_export_many(mg_ctx* ctx, mg_dense* d) {
         k_export_count<<<blocks_for(n_tiles_max, 1, 8), kThreads, 0, st>>>(a);
         k_export_split<<<blocks_for(n_tiles_max, 1, 8), kThreads, 0, st>>>(a);
         k_export_order<<<blocks_for(a.n_bins_max, kThreads / 32, 8), kThreads, 0, st>>>(a);
-        k_export_many_entries<<<blocks_for(d->h_hdr.hop_base[k], kThreads, 8), kThreads, 0, st>>>(a);
+        const int32_t n_sampled = d->h_hdr.hop_base[k];
+        a.nodes_per_warp = 32;
+        while (a.nodes_per_warp > 1 && n_sampled < (int64_t)a.nodes_per_warp * mg_grid(ctx, 8) * (kThreads / 32)) a.nodes_per_warp /= 2;
+        k_export_many_entries<<<blocks_for(n_sampled, kThreads / 32 * a.nodes_per_warp, 8), kThreads, 0, st>>>(a);
         ctx->launches += 5;
         }
         ctx->stream = user;
