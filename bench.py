@@ -422,8 +422,8 @@ def main():
     launches = ctx.kernel_launches() - launches0
 
     # ---- the same steps with the canonical export of every mini-batch inside the timed region -------------
-    for i in range(2):
-        run_steps(i, 1, False, export=True)      # allocates the export buffers
+    for i in range(3):
+        run_steps(i, 1, False, export=True)      # allocates the export buffers, one per sample handle
     barrier()
     ev4, ev5 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     ev4.record()
