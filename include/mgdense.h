@@ -319,7 +319,10 @@ int mg_forward(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out, int out_
  * output is read back from L2 instead of DRAM; H^k is the same, the intermediate layers are not kept.
  * Only the fused tensor-core layers (MG_GEMM_TF32, widths <= 256) use windows. */
 int mg_set_layer_window(mg_ctx* ctx, int32_t mini_batches);
-/* enable = 1 forces the whole-layer schedule whatever the window, so that mg_layer_output works. */
+/* enable = 1 forces the whole-layer schedule whatever the window, so that mg_layer_output and mg_backward work.  With MG_GEMM_TF32 the forward
+ * pass then also leaves, to save mg_backward work, a bit per intermediate output and, for the rows of later layers with more than three
+ * entries on average, their aggregates (one more row of the layer's input width each).  That memory is given back to whatever the context
+ * allocates and finds no room for; mg_backward then reads the rows instead. */
 int mg_keep_layer_outputs(mg_ctx* ctx, int enable);
 
 /* mg_forward with a HOST output whose device-to-host copy does not block the caller: the kernels are

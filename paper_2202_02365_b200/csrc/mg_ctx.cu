@@ -360,7 +360,7 @@ extern "C" int mg_destroy(mg_ctx* c) {
     free_out_graph(c);
     cudaFree(c->row_off); cudaFree(c->nbrs); cudaFree(c->d_slot_of_part); cudaFree(c->d_res_prefix); cudaFreeHost(c->h_flags);
     cudaFree(c->view_ws); cudaFree(c->d_part_start); cudaFree(c->d_part_of_node); cudaFree(c->d_local_of_node); cudaFree(c->d_nodes_by_part);
-    cudaFree(c->ws_x); cudaFree(c->ws_meta); cudaFree(c->ws_positive); cudaFree(c->ws_agg); cudaFree(c->ws_h[0]); cudaFree(c->ws_h[1]);
+    cudaFree(c->ws_x); cudaFree(c->ws_meta); cudaFree(c->ws_saved); cudaFree(c->ws_h[0]); cudaFree(c->ws_h[1]);
     cudaEventDestroy(c->ev_fwd_done); cudaEventDestroy(c->ev_out_done); cudaEventDestroy(c->ev_user);
     if (c->ev_backward) cudaEventDestroy(c->ev_backward);
     mg_reads_free(&c->array_reads);
@@ -440,8 +440,8 @@ static int rebuild_one_view(mg_ctx* c, bool all, const int64_t* row_off, const i
     }
     if (!*owned) {
         *view_off = nullptr; *view_nbrs = nullptr;
-        if (cudaMalloc((void**)view_off, sizeof(int64_t) * (c->n_nodes + 1)) != cudaSuccess ||
-            cudaMalloc((void**)view_nbrs, sizeof(int32_t) * std::max<int64_t>(n_edges, 1)) != cudaSuccess) {
+        if (mg_malloc(c, (void**)view_off, sizeof(int64_t) * (c->n_nodes + 1)) != cudaSuccess ||
+            mg_malloc(c, (void**)view_nbrs, sizeof(int32_t) * std::max<int64_t>(n_edges, 1)) != cudaSuccess) {
             cudaGetLastError();
             cudaFree(*view_off);
             *view_off = nullptr; *view_nbrs = nullptr;
@@ -460,7 +460,7 @@ static int rebuild_one_view(mg_ctx* c, bool all, const int64_t* row_off, const i
     if (c->view_ws_bytes < need) {
         cudaFree(c->view_ws);
         c->view_ws = nullptr; c->view_ws_bytes = 0;
-        if (cudaMalloc((void**)&c->view_ws, need) != cudaSuccess) { cudaGetLastError(); return mg_fail(c, MG_ERR_OOM, "scratch allocation for the in-buffer graph view failed"); }
+        if (mg_malloc(c, (void**)&c->view_ws, need) != cudaSuccess) { cudaGetLastError(); return mg_fail(c, MG_ERR_OOM, "scratch allocation for the in-buffer graph view failed"); }
         c->view_ws_bytes = need;
     }
     ViewArgs a;
@@ -516,8 +516,8 @@ static int upload_csr(mg_ctx* c, int64_t n_nodes, int64_t n_edges, const void* r
                       const int32_t* nbrs, int ptrs_are_device, int64_t** d_row_off, int32_t** d_nbrs) {
     const cudaMemcpyKind kind = ptrs_are_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     *d_row_off = nullptr; *d_nbrs = nullptr;
-    if (cudaMalloc((void**)d_row_off, sizeof(int64_t) * (n_nodes + 1)) != cudaSuccess ||
-        cudaMalloc((void**)d_nbrs, sizeof(int32_t) * std::max<int64_t>(n_edges, 1)) != cudaSuccess) {
+    if (mg_malloc(c, (void**)d_row_off, sizeof(int64_t) * (n_nodes + 1)) != cudaSuccess ||
+        mg_malloc(c, (void**)d_nbrs, sizeof(int32_t) * std::max<int64_t>(n_edges, 1)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(*d_row_off); *d_row_off = nullptr; *d_nbrs = nullptr;
         return mg_fail(c, MG_ERR_OOM, "allocation of the graph store failed");
@@ -529,7 +529,7 @@ static int upload_csr(mg_ctx* c, int64_t n_nodes, int64_t n_edges, const void* r
         e = cudaMemcpyAsync(*d_row_off, row_offsets, sizeof(int64_t) * (n_nodes + 1), kind, st);
     } else {
         int32_t* tmp = nullptr;
-        e = cudaMalloc((void**)&tmp, sizeof(int32_t) * (n_nodes + 1));
+        e = mg_malloc(c, (void**)&tmp, sizeof(int32_t) * (n_nodes + 1));
         if (e == cudaSuccess) e = cudaMemcpyAsync(tmp, row_offsets, sizeof(int32_t) * (n_nodes + 1), kind, st);
         if (e == cudaSuccess) {
             k_widen_offsets<<<mg_grid(c, 4), kThreads, 0, st>>>(tmp, *d_row_off, n_nodes + 1);
@@ -541,7 +541,7 @@ static int upload_csr(mg_ctx* c, int64_t n_nodes, int64_t n_edges, const void* r
     if (e == cudaSuccess && n_edges > 0) e = cudaMemcpyAsync(*d_nbrs, nbrs, sizeof(int32_t) * n_edges, kind, st);
     // validate on the device; only the two end offsets come back
     uint32_t* flags = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc((void**)&flags, sizeof(uint32_t));
+    if (e == cudaSuccess) e = mg_malloc(c, (void**)&flags, sizeof(uint32_t));
     if (e != cudaSuccess) { cudaGetLastError(); drop(); return mg_cuda_fail(c, e, "graph upload"); }
     cudaMemsetAsync(flags, 0, sizeof(uint32_t), st);
     k_check_graph<<<mg_grid(c, 8), kThreads, 0, st>>>(*d_row_off, n_nodes, *d_nbrs, n_edges, flags);
@@ -642,9 +642,9 @@ extern "C" int mg_set_partitioning(mg_ctx* c, int32_t n_parts, const uint8_t* pa
             local[(size_t)v] = (int32_t)(next[p] - c->part_start[p]);
             by_part[(size_t)next[p]++] = (int32_t)v;
         }
-        if (cudaMalloc((void**)&c->d_part_of_node, (size_t)N) != cudaSuccess ||
-            cudaMalloc((void**)&c->d_local_of_node, sizeof(int32_t) * (size_t)N) != cudaSuccess ||
-            cudaMalloc((void**)&c->d_nodes_by_part, sizeof(int32_t) * (size_t)N) != cudaSuccess) {
+        if (mg_malloc(c, (void**)&c->d_part_of_node, (size_t)N) != cudaSuccess ||
+            mg_malloc(c, (void**)&c->d_local_of_node, sizeof(int32_t) * (size_t)N) != cudaSuccess ||
+            mg_malloc(c, (void**)&c->d_nodes_by_part, sizeof(int32_t) * (size_t)N) != cudaSuccess) {
             cudaGetLastError();
             cudaFree(c->d_part_of_node); cudaFree(c->d_local_of_node); cudaFree(c->d_nodes_by_part);
             c->d_part_of_node = nullptr; c->d_local_of_node = nullptr; c->d_nodes_by_part = nullptr;
@@ -692,7 +692,7 @@ extern "C" int mg_load_features(mg_ctx* c, const void* table, int table_is_devic
             c->slots_owned = false;
         } else {
             const size_t bytes = (size_t)c->n_nodes * c->row_bytes;
-            if (cudaMalloc((void**)&c->slots, bytes) != cudaSuccess) { cudaGetLastError(); c->slots = nullptr; return mg_fail(c, MG_ERR_OOM, "feature table allocation failed"); }
+            if (mg_malloc(c, (void**)&c->slots, bytes) != cudaSuccess) { cudaGetLastError(); c->slots = nullptr; return mg_fail(c, MG_ERR_OOM, "feature table allocation failed"); }
             c->slots_owned = true;
             MG_CUDA(c, cudaMemcpyAsync(c->slots, table, bytes, cudaMemcpyHostToDevice, c->stream));
             MG_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -704,7 +704,7 @@ extern "C" int mg_load_features(mg_ctx* c, const void* table, int table_is_devic
     } else {
         c->n_slots = buffer_capacity_parts + 1;
         const size_t bytes = (size_t)c->n_slots * c->slot_bytes;
-        if (cudaMalloc((void**)&c->slots, bytes) != cudaSuccess) { cudaGetLastError(); c->slots = nullptr; return mg_fail(c, MG_ERR_OOM, "buffer slot allocation failed"); }
+        if (mg_malloc(c, (void**)&c->slots, bytes) != cudaSuccess) { cudaGetLastError(); c->slots = nullptr; return mg_fail(c, MG_ERR_OOM, "buffer slot allocation failed"); }
         c->slots_owned = true;
         c->host_table = (const char*)table;
         // whatever was resident for sampling only is reloaded into slots

@@ -419,10 +419,10 @@ extern "C" int mg_model_create(mg_ctx* ctx, int32_t k, const int32_t* dims, cons
     for (int l = 0; l <= k; ++l) m->dims[l] = dims[l];
     for (int l = 0; l < k; ++l) {
         const size_t di = dims[l], dn = dims[l + 1];
-        if (cudaMalloc((void**)&m->w_cat[l], sizeof(float) * 2 * di * dn) != cudaSuccess ||
-            cudaMalloc((void**)&m->w_cat_t[l], sizeof(float) * 2 * di * dn) != cudaSuccess ||
-            cudaMalloc((void**)&m->w_pad_t[l], sizeof(float) * 2 * ((di + 31) / 32 * 32) * dn) != cudaSuccess ||
-            cudaMalloc((void**)&m->bias[l], sizeof(float) * dn) != cudaSuccess) {
+        if (mg_malloc(ctx, (void**)&m->w_cat[l], sizeof(float) * 2 * di * dn) != cudaSuccess ||
+            mg_malloc(ctx, (void**)&m->w_cat_t[l], sizeof(float) * 2 * di * dn) != cudaSuccess ||
+            mg_malloc(ctx, (void**)&m->w_pad_t[l], sizeof(float) * 2 * ((di + 31) / 32 * 32) * dn) != cudaSuccess ||
+            mg_malloc(ctx, (void**)&m->bias[l], sizeof(float) * dn) != cudaSuccess) {
             cudaGetLastError();
             mg_model_free(m);
             return mg_fail(ctx, MG_ERR_OOM, "weight allocation failed");
@@ -447,7 +447,7 @@ extern "C" int mg_model_create(mg_ctx* ctx, int32_t k, const int32_t* dims, cons
         }
         const double rms = std::sqrt(sq / (double)(2 * di * dn));
         if (!(mx < 32768.0 && rms > 1.0 / 1024.0)) continue;
-        if (cudaMalloc(&m->w_pad_h[l], sizeof(uint16_t) * 2 * ((di + 63) / 64 * 64) * dn) != cudaSuccess) {
+        if (mg_malloc(ctx, (void**)&m->w_pad_h[l], sizeof(uint16_t) * 2 * ((di + 63) / 64 * 64) * dn) != cudaSuccess) {
             cudaGetLastError();
             mg_model_free(m);
             return mg_fail(ctx, MG_ERR_OOM, "weight allocation failed");
@@ -662,32 +662,36 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
         ctx->ws_x_bytes = have * sizeof(float);
     }
 
-    // The weights' gradients want the rows' aggregates again.  Where a row has several entries of a layer's outputs the forward pass leaves
-    // the aggregate behind: a row to write and to read in place of a row for each entry.  (Layer 1's rows have few entries and come from
-    // the table, where the other mini-batches' copies are as many: it gathers again.)
+    // What is left for the backward pass beside the kept outputs, in one block.  A bit for each of them: it takes them through a ReLU once more and
+    // only has to know which were above zero, a thirty-second of what reading the rows again takes.  And the rows' aggregates, which the weights'
+    // gradients want again, where a row has several entries of a layer's outputs: a row to write and to read in place of a row for each
+    // entry.  (Layer 1's rows have few entries and come from the table, where the other mini-batches' copies are as many: it gathers again.)
+    // Without room for the aggregates, or for either, the backward pass reads the rows.
     {
-        int64_t floats = 0;
+        int64_t words = 0, bits = 0;
+        const auto fused = [&](int l) { return ctx->keep_layers && m->precision == MG_GEMM_TF32 && mg_layer_fused_supported(m->dims[l - 1], m->dims[l]); };
         for (int l = 1; l <= k; ++l) {
-            const bool kept = ctx->keep_layers && l > 1 && m->precision == MG_GEMM_TF32 && mg_layer_fused_supported(m->dims[l - 1], m->dims[l]) &&
-                              (int64_t)d->h_hdr.ent_base[k - l + 1] > kKeepEntriesPerRow * d->h_hdr.rows_total[l];
-            ctx->agg_at[l] = kept ? floats : -1;
-            if (kept) floats += (int64_t)d->h_hdr.rows_total[l] * m->dims[l - 1];
+            ctx->positive_at[l] = l < k && fused(l) ? words : -1;
+            if (ctx->positive_at[l] >= 0) words += mg_positive_words(d->h_hdr.rows_total[l], m->dims[l]);
+        }
+        bits = words;
+        for (int l = 1; l <= k; ++l) {
+            ctx->agg_at[l] = l > 1 && fused(l) && (int64_t)d->h_hdr.ent_base[k - l + 1] > kKeepEntriesPerRow * d->h_hdr.rows_total[l] ? words : -1;
+            if (ctx->agg_at[l] >= 0) words += (int64_t)d->h_hdr.rows_total[l] * m->dims[l - 1];   // (widths are multiples of 4: 16-byte aligned starts)
         }
         ctx->agg_sum = m->sum_aggr;
-        if (floats > 0 && ctx->ws_agg_elems < (size_t)floats && mg_ensure(ctx, &ctx->ws_agg, &ctx->ws_agg_elems, (size_t)(floats + floats / 4)))
-            for (int l = 1; l <= k; ++l) ctx->agg_at[l] = -1;   // (no room: gathered again)
-    }
-    // Kept outputs go through a ReLU once more in the backward pass, which only has to know which values were above zero: the
-    // fused kernel leaves a bit for each, a thirty-second of what reading the rows again takes.
-    {
-        int64_t words = 0;
-        for (int l = 1; l <= k; ++l) {
-            const bool bits = ctx->keep_layers && l < k && m->precision == MG_GEMM_TF32 && mg_layer_fused_supported(m->dims[l - 1], m->dims[l]);
-            ctx->positive_at[l] = bits ? words : -1;
-            if (bits) words += mg_positive_words(d->h_hdr.rows_total[l], m->dims[l]);
+        if (ctx->ws_saved_elems < (size_t)words) {
+            cudaFree(ctx->ws_saved);
+            ctx->ws_saved = nullptr; ctx->ws_saved_elems = 0;
+            for (const int64_t want : {words, bits}) {
+                if (want < words) for (int l = 1; l <= k; ++l) ctx->agg_at[l] = -1;
+                const size_t room = (size_t)(want + want / 4);
+                if (want == 0 || cudaMalloc((void**)&ctx->ws_saved, room * sizeof(uint32_t)) == cudaSuccess) { ctx->ws_saved_elems = want ? room : 0; break; }
+                cudaGetLastError();
+                ctx->ws_saved = nullptr;
+            }
+            if (!ctx->ws_saved) for (int l = 1; l <= k; ++l) ctx->agg_at[l] = ctx->positive_at[l] = -1;
         }
-        if (words > 0 && ctx->ws_positive_elems < (size_t)words && mg_ensure(ctx, &ctx->ws_positive, &ctx->ws_positive_elems, (size_t)(words + words / 4)))
-            for (int l = 1; l <= k; ++l) ctx->positive_at[l] = -1;   // (no room: the rows are read)
     }
 
     const bool half = ctx->feat_dtype == MG_DTYPE_F16;
@@ -703,8 +707,8 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
                 rc = mg_layer_fused(ctx, d, l, d_in, d_out, m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
                                     (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], 0, M, 0,
                                     (l == 1 || f16_inter) ? m->w_pad_h[l - 1] : nullptr, f16_inter && l > 1, f16_inter && l < k,
-                                    ctx->positive_at[l] >= 0 ? ctx->ws_positive + ctx->positive_at[l] : nullptr,
-                                    ctx->agg_at[l] >= 0 ? ctx->ws_agg + ctx->agg_at[l] : nullptr);
+                                    ctx->positive_at[l] >= 0 ? ctx->ws_saved + ctx->positive_at[l] : nullptr,
+                                    ctx->agg_at[l] >= 0 ? reinterpret_cast<float*>(ctx->ws_saved + ctx->agg_at[l]) : nullptr);
             }
             if (rc) return rc;
             continue;
@@ -1325,7 +1329,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     if (!m->g_block) {
         m->g_elems = 0;
         for (int l = 0; l < k; ++l) m->g_elems += (size_t)(2 * m->dims[l] + 1) * m->dims[l + 1];
-        if (cudaMalloc((void**)&m->g_block, m->g_elems * sizeof(float)) != cudaSuccess) { cudaGetLastError(); m->g_block = nullptr; return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
+        if (mg_malloc(ctx, (void**)&m->g_block, m->g_elems * sizeof(float)) != cudaSuccess) { cudaGetLastError(); m->g_block = nullptr; return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
         float* g = m->g_block;
         for (int l = 0; l < k; ++l) {
             m->g_w_cat[l] = g; g += (size_t)2 * m->dims[l] * m->dims[l + 1];
@@ -1336,7 +1340,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     m->g_reads.queued = false;
     MG_CUDA(ctx, cudaMemsetAsync(m->g_block, 0, m->g_elems * sizeof(float), st));
     if (!m->zeros) {
-        if (cudaMalloc((void**)&m->zeros, sizeof(float) * 2 * 1024) != cudaSuccess) { cudaGetLastError(); return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
+        if (mg_malloc(ctx, (void**)&m->zeros, sizeof(float) * 2 * 1024) != cudaSuccess) { cudaGetLastError(); return mg_fail(ctx, MG_ERR_OOM, "gradient allocation failed"); }
         MG_CUDA(ctx, cudaMemsetAsync(m->zeros, 0, sizeof(float) * 2 * 1024, st));
     }
     // scratch: dH^1 .. dH^{k-1}, the X rows of a chunk (fp32 products only), dX of a layer, the turned-round entries of the layers whose dX is handed down
@@ -1435,7 +1439,8 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
             // dW += X^T dPre with X gathered again inside the kernel; the row metadata is what the forward pass left (its layers all
             // have it, mg_forward of this very model and sample was the last to write it)
             if ((rc = mg_layer_grad_weights(ctx, d, l, d_in, d_out, h_prev, dpre_all, ctx->ws_meta + meta_at, m->sum_aggr ? 1 : 0,
-                                            ctx->agg_at[l] >= 0 && ctx->agg_sum == m->sum_aggr ? ctx->ws_agg + ctx->agg_at[l] : nullptr, m->g_w_cat[l - 1]))) return rc;
+                                            ctx->agg_at[l] >= 0 && ctx->agg_sum == m->sum_aggr ? reinterpret_cast<const float*>(ctx->ws_saved + ctx->agg_at[l]) : nullptr,
+                                            m->g_w_cat[l - 1]))) return rc;
             // dX = dPre W^T on the tensor cores: the K-major operand the kernel wants is W itself ([2 d_in, d_out])
             if (g_in && (rc = mg_gemm_tf32(ctx, dpre_all, m->w_cat[l - 1], m->zeros, ctx->bw_dx, M, 2 * d_in, d_out, false))) return rc;
         }
@@ -1473,7 +1478,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         // dX -> the gradient of the layer's input rows
         const bool bits = l > 1 && ctx->positive_at[l - 1] >= 0;
         GatherArgs ga{geom, l, rows_in, ra.cnt + ra.in_at[l], ra.rev, ra.units + ra.unit_at[l], ra.n_units + l, ra.bad, ctx->bw_dx, d_in,
-                      l > 1 ? ctx->ws_h[0] + h_off[l - 1] : nullptr, bits ? ctx->ws_positive + ctx->positive_at[l - 1] : nullptr, g_in, l > 1 ? m->g_bias[l - 2] : nullptr};
+                      l > 1 ? ctx->ws_h[0] + h_off[l - 1] : nullptr, bits ? ctx->ws_saved + ctx->positive_at[l - 1] : nullptr, g_in, l > 1 ? m->g_bias[l - 2] : nullptr};
         // (groups of 16 rows, a warp per 128 columns; the units come on top, the loop takes what does not fit the grid)
         const int64_t warps = (rows_in + kGradRows - 1) / kGradRows * std::max(1, (d_in + 127) / 128);
         const int ggrid = (int)std::max<int64_t>(1, std::min<int64_t>(mg_grid(ctx, l > 1 ? 4 : 8), (warps + kThreads / 32 - 1) / (kThreads / 32) + 16));
@@ -1531,7 +1536,7 @@ extern "C" int mg_model_adagrad_step(mg_ctx* ctx, mg_model* m, float lr, float e
     if (!(eps > 0.f)) return mg_fail(ctx, MG_ERR_ARG, "eps must be positive");
     MG_CUDA(ctx, cudaSetDevice(ctx->device));
     if (!m->s_block) {   // accumulated squared gradients start at zero
-        if (cudaMalloc((void**)&m->s_block, m->g_elems * sizeof(float)) != cudaSuccess) {
+        if (mg_malloc(ctx, (void**)&m->s_block, m->g_elems * sizeof(float)) != cudaSuccess) {
             cudaGetLastError();
             m->s_block = nullptr;
             return mg_fail(ctx, MG_ERR_OOM, "optimizer state allocation failed");

@@ -427,15 +427,15 @@ extern "C" int mg_gat_model_create(mg_ctx* ctx, int32_t k, const int32_t* dims, 
     for (int l = 0; l <= k; ++l) m->dims[l] = dims[l];
     int widest = 4;
     for (int l = 1; l <= k; ++l) widest = std::max(widest, dims[l]);
-    bool ok = cudaMalloc((void**)&m->zeros, sizeof(float) * widest) == cudaSuccess &&
+    bool ok = mg_malloc(ctx, (void**)&m->zeros, sizeof(float) * widest) == cudaSuccess &&
               cudaMemsetAsync(m->zeros, 0, sizeof(float) * widest, ctx->stream) == cudaSuccess;
     for (int l = 0; l < k && ok; ++l) {
         const size_t di = dims[l], dn = dims[l + 1];
-        ok = cudaMalloc((void**)&m->w[l], sizeof(float) * di * dn) == cudaSuccess &&
-             cudaMalloc((void**)&m->w_t[l], sizeof(float) * di * dn) == cudaSuccess &&
-             cudaMalloc((void**)&m->a_src[l], sizeof(float) * dn) == cudaSuccess &&
-             cudaMalloc((void**)&m->a_dst[l], sizeof(float) * dn) == cudaSuccess &&
-             cudaMalloc((void**)&m->bias[l], sizeof(float) * dn) == cudaSuccess;
+        ok = mg_malloc(ctx, (void**)&m->w[l], sizeof(float) * di * dn) == cudaSuccess &&
+             mg_malloc(ctx, (void**)&m->w_t[l], sizeof(float) * di * dn) == cudaSuccess &&
+             mg_malloc(ctx, (void**)&m->a_src[l], sizeof(float) * dn) == cudaSuccess &&
+             mg_malloc(ctx, (void**)&m->a_dst[l], sizeof(float) * dn) == cudaSuccess &&
+             mg_malloc(ctx, (void**)&m->bias[l], sizeof(float) * dn) == cudaSuccess;
         if (!ok) break;
         cudaMemcpyAsync(m->w[l], w[l], sizeof(float) * di * dn, cudaMemcpyHostToDevice, ctx->stream);
         cudaMemcpyAsync(m->a_src[l], a_src[l], sizeof(float) * dn, cudaMemcpyHostToDevice, ctx->stream);
@@ -450,8 +450,8 @@ extern "C" int mg_gat_model_create(mg_ctx* ctx, int32_t k, const int32_t* dims, 
             for (size_t c = 0; c < dn; ++c) { s1 += (double)w[l][r * dn + c] * a_src[l][c]; s2 += (double)w[l][r * dn + c] * a_dst[l][c]; }
             us[r] = (float)s1; ud[r] = (float)s2;
         }
-        ok = cudaMalloc((void**)&m->u_src[l], sizeof(float) * di) == cudaSuccess &&
-             cudaMalloc((void**)&m->u_dst[l], sizeof(float) * di) == cudaSuccess &&
+        ok = mg_malloc(ctx, (void**)&m->u_src[l], sizeof(float) * di) == cudaSuccess &&
+             mg_malloc(ctx, (void**)&m->u_dst[l], sizeof(float) * di) == cudaSuccess &&
              cudaMemcpy(m->u_src[l], us.data(), sizeof(float) * di, cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemcpy(m->u_dst[l], ud.data(), sizeof(float) * di, cudaMemcpyHostToDevice) == cudaSuccess;
     }

@@ -136,16 +136,17 @@ struct mg_ctx {
     float* ws_x = nullptr; size_t ws_x_bytes = 0;
     float* ws_h[2] = {nullptr, nullptr}; size_t ws_h_bytes[2] = {0, 0};
     int4* ws_meta = nullptr; size_t ws_meta_elems = 0;   // row metadata of the fused layers (mg_layer_rows)
-    float* ws_agg = nullptr; size_t ws_agg_elems = 0;                // aggregates of the kept layers' rows
-    uint32_t* ws_positive = nullptr; size_t ws_positive_elems = 0;   // kept layer outputs: a bit per value, above zero
+    // what a forward pass that keeps its layers leaves to save the backward pass work: a bit per value of the outputs (above zero), then
+    // aggregates of the rows.  The backward pass does without where there is no memory for it (mg_malloc).
+    uint32_t* ws_saved = nullptr; size_t ws_saved_elems = 0;
 
     // forward schedule
     int32_t layer_window_batches = 0;  // mini-batches per window of the layer schedule; 0 = whole layers
     bool keep_layers = false;          // keep H^1..H^{k-1} for mg_layer_output (whole-layer schedule)
     bool layers_kept = false;          // what the last forward did
-    int64_t agg_at[MG_MAX_HOPS + 1] = {0};        // where layer l's rows of ws_agg start (floats); below zero: it left none
+    int64_t agg_at[MG_MAX_HOPS + 1] = {0};        // where layer l's aggregates start in ws_saved (32-bit words); below zero: it left none
     bool agg_sum = false;                         // ... by the model's aggregator at the time
-    int64_t positive_at[MG_MAX_HOPS + 1] = {0};   // where layer l's bits of ws_positive start (32-bit words); below zero: it left none
+    int64_t positive_at[MG_MAX_HOPS + 1] = {0};   // where layer l's bits start in ws_saved; below zero: it left none
 
     // asynchronous output copy of mg_forward_host_async
     cudaEvent_t ev_fwd_done = nullptr, ev_out_done = nullptr;
@@ -323,6 +324,17 @@ int mg_cuda_fail(mg_ctx* ctx, cudaError_t e, const char* what);
         if (e__ != cudaSuccess) return mg_cuda_fail(ctx, e__, #call); \
     } while (0)
 
+// Device memory.  What the context holds only to save work is given back before an allocation fails.
+static inline cudaError_t mg_malloc(mg_ctx* ctx, void** ptr, size_t bytes) {
+    cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e != cudaErrorMemoryAllocation || !ctx->ws_saved) return e;
+    cudaGetLastError();
+    cudaFree(ctx->ws_saved);   // (waits for kernels that use it)
+    ctx->ws_saved = nullptr; ctx->ws_saved_elems = 0;
+    for (int l = 0; l <= MG_MAX_HOPS; ++l) ctx->agg_at[l] = ctx->positive_at[l] = -1;
+    return cudaMalloc(ptr, bytes);
+}
+
 // grow-only device buffer
 template <typename T>
 static inline int mg_ensure(mg_ctx* ctx, T** ptr, size_t* have_elems, size_t need_elems) {
@@ -331,7 +343,7 @@ static inline int mg_ensure(mg_ctx* ctx, T** ptr, size_t* have_elems, size_t nee
     *ptr = nullptr;
     *have_elems = 0;
     if (need_elems == 0) need_elems = 1;
-    cudaError_t e = cudaMalloc((void**)ptr, need_elems * sizeof(T));
+    cudaError_t e = mg_malloc(ctx, (void**)ptr, need_elems * sizeof(T));
     if (e != cudaSuccess) {
         cudaGetLastError();
         return mg_fail(ctx, MG_ERR_OOM, "device allocation of %zu bytes failed", need_elems * sizeof(T));
@@ -391,7 +403,7 @@ static inline HostMemory mg_host_memory(const void* p, size_t bytes, const void*
     return HOST_MAPPED;
 }
 
-// 32-bit words of a layer in mg_ctx::ws_positive: bit r % 32 of word (r / 32) * width + c stands for row r, column c
+// 32-bit words of a layer among mg_ctx::ws_saved: bit r % 32 of word (r / 32) * width + c stands for row r, column c
 static inline int64_t mg_positive_words(int64_t rows, int width) { return (rows + 31) / 32 * width; }
 
 static inline int mg_grid(const mg_ctx* ctx, int ctas_per_sm) { return ctx->n_sms * ctas_per_sm; }

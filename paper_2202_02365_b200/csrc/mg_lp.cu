@@ -565,7 +565,7 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
     if (ctx->lp_ws_bytes < ws_bytes) {
         cudaFree(ctx->lp_ws);
         ctx->lp_ws = nullptr; ctx->lp_ws_bytes = 0;
-        if (cudaMalloc((void**)&ctx->lp_ws, ws_bytes + ws_bytes / 4) != cudaSuccess) {
+        if (mg_malloc(ctx, (void**)&ctx->lp_ws, ws_bytes + ws_bytes / 4) != cudaSuccess) {
             cudaGetLastError(); delete lp;
             return mg_fail(ctx, MG_ERR_OOM, "allocation of the link-prediction scratch failed");
         }
@@ -602,7 +602,7 @@ extern "C" int mg_lp_prepare(mg_ctx* ctx, const int32_t* src, const int32_t* rel
         cudaStreamWaitEvent(st, spare->idle);
         mg_reads_wait(&spare->reads, st);
         spare->reads.queued = false;
-    } else if (cudaMalloc((void**)&lp->block, blk_bytes) != cudaSuccess) {
+    } else if (mg_malloc(ctx, (void**)&lp->block, blk_bytes) != cudaSuccess) {
         cudaGetLastError(); delete lp;
         return mg_fail(ctx, MG_ERR_OOM, "allocation of the link-prediction batch failed");
     } else {
@@ -716,7 +716,7 @@ extern "C" int mg_distmult_score(mg_ctx* ctx, const mg_lp_batch* lp, const float
             if (ctx->dm_images_bytes < image_bytes) {
                 cudaFree(ctx->dm_images);
                 ctx->dm_images = nullptr; ctx->dm_images_bytes = 0;
-                if (cudaMalloc((void**)&ctx->dm_images, image_bytes) != cudaSuccess) {
+                if (mg_malloc(ctx, (void**)&ctx->dm_images, image_bytes) != cudaSuccess) {
                     cudaGetLastError();
                     return mg_fail(ctx, MG_ERR_OOM, "device allocation of %zu bytes failed", image_bytes);
                 }

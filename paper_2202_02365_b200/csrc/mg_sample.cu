@@ -1839,7 +1839,7 @@ template <typename T>
 static int dev_realloc(mg_ctx* ctx, T** p, size_t elems) {
     if (*p) cudaFree(*p);
     *p = nullptr;
-    if (cudaMalloc((void**)p, std::max<size_t>(elems, 1) * sizeof(T)) != cudaSuccess) {
+    if (mg_malloc(ctx, (void**)p, std::max<size_t>(elems, 1) * sizeof(T)) != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
         return mg_fail(ctx, MG_ERR_OOM, "device allocation of %zu bytes failed", elems * sizeof(T));

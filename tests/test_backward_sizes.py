@@ -310,3 +310,55 @@ def test_aggregator_set_between_the_passes():
         got.append([x.clone() for layer in ctx.backward(model, dense, d_out) for x in layer])
     for x, y in zip(*got):      # (the same operands, sums in any order)
         assert float((x.double() - y.double()).norm()) <= 1e-4 * float(x.double().norm())
+
+
+# what the forward pass leaves to save the backward pass work gives way where memory is short: to what the backward pass cannot do without, and it
+# is not left at all where there is no room for it (no error of a call that succeeds); the results are the same
+@pytest.mark.parametrize("short", ["backward", "forward"])
+def test_what_is_kept_to_save_work_gives_way(short):
+    graph = inputs.erdos_renyi_graph(N, 9 * N, seed=31)
+    dims, per, count = [16, 256, 8], 3_000, 48
+    targets = torch.cat([inputs.distinct_targets(N, per, seed=b) for b in range(count)]).cuda()
+    d_out = torch.randn((per * count, 8), generator=torch.Generator("cuda").manual_seed(35), device="cuda")
+    free = lambda: torch.cuda.mem_get_info()[0]
+
+    def step(keep, held, leave_forward=None, leave_backward=None):
+        def hold(leave):
+            if leave is not None:
+                held.append(torch.empty(free() - leave, dtype=torch.uint8, device="cuda"))
+        ctx = mg.Context(0)
+        ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+        ctx.load_features(inputs.normal_features(N, dims[0], seed=32, device="cuda"))
+        ctx.keep_layer_outputs(keep)
+        model = ctx.model(inputs.random_bias_layers(dims, seed=34))
+        dense = ctx.sample_many(targets, per * np.arange(count + 1), [7, 4], list(range(count)))
+        out = torch.empty_like(d_out)
+        hold(leave_forward)
+        at = [free()]
+        ctx.forward(model, dense, out)
+        at.append(free())
+        assert ctx.lib.mg_last_error(ctx.handle) in (None, b"")
+        if leave_forward is not None:
+            held.clear()
+            torch.cuda.empty_cache()
+        hold(leave_backward)
+        at.append(free())
+        grads = [x.clone() for layer in ctx.backward(model, dense, d_out) for x in layer]
+        at.append(free())
+        ctx.close()
+        return grads, at[0] - at[1], at[2] - at[3]
+
+    held = []
+    step(True, held)                                         # (kernels loaded, torch's own blocks there)
+    want, forward, backward = step(False, held)
+    _, forward_kept, backward_kept = step(True, held)
+    kept = forward_kept - forward
+    assert kept > 100 << 20 and backward_kept == backward > kept
+    try:
+        got, used, _ = step(True, held, forward + kept // 2 if short == "forward" else None, backward - kept // 2 if short == "backward" else None)
+        assert used < forward + kept // 2 if short == "forward" else used == forward_kept
+    finally:
+        held.clear()
+        torch.cuda.empty_cache()
+    for x, y in zip(want, got):      # (the same operands; sums over rows meet in any order)
+        assert float((x.double() - y.double()).norm()) <= 1e-4 * float(x.double().norm())
