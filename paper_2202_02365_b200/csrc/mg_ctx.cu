@@ -368,7 +368,7 @@ extern "C" int mg_destroy(mg_ctx* c) {
     cudaFree(c->lp_ws); cudaFree(c->dm_images);
     for (auto& s : c->lp_spare) { cudaFree(s.block); if (s.idle) cudaEventDestroy(s.idle); mg_reads_free(&s.reads); }
     cudaStreamDestroy(c->prep_stream);
-    cudaFree(c->bw_g); cudaFree(c->bw_x); cudaFree(c->bw_dx); cudaFree(c->bw_off); cudaFree(c->bw_rev);
+    cudaFree(c->bw_g); cudaFree(c->bw_x); cudaFree(c->bw_dx); cudaFree(c->bw_lists);
     cudaFree(c->gat_x); cudaFree(c->gat_z); cudaFree(c->gat_s); cudaFree(c->gat_h[0]); cudaFree(c->gat_h[1]);
     cudaStreamDestroy(c->sample_stream);
     cudaStreamDestroy(c->side);

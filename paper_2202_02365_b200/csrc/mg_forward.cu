@@ -1375,13 +1375,13 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     if (ctx->bw_g_elems < g_total && (rc = mg_ensure(ctx, &ctx->bw_g, &ctx->bw_g_elems, g_total + g_total / 4 + 16))) return rc;
     if (ctx->bw_x_elems < (size_t)max_x && (rc = mg_ensure(ctx, &ctx->bw_x, &ctx->bw_x_elems, (size_t)max_x + 16))) return rc;
     if (ctx->bw_dx_elems < (size_t)max_dx && (rc = mg_ensure(ctx, &ctx->bw_dx, &ctx->bw_dx_elems, (size_t)max_dx + 16))) return rc;
-    // cleared by one memset: the scan's ticket, the unit counts, whether it gave up, its states, the counts; then the entries' places
+    // one block.  Cleared by one memset: the scan's ticket, the unit counts, whether it gave up, its states, the counts; then the entries'
+    // places, then the lists and units
     const size_t cnt_at = ((MG_MAX_HOPS + 4) + 2 * (size_t)rev_tiles + 3) / 4 * 4;
     const size_t cleared = cnt_at + (size_t)in_total + 1;
-    const size_t need_off = cleared + (size_t)ent_total;
-    const size_t need_rev = (size_t)ent_total + (size_t)ra.unit_at[k + 1];
-    if (ctx->bw_off_elems < need_off && (rc = mg_ensure(ctx, &ctx->bw_off, &ctx->bw_off_elems, need_off + need_off / 4 + 16))) return rc;
-    if (ctx->bw_rev_elems < need_rev && (rc = mg_ensure(ctx, &ctx->bw_rev, &ctx->bw_rev_elems, need_rev + need_rev / 4 + 16))) return rc;
+    const size_t rev_at = (cleared + (size_t)ent_total + 1) / 2 * 2;
+    const size_t need_lists = rev_at + 2 * ((size_t)ent_total + (size_t)ra.unit_at[k + 1]);
+    if (ctx->bw_lists_elems < need_lists && (rc = mg_ensure(ctx, &ctx->bw_lists, &ctx->bw_lists_elems, need_lists + need_lists / 4 + 16))) return rc;
     const RowGeom geom{B, k, d->rowbase, d->cum, d->node_off};
     const bool half = ctx->feat_dtype == MG_DTYPE_F16;
     const int grid = mg_grid(ctx, 8);
@@ -1394,20 +1394,20 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         ra.g = geom;
         ra.meta = ctx->ws_meta + (ra.l0 > 1 ? (int64_t)d->h_hdr.rows_total[1] : 0);
         ra.ent_repr = d->ent_repr; ra.sum_aggr = m->sum_aggr ? 1 : 0;
-        ra.ticket = ctx->bw_off;
+        ra.ticket = ctx->bw_lists;
         ra.n_units = ra.ticket + 1;
         static_assert(MG_MAX_HOPS % 2 == 0, "the states are 8-byte aligned behind the counters");
-        ra.state = reinterpret_cast<uint64_t*>(ctx->bw_off + MG_MAX_HOPS + 4);
-        ra.cnt = ctx->bw_off + cnt_at;
+        ra.state = reinterpret_cast<uint64_t*>(ctx->bw_lists + MG_MAX_HOPS + 4);
+        ra.cnt = ctx->bw_lists + cnt_at;
         ra.pos = ra.cnt + in_total + 1;
-        ra.rev = ctx->bw_rev;
-        ra.units = ctx->bw_rev + ent_total;
+        ra.rev = reinterpret_cast<int2*>(ctx->bw_lists + rev_at);
+        ra.units = ra.rev + ent_total;
         ra.bad = ra.n_units + MG_MAX_HOPS + 1;
         const char* polls = getenv("MG_REV_POLLS");
         ra.polls = polls ? atoi(polls) : kChainPolls;
         ra.status = ctx->d_flags;
         for (int l = ra.l0; l <= k; ++l) { ra.g_in[l] = l > 1 ? ctx->bw_g + g_off[l - 1] : d_h0_dev; ra.d_in[l] = m->dims[l - 1]; }
-        MG_CUDA(ctx, cudaMemsetAsync(ctx->bw_off, 0, sizeof(uint32_t) * cleared, st));
+        MG_CUDA(ctx, cudaMemsetAsync(ctx->bw_lists, 0, sizeof(uint32_t) * cleared, st));
         ra.rows_per_warp = 4;
         while (ra.rows_per_warp < 32 && ra.out_at[k + 1] > (int64_t)ra.rows_per_warp * grid * (kThreads / 32)) ra.rows_per_warp *= 2;
         const int64_t per_block = (int64_t)ra.rows_per_warp * (kThreads / 32);
