@@ -1,4 +1,4 @@
-"""The fused layer kernel cuts a layer's rows into tiles of 64 or 128 per CTA by how many rows there are: row counts on either
+"""The fused layer kernel cuts a layer's rows into tiles of 32, 64 or 128 per CTA by how many rows there are: row counts on either
 side of every cut, with the weights in tensor memory and streamed, against the layer's definition in fp64."""
 import pytest
 import torch
@@ -81,3 +81,76 @@ def test_rows_on_either_side_of_the_smallest_tiles(graph, rows, d_in, d_out, hal
 @pytest.mark.parametrize("d_in,d_out", [(16, 300), (128, 512), (100, 260)])
 def test_rows_on_either_side_of_the_persistent_product(graph, rows, d_in, d_out):
     test_rows_on_either_side_of_the_tile_sizes(graph, rows, d_in, d_out, False, 4)
+
+
+def layers_over(view, feats, layers, combine):
+    """Layers over one mini-batch in fp64: combine(self rows, sum over their entries, how many, layer), a ReLU on all but the last."""
+    nio, rep, off = view.node_id_offsets.tolist(), view.repr_map.long(), view.nbr_offsets.long()
+    h = feats[view.node_ids.long()].double()
+    for l, layer in enumerate(layers):
+        first, drop = nio[l + 1] - nio[l], nio[l + 1] - nio[1]
+        n = h.shape[0] - first
+        lo, hi, cnt = int(off[drop]), int(off[drop + n]), off[drop + 1:drop + n + 1] - off[drop:drop + n]
+        dst = torch.repeat_interleave(torch.arange(n, device=h.device), cnt)
+        total = torch.zeros((n, h.shape[1]), dtype=torch.float64, device=h.device).index_add(0, dst, h[rep[lo:hi] - nio[l]])
+        h = combine(h[first:], total, cnt.double()[:, None], [x.double().cuda() for x in layer])
+        if l + 1 < len(layers):
+            h = h.relu()
+    return h
+
+
+def uniform_attention(own, total, count, layer):
+    return (own + total) / (count + 1) @ layer[0] + layer[3]
+
+
+def mean_aggregator(own, total, count, layer):
+    return own @ layer[0] + total / count.clamp(min=1) @ layer[1] + layer[2]
+
+
+# the persistent product with a column block narrower than 256 (other boxes, MMA shapes, tensor-memory sizes and accumulator strides), which
+# takes 296 blocks of 256 rows (148 SMs): the last row count by tile, one more, a ragged last block; K of a part of a slice to eight slices.
+# An attention layer without attention is such a product of the rows' means.
+@pytest.mark.parametrize("rows", [75_520, 75_521, 75_777])
+@pytest.mark.parametrize("d_in,d_out", [(16, 4), (100, 16), (256, 36), (32, 96), (100, 100), (64, 132), (256, 200), (36, 224)])
+def test_narrow_persistent_product(graph, rows, d_in, d_out):
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    feats = inputs.normal_features(N, d_in, seed=5, device="cuda")
+    ctx.load_features(feats)
+    ((w, _, b),) = inputs.random_bias_layers([d_in, d_out], seed=6)
+    layer = (w, torch.zeros(d_out), torch.zeros(d_out), b)
+    offs = [0, 38_000, rows]
+    targets = torch.cat([inputs.distinct_targets(N, hi - lo, seed=lo) for lo, hi in zip(offs[:-1], offs[1:])])
+    dense = ctx.sample_many(targets, offs, [3], [1, 2])
+    out = torch.full((rows + 1, d_out), 7.0, device="cuda")
+    ctx.gat_forward(ctx.gat_model([layer]), dense, out[:rows])
+    want = torch.cat([layers_over(dense.view(i), feats, [layer], uniform_attention) for i in range(2)])
+    # (as above: operands rounded to 10 bits, sums of up to 256 products)
+    err, rms = (out[:rows].double() - want).abs(), want.square().mean().sqrt()
+    assert float(err.square().mean().sqrt() / rms) < 1e-3 and float((err / torch.maximum(want.abs(), rms)).max()) < 6e-3
+    assert torch.equal(out[rows], torch.full_like(out[rows], 7.0))
+
+
+# the same product with a ReLU: the first of two layers, one wider than the fused kernel's and one of attention
+@pytest.mark.parametrize("dims,attention", [([16, 300, 8], False), ([16, 100, 8], True), ([36, 320, 8], True)])
+def test_persistent_product_before_a_relu(graph, dims, attention):
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    feats = inputs.normal_features(N, dims[0], seed=5, device="cuda")
+    ctx.load_features(feats)
+    layers = inputs.random_bias_layers(dims, seed=6)
+    if attention:
+        layers = [(w, torch.zeros_like(b), torch.zeros_like(b), b) for w, _, b in layers]
+    per = 30_000
+    targets = torch.cat([inputs.distinct_targets(N, per, seed=b) for b in range(3)])
+    dense = ctx.sample_many(targets, [0, per, 2 * per, 3 * per], [3, 2], [1, 2, 3])
+    assert int(dense.counts()[0][:, :2].sum()) > 75_520       # rows of the first layer
+    out = torch.empty((3 * per, dims[-1]), device="cuda")
+    if attention:
+        ctx.gat_forward(ctx.gat_model(layers), dense, out)
+    else:
+        ctx.forward(ctx.model(layers), dense, out)
+    want = torch.cat([layers_over(dense.view(i), feats, layers, uniform_attention if attention else mean_aggregator) for i in range(3)])
+    # two layers, each with operands rounded to 10 bits: the bounds above twice
+    err, rms = (out.double() - want).abs(), want.square().mean().sqrt()
+    assert float(err.square().mean().sqrt() / rms) < 2e-3 and float((err / torch.maximum(want.abs(), rms)).max()) < 12e-3

@@ -310,3 +310,25 @@ def test_exports_beside_the_layers_of_other_samples(graph):
             for key in keys:
                 assert torch.equal(getattr(v, key), want[key]), (g, b, key)
     c.close()
+
+
+# the same tables beside a tile that has both directions: as many mini-batches as need no more shared memory than a kernel has without asking,
+# one more, as many as a call may have
+@pytest.mark.parametrize("n_batches", [1_408, 1_409, 4_096])
+def test_largest_tiles_of_both_directions(graph, n_batches):
+    c = mg.Context(0)
+    c.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    other = inputs.transpose_csr(graph)
+    c.load_out_graph(other.row_offsets.cuda(), other.nbrs.cuda())
+    c.set_sample_direction("inout")
+    rows = [inputs.distinct_targets(N, 60 - b % 2, seed=b) for b in range(n_batches)]      # (hop 1: room for more nodes than 12 x 148 tiles of 1,024)
+    offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    d = c.sample_many(torch.cat(rows), offs, [9, 1], list(range(n_batches)),
+                      caps={"max_nodes_per_batch": 2_400, "max_nodes_total": 2_400 * n_batches, "max_entries_total": 2_400 * n_batches})
+    for b in (0, 1, n_batches // 2, n_batches - 1):
+        one = c.sample(rows[b], [9, 1], b)
+        x, y = d.view(b), one.view(0)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
+        one.free()
+    c.close()
