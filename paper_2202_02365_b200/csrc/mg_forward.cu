@@ -846,8 +846,8 @@ extern "C" int mg_layer_output(mg_ctx* ctx, const mg_model* m, mg_dense* d, int3
 // Backward pass through the GraphSage layers (Section 3: the gradients of a mini-batch update the model and the
 // base representations).  Chain rule through Algorithm 3 and Algorithm 2, layer k down to layer 1, whole layers at a time:
 //   dPre = dH^l (masked by H^l > 0 below the last layer),
-//   dW += X^T dPre with X = [self | aggregate] gathered again from H^{l-1} (kept by the forward pass), dbias += column
-//   sums of dPre, dX = dPre W^T,
+//   dW += X^T dPre with X = [self | aggregate] from H^{l-1} (kept by the forward pass): the self rows gathered again, the aggregates
+//   too unless the forward pass has left them, dbias += column sums of dPre, dX = dPre W^T,
 //   dH^{l-1}[row] = its self part of dX + the neighbour parts of every entry that names it, times 1 / count (1 for a sum).
 // A model with TF32 products takes dW and dX on the tensor cores (X, dPre and W as they lie in memory, of which the tensor cores
 // read ten bits of the mantissa; fp32 accumulate), one with fp32 products on CUDA cores, there with X in chunks of rows.  All
@@ -1436,7 +1436,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         int64_t meta_at = 0;   // the layer's rows in ws_meta
         for (int q = 1; q < l; ++q) meta_at += d->h_hdr.rows_total[q];
         if (m->precision == MG_GEMM_TF32) {
-            // dW += X^T dPre with X gathered again inside the kernel; the row metadata is what the forward pass left (its layers all
+            // dW += X^T dPre with X brought together inside the kernel; the row metadata is what the forward pass left (its layers all
             // have it, mg_forward of this very model and sample was the last to write it)
             if ((rc = mg_layer_grad_weights(ctx, d, l, d_in, d_out, h_prev, dpre_all, ctx->ws_meta + meta_at, m->sum_aggr ? 1 : 0,
                                             ctx->agg_at[l] >= 0 && ctx->agg_sum == m->sum_aggr ? reinterpret_cast<const float*>(ctx->ws_saved + ctx->agg_at[l]) : nullptr,

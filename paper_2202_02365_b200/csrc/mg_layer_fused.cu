@@ -852,9 +852,9 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
 }
 
 // ---- weight gradients: dW += [self | aggregate]^T dPre --------------------------------------------------------------------
-// The layer's operand is gathered again, block by block of 32 rows, straight into shared memory, and contracted over the rows with
-// the gradient rows that TMA brings; it never exists in memory (before: an aggregation kernel wrote it, 1 to 2 KB per row, and a
-// product over split chunks read it back).  Bound by the gather like the forward layer.  A CTA owns 128 input columns -- their
+// The layer's operand is brought together block by block of 32 rows in shared memory, and contracted over the rows with the gradient
+// rows that TMA brings: self rows are gathered, aggregates are gathered or, where the forward pass has left them (KEPT), come by TMA.
+// (Before: an aggregation kernel wrote all of it, 1 to 2 KB per row, and a product over split chunks read it back.)  Bound by the gather like the forward layer.  A CTA owns 128 input columns -- their
 // self and aggregate halves are the two M = 128 tiles of its accumulators, all 512 columns of tensor memory with 256 output
 // columns -- and every n_slices-th block of rows; at the end it adds its 256 x 256 sums to dW with 16-byte reductions.  24 mini-batches of
 // 1,000 targets on 2M nodes: 540k rows of 2 x 128 in 252 us (257 + 190 before), 91k + 24k rows of 2 x 256 in 188 us (178 + 100).

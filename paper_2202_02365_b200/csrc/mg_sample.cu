@@ -163,13 +163,14 @@ __global__ void __launch_bounds__(kThreads) k_begin(BeginArgs a) {
 // totals are chained through one 64-bit word per tile (decoupled look-back), and the block's warps then pick for the tile's
 // nodes from shared memory.  Before, these were five kernels with the row bounds, degrees and counts going through memory
 // between them (one mini-batch of three hops on 1M nodes: 48 -> 32 us; 128 mini-batches, last hop of 2.7M nodes: 315 -> 288
-// us).  A tile has as few nodes as keeps five blocks per SM busy (hop_tile): the picks of a warp's nodes are one chain after
+// us).  A tile has as few nodes as leave five tiles per SM (hop_tile): the picks of a warp's nodes are one chain after
 // the other, and a hop of 1,000 nodes took 21 us with 256 of them per block, 10 us with 32.  Tiles are handed out by a
 // counter, as chain_tiles wants it.
 // Hop 0 also enters the targets: residency and range checks, the id table (Algorithm 1 wants unique targets).  The other hops start from the
 // counts of new nodes per mini-batch: every block sums them up for itself (block 0 writes the sums down), and the tiles' nodes are
 // read from the mini-batches' runs of new ids and put one behind the other on the way (a kernel of its own for
-// that took 3.4 to 5 us per hop of one mini-batch, 26 us for the two inner hops of 128).
+// that took 3.4 to 5 us per hop of one mini-batch, 26 us for the two inner hops of 128).  Small calls gain a launch per hop; on large ones the
+// hops take up what the placing leaves: with k_place 170 -> 164 us for 32 mini-batches of 114,000 nodes, 467 -> 465 for 128.
 struct HopArgs {
     DenseHeader* hdr;
     int hop;
@@ -203,7 +204,8 @@ struct HopArgs {
     FeatGeom feat;
 };
 
-// Nodes of a tile.  Below 256 as few as give five blocks (what the registers allow) on each SM a tile; above 256
+// Nodes of a tile.  Below 256 as few as leave five tiles per SM (measured: with four the hop of one mini-batch takes 34.9 us instead of
+// 28.7; k_hop is declared for four blocks per SM and its 48 registers let five onto one: declared for five it loses loads in flight); above 256
 // where twelve tiles per SM are left all the same: the chain through the tiles costs about 13 ns each (2.7M nodes: 620 us with
 // tiles of 64, 475 with 128, 342 with 256, 288 with 1,024).
 constexpr int kTilesPerSm = 5, kTilesPerSmLarge = 12, kTileMax = 1024, kTileSets = kTileMax / kThreads;
@@ -1854,7 +1856,8 @@ static int dense_alloc(mg_ctx* ctx, mg_dense* d, int32_t B, int32_t k, int64_t c
                        int32_t table_size, int32_t smem_nb) {
     int rc;
     if (!d->hdr && (rc = dev_realloc(ctx, &d->hdr, 1))) return rc;
-    // sort scratch: a tile per 4096 keys, and one more per (mini-batch, delta) segment for the export's segmented sort
+    // scratch of the sort of one mini-batch and of the export's bins, segments and tiles: a tile per 4096 keys, and one more per (mini-batch,
+    // delta) segment
     const int64_t want_sort_tiles = (std::max(cap_nodes, d->cap_nodes) + kSortTile - 1) / kSortTile + (int64_t)B * (k + 1);
     const bool grow_sort = d->cap_nodes < cap_nodes || d->cap_sort_tiles < want_sort_tiles;
     if (d->cap_nodes < cap_nodes) {
