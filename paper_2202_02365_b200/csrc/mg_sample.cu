@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <utility>
 
 #include "mg_device.cuh"
 #include "mg_internal.cuh"
@@ -182,6 +183,7 @@ struct HopArgs {
     int32_t* ent_off;
     int32_t* ent_nbrs;
     int32_t* ent_repr;            // receives the batch id of the entry (k_insert turns it into the id-table slot)
+    int32_t batch_of_entry;       // (0: nobody reads it, and a thread per node leaves it out)
     const uint64_t* seeds;
     int64_t cap_entries;
     uint64_t* tile_state;
@@ -220,6 +222,18 @@ __host__ __device__ __forceinline__ int hop_tile(int64_t n, int n_sms) {
 }
 // shared memory per node of a tile: id, mini-batch, first entry; first edge and length of its row, once per direction
 __host__ __device__ __forceinline__ int hop_node_bytes(bool inout) { return 12 + (inout ? 24 : 12); }
+
+// Fanouts of up to six and of eleven to kThreadPicks are picked by a thread per node where the hop may have tiles of kThreads nodes and the tile
+// has kThreadTile at least, else by a group of lanes per node.  Lanes: one look-up in flight per lane and as many Philox calls as draws; threads:
+// a quarter of the calls and all of a node's look-ups in flight.  us, lanes / threads: 71,000 nodes of 20 in one mini-batch 47 / 23, 2.7M nodes of 5 302 / 297
+// (DRAM bursts of the picks), 0.5M 67 / 54, 128,000 of 15 36 / 27; fanouts of seven to ten gain nothing (0.3M of 10: 87 / 92: the picks and the row
+// bounds in flight leave room for four blocks per SM where lanes have five), nor do fewer nodes than that (18,600 of 5: 14 / 15).
+constexpr int kThreadPicks = 20, kThreadTile = 128;
+__host__ __device__ __forceinline__ bool hop_by_thread(int f, int tile_cap) { return tile_cap >= kThreads && (f <= 6 || f > 10) && f <= kThreadPicks; }
+// shared memory for the picks of a block's threads
+__host__ __device__ __forceinline__ size_t hop_pick_bytes(int f, int tile_cap, bool inout) {
+    return hop_by_thread(f, tile_cap) ? (size_t)kThreads * f * (inout ? 2 : 1) * sizeof(uint32_t) : 0;
+}
 
 // the mini-batch of target i: a 32-way search of the warp for its first target, then a walk
 __device__ __forceinline__ int target_batch(const int32_t* __restrict__ off, int B, int32_t first, int32_t i) {
@@ -266,6 +280,53 @@ __device__ __forceinline__ uint32_t floyd_pick(bool on, uint32_t d, int32_t f, i
     }
     *rank = r;
     return pick;
+}
+
+// Batcher's odd-even merge sort of N values as a list of exchanges, so that a thread can sort what it holds in registers.
+template <int N> struct SortNet {
+    int n;
+    int a[N <= 1 ? 1 : N * N], b[N <= 1 ? 1 : N * N];
+    constexpr SortNet() : n(0), a(), b() {
+        for (int p = 1; p < N; p *= 2)
+            for (int k = p; k >= 1; k /= 2)
+                for (int j = k % p; j + k < N; j += 2 * k)
+                    for (int i = 0; i < k && i + j + k < N; ++i)
+                        if ((i + j) / (2 * p) == (i + j + k) / (2 * p)) { a[n] = i + j; b[n] = i + j + k; ++n; }
+    }
+};
+template <int I, int J>
+__device__ __forceinline__ void exchange(uint32_t* x) {
+    const uint32_t lo = min(x[I], x[J]), hi = max(x[I], x[J]);
+    x[I] = lo; x[J] = hi;
+}
+template <int N, int... C>
+__device__ __forceinline__ void sort_values(uint32_t* x, std::integer_sequence<int, C...>) {
+    constexpr SortNet<N> net;
+    (exchange<net.a[C], net.b[C]>(x), ...);
+}
+
+// Floyd's subset algorithm, a thread per node: the same draws as floyd_pick's, a Philox call for every four of them.  pick[0 .. f) are
+// the picks in ascending order.
+template <int G>
+__device__ __forceinline__ void floyd_thread(uint32_t d, int32_t f, uint64_t seed, uint32_t v, uint32_t hop, uint32_t slot_base, uint32_t (&pick)[G]) {
+#pragma unroll
+    for (int c = 0; c < G; c += 4) {
+        uint32_t w[4];
+        philox4x32_10(v, 0u, hop, (slot_base + (uint32_t)c) >> 2, (uint32_t)seed, (uint32_t)(seed >> 32), w);
+#pragma unroll
+        for (int u = 0; u < 4 && c + u < G; ++u) pick[c + u] = w[u];
+    }
+#pragma unroll
+    for (int t = 0; t < G; ++t) {
+        const uint32_t jt = d - (uint32_t)f + (uint32_t)t;
+        const uint32_t x = __umulhi(pick[t], jt + 1u);
+        bool hit = false;
+#pragma unroll
+        for (int q = 0; q < t; ++q) hit |= pick[q] == x;
+        pick[t] = t < f ? (hit ? jt : x) : 0xFFFFFFFFu;
+    }
+    constexpr SortNet<G> net;
+    sort_values<G>(pick, std::make_integer_sequence<int, net.n>{});
 }
 
 // A hop's nodes per mini-batch, summed up over the mini-batches: the new nodes of hop - 1 are hop's.  Every block takes the sums for itself
@@ -319,7 +380,8 @@ __device__ __forceinline__ int64_t sum_new_nodes(const NewNodes& a, int32_t* nex
 // G lanes per node, fanout <= G <= 32; a warp holds 32 / G nodes (G need not divide 32: the lanes left over idle, and
 // G = 5 or 10 keeps 30 lanes busy where the next power of two keeps 20).  G = 0: any fanout up to MG_MAX_FANOUT, a node per
 // warp at a time, picks staged in shared memory.
-template <int G>
+// THREAD (G <= kThreadPicks): the form for hops of many nodes; small tiles in it are picked by groups of lanes all the same.
+template <int G, bool THREAD>
 __global__ void __launch_bounds__(kThreads, 4) k_hop(HopArgs a) {
     extern __shared__ __align__(16) uint8_t hop_sm[];   // the tile's nodes, then (G = 0) per warp x[f], pick[f]
     __shared__ uint32_t part[kTileParts];
@@ -357,49 +419,103 @@ __global__ void __launch_bounds__(kThreads, 4) k_hop(HopArgs a) {
         const int32_t tile = sh_tile;
         if (tile >= n_tiles) break;
         const int32_t n_here = min(tile_nodes, n - tile * tile_nodes);
-        // node t = q * 256 + thread of the tile
+        // node t = q * 256 + thread of the tile: its id and row bounds
         uint32_t inc[kTileSets];
+        if constexpr (THREAD) {
+            // the look-ups of all sets are in flight before the first is used
+            int32_t vs[kTileSets], bs[kTileSets];
+            uint32_t cnt[kTileSets];
 #pragma unroll
-        for (int q = 0; q < kTileSets; ++q) {
-            if (q >= sets) break;
-            const int32_t t = q * kThreads + (int32_t)threadIdx.x, local = tile * tile_nodes + t;
-            const bool node_ok = t < n_here;
-            int32_t v = 0, b = 0;
-            bool in_range = node_ok;
-            if (node_ok) {
-                if (a.hop == 0) v = targets[local];
-                else {
-                    b = upper_segment(next_off, a.B, lo + local);
-                    v = a.new_ids[list_at[b] + (lo + local - next_off[b])];
-                    a.nodes[lo + local] = v;
-                    a.node_batch[lo + local] = b;
+            for (int q = 0; q < kTileSets; ++q) {
+                const int32_t t = q * kThreads + (int32_t)threadIdx.x, local = tile * tile_nodes + t;
+                vs[q] = 0; bs[q] = 0; cnt[q] = 0;
+                if (q >= sets) continue;
+                if (a.hop == 0) {
+                    if (t < n_here) vs[q] = targets[local];
+                    if (t - lane < n_here) bs[q] = target_batch(a.tgt_off, a.B, local - lane, min(local, n - 1));
+                } else if (t < n_here) {
+                    bs[q] = upper_segment(next_off, a.B, lo + local);
+                    vs[q] = __ldg(a.new_ids + list_at[bs[q]] + (lo + local - next_off[bs[q]]));
                 }
             }
-            if (a.hop == 0) {
-                if (t - lane < n_here) b = target_batch(a.tgt_off, a.B, local - lane, min(local, n - 1));
-                in_range = node_ok && v >= 0 && (int64_t)v < a.n_nodes;
-            }
-            uint32_t cnt = 0;
-            if (in_range) {
-                const int64_t r0 = a.row_off[0][v];
-                const uint32_t d = (uint32_t)(a.row_off[0][v + 1] - r0);
-                cnt = min(d, (uint32_t)f);
-                node_r0[t] = r0;
-                node_deg[t] = d;
-                if (inout) {   // incoming + outgoing sampling: up to `fanout` of each list
-                    const int64_t q0 = a.row_off[1][v];
-                    const uint32_t dq = (uint32_t)(a.row_off[1][v + 1] - q0);
-                    cnt += min(dq, (uint32_t)f);
-                    node_r0[a.tile_cap + t] = q0;
-                    node_deg[a.tile_cap + t] = dq;
+#pragma unroll
+            for (int dir = 0; dir < 2; ++dir) {   // incoming + outgoing sampling: up to `fanout` of each list
+                if (dir == 1 && !inout) break;
+                const int64_t* __restrict__ off = a.row_off[dir];
+                int64_t r0[kTileSets], r1[kTileSets];
+#pragma unroll
+                for (int q = 0; q < kTileSets; ++q) {
+                    const int32_t t = q * kThreads + (int32_t)threadIdx.x;
+                    r0[q] = 0; r1[q] = 0;
+                    if (q < sets && t < n_here && (a.hop > 0 || (vs[q] >= 0 && (int64_t)vs[q] < a.n_nodes))) { r0[q] = __ldg(off + vs[q]); r1[q] = __ldg(off + vs[q] + 1); }
                 }
-            } else if (node_ok) {
-                node_r0[t] = 0; node_deg[t] = 0;
-                if (inout) { node_r0[a.tile_cap + t] = 0; node_deg[a.tile_cap + t] = 0; }
+#pragma unroll
+                for (int q = 0; q < kTileSets; ++q) {
+                    const int32_t t = q * kThreads + (int32_t)threadIdx.x;
+                    if (q >= sets || t >= n_here) continue;
+                    const uint32_t d = (uint32_t)(r1[q] - r0[q]);
+                    cnt[q] += min(d, (uint32_t)f);
+                    node_r0[dir * a.tile_cap + t] = r0[q];
+                    node_deg[dir * a.tile_cap + t] = d;
+                }
             }
-            if (node_ok) { node_id[t] = v; node_b[t] = b; node_out[t] = cnt; }
-            inc[q] = warp_incl_scan(cnt);
-            if (lane == 31) part[q * (kThreads / 32) + warp] = inc[q];
+#pragma unroll
+            for (int q = 0; q < kTileSets; ++q) {
+                if (q >= sets) break;
+                const int32_t t = q * kThreads + (int32_t)threadIdx.x, local = tile * tile_nodes + t;
+                if (t < n_here) {
+                    node_id[t] = vs[q]; node_b[t] = bs[q]; node_out[t] = cnt[q];
+                    if (a.hop > 0) {
+                        a.nodes[lo + local] = vs[q];
+                        a.node_batch[lo + local] = bs[q];
+                    }
+                }
+                inc[q] = warp_incl_scan(cnt[q]);
+                if (lane == 31) part[q * (kThreads / 32) + warp] = inc[q];
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < kTileSets; ++q) {
+                if (q >= sets) break;
+                const int32_t t = q * kThreads + (int32_t)threadIdx.x, local = tile * tile_nodes + t;
+                const bool node_ok = t < n_here;
+                int32_t v = 0, b = 0;
+                bool in_range = node_ok;
+                if (node_ok) {
+                    if (a.hop == 0) v = targets[local];
+                    else {
+                        b = upper_segment(next_off, a.B, lo + local);
+                        v = a.new_ids[list_at[b] + (lo + local - next_off[b])];
+                        a.nodes[lo + local] = v;
+                        a.node_batch[lo + local] = b;
+                    }
+                }
+                if (a.hop == 0) {
+                    if (t - lane < n_here) b = target_batch(a.tgt_off, a.B, local - lane, min(local, n - 1));
+                    in_range = node_ok && v >= 0 && (int64_t)v < a.n_nodes;
+                }
+                uint32_t cnt = 0;
+                if (in_range) {
+                    const int64_t r0 = a.row_off[0][v];
+                    const uint32_t d = (uint32_t)(a.row_off[0][v + 1] - r0);
+                    cnt = min(d, (uint32_t)f);
+                    node_r0[t] = r0;
+                    node_deg[t] = d;
+                    if (inout) {   // incoming + outgoing sampling: up to `fanout` of each list
+                        const int64_t q0 = a.row_off[1][v];
+                        const uint32_t dq = (uint32_t)(a.row_off[1][v + 1] - q0);
+                        cnt += min(dq, (uint32_t)f);
+                        node_r0[a.tile_cap + t] = q0;
+                        node_deg[a.tile_cap + t] = dq;
+                    }
+                } else if (node_ok) {
+                    node_r0[t] = 0; node_deg[t] = 0;
+                    if (inout) { node_r0[a.tile_cap + t] = 0; node_deg[a.tile_cap + t] = 0; }
+                }
+                if (node_ok) { node_id[t] = v; node_b[t] = b; node_out[t] = cnt; }
+                inc[q] = warp_incl_scan(cnt);
+                if (lane == 31) part[q * (kThreads / 32) + warp] = inc[q];
+            }
         }
         __syncthreads();
         // entries before each warp's nodes inside the tile, the tile's count; the tiles before this one
@@ -448,6 +564,51 @@ __global__ void __launch_bounds__(kThreads, 4) k_hop(HopArgs a) {
         }
         if (!fits) break;   // (uniform over the block)
         __syncthreads();
+        if (THREAD && tile_nodes >= kThreadTile) {
+            // a thread per node: a Philox call gives four draws, and all picks of a node are looked up together.  The warp's entries are
+            // put one behind the other in shared memory and written from there.
+            constexpr int GT = THREAD ? G : 1;
+            uint32_t* out = reinterpret_cast<uint32_t*>(node_out + a.tile_cap) + (size_t)warp * 32 * f * (inout ? 2 : 1);
+#pragma unroll 1
+            for (int t0 = warp * 32; t0 < n_here; t0 += kThreads) {
+                const int t = min(t0 + lane, n_here - 1);
+                const bool on = t0 + lane < n_here;
+                const uint32_t g0 = node_out[t], base = __shfl_sync(0xFFFFFFFFu, g0, 0);
+                const int32_t gb = node_b[t];
+                uint32_t at = g0 - base;
+#pragma unroll 1
+                for (int dir = 0; dir < (inout ? 2 : 1); ++dir) {   // (the second direction's picks follow the first's)
+                    const uint32_t d = on ? node_deg[dir * a.tile_cap + t] : 0u, cnt = min(d, (uint32_t)f);
+                    const int32_t* __restrict__ row = a.row_nbrs[dir] + node_r0[dir * a.tile_cap + t];
+                    uint32_t pick[GT];
+                    if (d > (uint32_t)f) floyd_thread<GT>(d, f, a.seeds[gb], (uint32_t)node_id[t], (uint32_t)a.hop, dir ? (uint32_t)MG_OUT_SLOT_BASE : 0u, pick);
+                    else {   // all neighbours, in row order
+#pragma unroll
+                        for (int j = 0; j < GT; ++j) pick[j] = (uint32_t)j;
+                    }
+#pragma unroll
+                    for (int j = 0; j < GT; ++j) if ((uint32_t)j < cnt) pick[j] = (uint32_t)__ldg(row + pick[j]);
+#pragma unroll
+                    for (int j = 0; j < GT; ++j) if ((uint32_t)j < cnt) out[at + j] = pick[j];
+                    at += cnt;
+                }
+                const uint32_t total = __reduce_max_sync(0xFFFFFFFFu, on ? at : 0u);
+                __syncwarp();
+                for (uint32_t i = lane; i < total; i += 32) a.ent_nbrs[base + i] = (int32_t)out[i];
+                if (a.batch_of_entry) {
+                    const int32_t b0 = __shfl_sync(0xFFFFFFFFu, gb, 0);
+                    if (__all_sync(0xFFFFFFFFu, gb == b0)) {
+                        for (uint32_t i = lane; i < total; i += 32) a.ent_repr[base + i] = b0;
+                    } else {
+                        __syncwarp();
+                        if (on) for (uint32_t i = g0 - base; i < at; ++i) out[i] = (uint32_t)gb;
+                        __syncwarp();
+                        for (uint32_t i = lane; i < total; i += 32) a.ent_repr[base + i] = (int32_t)out[i];
+                    }
+                }
+                __syncwarp();
+            }
+        } else
         // the picks: warp after warp takes nodes of the tile
         for (int dir = 0; dir < (inout ? 2 : 1); ++dir) {
             const int32_t* __restrict__ row_nbrs = a.row_nbrs[dir];
@@ -2000,20 +2161,33 @@ extern "C" int mg_sample_many(mg_ctx* ctx, const int32_t* targets, int targets_o
 
 
 // dynamic shared-memory limits of the sampler's kernels (not inside a stream capture)
-constexpr int kHopSmem = kTileMax * (12 + 24) + 8 * MG_MAX_BATCHES;   // of k_hop at most: a tile with both directions, the mini-batches' tables
+// The instance for a fanout, and for as many nodes per tile as the hop may have: the narrowest group of lanes that holds the fanout among
+// those that waste at most two lanes of a warp; a thread per node where the hop fills larger tiles.
+#define MG_HOP_KERNELS k_hop<2, false>, k_hop<3, false>, k_hop<4, false>, k_hop<5, false>, k_hop<6, false>, k_hop<8, false>, k_hop<10, false>, k_hop<16, false>, \
+                       k_hop<32, false>, k_hop<2, true>, k_hop<3, true>, k_hop<4, true>, k_hop<5, true>, k_hop<6, true>, k_hop<16, true>, k_hop<20, true>
+typedef void (*HopKernel)(HopArgs);
+static HopKernel hop_kernel(int f, int tile_cap) {
+    if (hop_by_thread(f, tile_cap))
+        return f <= 2 ? k_hop<2, true> : f == 3 ? k_hop<3, true> : f == 4 ? k_hop<4, true> : f == 5 ? k_hop<5, true> : f == 6 ? k_hop<6, true> : f <= 16 ? k_hop<16, true>
+               : k_hop<20, true>;
+    return f <= 2 ? k_hop<2, false> : f == 3 ? k_hop<3, false> : f == 4 ? k_hop<4, false> : f == 5 ? k_hop<5, false> : f == 6 ? k_hop<6, false> : f <= 8 ? k_hop<8, false>
+           : f <= 10 ? k_hop<10, false> : f <= 16 ? k_hop<16, false> : f <= 32 ? k_hop<32, false> : k_hop<0, false>;
+}
+
+// of k_hop at most: a tile with both directions, the mini-batches' tables, the picks of a thread per node
+constexpr int kHopSmem = kTileMax * (12 + 24) + 8 * MG_MAX_BATCHES + kThreads * kThreadPicks * 2 * 4;
 static int sample_kernel_limits(mg_ctx* ctx) {
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_dedupe_last<1024>, (int)(kDedupMaxSlots * 2 * sizeof(int32_t))));
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_dedupe_last<512>, kDedupSlots512 * 2 * (int)sizeof(int32_t)));
-    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_hop<0>, (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + kHopSmem));
+    MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)k_hop<0, false>, (int)((size_t)(kThreads / 32) * 2 * MG_MAX_FANOUT * sizeof(uint32_t)) + kHopSmem));
     return MG_OK;
 }
 
 // ... and of the others where the mini-batches' tables of k_hop, beside its tile, come to more than a kernel has without asking
 static int hop_kernel_limits(mg_ctx* ctx, int32_t n_batches, bool inout) {
-    if (kTileMax * hop_node_bytes(inout) + 8 * n_batches <= 47 * 1024) return MG_OK;   // (48 KiB, of which k_hop has some for itself)
-    const void* hops[] = {(const void*)k_hop<2>, (const void*)k_hop<3>, (const void*)k_hop<4>, (const void*)k_hop<5>, (const void*)k_hop<6>,
-                          (const void*)k_hop<8>, (const void*)k_hop<10>, (const void*)k_hop<16>, (const void*)k_hop<32>};
-    for (const void* hop : hops) MG_CUDA(ctx, mg_smem_limit(ctx, hop, kHopSmem));
+    if (kTileMax * hop_node_bytes(inout) + 8 * n_batches + (int)hop_pick_bytes(kThreadPicks, kTileMax, inout) <= 47 * 1024) return MG_OK;   // (48 KiB, of which k_hop has some for itself)
+    const HopKernel hops[] = {MG_HOP_KERNELS};
+    for (const HopKernel hop : hops) MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)hop, kHopSmem));
     return MG_OK;
 }
 
@@ -2211,22 +2385,14 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
         {
             ProfScope ps(ctx, PH_SAMPLE_PICK);
             HopArgs a{d->hdr, h, f, d->nodes, d->node_batch, {ctx->view_off, inout ? ctx->view_off_out : nullptr},
-                      {ctx->view_nbrs, ctx->view_nbrs_out}, d->ent_off, d->ent_nbrs, d->ent_repr, d->d_seeds, d->cap_entries, d->tile_state,
+                      {ctx->view_nbrs, ctx->view_nbrs_out}, d->ent_off, d->ent_nbrs, d->ent_repr, smem_hop ? 0 : 1, d->d_seeds, d->cap_entries, d->tile_state,
                       hop_tile(nodes_bound[h], ctx->n_sms), ctx->n_sms, B, k, d->new_ids, batch_cnt + (size_t)(h > 0 ? h - 1 : 0) * B, d->cap_nodes,
                       inner_limit, d->cum, d->node_off, d->node_off, d->hkeys, d->hvals, tg, ctx->n_nodes, mg_feat_geom(ctx)};
             const unsigned grid = blocks_for(nodes_bound[h], 32, 8);
-            const size_t sm = (size_t)a.tile_cap * hop_node_bytes(inout) + (h > 0 ? 8 * (size_t)B : 0);   // 36 KiB, and 32 at the largest number of mini-batches
-            // the narrowest group that holds the fanout among those that waste at most two lanes of a warp
-            if (f <= 2) k_hop<2><<<grid, kThreads, sm, st>>>(a);
-            else if (f == 3) k_hop<3><<<grid, kThreads, sm, st>>>(a);
-            else if (f == 4) k_hop<4><<<grid, kThreads, sm, st>>>(a);
-            else if (f == 5) k_hop<5><<<grid, kThreads, sm, st>>>(a);
-            else if (f == 6) k_hop<6><<<grid, kThreads, sm, st>>>(a);
-            else if (f <= 8) k_hop<8><<<grid, kThreads, sm, st>>>(a);
-            else if (f <= 10) k_hop<10><<<grid, kThreads, sm, st>>>(a);
-            else if (f <= 16) k_hop<16><<<grid, kThreads, sm, st>>>(a);
-            else if (f <= 32) k_hop<32><<<grid, kThreads, sm, st>>>(a);
-            else k_hop<0><<<grid, kThreads, sm + (size_t)(kThreads / 32) * 2 * f * sizeof(uint32_t), st>>>(a);   // 64 KiB more at the largest fanout
+            // (36 KiB, 32 at the largest number of mini-batches, 40 for the picks of a thread per node)
+            const size_t sm = (size_t)a.tile_cap * hop_node_bytes(inout) + (h > 0 ? 8 * (size_t)B : 0) + hop_pick_bytes(f, a.tile_cap, inout);
+            const HopKernel kern = hop_kernel(f, a.tile_cap);
+            kern<<<grid, kThreads, sm + (f > 32 ? (size_t)(kThreads / 32) * 2 * f * sizeof(uint32_t) : 0), st>>>(a);   // 64 KiB more at the largest fanout
             ctx->launches++;
         }
         {

@@ -69,6 +69,33 @@ def test_hops_on_either_side_of_the_tile_sizes(graph, ctx, total):
     one.free()
 
 
+# many nodes: a thread draws and looks up a node's picks (fanouts of up to six, eleven to twenty); few: a group of lanes does.  Fanouts on either
+# side, tiles of 128 and of 256 nodes, one list and both (degrees about 6 and, of the second list, about 20; rows shorter and longer than the fanout)
+@pytest.mark.parametrize("total", [90_001, 128 * 740 + 257])
+@pytest.mark.parametrize("direction", ["in", "inout"])
+def test_picks_by_threads_and_by_groups_of_lanes(graph, total, direction):
+    c = mg.Context(0)
+    c.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    c.load_features(torch.zeros((N, 4), device="cuda"))
+    if direction == "inout":
+        other = inputs.rmat_graph(N, 20 * N, seed=22)
+        c.load_out_graph(other.row_offsets.cuda(), other.nbrs.cuda())
+        c.set_sample_direction("inout")
+    per = 9_973
+    sizes = [per] * (total // per) + [total % per]
+    ids = [inputs.distinct_targets(N, n, seed=300 + i) for i, n in enumerate(sizes)]
+    offs = np.concatenate([[0], np.cumsum(sizes)])
+    for f in (1, 2, 4, 5, 6, 7, 11, 16, 17, 20, 21):
+        d = c.sample_many(torch.cat(ids).cuda(), offs, [f], [2 ** 40 + 7 * b for b in range(len(sizes))])
+        for b in (0, 1, len(sizes) - 1):
+            one = c.sample(ids[b].cuda(), [f], 2 ** 40 + 7 * b)
+            x, y = d.view(b), one.view(0)
+            for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+                assert torch.equal(getattr(x, key), getattr(y, key)), (f, key)
+            one.free()
+        d.free()
+
+
 # the last hop: through the global tables (little room in all); buckets in shared memory, one (a table of a few hundred nodes), several
 # with tables for blocks of 256, 512 and 1,024 threads, as many tables as a mini-batch may need, and more (global tables again); ids that are multiples of a Fibonacci
 # number, whose multiplicative hashes lie next to each other
