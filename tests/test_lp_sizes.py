@@ -79,6 +79,12 @@ def test_negative_scores_by_the_number_of_tiles(edges, chunks, negs, corrupt):
             assert float(err.norm() / want.norm()) < 1e-3 and float(err.abs().max() / want.square().mean().sqrt()) < 1e-2
 
 
+# rows of scores that start 32-byte aligned (stored as they are), 16-byte aligned, and neither; widths that end inside a slice of 32 columns
+@pytest.mark.parametrize("edges,chunks,negs", [(500, 2, 8), (131, 1, 104), (1_000, 3, 500), (300, 1, 996), (300, 1, 1_001)])
+def test_negative_scores_by_the_alignment_of_their_rows(edges, chunks, negs):
+    test_negative_scores_by_the_number_of_tiles(edges, chunks, negs, mg.CORRUPT_BOTH)
+
+
 # batches are prepared while the scores of the ones before are computed, in the blocks of freed batches: growing, shrinking, two alive at once
 @pytest.mark.parametrize("sizes", [[40_000] * 6, [100, 40_000, 300, 50_000, 20_000, 60_000]])
 def test_batches_prepared_beside_scores(sizes):
