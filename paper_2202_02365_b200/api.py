@@ -16,6 +16,7 @@ import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libmgdense.so")
+VIEWS_PATH = os.path.join(HERE, "_mgviews.so")
 
 MG_OK = 0
 ERR_NAMES = {-1: "MG_ERR_ARG", -2: "MG_ERR_STATE", -3: "MG_ERR_NONRESIDENT", -4: "MG_ERR_DUPLICATE",
@@ -53,18 +54,24 @@ class DenseArrays(C.Structure):
 
 
 _lib = None
+_views = None           # the native part of the binding (csrc/mg_views.cpp) ...
+_export_copy = 0        # ... and the entry point it calls
 
 
 def load_library(path: str = LIB_PATH) -> C.CDLL:
     """dlopen the library (works without a GPU; calls then fail with MG_ERR_CUDA)."""
-    global _lib
+    global _lib, _views, _export_copy
     if _lib is None:
-        if not os.path.exists(path):
-            raise RuntimeError(f"{path} is missing: run `python -m paper_2202_02365_b200.build` "
-                               "(there is no fallback implementation)")
-        _lib = C.CDLL(path)
-        _lib.mg_last_error.restype = C.c_char_p
-        _lib.mg_kernel_launches.restype = C.c_int64
+        for needed in (path, VIEWS_PATH):
+            if not os.path.exists(needed):
+                raise RuntimeError(f"{needed} is missing: run `python -m paper_2202_02365_b200.build` "
+                                   "(there is no fallback implementation)")
+        from . import _mgviews
+        lib = C.CDLL(path)
+        lib.mg_last_error.restype = C.c_char_p
+        lib.mg_kernel_launches.restype = C.c_int64
+        _views, _export_copy = _mgviews, C.cast(lib.mg_dense_export_copy_aligned, C.c_void_p).value
+        _lib = lib
     return _lib
 
 
@@ -207,14 +214,14 @@ class Dense:
 
     def export_view(self, batch: int = 0) -> DenseView:
         """Mini-batch `batch` of the last export_many, ready in the order of torch's current stream.  (The stream waits for the
-        export, not the host: 32 mini-batches' views are queued while the export runs, the whole call 1107 -> 910 us.)"""
-        arr, at, ctx = DenseArrays(), C.c_int32(batch), self.ctx
-        ref, copy = C.byref(arr), ctx.lib.mg_dense_export_copy_aligned
-        ctx._check(copy(ctx.handle, self.handle, at, ref, None, _ALIGN, None))
-        room = _room(arr)
-        out = torch.empty(sum(room), dtype=torch.int32, device=ctx.device)
-        ctx._check(copy(ctx.handle, self.handle, at, ref, _ptr(out), _ALIGN, _raw_stream(ctx.device)))
-        return DenseView(*_pieces(out, room)[::2])
+        export, not the host: 32 mini-batches' views are queued while the export runs, the whole call 1107 -> 910 us; one call into native
+        code per view, 875 -> 688.)"""
+        ctx = self.ctx
+        views = _views.export_view(_export_copy, ctx.handle.value or 0, self.handle.value or 0, batch, ctx.device.index,
+                                   torch._C._cuda_getCurrentRawStream(ctx.device.index))
+        if type(views) is int:
+            ctx._check(views)
+        return DenseView(*views)
 
     def free(self):
         if self.handle:

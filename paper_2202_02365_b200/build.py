@@ -1,4 +1,5 @@
-"""Builds libmgdense.so (sm_100a only) next to this file with nvcc; no JIT cache is used."""
+"""Builds libmgdense.so (sm_100a only) next to this file with nvcc, and _mgviews.so, the part of the binding that makes torch tensors, with
+g++; no JIT cache is used."""
 from __future__ import annotations
 
 import os
@@ -11,6 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmgdense.so")
+VIEWS = os.path.join(HERE, "_mgviews.so")
 OBJ_DIR = os.path.join(HERE, "build")
 
 NVCC_FLAGS = [
@@ -29,6 +31,17 @@ def _nvcc() -> str:
 
 def sources():
     return sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cu"))
+
+
+def _views_command(src: str):
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+    includes = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], *cpp_extension.include_paths()]
+    libs = cpp_extension.library_paths()
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            *[f for d in includes for f in ("-isystem", d)], src, "-o", VIEWS, *[f"-L{d}" for d in libs], "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10"]
 
 
 def _stale(target: str, deps) -> bool:
@@ -56,10 +69,12 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         if r.returncode != 0 or verbose:
             sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
         if r.returncode != 0:
-            raise RuntimeError("nvcc failed: " + " ".join(cmd))
+            raise RuntimeError("compiler failed: " + " ".join(cmd))
 
-    with ThreadPoolExecutor(max_workers=max(1, min(8, len(jobs)))) as ex:
-        list(ex.map(run, jobs))
+    views_src = os.path.join(CSRC, "mg_views.cpp")
+    views = [_views_command(views_src)] if force or _stale(VIEWS, [views_src, os.path.join(ROOT, "include", "mgdense.h")]) else []
+    with ThreadPoolExecutor(max_workers=max(1, min(8, len(jobs) + 1))) as ex:
+        list(ex.map(run, jobs + views))
     if jobs or force or _stale(LIB, objs):
         run([nvcc, "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a",
              "-Xcompiler", "-fPIC", "-lcudart_static", "-ldl", "-lpthread", "-lrt"])
