@@ -2254,7 +2254,11 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     int64_t min_nb = (cap_batch + kDedupMaxSlots - 1) / kDedupMaxSlots;
     while (min_nb <= kDedupMaxTables && dedup_slots_for((cap_batch + min_nb - 1) / min_nb) > kDedupMaxSlots) ++min_nb;
     const int64_t dedup_nb = min_nb <= kDedupMaxTables ? dedup_buckets(n_batches, cap_batch, min_nb, ctx->n_sms) : min_nb;
-    const int32_t dedup_slots = (int32_t)std::min<int64_t>(dedup_slots_for((cap_batch + dedup_nb - 1) / dedup_nb), kDedupMaxSlots);
+    // A block of 1,024 threads has its SM's shared memory to itself: its table is half as large again as it has to be, where there is room, and
+    // the probes are shorter (64,000 entries and 29,000 nodes in the buckets of 37 mini-batches 63 -> 58 us, 128 of 103,000 286 -> 273; the smaller
+    // blocks gain nothing, 49 -> 50).
+    const int32_t dedup_least = (int32_t)std::min<int64_t>(dedup_slots_for((cap_batch + dedup_nb - 1) / dedup_nb), kDedupMaxSlots);
+    const int32_t dedup_slots = dedup_least > kDedupSlots512 ? std::min(kDedupMaxSlots, (dedup_least * 3 / 2 + 127) / 128 * 128) : dedup_least;
     const bool smem_fits = min_nb <= kDedupMaxTables && dedup_nb * n_batches < (1ll << 24) && cap_entries + cap_nodes < (1ll << 31);
     // Small samples go through the global tables in any case: these stay in L2, and k_insert takes one launch where the shared tables
     // take two (room for 14,000 nodes: the whole call 94 -> 84 us, 80,000: 192 -> 175 us, 8 x 83,000: 893 -> 883 us, 64 x 42,000:
