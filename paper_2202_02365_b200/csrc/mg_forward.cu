@@ -22,6 +22,7 @@ int mg_gemm_tf32_status(mg_ctx* ctx);
 // mg_layer_fused.cu
 bool mg_layer_fused_supported(int d_in, int d_out);
 int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int4* meta, const int64_t* start /* [k + 2], layer l at start[l] */);
+bool mg_layer_rows_inline(const mg_ctx* ctx, const mg_dense* d);   // the layers' kernels do without it
 int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* w_pad_t, const float* bias,
                    const float* h_prev, float* h_out, float* h_out2 /* nullable: the rows once more */, int flags /* 1 = ReLU, 2 = sum instead of mean */, const int4* row_meta,
                    int64_t row_lo, int64_t row_hi, int64_t safe_src_row, const void* w_pad_h /* the layer's fp16 weights, nullable */,
@@ -579,8 +580,11 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
     for (int l = 1; l <= k; ++l) all_fused = all_fused && mg_layer_fused_supported(m->dims[l - 1], m->dims[l]);
     // row metadata of the layers the fused kernel runs, all in one launch
     const bool any_fused = m->precision == MG_GEMM_TF32;
+    // (few rows of one mini-batch: the layers' kernels look it up themselves, unless the profile is to have its phase)
     int64_t meta_at[MG_MAX_HOPS + 2] = {0};
-    if (any_fused && (rc = row_metadata(ctx, d, meta_at))) return rc;
+    const bool rows_inline = all_fused && !ctx->keep_layers && !ctx->prof_on && ctx->layer_window_batches == 0 && mg_layer_rows_inline(ctx, d);
+    ctx->meta_left = any_fused && !rows_inline;
+    if (ctx->meta_left && (rc = row_metadata(ctx, d, meta_at))) return rc;
     // H^k stays in the library's buffer (mg_layer_output, mg_backward) and goes to the caller's: the last layer's kernel
     // stores its tiles to both when it can (the copy behind it read and wrote the rows once more: 41 us for 128,000 rows of
     // 1 KB, and a launch).  Not into the feature table, which other tiles still read.
@@ -705,7 +709,7 @@ static int forward_pass(mg_ctx* ctx, const mg_model* m, mg_dense* d, float* out,
             {
                 ProfScope ps(ctx, l == 1 ? PH_AGG_L1 : PH_AGG_REST);
                 rc = mg_layer_fused(ctx, d, l, d_in, d_out, m->w_pad_t[l - 1], m->bias[l - 1], h_prev, h_out, l == k ? out2 : nullptr,
-                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), ctx->ws_meta + meta_at[l], 0, M, 0,
+                                    (l < k ? 1 : 0) | (m->sum_aggr ? 2 : 0), rows_inline ? nullptr : ctx->ws_meta + meta_at[l], 0, M, 0,
                                     (l == 1 || f16_inter) ? m->w_pad_h[l - 1] : nullptr, f16_inter && l > 1, f16_inter && l < k,
                                     ctx->positive_at[l] >= 0 ? ctx->ws_saved + ctx->positive_at[l] : nullptr,
                                     ctx->agg_at[l] >= 0 ? reinterpret_cast<float*>(ctx->ws_saved + ctx->agg_at[l]) : nullptr);
@@ -1385,7 +1389,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     const RowGeom geom{B, k, d->rowbase, d->cum, d->node_off};
     const bool half = ctx->feat_dtype == MG_DTYPE_F16;
     const int grid = mg_grid(ctx, 8);
-    if (m->precision == MG_GEMM_FP32) {   // (the forward pass of the others has left it)
+    if (!ctx->meta_left) {   // (most forward passes have left it)
         int64_t meta_at[MG_MAX_HOPS + 2] = {0};
         if ((rc = row_metadata(ctx, d, meta_at))) return rc;
     }

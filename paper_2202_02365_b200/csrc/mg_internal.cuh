@@ -135,7 +135,8 @@ struct mg_ctx {
     // forward workspaces (grown on demand)
     float* ws_x = nullptr; size_t ws_x_bytes = 0;
     float* ws_h[2] = {nullptr, nullptr}; size_t ws_h_bytes[2] = {0, 0};
-    int4* ws_meta = nullptr; size_t ws_meta_elems = 0;   // row metadata of the fused layers (mg_layer_rows)
+    int4* ws_meta = nullptr; size_t ws_meta_elems = 0;   // row metadata of the fused layers (mg_layer_rows) ...
+    bool meta_left = false;                              // ... of the last forward pass, where that did not look it up on the way
     // what a forward pass that keeps its layers leaves to save the backward pass work: a bit per value of the outputs (above zero), then
     // aggregates of the rows.  The backward pass does without where there is no memory for it (mg_malloc).
     uint32_t* ws_saved = nullptr; size_t ws_saved_elems = 0;

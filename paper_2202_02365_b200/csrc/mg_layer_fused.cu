@@ -91,7 +91,7 @@ struct FusedArgs {
     const int32_t* ent_off;
     const int32_t* ent_nbrs;
     const int32_t* ent_repr;
-    const int4* row_meta;        // [M] (self source row, first entry, entry count, first H^{l-1} row of the batch)
+    const int4* row_meta;        // [M] (self source row, first entry, entry count, first H^{l-1} row of the batch), or null: see row_of_sample
     // input rows
     const float* h_prev;         // layers >= 2: [rows of layer l-1, d_in]
     const char* src_base;        // layer 1: the feature buffer; later layers: h_prev
@@ -191,6 +191,27 @@ template <> struct PieceSum<true> {
     }
     static __device__ __forceinline__ uint4 self_operand(const uint4& r) { return r; }   // fp16 rows are operands as they are
 };
+
+// Row metadata of a sample of one mini-batch, as the planners take it from the sample themselves: lane h knows hop h's first row and first
+// node (there is no mini-batch to look up).  A row then takes the same round trip as from mg_layer_rows' table, and a call of few rows, which is a
+// chain of launches, has one launch less (two layers on a graph of 10,000: the whole call 73.3 -> 70.7 us; three on 1M nodes 154 -> 152.6).
+struct HopOfLane { int32_t row0, node0; };
+__device__ __forceinline__ HopOfLane hop_of_lane(const FusedArgs& a) {
+    const int lane = threadIdx.x & 31;
+    const bool on = lane <= a.k - a.layer;
+    return {on ? __ldg(a.cum + lane) : 0, on ? __ldg(a.node_off + 2 * lane) : 0};
+}
+template <bool FIRST>
+__device__ __forceinline__ int4 row_of_sample(const FusedArgs& a, HopOfLane hops, int32_t r, bool on) {
+    int32_t idx = 0;
+    for (int h = 0; h <= a.k - a.layer; ++h) {
+        const int32_t row0 = __shfl_sync(0xFFFFFFFFu, hops.row0, h), node0 = __shfl_sync(0xFFFFFFFFu, hops.node0, h);
+        if (r >= row0) idx = node0 + (r - row0);
+    }
+    if (!on) return make_int4(a.safe_src, 0, -1, 0);
+    const int32_t e0 = __ldg(a.ent_off + idx), e1 = __ldg(a.ent_off + idx + 1);
+    return make_int4(FIRST ? (int32_t)feat_row(a.feat, __ldg(a.nodes + idx)) : r, e0, e1 - e0, 0);
+}
 
 // A planner warp's work on one row block, lane = row: the rows' metadata, their entries translated to source rows, each row's
 // first kUnroll source rows, all in shared memory.
@@ -566,6 +587,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
         // and what the gather and epilogue warps touch comes behind the planners' barriers.  (The two instructions in every
         // warp cost the gather warps registers: the first layer of 128 mini-batches 1.81 -> 1.86 ms.)
         pdl_trigger();
+        HopOfLane hops = {0, 0};
+        if (ROWS < BM && !a.row_meta) hops = hop_of_lane(a);   // (the sample is older than the kernel before this one)
         pdl_wait();
         bool ok = true;
         for (uint32_t q = plw; ok; q += kPlanners) {
@@ -580,7 +603,8 @@ k_sage_layer_fused(const __grid_constant__ CUtensorMap map_w, const __grid_const
             if (!ok) break;
             const int64_t r = a.row_lo + t * TM + (q % kBlocks) * kBlockRows + lane;
             int4 rm = make_int4(a.safe_src, 0, -1, 0);
-            if (r < a.M) rm = __ldg(a.row_meta + r);   // (self source row, first entry, count, first H^{l-1} row of the batch)
+            if (ROWS < BM && !a.row_meta) rm = row_of_sample<FIRST>(a, hops, (int32_t)r, r < a.M);
+            else if (r < a.M) rm = __ldg(a.row_meta + r);   // (self source row, first entry, count, first H^{l-1} row of the batch)
             plan_block<FIRST>(a, keys, rm, meta[slot], src_rows[slot], first_rows[slot], &plan_total[slot]);
             if (lane == 0) mbar_arrive(&plan_full[slot]);
         }
@@ -1106,6 +1130,22 @@ static bool make_map_f16(CUtensorMap* map, const void* base, int64_t rows, int K
 
 bool mg_layer_fused_supported(int d_in, int d_out) { return d_out <= 256 && d_out % 4 == 0 && d_in % 4 == 0; }
 
+// Rows of a layer's tiles.  Halves per tile: the CTA pair with the most rows sets the time, and a row of a one-half tile costs about a seventh
+// more where its pair has several of them.  (The three layers of one mini-batch on 1M nodes, 23,400, 4,300 and 1,000 rows: 93 us in
+// 128-row tiles, the whole call 214 -> 195 us; 128 mini-batches keep them: 4.0 ms either way.)
+static int mg_layer_tile(const mg_ctx* ctx, int64_t rows) {
+    const int64_t pairs = ctx->n_sms / 2;
+    const int64_t rounds1 = (rows + 2 * HM * pairs - 1) / (2 * HM * pairs), rounds2 = (rows + 4 * HM * pairs - 1) / (4 * HM * pairs);
+    return rows <= 2 * kBlockRows * pairs ? kBlockRows : rounds1 * 8 < rounds2 * 14 ? HM : BM;
+}
+
+bool mg_layer_rows_inline(const mg_ctx* ctx, const mg_dense* d) {
+    if (d->n_batches != 1) return false;
+    for (int l = 1; l <= d->k; ++l)
+        if (mg_layer_tile(ctx, d->h_hdr.rows_total[l]) == BM) return false;
+    return true;
+}
+
 static void fill_args(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, FusedArgs* pa) {
     FusedArgs& a = *pa;
     const int B = d->n_batches;
@@ -1141,8 +1181,9 @@ int mg_layer_rows(mg_ctx* ctx, const mg_dense* d, int4* meta, const int64_t* sta
 // Runs layer `layer` (1-based) for the packed output rows [row_lo, row_hi).  h_prev and h_out are indexed by
 // GLOBAL packed row (callers that keep only a window of a layer pass pointers shifted accordingly).  h_out2 (nullable, 16-byte
 // aligned): receives the same rows.  positive (nullable): mg_positive_words of the layer; kept_agg (nullable, layers >= 2):
-// [rows of the layer, d_in].  The kernel is launched as a programmatic dependent of the one queued before it, which
-// must be mg_layer_rows' or another layer's.
+// [rows of the layer, d_in].  row_meta: the layer's part of mg_layer_rows' result, or null where mg_layer_rows_inline says so.  The kernel is
+// launched as a programmatic dependent of the one queued before it where that is mg_layer_rows' or another layer's: all layers but a
+// first one without row_meta, whose weights the kernel before it may have written.
 int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_out, const float* w_pad_t, const float* bias,
                    const float* h_prev, float* h_out, float* h_out2, int flags, const int4* row_meta, int64_t row_lo, int64_t row_hi,
                    int64_t safe_src_row, const void* w_pad_h, int in_f16, int out_f16, uint32_t* positive, float* kept_agg) {
@@ -1175,12 +1216,8 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     const int b_bytes = (a.BN / 2) * 128;       // each CTA of a pair stages half of the output columns
     const int n_chunks = 2 * a.d_in_pad / kce;
     a.sa = std::min(8, n_chunks);   // one group of (self, mean) slice pairs: 128 input columns
-    // Halves per tile: the CTA pair with the most rows sets the time, and a row of a one-half tile costs about a seventh more
-    // where its pair has several of them.  (The three layers of one mini-batch on 1M nodes, 23,400, 4,300 and 1,000 rows: 93 us in
-    // 128-row tiles, the whole call 214 -> 195 us; 128 mini-batches keep them: 4.0 ms either way.)
     const int64_t rows = row_hi - row_lo, pairs = ctx->n_sms / 2;
-    const int64_t rounds1 = (rows + 2 * HM * pairs - 1) / (2 * HM * pairs), rounds2 = (rows + 4 * HM * pairs - 1) / (4 * HM * pairs);
-    const int tile_rows = rows <= 2 * kBlockRows * pairs ? kBlockRows : rounds1 * 8 < rounds2 * 14 ? HM : BM, halves = tile_rows > HM ? 2 : 1;
+    const int tile_rows = mg_layer_tile(ctx, rows), halves = tile_rows > HM ? 2 : 1;
     a.sb = std::max(2, std::min({kMaxStages, n_chunks, ring_bytes(halves) / b_bytes}));
     // weights in tensor memory: TF32 operands, fp32 output, all of K in 256 columns, at most 256 output columns
     // ... and rows with few entries: a half tile of long rows is gathered for longer than its weight slices take to
@@ -1225,7 +1262,7 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     cudaLaunchAttribute pdl;
     pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &pdl; cfg.numAttrs = 1;
+    cfg.attrs = &pdl; cfg.numAttrs = layer > 1 || row_meta ? 1 : 0;
     MG_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, mw, mo, mo2, a));
     ctx->launches++;
     MG_CUDA(ctx, cudaGetLastError());

@@ -154,3 +154,52 @@ def test_persistent_product_before_a_relu(graph, dims, attention):
     # two layers, each with operands rounded to 10 bits: the bounds above twice
     err, rms = (out.double() - want).abs(), want.square().mean().sqrt()
     assert float(err.square().mean().sqrt() / rms) < 2e-3 and float((err / torch.maximum(want.abs(), rms)).max()) < 12e-3
+
+
+# few rows of one mini-batch: the layers' kernels look the rows up in the sample themselves; a second mini-batch of one node makes them use
+# the table made before, and the rows are the same bit for bit.  One to three hops, empty hops, a table in slots of a buffer
+@pytest.mark.parametrize("rows,fanouts", [(1, [3]), (33, [9, 4]), (700, [5, 3, 2]), (2_000, [0, 2]), (4_737, [2])])
+@pytest.mark.parametrize("slots", [False, True])
+def test_rows_looked_up_by_the_layers(graph, rows, fanouts, slots):
+    if 0 in fanouts:
+        graph = inputs.build_csr(torch.tensor([3]), torch.tensor([4]), N)      # (no neighbours to speak of)
+        fanouts = [1] * len(fanouts)
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    ctx.set_partitioning(4)
+    feats = inputs.normal_features(N, 36, seed=5)
+    if slots:
+        ctx.load_features(feats.pin_memory(), capacity_parts=3, backing=mg.BACKING_HOST)
+        ctx.set_resident([3, 0, 2])
+        pool = torch.cat([torch.arange(0, N // 4), torch.arange(N // 2, N)])
+    else:
+        ctx.load_features(feats.cuda(), capacity_parts=4)
+        ctx.set_resident([0, 1, 2, 3])
+        pool = torch.arange(N)
+    ids = pool[torch.randperm(len(pool), generator=torch.Generator().manual_seed(rows))[:rows + 1]].to(torch.int32)
+    dims = [36] + [64] * (len(fanouts) - 1) + [20]
+    model = ctx.model(inputs.random_bias_layers(dims, seed=6))
+    one, two = torch.empty((rows, 20), device="cuda"), torch.empty((rows + 1, 20), device="cuda")
+    before = ctx.kernel_launches()
+    ctx.forward(model, ctx.sample(ids[:rows], fanouts, seed=8), one)
+    alone = ctx.kernel_launches() - before
+    ctx.forward(model, ctx.sample_many(ids, [0, rows, rows + 1], fanouts, [8, 9]), two)
+    assert torch.equal(one, two[:rows])
+    assert ctx.kernel_launches() - before - alone > alone
+
+
+# the backward pass of such a pass makes the table itself
+def test_backward_behind_rows_looked_up_by_the_layers(graph):
+    got = []
+    for keep in (False, True):
+        ctx = mg.Context(0)
+        ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+        ctx.load_features(inputs.normal_features(N, 36, seed=5, device="cuda"))
+        ctx.keep_layer_outputs(keep)
+        model = ctx.model(inputs.random_bias_layers([36, 64, 20], seed=6))
+        dense = ctx.sample(inputs.distinct_targets(N, 500, seed=7), [5, 3], seed=8)
+        ctx.forward(model, dense, torch.empty((500, 20), device="cuda"))
+        got.append(ctx.backward(model, dense, inputs.normal_features(500, 20, seed=9, device="cuda")))
+    for a, b in zip(*got):
+        for x, y in zip(a, b):      # the same products of operands rounded to ten bits, summed in another order: a few 2^-24 of the norm
+            assert float((x.double() - y.double()).norm() / y.double().norm()) < 1e-5
