@@ -117,7 +117,7 @@ struct FusedArgs {
     uint32_t* error;
 };
 
-constexpr int kTsMaxEntriesPerRow = 8;   // layers with more entries per output row than this stream their weights
+constexpr int kTsMaxEntriesPerRow = 8, kTsMaxEntriesNarrow = 16;   // layers with more entries per output row than this stream their weights (narrow: at most 128 output columns)
 constexpr int kLaneEntries = 32;   // rows up to this long are translated by their own lane of the planner warp
 constexpr int kKeyCap = 704;    // source-row indices of a row block's entries cached in shared memory (22 per row: what still fits the 196 KB carve-out)
 
@@ -1222,9 +1222,10 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     // weights in tensor memory: TF32 operands, fp32 output, all of K in 256 columns, at most 256 output columns
     // ... and rows with few entries: a half tile of long rows is gathered for longer than its weight slices take to
     // arrive, so the stream costs nothing there, while the transposed epilogue does (measured: 5.3 entries per row,
-    // 2.03 -> 1.92 ms with the weights in tensor memory; 20 per row, 0.83 -> 0.90 ms)
+    // 2.03 -> 1.92 ms with the weights in tensor memory; 20 per row, 0.83 -> 0.90 ms).  That epilogue is half as long for up to 128 output
+    // columns: 71,000 rows of 11 entries, 100 -> 100 columns, 92 -> 87 us; 66,000 of 14, 32 to 128 columns, 72 -> 70 to 92 -> 87
     const int64_t layer_entries = d->h_hdr.ent_base[d->k - layer + 1], layer_rows = d->h_hdr.rows_total[layer];
-    const bool ts = n_chunks <= 8 && d_out <= 256 && layer_entries <= kTsMaxEntriesPerRow * layer_rows && !getenv("MG_FUSED_NO_TS");
+    const bool ts = n_chunks <= 8 && d_out <= 256 && layer_entries <= (d_out <= 128 ? kTsMaxEntriesNarrow : kTsMaxEntriesPerRow) * layer_rows && !getenv("MG_FUSED_NO_TS");
     if (ts) { a.tmem_cols = 512; a.sb = 0; a.w_rows = f16 ? (const void*)w_pad_h : (const void*)w_pad_t; }
     const size_t smem = (size_t)a.sa * stage_bytes(halves) + (size_t)a.sb * b_bytes + 1024;
     CUtensorMap mw;
