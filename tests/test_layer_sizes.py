@@ -203,3 +203,26 @@ def test_backward_behind_rows_looked_up_by_the_layers(graph):
     for a, b in zip(*got):
         for x, y in zip(a, b):      # the same products of operands rounded to ten bits, summed in another order: a few 2^-24 of the norm
             assert float((x.double() - y.double()).norm() / y.double().norm()) < 1e-5
+
+
+# rows of 9 to 16 entries on average keep their weights in tensor memory where the outputs are narrow, and stream them where they are not or where
+# the rows are longer; against the streamed form, bit for bit, and the definition
+@pytest.mark.parametrize("d_in,d_out", [(100, 100), (128, 128), (32, 4), (64, 132)])
+@pytest.mark.parametrize("fanout", [12, 40])
+def test_long_rows_of_narrow_outputs(monkeypatch, d_in, d_out, fanout):
+    g = inputs.erdos_renyi_graph(N, 22 * N, seed=33)
+    ctx = mg.Context(0)
+    ctx.load_graph(g.row_offsets.cuda(), g.nbrs.cuda())
+    feats = inputs.normal_features(N, d_in, seed=5, device="cuda")
+    ctx.load_features(feats)
+    (layer,) = inputs.random_bias_layers([d_in, d_out], seed=6)
+    rows = 20_001
+    dense = ctx.sample(inputs.distinct_targets(N, rows, seed=7), [fanout], seed=8)
+    out, streamed = torch.empty((rows, d_out), device="cuda"), torch.empty((rows, d_out), device="cuda")
+    ctx.forward(ctx.model([layer]), dense, out)
+    monkeypatch.setenv("MG_FUSED_NO_TS", "1")
+    ctx.forward(ctx.model([layer]), dense, streamed)
+    assert torch.equal(out, streamed)
+    want = last_layer(dense.view(0), feats, *layer)
+    # (operands rounded to 10 bits: as in test_rows_on_either_side_of_the_tile_sizes)
+    assert float((out.double() - want).norm() / want.norm()) < 1e-3
