@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(256) k_distmult_neg(NegArgs a) {
 // h[keep] (*) rel[r] are gathered once (eight warps), rounded to TF32 and written K-major with the 128-byte swizzle.
 // Then, block by block: one thread streams the operand images (two buffers), one thread issues the tcgen05 MMAs (fp32
 // accumulator in tensor memory, two buffers), and eight epilogue warps -- four from the start, four more once the left
-// operand is in place -- store the scores as coalesced row segments.  The score matrix (4 bytes per (edge, negative))
+// operand is in place -- store the scores, as full sectors from registers or as coalesced row segments.  The score matrix (4 bytes per (edge, negative))
 // is the bulk of the traffic; the contraction itself is small.  Every wait is bounded.
 constexpr int kTcGatherWarps = 8, kTcEpilogueWarps = 8;   // warps 4..7 gather first and store afterwards
 constexpr int kTcFirstGatherWarp = 4;
