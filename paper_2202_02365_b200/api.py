@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import warnings
 import weakref
 from dataclasses import dataclass
 
@@ -54,25 +55,36 @@ class DenseArrays(C.Structure):
 
 
 _lib = None
-_views = None           # the native part of the binding (csrc/mg_views.cpp) ...
+_views = None           # the native part of the binding (csrc/mg_views.cpp), False where it was not built ...
 _export_copy = 0        # ... and the entry point it calls
 
 
 def load_library(path: str = LIB_PATH) -> C.CDLL:
     """dlopen the library (works without a GPU; calls then fail with MG_ERR_CUDA)."""
-    global _lib, _views, _export_copy
+    global _lib
     if _lib is None:
-        for needed in (path, VIEWS_PATH):
-            if not os.path.exists(needed):
-                raise RuntimeError(f"{needed} is missing: run `python -m paper_2202_02365_b200.build` "
-                                   "(there is no fallback implementation)")
-        from . import _mgviews
-        lib = C.CDLL(path)
-        lib.mg_last_error.restype = C.c_char_p
-        lib.mg_kernel_launches.restype = C.c_int64
-        _views, _export_copy = _mgviews, C.cast(lib.mg_dense_export_copy_aligned, C.c_void_p).value
-        _lib = lib
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: run `python -m paper_2202_02365_b200.build` "
+                               "(there is no fallback implementation)")
+        _lib = C.CDLL(path)
+        _lib.mg_last_error.restype = C.c_char_p
+        _lib.mg_kernel_launches.restype = C.c_int64
     return _lib
+
+
+def _load_views():
+    """The native views, loaded by the first call that wants them: the library needs nothing of them.  Without them the same calls are made
+    from Python, at 13 us of host time a view instead of 8."""
+    global _views, _export_copy
+    if _views is None:
+        if os.path.exists(VIEWS_PATH):
+            from . import _mgviews
+            _export_copy = C.cast(load_library().mg_dense_export_copy_aligned, C.c_void_p).value
+            _views = _mgviews
+        else:
+            warnings.warn(f"{VIEWS_PATH} is missing (`python -m paper_2202_02365_b200.build` makes it): views of an export take longer", RuntimeWarning, stacklevel=3)
+            _views = False
+    return _views
 
 
 def _ptr(t: torch.Tensor | None):
@@ -217,11 +229,20 @@ class Dense:
         export, not the host: 32 mini-batches' views are queued while the export runs, the whole call 1107 -> 910 us; one call into native
         code per view, 875 -> 688.)"""
         ctx = self.ctx
-        views = _views.export_view(_export_copy, ctx.handle.value or 0, self.handle.value or 0, batch, ctx.device.index,
-                                   torch._C._cuda_getCurrentRawStream(ctx.device.index))
-        if type(views) is int:
-            ctx._check(views)
-        return DenseView(*views)
+        native = _views or _load_views()
+        if native:
+            views = native.export_view(_export_copy, ctx.handle.value or 0, self.handle.value or 0, batch, ctx.device.index,
+                                       torch._C._cuda_getCurrentRawStream(ctx.device.index))
+            if type(views) is int:
+                ctx._check(views)
+            return DenseView(*views)
+        arr, at, copy = DenseArrays(), C.c_int32(batch), ctx.lib.mg_dense_export_copy_aligned
+        ref = C.byref(arr)
+        ctx._check(copy(ctx.handle, self.handle, at, ref, None, _ALIGN, None))
+        room = _room(arr)
+        out = torch.empty(sum(room), dtype=torch.int32, device=ctx.device)
+        ctx._check(copy(ctx.handle, self.handle, at, ref, _ptr(out), _ALIGN, _raw_stream(ctx.device)))
+        return DenseView(*_pieces(out, room)[::2])
 
     def free(self):
         if self.handle:

@@ -47,6 +47,24 @@ def test_arrays_start_on_their_own_and_live_on_their_own(sample, export):
         assert int(weight.grad.sum()) == 2 * len(v.node_ids)
 
 
+# the same views where the native part was not built, and that it is missing is said
+@pytest.mark.gpu
+def test_export_views_without_the_native_part(sample, monkeypatch):
+    ctx, dense = sample
+    dense.export_many()
+    keys = ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map")
+    native = [dense.export_view(b) for b in range(3)]
+    monkeypatch.setattr(api, "_views", None)
+    monkeypatch.setattr(api, "VIEWS_PATH", api.VIEWS_PATH + ".missing")
+    with pytest.warns(RuntimeWarning, match="missing"):
+        plain = [dense.export_view(b) for b in range(3)]
+    for x, y in zip(native, plain):
+        for key in keys:
+            assert torch.equal(getattr(x, key), getattr(y, key)) and getattr(y, key).data_ptr() % 512 == 0
+    with pytest.raises(mg.MgError):
+        dense.export_view(3)
+
+
 @pytest.mark.gpu
 def test_gradients_may_be_changed_in_place(sample):
     ctx, dense = sample

@@ -2,6 +2,9 @@
 symbol the header declares; the binding refuses to run without a device."""
 import os
 import re
+import shutil
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -27,6 +30,18 @@ def test_builds_and_exports_every_declared_symbol():
     for name in names:
         assert hasattr(lib, name), name
     assert sorted(api.EXPORTS) == names
+
+
+# the library needs nothing of the native views: a copy of it loads, and plans, where they were not built
+def test_loads_without_the_native_views(tmp_path):
+    package = tmp_path / "paper_2202_02365_b200"
+    package.mkdir()
+    for name in ("__init__.py", "api.py", "build.py", "inputs.py", "libmgdense.so"):
+        shutil.copy(os.path.join(api.HERE, name), package / name)
+    code = ("import paper_2202_02365_b200 as mg; from paper_2202_02365_b200 import api; assert api.HERE != %r; "
+            "assert mg.load_library().mg_kernel_launches(None) == 0 and len(api.comet_plan(8, 4, 2, 1)['sets']) >= 1" % api.HERE)
+    ran = subprocess.run([sys.executable, "-c", code], cwd=tmp_path, capture_output=True, text=True)
+    assert ran.returncode == 0, ran.stderr[-2000:]
 
 
 @pytest.mark.skipif(torch.cuda.is_available(), reason="checks the no-GPU behaviour")
