@@ -7,6 +7,7 @@ CPU fallback: a missing library or a failing call raises.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 import warnings
 import weakref
@@ -17,7 +18,6 @@ import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libmgdense.so")
-VIEWS_PATH = os.path.join(HERE, "_mgviews.so")
 
 MG_OK = 0
 ERR_NAMES = {-1: "MG_ERR_ARG", -2: "MG_ERR_STATE", -3: "MG_ERR_NONRESIDENT", -4: "MG_ERR_DUPLICATE",
@@ -77,12 +77,16 @@ def _load_views():
     from Python, at 13 us of host time a view instead of 8."""
     global _views, _export_copy
     if _views is None:
-        if os.path.exists(VIEWS_PATH):
-            from . import _mgviews
+        from . import build
+        path = build.views_path()
+        if os.path.exists(path):
+            spec = importlib.util.spec_from_file_location(__package__ + "._mgviews", path)
+            views = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(views)
             _export_copy = C.cast(load_library().mg_dense_export_copy_aligned, C.c_void_p).value
-            _views = _mgviews
+            _views = views
         else:
-            warnings.warn(f"{VIEWS_PATH} is missing (`python -m paper_2202_02365_b200.build` makes it): views of an export take longer", RuntimeWarning, stacklevel=3)
+            warnings.warn(f"{path} is missing (`python -m paper_2202_02365_b200.build` makes it): views of an export take longer", RuntimeWarning, stacklevel=3)
             _views = False
     return _views
 

@@ -1,18 +1,18 @@
-"""Builds libmgdense.so (sm_100a only) next to this file with nvcc, and _mgviews.so, the part of the binding that makes torch tensors, with
-g++; no JIT cache is used."""
+"""Builds libmgdense.so (sm_100a only) next to this file with nvcc, and the native views (_mgviews.*.so), the part of the binding that makes
+torch tensors, with g++; no JIT cache is used."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmgdense.so")
-VIEWS = os.path.join(HERE, "_mgviews.so")
 OBJ_DIR = os.path.join(HERE, "build")
 
 NVCC_FLAGS = [
@@ -33,15 +33,19 @@ def sources():
     return sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cu"))
 
 
-def _views_command(src: str):
-    import sysconfig
+def views_path() -> str:
+    """The native views lay torch's and Python's structures out as their headers have them: a file of its own for each pair of versions."""
+    import torch
+    return os.path.join(HERE, f"_mgviews.{sysconfig.get_config_var('SOABI')}.torch-{torch.__version__}.so")
 
+
+def _views_command(src: str):
     import torch
     from torch.utils import cpp_extension
     includes = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], *cpp_extension.include_paths()]
     libs = cpp_extension.library_paths()
     return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-            *[f for d in includes for f in ("-isystem", d)], src, "-o", VIEWS, *[f"-L{d}" for d in libs], "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10"]
+            *[f for d in includes for f in ("-isystem", d)], src, "-o", views_path(), *[f"-L{d}" for d in libs], "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10"]
 
 
 def _stale(target: str, deps) -> bool:
@@ -72,7 +76,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
             raise RuntimeError("compiler failed: " + " ".join(cmd))
 
     views_src = os.path.join(CSRC, "mg_views.cpp")
-    views = [_views_command(views_src)] if force or _stale(VIEWS, [views_src, os.path.join(ROOT, "include", "mgdense.h")]) else []
+    views = [_views_command(views_src)] if force or _stale(views_path(), [views_src, os.path.join(ROOT, "include", "mgdense.h")]) else []
     with ThreadPoolExecutor(max_workers=max(1, min(8, len(jobs) + 1))) as ex:
         list(ex.map(run, jobs + views))
     if jobs or force or _stale(LIB, objs):

@@ -1,10 +1,12 @@
 """What the binding hands out and takes in: tensors with a start and an autograd life of their own, sizes as they were given."""
+import os
+
 import numpy as np
 import pytest
 import torch
 
 import paper_2202_02365_b200 as mg
-from paper_2202_02365_b200 import api, inputs
+from paper_2202_02365_b200 import api, build, inputs
 
 N = 5_000
 
@@ -55,7 +57,7 @@ def test_export_views_without_the_native_part(sample, monkeypatch):
     keys = ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map")
     native = [dense.export_view(b) for b in range(3)]
     monkeypatch.setattr(api, "_views", None)
-    monkeypatch.setattr(api, "VIEWS_PATH", api.VIEWS_PATH + ".missing")
+    monkeypatch.setattr(build, "views_path", lambda: os.path.join(build.HERE, "not_built.so"))
     with pytest.warns(RuntimeWarning, match="missing"):
         plain = [dense.export_view(b) for b in range(3)]
     for x, y in zip(native, plain):

@@ -5,12 +5,13 @@ import re
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 import pytest
 import torch
 
 import paper_2202_02365_b200 as mg
-from paper_2202_02365_b200 import api
+from paper_2202_02365_b200 import api, build
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -42,6 +43,22 @@ def test_loads_without_the_native_views(tmp_path):
             "assert mg.load_library().mg_kernel_launches(None) == 0 and len(api.comet_plan(8, 4, 2, 1)['sets']) >= 1" % api.HERE)
     ran = subprocess.run([sys.executable, "-c", code], cwd=tmp_path, capture_output=True, text=True)
     assert ran.returncode == 0, ran.stderr[-2000:]
+
+
+# native views that were built for another torch or another Python are not taken for those of this one: neither loaded nor left unbuilt
+def test_native_views_belong_to_their_versions(monkeypatch):
+    build.build()
+    assert os.path.exists(build.views_path())
+    for module, name, value in ((torch, "__version__", "0.0.0+other"), (sysconfig, "get_config_var", lambda name: "cpython-00-other")):
+        with monkeypatch.context() as m:
+            m.setattr(module, name, value)
+            m.setattr(api, "_views", None)
+            asked = []
+            m.setattr(build.subprocess, "run", lambda command, **_: asked.append(command) or subprocess.CompletedProcess(command, 0, "", ""))
+            build.build()
+            assert [c[c.index("-o") + 1] for c in asked] == [build.views_path()]      # (the library itself is as it was)
+            with pytest.warns(RuntimeWarning, match="missing"):
+                assert api._load_views() is False
 
 
 @pytest.mark.skipif(torch.cuda.is_available(), reason="checks the no-GPU behaviour")
