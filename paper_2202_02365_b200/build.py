@@ -75,13 +75,20 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         if r.returncode != 0:
             raise RuntimeError("compiler failed: " + " ".join(cmd))
 
-    views_src = os.path.join(CSRC, "mg_views.cpp")
-    views = [_views_command(views_src)] if force or _stale(views_path(), [views_src, os.path.join(ROOT, "include", "mgdense.h")]) else []
+    # (the library does without the views, so it is there whatever becomes of them, and the views need what the library does not: Python's headers)
+    views_src, views = os.path.join(CSRC, "mg_views.cpp"), None
     with ThreadPoolExecutor(max_workers=max(1, min(8, len(jobs) + 1))) as ex:
-        list(ex.map(run, jobs + views))
-    if jobs or force or _stale(LIB, objs):
-        run([nvcc, "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a",
-             "-Xcompiler", "-fPIC", "-lcudart_static", "-ldl", "-lpthread", "-lrt"])
+        if force or _stale(views_path(), [views_src, os.path.join(ROOT, "include", "mgdense.h")]):
+            if os.path.exists(os.path.join(sysconfig.get_paths()["include"], "Python.h")):
+                views = ex.submit(run, _views_command(views_src))
+            else:
+                sys.stderr.write("no Python.h: the native views are left out, and views of an export take longer\n")
+        list(ex.map(run, jobs))
+        if jobs or force or _stale(LIB, objs):
+            run([nvcc, "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a",
+                 "-Xcompiler", "-fPIC", "-lcudart_static", "-ldl", "-lpthread", "-lrt"])
+    if views:
+        views.result()
     return LIB
 
 

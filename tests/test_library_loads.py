@@ -61,6 +61,24 @@ def test_native_views_belong_to_their_versions(monkeypatch):
                 assert api._load_views() is False
 
 
+# the library is built where the views cannot be: without Python's headers, and where their compiler fails (which is said, behind the library)
+def test_builds_the_library_whatever_becomes_of_the_views(monkeypatch, tmp_path, capsys):
+    asked = []
+
+    def run(command, **_):
+        asked.append(command)
+        return subprocess.CompletedProcess(command, int(command[0] == "g++"), "", "")
+    monkeypatch.setattr(build.subprocess, "run", run)
+    with monkeypatch.context() as m:
+        m.setattr(sysconfig, "get_paths", lambda: {"include": str(tmp_path)})
+        assert build.build(force=True) == build.LIB
+    assert "Python.h" in capsys.readouterr().err and build.LIB in asked[-1] and all(c[0] != "g++" for c in asked)
+    asked.clear()
+    with pytest.raises(RuntimeError, match="compiler failed"):
+        build.build(force=True)
+    assert any(build.LIB in c for c in asked)
+
+
 @pytest.mark.skipif(torch.cuda.is_available(), reason="checks the no-GPU behaviour")
 def test_no_cpu_fallback():
     with pytest.raises(RuntimeError):
