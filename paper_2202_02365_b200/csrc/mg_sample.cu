@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kThreads) k_begin(BeginArgs a) {
 // totals are chained through one 64-bit word per tile (decoupled look-back), and the block's warps then pick for the tile's
 // nodes from shared memory.  Before, these were five kernels with the row bounds, degrees and counts going through memory
 // between them (one mini-batch of three hops on 1M nodes: 48 -> 32 us; 128 mini-batches, last hop of 2.7M nodes: 315 -> 288
-// us).  A tile has as few nodes as leave five tiles per SM (hop_tile): the picks of a warp's nodes are one chain after
+// us).  A tile has as few nodes as leave one for every block that the SMs hold (hop_tile): the picks of a warp's nodes are one chain after
 // the other, and a hop of 1,000 nodes took 21 us with 256 of them per block, 10 us with 32.  Tiles are handed out by a
 // counter, as chain_tiles wants it.
 // Hop 0 also enters the targets: residency and range checks, the id table (Algorithm 1 wants unique targets).  The other hops start from the
@@ -188,7 +188,7 @@ struct HopArgs {
     int64_t cap_entries;
     uint64_t* tile_state;
     int32_t tile_cap;             // nodes of a tile that the launch has shared memory for
-    int32_t n_sms;
+    int32_t n_sms, per_sm;        // (blocks of this instance that an SM holds)
     int32_t B, k;
     // hops > 0: the nodes are what k_insert found new in the hop before
     const int32_t* new_ids;       // by rank, mini-batch b's from the place of its first entry on
@@ -206,16 +206,22 @@ struct HopArgs {
     FeatGeom feat;
 };
 
-// Nodes of a tile.  Below 256 as few as leave five tiles per SM (measured: with four the hop of one mini-batch takes 34.9 us instead of
-// 28.7; k_hop is declared for four blocks per SM and its 48 registers let five onto one: declared for five it loses loads in flight); above 256
-// where twelve tiles per SM are left all the same: the chain through the tiles costs about 13 ns each (2.7M nodes: 620 us with
-// tiles of 64, 475 with 128, 342 with 256, 288 with 1,024).
-constexpr int kTilesPerSm = 5, kTilesPerSmLarge = 12, kTileMax = 1024, kTileSets = kTileMax / kThreads;
+// Blocks of k_hop that an SM holds by their registers.  Groups of lanes: five (declared for four they take 48 registers; declared for five they
+// lose loads in flight).  A thread per node: four of 64 registers, five for the fanouts that leave few look-ups in flight anyway (0.5M nodes of 2 in
+// blocks of 48 registers 57 us, of 64 registers 65).
+constexpr int kHopBlocks = 5;
+__host__ __device__ constexpr int hop_blocks(bool thread, int f) { return thread && f > 2 ? 4 : kHopBlocks; }
+
+// Nodes of a tile.  Below 256 as few as leave a tile for every block that the SMs hold (groups of lanes: with four per SM the hop of one
+// mini-batch takes 34.9 us instead of 28.7; a thread per node, where a fifth waits for a second wave: 94,000 nodes of 5 in tiles for four
+// 15 us, for five 21); above 256 where twelve tiles per SM are left all the same: the chain through the tiles costs about 13 ns each (2.7M nodes:
+// 620 us with tiles of 64, 475 with 128, 342 with 256, 288 with 1,024).
+constexpr int kTilesPerSmLarge = 12, kTileMax = 1024, kTileSets = kTileMax / kThreads;
 constexpr int kTileParts = kTileSets * kThreads / 32;
 static_assert(kTileParts <= 32, "one warp scans the tile's warp totals");
-__host__ __device__ __forceinline__ int hop_tile(int64_t n, int n_sms) {
+__host__ __device__ __forceinline__ int hop_tile(int64_t n, int n_sms, int per_sm) {
     for (int t = 32; t < kThreads; t <<= 1)
-        if (n <= (int64_t)t * kTilesPerSm * n_sms) return t;
+        if (n <= (int64_t)t * per_sm * n_sms) return t;
     for (int t = kTileMax; t > kThreads; t >>= 1)
         if (n > (int64_t)t * kTilesPerSmLarge * n_sms) return t;
     return kThreads;
@@ -229,10 +235,25 @@ __host__ __device__ __forceinline__ int hop_node_bytes(bool inout) { return 12 +
 // (DRAM bursts of the picks), 0.5M 67 / 54, 128,000 of 15 36 / 27; fanouts of seven to ten gain nothing (0.3M of 10: 87 / 92: the picks and the row
 // bounds in flight leave room for four blocks per SM where lanes have five), nor do fewer nodes than that (18,600 of 5: 14 / 15).
 constexpr int kThreadPicks = 20, kThreadTile = 128;
-__host__ __device__ __forceinline__ bool hop_by_thread(int f, int tile_cap) { return tile_cap >= kThreads && (f <= 6 || f > 10) && f <= kThreadPicks; }
+static bool hop_by_thread(int f, int64_t bound, int n_sms) { return hop_tile(bound, n_sms, kHopBlocks) >= kThreads && (f <= 6 || f > 10) && f <= kThreadPicks; }
 // shared memory for the picks of a block's threads
-__host__ __device__ __forceinline__ size_t hop_pick_bytes(int f, int tile_cap, bool inout) {
-    return hop_by_thread(f, tile_cap) ? (size_t)kThreads * f * (inout ? 2 : 1) * sizeof(uint32_t) : 0;
+static size_t hop_pick_bytes(int f, bool inout) { return (size_t)kThreads * f * (inout ? 2 : 1) * sizeof(uint32_t); }
+
+// How a hop of at most `bound` nodes is launched; `tables`: bytes of the mini-batches' tables.
+struct HopLaunch {
+    bool thread;        // a thread per node
+    int32_t per_sm;     // blocks that an SM holds
+    int32_t tile_cap;   // nodes of a tile at most
+    size_t smem;
+};
+static HopLaunch hop_launch(int f, int64_t bound, int n_sms, bool inout, size_t tables) {
+    HopLaunch l;
+    l.thread = hop_by_thread(f, bound, n_sms);
+    l.per_sm = hop_blocks(l.thread, f);
+    l.tile_cap = hop_tile(bound, n_sms, l.per_sm);
+    l.smem = tables + (size_t)l.tile_cap * hop_node_bytes(inout) + (l.thread ? hop_pick_bytes(f, inout) : 0);
+    if (f > 32) l.smem += (size_t)(kThreads / 32) * 2 * f * sizeof(uint32_t);   // (64 KiB at the largest fanout)
+    return l;
 }
 
 // the mini-batch of target i: a 32-way search of the warp for its first target, then a walk
@@ -382,7 +403,7 @@ __device__ __forceinline__ int64_t sum_new_nodes(const NewNodes& a, int32_t* nex
 // warp at a time, picks staged in shared memory.
 // THREAD (G <= kThreadPicks): the form for hops of many nodes; small tiles in it are picked by groups of lanes all the same.
 template <int G, bool THREAD>
-__global__ void __launch_bounds__(kThreads, 4) k_hop(HopArgs a) {
+__global__ void __launch_bounds__(kThreads, THREAD ? hop_blocks(true, G) : 4) k_hop(HopArgs a) {
     extern __shared__ __align__(16) uint8_t hop_sm[];   // the tile's nodes, then (G = 0) per warp x[f], pick[f]
     __shared__ uint32_t part[kTileParts];
     __shared__ int32_t sh_tile;
@@ -402,7 +423,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_hop(HopArgs a) {
         n = (int32_t)(end - lo);
     }
     // (an empty hop has one empty tile: it closes the entry range)
-    const int32_t tile_nodes = min(hop_tile(n, a.n_sms), a.tile_cap), n_tiles = max(1, (n + tile_nodes - 1) / tile_nodes);
+    const int32_t tile_nodes = min(hop_tile(n, a.n_sms, a.per_sm), a.tile_cap), n_tiles = max(1, (n + tile_nodes - 1) / tile_nodes);
     const int sets = (tile_nodes + kThreads - 1) / kThreads;   // nodes per thread
     int64_t* node_r0 = reinterpret_cast<int64_t*>(hop_sm + (a.hop > 0 ? 8 * (size_t)a.B : 0));   // [dirs][tile_cap]
     uint32_t* node_deg = reinterpret_cast<uint32_t*>(node_r0 + (inout ? 2 : 1) * a.tile_cap);   // [dirs][tile_cap]
@@ -2011,7 +2032,7 @@ static int dev_realloc(mg_ctx* ctx, T** p, size_t elems) {
 }
 
 // tiles of a hop at most (tiles below 256 nodes: at most five per SM)
-static size_t tile_states(const mg_ctx* ctx, int64_t cap_nodes) { return (size_t)cap_nodes / kThreads + (size_t)kTilesPerSm * ctx->n_sms + 2; }
+static size_t tile_states(const mg_ctx* ctx, int64_t cap_nodes) { return (size_t)cap_nodes / kThreads + (size_t)kHopBlocks * ctx->n_sms + 2; }
 
 static int dense_alloc(mg_ctx* ctx, mg_dense* d, int32_t B, int32_t k, int64_t cap_nodes, int64_t cap_entries,
                        int32_t table_size, int32_t smem_nb) {
@@ -2166,8 +2187,8 @@ extern "C" int mg_sample_many(mg_ctx* ctx, const int32_t* targets, int targets_o
 #define MG_HOP_KERNELS k_hop<2, false>, k_hop<3, false>, k_hop<4, false>, k_hop<5, false>, k_hop<6, false>, k_hop<8, false>, k_hop<10, false>, k_hop<16, false>, \
                        k_hop<32, false>, k_hop<2, true>, k_hop<3, true>, k_hop<4, true>, k_hop<5, true>, k_hop<6, true>, k_hop<16, true>, k_hop<20, true>
 typedef void (*HopKernel)(HopArgs);
-static HopKernel hop_kernel(int f, int tile_cap) {
-    if (hop_by_thread(f, tile_cap))
+static HopKernel hop_kernel(int f, bool thread) {
+    if (thread)
         return f <= 2 ? k_hop<2, true> : f == 3 ? k_hop<3, true> : f == 4 ? k_hop<4, true> : f == 5 ? k_hop<5, true> : f == 6 ? k_hop<6, true> : f <= 16 ? k_hop<16, true>
                : k_hop<20, true>;
     return f <= 2 ? k_hop<2, false> : f == 3 ? k_hop<3, false> : f == 4 ? k_hop<4, false> : f == 5 ? k_hop<5, false> : f == 6 ? k_hop<6, false> : f <= 8 ? k_hop<8, false>
@@ -2185,7 +2206,7 @@ static int sample_kernel_limits(mg_ctx* ctx) {
 
 // ... and of the others where the mini-batches' tables of k_hop, beside its tile, come to more than a kernel has without asking
 static int hop_kernel_limits(mg_ctx* ctx, int32_t n_batches, bool inout) {
-    if (kTileMax * hop_node_bytes(inout) + 8 * n_batches + (int)hop_pick_bytes(kThreadPicks, kTileMax, inout) <= 47 * 1024) return MG_OK;   // (48 KiB, of which k_hop has some for itself)
+    if (kTileMax * hop_node_bytes(inout) + 8 * n_batches + (int)hop_pick_bytes(kThreadPicks, inout) <= 47 * 1024) return MG_OK;   // (48 KiB, of which k_hop has some for itself)
     const HopKernel hops[] = {MG_HOP_KERNELS};
     for (const HopKernel hop : hops) MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)hop, kHopSmem));
     return MG_OK;
@@ -2388,15 +2409,15 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
         const bool smem_hop = smem_last && h == k - 1;
         {
             ProfScope ps(ctx, PH_SAMPLE_PICK);
+            const HopLaunch l = hop_launch(f, nodes_bound[h], ctx->n_sms, inout, h > 0 ? 8 * (size_t)B : 0);
             HopArgs a{d->hdr, h, f, d->nodes, d->node_batch, {ctx->view_off, inout ? ctx->view_off_out : nullptr},
                       {ctx->view_nbrs, ctx->view_nbrs_out}, d->ent_off, d->ent_nbrs, d->ent_repr, smem_hop ? 0 : 1, d->d_seeds, d->cap_entries, d->tile_state,
-                      hop_tile(nodes_bound[h], ctx->n_sms), ctx->n_sms, B, k, d->new_ids, batch_cnt + (size_t)(h > 0 ? h - 1 : 0) * B, d->cap_nodes,
+                      l.tile_cap, ctx->n_sms, l.per_sm, B, k, d->new_ids, batch_cnt + (size_t)(h > 0 ? h - 1 : 0) * B, d->cap_nodes,
                       inner_limit, d->cum, d->node_off, d->node_off, d->hkeys, d->hvals, tg, ctx->n_nodes, mg_feat_geom(ctx)};
-            const unsigned grid = blocks_for(nodes_bound[h], 32, 8);
-            // (36 KiB, 32 at the largest number of mini-batches, 40 for the picks of a thread per node)
-            const size_t sm = (size_t)a.tile_cap * hop_node_bytes(inout) + (h > 0 ? 8 * (size_t)B : 0) + hop_pick_bytes(f, a.tile_cap, inout);
-            const HopKernel kern = hop_kernel(f, a.tile_cap);
-            kern<<<grid, kThreads, sm + (f > 32 ? (size_t)(kThreads / 32) * 2 * f * sizeof(uint32_t) : 0), st>>>(a);   // 64 KiB more at the largest fanout
+            // (a thread per node: no block waits for another one to end just to find no tile left, 42,000 nodes of 3 12.1 -> 10.8 us)
+            const unsigned grid = blocks_for(nodes_bound[h], 32, l.thread ? l.per_sm : 8);
+            const HopKernel kern = hop_kernel(f, l.thread);
+            kern<<<grid, kThreads, l.smem, st>>>(a);
             ctx->launches++;
         }
         {

@@ -1,5 +1,7 @@
 """The sampler's work is cut by the size of a hop (nodes per tile, buckets of the last hop, table density): the sizes on
 either side of each cut, against the graph's own rows and against the same mini-batches sampled one at a time."""
+import json
+
 import numpy as np
 import pytest
 import torch
@@ -94,6 +96,48 @@ def test_picks_by_threads_and_by_groups_of_lanes(graph, total, direction):
                 assert torch.equal(getattr(x, key), getattr(y, key)), (f, key)
             one.free()
         d.free()
+
+
+def hops_launched(call, tmp_path):
+    """(blocks, blocks that the SMs hold at once, shared memory of those on one SM) of every k_hop that `call` launches."""
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    prof.export_chrome_trace(str(tmp_path / "trace.json"))
+    events = [e for e in json.load(open(tmp_path / "trace.json"))["traceEvents"] if e.get("cat") == "kernel" and "k_hop" in e["name"]]
+    launched = []
+    for e in sorted(events, key=lambda e: e["ts"]):
+        registers, smem = -(-e["args"]["registers per thread"] // 8) * 8, e["args"]["shared memory"] + 1024      # (a kilobyte of every block is the system's)
+        held = min(65536 // (256 * registers), 228 * 1024 // smem)
+        launched.append((e["args"]["grid"][0], held * torch.cuda.get_device_properties(0).multi_processor_count, held * smem))
+    return launched
+
+
+# the blocks of a hop that may be picked by a thread per node are all on the SMs at once, whatever the hop turns out to have: without caps far
+# less than its bound.  Tiles of every size in that form, fanouts on either side of its instances, one list and both
+@pytest.mark.parametrize("direction", ["in", "inout"])
+@pytest.mark.parametrize("targets", [4_200, 9_000, 30_000])
+def test_later_hops_that_have_less_than_their_bound(graph, direction, targets, tmp_path):
+    c = mg.Context(0)
+    c.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    c.load_features(torch.zeros((N, 4), device="cuda"))
+    other = inputs.rmat_graph(N, 20 * N, seed=22)
+    if direction == "inout":
+        c.load_out_graph(other.row_offsets.cuda(), other.nbrs.cuda())
+        c.set_sample_direction("inout")
+    ids = [inputs.distinct_targets(N, n, seed=n) for n in (targets - 1, 1)]
+    pair = torch.cat(ids).cuda()
+    for f in (1, 2, 3, 5, 6, 11, 16, 20):
+        d = c.sample_many(pair, [0, targets - 1, targets], [40, f], [3, 4])
+        one = c.sample(ids[1].cuda(), [40, f], 4)      # (the few nodes of the second mini-batch alone: a group of lanes per node)
+        x, y = d.view(1), one.view(0)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (f, key)
+        launched = hops_launched(lambda: c.sample_many(pair, [0, targets - 1, targets], [40, f], [3, 4], out=d), tmp_path)
+        assert len(launched) == 2 and launched[1][0] <= launched[1][1], (f, launched)
+        one.free()
+        d.free()
+    c.close()
 
 
 # the last hop: through the global tables (little room in all); buckets in shared memory, one (a table of a few hundred nodes), several
