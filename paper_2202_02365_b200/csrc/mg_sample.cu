@@ -239,7 +239,13 @@ static bool hop_by_thread(int f, int64_t bound, int n_sms) { return hop_tile(bou
 // shared memory for the picks of a block's threads
 static size_t hop_pick_bytes(int f, bool inout) { return (size_t)kThreads * f * (inout ? 2 : 1) * sizeof(uint32_t); }
 
-// How a hop of at most `bound` nodes is launched; `tables`: bytes of the mini-batches' tables.
+// Shared memory of the blocks on one SM, and what of it leaves look-ups a useful L1: the driver takes the smallest split that holds the blocks, and beyond
+// 196 KiB that is the one of 228, with 28 KiB left (2M nodes of 6 in both lists, four blocks of 48 KiB: 818 us, groups of lanes 552).  A thread per node stays below it:
+// in the largest tiles of which all blocks do, or, where the picks alone are too many, with fewer blocks.
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemWithL1 = 196 * 1024, kSmemOfBlock = 1024 + 256;   // (the system's part of a block and its static variables)
+
+// How a hop of at most `bound` nodes is launched; `tables`: bytes of the mini-batches' tables.  (us, always 1,024 nodes a tile / smaller ones: both lists,
+// 2M nodes of 6 818 / 424, 1M of 15 833 / 408; fewer blocks: 0.5M of 20 551 / 318, 94,000 of 20 147 / 70.)
 struct HopLaunch {
     bool thread;        // a thread per node
     int32_t per_sm;     // blocks that an SM holds
@@ -251,7 +257,15 @@ static HopLaunch hop_launch(int f, int64_t bound, int n_sms, bool inout, size_t 
     l.thread = hop_by_thread(f, bound, n_sms);
     l.per_sm = hop_blocks(l.thread, f);
     l.tile_cap = hop_tile(bound, n_sms, l.per_sm);
-    l.smem = tables + (size_t)l.tile_cap * hop_node_bytes(inout) + (l.thread ? hop_pick_bytes(f, inout) : 0);
+    auto room = [&](int tile) { return tables + (size_t)tile * hop_node_bytes(inout) + (l.thread ? hop_pick_bytes(f, inout) : 0); };
+    if (l.thread) {
+        int tile = l.tile_cap;
+        while (tile > kThreads && l.per_sm * (room(tile) + kSmemOfBlock) > kSmemWithL1) tile /= 2;
+        if (l.per_sm * (room(tile) + kSmemOfBlock) <= kSmemWithL1) l.tile_cap = tile;
+        else while (l.per_sm > 2 && l.per_sm * (room(l.tile_cap) + kSmemOfBlock) > kSmemWithL1) --l.per_sm;
+    }
+    l.smem = room(l.tile_cap);
+    if (l.thread && l.per_sm < hop_blocks(true, f)) l.smem = std::max(l.smem, kSmemPerSm / (l.per_sm + 1));   // (no room for one more)
     if (f > 32) l.smem += (size_t)(kThreads / 32) * 2 * f * sizeof(uint32_t);   // (64 KiB at the largest fanout)
     return l;
 }

@@ -135,8 +135,34 @@ def test_later_hops_that_have_less_than_their_bound(graph, direction, targets, t
             assert torch.equal(getattr(x, key), getattr(y, key)), (f, key)
         launched = hops_launched(lambda: c.sample_many(pair, [0, targets - 1, targets], [40, f], [3, 4], out=d), tmp_path)
         assert len(launched) == 2 and launched[1][0] <= launched[1][1], (f, launched)
+        assert launched[1][2] <= 196 * 1024, (f, launched)      # (above, the look-ups have next to no L1)
         one.free()
         d.free()
+    c.close()
+
+
+# both lists in hops of more than a million nodes: tiles of 1,024, 512 and 256 nodes by what the picks leave of the shared memory, and fewer blocks
+@pytest.mark.parametrize("fanout", [2, 4, 6, 12, 16, 20])
+def test_picks_by_threads_in_tiles_that_leave_room_for_them(graph, fanout, tmp_path):
+    c = mg.Context(0)
+    c.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    other = inputs.transpose_csr(graph)
+    c.load_out_graph(other.row_offsets.cuda(), other.nbrs.cuda())
+    c.set_sample_direction("inout")
+    n_batches, per = 700, 700
+    rows = [inputs.distinct_targets(N, per - b % 2, seed=b) for b in range(n_batches)]
+    offs = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    caps = {"max_nodes_per_batch": 60_000, "max_nodes_total": 16_000_000 + 4_000_000 * fanout, "max_entries_total": 16_000_000 + 6_000_000 * fanout}
+    d = c.sample_many(torch.cat(rows), offs, [3, fanout], list(range(n_batches)), caps=caps)
+    assert int(d.counts()[0][:, 1].sum()) > 1_818_624      # (tiles of 1,024 where they fit)
+    launched = hops_launched(lambda: c.sample_many(torch.cat(rows), offs, [3, fanout], list(range(n_batches)), caps=caps, out=d), tmp_path)
+    assert launched[1][0] <= launched[1][1] and launched[1][2] <= 196 * 1024, launched
+    for b in (0, 1, n_batches // 2, n_batches - 1):
+        one = c.sample(rows[b], [3, fanout], b)
+        x, y = d.view(b), one.view(0)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
+        one.free()
     c.close()
 
 
