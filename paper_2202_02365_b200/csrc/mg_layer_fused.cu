@@ -117,7 +117,7 @@ struct FusedArgs {
     uint32_t* error;
 };
 
-constexpr int kTsMaxEntriesPerRow = 8, kTsMaxEntriesNarrow = 16;   // layers with more entries per output row than this stream their weights (narrow: at most 128 output columns)
+constexpr int kTsMaxEntriesPerRow = 8, kTsMaxEntriesNarrow = 16;   // layers with more entries per output row than this stream their weights (narrow: at most 128 output columns; between the two mg_layer_narrow_ts decides)
 constexpr int kLaneEntries = 32;   // rows up to this long are translated by their own lane of the planner warp
 constexpr int kKeyCap = 704;    // source-row indices of a row block's entries cached in shared memory (22 per row: what still fits the 196 KB carve-out)
 
@@ -1139,6 +1139,23 @@ static int mg_layer_tile(const mg_ctx* ctx, int64_t rows) {
     return rows <= 2 * kBlockRows * pairs ? kBlockRows : rounds1 * 8 < rounds2 * 14 ? HM : BM;
 }
 
+// Whether a layer of 9 to 16 entries per row and at most 128 output columns keeps its weights in tensor memory, by what it gains there (time with
+// them there over time with them streamed; 9 and 16 entries, 600 to 130,000 rows, 16 to 256 input columns, fp32 and fp16 rows).  For it: no slice is
+// waited for, and half the epilogue of a wider layer.  Against it: all weights have to be there before a tile's first product.  That shows in the
+// one tile that a CTA has of a small first layer (a later layer's weights come in beside the layer before), and where there are no more slices than the
+// ring holds (n_chunks = 2), which arrive in time anyway.
+//   32-row tiles                      0.80 - 1.04; first layers of fp32 rows wider than 64 into more than 112 columns 0.98 - 1.06
+//   first layers, one tile per CTA    more than four slices and up to 112 columns 0.90 - 1.04, else 0.95 - 1.10
+//   ... several                       two slices 0.93 - 1.01 (65 to 112 columns) and 0.98 - 1.05 (others), more 0.88 - 1.03
+//   later layers                      two slices and one tile per CTA 0.96 - 1.05, else 0.80 - 1.03; that leave aggregates for the backward pass: up to
+//                                     four slices in 128-row tiles 1.02 - 1.08, else 0.81 - 1.01
+static bool mg_layer_narrow_ts(bool first, bool keep, bool f16, int n_chunks, int d_out, int tile_rows, bool one_tile) {
+    const bool two = n_chunks <= 2, wide = d_out > 112;
+    if (tile_rows == kBlockRows) return !first || !wide || f16 || n_chunks <= 4;
+    if (!first) return n_chunks > 4 || (keep ? tile_rows == HM : !two || !one_tile);
+    return one_tile ? n_chunks > 4 && !wide : !two || (d_out > 64 && !wide);
+}
+
 bool mg_layer_rows_inline(const mg_ctx* ctx, const mg_dense* d) {
     if (d->n_batches != 1) return false;
     for (int l = 1; l <= d->k; ++l)
@@ -1222,10 +1239,14 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     // weights in tensor memory: TF32 operands, fp32 output, all of K in 256 columns, at most 256 output columns
     // ... and rows with few entries: a half tile of long rows is gathered for longer than its weight slices take to
     // arrive, so the stream costs nothing there, while the transposed epilogue does (measured: 5.3 entries per row,
-    // 2.03 -> 1.92 ms with the weights in tensor memory; 20 per row, 0.83 -> 0.90 ms).  That epilogue is half as long for up to 128 output
-    // columns: 71,000 rows of 11 entries, 100 -> 100 columns, 92 -> 87 us; 66,000 of 14, 32 to 128 columns, 72 -> 70 to 92 -> 87
+    // 2.03 -> 1.92 ms with the weights in tensor memory; 20 per row, 0.83 -> 0.90 ms).  Up to 128 output columns: mg_layer_narrow_ts
+    // (71,000 rows of 11 entries, 100 -> 100 columns, 92 -> 87 us)
+    const bool first = layer == 1, half = first && ctx->feat_dtype == MG_DTYPE_F16, keep = positive || kept_agg;
+    const int64_t n_tiles = (rows + tile_rows - 1) / tile_rows;
     const int64_t layer_entries = d->h_hdr.ent_base[d->k - layer + 1], layer_rows = d->h_hdr.rows_total[layer];
-    const bool ts = n_chunks <= 8 && d_out <= 256 && layer_entries <= (d_out <= 128 ? kTsMaxEntriesNarrow : kTsMaxEntriesPerRow) * layer_rows && !getenv("MG_FUSED_NO_TS");
+    const bool few = layer_entries <= kTsMaxEntriesPerRow * layer_rows || (d_out <= 128 && layer_entries <= kTsMaxEntriesNarrow * layer_rows &&
+                                                                          mg_layer_narrow_ts(first, keep, f16, n_chunks, d_out, tile_rows, n_tiles <= 2 * pairs));
+    const bool ts = n_chunks <= 8 && d_out <= 256 && few && !getenv("MG_FUSED_NO_TS");
     if (ts) { a.tmem_cols = 512; a.sb = 0; a.w_rows = f16 ? (const void*)w_pad_h : (const void*)w_pad_t; }
     const size_t smem = (size_t)a.sa * stage_bytes(halves) + (size_t)a.sb * b_bytes + 1024;
     CUtensorMap mw;
@@ -1240,7 +1261,6 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
     CUtensorMap mo2 = mo;
     if (h_out2 && (out_f16 || !make_map_f32(&mo2, h_out2, row_hi, d_out, 32)))
         return mg_fail(ctx, MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the layer output");
-    const bool first = layer == 1, half = first && ctx->feat_dtype == MG_DTYPE_F16;
     typedef void (*Kernel)(CUtensorMap, CUtensorMap, CUtensorMap, FusedArgs);
     // (kept outputs are fp32: fp16 rows as a later layer's input have no instance that keeps)
 #define MG_FUSED_KERNELS(TS, ROWS, KEEP) \
@@ -1251,12 +1271,10 @@ int mg_layer_fused(mg_ctx* ctx, const mg_dense* d, int layer, int d_in, int d_ou
                                             {MG_FUSED_FORMS(false, BM), MG_FUSED_FORMS(true, BM)}};
 #undef MG_FUSED_FORMS
 #undef MG_FUSED_KERNELS
-    const bool keep = positive || kept_agg;
     if (keep && (in_f16 || out_f16)) return mg_fail(ctx, MG_ERR_STATE, "fp16 layer outputs are not kept");
     const int which = (first ? (f16 ? 2 : half ? 1 : 0) : (f16 ? 4 : 3)) + (keep ? 5 : 0);
     const Kernel kern = kernels[tile_rows == BM ? 2 : tile_rows == HM ? 1 : 0][ts][which];
     MG_CUDA(ctx, mg_smem_limit(ctx, (const void*)kern, fused_smem_limit(halves)));
-    const int64_t n_tiles = (rows + tile_rows - 1) / tile_rows;
     const int grid = 2 * (int)std::min<int64_t>((n_tiles + 1) / 2, pairs);   // CTA pairs
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kFusedThreads); cfg.dynamicSmemBytes = smem; cfg.stream = ctx->stream;

@@ -1,5 +1,8 @@
 """The fused layer kernel cuts a layer's rows into tiles of 32, 64 or 128 per CTA by how many rows there are: row counts on either
 side of every cut, with the weights in tensor memory and streamed, against the layer's definition in fp64."""
+import json
+import re
+
 import pytest
 import torch
 
@@ -226,3 +229,44 @@ def test_long_rows_of_narrow_outputs(monkeypatch, d_in, d_out, fanout):
     want = last_layer(dense.view(0), feats, *layer)
     # (operands rounded to 10 bits: as in test_rows_on_either_side_of_the_tile_sizes)
     assert float((out.double() - want).norm() / want.norm()) < 1e-3
+
+
+def layers_launched(call, tmp_path):
+    """Template arguments (FIRST, HALF, F16, TS, ROWS, KEEP) of every layer kernel that `call` launches."""
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    prof.export_chrome_trace(str(tmp_path / "trace.json"))
+    events = [e for e in json.load(open(tmp_path / "trace.json"))["traceEvents"] if e.get("cat") == "kernel" and "k_sage_layer_fused" in e["name"]]
+    return [re.search(r"k_sage_layer_fused<(.*?)>", e["name"]).group(1).split(", ") for e in sorted(events, key=lambda e: e["ts"])]
+
+
+# which layers keep their weights in tensor memory: rows of exactly as many entries as the rule allows and of one more; of 9 to 16, tiles of every height
+# with one of them per CTA and several, two slices of weights and more, widths on either side of the rule's, fp16 rows and intermediates, layers that keep their
+# outputs.  Where they are kept there, bit for bit what the streamed form gives.
+@pytest.mark.parametrize("rows,tile", [(1_000, 32), (9_472, 64), (18_901, 128), (18_945, 64), (28_417, 128)])
+@pytest.mark.parametrize("form,d_in,d_out,entries,kept", [
+    ("fp32", 100, 128, 8, "yyyyy"), ("fp32", 100, 132, 8, "yyyyy"), ("fp32", 100, 132, 9, "nnnnn"), ("fp32", 100, 112, 16, "yyyyy"), ("fp32", 100, 112, 17, "nnnnn"),
+    ("fp32", 100, 128, 9, "nnnyy"), ("fp32", 64, 128, 9, "ynnyy"), ("fp32", 32, 64, 9, "ynnnn"), ("fp32", 32, 100, 9, "ynnyy"), ("fp16", 256, 128, 16, "ynnyy"),
+    ("fp16", 256, 64, 9, "yyyyy"), ("later", 32, 128, 9, "ynnyy"), ("later", 64, 128, 9, "yyyyy"), ("fp16 later", 128, 128, 16, "yyyyy"), ("kept", 64, 64, 9, "yynyn"),
+    ("kept", 128, 64, 9, "yyyyy")])
+def test_weights_in_tensor_memory_by_entries_and_width(monkeypatch, tmp_path, rows, tile, form, d_in, d_out, entries, kept):
+    kept = kept[[1_000, 9_472, 18_901, 18_945, 28_417].index(rows)] == "y"
+    half, later = "fp16" in form, form in ("later", "fp16 later", "kept")
+    gen = torch.Generator().manual_seed(entries)
+    g = inputs.build_csr(torch.randint(N, (N * entries,), generator=gen), torch.arange(N).repeat_interleave(entries), N)
+    ctx = mg.Context(0)
+    ctx.load_graph(g.row_offsets.cuda(), g.nbrs.cuda())
+    width = 64 if later else d_in
+    ctx.load_features(inputs.normal_features(N, width, seed=5, device="cuda", dtype=torch.float16 if half else torch.float32))
+    ctx.keep_layer_outputs(form == "kept")
+    model = ctx.model(inputs.random_bias_layers([width, d_in, d_out] if later else [width, d_out], seed=6))
+    model.set_intermediates(torch.float16 if half else torch.float32)
+    dense = ctx.sample(inputs.distinct_targets(N, rows, seed=7), [entries, 2] if later else [entries], seed=8)
+    out, streamed = torch.empty((rows, d_out), device="cuda"), torch.empty((rows, d_out), device="cuda")
+    last = layers_launched(lambda: ctx.forward(model, dense, out), tmp_path)[-1]
+    assert last == [str(x).lower() for x in (not later, half, half, kept, tile, form == "kept")], last
+    if kept:
+        monkeypatch.setenv("MG_FUSED_NO_TS", "1")
+        assert layers_launched(lambda: ctx.forward(model, dense, streamed), tmp_path)[-1][3] == "false"
+        assert torch.equal(out, streamed)
