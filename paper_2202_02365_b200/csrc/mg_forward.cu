@@ -1389,7 +1389,7 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
     const RowGeom geom{B, k, d->rowbase, d->cum, d->node_off};
     const bool half = ctx->feat_dtype == MG_DTYPE_F16;
     const int grid = mg_grid(ctx, 8);
-    if (!ctx->meta_left) {   // (most forward passes have left it)
+    if (!ctx->meta_left) {   // (the forward pass was in fp32, or of few rows that its layers looked up themselves)
         int64_t meta_at[MG_MAX_HOPS + 2] = {0};
         if ((rc = row_metadata(ctx, d, meta_at))) return rc;
     }
@@ -1440,8 +1440,8 @@ extern "C" int mg_backward_begin(mg_ctx* ctx, mg_model* m, mg_dense* d, const fl
         int64_t meta_at = 0;   // the layer's rows in ws_meta
         for (int q = 1; q < l; ++q) meta_at += d->h_hdr.rows_total[q];
         if (m->precision == MG_GEMM_TF32) {
-            // dW += X^T dPre with X brought together inside the kernel; the row metadata is what the forward pass left (its layers all
-            // have it, mg_forward of this very model and sample was the last to write it)
+            // dW += X^T dPre with X brought together inside the kernel; the row metadata is what mg_forward of this very model and sample left, or
+            // was made above where its layers did without
             if ((rc = mg_layer_grad_weights(ctx, d, l, d_in, d_out, h_prev, dpre_all, ctx->ws_meta + meta_at, m->sum_aggr ? 1 : 0,
                                             ctx->agg_at[l] >= 0 && ctx->agg_sum == m->sum_aggr ? reinterpret_cast<const float*>(ctx->ws_saved + ctx->agg_at[l]) : nullptr,
                                             m->g_w_cat[l - 1]))) return rc;

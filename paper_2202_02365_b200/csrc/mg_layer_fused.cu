@@ -194,7 +194,7 @@ template <> struct PieceSum<true> {
 
 // Row metadata of a sample of one mini-batch, as the planners take it from the sample themselves: lane h knows hop h's first row and first
 // node (there is no mini-batch to look up).  A row then takes the same round trip as from mg_layer_rows' table, and a call of few rows, which is a
-// chain of launches, has one launch less (two layers on a graph of 10,000: the whole call 73.3 -> 70.7 us; three on 1M nodes 154 -> 152.6).
+// chain of launches, has one launch less (two layers on a graph of 10,000: the whole call 74.4 -> 71.5 us; three on 1M nodes: 155 us either way).
 struct HopOfLane { int32_t row0, node0; };
 __device__ __forceinline__ HopOfLane hop_of_lane(const FusedArgs& a) {
     const int lane = threadIdx.x & 31;

@@ -231,6 +231,32 @@ def test_long_rows_of_narrow_outputs(monkeypatch, d_in, d_out, fanout):
     assert float((out.double() - want).norm() / want.norm()) < 1e-3
 
 
+# the same of fp16 rows, of intermediates kept as fp16, of the sum and of both lists
+@pytest.mark.parametrize("half,between,aggregator,direction", [(True, False, "mean", "in"), (False, True, "mean", "in"), (True, True, "mean", "inout"),
+                                                               (False, False, "sum", "in"), (True, False, "sum", "inout")])
+@pytest.mark.parametrize("rows", [1, 700, 1_300])
+def test_rows_looked_up_by_the_layers_in_every_form(graph, rows, half, between, aggregator, direction):
+    ctx = mg.Context(0)
+    ctx.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    if direction == "inout":
+        other = inputs.transpose_csr(graph)
+        ctx.load_out_graph(other.row_offsets.cuda(), other.nbrs.cuda())
+        ctx.set_sample_direction(direction)
+    ctx.load_features(inputs.normal_features(N, 72, seed=5, device="cuda", dtype=torch.float16 if half else torch.float32))
+    ids = inputs.distinct_targets(N, rows + 1, seed=rows)
+    model = ctx.model(inputs.random_bias_layers([72, 128, 20], seed=6))
+    model.set_intermediates(torch.float16 if between else torch.float32)
+    model.set_aggregator(aggregator)
+    one, two = torch.empty((rows, 20), device="cuda"), torch.empty((rows + 1, 20), device="cuda")
+    alone, both = ctx.sample(ids[:rows], [3, 2], seed=8), ctx.sample_many(ids, [0, rows, rows + 1], [3, 2], [8, 9])
+    launches = [ctx.kernel_launches()]
+    for dense, out in ((alone, one), (both, two)):
+        ctx.forward(model, dense, out)
+        launches.append(ctx.kernel_launches())
+    assert torch.equal(one, two[:rows])
+    assert launches[1] - launches[0] == 2 and launches[2] - launches[1] == 3      # (two layers; the table and two layers)
+
+
 def layers_launched(call, tmp_path):
     """Template arguments (FIRST, HALF, F16, TS, ROWS, KEEP) of every layer kernel that `call` launches."""
     with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
