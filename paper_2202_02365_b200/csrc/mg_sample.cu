@@ -1017,18 +1017,15 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_entries(DedupArgs a) 
 }
 
 template <int kDedupThreads>
-__global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
+__global__ void __launch_bounds__(kDedupThreads, kDedupThreads == 1024 ? 2 : 1536 / kDedupThreads) k_dedupe_last(DedupArgs a) {
     extern __shared__ int32_t dedup_sm[];
     __shared__ uint32_t row_base, warp_tot[kDedupThreads / 32];
     __shared__ int32_t run_lo[2][kDedupMaxBuckets], run_start[2][kDedupMaxBuckets + 1];
     if (__syncthreads_or(a.hdr->status != 0)) return;   // (the whole block: another one may be setting it)
-    const uint32_t S = (uint32_t)a.S, nb = (uint32_t)a.nb;
-    int32_t* keys = dedup_sm;
-    int32_t* vals = dedup_sm + S;
+    const uint32_t nb = (uint32_t)a.nb;
     const int32_t b = (int32_t)(blockIdx.x / nb);
     const uint32_t bucket = blockIdx.x % nb;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint32_t i = threadIdx.x; i < S; i += kDedupThreads) keys[i] = -1;
     if (threadIdx.x < 2 * nb) {   // this bucket's runs of pairs, one per share: entries [0], earlier nodes [1] ...
         const uint32_t which = threadIdx.x / nb, r = threadIdx.x % nb;
         const int32_t* so = a.share_off + (((int64_t)which * a.B + b) * nb + r) * (nb + 1) + bucket;
@@ -1046,6 +1043,15 @@ __global__ void __launch_bounds__(kDedupThreads) k_dedupe_last(DedupArgs a) {
         if (r1 < nb) rs[r1 + 1] = (int32_t)end;
         if (lane == 0) rs[0] = 0;
     }
+    __syncthreads();
+    // the table: half as many slots again as there can be ids, no more than there is room for.  (As many as there is room for are cleared and looked through
+    // for nothing where callers leave much of it: 37 mini-batches in four times the room they take 85.6 -> 78.9 us, 32 larger ones 104 -> 94.5, 128 303 -> 289; in half as
+    // much again as they take, as before.)
+    const uint32_t ids = (uint32_t)run_start[0][nb] + (uint32_t)run_start[1][nb];
+    const uint32_t S = min((uint32_t)a.S, ids + ids / 2 + 32u);
+    int32_t* keys = dedup_sm;
+    int32_t* vals = dedup_sm + S;
+    for (uint32_t i = threadIdx.x; i < S; i += kDedupThreads) keys[i] = -1;
     __syncthreads();
     auto pair_at = [&](int which, int32_t i) -> int2* {   // i-th pair of the bucket: which share's run it falls in (run_start ascends)
         uint32_t lo = 0, hi = nb;                           // run_start[lo] <= i < run_start[hi]
@@ -2289,9 +2295,8 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
     int64_t min_nb = (cap_batch + kDedupMaxSlots - 1) / kDedupMaxSlots;
     while (min_nb <= kDedupMaxTables && dedup_slots_for((cap_batch + min_nb - 1) / min_nb) > kDedupMaxSlots) ++min_nb;
     const int64_t dedup_nb = min_nb <= kDedupMaxTables ? dedup_buckets(n_batches, cap_batch, min_nb, ctx->n_sms) : min_nb;
-    // A block of 1,024 threads has its SM's shared memory to itself: its table is half as large again as it has to be, where there is room, and
-    // the probes are shorter (64,000 entries and 29,000 nodes in the buckets of 37 mini-batches 63 -> 58 us, 128 of 103,000 286 -> 273; the smaller
-    // blocks gain nothing, 49 -> 50).
+    // Room for tables half as large again as they have to be, where blocks have 1,024 threads and there is that much: the probes are shorter (32 mini-batches of
+    // 84,500 nodes in as much room 106 -> 65 us, 128 357 -> 245; the smaller blocks gain nothing, 49 -> 50).  k_dedupe_last takes of it what its ids need.
     const int32_t dedup_least = (int32_t)std::min<int64_t>(dedup_slots_for((cap_batch + dedup_nb - 1) / dedup_nb), kDedupMaxSlots);
     const int32_t dedup_slots = dedup_least > kDedupSlots512 ? std::min(kDedupMaxSlots, (dedup_least * 3 / 2 + 127) / 128 * 128) : dedup_least;
     const bool smem_fits = min_nb <= kDedupMaxTables && dedup_nb * n_batches < (1ll << 24) && cap_entries + cap_nodes < (1ll << 31);
@@ -2441,7 +2446,8 @@ static int sample_begin_impl(mg_ctx* ctx, const int32_t* targets, int targets_on
                              d->ent_repr, d->pairs, d->share_off, d->cum, batch_cnt + (size_t)h * B, d->new_ids,
                              (int32_t)cap_batch, d->cap_entries};
                 k_bucket_entries<<<(unsigned)(B * dedup_nb), kBucketThreads, 0, st>>>(da);
-                // (threads so that the blocks that shared memory lets onto an SM come to 2,048 threads)
+                // (threads by table size: registers let six blocks of 256 threads onto an SM, three of 512 and two of 1,024, tables as many of the
+                // first two and, above 113 KB, one of the last)
                 const unsigned grid = (unsigned)(B * dedup_nb);
                 const size_t sm = (size_t)dedup_slots * 2 * sizeof(int32_t);
                 if (dedup_slots > kDedupSlots512) k_dedupe_last<1024><<<grid, 1024, sm, st>>>(da);

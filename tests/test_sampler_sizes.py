@@ -197,6 +197,25 @@ def test_last_hop_buckets(graph, ctx, room, n_batches):
     d.free()
 
 
+# the last hop's tables in shared memory have slots for what their buckets hold, up to the room there is: mini-batches of none, one, few and many
+# targets in one call, with just the room that the largest takes (16,009 nodes) each and with far more
+@pytest.mark.parametrize("room", [16_009, 60_000, 300_000])
+def test_last_hop_of_mini_batches_of_any_size(graph, ctx, room):
+    sizes = [2_000, 0, 1, 3, 60, 700, 0, 1_500] * 10
+    rows = [inputs.distinct_targets(N, n, seed=b) for b, n in enumerate(sizes)]
+    rows[3] = torch.tensor([0, 1, N - 1], dtype=torch.int32)
+    offs = np.concatenate([[0], np.cumsum(sizes)])
+    caps = {"max_nodes_per_batch": room, "max_nodes_total": 1_500_000, "max_entries_total": 2_000_000}
+    d = ctx.sample_many(torch.cat(rows), offs, [2, 3], list(range(len(sizes))), caps=caps)
+    for b in (*range(8), len(sizes) - 1):
+        one = ctx.sample(rows[b], [2, 3], b)
+        x, y = d.view(b), one.view(0)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
+        one.free()
+    d.free()
+
+
 # entries go into the id tables 128 at a time, an entry per thread, or (hops with room for more than the SMs hold at once that way) 512 at
 # a time: either form with blocks that touch a few mini-batches, and more mini-batches than a block keeps counts for
 @pytest.mark.parametrize("per,fanout", [(1, 14), (4, 13), (4, 14)])
