@@ -229,13 +229,14 @@ __host__ __device__ __forceinline__ int hop_tile(int64_t n, int n_sms, int per_s
 // shared memory per node of a tile: id, mini-batch, first entry; first edge and length of its row, once per direction
 __host__ __device__ __forceinline__ int hop_node_bytes(bool inout) { return 12 + (inout ? 24 : 12); }
 
-// Fanouts of up to six and of eleven to kThreadPicks are picked by a thread per node where the hop may have tiles of kThreads nodes and the tile
+// Fanouts of up to kThreadPicks are picked by a thread per node where the hop may have tiles of kThreads nodes and the tile
 // has kThreadTile at least, else by a group of lanes per node.  Lanes: one look-up in flight per lane and as many Philox calls as draws; threads:
 // a quarter of the calls and all of a node's look-ups in flight.  us, lanes / threads: 71,000 nodes of 20 in one mini-batch 47 / 23, 2.7M nodes of 5 302 / 297
-// (DRAM bursts of the picks), 0.5M 67 / 54, 128,000 of 15 36 / 27; fanouts of seven to ten gain nothing (0.3M of 10: 87 / 92: the picks and the row
-// bounds in flight leave room for four blocks per SM where lanes have five), nor do fewer nodes than that (18,600 of 5: 14 / 15).
+// (DRAM bursts of the picks), 0.5M 67 / 54, 128,000 of 15 36 / 27, 0.3M of 10 55 / 38, of 7 49 / 33, both lists 90 / 55 and 81 / 52.  Fewer nodes than that
+// gain nothing (18,600 of 5: 14 / 15); where a hop without caps has far less than its bound, 40,000 nodes of 10 19.6 / 14.1, 2,300 7.9 / 7.9, both lists
+// 69,600 44.7 / 31.9, 22,400 21.6 / 22.9.
 constexpr int kThreadPicks = 20, kThreadTile = 128;
-static bool hop_by_thread(int f, int64_t bound, int n_sms) { return hop_tile(bound, n_sms, kHopBlocks) >= kThreads && (f <= 6 || f > 10) && f <= kThreadPicks; }
+static bool hop_by_thread(int f, int64_t bound, int n_sms) { return hop_tile(bound, n_sms, kHopBlocks) >= kThreads && f <= kThreadPicks; }
 // shared memory for the picks of a block's threads
 static size_t hop_pick_bytes(int f, bool inout) { return (size_t)kThreads * f * (inout ? 2 : 1) * sizeof(uint32_t); }
 
@@ -2205,12 +2206,12 @@ extern "C" int mg_sample_many(mg_ctx* ctx, const int32_t* targets, int targets_o
 // The instance for a fanout, and for as many nodes per tile as the hop may have: the narrowest group of lanes that holds the fanout among
 // those that waste at most two lanes of a warp; a thread per node where the hop fills larger tiles.
 #define MG_HOP_KERNELS k_hop<2, false>, k_hop<3, false>, k_hop<4, false>, k_hop<5, false>, k_hop<6, false>, k_hop<8, false>, k_hop<10, false>, k_hop<16, false>, \
-                       k_hop<32, false>, k_hop<2, true>, k_hop<3, true>, k_hop<4, true>, k_hop<5, true>, k_hop<6, true>, k_hop<16, true>, k_hop<20, true>
+                       k_hop<32, false>, k_hop<2, true>, k_hop<3, true>, k_hop<4, true>, k_hop<5, true>, k_hop<6, true>, k_hop<8, true>, k_hop<10, true>, k_hop<16, true>, k_hop<20, true>
 typedef void (*HopKernel)(HopArgs);
 static HopKernel hop_kernel(int f, bool thread) {
     if (thread)
-        return f <= 2 ? k_hop<2, true> : f == 3 ? k_hop<3, true> : f == 4 ? k_hop<4, true> : f == 5 ? k_hop<5, true> : f == 6 ? k_hop<6, true> : f <= 16 ? k_hop<16, true>
-               : k_hop<20, true>;
+        return f <= 2 ? k_hop<2, true> : f == 3 ? k_hop<3, true> : f == 4 ? k_hop<4, true> : f == 5 ? k_hop<5, true> : f == 6 ? k_hop<6, true> : f <= 8 ? k_hop<8, true>
+               : f <= 10 ? k_hop<10, true> : f <= 16 ? k_hop<16, true> : k_hop<20, true>;
     return f <= 2 ? k_hop<2, false> : f == 3 ? k_hop<3, false> : f == 4 ? k_hop<4, false> : f == 5 ? k_hop<5, false> : f == 6 ? k_hop<6, false> : f <= 8 ? k_hop<8, false>
            : f <= 10 ? k_hop<10, false> : f <= 16 ? k_hop<16, false> : f <= 32 ? k_hop<32, false> : k_hop<0, false>;
 }

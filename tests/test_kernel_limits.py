@@ -89,3 +89,10 @@ def test_small_tiles_of_a_hop_are_all_in_work(program):
             assert held == per_sm and held * (smem + 1024 + 144) <= 196 * 1024, (bound, f, lists)
             assert smem <= 1024 * 36 + 256 * 20 * 2 * 4 + 8 * 4096
         assert -(-n // tile) <= n // 256 + 5 * 148 + 2            # (the tiles' states that a sample has room for)
+
+
+# a hop that may fill tiles of as many nodes as a block has threads is picked by a thread per node, whatever its fanout of up to twenty and its lists
+def test_large_hops_are_picked_by_a_thread_per_node(program):
+    ran = subprocess.run([program, "launches"], capture_output=True, text=True)
+    for bound, n, f, lists, thread, *_ in ([int(x) for x in line.split()] for line in ran.stdout.splitlines()):
+        assert thread == (bound > 128 * 5 * 148 and f <= 20), (bound, f, lists)
