@@ -411,8 +411,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_distmult_neg_tc(NegTcArgs ta)
         const int first_block = job_first, n_blocks = job_blocks;
         float* out = ta.out[job_side];
         // rows start 32-byte aligned: no way round through shared memory, which the MMAs read their operands from meanwhile (100 million scores of
-        // 50,000 edges and 1,000 negatives 142 -> 135 us, 5 million of 5,000 and 500 ones that are 16-byte aligned only: as before)
-        const bool vec8 = a.negs % 8 == 0 && (reinterpret_cast<uintptr_t>(out) & 31) == 0;
+        // 50,000 edges and 1,000 negatives 142 -> 135 us, 5 million of 5,000 and 500 ones that are 16-byte aligned only: as before).  Not rows of whole
+        // 128-byte lines: a slice's four sectors, one row after the other, are a line of its own that the other form stores at once (5,000 edges, 1,504
+        // negatives 34.9 us by sectors, 28.7 by lines, 4,000 75.6 and 61.5; every second row on a line, 2,000: 38.6 and 37.8)
+        const bool lines = a.negs % 32 == 0 && (reinterpret_cast<uintptr_t>(out) & 127) == 0;
+        const bool vec8 = a.negs % 8 == 0 && (reinterpret_cast<uintptr_t>(out) & 31) == 0 && !lines;
         const bool vec4 = a.negs % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;   // rows start 16-byte aligned
         for (int j = 0; j < n_blocks && ok; ++j) {
             const int buf = j & 1;

@@ -85,6 +85,12 @@ def test_negative_scores_by_the_alignment_of_their_rows(edges, chunks, negs):
     test_negative_scores_by_the_number_of_tiles(edges, chunks, negs, mg.CORRUPT_BOTH)
 
 
+# rows of whole 128-byte lines, which are stored by lines: within one slice of 32 columns and one block of them, several of each; every second row on a line
+@pytest.mark.parametrize("edges,chunks,negs", [(131, 1, 32), (300, 2, 128), (257, 3, 1_504), (300, 1, 2_048), (300, 1, 1_008)])
+def test_negative_scores_in_rows_of_whole_lines(edges, chunks, negs):
+    test_negative_scores_by_the_number_of_tiles(edges, chunks, negs, mg.CORRUPT_BOTH)
+
+
 # batches are prepared while the scores of the ones before are computed, in the blocks of freed batches: growing, shrinking, two alive at once
 @pytest.mark.parametrize("sizes", [[40_000] * 6, [100, 40_000, 300, 50_000, 20_000, 60_000]])
 def test_batches_prepared_beside_scores(sizes):
