@@ -215,12 +215,14 @@ __host__ __device__ constexpr int hop_blocks(bool thread, int f) { return thread
 // Nodes of a tile.  Below 256 as few as leave a tile for every block that the SMs hold (groups of lanes: with four per SM the hop of one
 // mini-batch takes 34.9 us instead of 28.7; a thread per node, where a fifth waits for a second wave: 94,000 nodes of 5 in tiles for four
 // 15 us, for five 21); above 256 where twelve tiles per SM are left all the same: the chain through the tiles costs about 13 ns each (2.7M nodes:
-// 620 us with tiles of 64, 475 with 128, 342 with 256, 288 with 1,024).
+// 620 us with tiles of 64, 475 with 128, 342 with 256, 288 with 1,024).  A thread per node has tiles of up to 512 for the first reason too: it takes
+// two nodes at little more than the time of one, and tiles of 256 came to a second wave (200,000 nodes of 1 23.0 -> 18.3 us, 18.7 by groups of lanes; of 5
+// 25.3 -> 17.8, both lists of 10 43.3 -> 37.9).
 constexpr int kTilesPerSmLarge = 12, kTileMax = 1024, kTileSets = kTileMax / kThreads;
 constexpr int kTileParts = kTileSets * kThreads / 32;
 static_assert(kTileParts <= 32, "one warp scans the tile's warp totals");
-__host__ __device__ __forceinline__ int hop_tile(int64_t n, int n_sms, int per_sm) {
-    for (int t = 32; t < kThreads; t <<= 1)
+__host__ __device__ __forceinline__ int hop_tile(int64_t n, int n_sms, int per_sm, bool thread = false) {
+    for (int t = 32; t < (thread ? kTileMax : kThreads); t <<= 1)
         if (n <= (int64_t)t * per_sm * n_sms) return t;
     for (int t = kTileMax; t > kThreads; t >>= 1)
         if (n > (int64_t)t * kTilesPerSmLarge * n_sms) return t;
@@ -229,13 +231,12 @@ __host__ __device__ __forceinline__ int hop_tile(int64_t n, int n_sms, int per_s
 // shared memory per node of a tile: id, mini-batch, first entry; first edge and length of its row, once per direction
 __host__ __device__ __forceinline__ int hop_node_bytes(bool inout) { return 12 + (inout ? 24 : 12); }
 
-// Fanouts of up to kThreadPicks are picked by a thread per node where the hop may have tiles of kThreads nodes and the tile
-// has kThreadTile at least, else by a group of lanes per node.  Lanes: one look-up in flight per lane and as many Philox calls as draws; threads:
+// Fanouts of up to kThreadPicks are picked by a thread per node where the hop may have tiles of kThreads nodes, else by a group of lanes per node.  Lanes: one look-up in flight per lane and as many Philox calls as draws; threads:
 // a quarter of the calls and all of a node's look-ups in flight.  us, lanes / threads: 71,000 nodes of 20 in one mini-batch 47 / 23, 2.7M nodes of 5 302 / 297
-// (DRAM bursts of the picks), 0.5M 67 / 54, 128,000 of 15 36 / 27, 0.3M of 10 55 / 38, of 7 49 / 33, both lists 90 / 55 and 81 / 52.  Fewer nodes than that
-// gain nothing (18,600 of 5: 14 / 15); where a hop without caps has far less than its bound, 40,000 nodes of 10 19.6 / 14.1, 2,300 7.9 / 7.9, both lists
-// 69,600 44.7 / 31.9, 22,400 21.6 / 22.9.
-constexpr int kThreadPicks = 20, kThreadTile = 128;
+// (DRAM bursts of the picks), 0.5M 67 / 54, 128,000 of 15 36 / 27, 0.3M of 10 55 / 38, of 7 49 / 33, both lists 90 / 55 and 81 / 52.  Hops without caps may
+// have far less than their bound: 2,320 nodes of 10 8.3 / 8.3, 22,000 of 5 13.3 / 9.4, of 20 23.3 / 16.2, both lists 22,400 of 5 15.5 / 12.0, of 12 23.9 / 24.3, of 20
+// 36.7 / 28.7, 69,600 of 10 44.8 / 32.0.  (There the small tiles had been left to groups of lanes, four blocks or fewer to an SM instead of five: 36.5 -> 45.)
+constexpr int kThreadPicks = 20;
 static bool hop_by_thread(int f, int64_t bound, int n_sms) { return hop_tile(bound, n_sms, kHopBlocks) >= kThreads && f <= kThreadPicks; }
 // shared memory for the picks of a block's threads
 static size_t hop_pick_bytes(int f, bool inout) { return (size_t)kThreads * f * (inout ? 2 : 1) * sizeof(uint32_t); }
@@ -257,7 +258,8 @@ static HopLaunch hop_launch(int f, int64_t bound, int n_sms, bool inout, size_t 
     HopLaunch l;
     l.thread = hop_by_thread(f, bound, n_sms);
     l.per_sm = hop_blocks(l.thread, f);
-    l.tile_cap = hop_tile(bound, n_sms, l.per_sm);
+    l.tile_cap = hop_tile(bound, n_sms, l.per_sm, l.thread);
+    if (l.thread && bound > (int64_t)kThreads * l.per_sm * n_sms) l.tile_cap = std::max(l.tile_cap, kTileMax / 2);   // (fewer nodes than the bound may want larger tiles)
     auto room = [&](int tile) { return tables + (size_t)tile * hop_node_bytes(inout) + (l.thread ? hop_pick_bytes(f, inout) : 0); };
     if (l.thread) {
         int tile = l.tile_cap;
@@ -416,7 +418,7 @@ __device__ __forceinline__ int64_t sum_new_nodes(const NewNodes& a, int32_t* nex
 // G lanes per node, fanout <= G <= 32; a warp holds 32 / G nodes (G need not divide 32: the lanes left over idle, and
 // G = 5 or 10 keeps 30 lanes busy where the next power of two keeps 20).  G = 0: any fanout up to MG_MAX_FANOUT, a node per
 // warp at a time, picks staged in shared memory.
-// THREAD (G <= kThreadPicks): the form for hops of many nodes; small tiles in it are picked by groups of lanes all the same.
+// THREAD (G <= kThreadPicks): a thread per node, for hops of many nodes.
 template <int G, bool THREAD>
 __global__ void __launch_bounds__(kThreads, THREAD ? hop_blocks(true, G) : 4) k_hop(HopArgs a) {
     extern __shared__ __align__(16) uint8_t hop_sm[];   // the tile's nodes, then (G = 0) per warp x[f], pick[f]
@@ -438,7 +440,7 @@ __global__ void __launch_bounds__(kThreads, THREAD ? hop_blocks(true, G) : 4) k_
         n = (int32_t)(end - lo);
     }
     // (an empty hop has one empty tile: it closes the entry range)
-    const int32_t tile_nodes = min(hop_tile(n, a.n_sms, a.per_sm), a.tile_cap), n_tiles = max(1, (n + tile_nodes - 1) / tile_nodes);
+    const int32_t tile_nodes = min(hop_tile(n, a.n_sms, a.per_sm, THREAD), a.tile_cap), n_tiles = max(1, (n + tile_nodes - 1) / tile_nodes);
     const int sets = (tile_nodes + kThreads - 1) / kThreads;   // nodes per thread
     int64_t* node_r0 = reinterpret_cast<int64_t*>(hop_sm + (a.hop > 0 ? 8 * (size_t)a.B : 0));   // [dirs][tile_cap]
     uint32_t* node_deg = reinterpret_cast<uint32_t*>(node_r0 + (inout ? 2 : 1) * a.tile_cap);   // [dirs][tile_cap]
@@ -600,10 +602,9 @@ __global__ void __launch_bounds__(kThreads, THREAD ? hop_blocks(true, G) : 4) k_
         }
         if (!fits) break;   // (uniform over the block)
         __syncthreads();
-        if (THREAD && tile_nodes >= kThreadTile) {
+        if constexpr (THREAD) {
             // a thread per node: a Philox call gives four draws, and all picks of a node are looked up together.  The warp's entries are
             // put one behind the other in shared memory and written from there.
-            constexpr int GT = THREAD ? G : 1;
             uint32_t* out = reinterpret_cast<uint32_t*>(node_out + a.tile_cap) + (size_t)warp * 32 * f * (inout ? 2 : 1);
 #pragma unroll 1
             for (int t0 = warp * 32; t0 < n_here; t0 += kThreads) {
@@ -616,16 +617,16 @@ __global__ void __launch_bounds__(kThreads, THREAD ? hop_blocks(true, G) : 4) k_
                 for (int dir = 0; dir < (inout ? 2 : 1); ++dir) {   // (the second direction's picks follow the first's)
                     const uint32_t d = on ? node_deg[dir * a.tile_cap + t] : 0u, cnt = min(d, (uint32_t)f);
                     const int32_t* __restrict__ row = a.row_nbrs[dir] + node_r0[dir * a.tile_cap + t];
-                    uint32_t pick[GT];
-                    if (d > (uint32_t)f) floyd_thread<GT>(d, f, a.seeds[gb], (uint32_t)node_id[t], (uint32_t)a.hop, dir ? (uint32_t)MG_OUT_SLOT_BASE : 0u, pick);
+                    uint32_t pick[G];
+                    if (d > (uint32_t)f) floyd_thread<G>(d, f, a.seeds[gb], (uint32_t)node_id[t], (uint32_t)a.hop, dir ? (uint32_t)MG_OUT_SLOT_BASE : 0u, pick);
                     else {   // all neighbours, in row order
 #pragma unroll
-                        for (int j = 0; j < GT; ++j) pick[j] = (uint32_t)j;
+                        for (int j = 0; j < G; ++j) pick[j] = (uint32_t)j;
                     }
 #pragma unroll
-                    for (int j = 0; j < GT; ++j) if ((uint32_t)j < cnt) pick[j] = (uint32_t)__ldg(row + pick[j]);
+                    for (int j = 0; j < G; ++j) if ((uint32_t)j < cnt) pick[j] = (uint32_t)__ldg(row + pick[j]);
 #pragma unroll
-                    for (int j = 0; j < GT; ++j) if ((uint32_t)j < cnt) out[at + j] = pick[j];
+                    for (int j = 0; j < G; ++j) if ((uint32_t)j < cnt) out[at + j] = pick[j];
                     at += cnt;
                 }
                 const uint32_t total = __reduce_max_sync(0xFFFFFFFFu, on ? at : 0u);

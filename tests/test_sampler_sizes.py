@@ -98,6 +98,29 @@ def test_picks_by_threads_and_by_groups_of_lanes(graph, total, direction):
         d.free()
 
 
+# a thread per node in the last tiles of 256 and 512 nodes that are all in work at once, and one node more (148 SMs, four blocks each, five for fanouts of
+# one and two), one list and both
+@pytest.mark.parametrize("fanout,total", [(3, 151_552), (3, 151_553), (20, 303_104), (20, 303_105), (1, 189_441), (2, 378_881)])
+@pytest.mark.parametrize("direction", ["in", "inout"])
+def test_tiles_of_a_thread_per_node(graph, fanout, total, direction):
+    c = mg.Context(0)
+    c.load_graph(graph.row_offsets.cuda(), graph.nbrs.cuda())
+    if direction == "inout":
+        other = inputs.transpose_csr(graph)
+        c.load_out_graph(other.row_offsets.cuda(), other.nbrs.cuda())
+        c.set_sample_direction("inout")
+    sizes = [60_001] * (total // 60_001) + [total % 60_001]
+    ids = [inputs.distinct_targets(N, n, seed=500 + i) for i, n in enumerate(sizes)]
+    d = c.sample_many(torch.cat(ids).cuda(), np.concatenate([[0], np.cumsum(sizes)]), [fanout], [2 ** 40 + 7 * b for b in range(len(sizes))])
+    for b in (0, len(sizes) - 2, len(sizes) - 1):
+        one = c.sample(ids[b].cuda(), [fanout], 2 ** 40 + 7 * b)
+        x, y = d.view(b), one.view(0)
+        for key in ("node_ids", "node_id_offsets", "nbrs", "nbr_offsets", "repr_map"):
+            assert torch.equal(getattr(x, key), getattr(y, key)), (b, key)
+        one.free()
+    c.close()
+
+
 def hops_launched(call, tmp_path):
     """(blocks, blocks that the SMs hold at once, shared memory of those on one SM) of every k_hop that `call` launches."""
     with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
