@@ -231,7 +231,7 @@ class Dense:
     def export_view(self, batch: int = 0) -> DenseView:
         """Mini-batch `batch` of the last export_many, ready in the order of torch's current stream.  (The stream waits for the
         export, not the host: 32 mini-batches' views are queued while the export runs, the whole call 1107 -> 910 us; one call into native
-        code per view, 875 -> 688.)"""
+        code per view, 866 -> 685.)"""
         ctx = self.ctx
         native = _views or _load_views()
         if native:
