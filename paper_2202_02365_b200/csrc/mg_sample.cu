@@ -233,7 +233,8 @@ __host__ __device__ __forceinline__ int hop_node_bytes(bool inout) { return 12 +
 
 // Fanouts of up to kThreadPicks are picked by a thread per node where the hop may have tiles of kThreads nodes, else by a group of lanes per node.  Lanes: one look-up in flight per lane and as many Philox calls as draws; threads:
 // a quarter of the calls and all of a node's look-ups in flight.  us, lanes / threads: 71,000 nodes of 20 in one mini-batch 47 / 23, 2.7M nodes of 5 302 / 297
-// (DRAM bursts of the picks), 0.5M 67 / 54, 128,000 of 15 36 / 27, 0.3M of 10 55 / 38, of 7 49 / 33, both lists 90 / 55 and 81 / 52.  Hops without caps may
+// (DRAM bursts of the picks), 0.5M 67 / 54, 128,000 of 15 36 / 27, 0.3M of 10 55 / 38, of 7 49 / 33, both lists 90 / 55 and 81 / 52; on 16M nodes,
+// whose look-ups are DRAM bursts, 0.32M of 10 88 / 91.  Hops without caps may
 // have far less than their bound: 2,320 nodes of 10 8.3 / 8.3, 22,000 of 5 13.3 / 9.4, of 20 23.3 / 16.2, both lists 22,400 of 5 15.5 / 12.0, of 12 23.9 / 24.3, of 20
 // 36.7 / 28.7, 69,600 of 10 44.8 / 32.0.  (There the small tiles had been left to groups of lanes, four blocks or fewer to an SM instead of five: 36.5 -> 45.)
 constexpr int kThreadPicks = 20;
@@ -1018,6 +1019,8 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_entries(DedupArgs a) 
     }
 }
 
+// (1,024 threads: 32 registers, a few of them spilled, for two blocks per SM where tables leave room for them: 64 mini-batches of 47,000 nodes in half as much room
+// again 76.3 -> 63.1 us; where they don't, 128 of 96,000 254 -> 258)
 template <int kDedupThreads>
 __global__ void __launch_bounds__(kDedupThreads, kDedupThreads == 1024 ? 2 : 1536 / kDedupThreads) k_dedupe_last(DedupArgs a) {
     extern __shared__ int32_t dedup_sm[];
